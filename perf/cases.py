@@ -107,16 +107,17 @@ def _draw_attention(rng):
     return c
 
 
-def _sampling(rng):
-    top_k = rng.choice([0, 0, 10, 10, 50])
+def _sampling(rng, V):
+    # a top-k keeps a small share of the vocabulary; a model of a few thousand tokens is sampled plainly
+    top_k = rng.choice([0, 0] + [k for k in (10, 10, 50) if V >= 1024 * k])
     return dict(temperature=rng.choice([1.0, 0.8, 0.6]), top_k=top_k,
                 top_p=rng.choice([1.0, 0.8, 0.95]) if top_k else 1.0)
 
 
 def _draw_verify(rng):
     c = dict(kind="verify", R=_log_int(rng, 1, 64), W_lo=rng.randint(1, 4), W_hi=rng.randint(4, 8),
-             tree=rng.choice(["chain", "chain", "wide"]), depth=rng.randint(1, 8), V=_vocabulary(rng),
-             **_sampling(rng))
+             tree=rng.choice(["chain", "chain", "wide"]), depth=rng.randint(1, 8), V=_vocabulary(rng))
+    c.update(_sampling(rng, c["V"]))
     if c["tree"] == "wide":
         c["depth"] = 6
     while work(c)["bytes"] > MAX_VERIFY_BYTES:
@@ -125,17 +126,17 @@ def _draw_verify(rng):
 
 
 def _draw_draft(rng):
-    w = rng.randint(1, 8)
-    return dict(kind="draft", R=_log_int(rng, 1, 64), W_lo=w, W_hi=w, gamma=rng.randint(2, 8), V=_vocabulary(rng),
-                **_sampling(rng))
+    w, V = rng.randint(1, 8), _vocabulary(rng)
+    return dict(kind="draft", R=_log_int(rng, 1, 64), W_lo=w, W_hi=w, gamma=rng.randint(2, 8), V=V,
+                **_sampling(rng, V))
 
 
 def _draw_step(rng):
     w = rng.randint(2, 8)
-    lo = _log_int(rng, 128, 2048)
+    lo, V = _log_int(rng, 128, 2048), _vocabulary(rng)
     Hq, Hkv = rng.choice([(32, 8), (32, 32), (40, 40)])
     return dict(kind="step", R=_log_int(rng, 1, 16), W_lo=w, W_hi=w, gamma=rng.randint(2, 5), Hq=Hq, Hkv=Hkv, d=128,
-                dtype="bf16", L_lo=lo, L_hi=rng.choice([lo, 2 * lo + 1]), V=_vocabulary(rng), **_sampling(rng))
+                dtype="bf16", L_lo=lo, L_hi=rng.choice([lo, 2 * lo + 1]), V=V, **_sampling(rng, V))
 
 
 def _draw_commit(rng):

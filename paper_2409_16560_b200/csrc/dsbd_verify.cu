@@ -953,6 +953,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     // when asked, appends them to the candidate list (order is irrelevant: the final choice is
     // by (key, cell)).
     auto sweep = [&](float th, bool collect) {
+        half_sync(model);                      // every thread has taken the previous sweep's count
         if (tl == 0) tp.n_cand = 0;
         half_sync(model);
         // this warp's tiles into L2 first (a tile is 32 lines of 128 bytes: one per lane), so that

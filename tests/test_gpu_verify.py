@@ -283,6 +283,27 @@ def test_warping_edge_settings(top_k, top_p):
     check_exempt(exempt, decisions)
 
 
+@pytest.mark.parametrize("V,top_k", [(1000, 10), (2432, 50), (3000, 64)])
+def test_top_k_near_the_number_of_tiles(V, top_k):
+    """Fewer tiles than kept cells: every tile is taken and the threshold is found by bisection over
+    counts that all threads of a half must read alike (a thread that read the next sweep's count took
+    another branch, and its half waited for it for good).  Every repetition must
+    give the first one's results."""
+    rng = np.random.default_rng(V)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=61, V=V, gamma=2, max_w=8)
+    prm.update(top_k=top_k, top_p=0.95, temperature=0.6, step=1)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    gpu, status = run_gpu_verify(forest, prm, *dev)
+    assert status == 0
+    for _ in range(40):
+        again, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        for k in ("out_width", "out_token", "out_parent", "node_status", "layer_width"):
+            assert np.array_equal(again[k], gpu[k]), k
+    ref = _oracle(forest, prm, zp, zq, rp, rq)
+    check_exempt(*compare_verify(ref, gpu, forest))
+
+
 def test_roots_only_forest_goes_straight_to_the_extra_layer():
     rng = np.random.default_rng(3)
     V, B = 2000, 3

@@ -145,6 +145,25 @@ def test_trees_with_more_than_128_query_rows(Hq, Hkv, sizes, L):
     attention_close(to_host_f32(out), ref, bf16=True)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("sizes,L,Hq,Hkv,amp", [
+    ([16, 4, 1, 2], [127, 128, 129, 1], 16, 4, 1.0),         # edges of the 128-token tiles, 64 rows
+    ([17, 4], [200, 333], 16, 4, 1.0),                       # 68 rows: the 128-row instance
+    ([9, 4], [2000, 3333], 8, 2, 12.0),                      # logits far above the first token's: references move
+    ([30, 4], [2000, 3333], 8, 2, 12.0),
+    ([6] * 30, list(range(1000, 3900, 97))[:30], 32, 8, 1.0),    # many cut units, different shares of the rows
+    ([1, 9] * 20, [300] * 40, 4, 4, 1.0),                    # equal lengths, whole units
+])
+def test_transposed_products(d, sizes, L, Hq, Hkv, amp):
+    rng = np.random.default_rng(d + len(sizes))
+    trees = [[-1] + [int(rng.integers(0, i)) for i in range(1, n)] for n in sizes]
+    forest, spec, t, poff = _custom(rng, trees, L, Hq, Hkv, d, torch.bfloat16)
+    t = {k: (v.float() * amp).to(torch.bfloat16) if k in ("q", "k_new", "k_prefix") else v for k, v in t.items()}
+    out = _gpu(forest, spec, t, poff)
+    nodes, ref = _oracle_beams(forest, spec, t, poff, list(range(len(trees))))
+    attention_close(to_host_f32(out), ref, bf16=True)
+
+
 def test_host_side_errors():
     rng = np.random.default_rng(0)
     forest, spec, t, poff = _custom(rng, [[-1, 0]], [8], 4, 4, 64, torch.bfloat16)

@@ -7,7 +7,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(BUILD_DIR, "libdsbd.so")
-SOURCES = ["dsbd_api.cu", "dsbd_verify.cu", "dsbd_attention.cu", "dsbd_attention_tc.cu", "dsbd_kv_commit.cu", "dsbd_forest.cu"]
+SOURCES = ["dsbd_api.cu", "dsbd_verify.cu", "dsbd_attention.cu", "dsbd_attention_tc.cu",
+           "dsbd_attention_tr.cu", "dsbd_kv_commit.cu", "dsbd_forest.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xptxas=-v", "-Xcompiler", "-fPIC",
               "-I", os.path.join(ROOT, "include"), "-I", CSRC] + os.environ.get("DSBD_NVCC_EXTRA", "").split()
@@ -82,7 +83,7 @@ def _build_variant(lib_path, tag, sources, define, force):
 def build_wait_test(force=False):
     """A second library for one test: the attention kernel compiled with DSBD_TEST_WAIT_TIMEOUT
     (short bounded waits, one tile never delivered).  Nothing but that test loads it."""
-    return _build_variant(WAIT_TEST_LIB, "waittest", ("dsbd_api.cu", "dsbd_attention.cu", "dsbd_attention_tc.cu"),
+    return _build_variant(WAIT_TEST_LIB, "waittest", ("dsbd_api.cu", "dsbd_attention.cu", "dsbd_attention_tc.cu", "dsbd_attention_tr.cu"),
                           "-DDSBD_TEST_WAIT_TIMEOUT", force)
 
 

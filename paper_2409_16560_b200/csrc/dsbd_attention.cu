@@ -221,11 +221,13 @@ int check(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
 
 extern "C" size_t dsbd_forest_attention_workspace(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
     if (check(f, d) != DSBD_OK) return 0;
+    if (attention_tr_supported(f, d)) return attention_tr_workspace(f, d);
     return attention_tc_supported(f, d) ? attention_tc_workspace(f, d) : 256;
 }
 
 extern "C" int dsbd_forest_attention_launches(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
     if (check(f, d) != DSBD_OK) return 0;
+    if (attention_tr_supported(f, d)) return attention_tr_launches(f, d);
     return attention_tc_supported(f, d) ? attention_tc_launches(f, d) : 1;
 }
 
@@ -245,6 +247,9 @@ extern "C" int dsbd_forest_attention(const dsbd_forest_t *f, const dsbd_attn_des
                            reinterpret_cast<uintptr_t>(v_prefix) | reinterpret_cast<uintptr_t>(out);
     if (bits & 15) return DSBD_ERR_UNSUPPORTED;
 
+    if (attention_tr_supported(f, d))
+        return launch_attention_tr(f, d, q, k_new, v_new, k_prefix, v_prefix, prefix_off, out, workspace,
+                                   workspace_bytes, status, stream);
     if (attention_tc_supported(f, d))
         return launch_attention_tc(f, d, q, k_new, v_new, k_prefix, v_prefix, prefix_off, out, workspace,
                                    workspace_bytes, status, stream);
@@ -269,7 +274,8 @@ extern "C" size_t dsbd_forest_attention_paged_workspace(const dsbd_forest_t *f, 
                                                         const dsbd_kv_pages_t *pages) {
     if (check(f, d) != DSBD_OK || !pages || pages->n_pages <= 0 || pages->n_layers < 0) return 0;
     if (!attention_tc_supported(f, d, pages->n_pages) || !attention_tc_layers_ok(f, d, pages)) return 0;
-    return attention_tc_workspace(f, d, pages->n_layers);
+    return attention_tr_supported(f, d, pages->n_pages) ? attention_tr_workspace(f, d, pages->n_layers)
+                                                        : attention_tc_workspace(f, d, pages->n_layers);
 }
 
 extern "C" int dsbd_forest_attention_paged(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const void *q,
@@ -285,12 +291,14 @@ extern "C" int dsbd_forest_attention_paged(const dsbd_forest_t *f, const dsbd_at
         return DSBD_ERR_INVALID_ARG;
     if (!attention_tc_supported(f, d, pages->n_pages)) return DSBD_ERR_UNSUPPORTED;
     if (pages->n_layers < 0 || !attention_tc_layers_ok(f, d, pages)) return DSBD_ERR_INVALID_ARG;
-    if (workspace_bytes < attention_tc_workspace(f, d, pages->n_layers) || !workspace)
+    const bool tr = attention_tr_supported(f, d, pages->n_pages);
+    if (!workspace || workspace_bytes < (tr ? attention_tr_workspace(f, d, pages->n_layers)
+                                            : attention_tc_workspace(f, d, pages->n_layers)))
         return DSBD_ERR_WORKSPACE_TOO_SMALL;
     const uintptr_t bits = reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(k_new) |
                            reinterpret_cast<uintptr_t>(v_new) | reinterpret_cast<uintptr_t>(k_pool) |
                            reinterpret_cast<uintptr_t>(v_pool) | reinterpret_cast<uintptr_t>(out);
     if (bits & 15) return DSBD_ERR_UNSUPPORTED;
-    return launch_attention_tc(f, d, q, k_new, v_new, k_pool, v_pool, prefix_off, out, workspace, workspace_bytes,
-                               status, stream, pages);
+    return (tr ? launch_attention_tr : launch_attention_tc)(f, d, q, k_new, v_new, k_pool, v_pool, prefix_off, out,
+                                                            workspace, workspace_bytes, status, stream, pages);
 }

@@ -26,4 +26,18 @@ int launch_attention_tc(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const
                         void *out, void *workspace, size_t workspace_bytes, int32_t *status, cudaStream_t stream,
                         const dsbd_kv_pages_t *pages = nullptr);
 
+// Layer count and strides of a paged call; ok: they can be served.
+struct LayerDims { int n_layers, pool_rows, new_rows; int64_t q_stride; bool ok; };
+LayerDims layer_dims(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const dsbd_kv_pages_t *pages);
+
+// The same for the kernel with transposed products (at most 64 query rows per tree and KV head, d = 64 or 128),
+// which is taken when it covers the problem.
+bool attention_tr_supported(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, int64_t n_pages = 0);
+size_t attention_tr_workspace(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, int n_layers = 1);
+int attention_tr_launches(const dsbd_forest_t *f, const dsbd_attn_desc_t *d);
+int launch_attention_tr(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const void *q, const void *k_new,
+                        const void *v_new, const void *k_prefix, const void *v_prefix, const int64_t *prefix_off,
+                        void *out, void *workspace, size_t workspace_bytes, int32_t *status, cudaStream_t stream,
+                        const dsbd_kv_pages_t *pages = nullptr);
+
 }  // namespace dsbd

@@ -1,83 +1,54 @@
-// Forest attention on the 5th-generation tensor cores (tcgen05 + TMEM + TMA), bf16, d = 64 or 128.
+// Forest attention on the 5th-generation tensor cores (tcgen05 + TMEM + TMA), bf16, d = 128: query rows on the
+// M side, for trees of more than 64 query rows per KV head (smaller ones: dsbd_attention_tr.cu).
 //
-// Work unit = (beam, KV head, row block): the query rows of the beam's draft tree that map to this KV
-// head (row = node * group + head; blocks of at most NMAX = 64 or 128 rows) against the beam's KV
-// prefix and then the tree's own keys and values under the ancestor-or-self mask.
+// Work unit = (beam, KV head): all query rows of the beam's draft tree that map to this KV head
+// (row = node * group + head, at most 128) against the beam's KV prefix, streamed once in
+// 64-token tiles, followed by one tile holding the tree's own keys/values under the
+// ancestor-or-self mask.
 //
-// A draft tree has few query rows (36 for nine nodes and four heads per KV head), so the products are
-// taken transposed: the TOKENS and the head dimension fill the 128 rows of an MMA and the query rows
-// are its N columns, as many as there are (a multiple of 16):
-//   S^T = K Q^T    (M = 128 tokens, N = rows, K = d)         both operands K-major in shared memory
-//   O^T += V^T P^T (M = d, N = rows, K = 128 tokens)         both operands MN-major in shared memory
-//
-// One CTA per SM, groups of four warps:
-//   softmax   NMAX / 32 groups, each with a share of the rows (at most 32 columns of S^T).  A thread owns
-//             one token (its TMEM lane) and walks its group's rows, so a tile's exponentials are spread over
-//             all 128 lanes however few rows there are.
-//   output    O^T / row sum -> global, or the partial result of a cut unit.  The accumulators are double
-//             buffered over the units, so the softmax goes straight on to the next unit.
-//   then one warp each: TMA producer (K and V tiles of 128 tokens, boxes of 64 tokens x 64 columns with
-//             128-byte swizzle, through two rings of shared-memory slots, and the unit's query rows), the
-//             issuer of S^T (as many tiles ahead as there are S^T buffers) and the issuer of O^T.
-// The last three run converged and only predicate the copy / MMA instructions on one lane: issued from
-// a branch of a single thread an MMA takes 95 cycles (the operands go to uniform registers lane by lane),
-// issued like this 41 to 50 at N = 16 to 64 (M = 128, K = 16), which is the operand traffic of A.  One
-// warp for both products took 2050 cycles a tile at d = 128, about as long as the tile's bytes take.
-//
-// A row's reference is its logit of the unit's first token, moved only when some logit exceeds it
-// by more than 2^40: the weights then stay inside the exponent range of bf16 and fp32, whose relative
-// precision does not depend on the scale.
-//
-// Work split: the tiles of a layer's units form one sequence (beam, KV head, row block), cut into equal
-// runs, one per CTA; a unit that straddles a cut leaves partial results that k_attn_combine merges.
-// Where whole units fill the CTAs about as evenly nothing is cut (make_plan).  Every CTA finds its own
-// start with one scan over the beams; there is no plan kernel.
-//
-// Every mbarrier wait is bounded; on a time-out the kernel records DSBD_DEV_TIMEOUT, lets its copies
-// and products land, frees its TMEM and returns.
-#include <cuda.h>
-#include <cuda_bf16.h>
+// CTA = 6 warps, two CTAs per SM:
+//   warps 0-3  softmax: warp w owns TMEM lanes 32w..32w+31 = query rows 32w..32w+31, one row per
+//              thread, so row max / row sum are thread-local.  They write O at a unit's end.
+//   warp 4     TMA producer: K and V tiles (2 x 64x64 bf16 boxes each, 128-byte swizzle) into a
+//              ring of shared-memory stages, completion on mbarriers; and the unit's query rows
+//              (two boxes of 64 columns x group heads x nodes of a 3-D map over q), issued as soon
+//              as the previous unit's last Q K^T product has completed, so that the copy runs
+//              behind that unit's last softmax, P V product and output write.
+//   warp 5     MMA issuer (one lane): S = Q K^T (M128 N64 K16 x 8, both operands K-major in
+//              shared memory) into one of two S buffers in TMEM, one tile ahead, so that it runs
+//              while the softmax warps work on the previous tile; after they have written P
+//              (bf16, over the S buffer they just read), O += P V (A from TMEM, B = the V tile
+//              as an MN-major shared-memory operand).
+// O stays in TMEM for the whole unit; its rows are rescaled only when a row maximum grows by
+// more than 2^8 (the rescale is a TMEM load/scale/store by the row's own thread).
+// Every mbarrier wait is bounded; on a time-out the kernel records DSBD_DEV_TIMEOUT, lets its
+// copies land, frees its TMEM and returns.
 #include <math.h>
 
 #include <algorithm>
 
-#include "dsbd_attention.cuh"
+#include "dsbd_tc.cuh"
 
 using namespace dsbd;
 
 namespace {
 
-constexpr int kBN = 64;                 // tokens per copied box (and per cache page)
-constexpr int kTile = 128;              // tokens per tile = the M rows of the S^T product
-constexpr int kMaxTree = DSBD_MAX_TREE_NODES_TC;
-constexpr uint32_t kHalfStride = kTile * 128;        // bytes of one 64-column half of a tile (or of 64 rows of P)
-constexpr float kMoveRef = 40.f;        // log2 of the factor by which a logit may exceed its row's reference
-
-// Shape of one kernel instance.  SPLIT: the probabilities enter the second product as the sum of two
-// bf16 terms (2^-17 relative); used at d = 64, where they were kept in fp32 by the kernel this one replaced.
-template <int D, int NMAX, bool SPLIT>
-struct Shape {
-    static constexpr int kGroups = NMAX / 32;                 // softmax groups of 128 threads
-    static constexpr int kThreads = kGroups * 128 + 256;
-    static constexpr int kHalves = D / 64;                    // 64-column halves of a row of Q, K or V
-    static constexpr uint32_t kSlot = kTile * D * 2;          // one K or V tile
-    static constexpr uint32_t kPTerm = NMAX / 64 * kHalfStride;                  // [64-row block][token][128 B]
-    static constexpr uint32_t kPBuf = (SPLIT ? 2 : 1) * kPTerm;
-    static constexpr int kPBufs = NMAX == 64 ? 2 : 1;
-    // query rows of one unit, or of two when they fit (a unit's copy then runs a whole unit ahead; with one
-    // buffer its latency, 2800 cycles while HBM is saturated, shows at every unit's start)
-    static constexpr uint32_t kQBytes = D == 64 ? (NMAX == 64 ? 16 : 21) * 1024 : (NMAX == 64 ? 21 : 52) * 1024;
-    // K and V have rings of their own: each is consumed in order by one issuer, so that a wait for a slot's
-    // next filling can never be satisfied by the one before it
-    static constexpr int kKSlots = D == 64 ? 4 : 2, kVSlots = D == 64 ? 4 : (NMAX == 64 ? 3 : 2);
-    // order: K ring, V ring, P, Q (at d = 64 the upper 64 rows of the V^T operand alias the 16 KB after a slot,
-    // which therefore must exist; rows of an MMA are independent and those rows are never read back)
-    static constexpr uint32_t kOffV = kKSlots * kSlot, kOffP = kOffV + kVSlots * kSlot, kOffQ = kOffP + kPBufs * kPBuf;
-    static constexpr uint32_t kSmem = kOffQ + kQBytes;
-    // TMEM: 256 columns of S^T buffers (four of 64 rows or two of 128), then O^T of two units
-    static constexpr uint32_t kTmemCols = 512, kColO = 256, kSBufs = 256 / NMAX;
-};
-
+constexpr int kD = 128;                 // head dim
+constexpr int kMaxStages = 3;
+constexpr int kRows = 128;              // UMMA M
+constexpr int kThreadsTc = 192;
+constexpr uint32_t kTileBytes = kBN * kD * 2;         // 16 KB per K or V tile (two 8 KB boxes)
+constexpr uint32_t kStageBytes = 2 * kTileBytes;      // K then V
+// Shared memory of one CTA: Q (QROWS rows x 256 B as two swizzled halves), the K/V stage ring,
+// then the mbarriers.  With at most 64 query rows only 64 rows of Q are stored: the MMA still
+// runs with M = 128, and the A-operand rows 64..127 then alias the bytes that follow Q.  Rows of
+// an MMA are independent and rows >= M are never read back, so whatever those bytes hold is
+// harmless; the 16 KB saved buy a third stage at two CTAs per SM.
+constexpr uint32_t smem_bytes(int qrows, int stages) { return qrows * kD * 2 + stages * kStageBytes; }
+constexpr uint32_t kTmemCols = 256;
+// TMEM columns: two S buffers of 64 fp32 columns (P, bf16 pairs, overwrites the first 32 columns
+// of its S buffer once S has been read), then O (128 fp32 columns).
+constexpr uint32_t kColS = 0, kColO = 128;
 #ifdef DSBD_TEST_WAIT_TIMEOUT
 // Test build only (a second library that no product path loads): waits give up after about a
 // millisecond and the producer leaves out one tile, so that a wait runs out without anything
@@ -88,82 +59,56 @@ constexpr long long kWaitCycles = 2000000ll;
 constexpr long long kWaitCycles = 2000000000ll;   // about a second
 #endif
 
-// What a run left for the merge.  tail: its last unit starts here and goes on in the next run; head_ends:
-// the part of a unit that the run began with is the last one of that unit.
-struct CutRec { int tail, head_ends, b, g, rb, pad0, pad1, pad2; };
+// One work item: the query rows of unit (b, g) against the prefix tokens [t0, t1) of its beam,
+// plus the tree tile when `last`.  A unit split into several items leaves partial results
+// (reference maximum, row sum, unnormalised O) that a second kernel merges.
+// Trees with more than 128 query rows (nodes x query heads per KV head) are cut into row blocks
+// of 128 rows; every row block is an item of its own that streams the same keys and values.
+struct AttnItem { int b, g, t0, t1, last, nparts, slot, rb; };
 
 struct TcArgs {
-    int B, N, Hq, Hkv, group;
-    int block_rows;                   // query rows per row block: whole nodes, at most NMAX
+    int B, N, Hq, Hkv, group, n_units;
+    int max_rows;                     // max over trees of nodes * group
+    int block_rows;                   // query rows per row block: whole nodes, at most the kernel's Q tile (64 or 128)
     int nodes_per_block;              // block_rows / group
-    int q_nodes, q_rows, q_bufs;      // nodes of a query box, rows (a multiple of 8) and number of the Q buffers
-    int n_layers;                     // >= 1: transformer layers in one launch (paged caches)
-    int runs;                         // runs per layer; CTA c takes run c % runs of the layers c / runs + k * layer_step
-    int layer_step;
-    int uni_nt;                       // > 0: every unit has one row block and this many tiles
-    int whole;                        // runs are whole units: nothing is cut
-    int reread;                       // some tree has several row blocks: its prefix is read more than once
-    float scale_log2;                 // scale * log2(e)
+    int row_blocks;                   // ceil(max_rows / block_rows)
+    const AttnItem *items;            // nullptr: one item per unit, in unit order
+    const int *n_items;               // device count of items (with items)
+    float *partial;                   // [slot][max_rows][130]: m_ref, l, O[128]
+    float scale_log2;
     const int32_t *beam_node_off, *parent;
     const int64_t *prefix_off;
     const int32_t *page_table;        // paged caches: page ids of beam b at page_off[b] ..; nullptr: packed
     const int64_t *page_off;
+    const __nv_bfloat16 *q;
     __nv_bfloat16 *out;
     int32_t *status;
-    // layer l uses the same page tables and forest; its pools, new keys/values, queries and outputs lie
-    // l strides further
+    // several transformer layers in one launch (paged caches): layer l uses the same plan, page
+    // tables and forest; its pools, new keys/values, queries and outputs lie l strides further
+    int n_layers;                     // >= 1
     int pool_layer_rows;              // rows of the pool map between consecutive layers
     int new_layer_rows;               // rows of the k_new / v_new maps between consecutive layers
     int64_t q_layer_stride;           // elements between consecutive layers' q (and out)
     int q_layer_nodes;                // the same in nodes (rows of the query map between consecutive layers)
-    CutRec *recs;                     // [n_layers * runs]
-    float *partial;                   // [2 * n_layers * runs][NMAX][D + 2]: reference, row sum, O; run i's first
-                                      // unit in slot 2 i, its last one in slot 2 i + 1
+    int slots_per_layer;              // partial-result slots of one layer
+    // Tail split of a batch of equal-length units in unit order (no plan kernel): the units from
+    // tail_first on -- those that would leave most CTAs idle in a last, partly filled round --
+    // are cut into tail_k parts each, so that the last round has work for (nearly) every CTA.
+    int tail_first, tail_k;           // tail_k == 0: off
+    // Ragged batch of whole units without a plan kernel: every CTA ranks the units by tile count
+    // itself (longest first, ties by unit number, rounds alternating in direction) and keeps the
+    // entries of its own column.  rank_units = number of units, 0 = off.
+    int rank_units;
 };
 
-constexpr int kMaxSlots = 4;
+constexpr int kMaxRanked = 8;             // items of one CTA when it ranks the units itself
 struct Barriers {
-    unsigned long long k_full[kMaxSlots], k_empty[kMaxSlots], v_full[kMaxSlots], v_empty[kMaxSlots];
-    unsigned long long s_full[4], p_full[4], pv_done[2], q_full[2], q_empty[2];
-    unsigned long long sum_full[2], o_full[2], o_empty[2];     // by unit parity
-    unsigned long long drain[2];
+    unsigned long long kv_full[kMaxStages], kv_empty[kMaxStages], s_full[2], p_full[2], pv_done, q_full, q_empty, o_full;
     uint32_t tmem_base;
     int abort;
-    int scan[32];                          // warp sums of the start-up scan
-    int start[3];                          // beam, unit inside the beam, tile inside the unit
-    int run;                               // tiles of the run
-};
-// (The groups are not in step: what a group changes on its own is its own, since the share of the rows that a
-// column belongs to differs from unit to unit.)
-struct SoftmaxShared {
-    float negref[4][32];                   // [group] minus the row references (log2 units)
-    float ref[2][128];                     // [unit parity] the references a unit ended with
-    float red[2][4][128];                  // [unit parity] row sums per warp quarter
-    float colmax[4][4][32];                // [group] column maxima per warp quarter
-    float move[4][32];                     // [group] rescale factors when references move
-    float fac[128];                        // 1 / row sum
-    int rowoff[128];                       // output offset of a row inside its block
-    int16_t par[4][kMaxTree];              // [group] the tree's parents, local
-    uint32_t see[4][kMaxTree];             // [group] tree token j: the group's rows that see it
+    int my_units[kMaxRanked];             // rank mode: the unit of this CTA's k-th item, -1 for none
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(void *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive(void *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(void *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
 // Bounded wait: false if it gave up (time-out here, or another role already aborted).
 __device__ __forceinline__ bool mbar_wait(void *bar, uint32_t parity, Barriers *sb, int32_t *status) {
     if (mbar_try(bar, parity)) return true;
@@ -178,947 +123,703 @@ __device__ __forceinline__ bool mbar_wait(void *bar, uint32_t parity, Barriers *
     return false;
 }
 
-// Copies, products and commits are issued by whole warps with one lane's predicate (`on`).
-__device__ __forceinline__ void mbar_expect_tx_if(bool on, void *bar, uint32_t bytes) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t"
-        "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}"
-        ::"r"(smem_u32(bar)), "r"(bytes), "r"((uint32_t)on) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(bool on, uint32_t dst, const CUtensorMap *map, int x, int y, void *bar) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t"
-        "@p cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)), "r"((uint32_t)on) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d_hint(bool on, uint32_t dst, const CUtensorMap *map, int x, int y, void *bar,
-                                                 uint64_t pol) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %6, 0;\n\t"
-        "@p cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;\n\t}"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(pol), "r"((uint32_t)on) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(bool on, uint32_t dst, const CUtensorMap *map, int x, int y, int z, void *bar) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %6, 0;\n\t"
-        "@p cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n\t}"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "r"((uint32_t)on) : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(bool on, void *bar) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-        "@p tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
-        ::"r"(smem_u32(bar)), "r"((uint32_t)on) : "memory");
-}
-__device__ __forceinline__ void mma_ss(bool on, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.u32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc), "r"((uint32_t)on) : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *v) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *v) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-        : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t *v) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-        ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-        : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptors (128-byte swizzle, 8-row groups 1024 bytes apart).
-__device__ __forceinline__ uint64_t desc_k_major(uint32_t saddr) {
-    // leading offset unused for swizzled K-major (1), stride offset 1024 B, version 1, SWIZZLE_128B
-    return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ uint64_t desc_mn_major(uint32_t saddr, uint32_t lbo_bytes) {
-    // leading offset = distance between 64-element groups along N, stride offset = 8 k-rows
-    return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) |
-           ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-// M rows, N columns, fp32 accumulators, bf16 operands; MN-major operands are transposed in shared memory.
-__host__ __device__ constexpr uint32_t instr_desc(int M, int N, int a_mn_major, int b_mn_major) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn_major << 15) | ((uint32_t)b_mn_major << 16) |
-           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ float ex2_ftz(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t *>(&v);
-}
-__device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
-
-// Barrier of the 128 threads of group g (softmax groups, then the output warps; id 0 is __syncthreads),
-// plain and with an OR.  The warps arrive, and leave, converged: the TMEM accesses between the barriers
-// need whole warps.
-__device__ __forceinline__ void group_sync(int g) {
-    __syncwarp();
-    asm volatile("barrier.cta.sync.aligned %0, 128;" ::"r"(g + 1) : "memory");
-}
-__device__ __forceinline__ bool group_any(int g, bool v) {
-    uint32_t r;
-    __syncwarp();
-    asm volatile(
-        "{\n\t.reg .pred a, b;\n\tsetp.ne.u32 a, %1, 0;\n\t"
-        "barrier.cta.red.or.pred.aligned b, %2, 128, a;\n\tselp.u32 %0, 1, 0, b;\n\t}"
-        : "=r"(r) : "r"((uint32_t)v), "r"(g + 1) : "memory");
-    return r != 0;
-}
-// A bounded wait by a converged warp: the same answer on every lane.
+// The same wait by a converged warp: the same answer on every lane.
 __device__ __forceinline__ bool warp_wait(void *bar, uint32_t parity, Barriers *sb, int32_t *status) {
     return __all_sync(kFull, mbar_wait(bar, parity, sb, status));
 }
-// After a time-out: waits (again with a limit) until the products this warp has issued are done, so that TMEM
-// and shared memory can be given back.
-__device__ __forceinline__ void drain(bool on, void *bar) {
-    tc_commit(on, bar);
-    const long long t0 = clock64();
-    while (!__all_sync(kFull, mbar_try(bar, 0)))
-        if (__any_sync(kFull, clock64() - t0 > kWaitCycles)) break;
+
+__device__ __forceinline__ int item_count(const TcArgs &a) {
+    if (a.items) return *a.n_items;
+    if (a.rank_units) return (a.rank_units + (int)gridDim.x - 1) / (int)gridDim.x * (int)gridDim.x;
+    if (a.tail_k) return a.tail_first + (a.n_units - a.tail_first) * a.tail_k;
+    return a.n_units * a.row_blocks;
+}
+// The item, with b = -1 when there is nothing to do: a padding entry of the plan, or a row block
+// beyond the rows of this tree.  All three roles of the CTA skip such items alike.
+__device__ __forceinline__ AttnItem get_item(const TcArgs &a, int it, const Barriers &sb) {
+    AttnItem x;
+    if (a.items) {
+        x = a.items[it];
+    } else if (a.rank_units) {
+        // (every item index a CTA asks for is in its own column: it % grid == blockIdx.x)
+        const int u = sb.my_units[it / (int)gridDim.x];
+        x.rb = 0; x.b = -1; x.g = 0; x.t0 = 0; x.t1 = 0; x.last = 1; x.nparts = 1; x.slot = 0;
+        if (u >= 0) {
+            x.b = u / a.Hkv; x.g = u - x.b * a.Hkv;
+            x.t1 = (int)(a.prefix_off[x.b + 1] - a.prefix_off[x.b]);
+        }
+    } else if (a.tail_k && it >= a.tail_first) {
+        // part p of tail unit u: equal parts of whole tiles, the tree tile with the last part
+        const int r = it - a.tail_first, u = a.tail_first + r / a.tail_k, p = r - (r / a.tail_k) * a.tail_k;
+        x.rb = 0;
+        x.b = u / a.Hkv; x.g = u - x.b * a.Hkv;
+        const int L = (int)(a.prefix_off[x.b + 1] - a.prefix_off[x.b]);
+        const int plen = ((L + a.tail_k - 1) / a.tail_k + kBN - 1) / kBN * kBN;
+        x.t0 = min(p * plen, L); x.t1 = min(x.t0 + plen, L);
+        x.last = (p == a.tail_k - 1); x.nparts = a.tail_k; x.slot = r;
+    } else {
+        const int u = it / a.row_blocks;
+        x.rb = it - u * a.row_blocks;
+        x.b = u / a.Hkv; x.g = u - x.b * a.Hkv;
+        x.t0 = 0; x.t1 = (int)(a.prefix_off[x.b + 1] - a.prefix_off[x.b]);
+        x.last = 1; x.nparts = 1; x.slot = 0;
+    }
+    if (x.b >= 0 && x.rb > 0 &&
+        x.rb * a.block_rows >= (a.beam_node_off[x.b + 1] - a.beam_node_off[x.b]) * a.group)
+        x.b = -1;
+    return x;
 }
 
-// Combines 8 columns over the 32 lanes with 9 shuffles; lane i ends up with column i & 7 in v[0].
-template <class F>
-__device__ __forceinline__ void fold8(float *v, int lane, F op) {
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < o; ++i) {
-            const float send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
-            v[i] = op(keep, __shfl_xor_sync(kFull, send, o));
-        }
-    }
-    v[0] = op(v[0], __shfl_xor_sync(kFull, v[0], 8));
-    v[0] = op(v[0], __shfl_xor_sync(kFull, v[0], 16));
+// Tiles of 64 tokens that hold the tree's own keys and values (trees of up to 128 nodes).
+__device__ __forceinline__ int tree_tiles(const TcArgs &a, int b) {
+    return (a.beam_node_off[b + 1] - a.beam_node_off[b] + kBN - 1) / kBN;
 }
 
-// The part of one unit that a run holds: tiles [t0, t1) of the unit's nt.
-struct Seg { int layer, b, g, rb, t0, t1, nt, nhp, nh, L, n_lo, n_tree; };
-
-// Facts of a beam: prefix length, tree, boxes of 64 tokens (the prefix's, then the tree's), tiles of a
-// unit (two boxes each), row blocks.
-struct BeamFacts { int L, n_lo, n_tree, nhp, nh, nt, nrb; };
-__device__ __forceinline__ BeamFacts beam_facts(const TcArgs &a, int b) {
-    BeamFacts f;
-    f.L = (int)(a.prefix_off[b + 1] - a.prefix_off[b]);
-    f.n_lo = a.beam_node_off[b];
-    f.n_tree = min(max(a.beam_node_off[b + 1] - f.n_lo, 0), kMaxTree);
-    f.nhp = (f.L + kBN - 1) / kBN;
-    f.nh = f.nhp + (f.n_tree + kBN - 1) / kBN;
-    f.nt = (f.nh + 1) / 2;
-    f.nrb = max(1, (f.n_tree * a.group + a.block_rows - 1) / a.block_rows);
-    return f;
-}
-
-// Walks the runs of this CTA (one per layer that it serves); producer, MMA issuers, softmax groups and output
-// warps each keep one and see the same segments.
-struct Cursor {
-    int left, layer, b, k, toff, loaded;
-    BeamFacts f;
-    __device__ __forceinline__ Cursor(const TcArgs &a, const Barriers &sb) {
-        layer = (int)blockIdx.x / a.runs;
-        loaded = -1;
-        rewind(sb);
-    }
-    __device__ __forceinline__ void rewind(const Barriers &sb) {
-        left = sb.run; b = sb.start[0]; k = sb.start[1]; toff = sb.start[2];
-    }
-    __device__ __forceinline__ bool next(const TcArgs &a, const Barriers &sb, Seg &s) {
-        while (layer < a.n_layers) {
-            if (left <= 0 || b >= a.B) {
-                layer += a.layer_step;
-                rewind(sb);
-                if (left <= 0) return false;
-                continue;
-            }
-            if (loaded != b) { f = beam_facts(a, b); loaded = b; }
-            s.layer = layer; s.b = b; s.g = f.nrb == 1 ? k : k / f.nrb; s.rb = k - s.g * f.nrb;
-            s.t0 = toff; s.nt = f.nt; s.t1 = min(f.nt, toff + left);
-            s.nhp = f.nhp; s.nh = f.nh; s.L = f.L; s.n_lo = f.n_lo; s.n_tree = f.n_tree;
-            left -= s.t1 - s.t0;
-            toff = 0;
-            if (++k == f.nrb * a.Hkv) { k = 0; ++b; }
-            if (s.t1 > s.t0) return true;
-        }
-        return false;
-    }
-};
-
-// Finds the run of this CTA: first unit and tile, number of tiles (all threads).
-template <int kThreads>
-__device__ void find_run(const TcArgs &a, Barriers &sb) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int r = (int)blockIdx.x % a.runs, G = a.runs;
-    const int units = a.B * a.Hkv;                            // (where row blocks are one per tree)
-    if (a.uni_nt > 0 || a.whole) {
-        if (tid == 0) {
-            const int nt = a.uni_nt;
-            int lo, hi, unit;
-            if (a.whole) {
-                unit = (int)((int64_t)units * r / G);
-                lo = unit * nt; hi = (int)((int64_t)units * (r + 1) / G) * nt;
-                if (nt == 0) { lo = 0; hi = beam_facts(a, unit / a.Hkv).nt; }      // ragged: one unit per run
-            } else {
-                lo = (int)((int64_t)units * nt * r / G); hi = (int)((int64_t)units * nt * (r + 1) / G);
-                unit = lo / nt;
-            }
-            sb.start[0] = unit / a.Hkv; sb.start[1] = unit % a.Hkv; sb.start[2] = a.whole ? 0 : lo - unit * nt;
-            sb.run = hi - lo;
-        }
-        __syncthreads();
-        return;
-    }
-    // tiles before every thread's share of the beams
-    const int per = (a.B + kThreads - 1) / kThreads;
-    const int b0 = min(tid * per, a.B), b1 = min(b0 + per, a.B);
-    int sum = 0;
-    for (int b = b0; b < b1; ++b) {
-        const BeamFacts f = beam_facts(a, b);
-        sum += f.nt * f.nrb * a.Hkv;
-    }
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) sb.scan[warp] = incl;
-    if (tid == 0) { sb.start[0] = 0; sb.start[1] = 0; sb.start[2] = 0; sb.run = 0; }
-    __syncthreads();
-    int before = incl - sum, total = 0;
-    for (int w = 0; w < kThreads / 32; ++w) { if (w < warp) before += sb.scan[w]; total += sb.scan[w]; }
-    const int lo = (int)((int64_t)total * r / G), hi = (int)((int64_t)total * (r + 1) / G);
-    if (lo < hi && lo >= before && lo < before + sum) {
-        int at = before;
-        for (int b = b0; b < b1; ++b) {
-            const BeamFacts f = beam_facts(a, b);
-            const int w = f.nt * f.nrb * a.Hkv;
-            if (lo < at + w) {
-                sb.start[0] = b; sb.start[1] = (lo - at) / f.nt; sb.start[2] = (lo - at) % f.nt;
-                sb.run = hi - lo;
-                break;
-            }
-            at += w;
-        }
-    }
-    __syncthreads();
-}
-
-template <int D, int NMAX, bool SPLIT>
-__global__ void __launch_bounds__(Shape<D, NMAX, SPLIT>::kThreads, 1)
+template <int QROWS, int kStages>
+__global__ void __launch_bounds__(kThreadsTc, 2)
 k_forest_attn_tc(const __grid_constant__ CUtensorMap map_kp, const __grid_constant__ CUtensorMap map_vp,
                  const __grid_constant__ CUtensorMap map_kn, const __grid_constant__ CUtensorMap map_vn,
                  const __grid_constant__ CUtensorMap map_q, TcArgs a) {
-    using S = Shape<D, NMAX, SPLIT>;
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char *p_s = smem + S::kOffP, *q_s = smem + S::kOffQ;
+    constexpr uint32_t kQBytes = QROWS * kD * 2;
+    unsigned char *q_s = smem;                               // [2 halves][QROWS rows][128 B], swizzled
+    unsigned char *stage_s = smem + kQBytes;                 // [stages][K 16 KB | V 16 KB]
     __shared__ Barriers sb;
-    __shared__ __align__(16) SoftmaxShared sx;
     const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    constexpr int kGroups = S::kGroups, kWarpOut = kGroups * 4, kWarpTma = kWarpOut + 4, kWarpS = kWarpTma + 1,
-                  kWarpO = kWarpTma + 2;
     if ((smem_u32(smem) & 1023u) != 0u) {                    // the swizzled operands need 1024-byte alignment
         if (threadIdx.x == 0) report(a.status, DSBD_DEV_BAD_FOREST);
         return;
     }
+
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kMaxSlots; ++s) {
-            mbar_init(&sb.k_full[s], 1); mbar_init(&sb.k_empty[s], 1);
-            mbar_init(&sb.v_full[s], 1); mbar_init(&sb.v_empty[s], 1);
-        }
-        for (int b = 0; b < 4; ++b) { mbar_init(&sb.s_full[b], 1); mbar_init(&sb.p_full[b], kGroups * 4); }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&sb.pv_done[b], 1); mbar_init(&sb.q_full[b], 1); mbar_init(&sb.q_empty[b], 1);
-            mbar_init(&sb.sum_full[b], kGroups * 4); mbar_init(&sb.o_full[b], 1); mbar_init(&sb.o_empty[b], 4);
-            mbar_init(&sb.drain[b], 1);
-        }
+        for (int s = 0; s < kStages; ++s) { mbar_init(&sb.kv_full[s], 1); mbar_init(&sb.kv_empty[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&sb.s_full[b], 1); mbar_init(&sb.p_full[b], 4); }
+        mbar_init(&sb.pv_done, 1);
+        mbar_init(&sb.q_full, 1);
+        mbar_init(&sb.q_empty, 1);
+        mbar_init(&sb.o_full, 1);
         sb.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == kWarpS) {
+    if (warp == 5) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sb.tmem_base)),
-                     "r"(S::kTmemCols) : "memory");
+                     "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // query rows past a block's last one are never copied in: keep them finite
-    for (uint32_t i = threadIdx.x * 16; i < S::kQBytes; i += S::kThreads * 16)
-        *reinterpret_cast<uint4 *>(q_s + i) = make_uint4(0u, 0u, 0u, 0u);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (threadIdx.x < 128) {
-        const int node = (int)threadIdx.x / a.group;
-        sx.rowoff[threadIdx.x] = (node * a.Hq + (int)threadIdx.x - node * a.group) * D;
-    }
-    // launched with programmatic stream serialization: what is above overlaps the kernel before
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     tc_fence_before();
-    find_run<S::kThreads>(a, sb);                            // (has the block barriers)
+    __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = __shfl_sync(kFull, *reinterpret_cast<volatile uint32_t *>(&sb.tmem_base), 0);
-    Cursor cur(a, sb);
-    Seg sg;
-    // NMAX = 128: 4 x 96 + 2 x 48 = the 6 x 80 registers per lane of the launch
-    if (kGroups == 4 && warp >= kWarpOut) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&sb.tmem_base);
 
-    if (warp == kWarpTma) {
-        // ------------------------------------------------------------ TMA producer
-        const bool on = lane == 0;
-        uint32_t n_k = 0, n_v = 0, unit = 0;                 // K and V tiles so far
-        bool ok = true;
-        // a prefix that is read once: its lines are the first to leave L2 again, so that the queries, the
-        // tree's keys and values and the metadata the units keep coming back to stay there (the row blocks
-        // of a big tree read the same prefix: ordinary policy)
-        uint64_t pol;
-        if (!a.reread) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-        else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
-        const uint32_t ring = smem_u32(smem);
-        while (ok && cur.next(a, sb, sg)) {
-            const int row0 = a.page_table ? 0 : (int)(a.prefix_off[sg.b] * a.Hkv + (int64_t)sg.g * sg.L);
-            const int32_t *pages = a.page_table ? a.page_table + a.page_off[sg.b] : nullptr;
-            int pg[2] = {0, 0};                              // pages of the next tile's two boxes
-            auto fetch_pages = [&](int h) {
-                if (!pages) return;
-                if (h < sg.nhp) pg[0] = pages[h];
-                if (h + 1 < sg.nhp) pg[1] = pages[h + 1];
-            };
-            fetch_pages(2 * sg.t0);
-            auto load_tile = [&](int j, int kv) -> bool {    // K or V of tile j into the next slot
-                const uint32_t slots = kv ? S::kVSlots : S::kKSlots, n = kv ? n_v : n_k, s = n % slots;
-                void *full = kv ? &sb.v_full[s] : &sb.k_full[s], *empty = kv ? &sb.v_empty[s] : &sb.k_empty[s];
-                if (!warp_wait(empty, ((n / slots) & 1) ^ 1, &sb, a.status)) return false;
-                if (kv) ++n_v; else ++n_k;
-                const int boxes = min(2, sg.nh - 2 * j);
-                const uint32_t dst = ring + (kv ? S::kOffV : 0) + s * S::kSlot;
-                mbar_expect_tx_if(on, full, (uint32_t)boxes * kBN * D * 2);
-#ifdef DSBD_TEST_WAIT_TIMEOUT
-                if (n == 1 && !kv && blockIdx.x == 0) return true;   // the bytes this barrier expects never come
-#endif
+    if (a.rank_units) {
+        // A counting sort by tile count in the (still idle) stage ring: position of a unit = units
+        // with more tiles + earlier units with as many.  Columns are mirrored in odd rounds so
+        // that the CTA with the longest item of one round gets the shortest of the next.  Every
+        // CTA computes the same order and keeps the entries of its own column.
+        int *nt_s = reinterpret_cast<int *>(stage_s);            // [n] tile count of each unit
+        int *start_s = nt_s + 2048;                              // [1024] first position of a tile count
+        const int n = a.rank_units, grid = (int)gridDim.x;
+        for (int i = threadIdx.x; i < 1024; i += kThreadsTc) start_s[i] = 0;
+        if (threadIdx.x < kMaxRanked) sb.my_units[threadIdx.x] = -1;
+        __syncthreads();
+        for (int u = threadIdx.x; u < n; u += kThreadsTc) {
+            const int b = u / a.Hkv;
+            const int nt = min((int)((a.prefix_off[b + 1] - a.prefix_off[b] + kBN - 1) / kBN), 1023);
+            nt_s[u] = nt;
+            atomicAdd(&start_s[nt], 1);                          // counts first
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // counts -> first positions, largest tile count first (lane l owns counts 32l .. 32l+31)
+            int cnt[32], mine = 0;
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    if (i >= boxes) break;
-                    const int h = 2 * j + i;
+            for (int i = 0; i < 32; ++i) { cnt[i] = start_s[1023 - (lane * 32 + i)]; mine += cnt[i]; }
+            int before = mine;
 #pragma unroll
-                    for (int hc = 0; hc < S::kHalves; ++hc) {
-                        const uint32_t to = dst + hc * kHalfStride + i * (kHalfStride / 2);
-                        if (h >= sg.nhp)
-                            tma_load_2d(on, to, kv ? &map_vn : &map_kn, sg.g * D + hc * 64,
-                                        sg.n_lo + (h - sg.nhp) * kBN + sg.layer * a.new_layer_rows, full);
-                        else
-                            tma_load_2d_hint(on, to, kv ? &map_vp : &map_kp, hc * 64,
-                                             pages ? (pg[i] * a.Hkv + sg.g) * kBN + sg.layer * a.pool_layer_rows
-                                                   : row0 + h * kBN, full, pol);
-                    }
-                }
-                return true;
-            };
-            // The first K tile does not have to wait for the query rows.  A Q buffer is free once the last S^T
-            // product of the unit that had it has completed.
-            ok = load_tile(sg.t0, 0);
-            const uint32_t qb = unit % a.q_bufs, q_use = unit / a.q_bufs;
-            if (ok) ok = warp_wait(&sb.q_empty[qb], (q_use & 1) ^ 1, &sb, a.status);
-            if (!ok) break;
-            {
-                const int z = sg.n_lo + sg.rb * a.nodes_per_block + sg.layer * a.q_layer_nodes;
-                mbar_expect_tx_if(on, &sb.q_full[qb], (uint32_t)(a.q_nodes * a.group) * D * 2);
-#pragma unroll
-                for (int hc = 0; hc < S::kHalves; ++hc)
-                    tma_load_3d(on, smem_u32(q_s) + (qb * S::kHalves + hc) * a.q_rows * 128, &map_q, hc * 64,
-                                sg.g * a.group, z, &sb.q_full[qb]);
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(kFull, before, o);
+                if (lane >= o) before += t;
             }
-            ++unit;
-            ok = load_tile(sg.t0, 1);
-            for (int j = sg.t0 + 1; j < sg.t1 && ok; ++j) {
-                fetch_pages(2 * j);
-                ok = load_tile(j, 0);
-                if (ok) ok = load_tile(j, 1);
+            before -= mine;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) { start_s[1023 - (lane * 32 + i)] = before; before += cnt[i]; }
+            __syncwarp();
+            // units in order, 32 at a time: equal counts inside a group keep their unit order
+            for (int base = 0; base < n; base += 32) {
+                const int u = base + lane;
+                const int nt = u < n ? nt_s[u] : -1 - lane;                  // idle lanes match nobody
+                const unsigned same = __match_any_sync(kFull, nt);
+                if (u < n) {
+                    const int pos = start_s[nt] + __popc(same & ((1u << lane) - 1));
+                    const int round = pos / grid;
+                    int col = pos - round * grid;
+                    if (round & 1) col = grid - 1 - col;
+                    if (col == (int)blockIdx.x && round < kMaxRanked) sb.my_units[round] = u;
+                }
+                __syncwarp();
+                if (u < n && lane == 31 - __clz(same)) start_s[nt] += __popc(same);   // one lane per count
+                __syncwarp();
             }
         }
-        if (!ok) {
-            // let the copies already issued land before the CTA goes away
-            auto land = [&](unsigned long long *full, uint32_t n, uint32_t slots) {
-                for (uint32_t k = 1; k <= slots && k <= n; ++k) {
+        __syncthreads();
+    }
+
+    if (warp == 4) {
+        // ------------------------------------------------------------ TMA producer
+        if (lane == 0) {
+            uint32_t tile = 0, unit = 0;
+            bool ok = true;
+            const int n_items = item_count(a);
+            // a prefix that is read once: its lines are the first to leave L2 again, so that the queries,
+            // the tree's keys and values and the metadata the units keep coming back to stay there
+            // (with several row blocks per unit the blocks read the same prefix: ordinary policy)
+            uint64_t pol_stream;
+            if (a.row_blocks == 1) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
+            else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol_stream));
+            for (int u = blockIdx.x; u < n_items * a.n_layers && ok; u += gridDim.x) {
+                const int layer = u / n_items;
+                const AttnItem item = get_item(a, u - layer * n_items, sb);
+                if (item.b < 0) continue;
+                const int b = item.b, g = item.g;
+                const int64_t L = a.prefix_off[b + 1] - a.prefix_off[b];
+                const int64_t row0 = a.prefix_off[b] * a.Hkv + (int64_t)g * L + item.t0;
+                // paged: tile j of the item is page t0/64 + j of the beam, one 64-row box of the pool
+                const int32_t *pages = a.page_table ? a.page_table + a.page_off[b] + item.t0 / kBN : nullptr;
+                int page_next = (pages && item.t1 > item.t0) ? pages[0] : 0;
+                const int nt_p = (item.t1 - item.t0 + kBN - 1) / kBN;
+                const int n_lo = a.beam_node_off[b];
+                const int nt = nt_p + (item.last ? tree_tiles(a, b) : 0);
+                // The unit's query rows: one box per 64-column half, rows = (node, query head of this
+                // KV head) in the order the MMA reads them.  The single Q buffer is free once the
+                // previous unit's last Q K^T product has completed, which is while that unit's last
+                // softmax, P V product and output write are still running: the copy hides behind them.
+                if (unit > 0) ok = mbar_wait(&sb.q_empty, (unit - 1) & 1, &sb, a.status);
+                if (!ok) break;
+                {
+                    const int z = n_lo + item.rb * a.nodes_per_block + layer * a.q_layer_nodes;
+                    mbar_expect_tx(&sb.q_full, (uint32_t)a.block_rows * kD * 2);
+                    tma_load_3d_one(q_s, &map_q, 0, g * a.group, z, &sb.q_full);
+                    tma_load_3d_one(q_s + QROWS * 128, &map_q, 64, g * a.group, z, &sb.q_full);
+                }
+                ++unit;
+                for (int j = 0; j < nt && ok; ++j, ++tile) {
+                    const int s = tile % kStages;
+                    const uint32_t par = (tile / kStages) & 1;
+                    ok = mbar_wait(&sb.kv_empty[s], par ^ 1, &sb, a.status);
+                    if (!ok) break;
+                    unsigned char *ks = stage_s + s * kStageBytes, *vs = ks + kTileBytes;
+                    mbar_expect_tx(&sb.kv_full[s], kStageBytes);
+#ifdef DSBD_TEST_WAIT_TIMEOUT
+                    if (tile == 1 && blockIdx.x == 0) continue;      // the bytes this barrier expects never come
+#endif
+                    if (j < nt_p) {
+                        int y = (int)(row0 + (int64_t)j * kBN);
+                        if (pages) {
+                            y = (page_next * a.Hkv + g) * kBN + layer * a.pool_layer_rows;
+                            if (j + 1 < nt_p) page_next = pages[j + 1];
+                        }
+                        tma_load_2d_hint_one(ks, &map_kp, 0, y, &sb.kv_full[s], pol_stream);
+                        tma_load_2d_hint_one(ks + kTileBytes / 2, &map_kp, 64, y, &sb.kv_full[s], pol_stream);
+                        tma_load_2d_hint_one(vs, &map_vp, 0, y, &sb.kv_full[s], pol_stream);
+                        tma_load_2d_hint_one(vs + kTileBytes / 2, &map_vp, 64, y, &sb.kv_full[s], pol_stream);
+                    } else {
+                        const int x = g * kD;                                  // tree tile j - nt_p
+                        const int y = n_lo + (j - nt_p) * kBN + layer * a.new_layer_rows;
+                        tma_load_2d_one(ks, &map_kn, x, y, &sb.kv_full[s]);
+                        tma_load_2d_one(ks + kTileBytes / 2, &map_kn, x + 64, y, &sb.kv_full[s]);
+                        tma_load_2d_one(vs, &map_vn, x, y, &sb.kv_full[s]);
+                        tma_load_2d_one(vs + kTileBytes / 2, &map_vn, x + 64, y, &sb.kv_full[s]);
+                    }
+                }
+            }
+            if (!ok) {
+                // let the copies already issued land before the CTA goes away
+                for (uint32_t k = 0; k < (uint32_t)kStages && k < tile; ++k) {
+                    const uint32_t t = tile - 1 - k;
                     const long long t0 = clock64();
-                    while (!mbar_try(&full[(n - k) % slots], ((n - k) / slots) & 1))
+                    while (!mbar_try(&sb.kv_full[t % kStages], (t / kStages) & 1))
                         if (clock64() - t0 > kWaitCycles) break;
                 }
-            };
-            land(sb.k_full, n_k, S::kKSlots);
-            land(sb.v_full, n_v, S::kVSlots);
-            land(sb.q_full, unit, (uint32_t)a.q_bufs);
+            }
         }
-    } else if (warp == kWarpS) {
-        // ------------------------------------------------------------ S^T issuer
+    } else if (warp == 5) {
+        // ------------------------------------------------------------ MMA issuer
+        // the warp stays converged and predicates the MMAs on one lane: issued from a branch of a single thread
+        // each takes 95 cycles, like this about 50
         const bool on = lane == 0;
+        {
+            constexpr uint32_t idesc_s = instr_desc(kRows, kBN, 0, 0);
+            constexpr uint32_t idesc_o = instr_desc(kRows, kD, 0, 1);
+            uint32_t tile = 0, unit = 0;
+            bool ok = true;
+            const uint64_t qd = desc_k_major(smem_u32(q_s));
+            const int n_items = item_count(a);
+            for (int u = blockIdx.x; u < n_items * a.n_layers && ok; u += gridDim.x) {
+                const AttnItem item = get_item(a, u % n_items, sb);
+                if (item.b < 0) continue;
+                const int nt = (item.t1 - item.t0 + kBN - 1) / kBN + (item.last ? tree_tiles(a, item.b) : 0);
+                ok = warp_wait(&sb.q_full, unit & 1, &sb, a.status);
+                // S(t) = Q K(t)^T into S buffer t & 1; issued one tile ahead of the P V product so
+                // that it runs while the softmax warps work on the previous tile
+                auto issue_s = [&](uint32_t t) -> bool {
+                    const int s = t % kStages;
+                    if (!warp_wait(&sb.kv_full[s], (t / kStages) & 1, &sb, a.status)) return false;
+                    tc_fence_after();
+                    const uint64_t kd = desc_k_major(smem_u32(stage_s + s * kStageBytes));
+#pragma unroll
+                    for (int ks = 0; ks < kD / 16; ++ks) {
+                        const uint64_t ad = qd + (uint64_t)((ks / 4) * ((QROWS * 128) >> 4) + (ks % 4) * 2);
+                        const uint64_t bd = kd + (uint64_t)((ks / 4) * ((kBN * 128) >> 4) + (ks % 4) * 2);
+                        mma_ss(on, tmem + kColS + (t & 1) * 64, ad, bd, idesc_s, ks > 0);
+                    }
+                    tc_commit(on, &sb.s_full[t & 1]);
+                    return true;
+                };
+                if (ok) ok = issue_s(tile);
+                if (ok && nt == 1) tc_commit(on, &sb.q_empty);       // the unit's last (only) Q K^T product
+                for (int j = 0; j < nt && ok; ++j, ++tile) {
+                    if (j + 1 < nt) {
+                        ok = issue_s(tile + 1);
+                        if (!ok) break;
+                        if (j + 2 == nt) tc_commit(on, &sb.q_empty);
+                    }
+                    const int s = tile % kStages;
+                    ok = warp_wait(&sb.p_full[tile & 1], (tile >> 1) & 1, &sb, a.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t vd = desc_mn_major(smem_u32(stage_s + s * kStageBytes) + kTileBytes, kBN * 128);
+#pragma unroll
+                    for (int ks = 0; ks < kBN / 16; ++ks)
+                        mma_ts(on, tmem + kColO, tmem + kColS + (tile & 1) * 64 + ks * 8,
+                               vd + (uint64_t)(ks * ((16 * 128) >> 4)), idesc_o, (j > 0 || ks > 0) ? 1u : 0u);
+                    tc_commit(on, &sb.kv_empty[s]);
+                    tc_commit(on, &sb.pv_done);
+                }
+                if (ok) tc_commit(on, &sb.o_full);
+                ++unit;
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ softmax warps
+        const int row = warp * 32 + lane;
+        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
         uint32_t tile = 0, unit = 0;
         bool ok = true;
-        while (ok && cur.next(a, sb, sg)) {
-            const int rows = min(a.block_rows, sg.n_tree * a.group - sg.rb * a.block_rows);
-            const uint32_t idesc = instr_desc(kTile, max(16, (rows + 15) & ~15), 0, 0);
-            const uint32_t qb = unit % a.q_bufs, q_half = (uint32_t)a.q_rows * 128;
-            const uint64_t qd = desc_k_major(smem_u32(q_s) + qb * S::kHalves * q_half);
-            ok = warp_wait(&sb.q_full[qb], (unit / a.q_bufs) & 1, &sb, a.status);
-            for (int j = sg.t0; j < sg.t1 && ok; ++j, ++tile) {
-                const uint32_t s = tile % S::kKSlots, sbuf = tile % S::kSBufs;
-                ok = warp_wait(&sb.k_full[s], (tile / S::kKSlots) & 1, &sb, a.status);
-                // The softmax has read what the buffer held.  With two P buffers, wait for the O^T product two
-                // tiles back, which came after: S^T then also says that the tile's P buffer is free
-                if (S::kPBufs == 2) {
-                    if (ok && tile >= 2) ok = warp_wait(&sb.pv_done[tile & 1], ((tile - 2) >> 1) & 1, &sb, a.status);
-                } else if (ok && tile >= S::kSBufs) {
-                    ok = warp_wait(&sb.p_full[sbuf], (tile / S::kSBufs - 1) & 1, &sb, a.status);
+        const int n_items = item_count(a);
+        for (int u = blockIdx.x; u < n_items * a.n_layers && ok; u += gridDim.x) {
+            const AttnItem item = get_item(a, u % n_items, sb);
+            if (item.b < 0) continue;
+            const int b = item.b, g = item.g;
+            const int64_t L = item.t1;                         // tokens beyond t1 belong to other items
+            const int nt_p = (item.t1 - item.t0 + kBN - 1) / kBN;
+            const int n_lo = a.beam_node_off[b];
+            const int n_tree = a.beam_node_off[b + 1] - n_lo;
+            const int nt = nt_p + (item.last ? (n_tree + kBN - 1) / kBN : 0);
+            const int M = n_tree * a.group;
+            const int r0 = item.rb * a.block_rows;              // first row of this row block
+            // (the MMA's rows from block_rows on hold no query of this block: never active)
+            const bool warp_active = warp * 32 < a.block_rows && r0 + warp * 32 < M;
+            const bool active = row < a.block_rows && r0 + row < M;
+            const int node = active ? (r0 + row) / a.group : 0;
+            const int hq = g * a.group + (active ? r0 + row - node * a.group : 0);
+            // ancestor-or-self mask of this row's node: walk up the tree
+            unsigned long long anc_lo = 0ull, anc_hi = 0ull;       // nodes 0..63, 64..127
+            {
+                int n = node;
+                for (int hop = 0; hop < 2 * kBN && n >= 0 && n < n_tree; ++hop) {
+                    if (n < 64) anc_lo |= 1ull << n; else anc_hi |= 1ull << (n - 64);
+                    const int par = a.parent[n_lo + n];
+                    if (par >= n_lo + n) { report(a.status, DSBD_DEV_BAD_FOREST); break; }
+                    n = par < 0 ? -1 : par - n_lo;
                 }
+            }
+            float m_ref = -INFINITY, l_run = 0.f;
+            for (int j = 0; j < nt && ok; ++j, ++tile) {
+                ok = mbar_wait(&sb.s_full[tile & 1], (tile >> 1) & 1, &sb, a.status);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t kd = desc_k_major(smem_u32(smem + s * S::kSlot));
-#pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks)
-                    mma_ss(on, tmem + sbuf * NMAX, kd + (uint64_t)((ks / 4) * (kHalfStride >> 4) + (ks % 4) * 2),
-                           qd + (uint64_t)((ks / 4) * (q_half >> 4) + (ks % 4) * 2), idesc, ks > 0);
-                tc_commit(on, &sb.k_empty[s]);
-                tc_commit(on, &sb.s_full[sbuf]);
-                if (j + 1 == sg.t1) tc_commit(on, &sb.q_empty[qb]);          // the unit's last S^T product
-            }
-            ++unit;
-        }
-        if (!ok) drain(on, &sb.drain[0]);
-    } else if (warp == kWarpO) {
-        // ------------------------------------------------------------ O^T issuer
-        const bool on = lane == 0;
-        uint32_t tile = 0, unit = 0;
-        bool ok = true;
-        while (ok && cur.next(a, sb, sg)) {
-            const int rows = min(a.block_rows, sg.n_tree * a.group - sg.rb * a.block_rows);
-            const uint32_t idesc = instr_desc(128, max(16, (rows + 15) & ~15), 1, 1);
-            const uint32_t col = tmem + S::kColO + (unit & 1) * NMAX;
-            // the accumulators were last used two units ago
-            ok = warp_wait(&sb.o_empty[unit & 1], ((unit >> 1) & 1) ^ 1, &sb, a.status);
-            for (int j = sg.t0; j < sg.t1 && ok; ++j, ++tile) {
-                const uint32_t s = tile % S::kVSlots;
-                ok = warp_wait(&sb.v_full[s], (tile / S::kVSlots) & 1, &sb, a.status) &&
-                     warp_wait(&sb.p_full[tile % S::kSBufs], (tile / S::kSBufs) & 1, &sb, a.status);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t vd = desc_mn_major(smem_u32(smem + S::kOffV + s * S::kSlot), kHalfStride);
-                const bool both = sg.nh - 2 * j >= 2;        // a lone box: 64 tokens
-                const uint32_t acc = j > sg.t0 ? 1u : 0u;
-#pragma unroll
-                for (int term = 0; term < (SPLIT ? 2 : 1); ++term) {
-                    const uint64_t pd = desc_mn_major(
-                        smem_u32(p_s + (tile % S::kPBufs) * S::kPBuf + term * S::kPTerm), kHalfStride);
-#pragma unroll
-                    for (int ks = 0; ks < kTile / 16; ++ks)
-                        mma_ss(on && (ks < 4 || both), col, vd + (uint64_t)(ks * ((16 * 128) >> 4)),
-                               pd + (uint64_t)(ks * ((16 * 128) >> 4)), idesc, (term + ks > 0) ? 1u : acc);
-                }
-                tc_commit(on, &sb.v_empty[s]);
-                tc_commit(on, &sb.pv_done[tile & 1]);
-            }
-            if (ok) tc_commit(on, &sb.o_full[unit & 1]);
-            ++unit;
-        }
-        if (!ok) drain(on, &sb.drain[1]);
-    } else if (warp >= kWarpOut && warp < kWarpTma) {
-        // ------------------------------------------------------------ output
-        const int q = warp & 3, tid = threadIdx.x & 127;
-        const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        uint32_t unit = 0;
-        CutRec rec = {};
-        int rec_layer = (int)blockIdx.x / a.runs;
-        auto put_rec = [&](int layer) {
-            if (!a.whole && tid == 0) a.recs[layer * a.runs + (int)blockIdx.x % a.runs] = rec;
-        };
-        while (cur.next(a, sb, sg)) {
-            if (sg.layer != rec_layer) { put_rec(rec_layer); rec = CutRec{}; rec_layer = sg.layer; }
-            const int rows = min(a.block_rows, sg.n_tree * a.group - sg.rb * a.block_rows);
-            const uint32_t ub = unit & 1;
-            const uint32_t o_addr = tmem + lane_base + S::kColO + ub * NMAX;
-            bool ok = warp_wait(&sb.sum_full[ub], (unit >> 1) & 1, &sb, a.status);
-            if (ok) ok = warp_wait(&sb.o_full[ub], (unit >> 1) & 1, &sb, a.status);
-            if (group_any(kGroups, !ok)) break;
-            tc_fence_after();
-            const bool whole = sg.t0 == 0 && sg.t1 == sg.nt;
-            float *part = a.partial;
-            if (!whole) {
-                part += (2 * ((int64_t)sg.layer * a.runs + (int)blockIdx.x % a.runs) + (sg.t0 == 0 ? 1 : 0)) *
-                        NMAX * (D + 2);
-                if (sg.t0 > 0) rec.head_ends = sg.t1 == sg.nt;
-                else { rec.tail = 1; rec.b = sg.b; rec.g = sg.g; rec.rb = sg.rb; }
-            }
-            if (tid < rows) {
-                const float sum = (sx.red[ub][0][tid] + sx.red[ub][1][tid]) + (sx.red[ub][2][tid] + sx.red[ub][3][tid]);
-                if (whole) {
-                    sx.fac[tid] = 1.f / sum;
-                } else {
-                    sx.fac[tid] = 1.f;
-                    part[tid * (D + 2)] = sum > 0.f ? sx.ref[ub][tid] : -INFINITY;
-                    part[tid * (D + 2) + 1] = sum;
-                }
-            }
-            group_sync(kGroups);
-            if (tid < D) {                                   // (d = 64: lanes 64.. hold aliased rows; whole warps)
-                __nv_bfloat16 *dst = a.out + (int64_t)sg.layer * a.q_layer_stride +
-                                     ((int64_t)(sg.n_lo + sg.rb * a.nodes_per_block) * a.Hq + sg.g * a.group) * D +
-                                     (tid & ~1);
-                const int nch = (rows + 15) / 16;
-#pragma unroll 1
-                for (int ch = 0; ch < nch; ++ch) {
-                    uint32_t ov[16];
-                    tmem_ld16(o_addr + ch * 16, ov);
+                if (warp_active) {
+                    uint32_t sv[2][32];
+                    const uint32_t s_col = kColS + (tile & 1) * 64;
+                    tmem_ld32(tmem + lane_base + s_col, sv[0]);
+                    tmem_ld32(tmem + lane_base + s_col + 32, sv[1]);
                     tmem_wait_ld();
-                    float v[16];
-#pragma unroll
-                    for (int c = 0; c < 16; c += 4) {
-                        const float4 f = *reinterpret_cast<const float4 *>(&sx.fac[ch * 16 + c]);
-                        v[c] = __uint_as_float(ov[c]) * f.x; v[c + 1] = __uint_as_float(ov[c + 1]) * f.y;
-                        v[c + 2] = __uint_as_float(ov[c + 2]) * f.z; v[c + 3] = __uint_as_float(ov[c + 3]) * f.w;
+                    float mx = -INFINITY;
+                    const bool tree = (j >= nt_p);
+                    // visibility of the tile's 64 tokens for this row, as a bit mask
+                    unsigned long long vis;
+                    if (tree) {
+                        const int jt = j - nt_p, left = n_tree - jt * kBN;
+                        vis = (jt ? anc_hi : anc_lo) & (left >= 64 ? ~0ull : ((1ull << left) - 1));
                     }
-                    if (whole) {
-                        // two lanes swap halves of two rows, so that each stores a pair of columns of one row
+                    else {
+                        const int64_t left = L - item.t0 - (int64_t)j * kBN;
+                        vis = left >= 64 ? ~0ull : ((1ull << left) - 1);
+                    }
+                    // The softmax warps set the pace of a unit (one row per thread, 64 columns in sequence),
+                    // so the common tile -- every token visible -- does no masking, the scale is folded
+                    // into the exponent's fma, and the exponential is the bare ex2.approx.
+                    if (vis != ~0ull) {
 #pragma unroll
-                        for (int c = 0; c < 16; c += 2) {
-                            const int row = ch * 16 + c + (lane & 1);
-                            const float swap = __shfl_xor_sync(kFull, (lane & 1) ? v[c] : v[c + 1], 1);
-                            const uint32_t w = (lane & 1) ? pack_bf16(swap, v[c + 1]) : pack_bf16(v[c], swap);
-                            if (row < rows) *reinterpret_cast<uint32_t *>(dst + sx.rowoff[row]) = w;
+                        for (int c = 0; c < 64; ++c)
+                            if (!((vis >> c) & 1ull)) sv[c >> 5][c & 31] = 0xff800000u;      // -inf: weight 0
+                    }
+                    {   // four independent chains: this warp has its scheduler nearly to itself, so a
+                        // 64-long dependent chain would be pure latency
+                        float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                        for (int c = 0; c < 64; ++c) m4[c & 3] = fmaxf(m4[c & 3], __uint_as_float(sv[c >> 5][c & 31]));
+                        mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+                    }
+                    mx *= a.scale_log2;                                  // scale > 0 (checked by the host)
+                    // lazy rescale: move the reference only when some row of the warp needs it
+                    const bool need = mx > m_ref + 8.f;
+                    if (__any_sync(kFull, need)) {
+                        // O is about to be rescaled in place: the previous tile's P V must have landed
+                        if (j > 0 && !mbar_wait(&sb.pv_done, (tile - 1) & 1, &sb, a.status)) { ok = false; }
+                        tc_fence_after();
+                        const float m_new = need ? mx : m_ref;
+                        const float f = (m_ref == -INFINITY) ? 0.f : exp2f(m_ref - m_new);
+                        l_run *= f;
+                        if (j > 0) {
+#pragma unroll
+                            for (int cc = 0; cc < 4; ++cc) {
+                                uint32_t ov[32];
+                                tmem_ld32(tmem + lane_base + kColO + cc * 32, ov);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * f);
+                                tmem_st32(tmem + lane_base + kColO + cc * 32, ov);
+                            }
                         }
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 16; ++c)
-                            if (ch * 16 + c < rows) part[(ch * 16 + c) * (D + 2) + 2 + tid] = v[c];
+                        m_ref = m_new;
                     }
-                    __syncwarp();
+                    uint32_t pv[32];
+                    const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
+                    float l4[4] = {0.f, 0.f, 0.f, 0.f};                  // (independent chains again)
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) {
+                        const float p0 = ex2_ftz(fmaf(__uint_as_float(sv[(2 * c) >> 5][(2 * c) & 31]), a.scale_log2, -m_use));
+                        const float p1 = ex2_ftz(fmaf(__uint_as_float(sv[(2 * c + 1) >> 5][(2 * c + 1) & 31]), a.scale_log2, -m_use));
+                        const uint32_t pk = pack_bf16(p0, p1);
+                        // the row sum must match what the tensor core will see: the rounded values
+                        l4[c & 1] += __uint_as_float(pk << 16);
+                        l4[2 + (c & 1)] += __uint_as_float(pk & 0xffff0000u);
+                        pv[c] = pk;
+                    }
+                    l_run += (l4[0] + l4[1]) + (l4[2] + l4[3]);
+                    tmem_st32(tmem + lane_base + s_col, pv);
+                    tmem_wait_st();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sb.p_full[tile & 1]);
+            }
+            if (!ok) break;
+            // ---- unit done: O / l -> global
+            ok = mbar_wait(&sb.o_full, unit & 1, &sb, a.status);
+            if (!ok) break;
+            tc_fence_after();
+            if (warp_active) {
+                const int layer = u / n_items;
+                if (item.nparts == 1) {
+                    const float inv = active ? 1.f / l_run : 0.f;
+                    __nv_bfloat16 *dst = a.out + (int64_t)layer * a.q_layer_stride +
+                                         ((int64_t)(n_lo + node) * a.Hq + hq) * kD;
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) {
+                        uint32_t ov[32];
+                        tmem_ld32(tmem + lane_base + kColO + cc * 32, ov);
+                        tmem_wait_ld();
+                        if (active) {
+#pragma unroll
+                            for (int c = 0; c < 32; c += 8) {
+                                uint4 w;
+                                w.x = pack_bf16(__uint_as_float(ov[c]) * inv, __uint_as_float(ov[c + 1]) * inv);
+                                w.y = pack_bf16(__uint_as_float(ov[c + 2]) * inv, __uint_as_float(ov[c + 3]) * inv);
+                                w.z = pack_bf16(__uint_as_float(ov[c + 4]) * inv, __uint_as_float(ov[c + 5]) * inv);
+                                w.w = pack_bf16(__uint_as_float(ov[c + 6]) * inv, __uint_as_float(ov[c + 7]) * inv);
+                                *reinterpret_cast<uint4 *>(dst + cc * 32 + c) = w;
+                            }
+                        }
+                    }
+                } else {
+                    // partial result of this part of the unit: reference maximum, row sum, raw O
+                    float *dst = a.partial +
+                                 (((int64_t)layer * a.slots_per_layer + item.slot) * a.max_rows + r0 + row) * 130;
+                    if (active) { dst[0] = m_ref; dst[1] = l_run; }
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) {
+                        uint32_t ov[32];
+                        tmem_ld32(tmem + lane_base + kColO + cc * 32, ov);
+                        tmem_wait_ld();
+                        if (active) {
+#pragma unroll
+                            for (int c = 0; c < 32; c += 2)
+                                *reinterpret_cast<float2 *>(dst + 2 + cc * 32 + c) =
+                                    make_float2(__uint_as_float(ov[c]), __uint_as_float(ov[c + 1]));
+                        }
+                    }
                 }
             }
             tc_fence_before();
-            group_sync(kGroups);                             // (the factors are read before they are written again)
-            if (lane == 0) mbar_arrive(&sb.o_empty[ub]);
-            ++unit;
-        }
-        put_rec(rec_layer);
-    } else if (warp < kWarpOut) {
-        if (kGroups == 4) asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
-        // ------------------------------------------------------------ softmax groups
-        const int grp = warp >> 2, q = warp & 3, tok = threadIdx.x & 127;     // token inside the tile = TMEM lane
-        const int box = tok >> 6, in_box = tok & 63;
-        const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        uint32_t tile = 0, unit = 0;
-        int mask_b = -1, mask_rb = -1;                       // the tree whose mask this group holds
-        bool ok = true;
-        while (cur.next(a, sb, sg)) {
-            // the group's columns: chunks of 8 rows, shared out evenly
-            const int rows = min(a.block_rows, sg.n_tree * a.group - sg.rb * a.block_rows);
-            const int n8 = (rows + 7) / 8, per = (n8 + kGroups - 1) / kGroups;
-            const int cbase = grp * per * 8, nch = min(max(n8 - grp * per, 0), per);
-            const uint32_t o_addr = tmem + lane_base + S::kColO + (unit & 1) * NMAX + cbase;
-            float l[32];
-#pragma unroll
-            for (int c = 0; c < 32; ++c) l[c] = 0.f;
-            for (int j = sg.t0; j < sg.t1; ++j, ++tile) {
-                // what this thread's token is: a prefix token every row sees, a tree token some rows see,
-                // or nothing
-                const int h = 2 * j + box;
-                const bool plain = (2 * j + 2) * kBN <= sg.L;
-                uint32_t see = ~0u;
-                if (!plain) {
-                    if (2 * j + 2 > sg.nhp && (mask_b != sg.b || mask_rb != sg.rb)) {
-                        // which rows of the group see tree token j: the rows whose node has j on its path to
-                        // the root (kept over the KV heads of a beam)
-                        mask_b = sg.b; mask_rb = sg.rb;
-                        if (tok < sg.n_tree) {
-                            const int par = a.parent[sg.n_lo + tok];
-                            int p = par - sg.n_lo;
-                            if (par < 0 || p < 0) p = -1;
-                            else if (p >= tok) { report(a.status, DSBD_DEV_BAD_FOREST); p = -1; }
-                            sx.par[grp][tok] = (int16_t)p;
-                        }
-                        sx.see[grp][tok] = 0u;
-                        group_sync(grp);
-                        if (tok < 32 && tok < nch * 8 && cbase + tok < rows)
-                            for (int n = (sg.rb * a.block_rows + cbase + tok) / a.group; n >= 0; n = sx.par[grp][n])
-                                atomicOr(&sx.see[grp][n], 1u << tok);
-                        group_sync(grp);
-                    }
-                    const int jt = (h - sg.nhp) * kBN + in_box;
-                    if (h < sg.nhp) {
-                        if (h * kBN + in_box >= sg.L) see = 0u;
-                    } else if (h < sg.nh && jt < sg.n_tree) {
-                        see = sx.see[grp][jt];
-                    } else {
-                        see = 0u;
-                    }
-                }
-                ok = warp_wait(&sb.s_full[tile % S::kSBufs], (tile / S::kSBufs) & 1, &sb, a.status);
-                tc_fence_after();
-                const bool work = ok && nch > 0 && h < sg.nh;   // (a lone box leaves the upper two warps idle)
-                const uint32_t s_addr = tmem + lane_base + (tile % S::kSBufs) * NMAX + cbase;
-                // the first tile sets the references: the logits of its first token when every row sees it (a
-                // prefix token or the root), else the maxima
-                bool set = j == sg.t0 && 2 * j > sg.nhp;
-                if (j == sg.t0) {
-                    if (!set) {
-                        if (q == 0 && work) {
-#pragma unroll 1
-                            for (int ch = 0; ch < nch; ++ch) {
-                                uint32_t v[8];
-                                tmem_ld8(s_addr + ch * 8, v);
-                                tmem_wait_ld();
-                                if (tok == 0) {
-#pragma unroll
-                                    for (int c = 0; c < 8; c += 4)
-                                        *reinterpret_cast<float4 *>(&sx.negref[grp][ch * 8 + c]) =
-                                            make_float4(-__uint_as_float(v[c]) * a.scale_log2, -__uint_as_float(v[c + 1]) * a.scale_log2,
-                                                        -__uint_as_float(v[c + 2]) * a.scale_log2, -__uint_as_float(v[c + 3]) * a.scale_log2);
-                                }
-                                __syncwarp();
-                            }
-                        }
-                    } else if (tok < nch * 8) {
-                        sx.negref[grp][tok] = 0.f;
-                    }
-                    group_sync(grp);
-                }
-                // one P buffer: it is free once the last product has landed
-                if (S::kPBufs == 1 && ok && tile >= 1)
-                    ok = warp_wait(&sb.pv_done[(tile - 1) & 1], ((tile - 1) >> 1) & 1, &sb, a.status);
-                // the weights: bf16 pairs (SPLIT: the sums of their two terms) of the group's rows
-                uint32_t w[SPLIT ? 32 : 16];
-                float over = 0.f;                            // how far logits exceed the references
-                for (int attempt = 0; ; ++attempt) {
-                    if (work && ok) {
-                        over = 0.f;
-                        uint32_t sv[32];
-#pragma unroll
-                        for (int ch = 0; ch < 4; ++ch)
-                            if (ch < nch) tmem_ld8(s_addr + ch * 8, sv + ch * 8);
-                        tmem_wait_ld();
-                        if (!plain) {
-#pragma unroll
-                            for (int c = 0; c < 32; ++c)
-                                if (!((see >> c) & 1u)) sv[c] = 0xff800000u;           // -inf: weight 0
-                        }
-#pragma unroll
-                        for (int ch = 0; ch < 4; ++ch) {
-                            if (ch >= nch) break;
-                            uint32_t pk[4], lo[4];
-#pragma unroll
-                            for (int i = 0; i < 2; ++i) {
-                                const int c = ch * 8 + 4 * i;
-                                const float4 nr = *reinterpret_cast<const float4 *>(&sx.negref[grp][c]);
-                                const float d0 = fmaf(__uint_as_float(sv[c]), a.scale_log2, nr.x);
-                                const float d1 = fmaf(__uint_as_float(sv[c + 1]), a.scale_log2, nr.y);
-                                const float d2 = fmaf(__uint_as_float(sv[c + 2]), a.scale_log2, nr.z);
-                                const float d3 = fmaf(__uint_as_float(sv[c + 3]), a.scale_log2, nr.w);
-                                over = fmaxf(over, fmaxf(fmaxf(d0, d1), fmaxf(d2, d3)));
-                                const float p0 = ex2_ftz(d0), p1 = ex2_ftz(d1), p2 = ex2_ftz(d2), p3 = ex2_ftz(d3);
-                                pk[2 * i] = pack_bf16(p0, p1);
-                                pk[2 * i + 1] = pack_bf16(p2, p3);
-                                if (SPLIT) {
-                                    lo[2 * i] = pack_bf16(p0 - bf16_lo(pk[2 * i]), p1 - bf16_hi(pk[2 * i]));
-                                    lo[2 * i + 1] = pack_bf16(p2 - bf16_lo(pk[2 * i + 1]), p3 - bf16_hi(pk[2 * i + 1]));
-                                }
-                            }
-                            const int r8 = cbase / 8 + ch;   // eight rows are one 16-byte piece of the token's line
-                            unsigned char *to = p_s + (tile % S::kPBufs) * S::kPBuf + (r8 >> 3) * kHalfStride + tok * 128 +
-                                                (((r8 & 7) ^ (tok & 7)) << 4);
-                            *reinterpret_cast<uint4 *>(to) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                            if (SPLIT) *reinterpret_cast<uint4 *>(to + S::kPTerm) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                if (SPLIT) {
-                                    w[(ch * 8 + 2 * i) % (SPLIT ? 32 : 16)] = __float_as_uint(bf16_lo(pk[i]) + bf16_lo(lo[i]));
-                                    w[(ch * 8 + 2 * i + 1) % (SPLIT ? 32 : 16)] = __float_as_uint(bf16_hi(pk[i]) + bf16_hi(lo[i]));
-                                } else {
-                                    w[ch * 4 + i] = pk[i];
-                                }
-                            }
-                        }
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    }
-                    if (!group_any(grp, !ok || over > kMoveRef || set) || attempt == 2) break;
-                    // rare: some reference has to move (or a wait ran out): O^T is rescaled, so the previous
-                    // product must have landed
-                    if (ok && j > sg.t0) ok = warp_wait(&sb.pv_done[(tile - 1) & 1], ((tile - 1) >> 1) & 1, &sb, a.status);
-                    if (group_any(grp, !ok)) { ok = false; break; }
-                    tc_fence_after();
-#pragma unroll 1
-                    for (int ch = 0; ch < nch; ++ch) {       // the columns' maxima over the tile's tokens
-                        uint32_t v[8];
-                        if (work) tmem_ld8(s_addr + ch * 8, v);
-                        tmem_wait_ld();
-                        float f[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            f[i] = work && ((see >> (ch * 8 + i)) & 1u) ? __uint_as_float(v[i]) : -INFINITY;
-                        fold8(f, lane, [](float x, float y) { return fmaxf(x, y); });
-                        if (lane < 8) sx.colmax[grp][q][ch * 8 + lane] = f[0];
-                        __syncwarp();
-                    }
-                    group_sync(grp);
-                    if (tok < nch * 8) {
-                        const float m = fmaxf(fmaxf(sx.colmax[grp][0][tok], sx.colmax[grp][1][tok]),
-                                              fmaxf(sx.colmax[grp][2][tok], sx.colmax[grp][3][tok])) *
-                                        a.scale_log2;        // scale > 0 (checked by the host)
-                        const float nr = sx.negref[grp][tok];
-                        const bool move = set ? m > -INFINITY : m + nr > 0.f;
-                        sx.move[grp][tok] = move ? exp2f(-(m + nr)) : 1.f;
-                        if (move) sx.negref[grp][tok] = -m;
-                    }
-                    set = false;
-                    group_sync(grp);
-                    if (j > sg.t0) {
-#pragma unroll
-                        for (int ch = 0; ch < 4; ++ch) {
-                            if (ch >= nch) break;
-                            uint32_t ov[8];
-                            tmem_ld8(o_addr + ch * 8, ov);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) {
-                                const float f = sx.move[grp][ch * 8 + c];
-                                ov[c] = __float_as_uint(__uint_as_float(ov[c]) * f);
-                                l[ch * 8 + c] *= f;
-                            }
-                            tmem_st8(o_addr + ch * 8, ov);
-                        }
-                        tmem_wait_st();
-                    }
-                }
-                if (!ok) break;
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sb.p_full[tile % S::kSBufs]);
-                if (work) {
-                    // (the row sum must match what the tensor core sees: the rounded values)
-#pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
-                        if (ch >= nch) break;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int c = ch * 8 + 2 * i;
-                            l[c] += SPLIT ? __uint_as_float(w[c % (SPLIT ? 32 : 16)]) : bf16_lo(w[ch * 4 + i]);
-                            l[c + 1] += SPLIT ? __uint_as_float(w[(c + 1) % (SPLIT ? 32 : 16)]) : bf16_hi(w[ch * 4 + i]);
-                        }
-                    }
-                }
-            }
-            if (!ok) break;
-            // ---- the unit's (or the part's) end: references and row sums over the tokens for the output warps,
-            // which have read those of the unit before the previous one
-            const uint32_t ub = unit & 1;
-            ok = warp_wait(&sb.o_empty[ub], ((unit >> 1) & 1) ^ 1, &sb, a.status);
-#pragma unroll
-            for (int ch = 0; ch < 4; ++ch) {
-                if (ch >= nch) break;
-                fold8(l + ch * 8, lane, [](float x, float y) { return x + y; });
-                if (lane < 8) sx.red[ub][q][cbase + ch * 8 + lane] = l[ch * 8];
-            }
-            if (tok < nch * 8) sx.ref[ub][cbase + tok] = -sx.negref[grp][tok];
-            // (read before the next unit sets new references)
-            if (group_any(grp, !ok)) { ok = false; break; }
-            if (lane == 0) mbar_arrive(&sb.sum_full[ub]);
             ++unit;
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == kWarpS) {
+    if (warp == 5) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
 }
 
-// Merge of the units that were cut: block (i, y, layer) takes the unit that starts as the last one of run i,
-// warps over its rows; out = sum_p O_p 2^(m_p - m) / sum_p l_p 2^(m_p - m).
-constexpr int kMergeThreads = 256;
-template <int D, int NMAX>
-__global__ void __launch_bounds__(kMergeThreads)
-k_attn_combine(TcArgs a) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int layer = blockIdx.z, i0 = layer * a.runs + (int)blockIdx.x, end = (layer + 1) * a.runs - 1;
-    const CutRec rec = a.recs[i0];
-    if (!rec.tail) return;
-    int last = min(i0 + 1, end);                             // the runs that hold the other parts
-    while (last < end && !a.recs[last].head_ends) ++last;
-    const int n_lo = a.beam_node_off[rec.b];
-    const int n_tree = min(a.beam_node_off[rec.b + 1] - n_lo, kMaxTree);
-    const int rows = min(a.block_rows, n_tree * a.group - rec.rb * a.block_rows);
-    const int lane = threadIdx.x & 31;
-    constexpr int kPer = D / 32;                             // values per lane: 2 (d = 64) or 4
-    for (int row = (blockIdx.y * kMergeThreads + threadIdx.x) >> 5; row < rows; row += gridDim.y * kMergeThreads / 32) {
-        auto part = [&](int i) { return a.partial + ((2 * (int64_t)i + (i == i0 ? 1 : 0)) * NMAX + row) * (D + 2); };
-        float m = -INFINITY;
-        for (int i = i0; i <= last; ++i) m = fmaxf(m, part(i)[0]);
-        float l = 0.f, o[kPer] = {};
-        for (int i = i0; i <= last; ++i) {
-            const float *src = part(i);
-            if (src[0] == -INFINITY) continue;
-            const float w = exp2f(src[0] - m);
-            l += src[1] * w;
-#pragma unroll
-            for (int e = 0; e < kPer; e += 2) {
-                const float2 x = *reinterpret_cast<const float2 *>(src + 2 + lane * kPer + e);
-                o[e] += x.x * w; o[e + 1] += x.y * w;
+// ---------------------------------------------------------------------------------------
+// Work plan for ragged or small batches: every unit's prefix is cut into parts of at most
+// `chunk` tokens (equal parts, multiples of 64), and the items are ordered by decreasing tile
+// count, so that handing item i to CTA i mod grid spreads the work evenly.
+// ---------------------------------------------------------------------------------------
+struct UnitParts { int first_slot, nparts; };
+
+__device__ __forceinline__ void unit_parts(int64_t L, int chunk, int *np, int *plen) {
+    int n = (int)((L + chunk - 1) / chunk);
+    if (n < 1) n = 1;
+    const int64_t per = (L + n - 1) / n;
+    *np = n;
+    *plen = (int)((per + kBN - 1) / kBN) * kBN;
+}
+
+__global__ void __launch_bounds__(1024)
+k_attn_plan(int B, int Hkv, const int64_t *__restrict__ prefix_off, const int32_t *__restrict__ beam_node_off,
+            int group, int block_rows, int chunk, int grid, AttnItem *__restrict__ items,
+            int *__restrict__ n_items, UnitParts *__restrict__ units) {
+    __shared__ int bucket[1024];
+    __shared__ int scan[1024];
+    __shared__ int carry;
+    const int tid = threadIdx.x, n_units = B * Hkv;
+    // row blocks a tree really has: only those become items
+    auto blocks_of = [&](int b) {
+        const int rows = (beam_node_off[b + 1] - beam_node_off[b]) * group;
+        return rows > block_rows ? (rows + block_rows - 1) / block_rows : 1;
+    };
+    bucket[tid] = 0;
+    if (tid == 0) carry = 0;
+    __syncthreads();
+    // slots: exclusive scan of the part counts over the units, 1024 units at a time
+    for (int base = 0; base < n_units; base += 1024) {
+        const int u = base + tid;
+        int np = 0, plen = 0;
+        if (u < n_units) {
+            const int b = u / Hkv;
+            unit_parts(prefix_off[b + 1] - prefix_off[b], chunk, &np, &plen);
+        }
+        scan[tid] = np;
+        __syncthreads();
+        for (int o = 1; o < 1024; o <<= 1) {
+            const int v = tid >= o ? scan[tid - o] : 0;
+            __syncthreads();
+            scan[tid] += v;
+            __syncthreads();
+        }
+        if (u < n_units) {
+            units[u].first_slot = carry + scan[tid] - np;
+            units[u].nparts = np;
+            const int b = u / Hkv;
+            const int64_t L = prefix_off[b + 1] - prefix_off[b];
+            for (int p = 0; p < np; ++p) {
+                const int64_t t0 = (int64_t)p * plen;
+                const int64_t t1 = t0 + plen < L ? t0 + plen : L;
+                int nt = (int)((t1 - t0 + kBN - 1) / kBN) + (p == np - 1);
+                atomicAdd(&bucket[nt < 1023 ? nt : 1023], blocks_of(b));
             }
         }
+        __syncthreads();
+        if (tid == 0) carry += scan[1023];
+        __syncthreads();
+    }
+    // start of every bucket in the output, largest tile count first
+    scan[tid] = bucket[1023 - tid];
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {
+        const int v = tid >= o ? scan[tid - o] : 0;
+        __syncthreads();
+        scan[tid] += v;
+        __syncthreads();
+    }
+    const int start = scan[tid] - bucket[1023 - tid];
+    const int total_items = scan[1023];          // all buckets together
+    __syncthreads();
+    bucket[1023 - tid] = start;                 // bucket[k] becomes the cursor of tile count k
+    // The list is read in rounds of `grid` items, CTA k taking entry k of every round.  Odd rounds
+    // are stored back to front, so that the CTA with the longest item of one round gets the
+    // shortest of the next; the last round is padded with empty entries (b = -1).
+    const int padded = (total_items + grid - 1) / grid * grid;
+    for (int i = total_items - total_items % grid + tid; i < padded; i += 1024) items[i].b = -1;
+    if (tid == 0) *n_items = padded;
+    __syncthreads();
+    for (int u = tid; u < n_units; u += 1024) {
+        const int b = u / Hkv, g = u - b * Hkv;
+        const int64_t L = prefix_off[b + 1] - prefix_off[b];
+        int np, plen;
+        unit_parts(L, chunk, &np, &plen);
+        for (int p = 0; p < np; ++p) {
+            const int64_t t0 = (int64_t)p * plen;
+            const int64_t t1 = t0 + plen < L ? t0 + plen : L;
+            const int nt = (int)((t1 - t0 + kBN - 1) / kBN) + (p == np - 1);
+            const int nrb = blocks_of(b);
+            for (int rb = 0; rb < nrb; ++rb) {
+                int pos = atomicAdd(&bucket[nt < 1023 ? nt : 1023], 1);
+                const int round = pos / grid;
+                if (round & 1) pos = round * grid + (grid - 1 - (pos - round * grid));
+                AttnItem it;
+                it.b = b; it.g = g; it.t0 = (int)t0; it.t1 = (int)t1; it.last = (p == np - 1);
+                it.nparts = np; it.slot = units[u].first_slot + p; it.rb = rb;
+                items[pos] = it;
+            }
+        }
+    }
+}
+
+// Merge the parts of every split unit: out = sum_c O_c 2^(m_c - m) / sum_c l_c 2^(m_c - m).
+__global__ void __launch_bounds__(128)
+k_attn_combine(TcArgs a, const UnitParts *__restrict__ units) {
+    const int layer = blockIdx.y;
+    int u = blockIdx.x;
+    UnitParts up;
+    if (units) {
+        up = units[u];
+    } else {                                             // tail split: block i merges tail unit i
+        up.first_slot = u * a.tail_k; up.nparts = a.tail_k;
+        u += a.tail_first;
+    }
+    if (up.nparts <= 1) return;
+    const int b = u / a.Hkv, g = u - b * a.Hkv;
+    a.partial += (int64_t)layer * a.slots_per_layer * a.max_rows * 130;
+    a.out += (int64_t)layer * a.q_layer_stride;
+    const int n_lo = a.beam_node_off[b];
+    const int M = (a.beam_node_off[b + 1] - n_lo) * a.group;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int row = warp; row < M; row += 4) {
+        float m = -INFINITY;
+        for (int c = 0; c < up.nparts; ++c)
+            m = fmaxf(m, a.partial[((int64_t)(up.first_slot + c) * a.max_rows + row) * 130]);
+        float l = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < up.nparts; ++c) {
+            const float *src = a.partial + ((int64_t)(up.first_slot + c) * a.max_rows + row) * 130;
+            const float w = src[0] == -INFINITY ? 0.f : exp2f(src[0] - m);
+            l += src[1] * w;
+            const float2 x = *reinterpret_cast<const float2 *>(src + 2 + lane * 4);
+            const float2 y = *reinterpret_cast<const float2 *>(src + 4 + lane * 4);
+            o.x += x.x * w; o.y += x.y * w; o.z += y.x * w; o.w += y.y * w;
+        }
         const float inv = 1.f / l;
-        const int r = rec.rb * a.block_rows + row, node = r / a.group, hq = rec.g * a.group + (r - node * a.group);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(a.out + (int64_t)layer * a.q_layer_stride +
-                                                     ((int64_t)(n_lo + node) * a.Hq + hq) * D + lane * kPer);
-#pragma unroll
-        for (int e = 0; e < kPer; e += 2) dst[e / 2] = pack_bf16(o[e] * inv, o[e + 1] * inv);
+        const int node = row / a.group, hq = g * a.group + (row - node * a.group);
+        __nv_bfloat16 *dst = a.out + ((int64_t)(n_lo + node) * a.Hq + hq) * kD + lane * 4;
+        uint2 w2;
+        w2.x = pack_bf16(o.x * inv, o.y * inv);
+        w2.y = pack_bf16(o.z * inv, o.w * inv);
+        *reinterpret_cast<uint2 *>(dst) = w2;
     }
 }
 
-typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                             const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                             CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeFn encode_fn() {
-    static EncodeFn fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeFn>(p);
-    }
-    return fn;
-}
-
-// [rows, cols] bf16 row-major with `pitch` bytes between rows; boxes of 64 cols x 64 rows.
-bool make_map(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint64_t pitch) {
-    EncodeFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {cols, rows};
-    const cuuint64_t strides[1] = {pitch};
-    const cuuint32_t box[2] = {64, (cuuint32_t)kBN};
-    const cuuint32_t el[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, el,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// q as [nodes, Hq, d] bf16: boxes of 64 columns x `group` heads x `nodes` nodes, i.e. the query rows
-// of one KV head for a run of nodes, in (node, head) order.
-bool make_map_q(CUtensorMap *m, const void *base, uint64_t d, uint64_t Hq, uint64_t nodes_total, uint32_t group,
-                uint32_t nodes) {
-    EncodeFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {d, Hq, nodes_total};
-    const cuuint64_t strides[2] = {d * 2, Hq * d * 2};
-    const cuuint32_t box[3] = {64, group, nodes};
-    const cuuint32_t el[3] = {1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, el,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Launch shape shared by the workspace query and the launch.  It does not depend on the number of layers
-// of a call (nor do the results).
+// Launch shape shared by the workspace query and the launch.
 struct TcPlan {
-    int nmax;                 // query rows of the kernel instance: 64 or 128
-    int block_rows;           // rows of a row block: whole nodes (the copy engine fetches them as a box of
-                              // nodes x heads), as many as nmax holds
-    int row_blocks;           // of the largest tree
-    int q_nodes, q_rows;      // nodes and rows (a multiple of 8) of a block's query box
-    int runs, uni_nt;
-    int sms;
-    bool whole;               // no unit is cut: no partial results, no merge
+    int grid, chunk;          // chunk == 0: one item per unit in unit order, no plan kernel
+    bool split;               // units are cut into parts (partials + combine kernel)
+    int tail_first, tail_k;   // chunk == 0 only: the units from tail_first on are cut into tail_k parts
+    bool rank;                // chunk == 0 only: the CTAs order the (ragged) units themselves
+    int64_t items_max;
+    size_t off_items, off_units, off_partial, total;
 };
 
-// Cutting units into equal runs costs partial results and the merge kernel: about as long as kCutTiles
-// tiles of one CTA.  A run of fewer than kMinTiles tiles is not worth another CTA.
-constexpr int64_t kCutTiles = 6, kMinTiles = 8;
+// Query rows per row block.  Trees of up to 64 rows take the 64-row tile (two CTAs per SM).  So do
+// forests whose AVERAGE tree has at most 64 rows even when the largest is bigger (a sampled
+// forest puts most drafts under a few roots and leaves the other trees tiny): the big trees then
+// run as several 64-row blocks, the many small ones at the faster shape.
+int tile_rows_for(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
+    const int group = d->Hq / d->Hkv;
+    if (f->max_tree_nodes * group <= 64) return 64;
+    return ((int64_t)f->N * group <= (int64_t)64 * f->B && group <= 64) ? 64 : kRows;
+}
+// Rows of a row block: whole nodes (the copy engine fetches a block's query rows as a box of nodes x
+// heads), as many as the tile holds.
+int block_rows_for(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
+    const int group = d->Hq / d->Hkv;
+    return tile_rows_for(f, d) / group * group;
+}
 
-TcPlan make_plan(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
+TcPlan make_plan(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, int n_layers = 1) {
     TcPlan p = {};
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int group = d->Hq / d->Hkv, rows = f->max_tree_nodes * group;
-    p.sms = sms;
-    p.nmax = rows <= 64 ? 64 : 128;
-    p.block_rows = p.nmax / group * group;
-    p.row_blocks = (rows + p.block_rows - 1) / p.block_rows;
-    p.q_nodes = std::min(p.block_rows / group, f->max_tree_nodes);
-    p.q_rows = (p.q_nodes * group + 7) / 8 * 8;
-    const int tree_boxes = (f->max_tree_nodes + kBN - 1) / kBN;
-    const int64_t max_nt = ((d->max_prefix + kBN - 1) / kBN + tree_boxes + 1) / 2;
-    const int64_t units = (int64_t)f->B * d->Hkv;
-    const bool uniform = p.row_blocks == 1 && tree_boxes == 1 && d->max_prefix * f->B == d->total_prefix;
-    // tiles of a layer (ragged: a lower bound)
-    const int64_t tiles = uniform ? units * max_nt : std::max<int64_t>(units, d->total_prefix / kTile * d->Hkv);
-    const int64_t cut_len = std::max<int64_t>((tiles + sms - 1) / sms, kMinTiles) + kCutTiles;
-    int64_t runs = std::min<int64_t>(sms, std::max<int64_t>(tiles / kMinTiles, 1));
-    if (uniform) {
-        p.uni_nt = (int)max_nt;
-        p.whole = (units + sms - 1) / sms * max_nt <= cut_len;
-    } else {
-        p.whole = p.row_blocks == 1 && units <= sms && max_nt <= cut_len;
+    const int group = d->Hq / d->Hkv;
+    const int block_rows = block_rows_for(f, d);
+    const bool small_q = tile_rows_for(f, d) == 64;
+    p.grid = small_q ? 2 * sms : sms;
+    const int row_blocks = (f->max_tree_nodes * group + block_rows - 1) / block_rows;
+    const int64_t n_units = (int64_t)f->B * d->Hkv * row_blocks;     // counted with their row blocks
+    // Splitting a unit costs a pipeline drain, a Q reload and a partial result per part, so it
+    // pays only when there are fewer units than CTAs: then the prefix is cut so that about two
+    // items per CTA exist, in parts of at least 512 tokens.  Ragged batches with enough units
+    // are only re-ordered (longest first, rounds alternating in direction).
+    int64_t c = (int64_t)d->total_prefix * d->Hkv / (2ll * p.grid);
+    if (c < 512) c = 512;
+    c = (c + kBN - 1) / kBN * kBN;
+    p.split = n_units < p.grid && c < d->max_prefix;
+    const bool ragged = (int64_t)d->max_prefix * f->B * 100 > (int64_t)d->total_prefix * 115;
+    // trees with several row blocks always go through the plan, which lists only the blocks that
+    // exist (in unit order most (unit, block) pairs of a ragged forest would be empty, and the
+    // CTAs whose stride hits the first blocks would do all the work)
+    if (!p.split && !(ragged && n_units > p.grid) && row_blocks == 1) {
+        p.chunk = 0;
+        p.items_max = n_units;
+        if (p.grid > n_units) p.grid = (int)n_units;
+        p.total = 256;
+        // Equal-length units that do not fill the last round of CTAs: cut the units of that round
+        // into parts so that (nearly) every CTA has a part of it.  1024 units on 296 CTAs are 3.46
+        // rounds: whole units would take the time of 4, with the last 136 units in 2 parts 3.5.
+        const int rem = (int)(n_units % p.grid);
+        const bool uniform = (int64_t)d->max_prefix * f->B == d->total_prefix;
+        if (uniform && n_units > p.grid && rem > 0) {
+            const int tiles = (int)((d->max_prefix + kBN - 1) / kBN);
+            int k = p.grid / rem;
+            if (k > 8) k = 8;
+            if (k > tiles / 8) k = tiles / 8;               // parts of at least 8 tiles
+            if (k >= 2) {
+                p.tail_first = (int)n_units - rem;
+                p.tail_k = k;
+                p.items_max = (int64_t)p.tail_first + (int64_t)rem * k;
+                p.off_partial = 256;
+                p.total = align_up(256 + sizeof(float) * 130 * (size_t)n_layers * (size_t)rem * k *
+                                             (size_t)(f->max_tree_nodes * group), 256);
+            }
+        }
+        return p;
     }
-    if (p.whole) runs = std::min<int64_t>(units, sms);       // (ragged: one unit each)
-    p.runs = (int)runs;
+    // a ragged batch of whole units, few enough per CTA: no plan kernel, every CTA ranks the units
+    // itself at its start (a few microseconds in parallel instead of a serial kernel ahead of it)
+    if (!p.split && row_blocks == 1 && n_units <= 2048 && n_units <= (int64_t)kMaxRanked * p.grid) {
+        p.chunk = 0;
+        p.rank = true;
+        p.items_max = n_units;
+        p.total = 256;
+        return p;
+    }
+    if (!p.split) c = (int64_t)1 << 30;                  // one part per unit
+    p.chunk = (int)c;
+    p.items_max = (p.split ? (int64_t)d->Hkv * row_blocks * (d->total_prefix / c + f->B) : n_units) + p.grid;
+    if (p.grid > p.items_max - p.grid) p.grid = (int)(p.items_max - p.grid);
+    if (p.grid < 1) p.grid = 1;
+    size_t off = 256;
+    p.off_items = off;   off = align_up(off + sizeof(AttnItem) * (size_t)p.items_max, 256);
+    p.off_units = off;   off = align_up(off + sizeof(UnitParts) * (size_t)f->B * d->Hkv, 256);
+    p.off_partial = off;
+    if (p.split)
+        off = align_up(off + sizeof(float) * 130 * (size_t)n_layers * (size_t)p.items_max *
+                                 (size_t)(f->max_tree_nodes * group), 256);
+    p.total = off;
     return p;
-}
-
-size_t partial_offset(const TcPlan &p, int n_layers) { return align_up(sizeof(CutRec) * (size_t)p.runs * n_layers, 256); }
-size_t workspace_of(const TcPlan &p, int n_layers, int d) {
-    if (p.whole) return 256;
-    return align_up(partial_offset(p, n_layers) + sizeof(float) * 2 * (size_t)p.runs * n_layers * p.nmax * (d + 2), 256);
-}
-
-template <int D, int NMAX, bool SPLIT>
-int launch(const TcPlan &p, const CUtensorMap (&maps)[5], TcArgs a, cudaStream_t stream) {
-    using S = Shape<D, NMAX, SPLIT>;
-    if (cudaFuncSetAttribute(k_forest_attn_tc<D, NMAX, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)S::kSmem) != cudaSuccess)
-        return DSBD_ERR_CUDA;
-    // (an S^T product reads up to 8 rows past a buffer's last one: columns that nobody uses)
-    a.q_bufs = (uint32_t)(2 * S::kHalves * p.q_rows + 8) * 128 <= S::kQBytes ? 2 : 1;
-    // several layers: as many side by side as the SMs hold, each CTA with the same run of its layers
-    a.layer_step = std::max(1, std::min(a.n_layers, p.sms / p.runs));
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.runs * a.layer_step));
-    cfg.blockDim = dim3(S::kThreads);
-    cfg.dynamicSmemBytes = S::kSmem;
-    cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, k_forest_attn_tc<D, NMAX, SPLIT>, maps[0], maps[1], maps[2], maps[3], maps[4], a) !=
-        cudaSuccess)
-        return DSBD_ERR_CUDA;
-    if (p.whole) return DSBD_OK;
-    cfg.gridDim = dim3((unsigned)p.runs, (unsigned)((p.block_rows + 31) / 32), (unsigned)a.n_layers);
-    cfg.blockDim = dim3(kMergeThreads);
-    cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, k_attn_combine<D, NMAX>, a) == cudaSuccess ? DSBD_OK : DSBD_ERR_CUDA;
 }
 
 }  // namespace
@@ -1127,8 +828,6 @@ namespace dsbd {
 
 // Layer count and strides of a paged call, checked: the layers of one call share one tensor map
 // per operand, so a layer stride must be a whole number of map rows.
-struct LayerDims { int n_layers, pool_rows, new_rows; int64_t q_stride; bool ok; };
-
 LayerDims layer_dims(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const dsbd_kv_pages_t *pages) {
     LayerDims L = {1, 0, 0, 0, true};
     if (!pages || pages->n_layers <= 1) return L;
@@ -1147,13 +846,11 @@ LayerDims layer_dims(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const ds
 }
 
 bool attention_tc_supported(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, int64_t n_pages) {
-    if (d->dtype != DSBD_DTYPE_BF16) return false;
-    // heads of 64: packed caches, trees of one tree box (the limits of the entry point for d = 64)
-    if (d->d == 64 ? (n_pages > 0 || f->max_tree_nodes > DSBD_MAX_TREE_NODES) : d->d != 128) return false;
-    if (d->Hq / d->Hkv > 128) return false;                                  // a node's rows fit one row block
+    if (d->dtype != DSBD_DTYPE_BF16 || d->d != kD) return false;
+    if (d->Hq / d->Hkv > kRows) return false;                                // a node's rows fit one tile
     if (!(d->scale > 0.f)) return false;                                     // the row maximum is taken before scaling
-    if (f->max_tree_nodes * (d->Hq / d->Hkv) > 1024) return false;
-    if (f->max_tree_nodes > kMaxTree) return false;
+    if (f->max_tree_nodes * (d->Hq / d->Hkv) > kRows * 8) return false;      // up to 8 row blocks
+    if (f->max_tree_nodes > 2 * kBN) return false;                           // two tree tiles
     if (d->total_prefix <= 0) return false;
     // row coordinates of the K/V maps are 32-bit
     const int64_t rows = n_pages > 0 ? n_pages * d->Hkv * kBN : (int64_t)d->total_prefix * d->Hkv;
@@ -1166,57 +863,98 @@ bool attention_tc_layers_ok(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, c
 }
 
 size_t attention_tc_workspace(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, int n_layers) {
-    return workspace_of(make_plan(f, d), n_layers < 1 ? 1 : n_layers, d->d);
+    return make_plan(f, d, n_layers < 1 ? 1 : n_layers).total;
 }
 
-int attention_tc_launches(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) { return make_plan(f, d).whole ? 1 : 2; }
+int attention_tc_launches(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
+    const TcPlan p = make_plan(f, d);
+    return 1 + (p.chunk > 0 ? 1 : 0) + (p.split || p.tail_k ? 1 : 0);
+}
 
 int launch_attention_tc(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const void *q, const void *k_new,
                         const void *v_new, const void *k_prefix, const void *v_prefix, const int64_t *prefix_off,
                         void *out, void *workspace, size_t workspace_bytes, int32_t *status, cudaStream_t stream,
                         const dsbd_kv_pages_t *pages) {
+    CUtensorMap kp, vp, kn, vn, qm;
     const LayerDims LD = layer_dims(f, d, pages);
     if (!LD.ok) return DSBD_ERR_INVALID_ARG;
     const int nl = LD.n_layers;
-    const TcPlan plan = make_plan(f, d);
-    if (workspace_bytes < workspace_of(plan, nl, d->d)) return DSBD_ERR_WORKSPACE_TOO_SMALL;
-    if (!plan.whole && (reinterpret_cast<uintptr_t>(workspace) & 255)) return DSBD_ERR_INVALID_ARG;
     // one map per operand over all layers: layer l starts l * (layer stride in rows) further down
-    const uint64_t D = (uint64_t)d->d;
     const uint64_t prows = pages ? (uint64_t)pages->n_pages * d->Hkv * kBN + (uint64_t)(nl - 1) * LD.pool_rows
                                  : (uint64_t)d->total_prefix * d->Hkv;
     const uint64_t nrows = (uint64_t)f->N + (uint64_t)(nl - 1) * LD.new_rows;
-    const int group = d->Hq / d->Hkv;
-    const int64_t q_layer_nodes = nl > 1 ? LD.q_stride / ((int64_t)d->Hq * d->d) : 0;
-    if ((uint64_t)f->N + (uint64_t)(nl - 1) * q_layer_nodes >= ((uint64_t)1 << 31)) return DSBD_ERR_UNSUPPORTED;
-    CUtensorMap maps[5];
-    if (!make_map(&maps[0], k_prefix, D, prows, D * 2) || !make_map(&maps[1], v_prefix, D, prows, D * 2) ||
-        !make_map(&maps[2], k_new, (uint64_t)d->Hkv * D, nrows, (uint64_t)d->Hkv * D * 2) ||
-        !make_map(&maps[3], v_new, (uint64_t)d->Hkv * D, nrows, (uint64_t)d->Hkv * D * 2) ||
-        !make_map_q(&maps[4], q, D, (uint64_t)d->Hq, (uint64_t)f->N + (uint64_t)(nl - 1) * q_layer_nodes,
-                    (uint32_t)group, (uint32_t)plan.q_nodes))
+    if (!make_map(&kp, k_prefix, kD, prows, kD * 2) || !make_map(&vp, v_prefix, kD, prows, kD * 2) ||
+        !make_map(&kn, k_new, (uint64_t)d->Hkv * kD, nrows, (uint64_t)d->Hkv * kD * 2) ||
+        !make_map(&vn, v_new, (uint64_t)d->Hkv * kD, nrows, (uint64_t)d->Hkv * kD * 2))
         return DSBD_ERR_CUDA;
+    const int group = d->Hq / d->Hkv, block_rows = block_rows_for(f, d);
+    const int64_t q_layer_nodes = nl > 1 ? LD.q_stride / ((int64_t)d->Hq * kD) : 0;
+    if ((uint64_t)f->N + (uint64_t)(nl - 1) * q_layer_nodes >= ((uint64_t)1 << 31)) return DSBD_ERR_UNSUPPORTED;
+    if (!make_map_q(&qm, q, kD, (uint64_t)d->Hq, (uint64_t)f->N + (uint64_t)(nl - 1) * q_layer_nodes, (uint32_t)group,
+                    (uint32_t)(block_rows / group)))
+        return DSBD_ERR_CUDA;
+    const TcPlan plan = make_plan(f, d, nl);
+    if (workspace_bytes < plan.total) return DSBD_ERR_WORKSPACE_TOO_SMALL;
+    char *ws = static_cast<char *>(workspace);
     TcArgs a = {};
-    a.B = f->B; a.N = f->N; a.Hq = d->Hq; a.Hkv = d->Hkv; a.group = group;
-    a.block_rows = plan.block_rows;
-    a.nodes_per_block = plan.block_rows / group;
-    a.q_nodes = plan.q_nodes; a.q_rows = plan.q_rows;
-    a.runs = plan.runs; a.uni_nt = plan.uni_nt; a.whole = plan.whole;
-    a.reread = plan.row_blocks > 1;
+    a.B = f->B; a.N = f->N; a.Hq = d->Hq; a.Hkv = d->Hkv; a.group = d->Hq / d->Hkv;
+    a.n_units = f->B * d->Hkv;
+    a.max_rows = f->max_tree_nodes * a.group;
+    a.block_rows = block_rows;
+    a.nodes_per_block = block_rows / group;
+    a.row_blocks = (a.max_rows + a.block_rows - 1) / a.block_rows;
     a.scale_log2 = d->scale * 1.4426950408889634f;
     a.beam_node_off = f->beam_node_off; a.parent = f->parent; a.prefix_off = prefix_off;
     if (pages) { a.page_table = pages->page_table; a.page_off = pages->page_off; }
+    a.q = static_cast<const __nv_bfloat16 *>(q);
     a.out = static_cast<__nv_bfloat16 *>(out);
     a.status = status;
     a.n_layers = nl; a.pool_layer_rows = LD.pool_rows; a.new_layer_rows = LD.new_rows;
     a.q_layer_stride = LD.q_stride;
     a.q_layer_nodes = (int)q_layer_nodes;
-    a.recs = static_cast<CutRec *>(workspace);
-    a.partial = reinterpret_cast<float *>(static_cast<char *>(workspace) + partial_offset(plan, nl));
-    if (d->d == 64)
-        return plan.nmax == 64 ? launch<64, 64, true>(plan, maps, a, stream) : launch<64, 128, true>(plan, maps, a, stream);
-    return plan.nmax == 64 ? launch<128, 64, false>(plan, maps, a, stream)
-                           : launch<128, 128, false>(plan, maps, a, stream);
+    a.slots_per_layer = plan.tail_k ? (a.n_units - plan.tail_first) * plan.tail_k : (int)plan.items_max;
+    a.tail_first = plan.tail_first; a.tail_k = plan.tail_k;
+    a.rank_units = plan.rank ? a.n_units : 0;
+    if (plan.tail_k) {
+        if (reinterpret_cast<uintptr_t>(workspace) & 255) return DSBD_ERR_INVALID_ARG;
+        a.partial = reinterpret_cast<float *>(ws + plan.off_partial);
+    }
+    UnitParts *units = nullptr;
+    if (plan.chunk > 0) {
+        if (reinterpret_cast<uintptr_t>(workspace) & 255) return DSBD_ERR_INVALID_ARG;
+        AttnItem *items = reinterpret_cast<AttnItem *>(ws + plan.off_items);
+        units = reinterpret_cast<UnitParts *>(ws + plan.off_units);
+        int *n_items = reinterpret_cast<int *>(ws);
+        k_attn_plan<<<1, 1024, 0, stream>>>(f->B, d->Hkv, prefix_off, f->beam_node_off, a.group, a.block_rows,
+                                            plan.chunk, plan.grid, items, n_items, units);
+        a.items = items;
+        a.n_items = n_items;
+        a.partial = reinterpret_cast<float *>(ws + plan.off_partial);
+    }
+    // more layers mean more items for the same plan: the grid may grow back to the SM-filling size
+    int grid = plan.grid;
+    if (nl > 1) {
+        int dev = 0, sms = 148;
+        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int full = tile_rows_for(f, d) == 64 ? 2 * sms : sms;
+        if (plan.chunk == 0) grid = (int)std::min<int64_t>((int64_t)plan.items_max * nl, full);
+    }
+    // up to 64 query rows: 16 KB of Q, three stages, two CTAs per SM; more rows: one CTA per SM
+    const bool small_q = tile_rows_for(f, d) == 64;
+#define DSBD_LAUNCH_TC(QR, ST)                                                                              \
+    do {                                                                                                   \
+        constexpr uint32_t bytes = smem_bytes(QR, ST);                                                     \
+        if (cudaFuncSetAttribute(k_forest_attn_tc<QR, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
+                                 (int)bytes) != cudaSuccess)                                               \
+            return DSBD_ERR_CUDA;                                                                          \
+        k_forest_attn_tc<QR, ST><<<grid, kThreadsTc, bytes, stream>>>(kp, vp, kn, vn, qm, a);                  \
+    } while (0)
+    if (small_q) DSBD_LAUNCH_TC(64, 3);
+    else DSBD_LAUNCH_TC(128, 3);
+#undef DSBD_LAUNCH_TC
+    if (plan.split) k_attn_combine<<<dim3(a.n_units, nl), 128, 0, stream>>>(a, units);
+    else if (plan.tail_k) k_attn_combine<<<dim3(a.n_units - plan.tail_first, nl), 128, 0, stream>>>(a, nullptr);
+    return cudaGetLastError() == cudaSuccess ? DSBD_OK : DSBD_ERR_CUDA;
 }
 
 }  // namespace dsbd

@@ -64,7 +64,7 @@ struct Shape {
     static constexpr uint32_t kPTerm = kHalfStride;                                     // [token][128 B]
     static constexpr uint32_t kPBuf = (kSplit ? 2 : 1) * kPTerm;
     static constexpr int kPBufs = 2;
-    static constexpr bool kSWaits = D == 64;                  // S^T waits until the tile's P buffer is free
+    static constexpr bool kSWaits = D == 64 || NMAX == 64;                  // S^T waits until the tile's P buffer is free
     // query rows of one unit, or of two when they fit (a unit's copy then runs a whole unit ahead; with one
     // buffer its latency, 2800 cycles while HBM is saturated, shows at every unit's start)
     static constexpr uint32_t kQBytes = (D == 64 ? 17 : 21) * 1024;
@@ -101,6 +101,7 @@ struct TcArgs {
     int n_layers;                     // >= 1: transformer layers in one launch (paged caches)
     int runs;                         // runs per layer; CTA c takes run c % runs of the layers c / runs + k * layer_step
     int layer_step;
+    int unit_cost;                    // tiles that a unit's start and end are worth
     int uni_nt;                       // > 0: every unit has one row block and this many tiles
     int whole;                        // runs are whole units: nothing is cut
     int reread;                       // some tree has several row blocks: its prefix is read more than once
@@ -143,8 +144,8 @@ struct Barriers {
     uint32_t tmem_base;
     int abort;
     int scan[32];                          // warp sums of the start-up scan
-    int start[3];                          // beam, unit inside the beam, tile inside the unit
-    int run;                               // tiles of the run
+    int start[3];                          // beam, unit inside the beam, cost offset inside the unit
+    int run;                               // cost of the run
 };
 // (The groups are not in step: what a group changes on its own is its own, since the share of the rows that a
 // column belongs to differs from unit to unit.)
@@ -204,6 +205,28 @@ __device__ __forceinline__ void drain(bool on, void *bar) {
     land(bar, 0);
 }
 
+// Two fp32 operations an instruction (sm_100), and a maximum of three.
+struct F2 { float x, y; };
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 d;
+    asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+        "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 d;
+    asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+        "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 // Combines 8 columns over the 32 lanes with 9 shuffles; lane i ends up with column i & 7 in v[0].
 template <class F>
 __device__ __forceinline__ void fold8(float *v, int lane, F op) {
@@ -238,8 +261,10 @@ __device__ __forceinline__ BeamFacts beam_facts(const TcArgs &a, int b) {
 // Walks the runs of this CTA.  One warp does and hands the segments to the others, so that the beams' data
 // is fetched ahead and the walk's code exists once (with a copy in every role the kernel outgrew the
 // instruction cache: a fifth of all stalls at three tiles a unit).
+// Ragged runs are equal in cost: a unit costs its tiles plus unit_cost for its start and end (without it the
+// CTAs that met the short prefixes of a batch of 99 to 4911 tokens ended at 172 us, the median at 128).
 struct Cursor {
-    int left, layer, b, k, toff, loaded;
+    int left, layer, b, k, at, loaded;       // at: cost offset inside the unit
     BeamFacts f;
     __device__ __forceinline__ Cursor(const TcArgs &a, const Barriers &sb) {
         layer = a.whole && a.uni_nt ? 0 : (int)blockIdx.x / a.runs;
@@ -248,7 +273,7 @@ struct Cursor {
         if (a.whole && a.uni_nt) { layer = b / a.B; b -= layer * a.B; }      // the layers' units are one sequence
     }
     __device__ __forceinline__ void rewind(const Barriers &sb) {
-        left = sb.run; b = sb.start[0]; k = sb.start[1]; toff = sb.start[2];
+        left = sb.run; b = sb.start[0]; k = sb.start[1]; at = sb.start[2];
     }
     __device__ __forceinline__ bool next(const TcArgs &a, const Barriers &sb, Seg &s) {
         while (layer < a.n_layers) {
@@ -265,12 +290,13 @@ struct Cursor {
             }
             if (loaded != b) { f = beam_facts(a, b); loaded = b; }
             s.layer = layer; s.b = b; s.g = f.nrb == 1 ? k : k / f.nrb; s.rb = k - s.g * f.nrb;
-            s.t0 = toff; s.t1 = min(f.nt, toff + left);
+            const int extra = a.uni_nt ? 0 : a.unit_cost, stop = min(f.nt + extra, at + left);
+            s.t0 = max(at - extra, 0); s.t1 = max(stop - extra, 0);
             s.whole = s.t0 == 0 && s.t1 == f.nt; s.last = s.t1 == f.nt;
             s.nhp = f.nhp; s.nh = f.nh; s.L = f.L; s.n_lo = f.n_lo; s.n_tree = f.n_tree;
             s.rows = min(a.block_rows, f.n_tree * a.group - s.rb * a.block_rows);
-            left -= s.t1 - s.t0;
-            toff = 0;
+            left -= stop - at;
+            at = 0;
             if (++k == f.nrb * a.Hkv) { k = 0; ++b; }
             if (s.t1 > s.t0) return true;
         }
@@ -305,7 +331,7 @@ __device__ void find_run(const TcArgs &a, Barriers &sb) {
             if (a.whole) {
                 unit = share(units, r, G);
                 lo = 0; hi = (share(units, r + 1, G) - unit) * nt;
-                if (nt == 0) { hi = beam_facts(a, unit / a.Hkv).nt; }      // ragged: one unit per run
+                if (nt == 0) { hi = beam_facts(a, unit / a.Hkv).nt + a.unit_cost; }      // ragged: one unit per run
             } else {
                 lo = share(units * nt, r, G); hi = share(units * nt, r + 1, G);
                 unit = lo / nt;
@@ -316,14 +342,14 @@ __device__ void find_run(const TcArgs &a, Barriers &sb) {
         __syncthreads();
         return;
     }
-    // tiles before every thread's share of the beams
+    // cost before every thread's share of the beams
     const int per = (a.B + kThreads - 1) / kThreads;
     const int b0 = min(tid * per, a.B), b1 = min(b0 + per, a.B);
     int sum = 0;
 #pragma unroll 1
     for (int b = b0; b < b1; ++b) {
         const BeamFacts f = beam_facts(a, b);
-        sum += f.nt * f.nrb * a.Hkv;
+        sum += (f.nt + a.unit_cost) * f.nrb * a.Hkv;
     }
     int incl = sum;
 #pragma unroll
@@ -343,9 +369,9 @@ __device__ void find_run(const TcArgs &a, Barriers &sb) {
 #pragma unroll 1
         for (int b = b0; b < b1; ++b) {
             const BeamFacts f = beam_facts(a, b);
-            const int w = f.nt * f.nrb * a.Hkv;
+            const int cost = f.nt + a.unit_cost, w = cost * f.nrb * a.Hkv;
             if (lo < at + w) {
-                sb.start[0] = b; sb.start[1] = (lo - at) / f.nt; sb.start[2] = (lo - at) % f.nt;
+                sb.start[0] = b; sb.start[1] = (lo - at) / cost; sb.start[2] = (lo - at) % cost;
                 sb.run = hi - lo;
                 break;
             }
@@ -502,9 +528,9 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
             for (int j = sg.t0; j < sg.t1 && ok; ++j, ++tile) {
                 const uint32_t s = tile % S::kKSlots, sbuf = tile % S::kSBufs;
                 ok = warp_wait(&sb.k_full[s], (tile / S::kKSlots) & 1, &sb);
-                // The softmax has read what the buffer held.  d = 64, where the softmax sets the pace: wait for the
-                // O^T product two tiles back, which came after; S^T then also says that the tile's P buffer is
-                // free.  d = 128, where HBM does: no longer than needed, so that the K slot is free early.
+                // The softmax has read what the buffer held.  Where the softmax sets the pace (d = 64, more than 32
+                // rows): wait for the O^T product two tiles back, which came after; S^T then also says that the
+                // tile's P buffer is free.  Where HBM does: no longer than needed, so that the K slot is free early.
                 if (S::kSWaits) {
                     if (ok && tile >= 2) ok = warp_wait(&sb.pv_done[tile & 1], ((tile - 2) >> 1) & 1, &sb);
                 } else if (ok && tile >= S::kSBufs) {
@@ -762,12 +788,12 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                             for (int i = 0; i < 2; ++i) {
                                 const int c = ch * 8 + 4 * i;
                                 const float4 nr = *reinterpret_cast<const float4 *>(&sx.negref[grp][c]);
-                                const float d0 = fmaf(__uint_as_float(sv[c]), a.scale_log2, nr.x);
-                                const float d1 = fmaf(__uint_as_float(sv[c + 1]), a.scale_log2, nr.y);
-                                const float d2 = fmaf(__uint_as_float(sv[c + 2]), a.scale_log2, nr.z);
-                                const float d3 = fmaf(__uint_as_float(sv[c + 3]), a.scale_log2, nr.w);
-                                over = fmaxf(over, fmaxf(fmaxf(d0, d1), fmaxf(d2, d3)));
-                                const float p0 = ex2_ftz(d0), p1 = ex2_ftz(d1), p2 = ex2_ftz(d2), p3 = ex2_ftz(d3);
+                                const F2 sc = {a.scale_log2, a.scale_log2};
+                                const F2 da = fma2(F2{__uint_as_float(sv[c]), __uint_as_float(sv[c + 1])}, sc, F2{nr.x, nr.y});
+                                const F2 db = fma2(F2{__uint_as_float(sv[c + 2]), __uint_as_float(sv[c + 3])}, sc, F2{nr.z, nr.w});
+                                over = max3(over, da.x, da.y);
+                                over = max3(over, db.x, db.y);
+                                const float p0 = ex2_ftz(da.x), p1 = ex2_ftz(da.y), p2 = ex2_ftz(db.x), p3 = ex2_ftz(db.y);
                                 pk[2 * i] = pack_bf16(p0, p1);
                                 pk[2 * i + 1] = pack_bf16(p2, p3);
                                 if (S::kSplit) {
@@ -851,8 +877,10 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
                             const int c = ch * 8 + 2 * i;
-                            l[c] += S::kSplit ? __uint_as_float(w[c % kW]) : bf16_lo(w[ch * 4 + i]);
-                            l[c + 1] += S::kSplit ? __uint_as_float(w[(c + 1) % kW]) : bf16_hi(w[ch * 4 + i]);
+                            const F2 wt = S::kSplit ? F2{__uint_as_float(w[c % kW]), __uint_as_float(w[(c + 1) % kW])}
+                                                    : F2{bf16_lo(w[(ch * 4 + i) % kW]), bf16_hi(w[(ch * 4 + i) % kW])};
+                            const F2 t = add2(F2{l[c], l[c + 1]}, wt);
+                            l[c] = t.x; l[c + 1] = t.y;
                         }
                     }
                 }
@@ -1073,6 +1101,8 @@ int launch_attention_tr(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const
     a.nodes_per_block = plan.block_rows / group;
     a.q_nodes = plan.q_nodes; a.q_rows = plan.q_rows;
     a.runs = plan.runs; a.uni_nt = plan.uni_nt; a.whole = plan.whole;
+    // (tiles of 64-wide heads are half as long: 222 us at 1, 195 at 2 for 33 x 2-5 beams of 92 to 6875 tokens)
+    a.unit_cost = d->d == 64 ? 2 : 1;
     a.reread = plan.row_blocks > 1;
     a.scale_log2 = d->scale * 1.4426950408889634f;
     a.beam_node_off = f->beam_node_off; a.parent = f->parent; a.prefix_off = prefix_off;

@@ -304,120 +304,82 @@ __device__ double ordered_sum(const double *v, int n, int lane) {
 }
 
 // Inverse-CDF search over tile masses (canonical order).  mass(i) must be the same on every
-// lane.  Returns the tile holding the first cell whose running sum reaches target, and the
-// mass before that tile; if rounding leaves the target beyond the total, the last tile with
-// mass.  -1 if there is no mass at all.
+// lane.  Returns the tile holding the first cell whose running sum reaches the target, and the
+// target minus the mass before that tile; if rounding leaves the target beyond the total, the last
+// tile with mass.  -1 if there is no mass at all.  The target is u * total when of_total, else u.
+// Every round cuts the range by 32: a lane sums its share (its loads are independent, one memory
+// latency a round instead of one per 32 tiles), the lanes' sums are scanned, one lane is chosen.
 template <class F>
-__device__ int locate_tile(F mass, int n, double target, int lane, double *before) {
-    double running = 0.0, last_before = 0.0;
-    int last = -1;
-    for (int base = 0; base < n; base += 32) {
-        const int i = base + lane;
-        const double v = i < n ? mass(i) : 0.0;
+__device__ int locate_tile(F mass, int n, double u, bool of_total, int lane, double *rest) {
+    int lo = 0, len = n;
+    double target = u;
+    while (true) {
+        const int per = (len + 31) >> 5, i0 = lo + lane * per, i1 = min(i0 + per, lo + len);
+        double v = 0.0;
+#pragma unroll 4
+        for (int i = i0; i < i1; ++i) v += mass(i);
         const double incl = warp_scan(v, lane);
-        const bool hit = v > 0.0 && running + incl >= target;
-        const unsigned hits = __ballot_sync(kFull, hit);
-        if (hits) {
-            const int l = __ffs(hits) - 1;
-            *before = running + __shfl_sync(kFull, incl - v, l);
-            return base + l;
-        }
+        if (of_total) { target = u * __shfl_sync(kFull, incl, 31); of_total = false; }
         const unsigned pos = __ballot_sync(kFull, v > 0.0);
-        if (pos) {
-            const int l = 31 - __clz(pos);
-            last = base + l;
-            last_before = running + __shfl_sync(kFull, incl - v, l);
-        }
-        running += __shfl_sync(kFull, incl, 31);
+        if (!pos) return -1;
+        const unsigned hits = __ballot_sync(kFull, v > 0.0 && incl >= target);
+        const int l = hits ? __ffs(hits) - 1 : 31 - __clz(pos);
+        target -= __shfl_sync(kFull, incl - v, l);
+        lo += l * per;
+        len = min(per, len - l * per);
+        if (per == 1) { *rest = target; return lo; }
     }
-    *before = last_before;
-    return last;
 }
 
 // Inverse-CDF search inside one tile of row `row` (and its q row when s > 0): the first
 // token whose running mass reaches `target`, else the last token with mass.  -1: no mass.
-__device__ int locate_token(const VerifyArgs &a, int row, int t, const RowOff &ro, float s,
-                            double target, int lane) {
-    const float *rp = a.zp + (int64_t)row * a.stride;
-    const float *rq = a.zq + (int64_t)row * a.stride;
-    double running = 0.0;
-    int last = -1;
-    for (int it = 0; it < 8; ++it) {
-        const int e = t * kTile + it * 128 + lane * 4;
-        float mss[4];
-        double loc = 0.0;
+// A lane sums 32 consecutive tokens (two batches of independent loads), then the lanes take the 32 tokens
+// of the lane that was hit.
+__device__ __noinline__ int locate_token(const float *__restrict__ rp, const float *__restrict__ rq, int V, float k2,
+                                         int t, const RowOff ro, float s, double target, int lane) {
+    const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
+    const int e0 = t * kTile + lane * 32;
+    auto mass = [&](float zp, float zq) { return s > 0.f ? cell_mass(zp, zq, k2, ro, s) : exp2f(fmaf(zp, k2, ro.bp)) * ro.cp; };
+    double v = 0.0;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        float4 zp[4], zq[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float mv = 0.f;
-            if (e + c < a.V) {
-                const float zpv = __ldg(rp + e + c);
-                mv = (s > 0.f) ? cell_mass(zpv, __ldg(rq + e + c), a.k2, ro, s)
-                               : exp2f(fmaf(zpv, a.k2, ro.bp)) * ro.cp;
-            }
-            mss[c] = mv;
-            loc += (double)mv;
-        }
-        const double incl = warp_scan(loc, lane);
-        const bool hit = loc > 0.0 && running + incl >= target;
-        const unsigned hits = __ballot_sync(kFull, hit);
-        if (hits) {
-            const int l = __ffs(hits) - 1;
-            int tok = -1;
-            if (lane == l) {
-                double cum = running + incl - loc;
-                int lastpos = -1;
-                for (int c = 0; c < 4; ++c) {
-                    cum += (double)mss[c];
-                    if (mss[c] > 0.f) {
-                        lastpos = c;
-                        if (cum >= target) { tok = e + c; break; }
-                    }
+        for (int i = 0; i < 4; ++i) {
+            const int e = e0 + half * 16 + i * 4;
+            zq[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (al && e + 3 < V) {
+                zp[i] = __ldg(reinterpret_cast<const float4 *>(rp + e));
+                if (s > 0.f) zq[i] = __ldg(reinterpret_cast<const float4 *>(rq + e));
+            } else {
+                const float ninf = -INFINITY;
+                zp[i].x = e < V ? __ldg(rp + e) : ninf;         zp[i].y = e + 1 < V ? __ldg(rp + e + 1) : ninf;
+                zp[i].z = e + 2 < V ? __ldg(rp + e + 2) : ninf; zp[i].w = e + 3 < V ? __ldg(rp + e + 3) : ninf;
+                if (s > 0.f) {
+                    zq[i].x = e < V ? __ldg(rq + e) : ninf;         zq[i].y = e + 1 < V ? __ldg(rq + e + 1) : ninf;
+                    zq[i].z = e + 2 < V ? __ldg(rq + e + 2) : ninf; zq[i].w = e + 3 < V ? __ldg(rq + e + 3) : ninf;
                 }
-                if (tok < 0) tok = e + lastpos;
             }
-            return __shfl_sync(kFull, tok, l);
         }
-        const unsigned pos = __ballot_sync(kFull, loc > 0.0);
-        if (pos) {
-            const int l = 31 - __clz(pos);
-            int lp = -1;
-            if (lane == l)
-                for (int c = 0; c < 4; ++c) if (mss[c] > 0.f) lp = e + c;
-            last = __shfl_sync(kFull, lp, l);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            v += (double)mass(zp[i].x, zq[i].x); v += (double)mass(zp[i].y, zq[i].y);
+            v += (double)mass(zp[i].z, zq[i].z); v += (double)mass(zp[i].w, zq[i].w);
         }
-        running += __shfl_sync(kFull, incl, 31);
     }
-    return last;
-}
-
-// Writes output beam number `index` of request r (the caller has checked the slot range).
-__device__ void emit_at(const VerifyArgs &a, int r, int index, int parent, int node, int tok, int source) {
-    {
-        const int s = a.out.out_off[r] + index;
-        // the tree of a node: walk to the root, then find which beam starts there
-        int root = parent;
-        while (a.parent[root] >= 0) root = a.parent[root];
-        int lo = a.req_beam_off[r], hi = a.req_beam_off[r + 1];
-        int beam = lo;
-        for (int b = lo; b < hi; ++b) if (a.beam_node_off[b] == root) beam = b;
-        a.out.out_parent[s] = parent;
-        a.out.out_node[s] = node;
-        a.out.out_root_beam[s] = beam;
-        a.out.out_token[s] = tok;
-        a.out.out_source[s] = source;
-        const double lp = (double)a.zp[(int64_t)parent * a.stride + tok] * a.inv_tau - a.lse[parent];
-        const double lq = (double)a.zq[(int64_t)parent * a.stride + tok] * a.inv_tau - a.lse[a.N + parent];
-        a.out.out_logp[s] = (float)(a.score[parent] + lp);
-        a.out.out_logq[s] = (float)(a.score[a.N + parent] + lq);
+    int first = 0;                                               // the hit lane's first token
+    for (int level = 0; ; ++level) {
+        const double incl = warp_scan(v, lane);
+        const unsigned pos = __ballot_sync(kFull, v > 0.0);
+        if (!pos) return -1;
+        const unsigned hits = __ballot_sync(kFull, v > 0.0 && incl >= target);
+        const int l = hits ? __ffs(hits) - 1 : 31 - __clz(pos);
+        if (level) return first + l;
+        target -= __shfl_sync(kFull, incl - v, l);
+        first = t * kTile + l * 32;
+        const int e = first + lane;
+        v = e < V ? (double)mass(__ldg(rp + e), s > 0.f ? __ldg(rq + e) : 0.f) : 0.0;
     }
-}
-
-__device__ void emit_output(const VerifyArgs &a, int r, int *n_out, int parent, int node, int tok,
-                            int source, bool writer, int *err) {
-    const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
-    if (*n_out >= cap) { *err = DSBD_DEV_CAPACITY; return; }
-    if (writer) emit_at(a, r, *n_out, parent, node, tok, source);
-    (*n_out)++;
 }
 
 // Beam weights of the live set: softmax of the cumulative scores over A (Eq. 1 factorised).
@@ -429,8 +391,41 @@ struct NodeCache {
     double score_p[kCacheNodes], score_q[kCacheNodes], lse_p[kCacheNodes], lse_q[kCacheNodes];
     int16_t parent[kCacheNodes];          // local index of the parent, -1 for a root
     uint8_t depth[kCacheNodes];
+    uint8_t tree[kCacheNodes];            // tree of the node, inside the request
+    int root[kMaxLive];                   // first node of every tree
     int on;
 };
+
+// Writes output beam number `index` of request r (the caller has checked the slot range).  nc: the
+// request's node cache or nullptr; n_lo: first node of the request.
+__device__ void emit_at(const VerifyArgs &a, int r, int index, int parent, int node, int tok, int source,
+                        const NodeCache *nc, int n_lo) {
+    const int s = a.out.out_off[r] + index;
+    const float zp = a.zp[(int64_t)parent * a.stride + tok], zq = a.zq[(int64_t)parent * a.stride + tok];
+    const int lo = a.req_beam_off[r];
+    int beam = lo;
+    double lse_p, lse_q, score_p, score_q;
+    if (nc) {
+        const int i = parent - n_lo;
+        beam += nc->tree[i];
+        lse_p = nc->lse_p[i]; lse_q = nc->lse_q[i]; score_p = nc->score_p[i]; score_q = nc->score_q[i];
+    } else {
+        // the tree of a node: walk to the root, then find which beam starts there
+        int root = parent;
+        while (a.parent[root] >= 0) root = a.parent[root];
+        const int hi = a.req_beam_off[r + 1];
+        for (int b = lo; b < hi; ++b) if (a.beam_node_off[b] == root) beam = b;
+        lse_p = a.lse[parent]; lse_q = a.lse[a.N + parent]; score_p = a.score[parent]; score_q = a.score[a.N + parent];
+    }
+    a.out.out_parent[s] = parent;
+    a.out.out_node[s] = node;
+    a.out.out_root_beam[s] = beam;
+    a.out.out_token[s] = tok;
+    a.out.out_source[s] = source;
+    a.out.out_logp[s] = (float)(score_p + ((double)zp * a.inv_tau - lse_p));
+    a.out.out_logq[s] = (float)(score_q + ((double)zq * a.inv_tau - lse_q));
+}
+
 
 // Natural log of the softmax of n scores, by one warp (lanes over the scores).
 __device__ __forceinline__ void log_softmax_warp(const double *s, int n, int lane, double *out) {
@@ -739,40 +734,34 @@ __device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, unsign
     }
 }
 
-// One completion draw (residual if s_res > 0 else p_beam) by warp 0; returns the token or -1
+// One completion draw (residual if s_res > 0 else p_beam) by one warp; returns the token or -1
 // and the index of the live parent.
 __device__ int draw_cell(const VerifyArgs &a, const Shared &sh, double u, bool use_res, float s_res,
-                         double z_res, const double *res_sums, int lane, int *ia_out) {
-    int tile = -1;
-    double before = 0.0, target;
+                         const double *res_sums, int lane, int *ia_out) {
+    int ia, t;
+    double target;
     if (use_res) {
-        target = u * z_res;
-        tile = locate_tile([&](int i) { return __ldcg(res_sums + i); }, sh.nA * a.T, target, lane, &before);
+        const int tile = locate_tile([&](int i) { return __ldcg(res_sums + i); }, sh.nA * a.T, u, true, lane, &target);
+        if (tile < 0) return -1;
+        ia = tile / a.T; t = tile - ia * a.T;
     } else {
         // p_beam: first the live parent (its row holds exactly its beam weight), then the tile
-        double z = 0.0;
-        for (int i = 0; i < sh.nA; ++i) z += sh.wp[i];
-        target = u * z;
-        double row_before = 0.0;
-        const int ia = locate_tile([&](int i) { return sh.wp[i]; }, sh.nA, target, lane, &row_before);
+        ia = locate_tile([&](int i) { return sh.wp[i]; }, sh.nA, u, true, lane, &target);
         if (ia < 0) return -1;
-        const int T = a.T, row = sh.A[ia];
+        const int row = sh.A[ia];
         const double wpa = sh.wp[ia], lse_row = a.lse[row];
-        double in_row = 0.0;
-        const int t = locate_tile([&](int i) {
-            const TileStat ts = a.stats[(int64_t)row * T + i];
+        const TileStat *st = a.stats + (int64_t)row * a.T;
+        t = locate_tile([&](int i) {
+            const TileStat ts = st[i];
             if (!(ts.sum > 0.f)) return 0.0;
             return wpa * (double)ts.sum * exp((double)ts.mx * a.inv_tau - lse_row);
-        }, T, target - row_before, lane, &in_row);
+        }, a.T, target, false, lane, &target);
         if (t < 0) return -1;
-        tile = ia * T + t;
-        before = row_before + in_row;
     }
-    if (tile < 0) return -1;
-    const int ia = tile / a.T;
     *ia_out = ia;
     const RowOff ro = {sh.bp[ia], sh.bq[ia], sh.cp[ia], sh.cq[ia], sh.dc[ia]};
-    return locate_token(a, sh.A[ia], tile - ia * a.T, ro, use_res ? s_res : 0.f, target - before, lane);
+    const int64_t row = (int64_t)sh.A[ia] * a.stride;
+    return locate_token(a.zp + row, a.zq + row, a.V, a.k2, t, ro, use_res ? s_res : 0.f, target, lane);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1320,6 +1309,8 @@ k_verify(VerifyArgs a) {
     }
     // Every CTA of the cluster takes identical decisions from identical data, so each keeps its
     // own copy of the node statuses and only rank 0 writes results.
+    const int n_trees = min(b_hi - b_lo, kMaxLive);
+    if (!a.select_mode && (int)threadIdx.x < n_trees) nc.root[threadIdx.x] = a.beam_node_off[b_lo + threadIdx.x];
     const int n_layers = a.select_mode ? 1 : a.gamma;
     const int n_req_nodes = n_hi - n_lo;
     const bool st_ok = n_req_nodes <= kMaxLive * kMaxLive;
@@ -1339,6 +1330,9 @@ k_verify(VerifyArgs a) {
             nc.lse_p[i] = a.lse[n];       nc.lse_q[i] = a.lse[a.N + n];
             nc.parent[i] = (int16_t)((par >= n_lo && par < n) ? par - n_lo : -1);
             nc.depth[i] = (uint8_t)min(max(a.depth[n], 0), 255);
+            int tree = 0;
+            while (tree + 1 < n_trees && nc.root[tree + 1] <= n) ++tree;
+            nc.tree[i] = (uint8_t)tree;
         }
     __syncthreads();
     // node data by local index, from the cache when there is one
@@ -1661,41 +1655,47 @@ k_verify(VerifyArgs a) {
             const int W = sh.W, count = sh.count, j = sh.run_j;
             int err = 0;
             if (count < W) {
-                if (lane == 0)
-                    for (int i = 0; i < count && !err; ++i)
-                        emit_output(a, r, &n_out, a.parent[sh.acc[i]], sh.acc[i], a.token[sh.acc[i]],
-                                    DSBD_SRC_DRAFT, writer, &err);
-                n_out = __shfl_sync(kFull, n_out, 0);
-                err = __shfl_sync(kFull, err, 0);
-                int fill = 0;
-                // unwarped: warp 0 makes the residual draw, the p_beam fills (independent draws)
-                // are then spread over the warps of the CTA
-                const int kk_end = warped ? W : count + 1;
-                for (int kk = count; kk < kk_end && !err; ++kk) {
-                    const bool residual = (kk == count);
-                    const bool use_res = residual && j > 1;
-                    const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l,
-                                                      residual ? 1u : 2u, residual ? 0u : (uint32_t)fill);
-                    int ia = 0, tok;
-                    if (warped) {
-                        int pick = -1;
-                        if (lane == 0) pick = draw_support(wsup, u, use_res ? sh.s_arr[j - 1] : 0.0);
-                        pick = __shfl_sync(kFull, pick, 0);
-                        tok = -1;
-                        if (pick >= 0) { ia = wsup.cell[0][pick] / a.V; tok = wsup.cell[0][pick] - ia * a.V; }
-                    } else {
-                        double z_res = 0.0;
-                        if (use_res) z_res = ordered_sum(res_sums, sh.nA * a.T, lane);
-                        tok = draw_cell(a, sh, u, use_res, use_res ? (float)sh.s_arr[j - 1] : 0.f, z_res, res_sums,
-                                        lane, &ia);
+                // accepted drafts, then the residual draw, then fills from p_beam: warp 0 makes the residual draw
+                // (lane 0 when the joint is warped), the other outputs are independent of one another and
+                // spread over lanes or, for unwarped fills, over the warps of the CTA
+                const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
+                const NodeCache *cache = cached ? &nc : nullptr;
+                const int n_acc = min(count, max(cap - n_out, 0));
+                if (writer)
+                    for (int i = lane; i < n_acc; i += 32)
+                        emit_at(a, r, n_out + i, a.parent[sh.acc[i]], sh.acc[i], a.token[sh.acc[i]], DSBD_SRC_DRAFT, cache,
+                                n_lo);
+                n_out += n_acc;
+                if (n_acc < count) err = DSBD_DEV_CAPACITY;
+                const bool use_res = j > 1;
+                const float s_res = use_res ? (float)sh.s_arr[j - 1] : 0.f;
+                if (warped && !err) {
+                    const int want = W - count, n_draw = min(want, max(cap - n_out, 0));
+                    for (int kk = lane; kk < n_draw; kk += 32) {
+                        const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, kk ? 2u : 1u,
+                                                          kk ? (uint32_t)(kk - 1) : 0u);
+                        const int pick = draw_support(wsup, u, kk == 0 && use_res ? sh.s_arr[j - 1] : 0.0);
+                        if (pick < 0) { err = DSBD_DEV_EXHAUSTED; continue; }
+                        const int ia = wsup.cell[0][pick] / a.V, tok = wsup.cell[0][pick] - ia * a.V;
+                        if (writer)
+                            emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, kk ? DSBD_SRC_FILL : DSBD_SRC_RESIDUAL, cache, n_lo);
                     }
-                    if (tok < 0) { err = DSBD_DEV_EXHAUSTED; break; }
-                    if (lane == 0)
-                        emit_output(a, r, &n_out, sh.A[ia], -1, tok, residual ? DSBD_SRC_RESIDUAL : DSBD_SRC_FILL,
-                                    writer, &err);
-                    n_out = __shfl_sync(kFull, n_out, 0);
-                    err = __shfl_sync(kFull, err, 0);
-                    if (!residual) ++fill;
+                    if (__any_sync(kFull, err)) err = DSBD_DEV_EXHAUSTED;
+                    else {
+                        n_out += n_draw;
+                        if (n_draw < want) err = DSBD_DEV_CAPACITY;
+                    }
+                } else if (!err) {
+                    const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 1u, 0u);
+                    int ia = 0;
+                    const int tok = draw_cell(a, sh, u, use_res, s_res, res_sums, lane, &ia);
+                    if (tok < 0) err = DSBD_DEV_EXHAUSTED;
+                    else if (n_out >= cap) err = DSBD_DEV_CAPACITY;
+                    else {
+                        if (lane == 0 && writer)
+                            emit_at(a, r, n_out, sh.A[ia], -1, tok, DSBD_SRC_RESIDUAL, cache, n_lo);
+                        ++n_out;
+                    }
                 }
                 if (lane == 0) {
                     sh.done = 1;
@@ -1732,9 +1732,10 @@ k_verify(VerifyArgs a) {
             for (int f = warp; f < n_draw; f += kVWarps) {
                 const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 2u, (uint32_t)f);
                 int ia = 0;
-                const int tok = draw_cell(a, sh, u, false, 0.f, 0.0, nullptr, lane, &ia);
+                const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, lane, &ia);
                 if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
-                else if (lane == 0 && writer) emit_at(a, r, base + f, sh.A[ia], -1, tok, DSBD_SRC_FILL);
+                else if (lane == 0 && writer)
+                    emit_at(a, r, base + f, sh.A[ia], -1, tok, DSBD_SRC_FILL, cached ? &nc : nullptr, n_lo);
             }
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -1773,9 +1774,10 @@ k_verify(VerifyArgs a) {
             const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1) + a.extra_layer_bias, 3u,
                                               (uint32_t)kk);
             int ia = 0;
-            const int tok = draw_cell(a, sh, u, false, 0.f, 0.0, nullptr, lane, &ia);
+            const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, lane, &ia);
             if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
-            else if (lane == 0 && writer) emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA);
+            else if (lane == 0 && writer)
+                emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
         }
         __syncthreads();
         if (!sh.err) {
@@ -1783,25 +1785,26 @@ k_verify(VerifyArgs a) {
             if (W_nom > n_draw && threadIdx.x == 0) sh.err = DSBD_DEV_CAPACITY;
         }
     } else if (extra && warp == 0) {
+        // independent draws from the support, one lane each
         int err = extra_err;
         if (writer && lane == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
-        for (int kk = 0; kk < W_nom && !err; ++kk) {
+        const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
+        const int n_draw = err ? 0 : min(W_nom, max(cap - n_out, 0));
+        for (int kk = lane; kk < n_draw; kk += 32) {
             const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1) + a.extra_layer_bias, 3u,
                                               (uint32_t)kk);
-            int ia = 0, tok;
-            if (a.top_k > 0) {
-                int pick = -1;
-                if (lane == 0) pick = draw_support(wsx, u, 0.0);
-                pick = __shfl_sync(kFull, pick, 0);
-                tok = -1;
-                if (pick >= 0) { ia = wsx.cell[0][pick] / a.V; tok = wsx.cell[0][pick] - ia * a.V; }
-            } else {
-                tok = draw_cell(a, sh, u, false, 0.f, 0.0, nullptr, lane, &ia);
+            const int pick = draw_support(wsx, u, 0.0);
+            if (pick < 0) { err = DSBD_DEV_EXHAUSTED; continue; }
+            const int ia = wsx.cell[0][pick] / a.V, tok = wsx.cell[0][pick] - ia * a.V;
+            if (writer)
+                emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
+        }
+        if (!extra_err) {
+            if (__any_sync(kFull, err)) err = DSBD_DEV_EXHAUSTED;
+            else {
+                n_out += n_draw;
+                if (n_draw < W_nom) err = DSBD_DEV_CAPACITY;
             }
-            if (tok < 0) { err = DSBD_DEV_EXHAUSTED; break; }
-            if (lane == 0) emit_output(a, r, &n_out, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, writer, &err);
-            n_out = __shfl_sync(kFull, n_out, 0);
-            err = __shfl_sync(kFull, err, 0);
         }
         if (lane == 0 && err) sh.err = err;
     }

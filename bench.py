@@ -300,7 +300,7 @@ def _side_workload(dsbd, inputs, dev, name, steps, warmup, top_k=0, top_p=1.0, p
 
 
 PHASE_NAMES = {1: "start", 2: "prologue / previous layer's completion", 3: "layer set-up", 4: "histogram pass",
-               5: "merge across the cluster", 6: "image into shared memory", 7: "suffix sums", 8: "residual chain",
+               5: "merge across the cluster", 7: "image and suffix sums", 8: "residual chain",
                9: "width and accept loop", 10: "residual pass for a completion draw", 11: "completion draws",
                12: "extra layer and final writes"}
 

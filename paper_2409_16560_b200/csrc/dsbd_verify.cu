@@ -95,6 +95,8 @@ k_tile_stats(const float *__restrict__ zp, const float *__restrict__ zq, int64_t
              const int32_t *__restrict__ n_rows_dev, float k2, TileStat *__restrict__ stats,
              int one_model = 0) {
     // one_model: zq is the same tensor as zp; read it once and store the statistics for both
+    // a kernel launched with programmatic stream serialization may be set up while the last blocks run
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -193,7 +195,8 @@ struct VerifyArgs {
     const double *lse;        // [2][N]
     const double *score;      // [2][N]
     const int32_t *depth;     // [N]
-    double *tile_sums;        // [R][2][max_m][max_live*T]
+    double *tile_sums;        // [R][2][max_m+1][max_live*T]: per bank the histogram pass's sums (half tiles may take
+                              // two slots), then those of the exact pass at j >= 2 in slot j
     unsigned long long *hist; // [R][2 banks][kBins+1] fixed-point ratio histograms (p<<32 | q)
     unsigned long long *dbg;  // phase time stamps (DSBD_PHASE_TIMING builds only)
     // verify mode computes the row and tree statistics of its own request first
@@ -224,8 +227,9 @@ struct Shared {
     int acc[kMaxLive];
     // log2 of (beam weight / sum of the row's exponentials), split so that the cell masses do not
     // inherit the rounding of one large float: bp/bq hold the nearest integer (exact in fp32), cp/cq
-    // the factor 2^(remainder) in [2^-0.5, 2^0.5], dc = log2(cp/cq)
-    float bp[kMaxLive], bq[kMaxLive], cp[kMaxLive], cq[kMaxLive], dc[kMaxLive];
+    // the factor 2^(remainder) in [2^-0.5, 2^0.5], rp/rq the remainders
+    float bp[kMaxLive], bq[kMaxLive], cp[kMaxLive], cq[kMaxLive];
+    double rp[kMaxLive], rq[kMaxLive];
     double lwp[kMaxLive], lwq[kMaxLive];    // natural log of the beam weights
     double wp[kMaxLive];
     double s_arr[kMaxLive + 2];             // s_0 .. s_m
@@ -234,13 +238,13 @@ struct Shared {
     double first[kMaxLive + 1];             // alpha_i prod_{j<i}(1-alpha_j)
     double col_a[kMaxLive + 1], col_b[kMaxLive + 1];
     double tail[kMaxLive + 2];
-    int bank, need_exact, res_j, run_j, chain_pos;
+    int bank, halves, need_exact, res_j, run_j, chain_pos;
     int n_out, n_fill;                      // output beams so far; p_beam fills left to the whole CTA
     int n_layers, n_tests, n_exact, n_respass;
     int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows consulted
     unsigned long long wtot_p[kVWarps], wtot_q[kVWarps];
     double n_cells;                         // cells that entered the layer's histogram
-    unsigned long long w_tot[10];           // sums of one histogram pass: see histogram_pass / hist_merge
+    unsigned long long w_tot[2][10];        // per bank, sums of one histogram pass: see histogram_pass / hist_fold_over
     int wrapped, n_wrapped;                 // a w word of the layer's histogram wrapped; layers where that happened
     double rho[kMaxLive], uu[kMaxLive];     // per live draft: p_beam/q_beam and its uniform
 };
@@ -262,6 +266,10 @@ __device__ __forceinline__ void split_offset(double b, float *bi, float *c, doub
     }
 }
 
+__device__ __forceinline__ RowOff row_off(const Shared &sh, int i) {
+    return RowOff{sh.bp[i], sh.bq[i], sh.cp[i], sh.cq[i], (float)(sh.rp[i] - sh.rq[i])};
+}
+
 // One cluster-wide pass: tile sums of max(p_beam - s q_beam, 0) over the live rows.
 __device__ void residual_pass(const VerifyArgs &a, const Shared &sh, float s, double *sums,
                               int cta_rank, int n_cta) {
@@ -275,7 +283,7 @@ __device__ void residual_pass(const VerifyArgs &a, const Shared &sh, float s, do
         const float *rp = a.zp + (int64_t)row * a.stride;
         const float *rq = a.zq + (int64_t)row * a.stride;
         const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
-        const RowOff ro = {sh.bp[i], sh.bq[i], sh.cp[i], sh.cq[i], sh.dc[i]};
+        const RowOff ro = row_off(sh, i);
         float acc = 0.f;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -393,7 +401,6 @@ struct NodeCache {
     uint8_t depth[kCacheNodes];
     uint8_t tree[kCacheNodes];            // tree of the node, inside the request
     int root[kMaxLive];                   // first node of every tree
-    int on;
 };
 
 // Writes output beam number `index` of request r (the caller has checked the slot range).  nc: the
@@ -440,21 +447,17 @@ __device__ __forceinline__ void log_softmax_warp(const double *s, int n, int lan
     __syncwarp();
 }
 
+// The weights of one model (0: p, 1: q) over the live set, by one warp; the two models' warps work side by side.
 // nc: the request's node cache or nullptr; n_lo: first node of the request.
-__device__ void live_weights(const VerifyArgs &a, Shared &sh, const double *sp, const double *sq, int lane,
-                             const NodeCache *nc = nullptr, int n_lo = 0) {
-    log_softmax_warp(sp, sh.nA, lane, sh.lwp);
-    log_softmax_warp(sq, sh.nA, lane, sh.lwq);
+__device__ void live_weights(const VerifyArgs &a, Shared &sh, int model, const double *scores, int lane,
+                             const NodeCache *nc, int n_lo) {
+    double *lw = model ? sh.lwq : sh.lwp;
+    log_softmax_warp(scores, sh.nA, lane, lw);
+    const double *lse = nc ? (model ? nc->lse_q : nc->lse_p) - n_lo : a.lse + (int64_t)model * a.N;
     for (int i = lane; i < sh.nA; i += 32) {
-        const double lwp = sh.lwp[i], lwq = sh.lwq[i];
-        sh.wp[i] = exp(lwp);
-        const int row = sh.A[i];
-        double rest_p, rest_q;
-        const double lse_p = nc ? nc->lse_p[row - n_lo] : a.lse[row];
-        const double lse_q = nc ? nc->lse_q[row - n_lo] : a.lse[a.N + row];
-        split_offset((lwp - lse_p) / kLn2, &sh.bp[i], &sh.cp[i], &rest_p);
-        split_offset((lwq - lse_q) / kLn2, &sh.bq[i], &sh.cq[i], &rest_q);
-        sh.dc[i] = (float)(rest_p - rest_q);
+        if (!model) sh.wp[i] = exp(lw[i]);
+        split_offset((lw[i] - lse[sh.A[i]]) * (1.0 / kLn2), model ? &sh.bq[i] : &sh.bp[i],
+                     model ? &sh.cq[i] : &sh.cp[i], model ? &sh.rq[i] : &sh.rp[i]);
     }
     __syncwarp();
 }
@@ -629,119 +632,128 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
 // One cluster-wide pass over the live rows; every CTA fills its own shared-memory histogram.
 // tot (shared memory, zero before the call): [0] what the CTA added to its w words (p and q).
 __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float binscale, const HistSmem &h,
-                               double *sums1, int cta_rank, int n_cta, unsigned long long *tot) {
+                               double *sums1, int cta_rank, int n_cta, int halves, unsigned long long *tot) {
+    // halves = 2: an item is a half tile (when the cluster has a warp for each), with a sum of its own
     const int lane = threadIdx.x & 31;
     const int warp = cta_rank * kVWarps + (threadIdx.x >> 5);
     const int nwarps = n_cta * kVWarps;
-    const int items = sh.nA * a.T;
+    const int items = sh.nA * a.T * halves;
     PassSums ps = {0ull};
     const uint32_t magic_bits = __float_as_uint(kBinMagic);
     const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(h.wp) - (magic_bits << 2);
     const uint32_t over_bits = magic_bits + (uint32_t)(kBins + ((threadIdx.x >> 5) & 15) * 16 + (threadIdx.x & 15));
     const float half_bin = 0.5f / binscale;                      // half a bin in log2 units
     const float top = (float)kBins / binscale - half_bin;        // log2 of the last edge (minus the half), as the bins see it
+    const int row_items = a.T * halves;
     for (int item = warp; item < items; item += nwarps) {
-        const int i = item / a.T, t = item - i * a.T;
+        const int i = item / row_items, t = item - i * row_items;
         const int row = sh.A[i];
         const float *rp = a.zp + (int64_t)row * a.stride;
         const float *rq = a.zq + (int64_t)row * a.stride;
         const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
-        const RowOff ro = {sh.bp[i], sh.bq[i], sh.cp[i], sh.cq[i], sh.dc[i]};
-        float res1u = 0.f;                               // sum of (p - q)+ over the tile in units: residual mass at s = 1
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
+        const RowOff ro = row_off(sh, i);
+        float res1u = 0.f;                               // sum of (p - q)+ over the item in units: residual mass at s = 1
+        int e0 = t * (kTile / halves);
+#pragma unroll 1
+        for (int half = halves; half < 3; ++half, e0 += kTile / 2) {
             float4 vp[4], vq[4];
-            const int e0 = t * kTile + half * (kTile / 2);
             load_half_tile(rp, e0, a.V, al, lane, vp);
             load_half_tile(rq, e0, a.V, al, lane, vq);
             hist_half_tile(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, res1u, ps, over_bits);
         }
-        // tile sums of the residual after ONE rejection (s_1 = 1): what a completion draw at run
+        // the items' sums of the residual after ONE rejection (s_1 = 1): what a completion draw at run
         // position 2 searches, so that this common case needs no second pass over the rows
         const double tot1 = warp_sum((double)res1u) * kUnfix;
         if (lane == 0) sums1[item] = tot1;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ps.tot += __shfl_xor_sync(kFull, ps.tot, o);
-    if (lane == 0 && ps.tot) atomicAdd(tot, ps.tot);
+    if (lane == 0 && ps.tot) atomicAdd(tot, ps.tot);         // (tot[0]: what the CTA's threads added to its w words)
 }
 
-// Merge of the cluster's histograms, after a cluster barrier that follows the pass: every CTA sums
-// one slice of the bins over all CTAs' shared memory (distributed shared memory loads, no atomics)
-// and stores the 64-bit sums, in units of 2^-44, to the global image, which therefore needs no
-// clearing; the last CTA also folds the copies of the last bin.  Returns through tot[9] whether
-// any CTA's w words wrapped (each CTA checks its own words against what its threads added, tot[0]).
-// The caller puts a cluster barrier behind this before anyone reads the image or reuses the arrays.
-__device__ void hist_check_local(const HistSmem &h, unsigned long long *tot, unsigned long long *warp_p,
-                                 unsigned long long *warp_q) {
-    unsigned long long sp = 0ull, sq = 0ull;
-    for (int i = threadIdx.x; i < kBins + kOverSlots; i += blockDim.x) { sp += h.wp[i]; sq += h.wq[i]; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        sp += __shfl_xor_sync(kFull, sp, o);
-        sq += __shfl_xor_sync(kFull, sq, o);
-    }
-    if ((threadIdx.x & 31) == 0) { warp_p[threadIdx.x >> 5] = sp; warp_q[threadIdx.x >> 5] = sq; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        sp = sq = 0ull;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { sp += warp_p[w]; sq += warp_q[w]; }
-        tot[6] = (tot[0] != sp + sq) ? 1ull : 0ull;               // a wrapped word lowers sp + sq by 2^32
-    }
-}
-
-__device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *gh,
-                           unsigned long long *tot, int cta_rank, int n_cta) {
-    const int per = (kBins + n_cta - 1) / n_cta;
-    const int lo = cta_rank * per, hi = min(lo + per, kBins);
-    for (int i = lo + (int)threadIdx.x; i < hi; i += blockDim.x) {
-        unsigned long long P = 0ull, Q = 0ull;
-        for (int c = 0; c < n_cta; ++c) {
-            const uint32_t *wp = cluster.map_shared_rank(h.wp, c), *wq = cluster.map_shared_rank(h.wq, c);
-            const uint32_t *bp = cluster.map_shared_rank(h.bp, c), *bq = cluster.map_shared_rank(h.bq, c);
-            P += ((unsigned long long)bp[i] << 16) + wp[i];
-            Q += ((unsigned long long)bq[i] << 16) + wq[i];
-        }
-        gh[2 * i] = P;
-        gh[2 * i + 1] = Q;
-    }
-    if (cta_rank == n_cta - 1) {
-        // the copies of the last bin (one per warp and half-warp lane, in every CTA) are one bin again
-        unsigned long long P = 0ull, Q = 0ull;
-        for (int i = kBins + (int)threadIdx.x; i < kBins + kOverSlots; i += blockDim.x)
-            for (int c = 0; c < n_cta; ++c) {
-                const uint32_t *wp = cluster.map_shared_rank(h.wp, c), *wq = cluster.map_shared_rank(h.wq, c);
-                const uint32_t *bp = cluster.map_shared_rank(h.bp, c), *bq = cluster.map_shared_rank(h.bq, c);
-                P += ((unsigned long long)bp[i] << 16) + wp[i];
-                Q += ((unsigned long long)bq[i] << 16) + wq[i];
-            }
+// The copies of the last bin (rho beyond the last edge), folded by each CTA and added to every CTA's total
+// (tot[7], tot[8]); before the cluster barrier that follows the pass.  Also tot[6] += what the CTA's threads
+// added to w words minus what these copies hold of it.
+__device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *tot, int n_cta) {
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < kOverSlots) {
+        const int i = kBins + (int)threadIdx.x;
+        unsigned long long w = (unsigned long long)h.wp[i] + h.wq[i];
+        unsigned long long P = ((unsigned long long)h.bp[i] << 16) + h.wp[i], Q = ((unsigned long long)h.bq[i] << 16) + h.wq[i];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
+            w += __shfl_xor_sync(kFull, w, o);
             P += __shfl_xor_sync(kFull, P, o);
             Q += __shfl_xor_sync(kFull, Q, o);
         }
-        if ((threadIdx.x & 31) == 0 && threadIdx.x < kOverSlots) {
-            if (P) atomicAdd(tot + 7, P);
-            if (Q) atomicAdd(tot + 8, Q);
+        if (threadIdx.x < 32) w -= tot[0];
+        if (lane < n_cta) {
+            unsigned long long *to = cluster.map_shared_rank(tot, lane);
+            if (w) atomicAdd(to + 6, 0ull - w);
+            if (P) atomicAdd(to + 7, P);
+            if (Q) atomicAdd(to + 8, Q);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) { gh[2 * kBins] = tot[7]; gh[2 * kBins + 1] = tot[8]; }
     }
-    if (threadIdx.x == 0) {
-        unsigned long long wrapped = 0ull;
-        for (int c = 0; c < n_cta; ++c) wrapped |= cluster.map_shared_rank(tot, c)[6];
-        tot[9] = wrapped;
+}
+
+// Merge of the cluster's histograms, after a cluster barrier that follows the pass: every CTA sums one slice of
+// the bins over all CTAs' shared memory (16-byte distributed shared memory loads, no atomics) and stores the
+// 64-bit sums, in units of 2^-44, to the global image, which therefore needs no clearing.  A lane takes four
+// bins of two CTAs, so that all its loads are in flight together; the lanes that share bins add up by shuffles
+// (bound by latency: two barriers and one round of remote loads, 6 us for 8 CTAs, 8 for 16; a thread that
+// walked all CTAs' words of one bin took 7 and 9, with a sweep for the wraps before the first barrier).
+// tot[6] of every CTA then holds what all threads added to w words minus what the words hold: zero unless a
+// word wrapped (a wrap lowers the words by 2^32).  The caller puts a cluster barrier behind this before
+// anyone reads the image or tot[6] or reuses the arrays.
+__device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *gh,
+                           unsigned long long *tot, int cta_rank, int n_cta) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int share = n_cta > 1 ? n_cta / 2 : 1;             // lanes that share four bins
+    const int quads = kBins / 4 / n_cta, per_warp = 32 / share;
+    unsigned long long wsum = 0ull;
+    for (int base = warp * per_warp; base < quads; base += kVWarps * per_warp) {
+        const int i = 4 * (cta_rank * quads + base + lane % per_warp);
+        unsigned long long P[4] = {}, Q[4] = {};
+        for (int c = lane / per_warp; c < n_cta; c += share) {
+            const uint4 wp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wp, c) + i);
+            const uint4 wq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wq, c) + i);
+            const uint4 bp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bp, c) + i);
+            const uint4 bq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bq, c) + i);
+            P[0] += ((unsigned long long)bp.x << 16) + wp.x; P[1] += ((unsigned long long)bp.y << 16) + wp.y;
+            P[2] += ((unsigned long long)bp.z << 16) + wp.z; P[3] += ((unsigned long long)bp.w << 16) + wp.w;
+            Q[0] += ((unsigned long long)bq.x << 16) + wq.x; Q[1] += ((unsigned long long)bq.y << 16) + wq.y;
+            Q[2] += ((unsigned long long)bq.z << 16) + wq.z; Q[3] += ((unsigned long long)bq.w << 16) + wq.w;
+            wsum += (unsigned long long)wp.x + wp.y + wp.z + wp.w;
+            wsum += (unsigned long long)wq.x + wq.y + wq.z + wq.w;
+        }
+        for (int o = per_warp; o < 32; o <<= 1) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                P[k] += __shfl_xor_sync(kFull, P[k], o);
+                Q[k] += __shfl_xor_sync(kFull, Q[k], o);
+            }
+        }
+        if (lane < per_warp) {
+            ulonglong2 *to = reinterpret_cast<ulonglong2 *>(gh + 2 * i);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) to[k] = make_ulonglong2(P[k], Q[k]);
+        }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(kFull, wsum, o);
+    if (lane < n_cta && wsum) atomicAdd(cluster.map_shared_rank(tot, lane) + 6, 0ull - wsum);
 }
 
 // One completion draw (residual if s_res > 0 else p_beam) by one warp; returns the token or -1
 // and the index of the live parent.
 __device__ int draw_cell(const VerifyArgs &a, const Shared &sh, double u, bool use_res, float s_res,
-                         const double *res_sums, int lane, int *ia_out) {
+                         const double *res_sums, int halves, int lane, int *ia_out) {
     int ia, t;
     double target;
     if (use_res) {
-        const int tile = locate_tile([&](int i) { return __ldcg(res_sums + i); }, sh.nA * a.T, u, true, lane, &target);
+        // (res_sums: one per tile, or two when the pass that wrote them worked on half tiles)
+        auto sum = [&](int i) { return halves == 1 ? __ldcg(res_sums + i) : __ldcg(res_sums + 2 * i) + __ldcg(res_sums + 2 * i + 1); };
+        const int tile = locate_tile(sum, sh.nA * a.T, u, true, lane, &target);
         if (tile < 0) return -1;
         ia = tile / a.T; t = tile - ia * a.T;
     } else {
@@ -759,7 +771,7 @@ __device__ int draw_cell(const VerifyArgs &a, const Shared &sh, double u, bool u
         if (t < 0) return -1;
     }
     *ia_out = ia;
-    const RowOff ro = {sh.bp[ia], sh.bq[ia], sh.cp[ia], sh.cq[ia], sh.dc[ia]};
+    const RowOff ro = row_off(sh, ia);
     const int64_t row = (int64_t)sh.A[ia] * a.stride;
     return locate_token(a.zp + row, a.zq + row, a.V, a.k2, t, ro, use_res ? s_res : 0.f, target, lane);
 }
@@ -1137,9 +1149,6 @@ k_verify(VerifyArgs a) {
     const HistSmem hs = hist_arrays(hp);
     unsigned long long *sufP = reinterpret_cast<unsigned long long *>(dyn_smem), *sufQ = sufP + kHistWords;
 
-    // launched with programmatic stream serialization: everything before this line overlaps the
-    // tail of the kernel ahead in the stream, nothing after it may run before that kernel is done
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int b_lo = a.req_beam_off[r], b_hi = a.req_beam_off[r + 1];
     const int n_lo = a.beam_node_off[b_lo], n_hi = a.beam_node_off[b_hi];
     int W_min = a.W_min_r ? a.W_min_r[r] : a.W_min;
@@ -1149,7 +1158,7 @@ k_verify(VerifyArgs a) {
     // reported (after the set-up below) and the request is not verified
     const bool bad_widths = a.check_widths && (W_min < 1 || W_max < W_min || W_nom < 1);
     if (bad_widths) { W_min = W_max = W_nom = 1; }
-    double *sums_base = a.tile_sums + (int64_t)r * 2 * a.max_m * ((int64_t)a.max_live * a.T);
+    double *sums_base = a.tile_sums + (int64_t)r * 2 * (a.max_m + 1) * ((int64_t)a.max_live * a.T);
     const int64_t slot_stride = (int64_t)a.max_live * a.T;
     unsigned long long *ghist = a.hist + (int64_t)r * 2 * kHistLen;        // [2 banks][kHistLen]
     const int hist_len = kHistLen;
@@ -1159,19 +1168,103 @@ k_verify(VerifyArgs a) {
 #endif
 
     TS(1);
+    // (a CTA may store into another's shared memory once that CTA runs: arrived here, waited for below)
+    if (threadIdx.x < 20) sh.w_tot[threadIdx.x / 10][threadIdx.x % 10] = 0ull;
+    cluster.barrier_arrive();
+    // Launched with programmatic stream serialization: everything before griddepcontrol.wait overlaps the tail of
+    // the dense pass ahead in the stream, whose grid started when all earlier work was done.  So what earlier
+    // kernels and the caller left may be read here, the tile statistics only after the wait.
+    const int n_req_nodes = n_hi - n_lo, n_trees = min(b_hi - b_lo, kMaxLive);
+    const bool cached = !a.select_mode && n_req_nodes <= kCacheNodes && a.gamma < 256;
     if (!a.select_mode) {
-        // ---- log-sum-exp of every row of the request from the dense pass's tile statistics ----
-        const int n_req = n_hi - n_lo;
+        const int n_req = n_req_nodes;
         const int cw = cta_rank * kVWarps + warp, ncw = n_cta * kVWarps;
+        // Small requests (as many nodes as the cache holds): every CTA of the cluster keeps the request's nodes in shared memory and computes all of
+        // their scores itself; the log-sum-exps, shared out over the cluster's warps, are stored into every
+        // CTA's copy.  One cluster barrier instead of three and no pass through global memory between them, and what
+        // the caller gave is read while the dense pass drains: 5.6 us instead of 8.5 (4 beams of 4 nodes, V = 32000),
+        // 9 instead of 15 with 84 nodes.  Node i is thread i's.
+        int par = -1, tok = -1;
+        float zp_tok = 0.f, zq_tok = 0.f;
+        if (cached) {
+            if ((int)threadIdx.x < n_trees) nc.root[threadIdx.x] = a.beam_node_off[b_lo + threadIdx.x];
+            const int i = threadIdx.x, n = n_lo + i;
+            if (i < n_req) {
+                par = a.parent[n];
+                if (par >= 0) {
+                    tok = a.token[n];
+                    if (par < n_lo || par >= n) { if (writer) report(a.status, DSBD_DEV_BAD_FOREST); tok = -2; }
+                    else if (tok < 0 || tok >= a.V) { if (writer) report(a.status, DSBD_DEV_BAD_TOKEN); tok = -2; }
+                    else {
+                        zp_tok = a.zp[(int64_t)par * a.stride + tok];
+                        zq_tok = a.zq[(int64_t)par * a.stride + tok];
+                    }
+                }
+                nc.parent[i] = (int16_t)((par >= n_lo && par < n) ? par - n_lo : -1);
+            }
+        }
+        cluster.barrier_wait();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        // ---- log-sum-exp of every row of the request from the dense pass's tile statistics ----
         for (int task = cw; task < 2 * n_req; task += ncw) {
             const int model = task / n_req, row = n_lo + (task - model * n_req);
             const double v = row_lse(a.stats + ((int64_t)model * a.N + row) * a.T, a.T, a.inv_tau, lane);
+            if (cached && lane < n_cta)
+                cluster.map_shared_rank(model ? nc.lse_q : nc.lse_p, lane)[row - n_lo] = v;
             if (lane == 0) {
                 a.lse_w[(int64_t)model * a.N + row] = v;
                 float *o = model ? a.out.lse_q : a.out.lse_p;
                 if (o) o[row] = (float)v;
             }
         }
+        if (cached) {
+            cluster.sync();
+            // ---- log-prob of every draft token given its parent, then every node sums its path to the root ----
+            double *slp = reinterpret_cast<double *>(hp), *slq = slp + kCacheNodes;     // (the histogram arrays are idle)
+            const int i = threadIdx.x;
+            if (i < n_req) {
+                double lp = 0.0, lq = 0.0;
+                if (tok == -2) lp = lq = -INFINITY;
+                else if (tok >= 0) {
+                    lp = (double)zp_tok * a.inv_tau - nc.lse_p[par - n_lo];
+                    lq = (double)zq_tok * a.inv_tau - nc.lse_q[par - n_lo];
+                }
+                slp[i] = lp; slq[i] = lq;
+            }
+            __syncthreads();
+            if (i < b_hi - b_lo && a.beam_node_off[b_lo + i] < n_hi) {
+                const int root = a.beam_node_off[b_lo + i];
+                if (writer && a.parent[root] != -1) report(a.status, DSBD_DEV_BAD_FOREST);
+                slp[root - n_lo] = (double)a.root_logp[b_lo + i];
+                slq[root - n_lo] = (double)a.root_logq[b_lo + i];
+            }
+            __syncthreads();
+            if (i < n_req) {
+                double sp = 0.0, sq = 0.0;
+                int dep = 0, cur = i;
+                while (true) {
+                    sp += slp[cur];
+                    sq += slq[cur];
+                    const int up = nc.parent[cur];
+                    if (up < 0) break;                                       // root or malformed
+                    cur = up;
+                    if (++dep > a.gamma) { if (writer) report(a.status, DSBD_DEV_BAD_FOREST); break; }
+                }
+                nc.score_p[i] = sp; nc.score_q[i] = sq;
+                nc.depth[i] = (uint8_t)min(dep, 255);
+                int tree = 0;
+                while (tree + 1 < n_trees && nc.root[tree + 1] <= n_lo + i) ++tree;
+                nc.tree[i] = (uint8_t)tree;
+                if (writer) {
+                    a.score_w[n_lo + i] = sp;
+                    a.score_w[a.N + n_lo + i] = sq;
+                    a.depth_w[n_lo + i] = dep;
+                    if (a.out.node_logp) a.out.node_logp[n_lo + i] = (float)sp;
+                    if (a.out.node_logq) a.out.node_logq[n_lo + i] = (float)sq;
+                }
+            }
+            __syncthreads();
+        } else {
         __threadfence();
         cluster.sync();
         // ---- log-prob of every draft token given its parent (all nodes at once) ----
@@ -1263,6 +1356,10 @@ k_verify(VerifyArgs a) {
         }
         __threadfence();
         cluster.sync();
+        }
+    } else {
+        cluster.barrier_wait();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
     }
 
     // ---- set-up ----
@@ -1290,56 +1387,63 @@ k_verify(VerifyArgs a) {
             } else {
                 sh.nA = b_hi - b_lo;
                 if (sh.nA > kMaxLive) { sh.err = DSBD_DEV_BAD_FOREST; sh.nA = 0; }
-                for (int i = 0; i < sh.nA; ++i) {
-                    sh.A[i] = a.beam_node_off[b_lo + i];
-                    sp_live[i] = a.score[sh.A[i]];
-                    sq_live[i] = a.score[a.N + sh.A[i]];
-                }
-                if (writer) {
-                    for (int l = 0; l <= a.gamma; ++l) a.out.layer_width[(int64_t)r * (a.gamma + 1) + l] = -1;
-                    a.out.l_last[r] = a.gamma + 1;
-                    a.out.out_width[r] = 0;
-                }
+            }
+        }
+        __syncwarp();
+        if (!a.select_mode) {
+            for (int i = lane; i < sh.nA; i += 32) {
+                const int root = a.beam_node_off[b_lo + i];
+                sh.A[i] = root;
+                sp_live[i] = cached ? nc.score_p[root - n_lo] : a.score[root];
+                sq_live[i] = cached ? nc.score_q[root - n_lo] : a.score[a.N + root];
+            }
+            if (writer) {
+                for (int l = lane; l <= a.gamma; l += 32) a.out.layer_width[(int64_t)r * (a.gamma + 1) + l] = -1;
+                if (lane == 0) { a.out.l_last[r] = a.gamma + 1; a.out.out_width[r] = 0; }
             }
         }
         __syncwarp();
         if (!a.select_mode && writer)
             for (int n = n_lo + lane; n < n_hi; n += 32)
-                a.out.node_status[n] = a.parent[n] < 0 ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+                a.out.node_status[n] = (cached ? nc.parent[n - n_lo] : a.parent[n]) < 0 ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     }
     // Every CTA of the cluster takes identical decisions from identical data, so each keeps its
     // own copy of the node statuses and only rank 0 writes results.
-    const int n_trees = min(b_hi - b_lo, kMaxLive);
-    if (!a.select_mode && (int)threadIdx.x < n_trees) nc.root[threadIdx.x] = a.beam_node_off[b_lo + threadIdx.x];
     const int n_layers = a.select_mode ? 1 : a.gamma;
-    const int n_req_nodes = n_hi - n_lo;
     const bool st_ok = n_req_nodes <= kMaxLive * kMaxLive;
     if (!a.select_mode)
         for (int n = threadIdx.x; n < n_req_nodes && st_ok; n += blockDim.x)
-            st[n] = a.parent[n_lo + n] < 0 ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
-    __threadfence();
-    cluster.sync();
+            st[n] = (cached ? nc.parent[n] : a.parent[n_lo + n]) < 0 ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+    __syncthreads();
     if (!a.select_mode && !st_ok && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
     if (bad_widths && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_PARAM;
-    const bool cached = !a.select_mode && n_req_nodes <= kCacheNodes && a.gamma < 256;
-    if (threadIdx.x == 0) nc.on = cached ? 1 : 0;
-    if (cached)
-        for (int i = threadIdx.x; i < n_req_nodes; i += blockDim.x) {
-            const int n = n_lo + i, par = a.parent[n];
-            nc.score_p[i] = a.score[n];   nc.score_q[i] = a.score[a.N + n];
-            nc.lse_p[i] = a.lse[n];       nc.lse_q[i] = a.lse[a.N + n];
-            nc.parent[i] = (int16_t)((par >= n_lo && par < n) ? par - n_lo : -1);
-            nc.depth[i] = (uint8_t)min(max(a.depth[n], 0), 255);
-            int tree = 0;
-            while (tree + 1 < n_trees && nc.root[tree + 1] <= n) ++tree;
-            nc.tree[i] = (uint8_t)tree;
-        }
     __syncthreads();
     // node data by local index, from the cache when there is one
     auto nd_depth = [&](int i) -> int { return cached ? (int)nc.depth[i] : a.depth[n_lo + i]; };
     auto nd_parent = [&](int i) -> int { return cached ? (int)nc.parent[i] : a.parent[n_lo + i] - n_lo; };
     auto nd_score = [&](int model, int i) -> double {
         return cached ? (model ? nc.score_q[i] : nc.score_p[i]) : a.score[(int64_t)model * a.N + n_lo + i];
+    };
+
+    // per live draft of layer l: index of its parent in A, rho = p_beam/q_beam of its cell, its uniform (one warp)
+    auto draft_tests = [&](int l, int m) {
+        for (int i = lane; i < m; i += 32) {
+            const int n = sh.S[i];
+            const int pl = nd_parent(n - n_lo), par = n_lo + pl;
+            int ai = 0;
+            while (ai < sh.nA && sh.A[ai] != par) ++ai;
+            sh.S_parent_idx[i] = ai;
+            const double lp = nd_score(0, n - n_lo) - nd_score(0, pl);
+            const double lq = nd_score(1, n - n_lo) - nd_score(1, pl);
+            double rho;
+            if (lq == -INFINITY || sh.lwq[ai] == -INFINITY)
+                rho = (lp > -INFINITY && sh.lwp[ai] > -INFINITY) ? INFINITY : 0.0;
+            else
+                rho = exp((sh.lwp[ai] - sh.lwq[ai]) + (lp - lq));
+            sh.rho[i] = rho;
+            sh.uu[i] = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 0u, (uint32_t)i);
+        }
+        __syncwarp();
     };
 
     for (int l = 1; l <= n_layers && !sh.done && !sh.err; ++l) {
@@ -1369,19 +1473,21 @@ k_verify(VerifyArgs a) {
                 }
                 if (m > kMaxLive) { if (lane == 0) sh.err = DSBD_DEV_BAD_FOREST; m = 0; }
                 __syncwarp();
-                if (lane == 0 && a.draft_rank) {
-                    // insertion sort by (draft_rank, node id); ids are already ascending
-                    for (int i = 1; i < m; ++i) {
-                        const int n = sh.S[i];
-                        const int key = a.draft_rank[n];
-                        int j = i - 1;
-                        while (j >= 0 && a.draft_rank[sh.S[j]] > key) { sh.S[j + 1] = sh.S[j]; --j; }
-                        sh.S[j + 1] = n;
+                if (a.draft_rank) {
+                    // order of (draft_rank, node id), ids being ascending: a draft's place is the number before it
+                    for (int i = lane; i < m; i += 32) sh.S_parent_idx[i] = a.draft_rank[sh.S[i]];
+                    __syncwarp();
+                    for (int i = lane; i < m; i += 32) {
+                        const int key = sh.S_parent_idx[i];
+                        int place = 0;
+                        for (int j = 0; j < m; ++j) place += sh.S_parent_idx[j] < key + (j < i);
+                        sh.acc[place] = sh.S[i];
                     }
+                    __syncwarp();
+                    for (int i = lane; i < m; i += 32) sh.S[i] = sh.acc[i];
                 }
             }
             __syncwarp();
-            live_weights(a, sh, sp_live, sq_live, lane, cached ? &nc : nullptr, n_lo);
             if (lane == 0) {
                 sh.m = m;
                 sh.s_arr[0] = 0.0;
@@ -1389,28 +1495,12 @@ k_verify(VerifyArgs a) {
                 sh.chain_len = 0;          // c_{j+1} is known for j = 1..chain_len
                 sh.bank = l & 1;
             }
-            // per live draft: index of its parent in A, rho = p_beam/q_beam of its cell, its uniform
-            if (!a.select_mode)
-                for (int i = lane; i < m; i += 32) {
-                    const int n = sh.S[i];
-                    const int pl = nd_parent(n - n_lo), par = n_lo + pl;
-                    int ai = 0;
-                    while (ai < sh.nA && sh.A[ai] != par) ++ai;
-                    sh.S_parent_idx[i] = ai;
-                    const double lp = nd_score(0, n - n_lo) - nd_score(0, pl);
-                    const double lq = nd_score(1, n - n_lo) - nd_score(1, pl);
-                    double rho;
-                    if (lq == -INFINITY || sh.lwq[ai] == -INFINITY)
-                        rho = (lp > -INFINITY && sh.lwp[ai] > -INFINITY) ? INFINITY : 0.0;
-                    else
-                        rho = exp((sh.lwp[ai] - sh.lwq[ai]) + (lp - lq));
-                    sh.rho[i] = rho;
-                    sh.uu[i] = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 0u, (uint32_t)i);
-                }
+        } else if (warp <= 2) {
+            live_weights(a, sh, warp - 1, warp == 1 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
+        } else {
+            uint4 *words = reinterpret_cast<uint4 *>(hp);
+            for (int i = threadIdx.x - 96; i < kHistArrays * kHistWords / 4; i += kVThreads - 96) words[i] = make_uint4(0, 0, 0, 0);
         }
-        for (int i = threadIdx.x; i < kHistArrays * kHistWords; i += blockDim.x) hp[i] = 0u;
-        if (threadIdx.x < 10) sh.w_tot[threadIdx.x] = 0ull;
-        if (threadIdx.x == 0) sh.wrapped = 0;
         __syncthreads();
         const int m = sh.m;
         TS(3);
@@ -1430,12 +1520,14 @@ k_verify(VerifyArgs a) {
                 else if (warp == 0) {
                     finish_supports(wsup, true, lane);
                     // rho of every live draft from the warped joints
-                    if (!a.select_mode)
+                    if (!a.select_mode) {
+                        draft_tests(l, m);
                         for (int i = lane; i < m; i += 32) {
                             const int cell = sh.S_parent_idx[i] * a.V + a.token[sh.S[i]];
                             const double pw = support_lookup(wsup, 0, cell), qw = support_lookup(wsup, 1, cell);
                             sh.rho[i] = qw > 0.0 ? pw / qw : (pw > 0.0 ? INFINITY : 0.0);
                         }
+                    }
                     // c_{j+1} = F(s_j) over the p support, lanes over cells
                     // (every lane keeps its at most two cells and the running s, c in registers)
                     const int ns = wsup.n[0];
@@ -1462,34 +1554,36 @@ k_verify(VerifyArgs a) {
             const double top = log2((double)(m > 2 ? m : 2));          // s_j <= j <= m
             const float binscale = (float)((double)kBins / top);
             unsigned long long *gh = ghist + sh.bank * hist_len;
-            histogram_pass(a, sh, binscale, hs, sums_base + ((int64_t)sh.bank * a.max_m) * slot_stride, cta_rank,
-                           n_cta, sh.w_tot);
+            unsigned long long *tot = sh.w_tot[sh.bank];
+            // half tiles as items where whole ones would leave a part of the last round's warps idle: a warp's own
+            // work is the pass's length there (V = 32000, 16 CTAs: 3 rows 4.5 us instead of 7)
+            const int tiles = sh.nA * a.T, nw = n_cta * kVWarps;
+            const int halves = (2 * tiles + nw - 1) / nw < 2 * ((tiles + nw - 1) / nw) ? 2 : 1;
+            histogram_pass(a, sh, binscale, hs, sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride, cta_rank,
+                           n_cta, halves, tot);
             __syncthreads();
-            hist_check_local(hs, sh.w_tot, sh.wtot_p, sh.wtot_q);
+            hist_fold_over(cluster, hs, tot, n_cta);
             TS(4);
             cluster.sync();                            // every CTA's histogram is complete
-            hist_merge(cluster, hs, gh, sh.w_tot, cta_rank, n_cta);
+            if (threadIdx.x < 10) sh.w_tot[sh.bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
+                                                       // the barrier below
+            hist_merge(cluster, hs, gh, tot, cta_rank, n_cta);
             cluster.sync();                            // the image is whole (the barrier orders the stores for
                                                        // the cluster); nobody reads the arrays any more
             TS(5);
-            // the merged histogram into shared memory (over the building arrays)
-            for (int i = threadIdx.x; i <= kBins; i += blockDim.x) {
-                sufP[i] = __ldcg(gh + 2 * i);
-                sufQ[i] = __ldcg(gh + 2 * i + 1);
-            }
-            if (threadIdx.x == 0) {
-                sh.n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
-                sh.wrapped = sh.w_tot[9] != 0ull;
-                if (sh.wrapped) ++sh.n_wrapped;
-            }
-            __syncthreads();
-            TS(6);
-            // in-place suffix sums: sufP[k] = p mass of the bins >= k (17 bins per thread)
+            // Suffix sums of the merged histogram into shared memory (over the building arrays): sufP[k] = p mass of
+            // the bins >= k.  A thread takes kPer consecutive bins in registers from the image to the sums, two bins a
+            // load (3.6 us; image, then sums in place through shared memory, took 3.8 to 4.5).
             {
-                constexpr int per = (kBins + 1 + kVThreads - 1) / kVThreads;
-                const int lo = min((int)threadIdx.x * per, kBins + 1), hi = min(lo + per, kBins + 1);
-                unsigned long long mp_ = 0ull, mq_ = 0ull;
-                for (int i = lo; i < hi; ++i) { mp_ += sufP[i]; mq_ += sufQ[i]; }
+                constexpr int kPer = kBins / kVThreads;
+                unsigned long long bp_[kPer], bq_[kPer], mp_ = 0ull, mq_ = 0ull;
+                const unsigned long long *src = gh + 2 * kPer * threadIdx.x;
+#pragma unroll
+                for (int i = 0; i < kPer; i += 2)
+                    asm volatile("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+                                 : "=l"(bp_[i]), "=l"(bq_[i]), "=l"(bp_[i + 1]), "=l"(bq_[i + 1]) : "l"(src + 2 * i) : "memory");
+#pragma unroll
+                for (int i = 0; i < kPer; ++i) { mp_ += bp_[i]; mq_ += bq_[i]; }
                 unsigned long long ap = mp_, aq = mq_;    // suffix scan inside the warp, top lane down
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -1497,16 +1591,32 @@ k_verify(VerifyArgs a) {
                     if (lane + o < 32) { ap += tp; aq += tq; }
                 }
                 if (lane == 0) { sh.wtot_p[warp] = ap; sh.wtot_q[warp] = aq; }
-                __syncthreads();
-                unsigned long long rp_ = ap - mp_, rq_ = aq - mq_;  // mass of the lanes above in this warp
-                for (int w = warp + 1; w < kVWarps; ++w) { rp_ += sh.wtot_p[w]; rq_ += sh.wtot_q[w]; }
-                for (int i = hi - 1; i >= lo; --i) {
-                    rp_ += sufP[i]; rq_ += sufQ[i];
-                    sufP[i] = rp_; sufQ[i] = rq_;
+                if (threadIdx.x == 0) {
+                    sh.n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
+                    sh.wrapped = tot[6] != 0ull;
+                    sh.halves = halves;
+                    if (sh.wrapped) ++sh.n_wrapped;
                 }
-                if (threadIdx.x == 0) { sufP[kBins + 1] = 0ull; sufQ[kBins + 1] = 0ull; }
+                __syncthreads();
+                unsigned long long rp_ = ap - mp_ + tot[7], rq_ = aq - mq_ + tot[8];  // bins above this thread's
+                for (int w = warp + 1; w < kVWarps; ++w) { rp_ += sh.wtot_p[w]; rq_ += sh.wtot_q[w]; }
+#pragma unroll
+                for (int i = kPer - 1; i >= 0; --i) {
+                    rp_ += bp_[i]; rq_ += bq_[i];
+                    bp_[i] = rp_; bq_[i] = rq_;
+                }
+#pragma unroll
+                for (int i = 0; i < kPer; i += 2) {
+                    *reinterpret_cast<ulonglong2 *>(sufP + kPer * threadIdx.x + i) = make_ulonglong2(bp_[i], bp_[i + 1]);
+                    *reinterpret_cast<ulonglong2 *>(sufQ + kPer * threadIdx.x + i) = make_ulonglong2(bq_[i], bq_[i + 1]);
+                }
+                if (threadIdx.x == 0) {
+                    sufP[kBins] = tot[7]; sufQ[kBins] = tot[8];
+                    sufP[kBins + 1] = 0ull; sufQ[kBins + 1] = 0ull;
+                }
             }
             __syncthreads();
+            if (warp == 1 && !a.select_mode) draft_tests(l, m);
 
             TS(7);
             int j0 = 1;
@@ -1526,7 +1636,9 @@ k_verify(VerifyArgs a) {
                             c_next = ((double)sufP[0] - (double)sufQ[0]) * kUnfix;
                             if (fix_err > kErrTol) { need = 1; break; }
                         } else {
-                            int k = (int)(log2(s_j) * (double)binscale);
+                            // (a float's logarithm can miss the bin only within 3e-7 of an edge; the bracket below
+                            // takes the edges 2e-6 wider)
+                            int k = (int)(log2f((float)s_j) * binscale);
                             if (k < 0) k = 0;
                             if (k >= kBins) { need = 1; break; }      // cannot happen for s_j <= m
                             const double Pa = (double)sufP[k + 1] * kUnfix, Qa = (double)sufQ[k + 1] * kUnfix;
@@ -1552,7 +1664,9 @@ k_verify(VerifyArgs a) {
                 if (!sh.need_exact) break;
                 const int j = sh.chain_pos;
                 if (threadIdx.x == 0) ++sh.n_exact;
-                double *sums = sums_base + ((int64_t)sh.bank * a.max_m + (j - 1)) * slot_stride;
+                // (at j = 1 these are the sums that the histogram pass left in slot 0)
+                double *sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride;
+                if (j == 1 && threadIdx.x == 0) sh.halves = 1;
                 residual_pass(a, sh, (float)sh.s_arr[j], sums, cta_rank, n_cta);
                 __threadfence();
                 cluster.sync();
@@ -1641,9 +1755,9 @@ k_verify(VerifyArgs a) {
 
         TS(9);
         // ---- a residual draw locates its tile through tile sums of max(p_beam - s_{j-1} q_beam, 0) ----
-        double *res_sums = sums_base + ((int64_t)sh.bank * a.max_m) * slot_stride;   // slot 0 of the bank
+        double *res_sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride;   // slot 0 of the bank
         if (!a.select_mode && !sh.err && !warped && sh.res_j > 2) {   // run position 2 is served by the histogram pass
-            if (threadIdx.x == 0) ++sh.n_respass;
+            if (threadIdx.x == 0) { ++sh.n_respass; sh.halves = 1; }
             residual_pass(a, sh, (float)sh.s_arr[sh.res_j - 1], res_sums, cta_rank, n_cta);
             __threadfence();
             cluster.sync();
@@ -1655,9 +1769,8 @@ k_verify(VerifyArgs a) {
             const int W = sh.W, count = sh.count, j = sh.run_j;
             int err = 0;
             if (count < W) {
-                // accepted drafts, then the residual draw, then fills from p_beam: warp 0 makes the residual draw
-                // (lane 0 when the joint is warped), the other outputs are independent of one another and
-                // spread over lanes or, for unwarped fills, over the warps of the CTA
+                // accepted drafts, then the residual draw, then fills from p_beam, all independent of one another:
+                // spread over lanes when the joint is warped, else over the warps of the CTA (below)
                 const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
                 const NodeCache *cache = cached ? &nc : nullptr;
                 const int n_acc = min(count, max(cap - n_out, 0));
@@ -1668,7 +1781,6 @@ k_verify(VerifyArgs a) {
                 n_out += n_acc;
                 if (n_acc < count) err = DSBD_DEV_CAPACITY;
                 const bool use_res = j > 1;
-                const float s_res = use_res ? (float)sh.s_arr[j - 1] : 0.f;
                 if (warped && !err) {
                     const int want = W - count, n_draw = min(want, max(cap - n_out, 0));
                     for (int kk = lane; kk < n_draw; kk += 32) {
@@ -1685,23 +1797,12 @@ k_verify(VerifyArgs a) {
                         n_out += n_draw;
                         if (n_draw < want) err = DSBD_DEV_CAPACITY;
                     }
-                } else if (!err) {
-                    const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 1u, 0u);
-                    int ia = 0;
-                    const int tok = draw_cell(a, sh, u, use_res, s_res, res_sums, lane, &ia);
-                    if (tok < 0) err = DSBD_DEV_EXHAUSTED;
-                    else if (n_out >= cap) err = DSBD_DEV_CAPACITY;
-                    else {
-                        if (lane == 0 && writer)
-                            emit_at(a, r, n_out, sh.A[ia], -1, tok, DSBD_SRC_RESIDUAL, cache, n_lo);
-                        ++n_out;
-                    }
                 }
                 if (lane == 0) {
                     sh.done = 1;
                     if (writer) a.out.l_last[r] = l;
                     sh.n_out = n_out;
-                    sh.n_fill = (!warped && !err) ? W - count - 1 : 0;
+                    sh.n_fill = (!warped && !err) ? W - count : 0;
                 }
             } else {
                 // the accepted drafts, ascending node id, are the next layer's input beams
@@ -1724,18 +1825,20 @@ k_verify(VerifyArgs a) {
         }
         __syncthreads();
         if (!a.select_mode && sh.done && sh.n_fill > 0 && !sh.err) {
-            // fill f is output beam n_out + f, drawn from p_beam with its own uniform
+            // draw f is output beam n_out + f: the residual draw at the run position where the layer ended, then the
+            // fills from p_beam, each with its own uniform
             const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
-            const int base = sh.n_out, want = sh.n_fill;
+            const int base = sh.n_out, want = sh.n_fill, j = sh.run_j;
             const int n_draw = min(want, max(cap - base, 0));
             __syncthreads();
             for (int f = warp; f < n_draw; f += kVWarps) {
-                const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 2u, (uint32_t)f);
+                const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, f ? 2u : 1u, f ? (uint32_t)(f - 1) : 0u);
+                const bool use_res = f == 0 && j > 1;
                 int ia = 0;
-                const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, lane, &ia);
+                const int tok = draw_cell(a, sh, u, use_res, use_res ? (float)sh.s_arr[j - 1] : 0.f, res_sums, sh.halves, lane, &ia);
                 if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
                 else if (lane == 0 && writer)
-                    emit_at(a, r, base + f, sh.A[ia], -1, tok, DSBD_SRC_FILL, cached ? &nc : nullptr, n_lo);
+                    emit_at(a, r, base + f, sh.A[ia], -1, tok, f ? DSBD_SRC_FILL : DSBD_SRC_RESIDUAL, cached ? &nc : nullptr, n_lo);
             }
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -1753,7 +1856,7 @@ k_verify(VerifyArgs a) {
     WarpScratch &wsx = *reinterpret_cast<WarpScratch *>(hq);
     int extra_err = 0;
     if (extra) {
-        if (warp == 0) live_weights(a, sh, sp_live, sq_live, lane);
+        if (warp < 2) live_weights(a, sh, warp, warp == 0 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
         __syncthreads();
         if (a.top_k > 0) {
             if (warp < kHalf / 32) {                            // one model only: the first half builds it
@@ -1774,7 +1877,7 @@ k_verify(VerifyArgs a) {
             const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1) + a.extra_layer_bias, 3u,
                                               (uint32_t)kk);
             int ia = 0;
-            const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, lane, &ia);
+            const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, 1, lane, &ia);
             if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
             else if (lane == 0 && writer)
                 emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
@@ -1842,7 +1945,7 @@ Layout make_layout(const dsbd_forest_t *f, int V) {
     L.score = off; off = align_up(off + sizeof(double) * 2 * (size_t)f->N, 256);
     L.depth = off; off = align_up(off + sizeof(int32_t) * (size_t)f->N, 256);
     L.sums = off;
-    off = align_up(off + sizeof(double) * (size_t)f->R * 2 * L.max_m * (size_t)L.max_live * L.T, 256);
+    off = align_up(off + sizeof(double) * (size_t)f->R * 2 * (L.max_m + 1) * (size_t)L.max_live * L.T, 256);
     L.hist = off;
     off = align_up(off + sizeof(unsigned long long) * (size_t)f->R * 2 * kHistLen, 256);
 #ifdef DSBD_PHASE_TIMING

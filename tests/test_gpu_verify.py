@@ -78,9 +78,9 @@ def test_c5_all_requests(top_k, top_p):
     check_exempt(exempt, decisions)
 
 
-def _random_problem(rng, R, V, gamma, max_w, stride_pad=0, ninf_frac=0.0, tree="chain"):
+def _random_problem(rng, R, V, gamma, max_w, stride_pad=0, ninf_frac=0.0, tree="chain", min_w=1):
     widths = rng.integers(1, max_w + 1, size=R)
-    spec = dict(R=R, W=(1, max_w), tree=inputs._chain(gamma) if tree == "chain" else inputs._binary(gamma),
+    spec = dict(R=R, W=(min_w, max_w), tree=inputs._chain(gamma) if tree == "chain" else inputs._binary(gamma),
                 prefix=(1, 1))
     forest, widths, _ = inputs.build_forest(spec, rng)
     N, B = forest["N"], forest["B"]
@@ -302,6 +302,27 @@ def test_top_k_near_the_number_of_tiles(V, top_k):
             assert np.array_equal(again[k], gpu[k]), k
     ref = _oracle(forest, prm, zp, zq, rp, rq)
     check_exempt(*compare_verify(ref, gpu, forest))
+
+
+@pytest.mark.parametrize("beams,gamma,V", [(15, 16, 512), (16, 15, 513), (16, 15, 1500), (6, 42, 700)])
+def test_requests_around_the_node_cache_and_half_tiles(beams, gamma, V):
+    """255, 256 and 258 nodes in a request (up to 256 are kept in every CTA's shared memory), at
+    vocabularies where the histogram pass takes half tiles (one row tile, its second half empty, with one
+    token, ragged) and where it takes whole ones; completion draws at every run position."""
+    rng = np.random.default_rng(V)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=3, V=V, gamma=gamma, max_w=beams, min_w=beams)
+    assert forest["N"] == 3 * beams * (gamma + 1)
+    forest["draft_rank"] = rng.integers(0, 4, forest["N"]).astype(np.int32)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = 0
+    for step in range(20):
+        prm.update(step=step, thresh=0.3 + 0.03 * step)
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+    check_exempt(exempt, decisions)
 
 
 def test_roots_only_forest_goes_straight_to_the_extra_layer():

@@ -523,9 +523,9 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
 //      overflow because a joint distribution sums to one.
 // A w word wraps once the small cells of ONE bin that ONE CTA added reach 2^-12 of the mass --
 // twenty times what a bin holds in ordinary data, but possible when the two models' rows are
-// proportional and every cell lands in the same bin.  A wrap is detected exactly: every thread
-// keeps the 64-bit total of what it added to the w words, and the CTA compares the sum of those
-// totals with the sum of its w words; a difference marks the layer, whose residual masses are
+// proportional and every cell lands in the same bin.  A wrap is always detected: every thread
+// keeps a total of the mass that it added, and the sum of those totals is compared with the sum of
+// all words; a difference marks the layer, whose residual masses are
 // then all computed by exact passes over the rows.
 // ---------------------------------------------------------------------------------------
 constexpr int kBins = 4096;
@@ -535,8 +535,6 @@ constexpr int kHistWords = kBins + kOverSlots + 16;  // bins 0..kBins-1, the cop
 static_assert(kHistWords % 4 == 0, "the arrays that share this memory need 16-byte alignment");
 constexpr float kFix = 17592186044416.f;          // 2^44
 constexpr double kUnfix = 1.0 / 17592186044416.0;
-constexpr float kBigCell = 1.f / 65536.f;         // 2^-16: cells from here on put their top part into the b word
-constexpr float kBigFix = 268435456.f;            // 2^28, the unit of the b word is 2^-28
 constexpr double kErrTol = 2.5e-7;                // error bound of F(s) above which it is recomputed exactly
 // global image of one histogram: P and Q of bin i at 2i, 2i+1 (units of 2^-44), two spare words
 constexpr int kHistLen = 2 * (kBins + 1) + 2;
@@ -554,19 +552,39 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// Per-thread sums of one histogram pass.
-struct PassSums {
-    unsigned long long tot;               // what went into the w words (p and q together)
-};
+// Two fp32 values in one 64-bit register: an instruction does both (rounding as the plain ones).
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    return v;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 
-// The cells of one half tile (4 x float4 per lane and model) into the histogram; adds their
-// (p - q)+, in units of 2^-44, to res1u.
+// The cells of one half tile (4 x float4 per lane and model) into the histogram; adds the p and the q mass of
+// its cells with p_beam > q_beam, in units of 2^-44, to sp and sq.
 // The work per cell decides the speed of this pass (it is bound by instruction issue, not by
-// memory), so the common case is straight-line code: masses are computed directly in units
-// (the row's factor 2^rest carries the 2^44), the bin comes from an fma onto 1.5 * 2^23 whose
-// low mantissa bits are then the integer (no conversion instruction), the two atomic adds, the
-// residual sum and the check sum are predicated on p_beam > q_beam inside one asm block, and only a
-// cell of at least 2^-16 (rare) takes a branch.
+// memory), so the common case is straight-line code, two cells to a packed instruction up to the exponentials:
+// masses are computed directly in units (the row's factor 2^rest carries the 2^44), the bin comes from an fma
+// onto 1.5 * 2^23 whose low mantissa bits are then the integer (no conversion instruction), the two atomic adds
+// and the two sums are predicated on p_beam > q_beam inside one asm block, and only cells
+// of at least 2^-16 take a branch, one for four cells.  (64 requests x 8 rows of 128256: 236 us to 210 for the
+// kernel against one cell to an instruction and a sum of integers to detect wraps.  Slower: eight cells at a time
+// or the loads of the next quarter tile in flight (spills at 64 registers), the split of big cells without a branch,
+// the next item prefetched into L2: 32 warps hide the loads already.)
 // wbase: shared-memory byte address of wp[0] minus 4 * (the bits of the fma's constant), so that
 // the address of a bin's word is wbase + 4 * (bits of the fma's result); the q array follows the p
 // array at kHistWords words, the b arrays at twice that.
@@ -575,62 +593,76 @@ constexpr float kBinMagic = 12582912.f;                         // 1.5 * 2^23
 constexpr float kBigUnits = 268435456.f;                        // 2^28 units = a cell of 2^-16
 __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const float4 (&vq)[4], float k2,
                                                const RowOff &o, float binscale, float half_bin, float top, uint32_t wbase,
-                                               float &res1u, PassSums &ps, uint32_t over_bits) {
+                                               uint32_t over_bits, float &sp, float &sq) {
     // dl = log2(rho) - half: the half bin (in log2 units) that turns the fma's round-to-nearest into
     // the bin's floor is part of the row offset, so p_beam > q_beam reads dl > -half
     const float bd = ((o.bp - o.bq) + o.dc) - half_bin;
     const float pass_thr = -half_bin;
     const float cpu = o.cp * kFix, cqu = o.cq * kFix;           // exact: powers of two
-    uint32_t t0 = 0u, t1 = 0u;                                  // each below 2^32: 8 cells x 2 x less than 2^28 units
+    const unsigned long long k22 = pack2(k2, k2), bd2 = pack2(bd, bd), bp2 = pack2(o.bp, o.bp), bq2 = pack2(o.bq, o.bq);
+    const unsigned long long cp2 = pack2(cpu, cpu), cq2 = pack2(cqu, cqu), neg2 = pack2(-1.f, -1.f);
+    const unsigned long long bs2 = pack2(binscale, binscale), mg2 = pack2(kBinMagic, kBinMagic);
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
-        const float zp4[4] = {vp[it].x, vp[it].y, vp[it].z, vp[it].w};
-        const float zq4[4] = {vq[it].x, vq[it].y, vq[it].z, vq[it].w};
+        float dl[4], pm[4], qm[4];
+        uint32_t addr[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float dl = fmaf(zp4[c] - zq4[c], k2, bd);     // NaN compares false
-            float pmu = ex2_approx(fmaf(zp4[c], k2, o.bp)) * cpu;
-            float qmu = ex2_approx(fmaf(zq4[c], k2, o.bq)) * cqu;
-            const float diff = fmaxf(pmu - qmu, 0.f);
+        for (int h = 0; h < 2; ++h) {
+            const float4 &zp = vp[it], &zq = vq[it];
+            const unsigned long long p2 = h & 1 ? pack2(zp.z, zp.w) : pack2(zp.x, zp.y);
+            const unsigned long long q2 = h & 1 ? pack2(zq.z, zq.w) : pack2(zq.x, zq.y);
+            const unsigned long long dl2 = fma2(fma2(q2, neg2, p2), k22, bd2);     // NaN compares false
+            const float2 d = unpack2(dl2), t = unpack2(fma2(dl2, bs2, mg2));
+            const float2 pe = unpack2(fma2(p2, k22, bp2)), qe = unpack2(fma2(q2, k22, bq2));
+            const float2 pu = unpack2(mul2(pack2(ex2_approx(pe.x), ex2_approx(pe.y)), cp2));
+            const float2 qu = unpack2(mul2(pack2(ex2_approx(qe.x), ex2_approx(qe.y)), cq2));
             // floor(log2(rho) * binscale) in the low bits (round to nearest of x - 0.5; an x that is a
             // whole number may fall to either side, both within the bins' edge tolerance)
-            const float tb = fmaf(dl, binscale, kBinMagic);
             // (all cells beyond the last edge in one word would wrap it: every warp and half-warp
             // lane has its own copy of that bin)
-            const uint32_t bits = dl < top ? __float_as_uint(tb) : over_bits;
-            const uint32_t addr = wbase + (bits << 2);
-            if (pmu >= kBigUnits && dl > pass_thr) {
-                // whole multiples of 2^-28 of a big cell go to the b word (units of 2^-28), the
-                // remainder (below 2^16 units) stays for the w word
-                const float hp = floorf(pmu * (1.f / 65536.f));
-                pmu = fmaf(-hp, 65536.f, pmu);
-                asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(addr), "n"(2 * kHistWords * 4), "r"((uint32_t)hp) : "memory");
-                if (qmu >= kBigUnits) {
-                    const float hq = floorf(qmu * (1.f / 65536.f));
-                    qmu = fmaf(-hq, 65536.f, qmu);
-                    asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(addr), "n"(3 * kHistWords * 4), "r"((uint32_t)hq) : "memory");
+            addr[2 * h] = wbase + ((d.x < top ? __float_as_uint(t.x) : over_bits) << 2);
+            addr[2 * h + 1] = wbase + ((d.y < top ? __float_as_uint(t.y) : over_bits) << 2);
+            dl[2 * h] = d.x; pm[2 * h] = pu.x; qm[2 * h] = qu.x;
+            dl[2 * h + 1] = d.y; pm[2 * h + 1] = pu.y; qm[2 * h + 1] = qu.y;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            asm("{\n\t.reg .pred p;\n\t"
+                "setp.gt.f32 p, %2, %5;\n\t"
+                "@p add.f32 %0, %0, %3;\n\t"
+                "@p add.f32 %1, %1, %4;\n\t}"
+                : "+f"(sp), "+f"(sq) : "f"(dl[c]), "f"(pm[c]), "f"(qm[c]), "f"(pass_thr));
+        const float big = fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3]));
+        if (big >= kBigUnits) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (pm[c] >= kBigUnits && dl[c] > pass_thr) {
+                    // whole multiples of 2^-28 of a big cell go to the b word (units of 2^-28), the
+                    // remainder (below 2^16 units) stays for the w word
+                    const float hp = floorf(pm[c] * (1.f / 65536.f));
+                    pm[c] = fmaf(-hp, 65536.f, pm[c]);
+                    asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(addr[c]), "n"(2 * kHistWords * 4), "r"((uint32_t)hp) : "memory");
+                    if (qm[c] >= kBigUnits) {
+                        const float hq = floorf(qm[c] * (1.f / 65536.f));
+                        qm[c] = fmaf(-hq, 65536.f, qm[c]);
+                        asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(addr[c]), "n"(3 * kHistWords * 4), "r"((uint32_t)hq) : "memory");
+                    }
                 }
-            }
-            const uint32_t ap = __float2uint_rn(pmu), aq = __float2uint_rn(qmu);
-            uint32_t &tacc = (it < 2) ? t0 : t1;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
             asm volatile(
                 "{\n\t.reg .pred p;\n\t"
-                "setp.gt.f32 p, %2, %8;\n\t"
-                "@p red.shared.add.u32 [%3], %4;\n\t"
-                "@p red.shared.add.u32 [%3+%6], %5;\n\t"
-                "@p add.f32 %0, %0, %7;\n\t"
-                "@p add.u32 %1, %1, %4;\n\t"
-                "@p add.u32 %1, %1, %5;\n\t}"
-                : "+f"(res1u), "+r"(tacc)
-                : "f"(dl), "r"(addr), "r"(ap), "r"(aq), "n"(kHistWords * 4), "f"(diff), "f"(pass_thr)
+                "setp.gt.f32 p, %0, %5;\n\t"
+                "@p red.shared.add.u32 [%1], %2;\n\t"
+                "@p red.shared.add.u32 [%1+%4], %3;\n\t}"
+                :: "f"(dl[c]), "r"(addr[c]), "r"(__float2uint_rn(pm[c])), "r"(__float2uint_rn(qm[c])), "n"(kHistWords * 4), "f"(pass_thr)
                 : "memory");
-        }
     }
-    ps.tot += (unsigned long long)t0 + t1;
 }
 
 // One cluster-wide pass over the live rows; every CTA fills its own shared-memory histogram.
-// tot (shared memory, zero before the call): [0] what the CTA added to its w words (p and q).
+// tot (shared memory, zero before the call): [0] the mass that the CTA added (p and q), from floating-point sums.
 __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float binscale, const HistSmem &h,
                                double *sums1, int cta_rank, int n_cta, int halves, unsigned long long *tot) {
     // halves = 2: an item is a half tile (when the cluster has a warp for each), with a sum of its own
@@ -638,7 +670,7 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float bins
     const int warp = cta_rank * kVWarps + (threadIdx.x >> 5);
     const int nwarps = n_cta * kVWarps;
     const int items = sh.nA * a.T * halves;
-    PassSums ps = {0ull};
+    unsigned long long added = 0ull;
     const uint32_t magic_bits = __float_as_uint(kBinMagic);
     const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(h.wp) - (magic_bits << 2);
     const uint32_t over_bits = magic_bits + (uint32_t)(kBins + ((threadIdx.x >> 5) & 15) * 16 + (threadIdx.x & 15));
@@ -652,40 +684,49 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float bins
         const float *rq = a.zq + (int64_t)row * a.stride;
         const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
         const RowOff ro = row_off(sh, i);
-        float res1u = 0.f;                               // sum of (p - q)+ over the item in units: residual mass at s = 1
+        double res1 = 0.0;                               // sum of (p - q)+ over the item in units: residual mass at s = 1
         int e0 = t * (kTile / halves);
 #pragma unroll 1
         for (int half = halves; half < 3; ++half, e0 += kTile / 2) {
             float4 vp[4], vq[4];
-            load_half_tile(rp, e0, a.V, al, lane, vp);
-            load_half_tile(rq, e0, a.V, al, lane, vq);
-            hist_half_tile(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, res1u, ps, over_bits);
+            if (al && e0 + kTile / 2 <= a.V) {
+#pragma unroll
+                for (int it = 0; it < 4; ++it) vp[it] = ldg_stream(reinterpret_cast<const float4 *>(rp + e0 + it * 128) + lane);
+#pragma unroll
+                for (int it = 0; it < 4; ++it) vq[it] = ldg_stream(reinterpret_cast<const float4 *>(rq + e0 + it * 128) + lane);
+            } else {
+                load_half_tile(rp, e0, a.V, false, lane, vp);
+                load_half_tile(rq, e0, a.V, false, lane, vq);
+            }
+            float sp = 0.f, sq = 0.f;
+            hist_half_tile(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sp, sq);
+            added += __float2ull_rn(sp + sq);
+            res1 += (double)sp - (double)sq;
         }
         // the items' sums of the residual after ONE rejection (s_1 = 1): what a completion draw at run
         // position 2 searches, so that this common case needs no second pass over the rows
-        const double tot1 = warp_sum((double)res1u) * kUnfix;
+        const double tot1 = warp_sum(res1) * kUnfix;
         if (lane == 0) sums1[item] = tot1;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ps.tot += __shfl_xor_sync(kFull, ps.tot, o);
-    if (lane == 0 && ps.tot) atomicAdd(tot, ps.tot);         // (tot[0]: what the CTA's threads added to its w words)
+    for (int o = 16; o > 0; o >>= 1) added += __shfl_xor_sync(kFull, added, o);
+    if (lane == 0 && added) atomicAdd(tot, added);
 }
 
 // The copies of the last bin (rho beyond the last edge), folded by each CTA and added to every CTA's total
 // (tot[7], tot[8]); before the cluster barrier that follows the pass.  Also tot[6] += what the CTA's threads
-// added to w words minus what these copies hold of it.
+// added minus what these copies hold of it.
 __device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *tot, int n_cta) {
     const int lane = threadIdx.x & 31;
     if (threadIdx.x < kOverSlots) {
         const int i = kBins + (int)threadIdx.x;
-        unsigned long long w = (unsigned long long)h.wp[i] + h.wq[i];
         unsigned long long P = ((unsigned long long)h.bp[i] << 16) + h.wp[i], Q = ((unsigned long long)h.bq[i] << 16) + h.wq[i];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            w += __shfl_xor_sync(kFull, w, o);
             P += __shfl_xor_sync(kFull, P, o);
             Q += __shfl_xor_sync(kFull, Q, o);
         }
+        unsigned long long w = P + Q;
         if (threadIdx.x < 32) w -= tot[0];
         if (lane < n_cta) {
             unsigned long long *to = cluster.map_shared_rank(tot, lane);
@@ -702,15 +743,16 @@ __device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, un
 // bins of two CTAs, so that all its loads are in flight together; the lanes that share bins add up by shuffles
 // (bound by latency: two barriers and one round of remote loads, 6 us for 8 CTAs, 8 for 16; a thread that
 // walked all CTAs' words of one bin took 7 and 9, with a sweep for the wraps before the first barrier).
-// tot[6] of every CTA then holds what all threads added to w words minus what the words hold: zero unless a
-// word wrapped (a wrap lowers the words by 2^32).  The caller puts a cluster barrier behind this before
+// tot[6] of every CTA then holds what all threads added, by their floating-point sums, minus what the words hold.
+// Without a wrap that is rounding: half a unit for each cell and 2^-20 of the mass (16 cells in a float sum), less
+// than 2^26 units; a wrap lowers the words by 2^32.  The caller puts a cluster barrier behind this before
 // anyone reads the image or tot[6] or reuses the arrays.
 __device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *gh,
                            unsigned long long *tot, int cta_rank, int n_cta) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int share = n_cta > 1 ? n_cta / 2 : 1;             // lanes that share four bins
     const int quads = kBins / 4 / n_cta, per_warp = 32 / share;
-    unsigned long long wsum = 0ull;
+    unsigned long long sum = 0ull;
     for (int base = warp * per_warp; base < quads; base += kVWarps * per_warp) {
         const int i = 4 * (cta_rank * quads + base + lane % per_warp);
         unsigned long long P[4] = {}, Q[4] = {};
@@ -723,8 +765,6 @@ __device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, unsign
             P[2] += ((unsigned long long)bp.z << 16) + wp.z; P[3] += ((unsigned long long)bp.w << 16) + wp.w;
             Q[0] += ((unsigned long long)bq.x << 16) + wq.x; Q[1] += ((unsigned long long)bq.y << 16) + wq.y;
             Q[2] += ((unsigned long long)bq.z << 16) + wq.z; Q[3] += ((unsigned long long)bq.w << 16) + wq.w;
-            wsum += (unsigned long long)wp.x + wp.y + wp.z + wp.w;
-            wsum += (unsigned long long)wq.x + wq.y + wq.z + wq.w;
         }
         for (int o = per_warp; o < 32; o <<= 1) {
 #pragma unroll
@@ -736,12 +776,15 @@ __device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, unsign
         if (lane < per_warp) {
             ulonglong2 *to = reinterpret_cast<ulonglong2 *>(gh + 2 * i);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) to[k] = make_ulonglong2(P[k], Q[k]);
+            for (int k = 0; k < 4; ++k) {
+                to[k] = make_ulonglong2(P[k], Q[k]);
+                sum += P[k] + Q[k];
+            }
         }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(kFull, wsum, o);
-    if (lane < n_cta && wsum) atomicAdd(cluster.map_shared_rank(tot, lane) + 6, 0ull - wsum);
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+    if (lane < n_cta && sum) atomicAdd(cluster.map_shared_rank(tot, lane) + 6, 0ull - sum);
 }
 
 // One completion draw (residual if s_res > 0 else p_beam) by one warp; returns the token or -1
@@ -1132,7 +1175,7 @@ constexpr size_t kVerifyDynSmem = kHistArrays * sizeof(uint32_t) * kHistWords;
 static_assert(2 * sizeof(unsigned long long) * kHistWords <= kVerifyDynSmem, "the suffix sums fit over the building arrays");
 
 __global__ void __launch_bounds__(kVThreads, 2)
-k_verify(VerifyArgs a) {
+k_verify(const __grid_constant__ VerifyArgs a) {
     cg::cluster_group cluster = cg::this_cluster();
     const int n_cta = (int)cluster.num_blocks();
     const int cta_rank = (int)cluster.block_rank();
@@ -1593,7 +1636,7 @@ k_verify(VerifyArgs a) {
                 if (lane == 0) { sh.wtot_p[warp] = ap; sh.wtot_q[warp] = aq; }
                 if (threadIdx.x == 0) {
                     sh.n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
-                    sh.wrapped = tot[6] != 0ull;
+                    sh.wrapped = (long long)tot[6] > (1ll << 31);
                     sh.halves = halves;
                     if (sh.wrapped) ++sh.n_wrapped;
                 }

@@ -829,16 +829,15 @@ __device__ int draw_cell(const VerifyArgs &a, const Shared &sh, double u, bool u
 // ---------------------------------------------------------------------------------------
 constexpr int kMaxTopK = 64;
 constexpr int kMaxCand = 680;      // candidate cells per model (two lists overlay one histogram array)
-constexpr int kHalf = 256;         // threads that build one model's support (the two models run side by side)
+constexpr int kHalf = kVThreads / 2;   // threads that build one model's support when the two models run side by side
 // scratch of one build_support instance
 struct SupportTmp {
     float off[kMaxLive];          // log(beam weight) - lse of each live row
     int sel[256];                 // tiles whose bound reaches the threshold
-    int rhist[256];               // radix select of the k-th largest tile bound
-    int n_sel, n_cand, err, n_finite, rk;
-    unsigned rprefix;
-    float theta;
-    double zsum;
+    unsigned lo[kVWarps], hi[kVWarps];   // per warp, images of the smallest finite and of the largest bound
+    int finite[kVWarps];          // per warp, finite bounds
+    int count[3];                 // of the bisection's rounds, in turn
+    int n_sel, n_cand, err;
 };
 struct WarpScratch {
     double prob[2][kMaxTopK];     // warped probabilities, most probable first (0: p, 1: q)
@@ -848,166 +847,124 @@ struct WarpScratch {
     int n[2];
     SupportTmp tmp[2];
 };
-constexpr int kBoundCache = 1152;  // tile bounds per model kept in shared memory behind the WarpScratch
-static_assert(((sizeof(WarpScratch) + 15) & ~size_t(15)) + 2 * kBoundCache * sizeof(float) <=
-                  (kBins + 2) * sizeof(uint32_t),
-              "the support scratch and the two bound caches overlay one histogram array");
+constexpr int kBoundCache = kHistWords;   // tile bounds kept in shared memory: the third (p) or fourth (q) histogram array
+static_assert(sizeof(WarpScratch) <= kHistWords * sizeof(uint32_t), "the support scratch overlays the second histogram array");
 static_assert(2 * kMaxCand * (sizeof(double) + sizeof(int)) <= (kBins + 2) * sizeof(uint32_t),
               "the two candidate lists overlay the other histogram array");
 
-// barrier of the kHalf threads that work on one model (ids 1 and 2; 0 is __syncthreads)
-__device__ __forceinline__ void half_sync(int half) {
-    asm volatile("bar.sync %0, %1;" ::"r"(half + 1), "r"(kHalf) : "memory");
+// barrier of the NT threads that work on one model (ids 1 and 2; 0 is __syncthreads)
+template <int NT>
+__device__ __forceinline__ void part_sync(int model) {
+    asm volatile("bar.sync %0, %1;" ::"r"(model + 1), "n"(NT) : "memory");
 }
 
-// Support of the warped joint of one model; called by the kHalf threads of half `model` of the CTA
-// (warps 0-7: p, warps 8-15: q), the two halves side by side on their own scratch.  hist_p / hist_q:
-// the two idle histogram arrays.  Returns 0 or a DSBD_DEV_* code (the same on every thread of the
-// half).
+// Support of the warped joint of one model by NT threads: a half of the CTA for each model (warps 0-7: p, warps
+// 8-15: q) side by side on their own scratch, or the whole CTA where only p is wanted.  hist_p / hist_q: the first two
+// of the idle histogram arrays.  Returns 0 or a DSBD_DEV_* code (the same on every thread of the part).
+// Latency decides (a chain of short steps between barriers): the threshold is a bisection whose rounds have one
+// barrier each and that stops at the first cut with k to k + 2 tiles above it, about 8 rounds.  Exact radix
+// selection (4 rounds of three barriers with colliding atomics), one warp that lists the tiles, one thread that cuts
+// at top-p and half the CTA for a draft layer's only model took, for a draft of 5 layers of 16 x 8 rows of 128256 with
+// top-k 10, 419 us instead of 337; 20 requests with top-k 50 took 169 instead of 144.  (As a function that is
+// not inlined, with generic loads: 363 and 165.)
+template <int NT>
 __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, uint32_t *hist_p, uint32_t *hist_q) {
     WarpScratch &ws = *reinterpret_cast<WarpScratch *>(hist_q);
     SupportTmp &tp = ws.tmp[model];
     double *cand_key = reinterpret_cast<double *>(hist_p) + model * kMaxCand;
     int *cand_cell = reinterpret_cast<int *>(reinterpret_cast<double *>(hist_p) + 2 * kMaxCand) + model * kMaxCand;
-    const int tl = threadIdx.x & (kHalf - 1);                 // thread and warp inside the half
+    const int tl = threadIdx.x & (NT - 1);                    // thread and warp inside the part
     const int lane = threadIdx.x & 31, warp = tl >> 5;
-    constexpr int kHalfWarps = kHalf / 32;
+    constexpr int kPartWarps = NT / 32;
     const int T = a.T, nt = sh.nA * T, k = a.top_k;
     const TileStat *stats = a.stats + (int64_t)model * a.N * T;
     const double *lw = model ? sh.lwq : sh.lwp;
     const double *lse = a.lse + (int64_t)model * a.N;
     const float *z = model ? a.zq : a.zp;
     const float inv_tau_f = (float)a.inv_tau;
-    for (int i = tl; i < sh.nA; i += kHalf) tp.off[i] = (float)(lw[i] - lse[sh.A[i]]);
+    for (int i = tl; i < sh.nA; i += NT) tp.off[i] = (float)(lw[i] - lse[sh.A[i]]);
+    if (tl < 3) tp.count[tl] = 0;
     if (tl == 0) { tp.n_sel = 0; tp.n_cand = 0; tp.err = 0; ws.n[model] = 0; }
-    half_sync(model);
+    part_sync<NT>(model);
     // float upper bound of log(joint probability) over tile i
     auto bound = [&](int i) -> float {
         const int ia = i / T;
         return fmaf(stats[(int64_t)sh.A[ia] * T + (i - ia * T)].mx, inv_tau_f, tp.off[ia]);
     };
-    // The k-th largest tile bound (with multiplicity: k tiles each hold a cell at least that
-    // large); with fewer than k finite bounds every tile counts.
-    float *bcache = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(&ws) +
-                                              ((sizeof(WarpScratch) + 15) & ~size_t(15))) + model * kBoundCache;
+    // order-preserving integer image of a float and back
+    auto image = [](float v) -> unsigned {
+        const unsigned b = __float_as_uint(v);
+        return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+    };
+    auto value = [](unsigned u) -> float { return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u); };
+    // A cut not above the k-th largest tile bound (with multiplicity: k tiles each hold a cell at least that
+    // large) and few tiles below it; with fewer than k finite bounds every tile counts.  Bounds that do not fit
+    // the cache are computed again in every round.
+    unsigned *bcache = hist_p + (2 + model) * kHistWords;
     const bool cached = nt <= kBoundCache;
-    if (cached) {
-        // all warps: bounds into shared memory, then a radix select over their order-preserving
-        // integer images, one byte per pass from the top
-        auto image = [](float v) -> unsigned {
-            const unsigned b = __float_as_uint(v);
-            return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-        };
-        if (tl == 0) { tp.rprefix = 0u; tp.rk = k; tp.n_finite = 0; }
-        half_sync(model);
+    {
+        unsigned lo = 0xffffffffu, hi = 0u;
         int finite = 0;
-        for (int i = tl; i < nt; i += kHalf) {
+#pragma unroll 4
+        for (int i = tl; i < nt; i += NT) {
             const float v = bound(i);
-            bcache[i] = v;
-            finite += v > -INFINITY;
+            const unsigned u = image(v);
+            if (cached) bcache[i] = u;
+            if (v > -INFINITY) { ++finite; lo = min(lo, u); hi = max(hi, u); }
         }
-        if (finite) atomicAdd(&tp.n_finite, finite);
-        for (int pass = 3; pass >= 0; --pass) {
-            for (int i = tl; i < 256; i += kHalf) tp.rhist[i] = 0;
-            half_sync(model);
-            const unsigned prefix = tp.rprefix;
-            for (int i = tl; i < nt; i += kHalf) {
-                const unsigned u = image(bcache[i]);
-                if (pass == 3 || (u >> (8 * (pass + 1))) == prefix) atomicAdd(&tp.rhist[(u >> (8 * pass)) & 255u], 1);
-            }
-            half_sync(model);
-            if (warp == 0) {
-                // the digit whose bin holds the rk-th largest: lane l owns bins 8l .. 8l+7; a suffix
-                // sum over the lanes finds the owning lane, which then walks its own bins
-                int mine = 0;
+        lo = __reduce_min_sync(kFull, lo); hi = __reduce_max_sync(kFull, hi); finite = __reduce_add_sync(kFull, finite);
+        if (lane == 0) { tp.lo[warp] = lo; tp.hi[warp] = hi; tp.finite[warp] = finite; }
+    }
+    part_sync<NT>(model);
+    unsigned lo = 0xffffffffu, hi = 0u;
+    int finite = 0;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) mine += tp.rhist[lane * 8 + q];
-                int above = mine;                              // bins of this lane and of the lanes above
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_down_sync(kFull, above, o);
-                    if (lane + o < 32) above += t;
-                }
-                const int need0 = tp.rk;
-                const bool owner = above >= need0 && above - mine < need0;
-                const unsigned who = __ballot_sync(kFull, owner);
-                if (who == 0u) {
-                    if (lane == 0) { tp.rprefix = prefix << 8; tp.rk = need0 - above; }   // fewer than rk values
-                } else if (owner) {
-                    int need = need0 - (above - mine), d = lane * 8 + 7;
-                    for (; d > lane * 8; --d) {
-                        if (tp.rhist[d] >= need) break;
-                        need -= tp.rhist[d];
-                    }
-                    tp.rk = need;
-                    tp.rprefix = (prefix << 8) | (unsigned)d;
-                }
-            }
-            half_sync(model);
+    for (int w = 0; w < kPartWarps; ++w) { lo = min(lo, tp.lo[w]); hi = max(hi, tp.hi[w]); finite += tp.finite[w]; }
+    if (finite >= k) {
+        // count(>= lo) >= k always holds; hi is above the k-th largest
+        ++hi;
+        for (int round = 0; hi - lo > 1; ++round) {
+            const unsigned mid = lo + (hi - lo) / 2;
+            int n = 0;
+            for (int i = tl; i < nt; i += NT) n += (cached ? bcache[i] : image(bound(i))) >= mid;
+            n = __reduce_add_sync(kFull, n);
+            if (lane == 0 && n) atomicAdd(&tp.count[round % 3], n);
+            if (tl == 0) tp.count[(round + 1) % 3] = 0;           // (last read two rounds ago)
+            part_sync<NT>(model);
+            n = tp.count[round % 3];
+            if (n >= k) { lo = mid; if (n <= k + 2) break; } else hi = mid;
         }
     }
-    if (warp == 0) {
-        float thr = INFINITY;
-        bool enough = true, any = false;
-        if (cached) {
-            const unsigned u = tp.rprefix;
-            thr = __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
-            enough = tp.n_finite >= k && thr > -INFINITY;
-            any = tp.n_finite > 0;
-        } else {
-            // too many live rows x tiles for the cache: k rounds of arg-max over distinct bounds
-            for (int kk = 0; kk < k; ++kk) {
-                float best = -INFINITY;
-                for (int i = lane; i < nt; i += 32) {
-                    const float v = bound(i);
-                    if (v < thr && v > best) best = v;
-                }
-                best = warp_max(best);
-                if (!(best > -INFINITY)) { enough = false; break; }
-                any = true;
-                thr = best;
+    const float thr = value(lo);
+    // the float keys carry an error of about 1e-5; the slack keeps the selection conservative
+    float theta = finite >= k ? thr - 5e-5f - 4e-6f * fabsf(thr) : -INFINITY;
+    if (finite > 0)
+        for (int i = tl; i < nt; i += NT) {
+            const float bv = cached ? value(bcache[i]) : bound(i);
+            if (bv >= theta && bv > -INFINITY) {
+                const int pos = atomicAdd(&tp.n_sel, 1);
+                if (pos < 256) tp.sel[pos] = i;
+                else tp.err = DSBD_DEV_CAPACITY;                  // hundreds of tiles tie at the cut
             }
         }
-        // the float keys carry an error of about 1e-5; the slack keeps the selection conservative
-        const float theta = enough ? thr - 5e-5f - 4e-6f * fabsf(thr) : -INFINITY;
-        int n_sel = 0;
-        if (any)
-            for (int base = 0; base < nt; base += 32) {
-                const int i = base + lane;
-                const float bv = i < nt ? (cached ? bcache[i] : bound(i)) : -INFINITY;
-                const bool hit = i < nt && bv >= theta && bv > -INFINITY;
-                const unsigned mask = __ballot_sync(kFull, hit);
-                if (hit) {
-                    const int pos = n_sel + __popc(mask & ((1u << lane) - 1));
-                    if (pos < 256) tp.sel[pos] = i;
-                }
-                n_sel += __popc(mask);
-            }
-        if (lane == 0) {
-            tp.theta = theta;
-            tp.n_sel = n_sel;
-            if (n_sel > 256) tp.err = DSBD_DEV_CAPACITY;       // hundreds of tiles tie at the cut
-        }
-    }
-    half_sync(model);
+    part_sync<NT>(model);
     if (tp.err) return tp.err;
-    float theta = tp.theta;
     const int n_sel = tp.n_sel;
     // One sweep over the selected tiles by all warps: counts the cells whose key reaches th and,
     // when asked, appends them to the candidate list (order is irrelevant: the final choice is
     // by (key, cell)).
     auto sweep = [&](float th, bool collect) {
-        half_sync(model);                      // every thread has taken the previous sweep's count
+        part_sync<NT>(model);                      // every thread has taken the previous sweep's count
         if (tl == 0) tp.n_cand = 0;
-        half_sync(model);
+        part_sync<NT>(model);
         // this warp's tiles into L2 first (a tile is 32 lines of 128 bytes: one per lane), so that
         // the dependent tile loads below do not each pay a trip to HBM
-        for (int sidx = warp; sidx < n_sel; sidx += kHalfWarps) {
+        for (int sidx = warp; sidx < n_sel; sidx += kPartWarps) {
             const int ti = tp.sel[sidx], ia = ti / T, t = ti - ia * T;
             const int e = t * kTile + lane * 32;
             if (e < a.V) asm volatile("prefetch.global.L2 [%0];" ::"l"(z + (int64_t)sh.A[ia] * a.stride + e));
         }
-        for (int sidx = warp; sidx < n_sel; sidx += kHalfWarps) {
+        for (int sidx = warp; sidx < n_sel; sidx += kPartWarps) {
             const int ti = tp.sel[sidx], ia = ti / T, t = ti - ia * T, row = sh.A[ia];
             const float *rowp = z + (int64_t)row * a.stride;
             const bool al = (reinterpret_cast<uintptr_t>(rowp) & 15) == 0;
@@ -1053,7 +1010,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
                 }
             }
         }
-        half_sync(model);
+        part_sync<NT>(model);
         return tp.n_cand;
     };
     int n_cand = sweep(theta, true);
@@ -1078,10 +1035,11 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     // cell ascending -- a total order, cells are unique) and, if fewer than k do, that count is its
     // place in the support
     if (n_cand > kMaxCand) n_cand = kMaxCand;
-    for (int jc = tl; jc < n_cand; jc += kHalf) {
+    for (int jc = tl; jc < n_cand; jc += NT) {
         const double key = cand_key[jc];
         const int cell = cand_cell[jc];
         int rank = 0;
+#pragma unroll 4
         for (int i = 0; i < n_cand; ++i) {
             const double ki = cand_key[i];
             rank += (ki > key) || (ki == key && cand_cell[i] < cell);
@@ -1091,62 +1049,56 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
             ws.cell[model][rank] = cell;
         }
     }
-    half_sync(model);
+    part_sync<NT>(model);
     if (warp == 0) {
+        // renormalise over the top k, then the top-p cut and its renormalisation: a lane has the places 2 lane, 2 lane + 1
         const int n_sup = n_cand < k ? n_cand : k;
-        // renormalise over the top k, then the top-p cut and its renormalisation (sorted order)
-        if (lane == 0) {
-            double zsum = 0.0;
-            for (int j = 0; j < n_sup; ++j) zsum += ws.prob[model][j];
-            int keep = n_sup;
-            if (a.top_p > 0.0 && a.top_p < 1.0 && zsum > 0.0) {
-                double cum = 0.0;
-                int j = 0;
-                for (; j < n_sup; ++j) {
-                    cum += ws.prob[model][j] / zsum;
-                    if (cum >= a.top_p) { ++j; break; }
-                }
-                keep = j;
-                zsum = 0.0;
-                for (int q = 0; q < keep; ++q) zsum += ws.prob[model][q];
-            }
-            ws.n[model] = keep;
-            tp.zsum = zsum;
+        const double p0 = 2 * lane < n_sup ? ws.prob[model][2 * lane] : 0.0;
+        const double p1 = 2 * lane + 1 < n_sup ? ws.prob[model][2 * lane + 1] : 0.0;
+        const double incl = warp_scan(p0 + p1, lane), cum0 = incl - p1;
+        double zsum = __shfl_sync(kFull, incl, 31);
+        int keep = n_sup;
+        if (a.top_p > 0.0 && a.top_p < 1.0 && zsum > 0.0) {
+            // the first place whose running sum reaches top_p is the last one kept
+            const unsigned b0 = __ballot_sync(kFull, cum0 < a.top_p * zsum), b1 = __ballot_sync(kFull, incl < a.top_p * zsum);
+            keep = min(n_sup, __popc(b0) + __popc(b1) + 1);
+            const double c0 = __shfl_sync(kFull, cum0, (keep - 1) / 2), c1 = __shfl_sync(kFull, incl, (keep - 1) / 2);
+            zsum = (keep & 1) ? c0 : c1;
         }
-        __syncwarp();
-        const double inv = tp.zsum > 0.0 ? 1.0 / tp.zsum : 0.0;
-        for (int j = lane; j < ws.n[model]; j += 32) ws.prob[model][j] *= inv;
+        const double inv = zsum > 0.0 ? 1.0 / zsum : 0.0;
+        if (2 * lane < keep) ws.prob[model][2 * lane] = p0 * inv;
+        if (2 * lane + 1 < keep) ws.prob[model][2 * lane + 1] = p1 * inv;
+        if (lane == 0) ws.n[model] = keep;
     }
-    half_sync(model);
+    part_sync<NT>(model);
     return 0;
 }
 
 __device__ __forceinline__ double support_lookup(const WarpScratch &ws, int model, int cell) {
-    for (int j = 0; j < ws.n[model]; ++j)
-        if (ws.cell[model][j] == cell) return ws.prob[model][j];
-    return 0.0;
+    int at = -1;
+    for (int j = 0, n = ws.n[model]; j < n; ++j) at = ws.cell[model][j] == cell ? j : at;      // (cells are unique)
+    return at >= 0 ? ws.prob[model][at] : 0.0;
 }
 
-// Inverse-CDF draw over the p support in canonical order; mass max(p~ - s q~, 0) (s = 0: p~).
-// By one thread.  Returns the index into the p support or -1.
-__device__ int draw_support(const WarpScratch &ws, double u, double s) {
+// Inverse-CDF draws over the p support in canonical order; mass max(p~ - s q~, 0) (s = 0: p~).  By one warp, one
+// draw for each lane that wants one (u per lane).  Returns the index into the p support or -1.
+__device__ int draw_support(const WarpScratch &ws, double u, double s, int lane) {
     const int n = ws.n[0];
-    double zsum = 0.0;
-    for (int o = 0; o < n; ++o) {
-        const int i = ws.order[o];
-        zsum += fmax(ws.prob[0][i] - s * ws.qat[i], 0.0);
-    }
-    if (!(zsum > 0.0)) return -1;
+    double w0 = 0.0, w1 = 0.0;                                // places 2 lane and 2 lane + 1
+    if (2 * lane < n) { const int i = ws.order[2 * lane]; w0 = fmax(ws.prob[0][i] - s * ws.qat[i], 0.0); }
+    if (2 * lane + 1 < n) { const int i = ws.order[2 * lane + 1]; w1 = fmax(ws.prob[0][i] - s * ws.qat[i], 0.0); }
+    const double incl = warp_scan(w0 + w1, lane), cum0 = incl - w1;
+    const double zsum = __shfl_sync(kFull, incl, 31);
+    const unsigned m0 = __ballot_sync(kFull, w0 > 0.0), m1 = __ballot_sync(kFull, w1 > 0.0);
     const double target = u * zsum;
-    double cum = 0.0;
-    int last = -1;
-    for (int o = 0; o < n; ++o) {
-        const int i = ws.order[o];
-        const double w = fmax(ws.prob[0][i] - s * ws.qat[i], 0.0);
-        cum += w;
-        if (w > 0.0) { last = i; if (cum >= target) return i; }
+    int pick = -1;
+    bool found = false;
+    for (int l = 0; 2 * l < n; ++l) {
+        const double c0 = __shfl_sync(kFull, cum0, l), c1 = __shfl_sync(kFull, incl, l);
+        if (!found && (m0 >> l & 1)) { pick = 2 * l; found = c0 >= target; }
+        if (!found && (m1 >> l & 1)) { pick = 2 * l + 1; found = c1 >= target; }
     }
-    return last;
+    return pick < 0 || !(zsum > 0.0) ? -1 : ws.order[pick];
 }
 
 // After build_support(p) [and q]: q~ at the p cells and the canonical order of the p support.
@@ -1555,7 +1507,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             if (!sh.err) {
                 // the first half of the warps builds the support of p, the second that of q, side by side
                 const int half = warp / (kHalf / 32);
-                const int e_half = build_support(a, sh, half, hp, hq);
+                const int e_half = build_support<kHalf>(a, sh, half, hp, hq);
                 if (e_half && (threadIdx.x & (kHalf - 1)) == 0) wsup.tmp[half].err = e_half;
                 __syncthreads();
                 const int e = wsup.tmp[0].err ? wsup.tmp[0].err : wsup.tmp[1].err;
@@ -1826,10 +1778,16 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 const bool use_res = j > 1;
                 if (warped && !err) {
                     const int want = W - count, n_draw = min(want, max(cap - n_out, 0));
-                    for (int kk = lane; kk < n_draw; kk += 32) {
+                    for (int k0 = 0; k0 < n_draw; k0 += 32) {
+                        const int kk = k0 + lane;
                         const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, kk ? 2u : 1u,
                                                           kk ? (uint32_t)(kk - 1) : 0u);
-                        const int pick = draw_support(wsup, u, kk == 0 && use_res ? sh.s_arr[j - 1] : 0.0);
+                        int pick = draw_support(wsup, u, 0.0, lane);
+                        if (k0 == 0 && use_res) {
+                            const int of_res = draw_support(wsup, u, sh.s_arr[j - 1], lane);
+                            if (kk == 0) pick = of_res;
+                        }
+                        if (kk >= n_draw) continue;
                         if (pick < 0) { err = DSBD_DEV_EXHAUSTED; continue; }
                         const int ia = wsup.cell[0][pick] / a.V, tok = wsup.cell[0][pick] - ia * a.V;
                         if (writer)
@@ -1902,12 +1860,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         if (warp < 2) live_weights(a, sh, warp, warp == 0 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
         __syncthreads();
         if (a.top_k > 0) {
-            if (warp < kHalf / 32) {                            // one model only: the first half builds it
-                const int e_half = build_support(a, sh, 0, hp, hq);
-                if (e_half && threadIdx.x == 0) wsx.tmp[0].err = e_half;
-            }
-            __syncthreads();
-            extra_err = wsx.tmp[0].err;
+            extra_err = build_support<kVThreads>(a, sh, 0, hp, hq);       // one model only: by the whole CTA
             if (!extra_err && warp == 0) finish_supports(wsx, false, lane);
         }
     }
@@ -1936,10 +1889,12 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         if (writer && lane == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
         const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
         const int n_draw = err ? 0 : min(W_nom, max(cap - n_out, 0));
-        for (int kk = lane; kk < n_draw; kk += 32) {
+        for (int k0 = 0; k0 < n_draw; k0 += 32) {
+            const int kk = k0 + lane;
             const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1) + a.extra_layer_bias, 3u,
                                               (uint32_t)kk);
-            const int pick = draw_support(wsx, u, 0.0);
+            const int pick = draw_support(wsx, u, 0.0, lane);
+            if (kk >= n_draw) continue;
             if (pick < 0) { err = DSBD_DEV_EXHAUSTED; continue; }
             const int ia = wsx.cell[0][pick] / a.V, tok = wsx.cell[0][pick] - ia * a.V;
             if (writer)

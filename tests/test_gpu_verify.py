@@ -325,6 +325,24 @@ def test_requests_around_the_node_cache_and_half_tiles(beams, gamma, V):
     check_exempt(exempt, decisions)
 
 
+@pytest.mark.parametrize("beams,V,top_k,top_p", [(64, 72000, 10, 0.8), (64, 72000, 64, 0.9), (36, 121900, 1, 1.0)])
+def test_warped_layers_with_more_tiles_than_the_bound_cache(beams, V, top_k, top_p):
+    """64 x 71 = 4544 tile bounds, more than are kept in shared memory (4368), and 36 x 120 = 4320, just fewer."""
+    rng = np.random.default_rng(V + top_k)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=1, V=V, gamma=1, max_w=beams, min_w=beams)
+    prm.update(top_k=top_k, top_p=top_p)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = 0
+    for step in range(2):
+        prm["step"] = step
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+    check_exempt(exempt, decisions)
+
+
 def test_roots_only_forest_goes_straight_to_the_extra_layer():
     rng = np.random.default_rng(3)
     V, B = 2000, 3

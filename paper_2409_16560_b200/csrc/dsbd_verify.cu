@@ -94,7 +94,6 @@ k_tile_stats(const float *__restrict__ zp, const float *__restrict__ zq, int64_t
              int T, int N, int n_rows, const int32_t *__restrict__ rows,
              const int32_t *__restrict__ n_rows_dev, float k2, TileStat *__restrict__ stats,
              int one_model = 0) {
-    // one_model: zq is the same tensor as zp; read it once and store the statistics for both
     // a kernel launched with programmatic stream serialization may be set up while the last blocks run
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;
@@ -131,7 +130,6 @@ k_tile_stats(const float *__restrict__ zp, const float *__restrict__ zq, int64_t
         if (lane == 0) {
             TileStat s; s.mx = mx; s.sum = sum;
             stats[((int64_t)model * N + row) * T + t] = s;
-            if (one_model) stats[((int64_t)N + row) * T + t] = s;
         }
     }
 }
@@ -205,7 +203,6 @@ struct VerifyArgs {
     const float *root_logp, *root_logq;
     int max_m, max_live;
     int check_widths;            // verification / width selection: per-request widths are validated
-    uint32_t extra_layer_bias;   // added to the layer number in the Philox counter of the extra layer
     // outputs
     dsbd_verify_out_t out;
     int32_t *status;
@@ -1870,7 +1867,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         const int n_draw = min(W_nom, max(cap - n_out, 0));
         if (writer && threadIdx.x == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
         for (int kk = warp; kk < n_draw; kk += kVWarps) {
-            const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1) + a.extra_layer_bias, 3u,
+            const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1), 3u,
                                               (uint32_t)kk);
             int ia = 0;
             const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, 1, lane, &ia);
@@ -1891,7 +1888,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         const int n_draw = err ? 0 : min(W_nom, max(cap - n_out, 0));
         for (int k0 = 0; k0 < n_draw; k0 += 32) {
             const int kk = k0 + lane;
-            const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1) + a.extra_layer_bias, 3u,
+            const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1), 3u,
                                               (uint32_t)kk);
             const int pick = draw_support(wsx, u, 0.0, lane);
             if (kk >= n_draw) continue;
@@ -2123,59 +2120,116 @@ extern "C" int dsbd_node_stats(const dsbd_forest_t *f, const dsbd_verify_params_
 }
 
 // ---------------------------------------------------------------------------------------
-// dsbd_draft_layer: a beam-sampling step of the small model is the "extra layer" of the
-// verification kernel on a forest that has only roots (the current beams), with the small
-// model's logits standing for both models: W_S inverse-CDF draws from T o q_beam.
+// dsbd_draft_layer: a beam-sampling step of the small model is the extra layer of the
+// verification on the current beams, with one model: W_S inverse-CDF draws from T o q_beam.
+// One CTA per request after the dense pass over the beams' rows.  What is left is a chain of short steps on a
+// few thousand numbers, so a CTA that does them alone beats the verification kernel's cluster, whose CTAs all
+// repeat the chain between barriers (and which needed a launch for the root-only forest it walked): with top-k 10
+// over 16 x 8 rows of 128256 the kernel takes 16 us instead of 43, unwarped over 8 x 4 rows of 32000 9 instead of 15.5.
 // ---------------------------------------------------------------------------------------
 namespace {
-__global__ void k_draft_init(int n_beams, int32_t *beam_node_off, int32_t *parent) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i <= n_beams) beam_node_off[i] = i;
-    if (i < n_beams) parent[i] = -1;
+struct DraftArgs {
+    VerifyArgs v;             // what the shared steps read: V, T, k2, inv_tau, seed, step, top_k, top_p, zp, stride, stats, lse
+    uint32_t layer;           // layer number in the Philox counter
+    const float *beam_logq;
+    int W;
+    const int32_t *W_r, *out_off;
+    int32_t *out_parent, *out_token;
+    float *out_logq;
+    int32_t *req_error;
+};
+
+__global__ void __launch_bounds__(kVThreads)
+k_draft(const __grid_constant__ DraftArgs d) {
+    const VerifyArgs &a = d.v;
+    __shared__ Shared sh;
+    __shared__ double score[kMaxLive], lse[kMaxLive];
+    __shared__ int s_err;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    uint32_t *hp = reinterpret_cast<uint32_t *>(dyn_smem), *hq = hp + kHistWords;
+    const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b_lo = a.req_beam_off[r], o_lo = d.out_off[r], cap = d.out_off[r + 1] - o_lo;
+    const int W = d.W_r ? d.W_r[r] : d.W;
+    int nA = a.req_beam_off[r + 1] - b_lo, err = 0;
+    if (nA > kMaxLive) { err = DSBD_DEV_BAD_FOREST; nA = 0; }
+    if (threadIdx.x < nA) {
+        sh.A[threadIdx.x] = b_lo + threadIdx.x;
+        score[threadIdx.x] = (double)d.beam_logq[b_lo + threadIdx.x];
+    }
+    if (threadIdx.x == 0) { sh.nA = nA; s_err = 0; }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int i = warp; i < nA; i += kVWarps) {
+        const double v = row_lse(a.stats + (int64_t)(b_lo + i) * a.T, a.T, a.inv_tau, lane);
+        if (lane == 0) { lse[i] = v; a.lse_w[b_lo + i] = v; }
+    }
+    __syncthreads();
+    if (warp == 0) live_weights(a, sh, 0, score, lane, nullptr, 0);
+    __syncthreads();
+    const int n_draw = err ? 0 : min(W, max(cap, 0));
+    auto emit = [&](int kk, int ia, int tok) {
+        const float z = a.zp[(int64_t)(b_lo + ia) * a.stride + tok];
+        d.out_parent[o_lo + kk] = b_lo + ia;
+        d.out_token[o_lo + kk] = tok;
+        d.out_logq[o_lo + kk] = (float)(score[ia] + ((double)z * a.inv_tau - lse[ia]));
+    };
+    if (a.top_k > 0) {
+        WarpScratch &ws = *reinterpret_cast<WarpScratch *>(hq);
+        if (!err) err = build_support<kVThreads>(a, sh, 0, hp, hq);
+        if (!err && warp == 0) {
+            finish_supports(ws, false, lane);
+            for (int k0 = 0; k0 < n_draw; k0 += 32) {
+                const int kk = k0 + lane;
+                const double u = decision_uniform(a.seed, a.step, (uint32_t)r, d.layer, 3u, (uint32_t)kk);
+                const int pick = draw_support(ws, u, 0.0, lane);
+                if (kk >= n_draw) continue;
+                if (pick < 0) { s_err = DSBD_DEV_EXHAUSTED; continue; }
+                const int ia = ws.cell[0][pick] / a.V;
+                emit(kk, ia, ws.cell[0][pick] - ia * a.V);
+            }
+        }
+    } else {
+        for (int kk = warp; kk < n_draw; kk += kVWarps) {
+            const double u = decision_uniform(a.seed, a.step, (uint32_t)r, d.layer, 3u, (uint32_t)kk);
+            int ia = 0;
+            const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, 1, lane, &ia);
+            if (lane == 0) {
+                if (tok < 0) s_err = DSBD_DEV_EXHAUSTED;
+                else emit(kk, ia, tok);
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (!err) err = s_err;
+        if (!err && n_draw < W) err = DSBD_DEV_CAPACITY;
+        if (d.req_error) d.req_error[r] = err;
+        if (err) report(a.status, err);
+    }
 }
 
 struct DraftLayout {
-    Layout v;
-    size_t beam_node_off, parent, l_last, out_width, layer_width, node_status, out_node, out_root_beam,
-        out_source, out_logp, total;
+    size_t stats, lse, total;
+    int T;
 };
-
-dsbd_forest_t draft_forest(int R, int n_beams, const dsbd_draft_params_t *p) {
-    dsbd_forest_t f = {};
-    f.R = R; f.B = n_beams; f.N = n_beams; f.max_depth = 0;
-    f.max_tree_nodes = 1; f.max_req_beams = p->max_req_beams; f.max_layer_nodes = 0;
-    return f;
-}
 
 bool draft_args_ok(int R, int n_beams, const dsbd_draft_params_t *p) {
     return p && R > 0 && n_beams > 0 && p->V > 0 && p->temperature > 0.f && p->n_slots > 0 &&
            p->max_req_beams > 0 && (p->W_S >= 0 || p->W_S_r) && p->layer >= 0 && p->top_k >= 0;
 }
 
-DraftLayout make_draft_layout(int R, int n_beams, const dsbd_draft_params_t *p) {
+DraftLayout make_draft_layout(int n_beams, const dsbd_draft_params_t *p) {
     DraftLayout D;
-    const dsbd_forest_t f = draft_forest(R, n_beams, p);
-    D.v = make_layout(&f, p->V);
-    size_t off = D.v.total;
-    auto take = [&](size_t bytes) { const size_t at = off; off = align_up(off + bytes, 256); return at; };
-    D.beam_node_off = take(sizeof(int32_t) * ((size_t)n_beams + 1));
-    D.parent = take(sizeof(int32_t) * (size_t)n_beams);
-    D.l_last = take(sizeof(int32_t) * (size_t)R);
-    D.out_width = take(sizeof(int32_t) * (size_t)R);
-    D.layer_width = take(sizeof(int32_t) * (size_t)R);
-    D.node_status = take((size_t)n_beams);
-    D.out_node = take(sizeof(int32_t) * (size_t)p->n_slots);
-    D.out_root_beam = take(sizeof(int32_t) * (size_t)p->n_slots);
-    D.out_source = take(sizeof(int32_t) * (size_t)p->n_slots);
-    D.out_logp = take(sizeof(float) * (size_t)p->n_slots);
-    D.total = off;
+    D.T = (p->V + kTile - 1) / kTile;
+    D.stats = 0;
+    D.lse = align_up(sizeof(TileStat) * (size_t)n_beams * D.T, 256);
+    D.total = align_up(D.lse + sizeof(double) * (size_t)n_beams, 256);
     return D;
 }
 }  // namespace
 
 extern "C" size_t dsbd_draft_workspace(int32_t R, int32_t n_beams, const dsbd_draft_params_t *p) {
     if (!draft_args_ok(R, n_beams, p)) return 0;
-    return make_draft_layout(R, n_beams, p).total;
+    return make_draft_layout(n_beams, p).total;
 }
 
 extern "C" int dsbd_draft_layer(int32_t R, int32_t n_beams, const int32_t *req_beam_off,
@@ -2190,61 +2244,47 @@ extern "C" int dsbd_draft_layer(int32_t R, int32_t n_beams, const int32_t *req_b
         return DSBD_ERR_INVALID_ARG;
     if (p->max_req_beams > DSBD_MAX_LIVE || p->top_k > 64) return DSBD_ERR_UNSUPPORTED;
     if (p->top_k == 0 && p->top_p > 0.f && p->top_p < 1.f) return DSBD_ERR_UNSUPPORTED;
-    const DraftLayout D = make_draft_layout(R, n_beams, p);
+    const DraftLayout D = make_draft_layout(n_beams, p);
     if (workspace_bytes < D.total) return DSBD_ERR_WORKSPACE_TOO_SMALL;
     if (reinterpret_cast<uintptr_t>(workspace) & 255) return DSBD_ERR_INVALID_ARG;
     char *ws = static_cast<char *>(workspace);
-    const Layout &L = D.v;
-    TileStat *stats = reinterpret_cast<TileStat *>(ws + L.stats);
-    double *lse = reinterpret_cast<double *>(ws + L.lse);
-    double *score = reinterpret_cast<double *>(ws + L.score);
-    int32_t *depth = reinterpret_cast<int32_t *>(ws + L.depth);
-    int32_t *beam_node_off = reinterpret_cast<int32_t *>(ws + D.beam_node_off);
-    int32_t *parent = reinterpret_cast<int32_t *>(ws + D.parent);
-    const double inv_tau = 1.0 / (double)p->temperature;
-    const float k2 = (float)((double)kLog2e * inv_tau);
-
-    k_draft_init<<<(n_beams + 1 + 255) / 256, 256, 0, stream>>>(n_beams, beam_node_off, parent);
-    const int64_t items = (int64_t)n_beams * L.T;
-    k_tile_stats<<<stats_grid(items), kThreads, 0, stream>>>(logits_q, logits_q, row_stride, p->V, L.T, n_beams,
-                                                            n_beams, nullptr, nullptr, k2, stats, 1);
-    if (cudaGetLastError() != cudaSuccess) return DSBD_ERR_CUDA;
-
-    VerifyArgs a = {};
-    a.R = R; a.N = n_beams; a.gamma = 0;
-    a.req_beam_off = req_beam_off; a.beam_node_off = beam_node_off; a.parent = parent;
-    a.token = nullptr; a.draft_rank = nullptr;
-    a.V = p->V; a.T = L.T; a.k2 = k2; a.inv_tau = inv_tau; a.thresh = 0.5;
-    a.W_min = 1; a.W_max = 1; a.W_nom = p->W_S; a.W_nom_r = p->W_S_r;
+    DraftArgs d = {};
+    VerifyArgs &a = d.v;
+    a.R = R; a.N = n_beams;
+    a.req_beam_off = req_beam_off;
+    a.V = p->V; a.T = D.T;
+    a.inv_tau = 1.0 / (double)p->temperature;
+    a.k2 = (float)((double)kLog2e * a.inv_tau);
     a.seed = p->seed; a.step = p->step;
     a.top_k = p->top_k; a.top_p = (double)p->top_p;
-    a.zp = logits_q; a.zq = logits_q; a.stride = row_stride;
-    a.stats = stats; a.lse = lse; a.score = score; a.depth = depth;
-    a.tile_sums = reinterpret_cast<double *>(ws + L.sums);
-    a.max_m = L.max_m; a.max_live = L.max_live;
-    a.hist = reinterpret_cast<unsigned long long *>(ws + L.hist);
-#ifdef DSBD_PHASE_TIMING
-    a.dbg = reinterpret_cast<unsigned long long *>(ws + L.total) - (size_t)R * 256;
-#endif
-    a.extra_layer_bias = (1u << 29) + (uint32_t)p->layer - 1u;     // layer number 2^29 + layer
-    a.out = dsbd_verify_out_t{};
-    a.out.l_last = reinterpret_cast<int32_t *>(ws + D.l_last);
-    a.out.out_width = reinterpret_cast<int32_t *>(ws + D.out_width);
-    a.out.out_off = out_off;
-    a.out.out_parent = out_parent;
-    a.out.out_node = reinterpret_cast<int32_t *>(ws + D.out_node);
-    a.out.out_root_beam = reinterpret_cast<int32_t *>(ws + D.out_root_beam);
-    a.out.out_token = out_token;
-    a.out.out_logp = reinterpret_cast<float *>(ws + D.out_logp);
-    a.out.out_logq = out_logq;
-    a.out.out_source = reinterpret_cast<int32_t *>(ws + D.out_source);
-    a.out.node_status = reinterpret_cast<int8_t *>(ws + D.node_status);
-    a.out.layer_width = reinterpret_cast<int32_t *>(ws + D.layer_width);
-    a.out.req_error = req_error;
-    a.status = status; a.select_mode = 0;
-    a.lse_w = lse; a.score_w = score; a.depth_w = depth;
-    a.root_logp = beam_logq; a.root_logq = beam_logq;
-    return launch_verify(a, R, L.max_live * L.T, stream);
+    a.zp = a.zq = logits_q; a.stride = row_stride;
+    TileStat *stats = reinterpret_cast<TileStat *>(ws + D.stats);
+    a.stats = stats;
+    a.lse = a.lse_w = reinterpret_cast<double *>(ws + D.lse);
+    a.status = status;
+    d.layer = (1u << 29) + (uint32_t)p->layer;
+    d.beam_logq = beam_logq;
+    d.W = p->W_S; d.W_r = p->W_S_r;
+    d.out_off = out_off; d.out_parent = out_parent; d.out_token = out_token; d.out_logq = out_logq;
+    d.req_error = req_error;
+
+    const int64_t items = (int64_t)n_beams * D.T;
+    k_tile_stats<<<stats_grid(items), kThreads, 0, stream>>>(logits_q, logits_q, row_stride, p->V, D.T, n_beams,
+                                                            n_beams, nullptr, nullptr, a.k2, stats, 1);
+    if (cudaGetLastError() != cudaSuccess) return DSBD_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)R);
+    cfg.blockDim = dim3(kVThreads);
+    cfg.dynamicSmemBytes = p->top_k > 0 ? kVerifyDynSmem : 0;           // the support's scratch
+    cfg.stream = stream;
+    if (p->top_k > 0 && cudaFuncSetAttribute(k_draft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess)
+        return DSBD_ERR_CUDA;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;       // see launch_verify
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_draft, d) == cudaSuccess ? DSBD_OK : DSBD_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------------------------------

@@ -115,6 +115,14 @@ def test_the_largest_live_set():
     _case(rng, [64, 64], 1500, 64, 2, top_k=64, top_p=0.9)
 
 
+@pytest.mark.parametrize("beams,V,W_S", [([1], 1, 1), ([3, 1], 7, 33), ([17, 16, 15], 1025, [31, 32, 65]), ([64], 70700, 9)])
+@pytest.mark.parametrize("top_k", [0, 3, 64])
+def test_widths_around_the_warps(beams, V, W_S, top_k):
+    """One token and one beam, more draws than lanes or warps, a support of every cell, 64 x 70 tile bounds (more
+    than are kept in shared memory)."""
+    _case(np.random.default_rng(V + top_k), beams, V, W_S, 2, top_k=top_k, top_p=0.9 if top_k else 1.0)
+
+
 def test_capacity_error_is_per_request():
     rng = np.random.default_rng(6)
     rbo, z, s = _problem(rng, [2, 3], 1000)

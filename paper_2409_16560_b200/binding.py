@@ -148,9 +148,21 @@ def _ptr(t):
 
 
 def _stream(stream):
+    # (the raw handle: making the Stream object takes 3 us, an eighth of a call's host time)
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream
+
+
+def _widest(off):
+    """Largest difference of neighbours (short arrays are faster as a list: 0.6 us, np.diff and max 2.3)."""
+    off = np.asarray(off)
+    d = off[1:] - off[:-1]
+    return max(d.tolist()) if 0 < len(d) <= 64 else int(d.max()) if len(d) else 0
+
+
+def _workspace(need, device):
+    return torch.empty(max(int(need), 256), dtype=torch.uint8, device=device)
 
 
 def _require_cuda(*tensors):
@@ -220,24 +232,15 @@ class Forest:
         self.device = device
 
     def struct(self):
-        f = ForestT()
-        f.R, f.B, f.N, f.max_depth = self.R, self.B, self.N, self.max_depth
-        for k in ("req_beam_off", "beam_node_off", "parent", "token", "draft_rank"):
-            setattr(f, k, _ptr(self.dev[k]))
-        f.max_tree_nodes = self.max_tree_nodes
-        f.max_req_beams = self.max_req_beams
-        f.max_layer_nodes = self.max_layer_nodes
-        return f
+        dev = self.dev
+        return ForestT(self.R, self.B, self.N, self.max_depth, _ptr(dev["req_beam_off"]), _ptr(dev["beam_node_off"]),
+                       _ptr(dev["parent"]), _ptr(dev["token"]), _ptr(dev["draft_rank"]), self.max_tree_nodes,
+                       self.max_req_beams, self.max_layer_nodes)
 
 
 def _attn_desc(Hq, Hkv, d, dtype, scale, prefix_off_host):
-    desc = AttnDescT()
-    desc.Hq, desc.Hkv, desc.d = Hq, Hkv, d
-    desc.dtype = DTYPE_BF16 if dtype == torch.bfloat16 else DTYPE_F32
-    desc.scale = float(scale)
-    desc.total_prefix = int(prefix_off_host[-1])
-    desc.max_prefix = int(np.diff(prefix_off_host).max()) if len(prefix_off_host) > 1 else 0
-    return desc
+    return AttnDescT(Hq, Hkv, d, DTYPE_BF16 if dtype == torch.bfloat16 else DTYPE_F32, float(scale),
+                     int(prefix_off_host[-1]), _widest(prefix_off_host))
 
 
 def forest_attention_workspace(forest, Hq, Hkv, d, dtype, scale, prefix_off_host):
@@ -261,9 +264,8 @@ def forest_attention(forest, Hq, Hkv, d, scale, q, k_new, v_new, k_prefix, v_pre
     desc = _attn_desc(Hq, Hkv, d, q.dtype, scale, prefix_off_host)
     if out is None:
         out = torch.empty_like(q)
-    need = int(load().dsbd_forest_attention_workspace(C.addressof(f), C.addressof(desc)))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device)
+        workspace = _workspace(load().dsbd_forest_attention_workspace(C.addressof(f), C.addressof(desc)), q.device)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=q.device)
     rc = load().dsbd_forest_attention(C.addressof(f), C.addressof(desc), _ptr(q), _ptr(k_new), _ptr(v_new),
@@ -301,7 +303,7 @@ def forest_build(req_beam_off, req_beam_off_host, gamma, W_S, draw_parent, draw_
         raise DsbdError("dsbd_forest_build", rc)
     f = Forest.from_device(R, B, N, gamma, arrays,
                            max_tree_nodes=int(largest.item()) if exact else 1 + gamma * W_S,
-                           max_req_beams=int(np.diff(rbo).max()), max_layer_nodes=W_S)
+                           max_req_beams=_widest(rbo), max_layer_nodes=W_S)
     return f, node_of_draw, status
 
 
@@ -330,9 +332,8 @@ def forest_attention_paged(forest, Hq, Hkv, d, scale, q, k_new, v_new, k_pool, v
         assert out.stride(0) == q.stride(0)
         pages.pool_layer_stride, pages.new_layer_stride = int(k_pool.stride(0)), int(k_new.stride(0))
         pages.q_layer_stride = int(q.stride(0))
-    need = int(load().dsbd_forest_attention_paged_workspace(C.addressof(f), C.addressof(desc), C.addressof(pages)))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=q.device)
+        workspace = _workspace(load().dsbd_forest_attention_paged_workspace(C.addressof(f), C.addressof(desc), C.addressof(pages)), q.device)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=q.device)
     rc = load().dsbd_forest_attention_paged(C.addressof(f), C.addressof(desc), _ptr(q), _ptr(k_new), _ptr(v_new),
@@ -360,22 +361,16 @@ def draft_layer(req_beam_off, req_beam_off_host, params, layer, W_S, logits_q, b
     dev = logits_q.device
     rbo = np.asarray(req_beam_off_host)
     R, n_beams = len(rbo) - 1, int(rbo[-1])
-    p = DraftParamsT()
-    p.V = int(params["V"])
-    p.temperature = float(params.get("temperature", 1.0))
+    width, width_r = W_S, None                 # (W_S itself stays: it may be the tensor's last reference)
     if torch.is_tensor(W_S):
         _require_cuda(W_S)
         assert W_S.dtype == torch.int32
-        p.W_S, p.W_S_r = 0, _ptr(W_S)
-    else:
-        p.W_S = int(W_S)
-    p.seed, p.step, p.layer = int(params.get("seed", 0)), int(params.get("step", 0)), int(layer)
-    p.top_k, p.top_p = int(params.get("top_k", 0)), float(params.get("top_p", 1.0))
-    p.n_slots = int(n_slots)
-    p.max_req_beams = int(np.diff(rbo).max())
-    need = int(load().dsbd_draft_workspace(R, n_beams, C.addressof(p)))
+        width, width_r = 0, _ptr(W_S)
+    p = DraftParamsT(int(params["V"]), float(params.get("temperature", 1.0)), int(width), width_r,
+                     int(params.get("seed", 0)), int(params.get("step", 0)), int(layer), int(params.get("top_k", 0)),
+                     float(params.get("top_p", 1.0)), int(n_slots), _widest(rbo))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+        workspace = _workspace(load().dsbd_draft_workspace(R, n_beams, C.addressof(p)), dev)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=dev)
     res = out if out is not None else dict(
@@ -414,9 +409,8 @@ def kv_commit(forest, Hkv, d, out_off, out_width, out_parent, out_root_beam, out
         k_dst = torch.empty(int(dst_capacity) * Hkv * d, dtype=k_new.dtype, device=dev)
     if v_dst is None:
         v_dst = torch.empty(int(dst_capacity) * Hkv * d, dtype=k_new.dtype, device=dev)
-    need = int(load().dsbd_kv_commit_workspace(C.addressof(f), C.addressof(p)))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+        workspace = _workspace(load().dsbd_kv_commit_workspace(C.addressof(f), C.addressof(p)), dev)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=dev)
     if out is not None:
@@ -461,9 +455,8 @@ def kv_commit_paged(forest, Hkv, d, out_off, out_width, out_parent, out_root_bea
         assert k_new.dim() == 4 and k_new.shape[0] == p.n_layers
     pages.page_table, pages.page_off = _ptr(page_table), _ptr(page_off)
     pages.n_pages = int(k_pool.shape[-4])
-    need = int(load().dsbd_kv_commit_paged_workspace(C.addressof(f), C.addressof(p), pages.n_pages))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+        workspace = _workspace(load().dsbd_kv_commit_paged_workspace(C.addressof(f), C.addressof(p), pages.n_pages), dev)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=dev)
     res = out if out is not None else dict(
@@ -486,25 +479,18 @@ def kv_commit_paged(forest, Hkv, d, out_off, out_width, out_parent, out_root_bea
 
 
 def _params(params, keep):
-    p = VerifyParamsT()
-    p.V = int(params["V"])
-    p.temperature = float(params.get("temperature", 1.0))
-    p.thresh = float(params.get("thresh", 0.7))
-    p.W_min = int(params.get("W_min", 1))
-    p.W_max = int(params.get("W_max", 1 << 30))
-    p.W_nom = int(params.get("W_nom", 1))
+    get = params.get
+    per_request = []
     for name in ("W_min_r", "W_max_r", "W_nom_r"):
-        t = params.get(name)
+        t = get(name)
         if t is not None:
             _require_cuda(t)
             assert t.dtype == torch.int32
             keep.append(t)
-            setattr(p, name, _ptr(t))
-    p.seed = int(params.get("seed", 0))
-    p.step = int(params.get("step", 0))
-    p.top_k = int(params.get("top_k", 0))
-    p.top_p = float(params.get("top_p", 1.0))
-    return p
+        per_request.append(_ptr(t))
+    return VerifyParamsT(int(params["V"]), float(get("temperature", 1.0)), float(get("thresh", 0.7)),
+                         int(get("W_min", 1)), int(get("W_max", 1 << 30)), int(get("W_nom", 1)), *per_request,
+                         int(get("seed", 0)), int(get("step", 0)), int(get("top_k", 0)), float(get("top_p", 1.0)))
 
 
 def verify_workspace(forest, params):
@@ -566,12 +552,9 @@ def verify_step(forest, params, logits_p, logits_q, root_logp, root_logq, out, w
     keep = []
     f = forest.struct()
     p = _params(params, keep)
-    o = VerifyOutT()
-    for name in _OUT_FIELDS:
-        setattr(o, name, _ptr(out[name]))
-    need = int(load().dsbd_verify_workspace(C.addressof(f), C.addressof(p)))
+    o = VerifyOutT(*[_ptr(out[name]) for name in _OUT_FIELDS])
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=logits_p.device)
+        workspace = _workspace(load().dsbd_verify_workspace(C.addressof(f), C.addressof(p)), logits_p.device)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=logits_p.device)
     stride = int(row_stride) if row_stride is not None else logits_p.stride(0)
@@ -594,9 +577,8 @@ def node_stats(forest, params, logits_p, logits_q, lse_p=None, lse_q=None, works
         lse_p = torch.empty(forest.N, dtype=torch.float32, device=dev)
     if lse_q is None:
         lse_q = torch.empty(forest.N, dtype=torch.float32, device=dev)
-    need = int(load().dsbd_verify_workspace(C.addressof(f), C.addressof(p)))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+        workspace = _workspace(load().dsbd_verify_workspace(C.addressof(f), C.addressof(p)), dev)
     rc = load().dsbd_node_stats(C.addressof(f), C.addressof(p), _ptr(logits_p), _ptr(logits_q),
                                 logits_p.stride(0), _ptr(lse_p), _ptr(lse_q), _ptr(workspace),
                                 workspace.numel(), _stream(stream))
@@ -636,9 +618,8 @@ def select_width(forest, params, logits_p, logits_q, node_logp, node_logq, live_
     width = torch.zeros(forest.R, dtype=torch.int32, device=dev)
     alpha = torch.zeros(forest.R, out_stride, dtype=torch.float32, device=dev) if want_alpha else None
     tail = torch.zeros(forest.R, out_stride, dtype=torch.float32, device=dev) if want_alpha else None
-    need = int(load().dsbd_verify_workspace(C.addressof(f), C.addressof(p)))
     if workspace is None:
-        workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+        workspace = _workspace(load().dsbd_verify_workspace(C.addressof(f), C.addressof(p)), dev)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=dev)
     rc = load().dsbd_select_width(C.addressof(f), C.addressof(p), _ptr(logits_p), _ptr(logits_q),

@@ -7,7 +7,7 @@
 // prefix is streamed once per unit.
 //
 // k_forest_attn_simt  fp32-accumulating CUDA-core kernel for any dtype: K/V tiles are staged
-//                     in shared memory with 128-bit loads, one thread pair per query row.
+//                     in shared memory with 128-bit loads, one to four thread pairs per query row.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -18,23 +18,24 @@ using namespace dsbd;
 
 namespace {
 
-constexpr int kRowsPerBlock = 64;     // query rows per CTA (two threads each)
+constexpr int kThreads = 128;
+constexpr int kRowsPerBlock = 64;     // query rows per CTA at two threads a row
 constexpr int kTok = 32;              // tokens per staged tile
+constexpr int kChunk = 8;             // tokens a thread takes between two updates of its running maximum
 
 template <class T> struct Elem;
 template <> struct Elem<float> {
     static constexpr int kPerVec = 4;
-    __device__ static void load(const float *p, float *dst) {
-        const float4 v = *reinterpret_cast<const float4 *>(p);
-        dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w;
+    __device__ static void widen(const uint4 &v, float *dst) {
+        dst[0] = __uint_as_float(v.x); dst[1] = __uint_as_float(v.y);
+        dst[2] = __uint_as_float(v.z); dst[3] = __uint_as_float(v.w);
     }
     __device__ static float to_float(float v) { return v; }
     __device__ static float from_float(float v) { return v; }
 };
 template <> struct Elem<__nv_bfloat16> {
     static constexpr int kPerVec = 8;
-    __device__ static void load(const __nv_bfloat16 *p, float *dst) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(p);
+    __device__ static void widen(const uint4 &v, float *dst) {
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -55,34 +56,28 @@ struct AttnArgs {
     void *out;
     int32_t *status;
     int row_blocks;
+    int splits;                    // thread pairs per query row
 };
 
-// Stage `cnt` (<= kTok) rows of d elements, row i at src + i*row_stride, into fp32 smem.
+// A row belongs to `splits` pairs of neighbouring threads; a pair takes every splits-th token, its two threads
+// every other four elements of it.  This kernel serves small calls, whose time is latency: few CTAs, each a
+// chain of tiles.  So the next tile's K and V are on their way in registers while one is worked on, small trees use
+// the threads that have no row of their own for tokens (4 pairs up to 16 rows, 2 up to 32: a tile's work is the
+// chain's step), and the parents are read at once.  Smem rows are padded by 32 bytes: the 16-byte words that
+// the pairs of a row and the threads of a pair read together lie in different banks.
+// fp32, one thread pair a row, tiles loaded when needed, parents read one by one against this: 2 beams x 15 nodes x
+// 4 heads of 64 after 64 tokens 22.7 and 13.7 us a call; 8 requests, 6 nodes, 8 heads of 64 after 200-600 tokens
+// 174 and 47; 40 requests, 24 rows a unit 507 and 143; heads of 128 in groups of 4 334 and 158.
 template <class T, int D>
-__device__ void stage_rows(const T *src, int64_t row_stride, int cnt, float *dst, int tid, int nthreads) {
-    constexpr int PV = Elem<T>::kPerVec;
-    constexpr int VPR = D / PV;           // vectors per row
-    for (int i = tid; i < kTok * VPR; i += nthreads) {
-        const int row = i / VPR, c = (i - row * VPR) * PV;
-        float tmp[PV];
-        if (row < cnt) {
-            Elem<T>::load(src + (int64_t)row * row_stride + c, tmp);
-        } else {
-#pragma unroll
-            for (int e = 0; e < PV; ++e) tmp[e] = 0.f;
-        }
-#pragma unroll
-        for (int e = 0; e < PV; ++e) dst[row * D + c + e] = tmp[e];
-    }
-}
-
-template <class T, int D>
-__global__ void __launch_bounds__(2 * kRowsPerBlock)
+__global__ void __launch_bounds__(kThreads)
 k_forest_attn_simt(AttnArgs a) {
-    constexpr int H = D / 2;              // elements per thread of the pair
-    extern __shared__ float smem[];
-    float *ks = smem;                     // [kTok][D]
-    float *vs = smem + kTok * D;          // [kTok][D]
+    constexpr int H = D / 2;              // elements per thread of a pair
+    constexpr int RS = D + 8;             // floats from one staged row to the next
+    constexpr int PV = Elem<T>::kPerVec, VPR = D / PV, NV = kTok * VPR / kThreads;
+    extern __shared__ __align__(16) float smem[];
+    float *ks = smem;                     // [kTok][RS]
+    float *vs = smem + kTok * RS;         // [kTok][RS]
+    __shared__ int par_s[DSBD_MAX_TREE_NODES];
     __shared__ unsigned long long anc[DSBD_MAX_TREE_NODES];
 
     int unit = blockIdx.x;
@@ -92,37 +87,9 @@ k_forest_attn_simt(AttnArgs a) {
     const int n_lo = a.beam_node_off[b];
     const int n_tree = a.beam_node_off[b + 1] - n_lo;
     const int M = n_tree * a.group;
-    if (rb * kRowsPerBlock >= M) return;
-    const int tid = threadIdx.x, nthreads = blockDim.x;
-
-    // ancestor-or-self bitmasks of the tree: anc[i] = anc[parent(i)] | bit(i)
-    if (tid == 0) {
-        for (int i = 0; i < n_tree; ++i) {
-            const int par = a.parent[n_lo + i];
-            unsigned long long m = 1ull << i;
-            if (par >= n_lo && par < n_lo + i) m |= anc[par - n_lo];
-            else if (par != -1 || i != 0) report(a.status, DSBD_DEV_BAD_FOREST);
-            anc[i] = m;
-        }
-    }
-
-    const int row = rb * kRowsPerBlock + (tid >> 1);     // query row inside the unit
-    const int half = tid & 1;
-    const bool active = row < M;
-    const int node = active ? row / a.group : 0;          // tree-local node
-    const int hq = g * a.group + (active ? row % a.group : 0);
-    const T *Q = static_cast<const T *>(a.q);
-    float qv[H], o[H];
-#pragma unroll
-    for (int c = 0; c < H; ++c) {
-        qv[c] = active ? Elem<T>::to_float(Q[((int64_t)(n_lo + node) * a.Hq + hq) * D + half * H + c]) *
-                             a.scale_log2
-                       : 0.f;
-        o[c] = 0.f;
-    }
-    float mrun = -INFINITY, lrun = 0.f;
-    __syncthreads();
-    const unsigned long long my_anc = anc[node];
+    const int rows = kRowsPerBlock / a.splits;
+    if (rb * rows >= M) return;
+    const int tid = threadIdx.x;
 
     const int64_t L = a.prefix_off[b + 1] - a.prefix_off[b];
     const T *kp = static_cast<const T *>(a.k_prefix) + (a.prefix_off[b] * a.Hkv + (int64_t)g * L) * D;
@@ -130,80 +97,155 @@ k_forest_attn_simt(AttnArgs a) {
     const T *kn = static_cast<const T *>(a.k_new) + ((int64_t)n_lo * a.Hkv + g) * D;
     const T *vn = static_cast<const T *>(a.v_new) + ((int64_t)n_lo * a.Hkv + g) * D;
 
-    const int64_t total = L + n_tree;
-    for (int64_t t0 = 0; t0 < total; t0 += kTok) {
-        // a tile never straddles the prefix / tree boundary
-        const bool in_tree = t0 >= L;
-        int cnt;
-        if (!in_tree) {
-            cnt = (int)((L - t0) < kTok ? (L - t0) : kTok);
-            stage_rows<T, D>(kp + t0 * D, D, cnt, ks, tid, nthreads);
-            stage_rows<T, D>(vp + t0 * D, D, cnt, vs, tid, nthreads);
-        } else {
-            const int j0 = (int)(t0 - L);
-            cnt = (n_tree - j0) < kTok ? (n_tree - j0) : kTok;
-            stage_rows<T, D>(kn + (int64_t)j0 * a.Hkv * D, (int64_t)a.Hkv * D, cnt, ks, tid, nthreads);
-            stage_rows<T, D>(vn + (int64_t)j0 * a.Hkv * D, (int64_t)a.Hkv * D, cnt, vs, tid, nthreads);
-        }
-        __syncthreads();
-        float s[kTok];
-        float tmax = -INFINITY;
-#pragma unroll 4
-        for (int j = 0; j < kTok; ++j) {
-            const float4 *kr = reinterpret_cast<const float4 *>(ks + j * D + half * H);
-            float acc = 0.f;
+    // a tile never straddles the prefix / tree boundary
+    const int64_t p_tiles = (L + kTok - 1) / kTok, n_tiles = p_tiles + (n_tree + kTok - 1) / kTok;
+    uint4 kr[NV], vr[NV];
+    auto tile_tokens = [&](int64_t t) -> int {
+        return (int)(t < p_tiles ? min((int64_t)kTok, L - t * kTok) : min((int64_t)kTok, n_tree - (t - p_tiles) * kTok));
+    };
+    auto load = [&](int64_t t) {
+        const int cnt = tile_tokens(t);
+        const bool in_tree = t >= p_tiles;
+        const int64_t stride = in_tree ? (int64_t)a.Hkv * D : D;
+        const int64_t first = in_tree ? (t - p_tiles) * kTok * stride : t * kTok * stride;
+        const T *kt = (in_tree ? kn : kp) + first, *vt = (in_tree ? vn : vp) + first;
 #pragma unroll
-            for (int c = 0; c < H / 4; ++c) {
-                const float4 kv = kr[c];
-                acc = fmaf(qv[4 * c], kv.x, acc);
-                acc = fmaf(qv[4 * c + 1], kv.y, acc);
-                acc = fmaf(qv[4 * c + 2], kv.z, acc);
-                acc = fmaf(qv[4 * c + 3], kv.w, acc);
+        for (int i = 0; i < NV; ++i) {
+            const int at = i * kThreads + tid, row = at / VPR, c = (at - row * VPR) * PV;
+            kr[i] = row < cnt ? *reinterpret_cast<const uint4 *>(kt + row * stride + c) : make_uint4(0, 0, 0, 0);
+            vr[i] = row < cnt ? *reinterpret_cast<const uint4 *>(vt + row * stride + c) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    auto store = [&] {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int at = i * kThreads + tid, row = at / VPR, c = (at - row * VPR) * PV;
+            float k[PV], v[PV];
+            Elem<T>::widen(kr[i], k);
+            Elem<T>::widen(vr[i], v);
+#pragma unroll
+            for (int e = 0; e < PV; e += 4) {
+                *reinterpret_cast<float4 *>(ks + row * RS + c + e) = make_float4(k[e], k[e + 1], k[e + 2], k[e + 3]);
+                *reinterpret_cast<float4 *>(vs + row * RS + c + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
             }
-            acc += __shfl_xor_sync(kFull, acc, 1);
-            bool vis = j < cnt;
-            if (in_tree) vis = vis && ((my_anc >> ((int)(t0 - L) + j)) & 1ull);
-            s[j] = vis ? acc : -INFINITY;
-            tmax = fmaxf(tmax, s[j]);
         }
-        if (tmax > -INFINITY) {
-            const float mnew = fmaxf(mrun, tmax);
-            const float corr = exp2f(mrun - mnew);      // 0 when mrun == -inf
-            lrun *= corr;
+    };
+    load(0);
+
+    const int pair = tid >> 1, half = tid & 1;
+    const int split = pair % a.splits, row = rb * rows + pair / a.splits;   // query row inside the unit
+    const bool active = row < M;
+    const int node = active ? row / a.group : 0;          // tree-local node
+    const int hq = g * a.group + (active ? row % a.group : 0);
+    const T *Q = static_cast<const T *>(a.q) + ((int64_t)(n_lo + node) * a.Hq + hq) * D;
+    // element e of the thread's H: 4 (2 (e / 4) + half) + e % 4 of the row
+    float qv[H], o[H];
 #pragma unroll
-            for (int c = 0; c < H; ++c) o[c] *= corr;
-#pragma unroll 4
-            for (int j = 0; j < kTok; ++j) {
-                const float p = exp2f(s[j] - mnew);      // 0 for masked entries
-                lrun += p;
-                const float4 *vr = reinterpret_cast<const float4 *>(vs + j * D + half * H);
+    for (int e = 0; e < H; ++e) {
+        qv[e] = active ? Elem<T>::to_float(Q[4 * (2 * (e / 4) + half) + e % 4]) * a.scale_log2 : 0.f;
+        o[e] = 0.f;
+    }
+    float mrun = -INFINITY, lrun = 0.f;
+    if (tid < n_tree) par_s[tid] = a.parent[n_lo + tid];
+    __syncthreads();
+    // ancestor-or-self bitmasks of the tree
+    if (tid < n_tree) {
+        unsigned long long m = 0ull;
+        for (int i = tid; ;) {
+            m |= 1ull << i;
+            const int par = par_s[i];
+            if (par < n_lo || par >= n_lo + i) {
+                if (i == tid && (par != -1 || i != 0)) report(a.status, DSBD_DEV_BAD_FOREST);
+                break;
+            }
+            i = par - n_lo;
+        }
+        anc[tid] = m;
+    }
+    __syncthreads();
+    const unsigned long long my_anc = anc[node];
+
+    for (int64_t t = 0; t < n_tiles; ++t) {
+        store();
+        __syncthreads();
+        if (t + 1 < n_tiles) load(t + 1);
+        const int cnt = tile_tokens(t);
+        const unsigned visible = t < p_tiles ? kFull : (unsigned)(my_anc >> ((t - p_tiles) * kTok));
+#pragma unroll 1
+        for (int j0 = split; j0 < cnt; j0 += kChunk * a.splits) {
+            float s[kChunk];
+            float tmax = -INFINITY;
+#pragma unroll
+            for (int i = 0; i < kChunk; ++i) {
+                const int j = j0 + i * a.splits;
+                const float4 *row4 = reinterpret_cast<const float4 *>(ks + j * RS) + half;
+                float acc = 0.f;
 #pragma unroll
                 for (int c = 0; c < H / 4; ++c) {
-                    const float4 vv = vr[c];
-                    o[4 * c] = fmaf(p, vv.x, o[4 * c]);
-                    o[4 * c + 1] = fmaf(p, vv.y, o[4 * c + 1]);
-                    o[4 * c + 2] = fmaf(p, vv.z, o[4 * c + 2]);
-                    o[4 * c + 3] = fmaf(p, vv.w, o[4 * c + 3]);
+                    const float4 kv = row4[2 * c];
+                    acc = fmaf(qv[4 * c], kv.x, acc);
+                    acc = fmaf(qv[4 * c + 1], kv.y, acc);
+                    acc = fmaf(qv[4 * c + 2], kv.z, acc);
+                    acc = fmaf(qv[4 * c + 3], kv.w, acc);
                 }
+                s[i] = acc;
             }
-            mrun = mnew;
+            // (the pairs of a warp differ in their number of chunks: a pair's two threads do not)
+#pragma unroll
+            for (int i = 0; i < kChunk; ++i) {
+                const int j = j0 + i * a.splits;
+                s[i] += __shfl_xor_sync(3u << (tid & 30), s[i], 1);
+                if (j >= cnt || !(visible >> j & 1u)) s[i] = -INFINITY;
+                tmax = fmaxf(tmax, s[i]);
+            }
+            if (tmax > -INFINITY) {
+                const float mnew = fmaxf(mrun, tmax);
+                const float corr = exp2f(mrun - mnew);      // 0 when mrun == -inf
+                lrun *= corr;
+#pragma unroll
+                for (int e = 0; e < H; ++e) o[e] *= corr;
+#pragma unroll
+                for (int i = 0; i < kChunk; ++i) {
+                    const int j = j0 + i * a.splits;
+                    const float p = exp2f(s[i] - mnew);      // 0 for masked entries
+                    lrun += p;
+                    const float4 *row4 = reinterpret_cast<const float4 *>(vs + j * RS) + half;
+#pragma unroll
+                    for (int c = 0; c < H / 4; ++c) {
+                        const float4 vv = row4[2 * c];
+                        o[4 * c] = fmaf(p, vv.x, o[4 * c]);
+                        o[4 * c + 1] = fmaf(p, vv.y, o[4 * c + 1]);
+                        o[4 * c + 2] = fmaf(p, vv.z, o[4 * c + 2]);
+                        o[4 * c + 3] = fmaf(p, vv.w, o[4 * c + 3]);
+                    }
+                }
+                mrun = mnew;
+            }
         }
         __syncthreads();
-        if (!in_tree && t0 + kTok > L) t0 = L - kTok;   // next tile starts the tree part
     }
-    if (active) {
-        T *O = static_cast<T *>(a.out);
+    // the pairs of a row
+    for (int off = 2; off < 2 * a.splits; off *= 2) {
+        const float m2 = __shfl_xor_sync(kFull, mrun, off), l2 = __shfl_xor_sync(kFull, lrun, off);
+        const float mnew = fmaxf(mrun, m2);
+        const float c1 = mrun > -INFINITY ? exp2f(mrun - mnew) : 0.f, c2 = m2 > -INFINITY ? exp2f(m2 - mnew) : 0.f;
+        lrun = lrun * c1 + l2 * c2;
+#pragma unroll
+        for (int e = 0; e < H; ++e) o[e] = o[e] * c1 + __shfl_xor_sync(kFull, o[e], off) * c2;
+        mrun = mnew;
+    }
+    if (active && split == 0) {
+        T *O = static_cast<T *>(a.out) + ((int64_t)(n_lo + node) * a.Hq + hq) * D;
         const float inv = 1.f / lrun;
 #pragma unroll
-        for (int c = 0; c < H; ++c)
-            O[((int64_t)(n_lo + node) * a.Hq + hq) * D + half * H + c] = Elem<T>::from_float(o[c] * inv);
+        for (int e = 0; e < H; ++e) O[4 * (2 * (e / 4) + half) + e % 4] = Elem<T>::from_float(o[e] * inv);
     }
 }
 
 template <class T, int D>
 int launch_simt(const AttnArgs &a, int units, cudaStream_t stream) {
-    const size_t smem = sizeof(float) * 2 * kTok * D;
-    k_forest_attn_simt<T, D><<<units, 2 * kRowsPerBlock, smem, stream>>>(a);
+    const size_t smem = sizeof(float) * 2 * kTok * (D + 8);
+    k_forest_attn_simt<T, D><<<units, kThreads, smem, stream>>>(a);
     return cudaGetLastError() == cudaSuccess ? DSBD_OK : DSBD_ERR_CUDA;
 }
 
@@ -262,7 +304,8 @@ extern "C" int dsbd_forest_attention(const dsbd_forest_t *f, const dsbd_attn_des
     a.q = q; a.k_new = k_new; a.v_new = v_new; a.k_prefix = k_prefix; a.v_prefix = v_prefix;
     a.out = out; a.status = status;
     const int max_rows = f->max_tree_nodes * a.group;
-    a.row_blocks = (max_rows + kRowsPerBlock - 1) / kRowsPerBlock;
+    a.splits = max_rows <= kRowsPerBlock / 4 ? 4 : max_rows <= kRowsPerBlock / 2 ? 2 : 1;
+    a.row_blocks = (max_rows * a.splits + kRowsPerBlock - 1) / kRowsPerBlock;
     const int units = f->B * d->Hkv * a.row_blocks;
     if (d->dtype == DSBD_DTYPE_F32)
         return d->d == 64 ? launch_simt<float, 64>(a, units, stream) : launch_simt<float, 128>(a, units, stream);

@@ -98,6 +98,22 @@ def test_ragged_prefixes_and_tree_shapes(dtype, Hq, Hkv, d):
     attention_close(to_host_f32(out), ref, bf16=dtype == torch.bfloat16)
 
 
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 64), (torch.float32, 128), (torch.bfloat16, 64)])
+@pytest.mark.parametrize("max_rows", [1, 16, 17, 32, 33, 64])
+def test_cuda_core_kernel_row_splits(dtype, d, max_rows):
+    """Query rows around the sizes where a row has 4, 2 or 1 thread pairs, prefixes around the 32-token tile and
+    around the tokens that a pair takes between two updates (bf16 runs here with a group beyond the tensor cores')."""
+    rng = np.random.default_rng(max_rows + d)
+    rand_tree = lambda n: [-1] + [int(rng.integers(0, i)) for i in range(1, n)]
+    group = 1 if dtype == torch.float32 else 65
+    trees = [rand_tree(max_rows), [-1], rand_tree((max_rows + 1) // 2), rand_tree(max_rows)]
+    L = [31, 0, 33, 200] if max_rows % 2 else [32, 1, 7, 65]
+    forest, spec, t, poff = _custom(rng, trees, L, 2 * group, 2, d, dtype)
+    out = _gpu(forest, spec, t, poff)
+    nodes, ref = _oracle_beams(forest, spec, t, poff, list(range(len(trees))))
+    attention_close(to_host_f32(out), ref, bf16=dtype == torch.bfloat16)
+
+
 @pytest.mark.parametrize("Hq,Hkv,max_nodes", [(8, 2, 32), (16, 2, 16), (4, 4, 64), (32, 8, 9), (40, 40, 20)])
 def test_tensor_core_kernel_row_counts(Hq, Hkv, max_nodes):
     """bf16, d = 128: the tcgen05 kernel with 64-row and with 128-row query tiles (nodes x group

@@ -300,7 +300,8 @@ def _side_workload(dsbd, inputs, dev, name, steps, warmup, top_k=0, top_p=1.0, p
 
 
 PHASE_NAMES = {1: "start", 2: "prologue / previous layer's completion", 3: "layer set-up", 4: "histogram pass",
-               5: "merge across the cluster", 7: "image and suffix sums", 8: "residual chain",
+               5: "wait for the cluster's slices", 6: "wait for the cluster's passes",
+               7: "merge and suffix sums of a slice", 8: "residual chain",
                9: "width and accept loop", 10: "residual pass for a completion draw", 11: "completion draws",
                12: "extra layer and final writes"}
 

@@ -195,7 +195,6 @@ struct VerifyArgs {
     const int32_t *depth;     // [N]
     double *tile_sums;        // [R][2][max_m+1][max_live*T]: per bank the histogram pass's sums (half tiles may take
                               // two slots), then those of the exact pass at j >= 2 in slot j
-    unsigned long long *hist; // [R][2 banks][kBins+1] fixed-point ratio histograms (p<<32 | q)
     unsigned long long *dbg;  // phase time stamps (DSBD_PHASE_TIMING builds only)
     // verify mode computes the row and tree statistics of its own request first
     double *lse_w, *score_w;
@@ -240,9 +239,9 @@ struct Shared {
     int n_layers, n_tests, n_exact, n_respass;
     int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows consulted
     unsigned long long wtot_p[kVWarps], wtot_q[kVWarps];
-    double n_cells;                         // cells that entered the layer's histogram
+    unsigned long long slice_p[16], slice_q[16];   // mass of the bins of every CTA's slice
     unsigned long long w_tot[2][10];        // per bank, sums of one histogram pass: see histogram_pass / hist_fold_over
-    int wrapped, n_wrapped;                 // a w word of the layer's histogram wrapped; layers where that happened
+    int n_wrapped;                          // layers where a w word of the histogram wrapped
     double rho[kMaxLive], uu[kMaxLive];     // per live draft: p_beam/q_beam and its uniform
 };
 
@@ -533,9 +532,6 @@ static_assert(kHistWords % 4 == 0, "the arrays that share this memory need 16-by
 constexpr float kFix = 17592186044416.f;          // 2^44
 constexpr double kUnfix = 1.0 / 17592186044416.0;
 constexpr double kErrTol = 2.5e-7;                // error bound of F(s) above which it is recomputed exactly
-// global image of one histogram: P and Q of bin i at 2i, 2i+1 (units of 2^-44), two spare words
-constexpr int kHistLen = 2 * (kBins + 1) + 2;
-
 constexpr int kHistArrays = 4;
 struct HistSmem { uint32_t *wp, *wq, *bp, *bq; };
 
@@ -735,53 +731,97 @@ __device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, un
 }
 
 // Merge of the cluster's histograms, after a cluster barrier that follows the pass: every CTA sums one slice of
-// the bins over all CTAs' shared memory (16-byte distributed shared memory loads, no atomics) and stores the
-// 64-bit sums, in units of 2^-44, to the global image, which therefore needs no clearing.  A lane takes four
-// bins of two CTAs, so that all its loads are in flight together; the lanes that share bins add up by shuffles
-// (bound by latency: two barriers and one round of remote loads, 6 us for 8 CTAs, 8 for 16; a thread that
-// walked all CTAs' words of one bin took 7 and 9, with a sweep for the wraps before the first barrier).
-// tot[6] of every CTA then holds what all threads added, by their floating-point sums, minus what the words hold.
-// Without a wrap that is rounding: half a unit for each cell and 2^-20 of the mass (16 cells in a float sum), less
-// than 2^26 units; a wrap lowers the words by 2^32.  The caller puts a cluster barrier behind this before
-// anyone reads the image or tot[6] or reuses the arrays.
-__device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *gh,
-                           unsigned long long *tot, int cta_rank, int n_cta) {
+// the bins over all CTAs' shared memory.  A lane takes four bins of two CTAs (eight bins when there is one CTA), so
+// that all its loads are in flight together; the lanes that share bins add up by shuffles, and with 16 CTAs two
+// warps share bins.  The CTA's suffix sums (p and q mass of the slice's bins >= k, units of 2^-44) replace the words of
+// its own slice, which no other CTA reads here: w words the low, b words the high halves.  Every CTA
+// gets the slice's totals.  The caller puts a cluster barrier behind this before anyone looks at another's slice.
+// Bound by distributed shared memory (64 KB a CTA, 4.5 us), as long as an instruction takes at least 128 bytes from
+// each CTA it reads: with 64 bytes from each of 8, one warp to the bins, 16 CTAs took 7 to 10 us.  (512 bytes
+// an instruction and the sums of 2 to 8 warps through a stage of 16 KB were no faster with 8 CTAs, and the shared
+// memory came off the L1 cache: 64 requests x 8 rows of 128256 30 us slower.)
+__device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, Shared &sh, int cta_rank, int n_cta) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int share = n_cta > 1 ? n_cta / 2 : 1;             // lanes that share four bins
-    const int quads = kBins / 4 / n_cta, per_warp = 32 / share;
-    unsigned long long sum = 0ull;
-    for (int base = warp * per_warp; base < quads; base += kVWarps * per_warp) {
-        const int i = 4 * (cta_rank * quads + base + lane % per_warp);
-        unsigned long long P[4] = {}, Q[4] = {};
-        for (int c = lane / per_warp; c < n_cta; c += share) {
-            const uint4 wp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wp, c) + i);
-            const uint4 wq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wq, c) + i);
-            const uint4 bp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bp, c) + i);
-            const uint4 bq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bq, c) + i);
-            P[0] += ((unsigned long long)bp.x << 16) + wp.x; P[1] += ((unsigned long long)bp.y << 16) + wp.y;
-            P[2] += ((unsigned long long)bp.z << 16) + wp.z; P[3] += ((unsigned long long)bp.w << 16) + wp.w;
-            Q[0] += ((unsigned long long)bq.x << 16) + wq.x; Q[1] += ((unsigned long long)bq.y << 16) + wq.y;
-            Q[2] += ((unsigned long long)bq.z << 16) + wq.z; Q[3] += ((unsigned long long)bq.w << 16) + wq.w;
-        }
-        for (int o = per_warp; o < 32; o <<= 1) {
+    const int share = n_cta > 1 ? min(n_cta / 2, 4) : 1;     // lanes that share four bins
+    const int parts = n_cta > 8 ? 2 : 1;                     // warps that share them
+    const int per_warp = 32 / share, place = lane % per_warp, segs = kVWarps / parts;
+    const int seg = warp % segs, part = warp / segs;
+    const int n_bins = n_cta > 1 ? 4 : 8;                    // of a lane
+    const int i0 = cta_rank * (kBins / n_cta) + (seg * per_warp + place) * n_bins;
+    unsigned long long P[8] = {}, Q[8] = {};
+    auto add4 = [&](int c, int i, unsigned long long *p, unsigned long long *q) {
+        const uint4 wp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wp, c) + i);
+        const uint4 wq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wq, c) + i);
+        const uint4 bp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bp, c) + i);
+        const uint4 bq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bq, c) + i);
+        p[0] += ((unsigned long long)bp.x << 16) + wp.x; p[1] += ((unsigned long long)bp.y << 16) + wp.y;
+        p[2] += ((unsigned long long)bp.z << 16) + wp.z; p[3] += ((unsigned long long)bp.w << 16) + wp.w;
+        q[0] += ((unsigned long long)bq.x << 16) + wq.x; q[1] += ((unsigned long long)bq.y << 16) + wq.y;
+        q[2] += ((unsigned long long)bq.z << 16) + wq.z; q[3] += ((unsigned long long)bq.w << 16) + wq.w;
+    };
+    const int c0 = part * 8 + lane / per_warp;
+    if (n_cta > 1) {
+        add4(c0, i0, P, Q);
+        add4(c0 + share, i0, P, Q);
+    } else {
+        add4(0, i0, P, Q);
+        add4(0, i0 + 4, P + 4, Q + 4);
+    }
+    for (int o = per_warp; o < 32; o <<= 1) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                P[k] += __shfl_xor_sync(kFull, P[k], o);
-                Q[k] += __shfl_xor_sync(kFull, Q[k], o);
-            }
-        }
-        if (lane < per_warp) {
-            ulonglong2 *to = reinterpret_cast<ulonglong2 *>(gh + 2 * i);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                to[k] = make_ulonglong2(P[k], Q[k]);
-                sum += P[k] + Q[k];
-            }
+        for (int k = 0; k < 4; ++k) {
+            P[k] += __shfl_xor_sync(kFull, P[k], o);
+            Q[k] += __shfl_xor_sync(kFull, Q[k], o);
         }
     }
+    auto store4 = [&](int i, const unsigned long long *p, const unsigned long long *q, unsigned long long rp, unsigned long long rq) {
+        auto words = [&](uint32_t *low, uint32_t *high, const unsigned long long *v, unsigned long long r) {
+            *reinterpret_cast<uint4 *>(low + i) = make_uint4((uint32_t)(v[0] + r), (uint32_t)(v[1] + r), (uint32_t)(v[2] + r), (uint32_t)(v[3] + r));
+            *reinterpret_cast<uint4 *>(high + i) = make_uint4((uint32_t)((v[0] + r) >> 32), (uint32_t)((v[1] + r) >> 32),
+                                                             (uint32_t)((v[2] + r) >> 32), (uint32_t)((v[3] + r) >> 32));
+        };
+        words(h.wp, h.bp, p, rp);
+        words(h.wq, h.bq, q, rq);
+    };
+    if (parts == 2) {
+        // the second warp's sums through the slice itself, once the whole CTA has read its own words there
+        __syncthreads();
+        if (part == 1 && lane < per_warp) store4(i0, P, Q, 0ull, 0ull);
+        __syncthreads();
+        if (part == 0) {
+            const uint4 lp = *reinterpret_cast<const uint4 *>(h.wp + i0), up = *reinterpret_cast<const uint4 *>(h.bp + i0);
+            const uint4 lq = *reinterpret_cast<const uint4 *>(h.wq + i0), uq = *reinterpret_cast<const uint4 *>(h.bq + i0);
+            auto whole = [](uint32_t low, uint32_t high) { return ((unsigned long long)high << 32) | low; };
+            P[0] += whole(lp.x, up.x); P[1] += whole(lp.y, up.y); P[2] += whole(lp.z, up.z); P[3] += whole(lp.w, up.w);
+            Q[0] += whole(lq.x, uq.x); Q[1] += whole(lq.y, uq.y); Q[2] += whole(lq.z, uq.z); Q[3] += whole(lq.w, uq.w);
+        }
+    }
+    // suffix sums: in the lane, over the lanes' places, over the warps of part 0
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
-    if (lane < n_cta && sum) atomicAdd(cluster.map_shared_rank(tot, lane) + 6, 0ull - sum);
+    for (int k = 6; k >= 0; --k) { P[k] += P[k + 1]; Q[k] += Q[k + 1]; }
+    unsigned long long ap = P[0], aq = Q[0];
+    for (int o = 1; o < per_warp; o <<= 1) {
+        const unsigned long long tp = __shfl_down_sync(kFull, ap, o), tq = __shfl_down_sync(kFull, aq, o);
+        if (place + o < per_warp) { ap += tp; aq += tq; }
+    }
+    if (part == 0 && lane == 0) { sh.wtot_p[seg] = ap; sh.wtot_q[seg] = aq; }
+    __syncthreads();
+    if (part > 0) return;
+    unsigned long long rp = ap - P[0], rq = aq - Q[0];
+    for (int w = seg + 1; w < segs; ++w) { rp += sh.wtot_p[w]; rq += sh.wtot_q[w]; }
+    if (lane < per_warp) {
+        store4(i0, P, Q, rp, rq);
+        if (n_cta == 1) store4(i0 + 4, P + 4, Q + 4, rp, rq);
+    }
+    if (seg == 0) {
+        // place 0: the whole slice
+        const unsigned long long tp = __shfl_sync(kFull, P[0] + rp, 0), tq = __shfl_sync(kFull, Q[0] + rq, 0);
+        if (lane < n_cta) {
+            Shared *to = cluster.map_shared_rank(&sh, lane);
+            to->slice_p[cta_rank] = tp;
+            to->slice_q[cta_rank] = tq;
+        }
+    }
 }
 
 // One completion draw (residual if s_res > 0 else p_beam) by one warp; returns the token or -1
@@ -1119,9 +1159,8 @@ __device__ void finish_supports(WarpScratch &ws, bool have_q, int lane) {
 #endif
 
 // dynamic shared memory of k_verify: the histogram of a layer as four 32-bit arrays while it is
-// being built, then (over the same bytes) the 64-bit suffix sums of its p and q mass
+// being built, then (over the same bytes) this CTA's slice of the suffix sums of its p and q mass
 constexpr size_t kVerifyDynSmem = kHistArrays * sizeof(uint32_t) * kHistWords;
-static_assert(2 * sizeof(unsigned long long) * kHistWords <= kVerifyDynSmem, "the suffix sums fit over the building arrays");
 
 __global__ void __launch_bounds__(kVThreads, 2)
 k_verify(const __grid_constant__ VerifyArgs a) {
@@ -1139,7 +1178,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     uint32_t *hp = reinterpret_cast<uint32_t *>(dyn_smem), *hq = hp + kHistWords;     // first two digit arrays
     const HistSmem hs = hist_arrays(hp);
-    unsigned long long *sufP = reinterpret_cast<unsigned long long *>(dyn_smem), *sufQ = sufP + kHistWords;
 
     const int b_lo = a.req_beam_off[r], b_hi = a.req_beam_off[r + 1];
     const int n_lo = a.beam_node_off[b_lo], n_hi = a.beam_node_off[b_hi];
@@ -1152,8 +1190,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     if (bad_widths) { W_min = W_max = W_nom = 1; }
     double *sums_base = a.tile_sums + (int64_t)r * 2 * (a.max_m + 1) * ((int64_t)a.max_live * a.T);
     const int64_t slot_stride = (int64_t)a.max_live * a.T;
-    unsigned long long *ghist = a.hist + (int64_t)r * 2 * kHistLen;        // [2 banks][kHistLen]
-    const int hist_len = kHistLen;
     int n_out = 0;
 #ifdef DSBD_PHASE_TIMING
     int ts_n = 0;
@@ -1495,6 +1531,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         }
         __syncthreads();
         const int m = sh.m;
+        bool looked_up = false;
         TS(3);
 
         const bool warped = a.top_k > 0;
@@ -1545,7 +1582,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             // ---- one pass: ratio histogram of the layer over the live rows ----
             const double top = log2((double)(m > 2 ? m : 2));          // s_j <= j <= m
             const float binscale = (float)((double)kBins / top);
-            unsigned long long *gh = ghist + sh.bank * hist_len;
             unsigned long long *tot = sh.w_tot[sh.bank];
             // half tiles as items where whole ones would leave a part of the last round's warps idle: a warp's own
             // work is the pass's length there (V = 32000, 16 CTAs: 3 rows 4.5 us instead of 7)
@@ -1557,75 +1593,69 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             hist_fold_over(cluster, hs, tot, n_cta);
             TS(4);
             cluster.sync();                            // every CTA's histogram is complete
+            TS(6);
             if (threadIdx.x < 10) sh.w_tot[sh.bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
                                                        // the barrier below
-            hist_merge(cluster, hs, gh, tot, cta_rank, n_cta);
-            cluster.sync();                            // the image is whole (the barrier orders the stores for
-                                                       // the cluster); nobody reads the arrays any more
-            TS(5);
-            // Suffix sums of the merged histogram into shared memory (over the building arrays): sufP[k] = p mass of
-            // the bins >= k.  A thread takes kPer consecutive bins in registers from the image to the sums, two bins a
-            // load (3.6 us; image, then sums in place through shared memory, took 3.8 to 4.5).
-            {
-                constexpr int kPer = kBins / kVThreads;
-                unsigned long long bp_[kPer], bq_[kPer], mp_ = 0ull, mq_ = 0ull;
-                const unsigned long long *src = gh + 2 * kPer * threadIdx.x;
-#pragma unroll
-                for (int i = 0; i < kPer; i += 2)
-                    asm volatile("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];"
-                                 : "=l"(bp_[i]), "=l"(bq_[i]), "=l"(bp_[i + 1]), "=l"(bq_[i + 1]) : "l"(src + 2 * i) : "memory");
-#pragma unroll
-                for (int i = 0; i < kPer; ++i) { mp_ += bp_[i]; mq_ += bq_[i]; }
-                unsigned long long ap = mp_, aq = mq_;    // suffix scan inside the warp, top lane down
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long tp = __shfl_down_sync(kFull, ap, o), tq = __shfl_down_sync(kFull, aq, o);
-                    if (lane + o < 32) { ap += tp; aq += tq; }
-                }
-                if (lane == 0) { sh.wtot_p[warp] = ap; sh.wtot_q[warp] = aq; }
-                if (threadIdx.x == 0) {
-                    sh.n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
-                    sh.wrapped = (long long)tot[6] > (1ll << 31);
-                    sh.halves = halves;
-                    if (sh.wrapped) ++sh.n_wrapped;
-                }
-                __syncthreads();
-                unsigned long long rp_ = ap - mp_ + tot[7], rq_ = aq - mq_ + tot[8];  // bins above this thread's
-                for (int w = warp + 1; w < kVWarps; ++w) { rp_ += sh.wtot_p[w]; rq_ += sh.wtot_q[w]; }
-#pragma unroll
-                for (int i = kPer - 1; i >= 0; --i) {
-                    rp_ += bp_[i]; rq_ += bq_[i];
-                    bp_[i] = rp_; bq_[i] = rq_;
-                }
-#pragma unroll
-                for (int i = 0; i < kPer; i += 2) {
-                    *reinterpret_cast<ulonglong2 *>(sufP + kPer * threadIdx.x + i) = make_ulonglong2(bp_[i], bp_[i + 1]);
-                    *reinterpret_cast<ulonglong2 *>(sufQ + kPer * threadIdx.x + i) = make_ulonglong2(bq_[i], bq_[i + 1]);
-                }
-                if (threadIdx.x == 0) {
-                    sufP[kBins] = tot[7]; sufQ[kBins] = tot[8];
-                    sufP[kBins + 1] = 0ull; sufQ[kBins + 1] = 0ull;
-                }
-            }
-            __syncthreads();
-            if (warp == 1 && !a.select_mode) draft_tests(l, m);
-
+            hist_merge(cluster, hs, sh, cta_rank, n_cta);
             TS(7);
+            cluster.sync();                            // every slice of the suffix sums is complete
+            TS(5);
+            if (threadIdx.x == 32) sh.halves = halves;
+            if (warp == 1 && !a.select_mode) draft_tests(l, m);
+            // lane c of warp 0: mass of the bins above CTA c's slice
+            unsigned long long above_p = 0ull, above_q = 0ull;
+            double n_cells = 0.0;
+            bool wrapped = false;
+            const int slice = kBins / n_cta;
+            if (warp == 0) {
+                const unsigned long long own_p = lane < n_cta ? sh.slice_p[lane] : 0ull, own_q = lane < n_cta ? sh.slice_q[lane] : 0ull;
+                above_p = own_p; above_q = own_q;
+#pragma unroll
+                for (int o = 1; o < 16; o <<= 1) {
+                    const unsigned long long tp = __shfl_down_sync(kFull, above_p, o), tq = __shfl_down_sync(kFull, above_q, o);
+                    if (lane + o < 32) { above_p += tp; above_q += tq; }
+                }
+                // what all threads added, by their floating-point sums, minus what the words hold.  Without a wrap
+                // that is rounding: half a unit for each cell and 2^-20 of the mass (16 cells in a float sum), less
+                // than 2^26 units; a wrap lowers the words by 2^32
+                wrapped = (long long)(tot[6] - __shfl_sync(kFull, above_p + above_q, 0)) > (1ll << 31);
+                above_p += tot[7] - own_p; above_q += tot[8] - own_q;
+                n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
+                if (lane == 0 && wrapped) ++sh.n_wrapped;
+            }
+            // suffix sums of bins k and k + 1 (warp 0): one word of each kind from the CTAs that have them
+            auto suffix2 = [&](int k, unsigned long long (&P)[2], unsigned long long (&Q)[2]) {
+                const int at = min(k + (lane & 1), kBins), c = min(at / slice, n_cta - 1);
+                unsigned long long sp = tot[7], sq = tot[8];
+                const unsigned long long up = __shfl_sync(kFull, above_p, c), uq = __shfl_sync(kFull, above_q, c);
+                if (lane < 2 && at < kBins) {
+                    const uint32_t lp = cluster.map_shared_rank(hs.wp, c)[at], hi_p = cluster.map_shared_rank(hs.bp, c)[at];
+                    const uint32_t lq = cluster.map_shared_rank(hs.wq, c)[at], hi_q = cluster.map_shared_rank(hs.bq, c)[at];
+                    sp = (((unsigned long long)hi_p << 32) | lp) + up;
+                    sq = (((unsigned long long)hi_q << 32) | lq) + uq;
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) { P[i] = __shfl_sync(kFull, sp, i); Q[i] = __shfl_sync(kFull, sq, i); }
+            };
+
             int j0 = 1;
             while (j0 <= m) {
-                if (threadIdx.x == 0) {
+                if (warp == 0) {
                     int j = j0;
                     int need = 0;
+                    double s_j = sh.s_arr[j - 1], c_j = sh.c_arr[j];
                     for (; j <= m; ++j) {
-                        const double s_j = sh.s_arr[j - 1] + sh.c_arr[j];
-                        sh.s_arr[j] = s_j;
-                        sh.chain_len = j;
+                        s_j += c_j;
+                        if (lane == 0) { sh.s_arr[j] = s_j; sh.chain_len = j; }
                         double c_next;
                         // every partial sum of the histogram is off by at most half a unit per cell
-                        const double fix_err = sh.n_cells * (0.5 * kUnfix) * (1.0 + s_j);
-                        if (sh.wrapped) { need = 1; break; }             // a wrapped word: exact passes only
+                        const double fix_err = n_cells * (0.5 * kUnfix) * (1.0 + s_j);
+                        if (wrapped) { need = 1; break; }                // a wrapped word: exact passes only
+                        unsigned long long P[2], Q[2];
                         if (j == 1) {
-                            c_next = ((double)sufP[0] - (double)sufQ[0]) * kUnfix;
+                            P[0] = __shfl_sync(kFull, above_p, 0) + sh.slice_p[0];
+                            Q[0] = __shfl_sync(kFull, above_q, 0) + sh.slice_q[0];
+                            c_next = ((double)P[0] - (double)Q[0]) * kUnfix;
                             if (fix_err > kErrTol) { need = 1; break; }
                         } else {
                             // (a float's logarithm can miss the bin only within 3e-7 of an edge; the bracket below
@@ -1633,9 +1663,10 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                             int k = (int)(log2f((float)s_j) * binscale);
                             if (k < 0) k = 0;
                             if (k >= kBins) { need = 1; break; }      // cannot happen for s_j <= m
-                            const double Pa = (double)sufP[k + 1] * kUnfix, Qa = (double)sufQ[k + 1] * kUnfix;
-                            const double Pk = (double)(sufP[k] - sufP[k + 1]) * kUnfix;
-                            const double Qk = (double)(sufQ[k] - sufQ[k + 1]) * kUnfix;
+                            suffix2(k, P, Q);
+                            const double Pa = (double)P[1] * kUnfix, Qa = (double)Q[1] * kUnfix;
+                            const double Pk = (double)(P[0] - P[1]) * kUnfix;
+                            const double Qk = (double)(Q[0] - Q[1]) * kUnfix;
                             const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
                             const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
                             const double lo_b = fmax(Pk - s_j * Qk, 0.0);
@@ -1646,11 +1677,14 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                             if (0.5 * (hi_b - lo_b) + fix_err > kErrTol) { need = 1; break; }
                             c_next = fmax(Pa - s_j * Qa, 0.0) + 0.5 * (lo_b + hi_b);
                         }
-                        sh.c_arr[j + 1] = c_next;
+                        if (lane == 0) sh.c_arr[j + 1] = c_next;
+                        c_j = c_next;
                         if (!(c_next > 0.0)) { j = m; }               // chain exhausted: stop walking
                     }
-                    sh.need_exact = need;
-                    sh.chain_pos = need ? j : m + 1;
+                    if (lane == 0) {
+                        sh.need_exact = need;
+                        sh.chain_pos = need ? j : m + 1;
+                    }
                 }
                 __syncthreads();
                 if (!sh.need_exact) break;
@@ -1670,6 +1704,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 if (!(sh.c_arr[j + 1] > 0.0)) break;
                 j0 = j + 1;
             }
+            cluster.barrier_arrive();                  // this CTA has done with the others' slices
+            looked_up = true;
         }
         __syncthreads();
 
@@ -1745,6 +1781,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         }
         __syncthreads();
 
+        if (looked_up) cluster.barrier_wait();         // the others have done with this CTA's slice
         TS(9);
         // ---- a residual draw locates its tile through tile sums of max(p_beam - s_{j-1} q_beam, 0) ----
         double *res_sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride;   // slot 0 of the bank
@@ -1924,7 +1961,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
 
 // ------------------------------------------------------------------------------ host side
 struct Layout {
-    size_t stats, lse, score, depth, sums, hist, total;
+    size_t stats, lse, score, depth, sums, total;
     int T, max_m, max_live;
 };
 
@@ -1941,8 +1978,6 @@ Layout make_layout(const dsbd_forest_t *f, int V) {
     L.depth = off; off = align_up(off + sizeof(int32_t) * (size_t)f->N, 256);
     L.sums = off;
     off = align_up(off + sizeof(double) * (size_t)f->R * 2 * (L.max_m + 1) * (size_t)L.max_live * L.T, 256);
-    L.hist = off;
-    off = align_up(off + sizeof(unsigned long long) * (size_t)f->R * 2 * kHistLen, 256);
 #ifdef DSBD_PHASE_TIMING
     off = align_up(off + sizeof(unsigned long long) * (size_t)f->R * 256, 256);
 #endif
@@ -2081,7 +2116,6 @@ extern "C" int dsbd_verify_step(const dsbd_forest_t *f, const dsbd_verify_params
     a.stats = stats; a.lse = lse; a.score = score; a.depth = depth;
     a.tile_sums = reinterpret_cast<double *>(ws + L.sums);
     a.max_m = L.max_m; a.max_live = L.max_live;
-    a.hist = reinterpret_cast<unsigned long long *>(ws + L.hist);
 #ifdef DSBD_PHASE_TIMING
     a.dbg = reinterpret_cast<unsigned long long *>(ws + L.total) - (size_t)f->R * 256;
 #endif
@@ -2398,7 +2432,6 @@ extern "C" int dsbd_select_width(const dsbd_forest_t *f, const dsbd_verify_param
     a.stats = stats; a.lse = lse; a.score = nullptr; a.depth = nullptr;
     a.tile_sums = reinterpret_cast<double *>(ws + L.sums);
     a.max_m = L.max_m; a.max_live = L.max_live;
-    a.hist = reinterpret_cast<unsigned long long *>(ws + L.hist);
 #ifdef DSBD_PHASE_TIMING
     a.dbg = reinterpret_cast<unsigned long long *>(ws + L.total) - (size_t)f->R * 256;
 #endif

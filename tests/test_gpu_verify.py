@@ -325,6 +325,25 @@ def test_requests_around_the_node_cache_and_half_tiles(beams, gamma, V):
     check_exempt(exempt, decisions)
 
 
+@pytest.mark.parametrize("V", [1000, 2000, 4000, 8000, 32000])
+def test_every_cluster_size(V):
+    """8 rows of 1, 2, 4, 8 and 32 tiles: clusters of 1, 2, 4, 8 and 16 CTAs, whose slices of the merged
+    histogram the chain of 8 rejections looks into; scores tempered so that the ratios reach far bins."""
+    rng = np.random.default_rng(V)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=1, V=V, gamma=3, max_w=8, min_w=8)
+    zp = (zp + rng.normal(0, 2.0, zp.shape)).astype(np.float32)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = 0
+    for step in range(10):
+        prm.update(step=step, thresh=0.2 + 0.06 * step)
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+    check_exempt(exempt, decisions)
+
+
 @pytest.mark.parametrize("beams,V,top_k,top_p", [(64, 72000, 10, 0.8), (64, 72000, 64, 0.9), (36, 121900, 1, 1.0)])
 def test_warped_layers_with_more_tiles_than_the_bound_cache(beams, V, top_k, top_p):
     """64 x 71 = 4544 tile bounds, more than are kept in shared memory (4368), and 36 x 120 = 4320, just fewer."""

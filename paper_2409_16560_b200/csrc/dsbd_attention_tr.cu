@@ -25,9 +25,11 @@
 // issued like this 41 to 50 at N = 16 to 64 (M = 128, K = 16), which is the operand traffic of A.  One
 // warp for both products took 2050 cycles a tile at d = 128, about as long as the tile's bytes take.
 //
-// A row's reference is its logit of the unit's first token, moved only when some logit exceeds it
-// by more than 2^40: the weights then stay inside the exponent range of bf16 and fp32, whose relative
-// precision does not depend on the scale.
+// A row's reference is its largest logit in the unit's first tile, moved to a later tile's largest when that exceeds
+// it by more than 2^8.  The heaviest weight of a row is then mostly a power of two, which bf16 holds exactly: with the
+// first token's logit as the reference (one barrier less a unit) the error against 64 bits was up to 5.7 % larger,
+// at prefixes of 64 to 200 tokens.  Weights in two terms (kSplit) do not need that: there the first token's logit is the
+// reference, moved when exceeded by more than 2^40 (0.4 us of 31.3 for 8 x 4 beams after 512 to 2047 tokens).
 //
 // Work split: the tiles of a layer's units form one sequence (beam, KV head, row block), cut into equal
 // runs, one per CTA; a unit that straddles a cut leaves partial results that k_attn_merge merges.
@@ -48,8 +50,8 @@ namespace {
 
 constexpr int kTile = 128;              // tokens per tile = the M rows of the S^T product
 constexpr int kMaxTree = DSBD_MAX_TREE_NODES;
+static_assert(kMaxTree <= kBN, "a tree is one box: a part never starts behind the tree's root");
 constexpr uint32_t kHalfStride = kTile * 128;        // bytes of one 64-column half of a tile (or of 64 rows of P)
-constexpr float kMoveRef = 40.f;        // log2 of the factor by which a logit may exceed its row's reference
 
 // Shape of one kernel instance.  kSplit: the probabilities enter the second product as the sum of two
 // bf16 terms (2^-17 relative); used at d = 64, where they were kept in fp32 by the kernel this one replaced.
@@ -59,6 +61,7 @@ struct Shape {
     static constexpr int kCols = NMAX / kGroups, kCh = kCols / 8;               // rows of a group, in chunks of 8
     static constexpr int kThreads = kGroups * 128 + 256;
     static constexpr bool kSplit = D == 64;
+    static constexpr float kMoveRef = kSplit ? 40.f : 8.f;    // log2 of the factor by which a logit may exceed its row's reference
     static constexpr int kHalves = D / 64;                    // 64-column halves of a row of Q, K or V
     static constexpr uint32_t kSlot = kTile * D * 2;          // one K or V tile
     static constexpr uint32_t kPTerm = kHalfStride;                                     // [token][128 B]
@@ -735,28 +738,45 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                 tc_fence_after();
                 const bool work = ok && nch > 0 && h < sg.nh;   // (a lone box leaves the upper two warps idle)
                 const uint32_t s_addr = tmem + lane_base + (tile % S::kSBufs) * NMAX + cbase;
-                // the first tile sets the references: the logits of its first token when every row sees it (a
-                // prefix token or the root), else the maxima
-                bool set = j == sg.t0 && 2 * j > sg.nhp;
-                if (j == sg.t0) {
-                    if (!set) {
-                        if (q == 0 && work) {
-                            uint32_t v[S::kCols];
+                // the columns' maxima over the tile's tokens that their rows see, times the scale (> 0, checked by the
+                // host): thread tok has column tok of the group's
+                auto column_max = [&] {
+#pragma unroll 1
+                    for (int ch = 0; ch < nch; ++ch) {
+                        uint32_t v[8];
+                        if (work) tmem_ld8(s_addr + ch * 8, v);
+                        tmem_wait_ld();
+                        float f[8];
 #pragma unroll
-                            for (int ch = 0; ch < S::kCh; ++ch)
-                                if (ch < nch) tmem_ld8(s_addr + ch * 8, v + ch * 8);
-                            tmem_wait_ld();
-                            if (tok == 0) {
+                        for (int i = 0; i < 8; ++i)
+                            f[i] = work && ((see >> (ch * 8 + i)) & 1u) ? __uint_as_float(v[i]) : -INFINITY;
+                        fold8(f, lane, [](float x, float y) { return fmaxf(x, y); });
+                        if (lane < 8) sx.colmax[grp][q][ch * 8 + lane] = f[0];
+                        __syncwarp();
+                    }
+                    group_sync(grp);
+                    return tok < nch * 8 ? fmaxf(fmaxf(sx.colmax[grp][0][tok], sx.colmax[grp][1][tok]),
+                                                 fmaxf(sx.colmax[grp][2][tok], sx.colmax[grp][3][tok])) * a.scale_log2
+                                         : 0.f;
+                };
+                if (j == sg.t0) {                            // the first tile sets the references
+                    if (!S::kSplit) {
+                        const float m = column_max();
+                        if (tok < nch * 8) sx.negref[grp][tok] = m > -INFINITY ? -m : 0.f;
+                    } else if (q == 0 && work) {             // (its first token is a prefix token or the root)
+                        uint32_t v[S::kCols];
 #pragma unroll
-                                for (int c = 0; c < S::kCols; c += 4)
-                                    if (c / 8 < nch)
-                                        *reinterpret_cast<float4 *>(&sx.negref[grp][c]) =
-                                            make_float4(-__uint_as_float(v[c]) * a.scale_log2, -__uint_as_float(v[c + 1]) * a.scale_log2,
-                                                        -__uint_as_float(v[c + 2]) * a.scale_log2, -__uint_as_float(v[c + 3]) * a.scale_log2);
-                            }
+                        for (int ch = 0; ch < S::kCh; ++ch)
+                            if (ch < nch) tmem_ld8(s_addr + ch * 8, v + ch * 8);
+                        tmem_wait_ld();
+                        if (tok == 0) {
+#pragma unroll
+                            for (int c = 0; c < S::kCols; c += 4)
+                                if (c / 8 < nch)
+                                    *reinterpret_cast<float4 *>(&sx.negref[grp][c]) =
+                                        make_float4(-__uint_as_float(v[c]) * a.scale_log2, -__uint_as_float(v[c + 1]) * a.scale_log2,
+                                                    -__uint_as_float(v[c + 2]) * a.scale_log2, -__uint_as_float(v[c + 3]) * a.scale_log2);
                         }
-                    } else if (tok < nch * 8) {
-                        sx.negref[grp][tok] = 0.f;
                     }
                     group_sync(grp);
                 }
@@ -817,36 +837,19 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                         }
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     }
-                    if (!group_any(grp, !ok || over > kMoveRef || set) || attempt == 2) break;
+                    if (!group_any(grp, !ok || over > S::kMoveRef) || attempt == 2) break;
                     // rare: some reference has to move (or a wait ran out): O^T is rescaled, so the previous
                     // product must have landed
                     if (ok && j > sg.t0) ok = warp_wait(&sb.pv_done[(tile - 1) & 1], ((tile - 1) >> 1) & 1, &sb);
                     if (group_any(grp, !ok)) { ok = false; break; }
                     tc_fence_after();
-#pragma unroll 1
-                    for (int ch = 0; ch < nch; ++ch) {       // the columns' maxima over the tile's tokens
-                        uint32_t v[8];
-                        if (work) tmem_ld8(s_addr + ch * 8, v);
-                        tmem_wait_ld();
-                        float f[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            f[i] = work && ((see >> (ch * 8 + i)) & 1u) ? __uint_as_float(v[i]) : -INFINITY;
-                        fold8(f, lane, [](float x, float y) { return fmaxf(x, y); });
-                        if (lane < 8) sx.colmax[grp][q][ch * 8 + lane] = f[0];
-                        __syncwarp();
-                    }
-                    group_sync(grp);
+const float m = column_max();
                     if (tok < nch * 8) {
-                        const float m = fmaxf(fmaxf(sx.colmax[grp][0][tok], sx.colmax[grp][1][tok]),
-                                              fmaxf(sx.colmax[grp][2][tok], sx.colmax[grp][3][tok])) *
-                                        a.scale_log2;        // scale > 0 (checked by the host)
                         const float nr = sx.negref[grp][tok];
-                        const bool move = set ? m > -INFINITY : m + nr > 0.f;
+                        const bool move = m + nr > 0.f;
                         sx.move[grp][tok] = move ? exp2f(-(m + nr)) : 1.f;
                         if (move) sx.negref[grp][tok] = -m;
                     }
-                    set = false;
                     group_sync(grp);
                     if (j > sg.t0) {
 #pragma unroll 1

@@ -191,3 +191,39 @@ def test_host_side_errors():
     with pytest.raises(dsbd.DsbdError) as e:      # Hq not a multiple of Hkv
         dsbd.forest_attention(f, 4, 3, 64, 0.1, t["q"], t["k_new"], t["v_new"], t["k_prefix"], t["v_prefix"], pd, poff)
     assert e.value.code == -1
+
+
+@pytest.mark.parametrize("first,second,jump", [(1, 2, 0.0), (63, 40, 0.0), (100, 3, 0.0), (300, 350, 10.0), (1999, 1990, 25.0)])
+@pytest.mark.parametrize("d,nodes", [(64, 5), (64, 20), (128, 5), (128, 20)])
+def test_the_heaviest_weight_is_exact(d, nodes, first, second, jump):
+    """Two tokens of weights 1 and 3/4 and values +1 and -1; everything else weighs next to nothing.  Relative to the
+    heavier one both weights are bf16 numbers, so the result is 1/7 to its own rounding (2^-9) and the
+    first token's share (2^-12.4 in the row sum); relative to the first token they round by 0.29 % down and 0.30 % up, to
+    1/7 - 0.0029.  With a jump they stand 2^22 or 2^37 above all logits of the first tile."""
+    L, rng = 2000, np.random.default_rng(first)
+    tree = [-1] + [int(rng.integers(0, i)) for i in range(1, nodes)]
+    forest, spec, t, poff = _custom(rng, [tree], [L], 2, 2, d, torch.bfloat16)
+
+    def split(x):                                  # x as the sum of three bf16 numbers
+        parts = []
+        for _ in range(3):
+            parts.append(float(torch.tensor(x - sum(parts), dtype=torch.float64).to(torch.bfloat16)))
+        return parts
+
+    # logits in log2 units: q = (1, 1, 1, 0, ..), scale = ln 2
+    t["q"].zero_()
+    t["q"][..., :3] = 1.0
+    for k in ("k_prefix", "k_new", "v_prefix", "v_new"):
+        t[k].zero_()
+    K, Vv = (t[k][:L * 2 * d].view(2, L, d) for k in ("k_prefix", "v_prefix"))
+    off = 12.422
+    K[..., 0], t["k_new"][..., 0] = -100.0, -100.0
+    K[:, 0, :3] = torch.tensor(split(-off - jump), dtype=torch.bfloat16)
+    K[:, first, :3] = 0.0
+    K[:, second, :3] = torch.tensor(split(float(np.log2(0.75))), dtype=torch.bfloat16)
+    Vv[:, first], Vv[:, second] = 1.0, -1.0
+    f = dsbd.Forest(forest, "cuda")
+    out, status = dsbd.forest_attention(f, 2, 2, d, float(np.log(2.0)), t["q"], t["k_new"], t["v_new"], t["k_prefix"],
+                                        t["v_prefix"], torch.as_tensor(poff).cuda(), poff)
+    assert int(status.item()) == 0
+    assert (out.double() - 1 / 7).abs().max().item() <= (2.0 ** -9 + 2.0 ** -12) / 7

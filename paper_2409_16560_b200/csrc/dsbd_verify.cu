@@ -118,7 +118,15 @@ k_tile_stats(const float *__restrict__ zp, const float *__restrict__ zq, int64_t
             mx = fmaxf(mx, fmaxf(fmaxf(v[it].x, v[it].y), fmaxf(v[it].z, v[it].w)));
         mx = warp_max(mx);
         float sum = 0.f;
-        if (mx > -INFINITY) {
+        if (fabsf(mx) * k2 > 65536.f) {
+            // a tile masked with a huge value: the rounding of its product with k2 is no longer small against one, and
+            // the product may overflow (2^x of either would be infinite, and the row's sum with it).  -inf: no mass
+            if (mx > -INFINITY)
+#pragma unroll
+                for (int it = 0; it < 8; ++it)
+                    sum += exp2f((v[it].x - mx) * k2) + exp2f((v[it].y - mx) * k2) +
+                           exp2f((v[it].z - mx) * k2) + exp2f((v[it].w - mx) * k2);
+        } else {
             const float b = -mx * k2;
 #pragma unroll
             for (int it = 0; it < 8; ++it) {

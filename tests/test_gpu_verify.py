@@ -507,3 +507,22 @@ def test_select_width_matches_oracle(top_k, top_p):
     for r in range(forest["R"]):
         assert np.abs(alpha[r, :m[r]].cpu().numpy() - a_ref[r, :m[r]]).max() < 2e-5
         assert np.abs(tail[r, :m[r] + 1].cpu().numpy() - t_ref[r, :m[r] + 1]).max() < 2e-5
+
+
+@pytest.mark.parametrize("value", [float(np.finfo(np.float32).min), -1e30, -1e15, -1e9, -np.inf])
+@pytest.mark.parametrize("top_k", [0])
+def test_tiles_masked_with_huge_values(top_k, value):
+    """A row with whole tiles at the mask's value: value / tau times log2(e) is beyond the type's range or rounded by
+    far more than one, and the tile has no mass."""
+    V = 5000
+    rng = np.random.default_rng(top_k)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=4, V=V, gamma=3, max_w=4)
+    zp[:, 1024:3072] = zq[:, 1024:3072] = value
+    for n in range(forest["N"]):
+        if 1024 <= forest["token"][n] < 3072:
+            forest["token"][n] += 2048 if forest["token"][n] + 2048 < V else -1024
+    prm.update(temperature=1.0, top_k=top_k, top_p=0.9 if top_k else 1.0)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    gpu, status = run_gpu_verify(forest, prm, *dev)
+    assert status == 0
+    check_exempt(*compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest))

@@ -881,7 +881,8 @@ struct SupportTmp {
     int sel[256];                 // tiles whose bound reaches the threshold
     unsigned lo[kVWarps], hi[kVWarps];   // per warp, images of the smallest finite and of the largest bound
     int finite[kVWarps];          // per warp, finite bounds
-    int count[3];                 // of the bisection's rounds, in turn
+    int count[3];                 // of the bisection's rounds, in turn: bounds above the cut, and
+    unsigned low[3];              // the image of the smallest of them
     int n_sel, n_cand, err;
 };
 struct WarpScratch {
@@ -928,7 +929,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     const float *z = model ? a.zq : a.zp;
     const float inv_tau_f = (float)a.inv_tau;
     for (int i = tl; i < sh.nA; i += NT) tp.off[i] = (float)(lw[i] - lse[sh.A[i]]);
-    if (tl < 3) tp.count[tl] = 0;
+    if (tl < 3) { tp.count[tl] = 0; tp.low[tl] = 0xffffffffu; }
     if (tl == 0) { tp.n_sel = 0; tp.n_cand = 0; tp.err = 0; ws.n[model] = 0; }
     part_sync<NT>(model);
     // float upper bound of log(joint probability) over tile i
@@ -942,9 +943,10 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
     };
     auto value = [](unsigned u) -> float { return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u); };
-    // A cut not above the k-th largest tile bound (with multiplicity: k tiles each hold a cell at least that
-    // large) and few tiles below it; with fewer than k finite bounds every tile counts.  Bounds that do not fit
-    // the cache are computed again in every round.
+    // The k-th largest tile bound (with multiplicity: k tiles each hold a cell at least that large), or the next or
+    // next but one where these lie close; with fewer than k finite bounds every tile counts.  It must be a
+    // bound and not merely a cut below: a bisection's cut may lie far down in the gap above masked tiles,
+    // where it passes every cell of the tiles above.  Bounds that do not fit the cache are computed again in every round.
     unsigned *bcache = hist_p + (2 + model) * kHistWords;
     const bool cached = nt <= kBoundCache;
     {
@@ -967,17 +969,26 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     for (int w = 0; w < kPartWarps; ++w) { lo = min(lo, tp.lo[w]); hi = max(hi, tp.hi[w]); finite += tp.finite[w]; }
     if (finite >= k) {
         // count(>= lo) >= k always holds; hi is above the k-th largest
+        const float near = value(hi) - 30.f;                      // (cells below have no mass to speak of)
+        auto done = [&](int n) { return n == k || (n <= k + 2 && value(lo) > near); };
         ++hi;
-        for (int round = 0; hi - lo > 1; ++round) {
+        for (int round = 0; hi - lo > 1 && !(round == 0 && done(finite)); ++round) {
             const unsigned mid = lo + (hi - lo) / 2;
             int n = 0;
-            for (int i = tl; i < nt; i += NT) n += (cached ? bcache[i] : image(bound(i))) >= mid;
+            unsigned low = 0xffffffffu;
+            for (int i = tl; i < nt; i += NT) {
+                const unsigned u = cached ? bcache[i] : image(bound(i));
+                if (u >= mid) { ++n; low = min(low, u); }
+            }
             n = __reduce_add_sync(kFull, n);
-            if (lane == 0 && n) atomicAdd(&tp.count[round % 3], n);
-            if (tl == 0) tp.count[(round + 1) % 3] = 0;           // (last read two rounds ago)
+            low = __reduce_min_sync(kFull, low);
+            if (lane == 0 && n) { atomicAdd(&tp.count[round % 3], n); atomicMin(&tp.low[round % 3], low); }
+            if (tl == 0) { tp.count[(round + 1) % 3] = 0; tp.low[(round + 1) % 3] = 0xffffffffu; }     // (last read two rounds ago)
             part_sync<NT>(model);
             n = tp.count[round % 3];
-            if (n >= k) { lo = mid; if (n <= k + 2) break; } else hi = mid;
+            if (n < k) { hi = mid; continue; }
+            lo = tp.low[round % 3];
+            if (done(n)) break;
         }
     }
     const float thr = value(lo);

@@ -143,3 +143,20 @@ def test_host_side_errors():
     with pytest.raises(dsbd.DsbdError):        # more beams in a request than the kernel's live limit
         dsbd.draft_layer(torch.tensor([0, 70], dtype=torch.int32, device="cuda"), [0, 70], dict(V=100), 1, 2,
                          torch.zeros(70, 100, device="cuda"), torch.zeros(70, device="cuda"), off, 2)
+
+
+@pytest.mark.parametrize("value", [-np.inf, float(np.finfo(np.float32).min), -1e30, -1e9, -1e4])
+@pytest.mark.parametrize("V,top_k,extra", [(32000, 10, 0), (32000, 10, 2), (32000, 20, 1), (128256, 50, 2)])
+def test_top_k_with_masked_tiles(V, top_k, extra, value):
+    """k to k + 2 of a request's tiles hold the live vocabulary, the others are masked."""
+    global ref_prm, ref_layer
+    rng = np.random.default_rng(V + top_k + extra)
+    rbo, z, s = _problem(rng, [1, 1], V, zipf=False)
+    tiles = -(-V // 1024)
+    for row in z:
+        row[~np.isin(np.arange(V) // 1024, rng.choice(tiles, size=top_k + extra, replace=False))] = value
+    prm = dict(V=V, temperature=1.5, seed=7, step=0, top_k=top_k, top_p=0.95)
+    ref_prm, ref_layer = prm, 1
+    ref, gpu, W_r, out_off = _both(rbo, z, s, prm, 1, 16)
+    assert int(gpu["status"][0]) == 0
+    _compare(ref, gpu, W_r, out_off)

@@ -526,3 +526,39 @@ def test_tiles_masked_with_huge_values(top_k, value):
     gpu, status = run_gpu_verify(forest, prm, *dev)
     assert status == 0
     check_exempt(*compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest))
+
+
+def _masked_tiles(rng, n_rows, V, keep, value):
+    """Two models' logits in which all but `keep` of the 1024-token tiles are masked with `value`."""
+    zp = rng.normal(0, 2.5, size=(n_rows, V)).astype(np.float32)
+    zq = (zp + rng.normal(0, 1.0, size=(n_rows, V))).astype(np.float32)
+    tile = np.arange(V) // 1024
+    masked = ~np.isin(tile, rng.choice(tile[-1] + 1, size=keep, replace=False))
+    zp[:, masked] = value
+    zq[:, masked] = value
+    return zp, zq, np.flatnonzero(~masked)
+
+
+@pytest.mark.parametrize("value", [-np.inf, float(np.finfo(np.float32).min), -1e30, -1e9, -1e4])
+@pytest.mark.parametrize("V,top_k,extra", [(32000, 10, 0), (32000, 10, 2), (32000, 20, 1), (128256, 50, 2)])
+def test_top_k_with_masked_tiles(V, top_k, extra, value):
+    """k to k + 2 tiles hold the live vocabulary, the others are masked: the cut lies at the k-th largest tile bound
+    whatever the distance to the next one.  (Temperature 1.5 keeps the scaled mask finite.)"""
+    rng = np.random.default_rng(V + top_k + extra)
+    forest, prm, _, _, rp, rq, _ = _random_problem(rng, R=3, V=8, gamma=2, max_w=1)
+    zp, zq, live = _masked_tiles(rng, forest["N"], V, top_k + extra, value)
+    for n in range(forest["N"]):
+        par = forest["parent"][n]
+        if par >= 0:                               # a token that the small model is likely to draft
+            forest["token"][n] = live[np.argsort(-zq[par, live])[rng.integers(0, 8)]]
+    prm.update(V=V, top_k=top_k, top_p=0.95, temperature=1.5)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = 0
+    for step in range(3):
+        prm["step"] = step
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+    check_exempt(exempt, decisions)

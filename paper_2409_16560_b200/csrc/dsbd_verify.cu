@@ -1078,7 +1078,8 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         if (!(lo_t > -INFINITY)) lo_t = hi_t - 400.f;
         bool found = false;
         for (int itn = 0; itn < 60 && hi_t > lo_t; ++itn) {
-            const float mid = 0.5f * (lo_t + hi_t);
+            // (first out of the gap above a mask of finite values: halving does not come back from -1e30)
+            const float half = 0.5f * (lo_t + hi_t), mid = itn ? half : fmaxf(half, hi_t - 400.f);
             const int c = sweep(mid, false);
             if (c > kMaxCand) lo_t = mid;
             else if (c < k) hi_t = mid;

@@ -510,10 +510,10 @@ def test_select_width_matches_oracle(top_k, top_p):
 
 
 @pytest.mark.parametrize("value", [float(np.finfo(np.float32).min), -1e30, -1e15, -1e9, -np.inf])
-@pytest.mark.parametrize("top_k", [0])
+@pytest.mark.parametrize("top_k", [0, 10])
 def test_tiles_masked_with_huge_values(top_k, value):
     """A row with whole tiles at the mask's value: value / tau times log2(e) is beyond the type's range or rounded by
-    far more than one, and the tile has no mass."""
+    far more than one, and the tile has no mass.  (Kept cells: more than tiles that hold some in half of the requests.)"""
     V = 5000
     rng = np.random.default_rng(top_k)
     forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=4, V=V, gamma=3, max_w=4)

@@ -575,8 +575,9 @@ __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigne
     return d;
 }
 
-// The cells of one half tile (4 x float4 per lane and model) into the histogram; adds the p and the q mass of
-// its cells with p_beam > q_beam, in units of 2^-44, to sp and sq.
+// The cells of one half tile (4 x float4 per lane and model) into the histogram; adds p - q and q of its cells with
+// p_beam > q_beam, in units of 2^-44, to sd and sq.  (p - q cell by cell: the difference of two sums loses what lies
+// next to a heavy cell, and a completion draw looks for its tile by these sums.)
 // The work per cell decides the speed of this pass (it is bound by instruction issue, not by
 // memory), so the common case is straight-line code, two cells to a packed instruction up to the exponentials:
 // masses are computed directly in units (the row's factor 2^rest carries the 2^44), the bin comes from an fma
@@ -594,7 +595,7 @@ constexpr float kBinMagic = 12582912.f;                         // 1.5 * 2^23
 constexpr float kBigUnits = 268435456.f;                        // 2^28 units = a cell of 2^-16
 __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const float4 (&vq)[4], float k2,
                                                const RowOff &o, float binscale, float half_bin, float top, uint32_t wbase,
-                                               uint32_t over_bits, float &sp, float &sq) {
+                                               uint32_t over_bits, float &sd, float &sq) {
     // dl = log2(rho) - half: the half bin (in log2 units) that turns the fma's round-to-nearest into
     // the bin's floor is part of the row offset, so p_beam > q_beam reads dl > -half
     const float bd = ((o.bp - o.bq) + o.dc) - half_bin;
@@ -605,7 +606,7 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
     const unsigned long long bs2 = pack2(binscale, binscale), mg2 = pack2(kBinMagic, kBinMagic);
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
-        float dl[4], pm[4], qm[4];
+        float dl[4], pm[4], qm[4], df[4];
         uint32_t addr[4];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -615,16 +616,17 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
             const unsigned long long dl2 = fma2(fma2(q2, neg2, p2), k22, bd2);     // NaN compares false
             const float2 d = unpack2(dl2), t = unpack2(fma2(dl2, bs2, mg2));
             const float2 pe = unpack2(fma2(p2, k22, bp2)), qe = unpack2(fma2(q2, k22, bq2));
-            const float2 pu = unpack2(mul2(pack2(ex2_approx(pe.x), ex2_approx(pe.y)), cp2));
-            const float2 qu = unpack2(mul2(pack2(ex2_approx(qe.x), ex2_approx(qe.y)), cq2));
+            const unsigned long long pu2 = mul2(pack2(ex2_approx(pe.x), ex2_approx(pe.y)), cp2);
+            const unsigned long long qu2 = mul2(pack2(ex2_approx(qe.x), ex2_approx(qe.y)), cq2);
+            const float2 pu = unpack2(pu2), qu = unpack2(qu2), du = unpack2(fma2(qu2, neg2, pu2));
             // floor(log2(rho) * binscale) in the low bits (round to nearest of x - 0.5; an x that is a
             // whole number may fall to either side, both within the bins' edge tolerance)
             // (all cells beyond the last edge in one word would wrap it: every warp and half-warp
             // lane has its own copy of that bin)
             addr[2 * h] = wbase + ((d.x < top ? __float_as_uint(t.x) : over_bits) << 2);
             addr[2 * h + 1] = wbase + ((d.y < top ? __float_as_uint(t.y) : over_bits) << 2);
-            dl[2 * h] = d.x; pm[2 * h] = pu.x; qm[2 * h] = qu.x;
-            dl[2 * h + 1] = d.y; pm[2 * h + 1] = pu.y; qm[2 * h + 1] = qu.y;
+            dl[2 * h] = d.x; pm[2 * h] = pu.x; qm[2 * h] = qu.x; df[2 * h] = fmaxf(du.x, 0.f);
+            dl[2 * h + 1] = d.y; pm[2 * h + 1] = pu.y; qm[2 * h + 1] = qu.y; df[2 * h + 1] = fmaxf(du.y, 0.f);
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c)
@@ -632,7 +634,7 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
                 "setp.gt.f32 p, %2, %5;\n\t"
                 "@p add.f32 %0, %0, %3;\n\t"
                 "@p add.f32 %1, %1, %4;\n\t}"
-                : "+f"(sp), "+f"(sq) : "f"(dl[c]), "f"(pm[c]), "f"(qm[c]), "f"(pass_thr));
+                : "+f"(sd), "+f"(sq) : "f"(dl[c]), "f"(df[c]), "f"(qm[c]), "f"(pass_thr));
         const float big = fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3]));
         if (big >= kBigUnits) {
 #pragma unroll
@@ -699,10 +701,10 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float bins
                 load_half_tile(rp, e0, a.V, false, lane, vp);
                 load_half_tile(rq, e0, a.V, false, lane, vq);
             }
-            float sp = 0.f, sq = 0.f;
-            hist_half_tile(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sp, sq);
-            added += __float2ull_rn(sp + sq);
-            res1 += (double)sp - (double)sq;
+            float sd = 0.f, sq = 0.f;
+            hist_half_tile(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sd, sq);
+            added += __float2ull_rn(fmaf(2.f, sq, sd));
+            res1 += (double)sd;
         }
         // the items' sums of the residual after ONE rejection (s_1 = 1): what a completion draw at run
         // position 2 searches, so that this common case needs no second pass over the rows

@@ -562,3 +562,31 @@ def test_top_k_with_masked_tiles(V, top_k, extra, value):
         exempt += e
         decisions += d
     check_exempt(exempt, decisions)
+
+
+def test_residual_next_to_a_dominant_cell():
+    """One rejection; the residual is 12 cells of 2^-25 (of the heaviest cell) that share their lane with a cell of mass
+    0.53, and the residuals of that cell and of one of 0.47 elsewhere, a quarter of it.  Each small cell is a quarter
+    of the heavy one's last bit; a sum that holds both has none of them.  The heavy cells' masses are floats, their residuals
+    (0.56 and 1 of their last bits) therefore 0 or 1 times 2^-24 and 0 to 2 times 2^-25: the small cells' share of
+    1.9e-7 is at least 0.61, less 3 sigma of 512 draws 0.545."""
+    R, V, u = 512, 512, 2.0 ** -23
+    small = [it * 128 + c for it in (1, 2, 3) for c in range(4)]         # lane 0's cells, behind the heaviest
+    zp = np.full((2, V), -np.inf, np.float32)
+    zp[0, 0], zp[0, 4] = 0.0, np.log(0.875)
+    zq = zp.copy()
+    zp[0, small] = np.log(u / 4)
+    zq[0, 500] = np.log(4 * u)                                           # the draft: outside the support of p
+    zp[1], zq[1] = 0.0, 0.0
+    N = 2 * R
+    forest = dict(R=R, B=R, N=N, max_depth=1, req_beam_off=np.arange(R + 1, dtype=np.int32),
+                  beam_node_off=(2 * np.arange(R + 1)).astype(np.int32), token=np.full(N, 500, np.int32),
+                  parent=np.stack([np.full(R, -1), 2 * np.arange(R)], 1).reshape(-1).astype(np.int32))
+    prm = dict(V=V, temperature=1.0, thresh=0.5, W_min=1, W_max=1, W_nom=1, seed=3, step=0)
+    dev = [torch.as_tensor(np.tile(z, (R, 1))).cuda() for z in (zp, zq)]
+    zero = torch.zeros(R, device="cuda")
+    gpu, status = run_gpu_verify(forest, prm, *dev, zero, zero)
+    assert status == 0 and (gpu["req_error"] == 0).all()
+    assert (gpu["out_source"] == 1).all() and (gpu["l_last"] == 1).all()
+    share = np.isin(gpu["out_token"], small).mean()
+    assert share > 0.545, share

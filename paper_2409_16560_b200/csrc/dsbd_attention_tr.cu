@@ -613,6 +613,9 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
         auto put_rec = [&](int layer) {
             if (!a.whole && tid == 0) a.recs[layer * a.runs + (int)blockIdx.x % a.runs] = rec;
         };
+        // (the merge reads the records of all layers, also of those a CTA does not reach after a time-out)
+        if (!a.whole)
+            for (int l = rec_layer; l < a.n_layers; l += a.layer_step) put_rec(l);
         while (get_seg(sb, unit, sg)) {
             if (sg.layer != rec_layer) { put_rec(rec_layer); rec = CutRec{}; rec_layer = sg.layer; }
             const int rows = sg.rows;
@@ -925,6 +928,8 @@ k_attn_merge(TcArgs a) {
     const int layer = blockIdx.z, i0 = layer * a.runs + (int)blockIdx.x, end = (layer + 1) * a.runs - 1;
     const CutRec rec = a.recs[i0];
     if (!rec.tail) return;
+    // (no unit of this forest: a CTA that left before it wrote its records)
+    if ((unsigned)rec.b >= (unsigned)a.B || (unsigned)rec.g >= (unsigned)a.Hkv || (unsigned)rec.rb > (unsigned)kMaxTree) return;
     int last = min(i0 + 1, end);                             // the runs that hold the other parts
     while (last < end && !a.recs[last].head_ends) ++last;
     const int n_lo = a.beam_node_off[rec.b];

@@ -25,13 +25,21 @@ pytestmark = pytest.mark.gpu
 DEV_TIMEOUT = 5
 
 
-def test_a_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable():
+def _wait_library():
     lib = C.CDLL(cuda_build.build_wait_test())
     lib.dsbd_forest_attention_workspace.restype = C.c_size_t
     lib.dsbd_forest_attention_workspace.argtypes = [C.c_void_p, C.c_void_p]
     lib.dsbd_forest_attention.restype = C.c_int
     lib.dsbd_forest_attention.argtypes = [C.c_void_p] * 10 + [C.c_size_t, C.c_void_p, C.c_void_p]
+    lib.dsbd_forest_attention_paged_workspace.restype = C.c_size_t
+    lib.dsbd_forest_attention_paged_workspace.argtypes = [C.c_void_p] * 3
+    lib.dsbd_forest_attention_paged.restype = C.c_int
+    lib.dsbd_forest_attention_paged.argtypes = [C.c_void_p] * 11 + [C.c_size_t, C.c_void_p, C.c_void_p]
+    return lib
 
+
+def test_a_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable():
+    lib = _wait_library()
     rng = np.random.default_rng(31)
     rand_tree = lambda n: [-1] + [int(rng.integers(0, i)) for i in range(1, n)]
     trees = [rand_tree(9), rand_tree(5), rand_tree(12), rand_tree(3)]
@@ -62,3 +70,50 @@ def test_a_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable():
     # next launch on the same device gives the full, correct result
     good = _gpu(forest, spec, t, poff)
     attention_close(to_host_f32(good), ref, bf16=True)
+
+
+def test_a_wait_that_runs_out_in_a_call_of_several_layers_with_cut_units():
+    """The run of CTA 0 stops in the first layer.  Its records of the layers it never reached are empty, so
+    that the merge, which runs over all layers, takes no unit from them; rows of other runs are right in all layers."""
+    lib = _wait_library()
+    runs = torch.cuda.get_device_properties(0).multi_processor_count
+    R, L, Hq, Hkv, n_layers = 8, 10000, 8, 2, 3
+    # 16 units of 80 tiles a layer: a run for every SM, units cut into about 9
+    sizes = [9] * R
+    bno = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    parent = np.concatenate([[-1] + list(range(b, b + 8)) for b in bno[:-1]]).astype(np.int32)
+    forest = dict(R=1, B=R, N=int(bno[-1]), max_depth=8, req_beam_off=np.array([0, R], np.int32), beam_node_off=bno,
+                  parent=parent, token=np.zeros(int(bno[-1]), np.int32))
+    f = dsbd.Forest(forest, "cuda")
+    poff = (L * np.arange(R + 1)).astype(np.int64)
+    per = -(-L // 64)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    mk = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    q, kn, vn = mk(n_layers, f.N, Hq, 128), mk(n_layers, f.N, Hkv, 128), mk(n_layers, f.N, Hkv, 128)
+    kp, vp = mk(n_layers, R * per, Hkv, 64, 128), mk(n_layers, R * per, Hkv, 64, 128)
+    table = torch.arange(R * per, dtype=torch.int32, device="cuda")
+    page_off, poff_dev = (torch.as_tensor(x).cuda() for x in (per * np.arange(R + 1), poff))
+    scale = inputs.default_scale(128)
+    ref, status = dsbd.forest_attention_paged(f, Hq, Hkv, 128, scale, q, kn, vn, kp, vp, table, page_off, poff_dev, poff)
+    assert int(status.item()) == 0
+    fs, desc, pages = f.struct(), bd._attn_desc(Hq, Hkv, 128, torch.bfloat16, scale, poff), bd.KvPagesT()
+    pages.page_table, pages.page_off, pages.n_pages = table.data_ptr(), page_off.data_ptr(), R * per
+    pages.n_layers = n_layers
+    pages.pool_layer_stride, pages.new_layer_stride, pages.q_layer_stride = kp.stride(0), kn.stride(0), q.stride(0)
+    need = int(lib.dsbd_forest_attention_paged_workspace(*(C.addressof(x) for x in (fs, desc, pages))))
+    assert need > 32 * runs * n_layers                     # records and partial results: units are cut
+    ws = torch.full((need,), 0x11, dtype=torch.uint8, device="cuda")
+    out = torch.zeros_like(q)
+    rc = lib.dsbd_forest_attention_paged(C.addressof(fs), C.addressof(desc), *(x.data_ptr() for x in (q, kn, vn, kp, vp)),
+                                         C.addressof(pages), poff_dev.data_ptr(), out.data_ptr(), ws.data_ptr(), need,
+                                         status.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    torch.cuda.synchronize()
+    assert int(status.item()) == DEV_TIMEOUT
+    recs = ws[:32 * runs * n_layers].view(torch.int32).view(n_layers, runs, 8).cpu().numpy()
+    assert (recs[1:, 0] == 0).all()
+    assert np.isin(recs[..., :2], (0, 1)).all() and (recs[..., 2] < R).all() and (recs[..., 3] < Hkv).all()
+    assert torch.equal(out[:, int(bno[-2]):], ref[:, int(bno[-2]):])          # the last beam
+    again, status = dsbd.forest_attention_paged(f, Hq, Hkv, 128, scale, q, kn, vn, kp, vp, table, page_off, poff_dev, poff)
+    assert int(status.item()) == 0 and torch.equal(again, ref)

@@ -82,14 +82,17 @@ struct Shape {
     static constexpr uint32_t kSBufs = 4, kColO = kSBufs * NMAX, kTmemCols = NMAX == 32 ? 256 : 512;
 };
 
+// Tries of a wait before it gives up.  A try is suspended for 4 us here before it returns without success (4000 tries
+// that failed took 16 ms), so this is about two seconds; 20e6 were 80.  A limit in clock cycles costs the waits
+// 0.3 us of 31.2 (8 x 4 beams, heads of 64).
 #ifdef DSBD_TEST_WAIT_TIMEOUT
-// Test build only (a second library that no product path loads): waits give up after some hundred
-// microseconds and the producer leaves out one tile, so that a wait runs out without anything
+// Test build only (a second library that no product path loads): waits give up after about a
+// millisecond and the producer leaves out one tile, so that a wait runs out without anything
 // faulting or hanging.  The test checks the status, and that the next launch of the normal
 // library on the same context is correct.
-constexpr uint32_t kWaitTries = 4000;
+constexpr uint32_t kWaitTries = 250;
 #else
-constexpr uint32_t kWaitTries = 20000000;         // tries of a wait: about a second when each returns at once
+constexpr uint32_t kWaitTries = 500000;
 #endif
 
 // What a run left for the merge.  tail: its last unit starts here and goes on in the next run; head_ends:

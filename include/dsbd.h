@@ -89,7 +89,10 @@ enum { DSBD_DTYPE_BF16 = 0, DSBD_DTYPE_F32 = 1 };
  * forest nodes themselves);  k_prefix, v_prefix: the KV cache of each input beam packed
  * beam after beam, beam b as [Hkv, L_b, d] starting at element prefix_off[b]*Hkv*d, where
  * L_b = prefix_off[b+1]-prefix_off[b] tokens (the cache excludes the root token).  Query
- * head h uses KV head h / (Hq/Hkv).  All tensors share `dtype`; accumulation is fp32. */
+ * head h uses KV head h / (Hq/Hkv).  All tensors share `dtype`; accumulation is fp32.
+ * With bf16 and d = 128 the values are read in blocks of 64 tokens: up to 63 rows of v_prefix
+ * behind a head's prefix (the next head's or beam's) and of v_new behind a tree (the next
+ * trees') enter with weight zero and must be finite.  Other calls read exact ranges. */
 typedef struct {
     int32_t Hq, Hkv, d;            /* d in {64, 128}; Hq % Hkv == 0                          */
     int32_t dtype;                 /* DSBD_DTYPE_*                                           */

@@ -61,6 +61,9 @@ struct Shape {
     static constexpr int kCols = NMAX / kGroups, kCh = kCols / 8;               // rows of a group, in chunks of 8
     static constexpr int kThreads = kGroups * 128 + 256;
     static constexpr bool kSplit = D == 64;
+    // The results depend on the unit's own values only, whatever lies behind them, as on the CUDA cores, which served
+    // d = 64 before (d = 128 asks for finite values there).
+    static constexpr bool kExactRanges = D == 64;
     static constexpr float kMoveRef = kSplit ? 40.f : 8.f;    // log2 of the factor by which a logit may exceed its row's reference
     static constexpr int kHalves = D / 64;                    // 64-column halves of a row of Q, K or V
     static constexpr uint32_t kSlot = kTile * D * 2;          // one K or V tile
@@ -569,8 +572,22 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
 #pragma unroll 1
             for (int j = sg.t0; j < sg.t1 && ok; ++j, ++tile) {
                 const uint32_t s = tile % S::kVSlots;
-                ok = warp_wait(&sb.v_full[s], (tile / S::kVSlots) & 1, &sb) &&
-                     warp_wait(&sb.p_full[tile % S::kSBufs], (tile / S::kSBufs) & 1, &sb);
+                ok = warp_wait(&sb.v_full[s], (tile / S::kVSlots) & 1, &sb);
+                if (S::kExactRanges && ok && (2 * j + 2) * kBN > sg.L) {      // (while the weights are worked out)
+                    // rows that a box holds past the end of the prefix or of the tree: the weights there are zero, but
+                    // zero times a NaN or an infinity of someone else's values is not
+#pragma unroll 1
+                    for (int i = 0; i < 2; ++i) {
+                        const int h = 2 * j + i, end = h < sg.nhp ? sg.L - h * kBN : sg.n_tree - (h - sg.nhp) * kBN;
+                        uint4 *box = reinterpret_cast<uint4 *>(smem + S::kOffV + s * S::kSlot + i * (kHalfStride / 2));
+                        if (h < sg.nh)
+#pragma unroll 1
+                            for (int e = end * 8 + lane; e < kBN * 8; e += 32) box[e] = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                }
+                if (ok) ok = warp_wait(&sb.p_full[tile % S::kSBufs], (tile / S::kSBufs) & 1, &sb);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t vd = desc_mn_major(smem_u32(smem + S::kOffV + s * S::kSlot), kHalfStride);

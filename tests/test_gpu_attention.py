@@ -227,3 +227,24 @@ def test_the_heaviest_weight_is_exact(d, nodes, first, second, jump):
                                         t["v_prefix"], torch.as_tensor(poff).cuda(), poff)
     assert int(status.item()) == 0
     assert (out.double() - 1 / 7).abs().max().item() <= (2.0 ** -9 + 2.0 ** -12) / 7
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("L", [[70, 200, 1, 128], [3000, 2500, 1000, 64]])
+def test_heads_of_64_do_not_see_their_neighbours_values(L, bad):
+    """bf16, d = 64: copies of 64 tokens reach into the next head's or beam's cache and tree; what lies there
+    does not reach the result, not even as zero times a NaN."""
+    rng = np.random.default_rng(L[0])
+    trees = [[-1] + [int(rng.integers(0, i)) for i in range(1, n)] for n in (5, 9, 3, 16)]
+    forest, spec, t, poff = _custom(rng, trees, L, 8, 2, 64, torch.bfloat16)
+    clean = _gpu(forest, spec, t, poff)
+    bno = forest["beam_node_off"]
+    # beam 1: head 1 of its cache, and its new tokens' head 1
+    s = int(poff[1]) * 2 * 64 + L[1] * 64
+    t["v_prefix"][s:s + L[1] * 64] = bad
+    t["v_new"][bno[1]:bno[2], 1] = bad
+    out = _gpu(forest, spec, t, poff)
+    hit = torch.zeros(out.shape[:2], dtype=torch.bool, device="cuda")
+    hit[bno[1]:bno[2], 4:] = True
+    assert not torch.isfinite(out[hit].float()).any()
+    assert torch.equal(out[~hit], clean[~hit])

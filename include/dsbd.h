@@ -107,7 +107,9 @@ typedef struct {
  * other tree or beam is visible ("topology-aware mask" extended from one tree to a forest,
  * with a separate KV cache per input beam).  prefix_off: [B+1] int64, tokens.
  * Errors: INVALID_ARG (null pointer, Hq % Hkv), UNSUPPORTED (d, dtype, tree larger than
- * DSBD_MAX_TREE_NODES, pointers not 16-byte aligned), WORKSPACE_TOO_SMALL. */
+ * DSBD_MAX_TREE_NODES, pointers not 16-byte aligned), WORKSPACE_TOO_SMALL.
+ * *status: DSBD_DEV_BAD_FOREST for a parent outside the node's tree (bf16 with d = 128 notices
+ * only a parent at or behind its own node and takes any other as none). */
 int dsbd_forest_attention(const dsbd_forest_t *forest, const dsbd_attn_desc_t *desc,
                           const void *q, const void *k_new, const void *v_new,
                           const void *k_prefix, const void *v_prefix, const int64_t *prefix_off,

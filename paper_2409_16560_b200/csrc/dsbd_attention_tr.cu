@@ -736,8 +736,10 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                         if (tok < sg.n_tree) {
                             const int par = a.parent[sg.n_lo + tok];
                             int p = par - sg.n_lo;
-                            if (par < 0 || p < 0) p = -1;
-                            else if (p >= tok) { report(a.status, DSBD_DEV_BAD_FOREST); p = -1; }
+                            // (the entry point's rules differ: d = 64 reports every parent outside the tree)
+                            const bool bad = D == 64 ? (p < 0 || p >= tok) && (tok > 0 || par != -1) : par >= 0 && p >= tok;
+                            if (bad) report(a.status, DSBD_DEV_BAD_FOREST);
+                            if (par < 0 || p < 0 || p >= tok) p = -1;
                             sx.par[grp][tok] = (int16_t)p;
                         }
                         if (tok < kMaxTree) sx.see[grp][tok] = 0u;

@@ -248,3 +248,18 @@ def test_heads_of_64_do_not_see_their_neighbours_values(L, bad):
     hit[bno[1]:bno[2], 4:] = True
     assert not torch.isfinite(out[hit].float()).any()
     assert torch.equal(out[~hit], clean[~hit])
+
+
+@pytest.mark.parametrize("node,parent", [(6, -1), (7, 1), (5, 4), (7, 7), (6, 8)])
+def test_heads_of_64_report_parents_outside_the_tree(node, parent):
+    """bf16, d = 64; trees of nodes 0-4 and 5-8: a second root, a parent in the earlier tree, a root with a parent,
+    a node that is its own parent, one that follows its node."""
+    rng = np.random.default_rng(node)
+    forest, spec, t, poff = _custom(rng, [[-1, 0, 1, 2, 3], [-1, 0, 1, 1]], [100, 300], 8, 2, 64, torch.bfloat16)
+    good = _gpu(forest, spec, t, poff)
+    f = dsbd.Forest(forest, "cuda")
+    f.dev["parent"][node] = parent
+    out, status = dsbd.forest_attention(f, 8, 2, 64, inputs.default_scale(64), t["q"], t["k_new"], t["v_new"],
+                                        t["k_prefix"], t["v_prefix"], torch.as_tensor(poff).cuda(), poff)
+    assert int(status.item()) == 4
+    assert torch.equal(out[:5], good[:5])                                # the other tree

@@ -1035,9 +1035,11 @@ TcPlan make_plan(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
 }
 
 size_t partial_offset(const TcPlan &p, int n_layers) { return align_up(sizeof(CutRec) * (size_t)p.runs * n_layers, 256); }
+// (d = 64 takes a workspace of any alignment, as it always has, and aligns it itself)
 size_t workspace_of(const TcPlan &p, int n_layers, int d) {
     if (p.whole) return 256;
-    return align_up(partial_offset(p, n_layers) + sizeof(float) * 2 * (size_t)p.runs * n_layers * p.nmax * (d + 2), 256);
+    return align_up(partial_offset(p, n_layers) + sizeof(float) * 2 * (size_t)p.runs * n_layers * p.nmax * (d + 2), 256) +
+           (d == 64 ? 256 : 0);
 }
 
 template <int D, int NMAX>
@@ -1109,7 +1111,8 @@ int launch_attention_tr(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const
     const int nl = LD.n_layers;
     const TcPlan plan = make_plan(f, d);
     if (workspace_bytes < workspace_of(plan, nl, d->d)) return DSBD_ERR_WORKSPACE_TOO_SMALL;
-    if (!plan.whole && (reinterpret_cast<uintptr_t>(workspace) & 255)) return DSBD_ERR_INVALID_ARG;
+    const uintptr_t ws = d->d == 64 ? align_up(reinterpret_cast<uintptr_t>(workspace), 256) : reinterpret_cast<uintptr_t>(workspace);
+    if (!plan.whole && (ws & 255)) return DSBD_ERR_INVALID_ARG;
     // one map per operand over all layers: layer l starts l * (layer stride in rows) further down
     const uint64_t D = (uint64_t)d->d;
     const uint64_t prows = pages ? (uint64_t)pages->n_pages * d->Hkv * kBN + (uint64_t)(nl - 1) * LD.pool_rows
@@ -1142,8 +1145,8 @@ int launch_attention_tr(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const
     a.n_layers = nl; a.pool_layer_rows = LD.pool_rows; a.new_layer_rows = LD.new_rows;
     a.q_layer_stride = LD.q_stride;
     a.q_layer_nodes = (int)q_layer_nodes;
-    a.recs = static_cast<CutRec *>(workspace);
-    a.partial = reinterpret_cast<float *>(static_cast<char *>(workspace) + partial_offset(plan, nl));
+    a.recs = reinterpret_cast<CutRec *>(ws);
+    a.partial = reinterpret_cast<float *>(ws + partial_offset(plan, nl));
     if (d->d == 64)
         return plan.nmax == 32 ? launch<64, 32>(plan, maps, a, stream) : launch<64, 64>(plan, maps, a, stream);
     return plan.nmax == 32 ? launch<128, 32>(plan, maps, a, stream) : launch<128, 64>(plan, maps, a, stream);

@@ -263,3 +263,19 @@ def test_heads_of_64_report_parents_outside_the_tree(node, parent):
                                         t["k_prefix"], t["v_prefix"], torch.as_tensor(poff).cuda(), poff)
     assert int(status.item()) == 4
     assert torch.equal(out[:5], good[:5])                                # the other tree
+
+
+@pytest.mark.parametrize("shift", [1, 8, 100])
+def test_heads_of_64_take_a_workspace_of_any_alignment(shift):
+    rng = np.random.default_rng(shift)
+    forest, spec, t, poff = _custom(rng, [[-1, 0, 1], [-1, 0]], [4000, 5000], 8, 2, 64, torch.bfloat16)
+    f = dsbd.Forest(forest, "cuda")
+    scale = inputs.default_scale(64)
+    assert dsbd.forest_attention_launches(f, 8, 2, 64, torch.bfloat16, scale, poff) == 2       # (units are cut)
+    need = dsbd.forest_attention_workspace(f, 8, 2, 64, torch.bfloat16, scale, poff)
+    buf = torch.full((need + shift,), 0x77, dtype=torch.uint8, device="cuda")
+    out, status = dsbd.forest_attention(f, 8, 2, 64, scale, t["q"], t["k_new"], t["v_new"], t["k_prefix"],
+                                        t["v_prefix"], torch.as_tensor(poff).cuda(), poff, workspace=buf[shift:])
+    assert int(status.item()) == 0
+    assert torch.equal(out, _gpu(forest, spec, t, poff))
+    assert (buf[:shift] == 0x77).all()

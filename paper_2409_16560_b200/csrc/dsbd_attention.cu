@@ -175,6 +175,7 @@ k_forest_attn_simt(AttnArgs a) {
         for (int j0 = split; j0 < cnt; j0 += kChunk * a.splits) {
             float s[kChunk];
             float tmax = -INFINITY;
+            bool any = false;                                    // some token counts (a NaN does, and is no maximum)
 #pragma unroll
             for (int i = 0; i < kChunk; ++i) {
                 const int j = j0 + i * a.splits;
@@ -197,8 +198,9 @@ k_forest_attn_simt(AttnArgs a) {
                 s[i] += __shfl_xor_sync(3u << (tid & 30), s[i], 1);
                 if (j >= cnt || !(visible >> j & 1u)) s[i] = -INFINITY;
                 tmax = fmaxf(tmax, s[i]);
+                any = any || s[i] != -INFINITY;
             }
-            if (tmax > -INFINITY) {
+            if (any) {
                 const float mnew = fmaxf(mrun, tmax);
                 const float corr = exp2f(mrun - mnew);      // 0 when mrun == -inf
                 lrun *= corr;

@@ -279,3 +279,18 @@ def test_heads_of_64_take_a_workspace_of_any_alignment(shift):
     assert int(status.item()) == 0
     assert torch.equal(out, _gpu(forest, spec, t, poff))
     assert (buf[:shift] == 0x77).all()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("max_rows,L,at", [(40, 25, 24), (40, 96, 40), (24, 49, 48), (8, 33, 32), (8, 1, 0)])
+def test_a_nan_key_reaches_its_rows(d, max_rows, L, at):
+    """A NaN among the keys makes every row that sees it NaN, also where it is the only token of the last group that a
+    pair of threads takes (splits 1, 2 and 4); another beam does not see it."""
+    rng = np.random.default_rng(d + max_rows)
+    trees = [[-1] + [int(rng.integers(0, i)) for i in range(1, max_rows)], [-1, 0]]
+    forest, spec, t, poff = _custom(rng, trees, [L, 40], 2, 2, d, torch.float32)
+    clean = _gpu(forest, spec, t, poff)
+    t["k_prefix"].view(-1, d)[at] = float("nan")                         # beam 0, head 0
+    out = _gpu(forest, spec, t, poff)
+    assert torch.isnan(out[:max_rows, 0]).all()
+    assert torch.equal(out[:, 1], clean[:, 1]) and torch.equal(out[max_rows:], clean[max_rows:])

@@ -401,7 +401,7 @@ __device__ __noinline__ int locate_token(const float *__restrict__ rp, const flo
 constexpr int kCacheNodes = 256;
 struct NodeCache {
     double score_p[kCacheNodes], score_q[kCacheNodes], lse_p[kCacheNodes], lse_q[kCacheNodes];
-    int16_t parent[kCacheNodes];          // local index of the parent, -1 for a root
+    int16_t parent[kCacheNodes];          // local index of the parent, -1 for a root, -2: none inside the request
     uint8_t depth[kCacheNodes];
     uint8_t tree[kCacheNodes];            // tree of the node, inside the request
     int root[kMaxLive];                   // first node of every tree
@@ -1250,7 +1250,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                         zq_tok = a.zq[(int64_t)par * a.stride + tok];
                     }
                 }
-                nc.parent[i] = (int16_t)((par >= n_lo && par < n) ? par - n_lo : -1);
+                nc.parent[i] = (int16_t)((par >= n_lo && par < n) ? par - n_lo : par < 0 ? -1 : -2);
             }
         }
         cluster.barrier_wait();
@@ -1413,6 +1413,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     }
 
     // ---- set-up ----
+    auto is_root = [&](int i) { return cached ? nc.parent[i] == -1 : a.parent[n_lo + i] < 0; };
     if (warp == 0) {
         if (lane == 0) {
             sh.err = 0; sh.done = 0; sh.n_out = 0; sh.n_fill = 0;
@@ -1455,7 +1456,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         __syncwarp();
         if (!a.select_mode && writer)
             for (int n = n_lo + lane; n < n_hi; n += 32)
-                a.out.node_status[n] = (cached ? nc.parent[n - n_lo] : a.parent[n]) < 0 ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+                a.out.node_status[n] = is_root(n - n_lo) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     }
     // Every CTA of the cluster takes identical decisions from identical data, so each keeps its
     // own copy of the node statuses and only rank 0 writes results.
@@ -1463,7 +1464,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     const bool st_ok = n_req_nodes <= kMaxLive * kMaxLive;
     if (!a.select_mode)
         for (int n = threadIdx.x; n < n_req_nodes && st_ok; n += blockDim.x)
-            st[n] = (cached ? nc.parent[n] : a.parent[n_lo + n]) < 0 ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+            st[n] = is_root(n) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     __syncthreads();
     if (!a.select_mode && !st_ok && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
     if (bad_widths && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_PARAM;

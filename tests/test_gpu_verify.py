@@ -590,3 +590,22 @@ def test_residual_next_to_a_dominant_cell():
     assert (gpu["out_source"] == 1).all() and (gpu["l_last"] == 1).all()
     share = np.isin(gpu["out_token"], small).mean()
     assert share > 0.545, share
+
+
+def test_a_node_with_a_malformed_parent_is_not_accepted():
+    """A parent at or behind its own node is reported; the node stays unreached, its descendants are pruned."""
+    rng = np.random.default_rng(2)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=1, V=600, gamma=4, max_w=3, min_w=3)
+    prm.update(W_min=1, W_min_r=None, thresh=0.3)
+    lo = int(forest["beam_node_off"][1])
+    forest["parent"] = forest["parent"].copy()
+    forest["parent"][lo + 1] = lo + 3
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    f = dsbd.Forest(dict(forest, parent=np.where(forest["parent"] == lo + 3, lo, forest["parent"])), "cuda")
+    f.dev["parent"] = torch.as_tensor(forest["parent"]).cuda()
+    prm_dev = dict(prm)
+    out = dsbd.alloc_verify_out(f, oracle.default_out_off(forest, prm), "cuda")
+    status = dsbd.verify_step(f, prm_dev, *dev, out)
+    assert int(status.item()) == 4
+    got = out["node_status"].cpu().numpy()[lo:lo + 5]
+    assert got[0] == 1 and got[1] == 0 and got[2] == 4, got

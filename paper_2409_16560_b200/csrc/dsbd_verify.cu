@@ -1531,7 +1531,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     for (int i = lane; i < m; i += 32) {
                         const int key = sh.S_parent_idx[i];
                         int place = 0;
-                        for (int j = 0; j < m; ++j) place += sh.S_parent_idx[j] < key + (j < i);
+                        for (int j = 0; j < m; ++j) place += sh.S_parent_idx[j] < key || (j < i && sh.S_parent_idx[j] == key);
                         sh.acc[place] = sh.S[i];
                     }
                     __syncwarp();

@@ -609,3 +609,21 @@ def test_a_node_with_a_malformed_parent_is_not_accepted():
     assert int(status.item()) == 4
     got = out["node_status"].cpu().numpy()[lo:lo + 5]
     assert got[0] == 1 and got[1] == 0 and got[2] == 4, got
+
+
+def test_draft_ranks_up_to_the_type_s_largest():
+    """Equal ranks go by node id, whatever their value."""
+    rng = np.random.default_rng(9)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=4, V=900, gamma=3, max_w=8, min_w=8)
+    big = np.iinfo(np.int32).max
+    forest["draft_rank"] = rng.choice([big, big, big - 1, 0, np.iinfo(np.int32).min], forest["N"]).astype(np.int32)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = 0
+    for step in range(10):
+        prm["step"] = step
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+    check_exempt(exempt, decisions)

@@ -74,3 +74,13 @@ def test_forest_depths_match_a_plain_walk():
         for i, p in enumerate(parent):
             ref[i] = 0 if p < 0 else ref[p] + 1
         assert np.array_equal(_node_depths(parent), ref)
+
+
+def test_the_current_stream_without_torch_s_raw_calls(monkeypatch):
+    """A torch without the raw calls is asked for its Stream object."""
+    import types
+    import torch
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=11))
+    assert binding._stream_reader(types.SimpleNamespace())() == 11
+    raw = types.SimpleNamespace(_cuda_getCurrentRawStream=lambda device: 70 + device, _cuda_getDevice=lambda: 2)
+    assert binding._stream_reader(raw)() == 72

@@ -118,8 +118,9 @@ int dsbd_forest_attention(const dsbd_forest_t *forest, const dsbd_attn_desc_t *d
 
 size_t dsbd_forest_attention_workspace(const dsbd_forest_t *forest, const dsbd_attn_desc_t *desc);
 
-/* How many kernels dsbd_forest_attention launches for this shape (1: the attention kernel; 2:
- * plus the merge of cut units), 0 for invalid arguments.  For launch accounting; host-only. */
+/* How many kernels dsbd_forest_attention launches for this shape, 0 for invalid arguments: the
+ * attention kernel, plus the merge of cut units, plus (trees of more than 64 query rows per KV
+ * head) a work plan: 1 to 3.  For launch accounting; host-only. */
 int dsbd_forest_attention_launches(const dsbd_forest_t *forest, const dsbd_attn_desc_t *desc);
 
 /* The same attention over PAGED caches.  The paper keeps one key-value cache per input beam and

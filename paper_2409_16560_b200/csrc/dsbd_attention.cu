@@ -66,8 +66,9 @@ struct AttnArgs {
 // chain's step), and the parents are read at once.  Smem rows are padded by 32 bytes: the 16-byte words that
 // the pairs of a row and the threads of a pair read together lie in different banks.
 // fp32, one thread pair a row, tiles loaded when needed, parents read one by one against this: 2 beams x 15 nodes x
-// 4 heads of 64 after 64 tokens 22.7 and 13.7 us a call; 8 requests, 6 nodes, 8 heads of 64 after 200-600 tokens
-// 174 and 47; 40 requests, 24 rows a unit 507 and 143; heads of 128 in groups of 4 334 and 158.
+// 4 heads of 64 after 64 tokens 22.7 and 13.7 us a call (10.4 since the binding takes less of it); 8 requests, 6 nodes, 8 heads of 64 after 200-600 tokens
+// 174 and 47; 40 requests, 24 rows a unit 507 and 143; heads of 128 in groups of 4 334 and 158 (fp32 at d = 128 spills
+// 84 bytes at 255 registers).
 template <class T, int D>
 __global__ void __launch_bounds__(kThreads)
 k_forest_attn_simt(AttnArgs a) {

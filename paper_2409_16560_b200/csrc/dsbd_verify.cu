@@ -394,8 +394,6 @@ __device__ __noinline__ int locate_token(const float *__restrict__ rp, const flo
     }
 }
 
-// Beam weights of the live set: softmax of the cumulative scores over A (Eq. 1 factorised).
-// Called by all lanes of one warp; beam i is handled by lane i % 32.
 // Per-node data of the request that every layer's set-up reads, kept in shared memory when the
 // request is small enough (otherwise the set-up reads the global arrays).
 constexpr int kCacheNodes = 256;
@@ -451,7 +449,8 @@ __device__ __forceinline__ void log_softmax_warp(const double *s, int n, int lan
     __syncwarp();
 }
 
-// The weights of one model (0: p, 1: q) over the live set, by one warp; the two models' warps work side by side.
+// The weights of one model (0: p, 1: q) over the live set: softmax of the cumulative scores over A (Eq. 1 factorised),
+// by one warp; the two models' warps work side by side.
 // nc: the request's node cache or nullptr; n_lo: first node of the request.
 __device__ void live_weights(const VerifyArgs &a, Shared &sh, int model, const double *scores, int lane,
                              const NodeCache *nc, int n_lo) {
@@ -2066,8 +2065,9 @@ int launch_verify(const VerifyArgs &args, int R, int tiles, cudaStream_t stream)
     attr[0].val.clusterDim.x = (unsigned)cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    // the clusters may be set up while the dense pass before them drains; the kernel waits for
-    // that grid's results (griddepcontrol.wait) before it reads anything
+    // the clusters may be set up while the dense pass before them drains.  Before griddepcontrol.wait the kernel
+    // reads what the caller gave (forest, widths, logits), after it the statistics: that holds as long as the dense pass
+    // itself is launched without this attribute, so that it starts when all earlier work in the stream is done
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
@@ -2122,6 +2122,7 @@ extern "C" int dsbd_verify_step(const dsbd_forest_t *f, const dsbd_verify_params
     const float k2 = (float)((double)kLog2e * inv_tau);
 
     const int64_t items = (int64_t)2 * f->N * L.T;
+    // (never with programmatic stream serialization: k_verify reads the caller's arrays before it waits for this grid)
     k_tile_stats<<<stats_grid(items), kThreads, 0, stream>>>(logits_p, logits_q, row_stride, p->V, L.T,
                                                             f->N, f->N, nullptr, nullptr, k2, stats);
     if (cudaGetLastError() != cudaSuccess) return DSBD_ERR_CUDA;
@@ -2326,6 +2327,7 @@ extern "C" int dsbd_draft_layer(int32_t R, int32_t n_beams, const int32_t *req_b
     d.req_error = req_error;
 
     const int64_t items = (int64_t)n_beams * D.T;
+    // (never with programmatic stream serialization: k_draft reads the caller's arrays before it waits for this grid)
     k_tile_stats<<<stats_grid(items), kThreads, 0, stream>>>(logits_q, logits_q, row_stride, p->V, D.T, n_beams,
                                                             n_beams, nullptr, nullptr, a.k2, stats, 1);
     if (cudaGetLastError() != cudaSuccess) return DSBD_ERR_CUDA;

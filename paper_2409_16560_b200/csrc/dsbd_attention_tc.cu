@@ -733,13 +733,11 @@ struct TcPlan {
     size_t off_items, off_units, off_partial, total;
 };
 
-// Query rows per row block.  Trees of up to 64 rows take the 64-row tile (two CTAs per SM).  So do
-// forests whose AVERAGE tree has at most 64 rows even when the largest is bigger (a sampled
-// forest puts most drafts under a few roots and leaves the other trees tiny): the big trees then
-// run as several 64-row blocks, the many small ones at the faster shape.
+// Query rows per row block.  Forests whose AVERAGE tree has at most 64 rows take the 64-row tile (two CTAs per
+// SM) although the largest is bigger (a sampled forest puts most drafts under a few roots and leaves the
+// other trees tiny): the big trees then run as several 64-row blocks, the many small ones at the faster shape.
 int tile_rows_for(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
     const int group = d->Hq / d->Hkv;
-    if (f->max_tree_nodes * group <= 64) return 64;
     return ((int64_t)f->N * group <= (int64_t)64 * f->B && group <= 64) ? 64 : kRows;
 }
 // Rows of a row block: whole nodes (the copy engine fetches a block's query rows as a box of nodes x

@@ -1015,10 +1015,9 @@ TcPlan make_plan(const dsbd_forest_t *f, const dsbd_attn_desc_t *d) {
     p.nmax = p.block_rows <= 32 ? 32 : 64;
     p.q_nodes = std::min(p.block_rows / group, f->max_tree_nodes);
     p.q_rows = (p.q_nodes * group + 7) / 8 * 8;
-    const int tree_boxes = (f->max_tree_nodes + kBN - 1) / kBN;
-    const int64_t max_nt = ((d->max_prefix + kBN - 1) / kBN + tree_boxes + 1) / 2;
+    const int64_t max_nt = ((d->max_prefix + kBN - 1) / kBN + 2) / 2;         // (the tree is one box)
     const int64_t units = (int64_t)f->B * d->Hkv;
-    const bool uniform = p.row_blocks == 1 && tree_boxes == 1 && d->max_prefix * f->B == d->total_prefix;
+    const bool uniform = p.row_blocks == 1 && d->max_prefix * f->B == d->total_prefix;
     // tiles of a layer (ragged: a lower bound)
     const int64_t tiles = uniform ? units * max_nt : std::max<int64_t>(units, d->total_prefix / kTile * d->Hkv);
     const int64_t cut_len = std::max<int64_t>((tiles + sms - 1) / sms, kMinTiles) + kCutTiles;

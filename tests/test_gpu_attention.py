@@ -102,7 +102,8 @@ def test_ragged_prefixes_and_tree_shapes(dtype, Hq, Hkv, d):
 @pytest.mark.parametrize("max_rows", [1, 16, 17, 32, 33, 64])
 def test_cuda_core_kernel_row_splits(dtype, d, max_rows):
     """Query rows around the sizes where a row has 4, 2 or 1 thread pairs, prefixes around the 32-token tile and
-    around the tokens that a pair takes between two updates (bf16 runs here with a group beyond the tensor cores')."""
+    around the tokens that a pair takes between two updates (bf16 comes here with a group beyond the tensor cores', that
+    is with 65 rows or more and one pair a row; without any prefix below)."""
     rng = np.random.default_rng(max_rows + d)
     rand_tree = lambda n: [-1] + [int(rng.integers(0, i)) for i in range(1, n)]
     group = 1 if dtype == torch.float32 else 65
@@ -112,6 +113,18 @@ def test_cuda_core_kernel_row_splits(dtype, d, max_rows):
     out = _gpu(forest, spec, t, poff)
     nodes, ref = _oracle_beams(forest, spec, t, poff, list(range(len(trees))))
     attention_close(to_host_f32(out), ref, bf16=dtype == torch.bfloat16)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("max_rows", [1, 16, 17, 32, 33, 64])
+def test_cuda_core_kernel_without_any_prefix(d, max_rows):
+    """bf16 trees of up to 64 rows whose beams have no cache: 4, 2 and 1 thread pairs a row."""
+    rng = np.random.default_rng(max_rows + d)
+    trees = [[-1] + [int(rng.integers(0, i)) for i in range(1, n)] for n in (max_rows, 1, (max_rows + 1) // 2)]
+    forest, spec, t, poff = _custom(rng, trees, [0, 0, 0], 2, 2, d, torch.bfloat16)
+    out = _gpu(forest, spec, t, poff)
+    nodes, ref = _oracle_beams(forest, spec, t, poff, list(range(len(trees))))
+    attention_close(to_host_f32(out), ref, bf16=True)
 
 
 @pytest.mark.parametrize("Hq,Hkv,max_nodes", [(8, 2, 32), (16, 2, 16), (4, 4, 64), (32, 8, 9), (40, 40, 20)])
@@ -164,9 +177,11 @@ def test_trees_with_more_than_128_query_rows(Hq, Hkv, sizes, L):
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("sizes,L,Hq,Hkv,amp", [
     ([16, 4, 1, 2], [127, 128, 129, 1], 16, 4, 1.0),         # edges of the 128-token tiles, 64 rows
-    ([17, 4], [200, 333], 16, 4, 1.0),                       # 68 rows: the 128-row instance
+    ([17, 4], [200, 333], 16, 4, 1.0),                       # 68 rows: at d = 128 rows on the M side, else two blocks
     ([9, 4], [2000, 3333], 8, 2, 12.0),                      # logits far above the first token's: references move
     ([30, 4], [2000, 3333], 8, 2, 12.0),
+    ([8, 4], [2000, 3333], 8, 2, 12.0),                      # the same with 32 rows: cut units,
+    ([8, 3] * 20, [300] * 40, 4, 4, 12.0),                   # whole ones
     ([6] * 30, list(range(1000, 3900, 97))[:30], 32, 8, 1.0),    # many cut units, different shares of the rows
     ([1, 9] * 20, [300] * 40, 4, 4, 1.0),                    # equal lengths, whole units
 ])

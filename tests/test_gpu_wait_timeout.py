@@ -1,6 +1,6 @@
-"""A bounded wait of the tensor-core attention kernel that runs out.
+"""A bounded wait of the tensor-core attention kernels that runs out.
 
-Every mbarrier wait of that kernel gives up after a limit, records DSBD_DEV_TIMEOUT, lets the
+Every mbarrier wait of these kernels gives up after a limit, records DSBD_DEV_TIMEOUT, lets the
 copies in flight land, frees its tensor memory and returns.  The product library offers no way
 to make a wait run out, so this test builds a second library from the same sources with
 DSBD_TEST_WAIT_TIMEOUT: the limit drops to about a millisecond and the copy producer of one CTA
@@ -38,11 +38,14 @@ def _wait_library():
     return lib
 
 
-def test_a_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable():
+@pytest.mark.parametrize("sizes", [[9, 5, 12, 3], [20, 17, 25, 18], [20, 2, 3, 2]])
+def test_a_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable(sizes):
+    """Trees of at most 48 query rows: the transposed kernel; of 68 to 100 and of 8 to 80: the 128-row and the 64-row
+    instance of the kernel with the rows on the M side (their units are cut: the combination follows)."""
     lib = _wait_library()
     rng = np.random.default_rng(31)
     rand_tree = lambda n: [-1] + [int(rng.integers(0, i)) for i in range(1, n)]
-    trees = [rand_tree(9), rand_tree(5), rand_tree(12), rand_tree(3)]
+    trees = [rand_tree(n) for n in sizes]
     L = [700, 300, 1000, 200]                              # every unit has several tiles
     forest, spec, t, poff = _custom(rng, trees, L, 8, 2, 128, torch.bfloat16)
     f = dsbd.Forest(forest, "cuda")
@@ -64,8 +67,8 @@ def test_a_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable():
         assert rc == 0
         torch.cuda.synchronize()                           # returns: the wait was bounded
         assert int(status.item()) == DEV_TIMEOUT
-    # 250 tries (4 us each) for the tile, and again for the copies in flight.  The product library's limit is 2000
-    # times this one: seconds
+    # about a millisecond (250 tries of 4 us, or 2e6 cycles) for the tile, and again for the copies in flight.  The
+    # product library's limits are 1000 and 2000 times these: a second or two
     assert begin.elapsed_time(end) < 8.0
     assert "wait" in dsbd.status_string(DEV_TIMEOUT)
     # the CTAs whose tiles all arrived did their work: the last tree's rows are right

@@ -882,8 +882,8 @@ struct SupportTmp {
     int sel[256];                 // tiles whose bound reaches the threshold
     unsigned lo[kVWarps], hi[kVWarps];   // per warp, images of the smallest finite and of the largest bound
     int finite[kVWarps];          // per warp, finite bounds
-    int count[3];                 // of the bisection's rounds, in turn: bounds above the cut, and
-    unsigned low[3];              // the image of the smallest of them
+    int count[3];                 // of the bisection's rounds, in turn
+    unsigned low;                 // image of the smallest bound from the cut on
     int n_sel, n_cand, err;
 };
 struct WarpScratch {
@@ -930,8 +930,8 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     const float *z = model ? a.zq : a.zp;
     const float inv_tau_f = (float)a.inv_tau;
     for (int i = tl; i < sh.nA; i += NT) tp.off[i] = (float)(lw[i] - lse[sh.A[i]]);
-    if (tl < 3) { tp.count[tl] = 0; tp.low[tl] = 0xffffffffu; }
-    if (tl == 0) { tp.n_sel = 0; tp.n_cand = 0; tp.err = 0; ws.n[model] = 0; }
+    if (tl < 3) tp.count[tl] = 0;
+    if (tl == 0) { tp.low = 0xffffffffu; tp.n_sel = 0; tp.n_cand = 0; tp.err = 0; ws.n[model] = 0; }
     part_sync<NT>(model);
     // float upper bound of log(joint probability) over tile i
     auto bound = [&](int i) -> float {
@@ -944,10 +944,9 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
     };
     auto value = [](unsigned u) -> float { return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u); };
-    // The k-th largest tile bound (with multiplicity: k tiles each hold a cell at least that large), or the next or
-    // next but one where these lie close; with fewer than k finite bounds every tile counts.  It must be a
-    // bound and not merely a cut below: a bisection's cut may lie far down in the gap above masked tiles,
-    // where it passes every cell of the tiles above.  Bounds that do not fit the cache are computed again in every round.
+    // A cut not above the k-th largest tile bound (with multiplicity: k tiles each hold a cell at least that
+    // large) with few tiles below it; with fewer than k finite bounds every tile counts.  Bounds that do not fit
+    // the cache are computed again in every round.
     unsigned *bcache = hist_p + (2 + model) * kHistWords;
     const bool cached = nt <= kBoundCache;
     {
@@ -969,43 +968,51 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
 #pragma unroll
     for (int w = 0; w < kPartWarps; ++w) { lo = min(lo, tp.lo[w]); hi = max(hi, tp.hi[w]); finite += tp.finite[w]; }
     if (finite >= k) {
-        // count(>= lo) >= k always holds; hi is above the k-th largest
-        const float near = value(hi) - 30.f;                      // (cells below have no mass to speak of)
-        auto done = [&](int n) { return n == k || (n <= k + 2 && value(lo) > near); };
+        // count(>= lo) >= k always holds; hi is above the k-th largest.  One or two too many are fine where they are close
+        // (cells 30 below the largest have no mass to speak of)
+        const float near = value(hi) - 30.f;
         ++hi;
-        for (int round = 0; hi - lo > 1 && !(round == 0 && done(finite)); ++round) {
+        for (int round = 0; hi - lo > 1; ++round) {
             const unsigned mid = lo + (hi - lo) / 2;
             int n = 0;
-            unsigned low = 0xffffffffu;
-            for (int i = tl; i < nt; i += NT) {
-                const unsigned u = cached ? bcache[i] : image(bound(i));
-                if (u >= mid) { ++n; low = min(low, u); }
-            }
+            for (int i = tl; i < nt; i += NT) n += (cached ? bcache[i] : image(bound(i))) >= mid;
             n = __reduce_add_sync(kFull, n);
-            low = __reduce_min_sync(kFull, low);
-            if (lane == 0 && n) { atomicAdd(&tp.count[round % 3], n); atomicMin(&tp.low[round % 3], low); }
-            if (tl == 0) { tp.count[(round + 1) % 3] = 0; tp.low[(round + 1) % 3] = 0xffffffffu; }     // (last read two rounds ago)
+            if (lane == 0 && n) atomicAdd(&tp.count[round % 3], n);
+            if (tl == 0) tp.count[(round + 1) % 3] = 0;           // (last read two rounds ago)
             part_sync<NT>(model);
             n = tp.count[round % 3];
             if (n < k) { hi = mid; continue; }
-            lo = tp.low[round % 3];
-            if (done(n)) break;
+            lo = mid;
+            if (n == k || (n <= k + 2 && value(lo) > near)) break;
         }
     }
-    const float thr = value(lo);
-    // the float keys carry an error of about 1e-5; the slack keeps the selection conservative
-    float theta = finite >= k ? thr - 5e-5f - 4e-6f * fabsf(thr) : -INFINITY;
-    if (finite > 0)
+    // The tiles from the cut on, and the smallest bound among them, which is the threshold: a cut may lie far down in
+    // the gap above masked tiles, where it would pass every cell of the tiles above.
+    // (the float keys carry an error of about 1e-5; the slack keeps the selection conservative)
+    auto slack = [](float t) -> float { return t - 5e-5f - 4e-6f * fabsf(t); };
+    float theta = -INFINITY, cut = finite >= k ? slack(value(lo)) : -INFINITY;
+    for (int again = 0; ; ++again) {
+        unsigned low = 0xffffffffu;
         for (int i = tl; i < nt; i += NT) {
             const float bv = cached ? value(bcache[i]) : bound(i);
-            if (bv >= theta && bv > -INFINITY) {
+            if (bv >= cut && bv > -INFINITY) {
                 const int pos = atomicAdd(&tp.n_sel, 1);
                 if (pos < 256) tp.sel[pos] = i;
-                else tp.err = DSBD_DEV_CAPACITY;                  // hundreds of tiles tie at the cut
+                if (image(bv) >= lo) low = min(low, image(bv));
             }
         }
-    part_sync<NT>(model);
-    if (tp.err) return tp.err;
+        low = __reduce_min_sync(kFull, low);
+        if (lane == 0 && low != 0xffffffffu) atomicMin(&tp.low, low);
+        part_sync<NT>(model);
+        if (finite >= k) theta = slack(value(tp.low));
+        if (tp.n_sel <= 256) break;
+        if (again) return DSBD_DEV_CAPACITY;                      // hundreds of tiles tie at the threshold
+        // (or closely below the cut)
+        part_sync<NT>(model);
+        if (tl == 0) tp.n_sel = 0;
+        cut = theta;
+        part_sync<NT>(model);
+    }
     const int n_sel = tp.n_sel;
     // One sweep over the selected tiles by all warps: counts the cells whose key reaches th and,
     // when asked, appends them to the candidate list (order is irrelevant: the final choice is

@@ -148,19 +148,15 @@ def _ptr(t):
 
 
 def _stream_reader(c):
-    """A call that gives the raw handle of the current stream: torch's own (making the Stream object takes 3 us, an
-    eighth of a call's host time) where this torch has it."""
+    """A call that gives the raw handle of a stream, or of the current one for None: by torch's own calls (making the
+    Stream object takes 3 us, an eighth of a call's host time) where this torch has them."""
     raw, device = getattr(c, "_cuda_getCurrentRawStream", None), getattr(c, "_cuda_getDevice", None)
     if raw is None or device is None:
-        return lambda: torch.cuda.current_stream().cuda_stream
-    return lambda: raw(device())
+        return lambda stream: (torch.cuda.current_stream() if stream is None else stream).cuda_stream
+    return lambda stream: raw(device()) if stream is None else stream.cuda_stream
 
 
-_current_stream = _stream_reader(torch._C)
-
-
-def _stream(stream):
-    return _current_stream() if stream is None else stream.cuda_stream
+_stream = _stream_reader(torch._C)
 
 
 def _widest(off):

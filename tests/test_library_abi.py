@@ -81,6 +81,8 @@ def test_the_current_stream_without_torch_s_raw_calls(monkeypatch):
     import types
     import torch
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=11))
-    assert binding._stream_reader(types.SimpleNamespace())() == 11
+    assert binding._stream_reader(types.SimpleNamespace())(None) == 11
     raw = types.SimpleNamespace(_cuda_getCurrentRawStream=lambda device: 70 + device, _cuda_getDevice=lambda: 2)
-    assert binding._stream_reader(raw)() == 72
+    for reader in (binding._stream_reader(types.SimpleNamespace()), binding._stream_reader(raw)):
+        assert reader(types.SimpleNamespace(cuda_stream=5)) == 5
+    assert binding._stream_reader(raw)(None) == 72

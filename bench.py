@@ -30,11 +30,11 @@ METRIC = "verified forest nodes/sec per decode step"
 UNIT = "nodes/s"
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) on the full C5 workload,
-# from ncu captures of the same kernels on 16 of the 64 requests, scaled by 64/16 (the traffic is
-# proportional to the number of requests).  verify_step_total = the dense pass plus the
-# per-request kernel, which re-reads the live rows.
-NCU_TRAFFIC_BYTES = {"C5": {"forest_attention": 8.665e9, "verify_dense_pass": 4.748e9,
-                            "verify_step_total": 4.748e9 + 0.740e9}}
+# from ncu captures of k_forest_attn_tr, k_tile_stats and k_verify on 16 of the 64 requests, scaled by 64/16
+# (the traffic is proportional to the number of requests).  verify_step_total = the dense pass plus the
+# per-request kernel, which re-reads the live rows (unwarped; with a top-k 0.018e9).
+NCU_TRAFFIC_BYTES = {"C5": {"forest_attention": 8.776e9, "verify_dense_pass": 4.748e9,
+                            "verify_step_total": 4.748e9 + 0.729e9}}
 
 
 def _peaks():

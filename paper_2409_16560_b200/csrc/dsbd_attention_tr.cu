@@ -27,8 +27,8 @@
 //
 // A row's reference is its largest logit in the unit's first tile, moved to a later tile's largest when that exceeds
 // it by more than 2^8.  The heaviest weight of a row is then mostly a power of two, which bf16 holds exactly: with the
-// first token's logit as the reference (one barrier less a unit) the error against 64 bits was up to 5.7 % larger,
-// at prefixes of 64 to 200 tokens.  Weights in two terms (kSplit) do not need that: there the first token's logit is the
+// first token's logit as the reference (one barrier less a unit) the error against 64 bits was up to 7.5 % larger,
+// at prefixes of about 70 tokens.  Weights in two terms (kSplit) do not need that: there the first token's logit is the
 // reference, moved when exceeded by more than 2^40 (0.4 us of 31.3 for 8 x 4 beams after 512 to 2047 tokens).
 //
 // Work split: the tiles of a layer's units form one sequence (beam, KV head, row block), cut into equal

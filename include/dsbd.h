@@ -222,8 +222,10 @@ typedef struct {
     float   *lse_q;
     int32_t *req_error;     /* [R]  0 or a DSBD_DEV_* code                                   */
     int32_t *req_stats;     /* [R*DSBD_REQ_STATS] or NULL, per request: 0 layers verified, 1 accept
-                                    tests made, 2 residual masses recomputed exactly by a pass over
-                                    the rows, 3 extra passes made for completion draws, 4 accept
+                                    tests made, 2 residual masses of the histogram recomputed exactly by a
+                                    pass over the rows, 3 extra passes made for completion draws (layers
+                                    whose width needs no residual mass make their passes on demand and
+                                    count in neither), 4 accept
                                     tests with |u - ratio| < 1e-5 (near ties), 5 logits row pairs
                                     consulted after the dense pass (live parents summed over the
                                     verified layers), 6 layers whose histogram overflowed a word and

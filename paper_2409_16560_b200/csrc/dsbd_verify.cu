@@ -243,6 +243,8 @@ struct Shared {
     double col_a[kMaxLive + 1], col_b[kMaxLive + 1];
     double tail[kMaxLive + 2];
     int bank, halves, need_exact, res_j, run_j, chain_pos;
+    int on_demand, next_i;                  // a layer of known width: its passes are made when the accept loop asks
+    long long warp_part[kVWarps], part[2][16];      // sums of an exact pass: of this CTA's warps; of every CTA, two passes in turn
     int n_out, n_fill;                      // output beams so far; p_beam fills left to the whole CTA
     int n_layers, n_tests, n_exact, n_respass;
     int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows consulted
@@ -272,47 +274,6 @@ __device__ __forceinline__ void split_offset(double b, float *bi, float *c, doub
 
 __device__ __forceinline__ RowOff row_off(const Shared &sh, int i) {
     return RowOff{sh.bp[i], sh.bq[i], sh.cp[i], sh.cq[i], (float)(sh.rp[i] - sh.rq[i])};
-}
-
-// One cluster-wide pass: tile sums of max(p_beam - s q_beam, 0) over the live rows.
-__device__ void residual_pass(const VerifyArgs &a, const Shared &sh, float s, double *sums,
-                              int cta_rank, int n_cta) {
-    const int lane = threadIdx.x & 31;
-    const int warp = cta_rank * kVWarps + (threadIdx.x >> 5);
-    const int nwarps = n_cta * kVWarps;
-    const int items = sh.nA * a.T;
-    for (int item = warp; item < items; item += nwarps) {
-        const int i = item / a.T, t = item - i * a.T;
-        const int row = sh.A[i];
-        const float *rp = a.zp + (int64_t)row * a.stride;
-        const float *rq = a.zq + (int64_t)row * a.stride;
-        const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
-        const RowOff ro = row_off(sh, i);
-        float acc = 0.f;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            float4 vp[4], vq[4];
-            load_half_tile(rp, t * kTile + half * (kTile / 2), a.V, al, lane, vp);
-            load_half_tile(rq, t * kTile + half * (kTile / 2), a.V, al, lane, vq);
-#pragma unroll
-            for (int it = 0; it < 4; ++it) {
-                acc += cell_mass(vp[it].x, vq[it].x, a.k2, ro, s);
-                acc += cell_mass(vp[it].y, vq[it].y, a.k2, ro, s);
-                acc += cell_mass(vp[it].z, vq[it].z, a.k2, ro, s);
-                acc += cell_mass(vp[it].w, vq[it].w, a.k2, ro, s);
-            }
-        }
-        const double tot = warp_sum((double)acc);
-        if (lane == 0) sums[item] = tot;
-    }
-}
-
-// Ordered sum of n doubles by one warp: lane-strided partial sums, then a butterfly.  The
-// order depends on n only, never on the launch shape.
-__device__ double ordered_sum(const double *v, int n, int lane) {
-    double acc = 0.0;
-    for (int i = lane; i < n; i += 32) acc += __ldcg(v + i);
-    return warp_sum(acc);
 }
 
 // Inverse-CDF search over tile masses (canonical order).  mass(i) must be the same on every
@@ -572,6 +533,61 @@ __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigne
     unsigned long long d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+
+// Items of a pass over n_tiles tiles by n_warps warps: 1, whole tiles; 2, half tiles, where whole ones would leave a part
+// of the last round's warps idle (a warp's own work is the pass's length: V = 32000, 16 CTAs, 3 rows: 4.5 us instead of 7).
+__device__ __forceinline__ int item_halves(int n_tiles, int n_warps) {
+    return (2 * n_tiles + n_warps - 1) / n_warps < 2 * ((n_tiles + n_warps - 1) / n_warps) ? 2 : 1;
+}
+
+// One cluster-wide pass: item sums of max(p_beam - s q_beam, 0) over the live rows.  Returns the sum of this warp's items
+// in units of 2^-60 (whole numbers, so that the total does not depend on the launch shape).
+// A function of its own: its three callers would each carry its unrolled loop.
+constexpr double kSumUnit = 1152921504606846976.0;               // 2^60
+__device__ __noinline__ long long residual_pass(const float *__restrict__ zp, const float *__restrict__ zq, int64_t stride,
+                                                int V, int T, float k2, const Shared &sh, double s, double *sums,
+                                                int warp, int nwarps, int halves) {
+    const int lane = threadIdx.x & 31;
+    const int row_items = T * halves, items = sh.nA * row_items;
+    // (s in two floats: one alone would be off by up to 2^-24 of s q_beam)
+    const float s_hi = (float)s, s_lo = (float)(s - (double)s_hi);
+    const unsigned long long k22 = pack2(k2, k2), hi2 = pack2(-s_hi, -s_hi), lo2 = pack2(-s_lo, -s_lo);
+    long long total = 0;
+    for (int item = warp; item < items; item += nwarps) {
+        const int i = item / row_items, t = item - i * row_items;
+        const int row = sh.A[i];
+        const float *rp = zp + (int64_t)row * stride;
+        const float *rq = zq + (int64_t)row * stride;
+        const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
+        const unsigned long long bp2 = pack2(sh.bp[i], sh.bp[i]), bq2 = pack2(sh.bq[i], sh.bq[i]);
+        const unsigned long long cp2 = pack2(sh.cp[i], sh.cp[i]), cq2 = pack2(sh.cq[i], sh.cq[i]);
+        double acc = 0.0;
+        int e0 = t * (kTile / halves);
+#pragma unroll 1
+        for (int half = halves; half < 3; ++half, e0 += kTile / 2) {
+            float4 vp[4], vq[4];
+            load_half_tile(rp, e0, V, al, lane, vp);
+            load_half_tile(rq, e0, V, al, lane, vq);
+            float sum = 0.f;
+#pragma unroll
+            for (int it = 0; it < 4; ++it)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 pe = unpack2(fma2(h ? pack2(vp[it].z, vp[it].w) : pack2(vp[it].x, vp[it].y), k22, bp2));
+                    const float2 qe = unpack2(fma2(h ? pack2(vq[it].z, vq[it].w) : pack2(vq[it].x, vq[it].y), k22, bq2));
+                    const unsigned long long p2 = mul2(pack2(exp2f(pe.x), exp2f(pe.y)), cp2);
+                    const unsigned long long q2 = mul2(pack2(exp2f(qe.x), exp2f(qe.y)), cq2);
+                    const float2 d = unpack2(fma2(lo2, q2, fma2(hi2, q2, p2)));
+                    sum += fmaxf(d.x, 0.f) + fmaxf(d.y, 0.f);
+                }
+            acc += (double)sum;
+        }
+        const double tot = warp_sum(acc);
+        if (lane == 0) sums[item] = tot;
+        total += __double2ll_rn(tot * kSumUnit);
+    }
+    return total;
 }
 
 // The cells of one half tile (4 x float4 per lane and model) into the histogram; adds p - q and q of its cells with
@@ -1186,6 +1202,9 @@ __device__ void finish_supports(WarpScratch &ws, bool have_q, int lane) {
 #define TS(slot) do {} while (0)
 #endif
 
+// Drafts behind the first rejection of a layer of known width up to which its residual masses are computed on demand.
+constexpr int kOnDemandLeft = 3;
+
 // dynamic shared memory of k_verify: the histogram of a layer as four 32-bit arrays while it is
 // being built, then (over the same bytes) this CTA's slice of the suffix sums of its p and q mass
 constexpr size_t kVerifyDynSmem = kHistArrays * sizeof(uint32_t) * kHistWords;
@@ -1218,7 +1237,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     if (bad_widths) { W_min = W_max = W_nom = 1; }
     double *sums_base = a.tile_sums + (int64_t)r * 2 * (a.max_m + 1) * ((int64_t)a.max_live * a.T);
     const int64_t slot_stride = (int64_t)a.max_live * a.T;
-    int n_out = 0;
+    int n_out = 0, n_pass = 0, n_hist = 0;
 #ifdef DSBD_PHASE_TIMING
     int ts_n = 0;
 #endif
@@ -1418,6 +1437,10 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
 
+    // Warped layers have no step in which the cluster works together, and only rank 0 writes: the others would
+    // build the same supports beside it.  (Nobody stores into their shared memory any more.)
+    if (a.top_k > 0 && !writer) return;
+
     // ---- set-up ----
     auto is_root = [&](int i) { return cached ? nc.parent[i] == -1 : a.parent[n_lo + i] < 0; };
     if (warp == 0) {
@@ -1550,6 +1573,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 sh.s_arr[0] = 0.0;
                 sh.c_arr[1] = 1.0;
                 sh.chain_len = 0;          // c_{j+1} is known for j = 1..chain_len
+                sh.next_i = sh.count = 0;
+                sh.run_j = 1;
                 sh.bank = l & 1;
             }
         } else if (warp <= 2) {
@@ -1560,8 +1585,62 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         }
         __syncthreads();
         const int m = sh.m;
-        bool looked_up = false;
+        bool looked_up = false, on_demand = false;
         TS(3);
+
+        // The accept loop (lane 0 of warp 0), from draft sh.next_i on.  on_demand: ends with sh.need_exact = 1 after a
+        // rejection whose residual mass c_{j+1} is not known yet.
+        auto accept_loop = [&](int W, bool on_demand) {
+            int i = sh.next_i, count = sh.count, j = sh.run_j, tests = 0, near = 0, need = 0;
+            for (; i < m && count < W && !need; ++i) {
+                const int n = sh.S[i];
+                const double rho = sh.rho[i];
+                double ratio;
+                if (j == 1) ratio = rho;
+                else ratio = fmax(rho - sh.s_arr[j - 1], 0.0) / sh.c_arr[j];
+                if (ratio > 1.0) ratio = 1.0;
+                const double u = sh.uu[i];
+                ++tests;
+                near += fabs(u - ratio) < 1e-5;
+                if (u <= ratio) {
+                    st[n - n_lo] = DSBD_NODE_ACCEPTED;
+                    if (writer) a.out.node_status[n] = DSBD_NODE_ACCEPTED;
+                    sh.acc[count++] = n;
+                    j = 1;
+                } else {
+                    st[n - n_lo] = DSBD_NODE_REJECTED;
+                    if (writer) a.out.node_status[n] = DSBD_NODE_REJECTED;
+                    // an empty residual means p' == q_beam: the rejected draft lay outside the
+                    // support of q_beam, there is nothing to subtract and p' stays
+                    if (on_demand && j > sh.chain_len) { sh.s_arr[j] = sh.s_arr[j - 1] + sh.c_arr[j]; need = 1; }
+                    else if (j <= sh.chain_len && sh.c_arr[j + 1] > 0.0) ++j;
+                }
+            }
+            sh.next_i = i;
+            sh.count = count;
+            sh.run_j = j;
+            sh.n_tests += tests;
+            sh.n_near += near;
+            sh.need_exact = need;
+        };
+        // F(s) by a pass of the whole cluster over the live rows, whose item sums go to `sums`
+        auto exact_pass = [&](double s, double *sums, int halves) {
+            const long long mine = residual_pass(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s, sums,
+                                                 cta_rank * kVWarps + warp, n_cta * kVWarps, halves);
+            if (lane == 0) sh.warp_part[warp] = mine;
+            __syncthreads();
+            if (warp == 0) {
+                long long v = lane < kVWarps ? sh.warp_part[lane] : 0ll;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+                if (lane < n_cta) cluster.map_shared_rank(&sh, lane)->part[n_pass & 1][cta_rank] = v;
+            }
+            cluster.sync();                            // (two buffers: who is here has read those of the pass before)
+            long long v = 0ll;
+            for (int c = 0; c < n_cta; ++c) v += sh.part[n_pass & 1][c];
+            ++n_pass;
+            return (double)v * (1.0 / kSumUnit);
+        };
 
         const bool warped = a.top_k > 0;
         WarpScratch &wsup = *reinterpret_cast<WarpScratch *>(hq);       // the histogram arrays are idle when warped
@@ -1607,15 +1686,52 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 }
             }
             __syncthreads();
-        } else if (m >= 1 && !sh.err) {
+        } else if (m >= 1 && !sh.err && !a.select_mode && (m <= W_min || W_max <= W_min)) {
+            // ---- the width is W_min whatever the residual masses are (W~ <= m): the drafts are tested at once.  Up to
+            // the first rejection that takes no pass over the rows at all, and every rejection one pass, without a histogram,
+            // whose sums also serve the completion draw.  With more than kOnDemandLeft drafts behind the first
+            // rejection the histogram is the better way: one pass of it costs two to three of these.  (Two live rows of
+            // 128256, 4 CTAs: a layer of accepted drafts 5 us instead of 38; a rejection 16 instead of 37.  64 requests x
+            // 8 rows 986 -> 922 us for the call, 16 ragged requests 222 -> 174, one request of V = 32000 60 -> 52.) ----
+            if (warp == 0) {
+                draft_tests(l, m);
+                const int W = W_min < W_max ? W_min : W_max;
+                int first = m;                         // the first rejection
+                for (int base = 0; base < m && first == m; base += 32) {
+                    const int i = base + lane;
+                    const unsigned rejects = __ballot_sync(kFull, i < m && sh.uu[i] > fmin(sh.rho[i], 1.0));
+                    if (rejects) first = base + __ffs(rejects) - 1;
+                }
+                if (lane == 0) {
+                    sh.on_demand = first >= W || m - 1 - first <= kOnDemandLeft;
+                    sh.need_exact = 0;
+                    if (sh.on_demand) accept_loop(W, true);
+                }
+            }
+            __syncthreads();
+            on_demand = sh.on_demand;
+            while (on_demand && sh.need_exact) {
+                const int j = sh.run_j;
+                const int halves = j == 1 ? item_halves(sh.nA * a.T, n_cta * kVWarps) : 1;   // (slot 0 has room for half tiles)
+                const double c_next = exact_pass(sh.s_arr[j], sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride, halves);
+                if (threadIdx.x == 0) {
+                    if (j == 1) sh.halves = halves;
+                    sh.c_arr[j + 1] = c_next;
+                    sh.chain_len = j;
+                    if (c_next > 0.0) sh.run_j = j + 1;
+                    accept_loop(W_min < W_max ? W_min : W_max, true);
+                }
+                __syncthreads();
+            }
+        }
+        if (m >= 1 && !sh.err && !warped && !on_demand) {
             // ---- one pass: ratio histogram of the layer over the live rows ----
             const double top = log2((double)(m > 2 ? m : 2));          // s_j <= j <= m
             const float binscale = (float)((double)kBins / top);
-            unsigned long long *tot = sh.w_tot[sh.bank];
-            // half tiles as items where whole ones would leave a part of the last round's warps idle: a warp's own
-            // work is the pass's length there (V = 32000, 16 CTAs: 3 rows 4.5 us instead of 7)
-            const int tiles = sh.nA * a.T, nw = n_cta * kVWarps;
-            const int halves = (2 * tiles + nw - 1) / nw < 2 * ((tiles + nw - 1) / nw) ? 2 : 1;
+            // (counted by histograms, not by layers: the other bank is cleared between the barriers of this one)
+            const int bank = n_hist++ & 1;
+            unsigned long long *tot = sh.w_tot[bank];
+            const int halves = item_halves(sh.nA * a.T, n_cta * kVWarps);
             histogram_pass(a, sh, binscale, hs, sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride, cta_rank,
                            n_cta, halves, tot);
             __syncthreads();
@@ -1623,7 +1739,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             TS(4);
             cluster.sync();                            // every CTA's histogram is complete
             TS(6);
-            if (threadIdx.x < 10) sh.w_tot[sh.bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
+            if (threadIdx.x < 10) sh.w_tot[bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
                                                        // the barrier below
             hist_merge(cluster, hs, sh, cta_rank, n_cta);
             TS(7);
@@ -1722,13 +1838,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 // (at j = 1 these are the sums that the histogram pass left in slot 0)
                 double *sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride;
                 if (j == 1 && threadIdx.x == 0) sh.halves = 1;
-                residual_pass(a, sh, (float)sh.s_arr[j], sums, cta_rank, n_cta);
-                __threadfence();
-                cluster.sync();
-                if (warp == 0) {
-                    const double c_next = ordered_sum(sums, sh.nA * a.T, lane);
-                    if (lane == 0) sh.c_arr[j + 1] = c_next;
-                }
+                const double c_next = exact_pass(sh.s_arr[j], sums, 1);
+                if (threadIdx.x == 0) sh.c_arr[j + 1] = c_next;
                 __syncthreads();
                 if (!(sh.c_arr[j + 1] > 0.0)) break;
                 j0 = j + 1;
@@ -1741,20 +1852,22 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         TS(8);
         // ---- width and accept loop (warp 0) ----
         if (warp == 0 && !sh.err) {
-            // alpha_j = 1 - c_{j+1}/c_j; once a residual has no mass every later alpha is 1
-            for (int j = 1 + lane; j <= m; j += 32) {
-                double al = 1.0;
-                if (j <= sh.chain_len && sh.c_arr[j] > 0.0 && sh.c_arr[j + 1] > 0.0)
-                    al = fmin(fmax(1.0 - sh.c_arr[j + 1] / sh.c_arr[j], 0.0), 1.0);
-                sh.alpha[j] = al;
+            int W = W_min < W_max ? W_min : W_max;
+            if (!on_demand) {
+                // alpha_j = 1 - c_{j+1}/c_j; once a residual has no mass every later alpha is 1
+                for (int j = 1 + lane; j <= m; j += 32) {
+                    double al = 1.0;
+                    if (j <= sh.chain_len && sh.c_arr[j] > 0.0 && sh.c_arr[j + 1] > 0.0)
+                        al = fmin(fmax(1.0 - sh.c_arr[j + 1] / sh.c_arr[j], 0.0), 1.0);
+                    sh.alpha[j] = al;
+                }
+                __syncwarp();
+                // (the verification only needs W~ up to W_max and can stop at the first tail below the
+                // threshold; dsbd_select_width returns the whole tail)
+                const int wt = width_rule(sh, m, a.thresh, lane, a.select_mode ? -1 : W_max);
+                W = wt > W_min ? wt : W_min;
+                if (W > W_max) W = W_max;
             }
-            if (lane == 0) sh.res_j = 0;
-            __syncwarp();
-            // (the verification only needs W~ up to W_max and can stop at the first tail below the
-            // threshold; dsbd_select_width returns the whole tail)
-            const int wt = width_rule(sh, m, a.thresh, lane, a.select_mode ? -1 : W_max);
-            int W = wt > W_min ? wt : W_min;
-            if (W > W_max) W = W_max;
             if (a.select_mode) {
                 if (writer && lane == 0) {
                     a.width_out[r] = W;
@@ -1768,44 +1881,18 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 if (lane == 0) sh.done = 1;
             } else if (lane == 0) {
                 if (writer) a.out.layer_width[(int64_t)r * (a.gamma + 1) + (l - 1)] = W;
-                int count = 0, j = 1, err = 0, tests = 0, near = 0;
-                for (int i = 0; i < m && count < W; ++i) {
-                    const int n = sh.S[i];
-                    const double rho = sh.rho[i];
-                    double ratio;
-                    if (j == 1) ratio = rho;
-                    else ratio = fmax(rho - sh.s_arr[j - 1], 0.0) / sh.c_arr[j];
-                    if (ratio > 1.0) ratio = 1.0;
-                    const double u = sh.uu[i];
-                    ++tests;
-                    near += fabs(u - ratio) < 1e-5;
-                    if (u <= ratio) {
-                        st[n - n_lo] = DSBD_NODE_ACCEPTED;
-                        if (writer) a.out.node_status[n] = DSBD_NODE_ACCEPTED;
-                        sh.acc[count++] = n;
-                        j = 1;
-                    } else {
-                        st[n - n_lo] = DSBD_NODE_REJECTED;
-                        if (writer) a.out.node_status[n] = DSBD_NODE_REJECTED;
-                        // an empty residual means p' == q_beam: the rejected draft lay outside the
-                        // support of q_beam, there is nothing to subtract and p' stays
-                        if (j <= sh.chain_len && sh.c_arr[j + 1] > 0.0) ++j;
-                    }
-                }
+                if (!on_demand) accept_loop(W, false);
+                const int count = sh.count, j = sh.run_j;
                 for (int i = 0; i < m; ++i)
                     if (st[sh.S[i] - n_lo] == DSBD_NODE_UNREACHED) {
                         st[sh.S[i] - n_lo] = DSBD_NODE_CUT;
                         if (writer) a.out.node_status[sh.S[i]] = DSBD_NODE_CUT;
                     }
                 sh.W = W;
-                sh.count = count;
-                sh.n_tests += tests;
-                sh.n_near += near;
                 sh.n_rows += sh.nA;
                 ++sh.n_layers;
-                sh.res_j = (count < W && j > 1) ? j : 0;   // residual draw at run position j needs tile sums
-                sh.run_j = j;
-                if (err) sh.err = err;
+                // a residual draw at run position j needs tile sums (a layer of known width has them)
+                sh.res_j = (count < W && j > 1 && !on_demand) ? j : 0;
             }
         }
         __syncthreads();
@@ -1813,12 +1900,13 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         if (looked_up) cluster.barrier_wait();         // the others have done with this CTA's slice
         TS(9);
         // ---- a residual draw locates its tile through tile sums of max(p_beam - s_{j-1} q_beam, 0) ----
-        double *res_sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride;   // slot 0 of the bank
+        // slot 0 of the bank; in a layer of known width that of the rejection before the draw
+        const int res_slot = on_demand && sh.run_j > 2 ? sh.run_j - 1 : 0;
+        double *res_sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1) + res_slot) * slot_stride;
         if (!a.select_mode && !sh.err && !warped && sh.res_j > 2) {   // run position 2 is served by the histogram pass
-            if (threadIdx.x == 0) { ++sh.n_respass; sh.halves = 1; }
-            residual_pass(a, sh, (float)sh.s_arr[sh.res_j - 1], res_sums, cta_rank, n_cta);
-            __threadfence();
-            cluster.sync();
+            const int halves = item_halves(sh.nA * a.T, n_cta * kVWarps);
+            if (threadIdx.x == 0) { ++sh.n_respass; sh.halves = halves; }
+            exact_pass(sh.s_arr[sh.res_j - 1], res_sums, halves);
         }
 
         TS(10);
@@ -1888,7 +1976,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             if (lane == 0 && err) sh.err = err;
         }
         __syncthreads();
-        if (!a.select_mode && sh.done && sh.n_fill > 0 && !sh.err) {
+        if (writer && !a.select_mode && sh.done && sh.n_fill > 0 && !sh.err) {
             // draw f is output beam n_out + f: the residual draw at the run position where the layer ended, then the
             // fills from p_beam, each with its own uniform
             const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
@@ -1899,9 +1987,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, f ? 2u : 1u, f ? (uint32_t)(f - 1) : 0u);
                 const bool use_res = f == 0 && j > 1;
                 int ia = 0;
-                const int tok = draw_cell(a, sh, u, use_res, use_res ? (float)sh.s_arr[j - 1] : 0.f, res_sums, sh.halves, lane, &ia);
+                const int tok = draw_cell(a, sh, u, use_res, use_res ? (float)sh.s_arr[j - 1] : 0.f, res_sums, res_slot ? 1 : sh.halves, lane, &ia);
                 if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
-                else if (lane == 0 && writer)
+                else if (lane == 0)
                     emit_at(a, r, base + f, sh.A[ia], -1, tok, f ? DSBD_SRC_FILL : DSBD_SRC_RESIDUAL, cached ? &nc : nullptr, n_lo);
             }
             __syncthreads();
@@ -1916,7 +2004,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
 
     TS(11);
     // ---- every layer passed: W_nom beams from p_beam^(gamma+1) ----
-    const bool extra = !a.select_mode && !sh.done && !sh.err;
+    const bool extra = writer && !a.select_mode && !sh.done && !sh.err;
     WarpScratch &wsx = *reinterpret_cast<WarpScratch *>(hq);
     int extra_err = 0;
     if (extra) {
@@ -1931,14 +2019,14 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         // W_nom independent draws from p_beam, one warp each
         const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
         const int n_draw = min(W_nom, max(cap - n_out, 0));
-        if (writer && threadIdx.x == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
+        if (threadIdx.x == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
         for (int kk = warp; kk < n_draw; kk += kVWarps) {
             const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1), 3u,
                                               (uint32_t)kk);
             int ia = 0;
             const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, 1, lane, &ia);
             if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
-            else if (lane == 0 && writer)
+            else if (lane == 0)
                 emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
         }
         __syncthreads();
@@ -1949,7 +2037,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     } else if (extra && warp == 0) {
         // independent draws from the support, one lane each
         int err = extra_err;
-        if (writer && lane == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
+        if (lane == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
         const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
         const int n_draw = err ? 0 : min(W_nom, max(cap - n_out, 0));
         for (int k0 = 0; k0 < n_draw; k0 += 32) {
@@ -1960,8 +2048,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             if (kk >= n_draw) continue;
             if (pick < 0) { err = DSBD_DEV_EXHAUSTED; continue; }
             const int ia = wsx.cell[0][pick] / a.V, tok = wsx.cell[0][pick] - ia * a.V;
-            if (writer)
-                emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
+            emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
         }
         if (!extra_err) {
             if (__any_sync(kFull, err)) err = DSBD_DEV_EXHAUSTED;

@@ -80,8 +80,9 @@ def test_c5_all_requests(top_k, top_p):
 
 def _random_problem(rng, R, V, gamma, max_w, stride_pad=0, ninf_frac=0.0, tree="chain", min_w=1):
     widths = rng.integers(1, max_w + 1, size=R)
-    spec = dict(R=R, W=(min_w, max_w), tree=inputs._chain(gamma) if tree == "chain" else inputs._binary(gamma),
-                prefix=(1, 1))
+    if isinstance(tree, str):
+        tree = inputs._chain(gamma) if tree == "chain" else inputs._binary(gamma)
+    spec = dict(R=R, W=(min_w, max_w), tree=tree, prefix=(1, 1))
     forest, widths, _ = inputs.build_forest(spec, rng)
     N, B = forest["N"], forest["B"]
     stride = V + stride_pad
@@ -323,6 +324,51 @@ def test_requests_around_the_node_cache_and_half_tiles(beams, gamma, V):
         exempt += e
         decisions += d
     check_exempt(exempt, decisions)
+
+
+@pytest.mark.parametrize("V,beams,W_min,W_max", [(1, 3, 3, 3), (1000, 2, 2, 8), (1025, 5, 8, 8), (4097, 6, 4, 4),
+                                                 (9000, 40, 3, 3), (33000, 4, 4, 9), (50257, 3, 3, 3)])
+def test_layers_of_known_width(V, beams, W_min, W_max):
+    """Layers whose width does not depend on the residual masses (at most W_min drafts, or W_min = W_max): no rejection,
+    a rejection with none, three, four and many drafts behind it (passes on demand up to three, the histogram from
+    four on), several rejections in a row, accepts between them; clusters of 1 to 16 CTAs, whole and half tiles, vocabularies of
+    one token, one more than a tile and rows that are not aligned."""
+    rng = np.random.default_rng(V + beams)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=4, V=V, gamma=3, max_w=beams, min_w=beams)
+    zp = (zp + rng.normal(0, 1.0, zp.shape)).astype(np.float32)
+    prm.update(W_min_r=None, W_min=W_min, W_max=W_max)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = 0
+    for step in range(12):
+        prm["step"] = step
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+    check_exempt(exempt, decisions)
+
+
+@pytest.mark.parametrize("V", [2000, 40000])
+def test_histograms_with_a_layer_of_known_width_between(V):
+    """A layer with a histogram, one that needs none, another with one: drafts that widen again behind a chain."""
+    rng = np.random.default_rng(V)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=4, V=V, gamma=4, max_w=5, min_w=5,
+                                                     tree=[-1, 0, 1, 2, 2, 2, 3, 4, 4, 5, 5, 5])
+    zq = (zp + rng.normal(0, 0.4, zp.shape)).astype(np.float32)      # most drafts are accepted
+    prm.update(W_min_r=None, W_min=2)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = deep = 0
+    for step in range(16):
+        prm.update(step=step, thresh=0.7 + 0.015 * step)
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+        deep += int((gpu["l_last"] >= 3).sum())
+    check_exempt(exempt, decisions)
+    assert deep > 0
 
 
 @pytest.mark.parametrize("V", [1000, 2000, 4000, 8000, 32000])

@@ -303,7 +303,7 @@ PHASE_NAMES = {1: "start", 2: "prologue / previous layer's completion", 3: "laye
                5: "wait for the cluster's slices", 6: "wait for the cluster's passes",
                7: "merge and suffix sums of a slice", 8: "residual chain",
                9: "width and accept loop", 10: "residual pass for a completion draw", 11: "completion draws",
-               12: "extra layer and final writes"}
+               12: "extra layer and final writes", 13: "wait for the dense pass", 14: "log-sum-exps"}
 
 
 def run_verify_phases(args):

@@ -250,6 +250,8 @@ struct Shared {
     int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows consulted
     unsigned long long wtot_p[kVWarps], wtot_q[kVWarps];
     unsigned long long slice_p[16], slice_q[16];   // mass of the bins of every CTA's slice
+    unsigned long long above_p[16], above_q[16];   // mass of the bins above every CTA's slice
+    double bin_log2, bin_width, bin_inv_width;     // of a bin: log2 of its upper over its lower edge; see the chain
     unsigned long long w_tot[2][10];        // per bank, sums of one histogram pass: see histogram_pass / hist_fold_over
     int n_wrapped;                          // layers where a w word of the histogram wrapped
     double rho[kMaxLive], uu[kMaxLive];     // per live draft: p_beam/q_beam and its uniform
@@ -1763,6 +1765,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             if (threadIdx.x < 10) sh.w_tot[bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
                                                        // the barrier below
             hist_merge(cluster, hs, n_bins, sh, cta_rank, n_cta);
+            if (threadIdx.x == kVThreads - 32) {
+                // bin k is [e_k, e_k+1], e_k = 2^(k bin_log2); its width over e_k, with both edges 2e-6 wider
+                const double step = top / (double)n_bins, w = exp2(step) * (1.0 + 2e-6) - (1.0 - 2e-6);
+                sh.bin_log2 = step; sh.bin_width = w; sh.bin_inv_width = 1.0 / w;
+            }
             TS(7);
             cluster.sync();                            // every slice of the suffix sums is complete
             TS(5);
@@ -1789,20 +1796,21 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
                 if (lane == 0 && wrapped) ++sh.n_wrapped;
             }
-            // suffix sums of bins k and k + 1 (warp 0): one word of each kind from the CTAs that have them
-            auto suffix2 = [&](int k, unsigned long long (&P)[2], unsigned long long (&Q)[2]) {
-                const int at = min(k + (lane & 1), n_bins), c = min(at / slice, n_cta - 1);
-                unsigned long long sp = tot[7], sq = tot[8];
-                const unsigned long long up = __shfl_sync(kFull, above_p, c), uq = __shfl_sync(kFull, above_q, c);
-                if (lane < 2 && at < n_bins) {
-                    const uint32_t lp = cluster.map_shared_rank(hs.wp, c)[at], hi_p = cluster.map_shared_rank(hs.bp, c)[at];
-                    const uint32_t lq = cluster.map_shared_rank(hs.wq, c)[at], hi_q = cluster.map_shared_rank(hs.bq, c)[at];
-                    sp = (((unsigned long long)hi_p << 32) | lp) + up;
-                    sq = (((unsigned long long)hi_q << 32) | lq) + uq;
-                }
-#pragma unroll
-                for (int i = 0; i < 2; ++i) { P[i] = __shfl_sync(kFull, sp, i); Q[i] = __shfl_sync(kFull, sq, i); }
+            if (warp == 0) {
+                if (lane < n_cta) { sh.above_p[lane] = above_p; sh.above_q[lane] = above_q; }
+                __syncwarp();
+            }
+            // suffix sums of bin k (warp 0; the same on every lane): one word of each kind from the CTA that has it
+            const int shift = 31 - __clz(slice);
+            auto suffix = [&](int k, unsigned long long &P, unsigned long long &Q) {
+                if (k >= n_bins) { P = tot[7]; Q = tot[8]; return; }
+                const int c = k >> shift;
+                const uint32_t lp = cluster.map_shared_rank(hs.wp, c)[k], hi_p = cluster.map_shared_rank(hs.bp, c)[k];
+                const uint32_t lq = cluster.map_shared_rank(hs.wq, c)[k], hi_q = cluster.map_shared_rank(hs.bq, c)[k];
+                P = (((unsigned long long)hi_p << 32) | lp) + sh.above_p[c];
+                Q = (((unsigned long long)hi_q << 32) | lq) + sh.above_q[c];
             };
+            const double bin_log2 = sh.bin_log2, width = sh.bin_width, inv_width = sh.bin_inv_width;
 
             int j0 = 1;
             while (j0 <= m) {
@@ -1824,19 +1832,22 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                             c_next = ((double)P[0] - (double)Q[0]) * kUnfix;
                             if (fix_err > kErrTol) { need = 1; break; }
                         } else {
-                            // (a float's logarithm can miss the bin only within 3e-7 of an edge; the bracket below
-                            // takes the edges 2e-6 wider)
-                            int k = (int)(log2f((float)s_j) * binscale);
+                            // (the approximate logarithm and exponential miss the bin and its edges by at most 8e-7; the
+                            // bracket below takes the edges 2e-6 wider)
+                            int k = (int)(__log2f((float)s_j) * binscale);
                             if (k < 0) k = 0;
                             if (k >= n_bins) { need = 1; break; }     // cannot happen for s_j <= m
-                            suffix2(k, P, Q);
+                            suffix(k, P[0], Q[0]);
+                            suffix(k + 1, P[1], Q[1]);
                             const double Pa = (double)P[1] * kUnfix, Qa = (double)Q[1] * kUnfix;
                             const double Pk = (double)(P[0] - P[1]) * kUnfix;
                             const double Qk = (double)(Q[0] - Q[1]) * kUnfix;
-                            const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
-                            const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
+                            const float e_log2 = (float)((double)k * bin_log2);
+                            const double e_k = (double)ex2_approx(e_log2), inv_e = (double)ex2_approx(-e_log2);
+                            const double r_lo = e_k * (1.0 - 2e-6);
                             const double lo_b = fmax(Pk - s_j * Qk, 0.0);
-                            double q_hi = (Pk - r_lo * Qk) / (r_hi - r_lo);
+                            double q_hi = (Pk - r_lo * Qk) * (inv_e * inv_width);        // / (r_hi - r_lo)
+                            const double r_hi = r_lo + e_k * width;
                             q_hi = fmin(fmax(q_hi, 0.0), Qk);
                             const double hi_b = fmax(q_hi * (r_hi - s_j), lo_b);
                             // the midpoint of the bracket is used: half its width plus the fixed-point term

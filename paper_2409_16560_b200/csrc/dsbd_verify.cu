@@ -556,6 +556,9 @@ __device__ __forceinline__ int item_halves(int n_tiles, int n_warps) {
 
 // One cluster-wide pass: item sums of max(p_beam - s q_beam, 0) over the live rows.  Returns the sum of this warp's items
 // in units of 2^-60 (whole numbers, so that the total does not depend on the launch shape).
+// Bound by latency: few clusters make such a pass at a time, a warp takes about 1.4 us a half tile.  The hardware's exponential
+// (results below 2^-126 are zero, as in the histogram) and straight-line loads for whole aligned halves: two rows of 128256
+// by 4 CTAs 17.3 -> 16.3 us, eight 62 -> 55.  (The next item prefetched into L2: no difference.)
 // A function of its own: its three callers would each carry its unrolled loop.
 constexpr double kSumUnit = 1152921504606846976.0;               // 2^60
 __device__ __noinline__ long long residual_pass(const float *__restrict__ zp, const float *__restrict__ zq, int64_t stride,
@@ -580,8 +583,15 @@ __device__ __noinline__ long long residual_pass(const float *__restrict__ zp, co
 #pragma unroll 1
         for (int half = halves; half < 3; ++half, e0 += kTile / 2) {
             float4 vp[4], vq[4];
-            load_half_tile(rp, e0, V, al, lane, vp);
-            load_half_tile(rq, e0, V, al, lane, vq);
+            if (al && e0 + kTile / 2 <= V) {
+#pragma unroll
+                for (int it = 0; it < 4; ++it) vp[it] = ldg_stream(reinterpret_cast<const float4 *>(rp + e0 + it * 128) + lane);
+#pragma unroll
+                for (int it = 0; it < 4; ++it) vq[it] = ldg_stream(reinterpret_cast<const float4 *>(rq + e0 + it * 128) + lane);
+            } else {
+                load_half_tile(rp, e0, V, false, lane, vp);
+                load_half_tile(rq, e0, V, false, lane, vq);
+            }
             float sum = 0.f;
 #pragma unroll
             for (int it = 0; it < 4; ++it)
@@ -589,8 +599,8 @@ __device__ __noinline__ long long residual_pass(const float *__restrict__ zp, co
                 for (int h = 0; h < 2; ++h) {
                     const float2 pe = unpack2(fma2(h ? pack2(vp[it].z, vp[it].w) : pack2(vp[it].x, vp[it].y), k22, bp2));
                     const float2 qe = unpack2(fma2(h ? pack2(vq[it].z, vq[it].w) : pack2(vq[it].x, vq[it].y), k22, bq2));
-                    const unsigned long long p2 = mul2(pack2(exp2f(pe.x), exp2f(pe.y)), cp2);
-                    const unsigned long long q2 = mul2(pack2(exp2f(qe.x), exp2f(qe.y)), cq2);
+                    const unsigned long long p2 = mul2(pack2(ex2_approx(pe.x), ex2_approx(pe.y)), cp2);
+                    const unsigned long long q2 = mul2(pack2(ex2_approx(qe.x), ex2_approx(qe.y)), cq2);
                     const float2 d = unpack2(fma2(lo2, q2, fma2(hi2, q2, p2)));
                     sum += fmaxf(d.x, 0.f) + fmaxf(d.y, 0.f);
                 }

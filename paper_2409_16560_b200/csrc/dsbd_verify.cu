@@ -14,7 +14,8 @@
 //                  fixed-point histogram of the cells' ratios p_beam/q_beam, from which all the
 //                  residual masses c_{j+1} = F(s_j) of the layer follow without touching the
 //                  rows again; the acceptance-count recursion; the accept loop; the
-//                  inverse-CDF completion draws.
+//                  inverse-CDF completion draws.  A layer whose width does not depend on the residual
+//                  masses tests its drafts at once and makes a plain pass for each rejection.
 //
 // The residual chain uses the closed form of the paper's recursion p_{k+1} = norm(max(p_k -
 // q_beam, 0)):  with F(s) = sum max(p_beam - s q_beam, 0), c_1 = 1, s_0 = 0, s_j = s_{j-1} + c_j
@@ -556,9 +557,9 @@ __device__ __forceinline__ int item_halves(int n_tiles, int n_warps) {
 
 // One cluster-wide pass: item sums of max(p_beam - s q_beam, 0) over the live rows.  Returns the sum of this warp's items
 // in units of 2^-60 (whole numbers, so that the total does not depend on the launch shape).
-// Bound by latency: few clusters make such a pass at a time, a warp takes about 1.4 us a half tile.  The hardware's exponential
+// Bound by latency: few clusters make such a pass at a time, a warp takes about 1.8 us a half tile.  The hardware's exponential
 // (results below 2^-126 are zero, as in the histogram) and straight-line loads for whole aligned halves: two rows of 128256
-// by 4 CTAs 17.3 -> 16.3 us, eight 62 -> 55.  (The next item prefetched into L2: no difference.)
+// by 4 CTAs 17.3 -> 16.3 us, eight 62 -> 57.  (The next item prefetched into L2: no difference.)
 // A function of its own: its three callers would each carry its unrolled loop.
 constexpr double kSumUnit = 1152921504606846976.0;               // 2^60
 __device__ __noinline__ long long residual_pass(const float *__restrict__ zp, const float *__restrict__ zq, int64_t stride,
@@ -1243,6 +1244,9 @@ constexpr int kOnDemandLeft = 3;
 // being built, then (over the same bytes) this CTA's slice of the suffix sums of its p and q mass
 constexpr size_t kVerifyDynSmem = kHistArrays * sizeof(uint32_t) * kHistWords;
 
+// Two instances, with warped joints and without: neither carries the other's code, whose registers it would spill around
+// (64 requests x 8 rows of 128256 with top-k 10: the call 781 -> 772 us).
+template <bool kWarped>
 __global__ void __launch_bounds__(kVThreads, 2)
 k_verify(const __grid_constant__ VerifyArgs a) {
     cg::cluster_group cluster = cg::this_cluster();
@@ -1475,7 +1479,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
 
     // Warped layers have no step in which the cluster works together, and only rank 0 writes: the others would
     // build the same supports beside it.  (Nobody stores into their shared memory any more.)
-    if (a.top_k > 0 && !writer) return;
+    if (kWarped && !writer) return;
 
     // ---- set-up ----
     auto is_root = [&](int i) { return cached ? nc.parent[i] == -1 : a.parent[n_lo + i] < 0; };
@@ -1678,7 +1682,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             return (double)v * (1.0 / kSumUnit);
         };
 
-        const bool warped = a.top_k > 0;
+        constexpr bool warped = kWarped;
         WarpScratch &wsup = *reinterpret_cast<WarpScratch *>(hq);       // the histogram arrays are idle when warped
         if (warped) {
             // ---- supports of T o p_beam and T o q_beam, then the whole chain on <= 64 cells ----
@@ -2056,12 +2060,12 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     if (extra) {
         if (warp < 2) live_weights(a, sh, warp, warp == 0 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
         __syncthreads();
-        if (a.top_k > 0) {
+        if (kWarped) {
             extra_err = build_support<kVThreads>(a, sh, 0, hp, hq);       // one model only: by the whole CTA
             if (!extra_err && warp == 0) finish_supports(wsx, false, lane);
         }
     }
-    if (extra && a.top_k == 0) {
+    if (extra && !kWarped) {
         // W_nom independent draws from p_beam, one warp each
         const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
         const int n_draw = min(W_nom, max(cap - n_out, 0));
@@ -2190,10 +2194,11 @@ int cluster_size_for(int tiles, int R) {
 }
 
 int launch_verify(const VerifyArgs &args, int R, int tiles, cudaStream_t stream) {
+    const auto kernel = args.top_k > 0 ? k_verify<true> : k_verify<false>;
     const int cs = cluster_size_for(tiles, R);
-    if (cs > 8 && cudaFuncSetAttribute(k_verify, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    if (cs > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return DSBD_ERR_CUDA;
-    if (cudaFuncSetAttribute(k_verify, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess)
         return DSBD_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(R * cs));
@@ -2212,7 +2217,7 @@ int launch_verify(const VerifyArgs &args, int R, int tiles, cudaStream_t stream)
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_verify, args) == cudaSuccess ? DSBD_OK : DSBD_ERR_CUDA;
+    return cudaLaunchKernelEx(&cfg, kernel, args) == cudaSuccess ? DSBD_OK : DSBD_ERR_CUDA;
 }
 
 int stats_grid(int64_t items) {

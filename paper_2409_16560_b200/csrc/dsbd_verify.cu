@@ -249,7 +249,9 @@ struct Shared {
     double tail[kMaxLive + 2];
     int bank, halves, need_exact, res_j, run_j, chain_pos;
     int on_demand, next_i;                  // a layer of known width: its passes are made when the accept loop asks
-    long long warp_part[kVWarps], part[2][16];      // sums of an exact pass: of this CTA's warps; of every CTA, two passes in turn
+    // sums of an exact pass, in units of 2^-60, 2^-120 (what the first leaves) and 2^-44 (q): of this CTA's warps; of every
+    // CTA, two passes in turn
+    long long warp_part[3][kVWarps], part[2][3][16];
     int n_out, n_fill;                      // output beams so far; p_beam fills left to the whole CTA
     int n_layers, n_tests, n_exact, n_respass;
     int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows consulted
@@ -264,9 +266,10 @@ struct Shared {
 
 // mass of one cell of the residual max(p_beam - s q_beam, 0); s == 0 gives p_beam
 struct RowOff { float bp, bq, cp, cq, dc; };
-__device__ __forceinline__ float cell_mass(float zp, float zq, float k2, const RowOff &o, float s) {
+__device__ __forceinline__ float cell_mass(float zp, float zq, float k2, const RowOff &o, float s, float *q) {
     const float a = exp2f(fmaf(zp, k2, o.bp)) * o.cp;
     const float b = exp2f(fmaf(zq, k2, o.bq)) * o.cq;
+    *q = b;
     return fmaxf(fmaf(-s, b, a), 0.f);
 }
 // Splits b = log2(weight) - lse*log2(e) (double) into its nearest integer and the factor 2^(rest).
@@ -319,7 +322,8 @@ __device__ __noinline__ int locate_token(const float *__restrict__ rp, const flo
                                          int t, const RowOff ro, float s, double target, int lane) {
     const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
     const int e0 = t * kTile + lane * 32;
-    auto mass = [&](float zp, float zq) { return s > 0.f ? cell_mass(zp, zq, k2, ro, s) : exp2f(fmaf(zp, k2, ro.bp)) * ro.cp; };
+    float q;
+    auto mass = [&](float zp, float zq) { return s > 0.f ? cell_mass(zp, zq, k2, ro, s, &q) : exp2f(fmaf(zp, k2, ro.bp)) * ro.cp; };
     double v = 0.0;
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
@@ -555,65 +559,6 @@ __device__ __forceinline__ int item_halves(int n_tiles, int n_warps) {
     return (2 * n_tiles + n_warps - 1) / n_warps < 2 * ((n_tiles + n_warps - 1) / n_warps) ? 2 : 1;
 }
 
-// One cluster-wide pass: item sums of max(p_beam - s q_beam, 0) over the live rows.  Returns the sum of this warp's items
-// in units of 2^-60 (whole numbers, so that the total does not depend on the launch shape).
-// Bound by latency: few clusters make such a pass at a time, a warp takes about 1.8 us a half tile.  The hardware's exponential
-// (results below 2^-126 are zero, as in the histogram) and straight-line loads for whole aligned halves: two rows of 128256
-// by 4 CTAs 17.3 -> 16.3 us, eight 62 -> 57.  (The next item prefetched into L2: no difference.)
-// A function of its own: its three callers would each carry its unrolled loop.
-constexpr double kSumUnit = 1152921504606846976.0;               // 2^60
-__device__ __noinline__ long long residual_pass(const float *__restrict__ zp, const float *__restrict__ zq, int64_t stride,
-                                                int V, int T, float k2, const Shared &sh, double s, double *sums,
-                                                int warp, int nwarps, int halves) {
-    const int lane = threadIdx.x & 31;
-    const int row_items = T * halves, items = sh.nA * row_items;
-    // (s in two floats: one alone would be off by up to 2^-24 of s q_beam)
-    const float s_hi = (float)s, s_lo = (float)(s - (double)s_hi);
-    const unsigned long long k22 = pack2(k2, k2), hi2 = pack2(-s_hi, -s_hi), lo2 = pack2(-s_lo, -s_lo);
-    long long total = 0;
-    for (int item = warp; item < items; item += nwarps) {
-        const int i = item / row_items, t = item - i * row_items;
-        const int row = sh.A[i];
-        const float *rp = zp + (int64_t)row * stride;
-        const float *rq = zq + (int64_t)row * stride;
-        const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
-        const unsigned long long bp2 = pack2(sh.bp[i], sh.bp[i]), bq2 = pack2(sh.bq[i], sh.bq[i]);
-        const unsigned long long cp2 = pack2(sh.cp[i], sh.cp[i]), cq2 = pack2(sh.cq[i], sh.cq[i]);
-        double acc = 0.0;
-        int e0 = t * (kTile / halves);
-#pragma unroll 1
-        for (int half = halves; half < 3; ++half, e0 += kTile / 2) {
-            float4 vp[4], vq[4];
-            if (al && e0 + kTile / 2 <= V) {
-#pragma unroll
-                for (int it = 0; it < 4; ++it) vp[it] = ldg_stream(reinterpret_cast<const float4 *>(rp + e0 + it * 128) + lane);
-#pragma unroll
-                for (int it = 0; it < 4; ++it) vq[it] = ldg_stream(reinterpret_cast<const float4 *>(rq + e0 + it * 128) + lane);
-            } else {
-                load_half_tile(rp, e0, V, false, lane, vp);
-                load_half_tile(rq, e0, V, false, lane, vq);
-            }
-            float sum = 0.f;
-#pragma unroll
-            for (int it = 0; it < 4; ++it)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float2 pe = unpack2(fma2(h ? pack2(vp[it].z, vp[it].w) : pack2(vp[it].x, vp[it].y), k22, bp2));
-                    const float2 qe = unpack2(fma2(h ? pack2(vq[it].z, vq[it].w) : pack2(vq[it].x, vq[it].y), k22, bq2));
-                    const unsigned long long p2 = mul2(pack2(ex2_approx(pe.x), ex2_approx(pe.y)), cp2);
-                    const unsigned long long q2 = mul2(pack2(ex2_approx(qe.x), ex2_approx(qe.y)), cq2);
-                    const float2 d = unpack2(fma2(lo2, q2, fma2(hi2, q2, p2)));
-                    sum += fmaxf(d.x, 0.f) + fmaxf(d.y, 0.f);
-                }
-            acc += (double)sum;
-        }
-        const double tot = warp_sum(acc);
-        if (lane == 0) sums[item] = tot;
-        total += __double2ll_rn(tot * kSumUnit);
-    }
-    return total;
-}
-
 // The cells of one half tile (4 x float4 per lane and model) into the histogram; adds p - q and q of its cells with
 // p_beam > q_beam, in units of 2^-44, to sd and sq.  (p - q cell by cell: the difference of two sums loses what lies
 // next to a heavy cell, and a completion draw looks for its tile by these sums.)
@@ -630,8 +575,11 @@ __device__ __noinline__ long long residual_pass(const float *__restrict__ zp, co
 // the address of a bin's word is wbase + 4 * (bits of the fma's result); the q array follows the p
 // array at kHistWords words, the b arrays at twice that.
 // (ex2.approx flushes results below 2^-126 to zero; a cell enters the sums from 2^-45 on.)
+// kBinned = false: the sums alone, by the same instructions, so that a draw finds the same tile whether the layer took
+// the histogram or a pass on demand.
 constexpr float kBinMagic = 12582912.f;                         // 1.5 * 2^23
 constexpr float kBigUnits = 268435456.f;                        // 2^28 units = a cell of 2^-16
+template <bool kBinned>
 __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const float4 (&vq)[4], float k2,
                                                const RowOff &o, float binscale, float half_bin, float top, uint32_t wbase,
                                                uint32_t over_bits, float &sd, float &sq) {
@@ -669,11 +617,14 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            asm("{\n\t.reg .pred p;\n\t"
-                "setp.gt.f32 p, %2, %5;\n\t"
-                "@p add.f32 %0, %0, %3;\n\t"
-                "@p add.f32 %1, %1, %4;\n\t}"
-                : "+f"(sd), "+f"(sq) : "f"(dl[c]), "f"(df[c]), "f"(qm[c]), "f"(pass_thr));
+            if (kBinned)
+                asm("{\n\t.reg .pred p;\n\t"
+                    "setp.gt.f32 p, %2, %5;\n\t"
+                    "@p add.f32 %0, %0, %3;\n\t"
+                    "@p add.f32 %1, %1, %4;\n\t}"
+                    : "+f"(sd), "+f"(sq) : "f"(dl[c]), "f"(df[c]), "f"(qm[c]), "f"(pass_thr));
+            else sd += dl[c] > pass_thr ? df[c] : 0.f;
+        if (!kBinned) continue;
         const float big = fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3]));
         if (big >= kBigUnits) {
 #pragma unroll
@@ -701,6 +652,111 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
                 :: "f"(dl[c]), "r"(addr[c]), "r"(__float2uint_rn(pm[c])), "r"(__float2uint_rn(qm[c])), "n"(kHistWords * 4), "f"(pass_thr)
                 : "memory");
     }
+}
+
+// One cluster-wide pass without a histogram: item sums of max(p_beam - s q_beam, 0) over the live rows.
+// kFirst: s = 1, in the arithmetic (and the half-tile items) of the histogram pass; half_bin is that of the layer's histogram.
+// Else: any s, in the arithmetic of the search inside a tile (cell_mass), so that a tile with a sum has a cell that the search
+// finds; whole tiles.  sh.warp_part gets the total of each warp's items as whole numbers: the order in which warps and CTAs add
+// up changes nothing, and a small F keeps its digits; and, unless kFirst, the q mass of the cells with p_beam > s q_beam.
+// Bound by latency: few clusters make such a pass at a time, a warp takes about 1.8 us a half tile.  Straight-line loads for whole
+// aligned halves.  (The next item prefetched into L2: no difference.  Totals in registers: spills, a call 1 per cent slower.)
+// Functions of their own: the callers would each carry the unrolled loop.
+constexpr double kSumUnit = 1152921504606846976.0;               // 2^60
+template <bool kFirst>
+__device__ __noinline__ void residual_pass(const float *__restrict__ zp, const float *__restrict__ zq, int64_t stride,
+                                                int V, int T, float k2, Shared &sh, float s, float half_bin, double *sums,
+                                                int warp, int nwarps, int halves) {
+    const int lane = threadIdx.x & 31;
+    const int row_items = T * halves, items = sh.nA * row_items;
+    if (lane < 3) sh.warp_part[lane][threadIdx.x >> 5] = 0ll;
+    __syncwarp();
+    for (int item = warp; item < items; item += nwarps) {
+        const int i = item / row_items, t = item - i * row_items;
+        const int row = sh.A[i];
+        const float *rp = zp + (int64_t)row * stride;
+        const float *rq = zq + (int64_t)row * stride;
+        const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
+        const RowOff ro = row_off(sh, i);
+        double res1 = 0.0;
+        float acc = 0.f, q_acc = 0.f;
+        int e0 = t * (kTile / halves);
+#pragma unroll 1
+        for (int half = halves; half < 3; ++half, e0 += kTile / 2) {
+            float4 vp[4], vq[4];
+            if (al && e0 + kTile / 2 <= V) {
+#pragma unroll
+                for (int it = 0; it < 4; ++it) vp[it] = ldg_stream(reinterpret_cast<const float4 *>(rp + e0 + it * 128) + lane);
+#pragma unroll
+                for (int it = 0; it < 4; ++it) vq[it] = ldg_stream(reinterpret_cast<const float4 *>(rq + e0 + it * 128) + lane);
+            } else {
+                load_half_tile(rp, e0, V, false, lane, vp);
+                load_half_tile(rq, e0, V, false, lane, vq);
+            }
+            if (kFirst) {
+                float sd = 0.f, sq = 0.f;
+                hist_half_tile<false>(vp, vq, k2, ro, 0.f, half_bin, 0.f, 0u, 0u, sd, sq);
+                res1 += (double)sd;
+            } else {
+                auto cell = [&](float vpc, float vqc) {
+                    float q;
+                    const float d = cell_mass(vpc, vqc, k2, ro, s, &q);
+                    acc += d;
+                    q_acc += d > 0.f ? q : 0.f;
+                };
+#pragma unroll
+                for (int it = 0; it < 4; ++it) {
+                    cell(vp[it].x, vq[it].x); cell(vp[it].y, vq[it].y);
+                    cell(vp[it].z, vq[it].z); cell(vp[it].w, vq[it].w);
+                }
+            }
+        }
+        const double tot = kFirst ? warp_sum(res1) * kUnfix : warp_sum((double)acc);
+        const double q = kFirst ? 0.0 : warp_sum((double)q_acc) * (double)kFix;
+        if (lane == 0) {
+            sums[item] = tot;
+            const long long hi = __double2ll_rn(tot * kSumUnit);
+            sh.warp_part[0][threadIdx.x >> 5] += hi;
+            sh.warp_part[1][threadIdx.x >> 5] += __double2ll_rn((tot * kSumUnit - (double)hi) * kSumUnit);
+            if (!kFirst) sh.warp_part[2][threadIdx.x >> 5] += __double2ll_rn(q);
+        }
+    }
+}
+
+// F(s) by a pass of the whole cluster over the live rows, whose item sums go to `sums`.  first: s = 1, with the sums that the
+// histogram pass would have left.  Else the cells meet s as one float, as in the search of a draw; what that leaves out of
+// F, the remainder of s times the q mass above, is taken off the total.  n_pass: passes of the kernel before this one.
+// want_total = false: the item sums alone, for a draw.
+__device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, double s, double *sums, bool first, float half_bin,
+                                          int halves, bool want_total, int n_pass) {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int n_cta = (int)cluster.num_blocks(), cta_rank = (int)cluster.block_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float s_hi = (float)s;
+    const int w = cta_rank * kVWarps + warp, nw = n_cta * kVWarps;
+    if (first) residual_pass<true>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, half_bin, sums, w, nw, halves);
+    else residual_pass<false>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, 0.f, sums, w, nw, halves);
+    if (!want_total) {
+        cluster.sync();
+        return 0.0;
+    }
+    __syncthreads();
+    if (warp < 3) {
+        long long v = lane < kVWarps ? sh.warp_part[warp][lane] : 0ll;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        if (lane < n_cta) cluster.map_shared_rank(&sh, lane)->part[n_pass & 1][warp][cta_rank] = v;
+    }
+    cluster.sync();                                    // (two buffers: who is here has read those of the pass before)
+    long long hi = 0ll, lo = 0ll, q = 0ll;
+    for (int c = 0; c < n_cta; ++c) {
+        hi += sh.part[n_pass & 1][0][c];
+        lo += sh.part[n_pass & 1][1][c];
+        q += sh.part[n_pass & 1][2][c];
+    }
+    const double total = ((double)lo * (1.0 / kSumUnit) + (double)hi) * (1.0 / kSumUnit);
+    const double rest = (s - (double)s_hi) * ((double)q * kUnfix);
+    return rest < total ? total - rest : total;
 }
 
 // One cluster-wide pass over the live rows; every CTA fills its own shared-memory histogram.
@@ -741,7 +797,7 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, int n_bins
                 load_half_tile(rq, e0, a.V, false, lane, vq);
             }
             float sd = 0.f, sq = 0.f;
-            hist_half_tile(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sd, sq);
+            hist_half_tile<true>(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sd, sq);
             added += __float2ull_rn(fmaf(2.f, sq, sd));
             res1 += (double)sd;
         }
@@ -1663,25 +1719,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             sh.n_near += near;
             sh.need_exact = need;
         };
-        // F(s) by a pass of the whole cluster over the live rows, whose item sums go to `sums`
-        auto exact_pass = [&](double s, double *sums, int halves) {
-            const long long mine = residual_pass(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s, sums,
-                                                 cta_rank * kVWarps + warp, n_cta * kVWarps, halves);
-            if (lane == 0) sh.warp_part[warp] = mine;
-            __syncthreads();
-            if (warp == 0) {
-                long long v = lane < kVWarps ? sh.warp_part[lane] : 0ll;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-                if (lane < n_cta) cluster.map_shared_rank(&sh, lane)->part[n_pass & 1][cta_rank] = v;
-            }
-            cluster.sync();                            // (two buffers: who is here has read those of the pass before)
-            long long v = 0ll;
-            for (int c = 0; c < n_cta; ++c) v += sh.part[n_pass & 1][c];
-            ++n_pass;
-            return (double)v * (1.0 / kSumUnit);
-        };
-
         constexpr bool warped = kWarped;
         WarpScratch &wsup = *reinterpret_cast<WarpScratch *>(hq);       // the histogram arrays are idle when warped
         if (warped) {
@@ -1753,7 +1790,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             while (on_demand && sh.need_exact) {
                 const int j = sh.run_j;
                 const int halves = j == 1 ? item_halves(sh.nA * a.T, n_cta * kVWarps) : 1;   // (slot 0 has room for half tiles)
-                const double c_next = exact_pass(sh.s_arr[j], sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride, halves);
+                const float half_bin = 0.5f / (float)((double)layer_bins(m, false) / log2((double)(m > 2 ? m : 2)));
+                const double c_next = exact_pass(a, sh, sh.s_arr[j], sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride,
+                                                 j == 1, half_bin, halves, true, n_pass++);
                 if (threadIdx.x == 0) {
                     if (j == 1) sh.halves = halves;
                     sh.c_arr[j + 1] = c_next;
@@ -1888,7 +1927,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 // (at j = 1 these are the sums that the histogram pass left in slot 0)
                 double *sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride;
                 if (j == 1 && threadIdx.x == 0) sh.halves = 1;
-                const double c_next = exact_pass(sh.s_arr[j], sums, 1);
+                const double c_next = exact_pass(a, sh, sh.s_arr[j], sums, false, 0.f, 1, true, n_pass++);
                 if (threadIdx.x == 0) sh.c_arr[j + 1] = c_next;
                 __syncthreads();
                 if (!(sh.c_arr[j + 1] > 0.0)) break;
@@ -1954,9 +1993,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         const int res_slot = on_demand && sh.run_j > 2 ? sh.run_j - 1 : 0;
         double *res_sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1) + res_slot) * slot_stride;
         if (!a.select_mode && !sh.err && !warped && sh.res_j > 2) {   // run position 2 is served by the histogram pass
-            const int halves = item_halves(sh.nA * a.T, n_cta * kVWarps);
-            if (threadIdx.x == 0) { ++sh.n_respass; sh.halves = halves; }
-            exact_pass(sh.s_arr[sh.res_j - 1], res_sums, halves);
+            if (threadIdx.x == 0) { ++sh.n_respass; sh.halves = 1; }
+            exact_pass(a, sh, sh.s_arr[sh.res_j - 1], res_sums, false, 0.f, 1, false, n_pass++);
         }
 
         TS(10);

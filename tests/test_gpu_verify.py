@@ -5,7 +5,7 @@ import torch
 
 import oracle
 import paper_2409_16560_b200 as dsbd
-from paper_2409_16560_b200 import inputs
+from paper_2409_16560_b200 import binding, inputs
 from parity_util import check_exempt, compare_verify, run_gpu_verify, to_host_f32
 
 pytestmark = pytest.mark.gpu
@@ -347,6 +347,45 @@ def test_layers_of_known_width(V, beams, W_min, W_max):
         exempt += e
         decisions += d
     check_exempt(exempt, decisions)
+
+
+@pytest.mark.parametrize("V,beams,seeds", [(128256, 2, 3), (50257, 2, 2), (1025, 2, 1)])
+def test_draws_behind_a_layer_of_known_width_are_those_of_a_histogram(V, beams, seeds):
+    """One layer of two drafts whose two beams are wanted: W_min = 2 says so beforehand (no histogram is built), a
+    threshold that every tail reaches says so afterwards.  The sums that a residual draw searches are the same numbers either
+    way (run position 2: those of the histogram pass; 3: the cells at s as one float), so every output is, bit for bit."""
+    R, steps = 64, 400
+    forest, _, _ = inputs.build_forest(dict(R=R, W=beams, tree=inputs._chain(1), prefix=(1, 1)), np.random.default_rng(V))
+    f = dsbd.Forest(forest, "cuda")
+    off = dsbd.default_out_off(forest, dict(W_max=beams, W_nom=beams))
+    drawn = 0
+    for seed in range(seeds):
+        gen = torch.Generator(device="cuda").manual_seed(1000 * V + seed)
+        zq = 2.0 * torch.randn(forest["N"], V, generator=gen, device="cuda")
+        zp = zq + 0.8 * torch.randn(forest["N"], V, generator=gen, device="cuda")
+        rp, rq = (torch.randn(forest["B"], generator=gen, device="cuda") for _ in range(2))
+        parent = torch.as_tensor(forest["parent"], device="cuda").long()
+        drafts = torch.nonzero(parent >= 0).squeeze(1)
+        f.dev["token"][drafts] = torch.multinomial(torch.softmax(zq[parent[drafts]], dim=1), 1, generator=gen).squeeze(1).to(torch.int32)
+        known = dict(V=V, temperature=1.0, thresh=0.7, W_min=beams, W_max=beams, W_nom=beams, seed=seed, step=0, top_k=0, top_p=1.0)
+        outs = [dsbd.alloc_verify_out(f, off, "cuda") for _ in range(2)]
+        ws = torch.empty(dsbd.verify_workspace(f, known), dtype=torch.uint8, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        moved = torch.zeros((), dtype=torch.int64, device="cuda")
+        n_drawn = torch.zeros((), dtype=torch.int64, device="cuda")
+        for step in range(steps):
+            for out, prm in zip(outs, (known, dict(known, W_min=1, thresh=1e-9))):
+                for name in ("out_token", "out_parent", "out_node", "out_root_beam", "out_source", "out_logp", "out_logq"):
+                    out[name].zero_()
+                dsbd.verify_step(f, dict(prm, step=step), zp, zq, rp, rq, out, workspace=ws, status=status)
+            for name in outs[0]:
+                if name != "req_stats":
+                    moved += (outs[0][name] != outs[1][name]).sum()
+            n_drawn += (outs[0]["out_source"] == binding.SRC_RESIDUAL).sum()
+        assert int(status) == 0 and int(outs[0]["req_error"].abs().sum()) == 0
+        assert int(moved) == 0, "%d outputs differ" % int(moved)
+        drawn += int(n_drawn)
+    assert drawn > 0.1 * R * steps * seeds
 
 
 @pytest.mark.parametrize("V", [2000, 40000])

@@ -496,14 +496,17 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
 //      cell only its remainder below 2^-28 (less than 2^16 units).
 //   b: units of 2^-28, the whole multiples of 2^-28 of the cells of at least 2^-16; it cannot
 //      overflow because a joint distribution sums to one.
-// A w word wraps once the small cells of ONE bin that ONE CTA added reach 2^-12 of the mass --
-// twenty times what a bin holds in ordinary data, but possible when the two models' rows are
-// proportional and every cell lands in the same bin.  A wrap is always detected: every thread
+// A w word wraps once the small cells of ONE bin that ONE CTA added reach 2^-12 of the mass.  Two models sigma nats
+// apart have up to 0.4 / sigma of their mass per nat, shared out over the cluster's CTAs, and a bin of a layer of m drafts is
+// ln(max(m, 2)) / 4096 nats wide: with 4 CTAs, 8 drafts and sigma = 1 that is a fifth of 2^-12, with 2 CTAs, 2 drafts and
+// sigma = 0.4 a third; the fullest bin holds about twice that.  The copies of the last bin take 256 times 2^-12, a sixteenth of
+// the mass.  Closer models or a flat vocabulary with one CTA (more requests than SMs), and rows that are proportional, where every cell
+// lands in the same bin, can reach it.  A wrap is always detected: every thread
 // keeps a total of the mass that it added, and the sum of those totals is compared with the sum of
 // all words; a difference marks the layer, whose residual masses are
 // then all computed by exact passes over the rows.
 // ---------------------------------------------------------------------------------------
-constexpr int kBins = 4096;                       // at most; layers of few drafts take fewer (layer_bins)
+constexpr int kBins = 4096;
 constexpr int kOverSlots = 256;                   // copies of the last bin (rho beyond the last edge): one per
                                                   // warp and half-warp lane, so that none collects enough to wrap
 constexpr int kHistWords = kBins + kOverSlots + 16;  // bins 0..kBins-1, the copies of bin kBins, spare words
@@ -516,13 +519,6 @@ struct HistSmem { uint32_t *wp, *wq, *bp, *bq; };
 
 __device__ __forceinline__ HistSmem hist_arrays(uint32_t *base) {
     return HistSmem{base, base + kHistWords, base + 2 * kHistWords, base + 3 * kHistWords};
-}
-
-// Bins of a layer of m drafts: they cover [1, max(m, 2)], and the bracket of a residual mass is as wide as a bin's square, so a
-// short range needs fewer (and the merge, which is bound by their words, is shorter).  Their width is at most 1/1024 of an
-// octave for m <= 4, as for 16 drafts (8: 1/1365, 64: 1/683).  dsbd_select_width, which returns the alphas, always takes all.
-__device__ __forceinline__ int layer_bins(int m, bool select_mode) {
-    return select_mode || m > 4 ? kBins : m > 2 ? kBins / 2 : kBins / 4;
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -761,7 +757,7 @@ __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, do
 
 // One cluster-wide pass over the live rows; every CTA fills its own shared-memory histogram.
 // tot (shared memory, zero before the call): [0] the mass that the CTA added (p and q), from floating-point sums.
-__device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, int n_bins, float binscale, const HistSmem &h,
+__device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float binscale, const HistSmem &h,
                                double *sums1, int cta_rank, int n_cta, int halves, unsigned long long *tot) {
     // halves = 2: an item is a half tile (when the cluster has a warp for each), with a sum of its own
     const int lane = threadIdx.x & 31;
@@ -773,7 +769,7 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, int n_bins
     const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(h.wp) - (magic_bits << 2);
     const uint32_t over_bits = magic_bits + (uint32_t)(kBins + ((threadIdx.x >> 5) & 15) * 16 + (threadIdx.x & 15));
     const float half_bin = 0.5f / binscale;                      // half a bin in log2 units
-    const float top = (float)n_bins / binscale - half_bin;       // log2 of the last edge (minus the half), as the bins see it
+    const float top = (float)kBins / binscale - half_bin;       // log2 of the last edge (minus the half), as the bins see it
     const int row_items = a.T * halves;
     for (int item = warp; item < items; item += nwarps) {
         const int i = item / row_items, t = item - i * row_items;
@@ -814,16 +810,11 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, int n_bins
 // The copies of the last bin (rho beyond the last edge), folded by each CTA and added to every CTA's total
 // (tot[7], tot[8]); before the cluster barrier that follows the pass.  Also tot[6] += what the CTA's threads
 // added minus what these copies hold of it.
-__device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, int n_bins, unsigned long long *tot, int n_cta) {
+__device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *tot, int n_cta) {
     const int lane = threadIdx.x & 31;
     if (threadIdx.x < kOverSlots) {
         const int i = kBins + (int)threadIdx.x;
         unsigned long long P = ((unsigned long long)h.bp[i] << 16) + h.wp[i], Q = ((unsigned long long)h.bq[i] << 16) + h.wq[i];
-        if (threadIdx.x == 0 && n_bins < kBins) {
-            // (a ratio within rounding of the last edge may give bin n_bins; with kBins that is the first copy)
-            P += ((unsigned long long)h.bp[n_bins] << 16) + h.wp[n_bins];
-            Q += ((unsigned long long)h.bq[n_bins] << 16) + h.wq[n_bins];
-        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             P += __shfl_xor_sync(kFull, P, o);
@@ -843,25 +834,24 @@ __device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, in
 // Merge of the cluster's histograms, after a cluster barrier that follows the pass: every CTA sums one slice of
 // the bins over all CTAs' shared memory.  A lane takes four bins of two CTAs (eight bins when there is one CTA), so
 // that all its loads are in flight together; the lanes that share bins add up by shuffles, and with 16 CTAs two
-// warps share bins; with fewer bins the last warps have none.  The CTA's suffix sums (p and q mass of the slice's bins >= k, units of 2^-44) replace the words of
+// warps share bins.  The CTA's suffix sums (p and q mass of the slice's bins >= k, units of 2^-44) replace the words of
 // its own slice, which no other CTA reads here: w words the low, b words the high halves.  Every CTA
 // gets the slice's totals.  The caller puts a cluster barrier behind this before anyone looks at another's slice.
-// Bound by distributed shared memory (64 KB a CTA with all bins, 4.4 us; 32 KB 3.1), as long as an instruction takes at least 128 bytes from
+// Bound by distributed shared memory (64 KB a CTA, 4.5 us), as long as an instruction takes at least 128 bytes from
 // each CTA it reads: with 64 bytes from each of 8, one warp to the bins, 16 CTAs took 7 to 10 us.  (512 bytes
 // an instruction and the sums of 2 to 8 warps through a stage of 16 KB were no faster with 8 CTAs, and the shared
 // memory came off the L1 cache: 64 requests x 8 rows of 128256 30 us slower.  Half the words to fetch, by b words
 // that are added at once in the CTA that will merge them: merge 4.4 -> 3.3 us, but the pass 110 -> 115 and, for one request
-// of V = 32000, 7.5 -> 9.5: an atomic add to another CTA's shared memory costs its warp more than a local one.)
-__device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, int n_bins, Shared &sh, int cta_rank, int n_cta) {
+// of V = 32000, 7.5 -> 9.5: an atomic add to another CTA's shared memory costs its warp more than a local one.  Half the
+// bins for layers of few drafts: merge 4.4 -> 3.1, but their w words wrap on ordinary data when one CTA has the whole layer.)
+__device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, Shared &sh, int cta_rank, int n_cta) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int share = n_cta > 1 ? min(n_cta / 2, 4) : 1;     // lanes that share four bins
     const int parts = n_cta > 8 ? 2 : 1;                     // warps that share them
-    const int per_warp = 32 / share, place = lane % per_warp;
-    const int lane_bins = n_cta > 1 ? 4 : 8, slice = n_bins / n_cta;
-    const int segs = slice / (per_warp * lane_bins);         // warps (of a part) with bins
-    const int seg = warp % (kVWarps / parts), part = warp / (kVWarps / parts);
-    const bool mine = seg < segs;
-    const int i0 = cta_rank * slice + (seg * per_warp + place) * lane_bins;
+    const int per_warp = 32 / share, place = lane % per_warp, segs = kVWarps / parts;
+    const int seg = warp % segs, part = warp / segs;
+    const int n_bins = n_cta > 1 ? 4 : 8;                    // of a lane
+    const int i0 = cta_rank * (kBins / n_cta) + (seg * per_warp + place) * n_bins;
     unsigned long long P[8] = {}, Q[8] = {};
     auto add4 = [&](int c, int i, unsigned long long *p, unsigned long long *q) {
         const uint4 wp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wp, c) + i);
@@ -873,15 +863,13 @@ __device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, int n_
         q[0] += ((unsigned long long)bq.x << 16) + wq.x; q[1] += ((unsigned long long)bq.y << 16) + wq.y;
         q[2] += ((unsigned long long)bq.z << 16) + wq.z; q[3] += ((unsigned long long)bq.w << 16) + wq.w;
     };
-    if (mine) {
-        const int c0 = part * 8 + lane / per_warp;
-        if (n_cta > 1) {
-            add4(c0, i0, P, Q);
-            add4(c0 + share, i0, P, Q);
-        } else {
-            add4(0, i0, P, Q);
-            add4(0, i0 + 4, P + 4, Q + 4);
-        }
+    const int c0 = part * 8 + lane / per_warp;
+    if (n_cta > 1) {
+        add4(c0, i0, P, Q);
+        add4(c0 + share, i0, P, Q);
+    } else {
+        add4(0, i0, P, Q);
+        add4(0, i0 + 4, P + 4, Q + 4);
     }
     for (int o = per_warp; o < 32; o <<= 1) {
 #pragma unroll
@@ -902,9 +890,9 @@ __device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, int n_
     if (parts == 2) {
         // the second warp's sums through the slice itself, once the whole CTA has read its own words there
         __syncthreads();
-        if (mine && part == 1 && lane < per_warp) store4(i0, P, Q, 0ull, 0ull);
+        if (part == 1 && lane < per_warp) store4(i0, P, Q, 0ull, 0ull);
         __syncthreads();
-        if (mine && part == 0) {
+        if (part == 0) {
             const uint4 lp = *reinterpret_cast<const uint4 *>(h.wp + i0), up = *reinterpret_cast<const uint4 *>(h.bp + i0);
             const uint4 lq = *reinterpret_cast<const uint4 *>(h.wq + i0), uq = *reinterpret_cast<const uint4 *>(h.bq + i0);
             auto whole = [](uint32_t low, uint32_t high) { return ((unsigned long long)high << 32) | low; };
@@ -920,9 +908,9 @@ __device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, int n_
         const unsigned long long tp = __shfl_down_sync(kFull, ap, o), tq = __shfl_down_sync(kFull, aq, o);
         if (place + o < per_warp) { ap += tp; aq += tq; }
     }
-    if (mine && part == 0 && lane == 0) { sh.wtot_p[seg] = ap; sh.wtot_q[seg] = aq; }
+    if (part == 0 && lane == 0) { sh.wtot_p[seg] = ap; sh.wtot_q[seg] = aq; }
     __syncthreads();
-    if (part > 0 || !mine) return;
+    if (part > 0) return;
     unsigned long long rp = ap - P[0], rq = aq - Q[0];
     for (int w = seg + 1; w < segs; ++w) { rp += sh.wtot_p[w]; rq += sh.wtot_q[w]; }
     if (lane < per_warp) {
@@ -1790,7 +1778,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             while (on_demand && sh.need_exact) {
                 const int j = sh.run_j;
                 const int halves = j == 1 ? item_halves(sh.nA * a.T, n_cta * kVWarps) : 1;   // (slot 0 has room for half tiles)
-                const float half_bin = 0.5f / (float)((double)layer_bins(m, false) / log2((double)(m > 2 ? m : 2)));
+                const float half_bin = 0.5f / (float)((double)kBins / log2((double)(m > 2 ? m : 2)));
                 const double c_next = exact_pass(a, sh, sh.s_arr[j], sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride,
                                                  j == 1, half_bin, halves, true, n_pass++);
                 if (threadIdx.x == 0) {
@@ -1806,25 +1794,24 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         if (m >= 1 && !sh.err && !warped && !on_demand) {
             // ---- one pass: ratio histogram of the layer over the live rows ----
             const double top = log2((double)(m > 2 ? m : 2));          // s_j <= j <= m
-            const int n_bins = layer_bins(m, a.select_mode != 0);
-            const float binscale = (float)((double)n_bins / top);
+            const float binscale = (float)((double)kBins / top);
             // (counted by histograms, not by layers: the other bank is cleared between the barriers of this one)
             const int bank = n_hist++ & 1;
             unsigned long long *tot = sh.w_tot[bank];
             const int halves = item_halves(sh.nA * a.T, n_cta * kVWarps);
-            histogram_pass(a, sh, n_bins, binscale, hs, sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride, cta_rank,
+            histogram_pass(a, sh, binscale, hs, sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride, cta_rank,
                            n_cta, halves, tot);
             __syncthreads();
-            hist_fold_over(cluster, hs, n_bins, tot, n_cta);
+            hist_fold_over(cluster, hs, tot, n_cta);
             TS(4);
             cluster.sync();                            // every CTA's histogram is complete
             TS(6);
             if (threadIdx.x < 10) sh.w_tot[bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
                                                        // the barrier below
-            hist_merge(cluster, hs, n_bins, sh, cta_rank, n_cta);
+            hist_merge(cluster, hs, sh, cta_rank, n_cta);
             if (threadIdx.x == kVThreads - 32) {
                 // bin k is [e_k, e_k+1], e_k = 2^(k bin_log2); its width over e_k, with both edges 2e-6 wider
-                const double step = top / (double)n_bins, w = exp2(step) * (1.0 + 2e-6) - (1.0 - 2e-6);
+                const double step = top / (double)kBins, w = exp2(step) * (1.0 + 2e-6) - (1.0 - 2e-6);
                 sh.bin_log2 = step; sh.bin_width = w; sh.bin_inv_width = 1.0 / w;
             }
             TS(7);
@@ -1836,7 +1823,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             unsigned long long above_p = 0ull, above_q = 0ull;
             double n_cells = 0.0;
             bool wrapped = false;
-            const int slice = n_bins / n_cta;
+            const int slice = kBins / n_cta;
             if (warp == 0) {
                 const unsigned long long own_p = lane < n_cta ? sh.slice_p[lane] : 0ull, own_q = lane < n_cta ? sh.slice_q[lane] : 0ull;
                 above_p = own_p; above_q = own_q;
@@ -1860,7 +1847,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             // suffix sums of bin k (warp 0; the same on every lane): one word of each kind from the CTA that has it
             const int shift = 31 - __clz(slice);
             auto suffix = [&](int k, unsigned long long &P, unsigned long long &Q) {
-                if (k >= n_bins) { P = tot[7]; Q = tot[8]; return; }
+                if (k >= kBins) { P = tot[7]; Q = tot[8]; return; }
                 const int c = k >> shift;
                 const uint32_t lp = cluster.map_shared_rank(hs.wp, c)[k], hi_p = cluster.map_shared_rank(hs.bp, c)[k];
                 const uint32_t lq = cluster.map_shared_rank(hs.wq, c)[k], hi_q = cluster.map_shared_rank(hs.bq, c)[k];
@@ -1893,7 +1880,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                             // bracket below takes the edges 2e-6 wider)
                             int k = (int)(__log2f((float)s_j) * binscale);
                             if (k < 0) k = 0;
-                            if (k >= n_bins) { need = 1; break; }     // cannot happen for s_j <= m
+                            if (k >= kBins) { need = 1; break; }     // cannot happen for s_j <= m
                             suffix(k, P[0], Q[0]);
                             suffix(k + 1, P[1], Q[1]);
                             const double Pa = (double)P[1] * kUnfix, Qa = (double)Q[1] * kUnfix;

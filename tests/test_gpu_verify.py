@@ -388,6 +388,26 @@ def test_draws_behind_a_layer_of_known_width_are_those_of_a_histogram(V, beams, 
     assert drawn > 0.1 * R * steps * seeds
 
 
+@pytest.mark.parametrize("beams,sigma", [(2, 0.38), (3, 0.5), (4, 0.7)])
+def test_words_of_a_layer_of_few_drafts_do_not_wrap(beams, sigma):
+    """100 requests: two CTAs add the whole layer to their histograms.  Two models sigma nats apart over a flat vocabulary put
+    0.4 / sigma of their mass per nat next to ratio 1, which is 0.9e-4 to 1.1e-4 for each CTA in a bin of ln(beams) / 4096 nats.
+    A bin has 20 cells or more, so the fullest of 4096 holds up to twice that: below the 2^-12 = 2.4e-4 at which a word wraps.
+    Of the 0.05 of the mass beyond the last edge, ratio `beams`, each of 2 x 256 words holds 1e-4 or less."""
+    V, R = 128256, 100
+    forest, _, _ = inputs.build_forest(dict(R=R, W=beams, tree=inputs._chain(1), prefix=(1, 1)), np.random.default_rng(R))
+    gen = torch.Generator(device="cuda").manual_seed(V + beams)
+    zp = 0.3 * torch.randn(forest["N"], V, generator=gen, device="cuda")
+    zq = zp + sigma * torch.randn(forest["N"], V, generator=gen, device="cuda")
+    rp = rq = torch.zeros(forest["B"], device="cuda")
+    prm = dict(V=V, temperature=1.0, thresh=0.7, W_min=1, W_max=beams, W_nom=beams, seed=5, step=0, top_k=0, top_p=1.0)
+    gpu, status = run_gpu_verify(forest, prm, zp, zq, rp, rq)
+    assert status == 0
+    assert int(gpu["req_stats"].reshape(R, -1)[:, 6].sum()) == 0
+    e, d = compare_verify(_oracle(forest, prm, *(to_host_f32(x) for x in (zp, zq, rp, rq))), gpu, forest)
+    check_exempt(e, d)
+
+
 @pytest.mark.parametrize("V", [2000, 40000])
 def test_histograms_with_a_layer_of_known_width_between(V):
     """A layer with a histogram, one that needs none, another with one: drafts that widen again behind a chain."""

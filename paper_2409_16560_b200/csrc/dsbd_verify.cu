@@ -258,7 +258,6 @@ struct Shared {
     unsigned long long wtot_p[kVWarps], wtot_q[kVWarps];
     unsigned long long slice_p[16], slice_q[16];   // mass of the bins of every CTA's slice
     unsigned long long above_p[16], above_q[16];   // mass of the bins above every CTA's slice
-    double bin_log2, bin_width, bin_inv_width;     // of a bin: log2 of its upper over its lower edge; see the chain
     unsigned long long w_tot[2][10];        // per bank, sums of one histogram pass: see histogram_pass / hist_fold_over
     int n_wrapped;                          // layers where a w word of the histogram wrapped
     double rho[kMaxLive], uu[kMaxLive];     // per live draft: p_beam/q_beam and its uniform
@@ -1809,11 +1808,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             if (threadIdx.x < 10) sh.w_tot[bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
                                                        // the barrier below
             hist_merge(cluster, hs, sh, cta_rank, n_cta);
-            if (threadIdx.x == kVThreads - 32) {
-                // bin k is [e_k, e_k+1], e_k = 2^(k bin_log2); its width over e_k, with both edges 2e-6 wider
-                const double step = top / (double)kBins, w = exp2(step) * (1.0 + 2e-6) - (1.0 - 2e-6);
-                sh.bin_log2 = step; sh.bin_width = w; sh.bin_inv_width = 1.0 / w;
-            }
             TS(7);
             cluster.sync();                            // every slice of the suffix sums is complete
             TS(5);
@@ -1854,7 +1848,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 P = (((unsigned long long)hi_p << 32) | lp) + sh.above_p[c];
                 Q = (((unsigned long long)hi_q << 32) | lq) + sh.above_q[c];
             };
-            const double bin_log2 = sh.bin_log2, width = sh.bin_width, inv_width = sh.bin_inv_width;
 
             int j0 = 1;
             while (j0 <= m) {
@@ -1876,9 +1869,10 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                             c_next = ((double)P[0] - (double)Q[0]) * kUnfix;
                             if (fix_err > kErrTol) { need = 1; break; }
                         } else {
-                            // (the approximate logarithm and exponential miss the bin and its edges by at most 8e-7; the
-                            // bracket below takes the edges 2e-6 wider)
-                            int k = (int)(__log2f((float)s_j) * binscale);
+                            // (up to s = 64 the bin found is off by at most 9e-7 of an edge: the logarithm's last place 3.3e-7, s as a
+                            // float 0.6e-7, the product with binscale 5e-7; an edge by 6e-7.  The bracket below takes the edges
+                            // 2e-6 wider.  Approximate logarithm and exponential, reciprocals for the division: 1 us less, 1.6e-6)
+                            int k = (int)(log2f((float)s_j) * binscale);
                             if (k < 0) k = 0;
                             if (k >= kBins) { need = 1; break; }     // cannot happen for s_j <= m
                             suffix(k, P[0], Q[0]);
@@ -1886,12 +1880,10 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                             const double Pa = (double)P[1] * kUnfix, Qa = (double)Q[1] * kUnfix;
                             const double Pk = (double)(P[0] - P[1]) * kUnfix;
                             const double Qk = (double)(Q[0] - Q[1]) * kUnfix;
-                            const float e_log2 = (float)((double)k * bin_log2);
-                            const double e_k = (double)ex2_approx(e_log2), inv_e = (double)ex2_approx(-e_log2);
-                            const double r_lo = e_k * (1.0 - 2e-6);
+                            const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
+                            const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
                             const double lo_b = fmax(Pk - s_j * Qk, 0.0);
-                            double q_hi = (Pk - r_lo * Qk) * (inv_e * inv_width);        // / (r_hi - r_lo)
-                            const double r_hi = r_lo + e_k * width;
+                            double q_hi = (Pk - r_lo * Qk) / (r_hi - r_lo);
                             q_hi = fmin(fmax(q_hi, 0.0), Qk);
                             const double hi_b = fmax(q_hi * (r_hi - s_j), lo_b);
                             // the midpoint of the bracket is used: half its width plus the fixed-point term

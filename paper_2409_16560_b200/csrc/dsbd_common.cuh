@@ -77,6 +77,15 @@ __device__ __forceinline__ float4 ldg_stream(const float4 *p) {
     return v;
 }
 
+// The same for a kernel that may be resident while the data is still being written, and waits for it: .nc is only for data
+// that nobody writes as long as the kernel runs.
+__device__ __forceinline__ float4 ld_stream(const float4 *p) {
+    float4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace dsbd

@@ -50,20 +50,34 @@ constexpr double kLn2 = 0.6931471805599453;
 
 struct TileStat { float mx; float sum; };   // max of the raw logits, sum exp((z-mx)/tau)
 
-__device__ __forceinline__ void load_tile(const float *__restrict__ row, int e0, int V, bool aligned,
-                                          int lane, float4 (&v)[8]) {
-    const float ninf = -INFINITY;
+// kWritten: the row may have been written while the kernel was resident already (it has waited since).  Its single words by
+// predicated loads: as plain conditional ones they took 6 registers more, and five draft layers of 16 x 8 rows 180 us instead of 173.
+template <bool kWritten>
+__device__ __forceinline__ void load_tile(const float *row, int e0, int V, bool aligned, int lane, float4 (&v)[8]) {
+    auto four = [&](int e) {
+        const float4 *p = reinterpret_cast<const float4 *>(row + e);
+        return kWritten ? ld_stream(p) : ldg_stream(p);
+    };
+    auto one = [&](int e) {
+        if (!kWritten) return e < V ? __ldg(row + e) : -INFINITY;
+        float x;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "setp.lt.s32 p, %2, %3;\n\t"
+                     "mov.f32 %0, 0fFF800000;\n\t"
+                     "@p ld.global.f32 %0, [%1];\n\t}"
+                     : "=&f"(x) : "l"(row + e), "r"(e), "r"(V));
+        return x;
+    };
+    if (aligned && e0 + kTile <= V) {
+#pragma unroll
+        for (int it = 0; it < 8; ++it) v[it] = four(e0 + it * 128 + lane * 4);
+        return;
+    }
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
         const int e = e0 + it * 128 + lane * 4;
-        if (aligned && e + 3 < V) {
-            v[it] = ldg_stream(reinterpret_cast<const float4 *>(row + e));
-        } else {
-            v[it].x = e < V ? __ldg(row + e) : ninf;
-            v[it].y = e + 1 < V ? __ldg(row + e + 1) : ninf;
-            v[it].z = e + 2 < V ? __ldg(row + e + 2) : ninf;
-            v[it].w = e + 3 < V ? __ldg(row + e + 3) : ninf;
-        }
+        if (aligned && e + 3 < V) v[it] = four(e);
+        else v[it] = make_float4(one(e), one(e + 1), one(e + 2), one(e + 3));
     }
 }
 
@@ -91,14 +105,12 @@ __device__ __forceinline__ void load_half_tile(const float *__restrict__ row, in
 // listed row outside [0, N) is skipped -- the kernel that consumes the list reports it).
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads)
-k_tile_stats(const float *__restrict__ zp, const float *__restrict__ zq, int64_t stride, int V,
-             int T, int N, int n_rows, const int32_t *__restrict__ rows,
-             const int32_t *__restrict__ n_rows_dev, float k2, TileStat *__restrict__ stats,
-             int one_model = 0) {
+k_tile_stats(const float *zp, const float *zq, int64_t stride, int V, int T, int N, int n_rows, const int32_t *rows,
+             const int32_t *n_rows_dev, float k2, TileStat *__restrict__ stats, int one_model = 0) {
     // Launched with programmatic stream serialization: its blocks are in place when the work ahead in the stream ends, and
-    // read nothing before (five draft layers of 16 x 8 rows of 128256: 183 -> 175 us).  In this order: the kernel behind it,
-    // which may be set up while the last blocks run, must not start (and read what the caller gave) before all earlier
-    // work is done.
+    // read nothing before (five draft layers of 16 x 8 rows of 128256: 183 -> 175 us); what they read then may have been
+    // written while they were in place, so not through .nc.  In this order: the kernel behind it, which may be set up while
+    // the last blocks run, must not start (and read what the caller gave) before all earlier work is done.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;
@@ -116,7 +128,7 @@ k_tile_stats(const float *__restrict__ zp, const float *__restrict__ zq, int64_t
         const float *z = (model ? zq : zp) + (int64_t)row * stride;
         const bool aligned = (reinterpret_cast<uintptr_t>(z) & 15) == 0;
         float4 v[8];
-        load_tile(z, t * kTile, V, aligned, lane, v);
+        load_tile<true>(z, t * kTile, V, aligned, lane, v);
         float mx = -INFINITY;
 #pragma unroll
         for (int it = 0; it < 8; ++it)
@@ -1127,7 +1139,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
             const float *rowp = z + (int64_t)row * a.stride;
             const bool al = (reinterpret_cast<uintptr_t>(rowp) & 15) == 0;
             float4 v[8];
-            load_tile(rowp, t * kTile, a.V, al, lane, v);
+            load_tile<false>(rowp, t * kTile, a.V, al, lane, v);
             const float off_f = tp.off[ia];
             const double off_d = lw[ia] - lse[row];
             unsigned hits = 0;                               // bit (it*4+c) of this lane's 32 cells

@@ -408,6 +408,42 @@ def test_words_of_a_layer_of_few_drafts_do_not_wrap(beams, sigma):
     check_exempt(e, d)
 
 
+@pytest.mark.parametrize("V,R", [(128256, 16), (5001, 2)])
+def test_inputs_written_right_before_the_call(V, R):
+    """Kernels of a call are in place before the work ahead of it in the stream ends: whatever that work writes (logits, tokens, root
+    scores), calls one behind the other see the values of their turn, as they do one at a time."""
+    rng = np.random.default_rng(V)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=R, V=V, gamma=2, max_w=3, min_w=3)
+    prm.update(W_min_r=None, W_min=2)
+    f, n = dsbd.Forest(forest, "cuda"), 3
+    first = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)] + [f.dev["token"].clone()]
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    sets = [first] + [[x + torch.randn(x.shape, generator=gen, device="cuda") for x in first[:4]] +
+                      [torch.randint(0, V, first[4].shape, generator=gen, device="cuda").to(torch.int32)] for _ in range(n - 1)]
+    live = [x.clone() for x in first[:4]] + [f.dev["token"]]
+    ws = torch.empty(dsbd.verify_workspace(f, prm), dtype=torch.uint8, device="cuda")
+    off = dsbd.default_out_off(forest, prm)
+
+    def call(k, status):
+        for dst, src in zip(live, sets[k % n]):
+            dst.copy_(src)
+        out = dsbd.alloc_verify_out(f, off, "cuda")
+        dsbd.verify_step(f, dict(prm, step=k), *live[:4], out, workspace=ws, status=status)
+        return out
+
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    alone = []
+    for k in range(24):
+        alone.append(call(k, status))
+        torch.cuda.synchronize()
+    behind = [call(k, status) for k in range(24)]
+    torch.cuda.synchronize()
+    assert int(status) == 0
+    for k in range(24):
+        for name in alone[k]:
+            assert torch.equal(alone[k][name], behind[k][name]), (k, name)
+
+
 @pytest.mark.parametrize("V", [2000, 40000])
 def test_histograms_with_a_layer_of_known_width_between(V):
     """A layer with a histogram, one that needs none, another with one: drafts that widen again behind a chain."""

@@ -48,6 +48,10 @@ constexpr int kMaxLive = DSBD_MAX_LIVE;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr double kLn2 = 0.6931471805599453;
 
+// A load before griddepcontrol.wait: from L2.
+template <class V>
+__device__ __forceinline__ V ld_early(const V *p) { return __ldcg(p); }
+
 struct TileStat { float mx; float sum; };   // max of the raw logits, sum exp((z-mx)/tau)
 
 // kWritten: the row may have been written while the kernel was resident already (it has waited since).  Its single words by
@@ -1319,11 +1323,15 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     uint32_t *hp = reinterpret_cast<uint32_t *>(dyn_smem), *hq = hp + kHistWords;     // first two digit arrays
     const HistSmem hs = hist_arrays(hp);
 
-    const int b_lo = a.req_beam_off[r], b_hi = a.req_beam_off[r + 1];
-    const int n_lo = a.beam_node_off[b_lo], n_hi = a.beam_node_off[b_hi];
-    int W_min = a.W_min_r ? a.W_min_r[r] : a.W_min;
-    int W_max = a.W_max_r ? a.W_max_r[r] : a.W_max;
-    int W_nom = a.W_nom_r ? a.W_nom_r[r] : a.W_nom;
+    // Launched with programmatic stream serialization: everything before griddepcontrol.wait overlaps the tail of the dense
+    // pass ahead in the stream.  That pass lets this kernel start only when each of its blocks has waited for all earlier work,
+    // so what earlier kernels and the caller left lies in L2 and may be read here, from there (ld_early: the pass's wait says
+    // nothing about this SM's L1); the tile statistics only after the wait.
+    const int b_lo = ld_early(a.req_beam_off + r), b_hi = ld_early(a.req_beam_off + r + 1);
+    const int n_lo = ld_early(a.beam_node_off + b_lo), n_hi = ld_early(a.beam_node_off + b_hi);
+    int W_min = a.W_min_r ? ld_early(a.W_min_r + r) : a.W_min;
+    int W_max = a.W_max_r ? ld_early(a.W_max_r + r) : a.W_max;
+    int W_nom = a.W_nom_r ? ld_early(a.W_nom_r + r) : a.W_nom;
     // per-request widths come from device memory: a width below 1 or a cap below the minimum is
     // reported (after the set-up below) and the request is not verified
     const bool bad_widths = a.check_widths && (W_min < 1 || W_max < W_min || W_nom < 1);
@@ -1339,9 +1347,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     // (a CTA may store into another's shared memory once that CTA runs: arrived here, waited for below)
     if (threadIdx.x < 20) sh.w_tot[threadIdx.x / 10][threadIdx.x % 10] = 0ull;
     cluster.barrier_arrive();
-    // Launched with programmatic stream serialization: everything before griddepcontrol.wait overlaps the tail of
-    // the dense pass ahead in the stream, whose grid started when all earlier work was done.  So what earlier
-    // kernels and the caller left may be read here, the tile statistics only after the wait.
     const int n_req_nodes = n_hi - n_lo, n_trees = min(b_hi - b_lo, kMaxLive);
     const bool cached = !a.select_mode && n_req_nodes <= kCacheNodes && a.gamma < 256;
     if (!a.select_mode) {
@@ -1355,17 +1360,17 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         int par = -1, tok = -1;
         float zp_tok = 0.f, zq_tok = 0.f;
         if (cached) {
-            if ((int)threadIdx.x < n_trees) nc.root[threadIdx.x] = a.beam_node_off[b_lo + threadIdx.x];
+            if ((int)threadIdx.x < n_trees) nc.root[threadIdx.x] = ld_early(a.beam_node_off + b_lo + threadIdx.x);
             const int i = threadIdx.x, n = n_lo + i;
             if (i < n_req) {
-                par = a.parent[n];
+                par = ld_early(a.parent + n);
                 if (par >= 0) {
-                    tok = a.token[n];
+                    tok = ld_early(a.token + n);
                     if (par < n_lo || par >= n) { if (writer) report(a.status, DSBD_DEV_BAD_FOREST); tok = -2; }
                     else if (tok < 0 || tok >= a.V) { if (writer) report(a.status, DSBD_DEV_BAD_TOKEN); tok = -2; }
                     else {
-                        zp_tok = a.zp[(int64_t)par * a.stride + tok];
-                        zq_tok = a.zq[(int64_t)par * a.stride + tok];
+                        zp_tok = ld_early(a.zp + (int64_t)par * a.stride + tok);
+                        zq_tok = ld_early(a.zq + (int64_t)par * a.stride + tok);
                     }
                 }
                 nc.parent[i] = (int16_t)((par >= n_lo && par < n) ? par - n_lo : par < 0 ? -1 : -2);
@@ -2240,7 +2245,7 @@ int launch_verify(const VerifyArgs &args, int R, int tiles, cudaStream_t stream)
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     // the clusters may be set up while the dense pass before them drains.  Before griddepcontrol.wait the kernel
-    // reads what the caller gave (forest, widths, logits), after it the statistics: the dense pass lets it start only
+    // reads what the caller gave (forest, widths, logits) from L2, after it the statistics: the dense pass lets it start only
     // when all earlier work in the stream is done
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
@@ -2394,13 +2399,14 @@ k_draft(const __grid_constant__ DraftArgs d) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     uint32_t *hp = reinterpret_cast<uint32_t *>(dyn_smem), *hq = hp + kHistWords;
     const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int b_lo = a.req_beam_off[r], o_lo = d.out_off[r], cap = d.out_off[r + 1] - o_lo;
-    const int W = d.W_r ? d.W_r[r] : d.W;
-    int nA = a.req_beam_off[r + 1] - b_lo, err = 0;
+    // (before the wait as in k_verify: what earlier work left, from L2)
+    const int b_lo = ld_early(a.req_beam_off + r), o_lo = ld_early(d.out_off + r), cap = ld_early(d.out_off + r + 1) - o_lo;
+    const int W = d.W_r ? ld_early(d.W_r + r) : d.W;
+    int nA = ld_early(a.req_beam_off + r + 1) - b_lo, err = 0;
     if (nA > kMaxLive) { err = DSBD_DEV_BAD_FOREST; nA = 0; }
     if (threadIdx.x < nA) {
         sh.A[threadIdx.x] = b_lo + threadIdx.x;
-        score[threadIdx.x] = (double)d.beam_logq[b_lo + threadIdx.x];
+        score[threadIdx.x] = (double)ld_early(d.beam_logq + b_lo + threadIdx.x);
     }
     if (threadIdx.x == 0) { sh.nA = nA; s_err = 0; }
     asm volatile("griddepcontrol.wait;" ::: "memory");

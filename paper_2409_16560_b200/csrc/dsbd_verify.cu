@@ -558,6 +558,11 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
     unsigned long long d;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -587,13 +592,15 @@ __device__ __forceinline__ int item_halves(int n_tiles, int n_warps) {
 // array at kHistWords words, the b arrays at twice that.
 // (ex2.approx flushes results below 2^-126 to zero; a cell enters the sums from 2^-45 on.)
 // kBinned = false: the sums alone, by the same instructions, so that a draw finds the same tile whether the layer took
-// the histogram or a pass on demand.
+// the histogram or a pass on demand; and in *units the total of p - q in units of 2^-60, by a compensated sum, so that the
+// residual mass is as exact as that of the histogram's whole units.  (Whole units, two conversions a cell: a pass 1.5 us longer, the
+// compensated sum 0.3.)
 constexpr float kBinMagic = 12582912.f;                         // 1.5 * 2^23
 constexpr float kBigUnits = 268435456.f;                        // 2^28 units = a cell of 2^-16
 template <bool kBinned>
 __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const float4 (&vq)[4], float k2,
                                                const RowOff &o, float binscale, float half_bin, float top, uint32_t wbase,
-                                               uint32_t over_bits, float &sd, float &sq) {
+                                               uint32_t over_bits, float &sd, float &sq, long long *units) {
     // dl = log2(rho) - half: the half bin (in log2 units) that turns the fma's round-to-nearest into
     // the bin's floor is part of the row offset, so p_beam > q_beam reads dl > -half
     const float bd = ((o.bp - o.bq) + o.dc) - half_bin;
@@ -602,6 +609,7 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
     const unsigned long long k22 = pack2(k2, k2), bd2 = pack2(bd, bd), bp2 = pack2(o.bp, o.bp), bq2 = pack2(o.bq, o.bq);
     const unsigned long long cp2 = pack2(cpu, cpu), cq2 = pack2(cqu, cqu), neg2 = pack2(-1.f, -1.f);
     const unsigned long long bs2 = pack2(binscale, binscale), mg2 = pack2(kBinMagic, kBinMagic);
+    unsigned long long sum = 0ull, rest = 0ull;
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
         float dl[4], pm[4], qm[4], df[4];
@@ -634,8 +642,20 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
                     "@p add.f32 %0, %0, %3;\n\t"
                     "@p add.f32 %1, %1, %4;\n\t}"
                     : "+f"(sd), "+f"(sq) : "f"(dl[c]), "f"(df[c]), "f"(qm[c]), "f"(pass_thr));
-            else sd += dl[c] > pass_thr ? df[c] : 0.f;
-        if (!kBinned) continue;
+            else {
+                df[c] = dl[c] > pass_thr ? df[c] : 0.f;
+                sd += df[c];
+            }
+        if (!kBinned) {
+            // compensated (Kahan), two cells to an instruction
+#pragma unroll
+            for (int c = 0; c < 4; c += 2) {
+                const unsigned long long y = fma2(rest, neg2, pack2(df[c], df[c + 1])), t = add2(sum, y);
+                rest = fma2(y, neg2, fma2(sum, neg2, t));
+                sum = t;
+            }
+            continue;
+        }
         const float big = fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3]));
         if (big >= kBigUnits) {
 #pragma unroll
@@ -663,13 +683,18 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
                 :: "f"(dl[c]), "r"(addr[c]), "r"(__float2uint_rn(pm[c])), "r"(__float2uint_rn(qm[c])), "n"(kHistWords * 4), "f"(pass_thr)
                 : "memory");
     }
+    if (!kBinned) {
+        const float2 t = unpack2(sum), e = unpack2(rest);
+        *units += __double2ll_rn((((double)t.x - (double)e.x) + ((double)t.y - (double)e.y)) * 65536.0);
+    }
 }
 
 // One cluster-wide pass without a histogram: item sums of max(p_beam - s q_beam, 0) over the live rows.
 // kFirst: s = 1, in the arithmetic (and the half-tile items) of the histogram pass; half_bin is that of the layer's histogram.
 // Else: any s, in the arithmetic of the search inside a tile (cell_mass), so that a tile with a sum has a cell that the search
-// finds; whole tiles.  sh.warp_part gets the total of each warp's items as whole numbers: the order in which warps and CTAs add
-// up changes nothing, and a small F keeps its digits; and, unless kFirst, the q mass of the cells with p_beam > s q_beam.
+// finds; whole tiles.  sh.warp_part gets the total of each warp's items as whole numbers, so the order in which warps and CTAs add
+// up changes nothing.  Unless kFirst, in two words, so that a small F keeps its digits, and the q mass of the cells with
+// p_beam > s q_beam.
 // Bound by latency: few clusters make such a pass at a time, a warp takes about 1.8 us a half tile.  Straight-line loads for whole
 // aligned halves.  (The next item prefetched into L2: no difference.  Totals in registers: spills, a call 1 per cent slower.)
 // Functions of their own: the callers would each carry the unrolled loop.
@@ -682,6 +707,7 @@ __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const f
     const int row_items = T * halves, items = sh.nA * row_items;
     if (lane < 3) sh.warp_part[lane][threadIdx.x >> 5] = 0ll;
     __syncwarp();
+    long long units = 0ll;
     for (int item = warp; item < items; item += nwarps) {
         const int i = item / row_items, t = item - i * row_items;
         const int row = sh.A[i];
@@ -706,7 +732,7 @@ __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const f
             }
             if (kFirst) {
                 float sd = 0.f, sq = 0.f;
-                hist_half_tile<false>(vp, vq, k2, ro, 0.f, half_bin, 0.f, 0u, 0u, sd, sq);
+                hist_half_tile<false>(vp, vq, k2, ro, 0.f, half_bin, 0.f, 0u, 0u, sd, sq, &units);
                 res1 += (double)sd;
             } else {
                 auto cell = [&](float vpc, float vqc) {
@@ -726,11 +752,18 @@ __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const f
         const double q = kFirst ? 0.0 : warp_sum((double)q_acc) * (double)kFix;
         if (lane == 0) {
             sums[item] = tot;
-            const long long hi = __double2ll_rn(tot * kSumUnit);
-            sh.warp_part[0][threadIdx.x >> 5] += hi;
-            sh.warp_part[1][threadIdx.x >> 5] += __double2ll_rn((tot * kSumUnit - (double)hi) * kSumUnit);
-            if (!kFirst) sh.warp_part[2][threadIdx.x >> 5] += __double2ll_rn(q);
+            if (!kFirst) {
+                const long long hi = __double2ll_rn(tot * kSumUnit);
+                sh.warp_part[0][threadIdx.x >> 5] += hi;
+                sh.warp_part[1][threadIdx.x >> 5] += __double2ll_rn((tot * kSumUnit - (double)hi) * kSumUnit);
+                sh.warp_part[2][threadIdx.x >> 5] += __double2ll_rn(q);
+            }
         }
+    }
+    if (kFirst) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) units += __shfl_xor_sync(kFull, units, o);
+        if (lane == 0) sh.warp_part[0][threadIdx.x >> 5] = units;
     }
 }
 
@@ -765,6 +798,7 @@ __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, do
         lo += sh.part[n_pass & 1][1][c];
         q += sh.part[n_pass & 1][2][c];
     }
+    if (first) return (double)hi * (1.0 / kSumUnit);
     const double total = ((double)lo * (1.0 / kSumUnit) + (double)hi) * (1.0 / kSumUnit);
     const double rest = (s - (double)s_hi) * ((double)q * kUnfix);
     return rest < total ? total - rest : total;
@@ -808,7 +842,7 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float bins
                 load_half_tile(rq, e0, a.V, false, lane, vq);
             }
             float sd = 0.f, sq = 0.f;
-            hist_half_tile<true>(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sd, sq);
+            hist_half_tile<true>(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sd, sq, nullptr);
             added += __float2ull_rn(fmaf(2.f, sq, sd));
             res1 += (double)sd;
         }

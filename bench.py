@@ -494,6 +494,7 @@ def main():
                     "extra_completion_passes_per_request": float(st[:, 3].mean()),
                     "near_tie_accept_tests": int(st[:, 4].sum()), "consulted_row_pairs_per_request": float(st[:, 5].mean()),
                     "overflowed_histograms": int(st[:, 6].sum()),
+                    "passes_on_demand_per_request": float(st[:, 7].mean()),
                     "output_beams_per_request": float(vout["out_width"].float().mean().item())}
 
     # the dense logits pass alone (the kernel the verify roofline is quoted on)

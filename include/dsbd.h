@@ -223,13 +223,13 @@ typedef struct {
     int32_t *req_error;     /* [R]  0 or a DSBD_DEV_* code                                   */
     int32_t *req_stats;     /* [R*DSBD_REQ_STATS] or NULL, per request: 0 layers verified, 1 accept
                                     tests made, 2 residual masses of the histogram recomputed exactly by a
-                                    pass over the rows, 3 extra passes made for completion draws (layers
-                                    whose width needs no residual mass make their passes on demand and
-                                    count in neither), 4 accept
+                                    pass over the rows, 3 extra passes made for completion draws, 4 accept
                                     tests with |u - ratio| < 1e-5 (near ties), 5 logits row pairs
                                     consulted after the dense pass (live parents summed over the
-                                    verified layers), 6 layers whose histogram overflowed a word and
-                                    fell back to exact passes, 7 reserved (0)                     */
+                                    layers that made a pass over their rows or looked for a warped support),
+                                    6 layers whose histogram overflowed a word and fell back to exact
+                                    passes, 7 passes on demand (layers whose width needs no residual mass
+                                    make one for a rejection, without a histogram; not in 2 or 3)  */
 } dsbd_verify_out_t;
 
 /* One verification step (Algorithm 1 with the dynamic width of Eqs. for P, P~, alpha_j, W_L):

@@ -270,7 +270,7 @@ struct Shared {
     long long warp_part[3][kVWarps], part[2][3][16];
     int n_out, n_fill;                      // output beams so far; p_beam fills left to the whole CTA
     int n_layers, n_tests, n_exact, n_respass;
-    int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows consulted
+    int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows of layers that looked into them
     unsigned long long wtot_p[kVWarps], wtot_q[kVWarps];
     unsigned long long slice_p[16], slice_q[16];   // mass of the bins of every CTA's slice
     unsigned long long above_p[16], above_q[16];   // mass of the bins above every CTA's slice
@@ -2008,7 +2008,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                         if (writer) a.out.node_status[sh.S[i]] = DSBD_NODE_CUT;
                     }
                 sh.W = W;
-                sh.n_rows += sh.nA;
+                if (m >= 1 && (!on_demand || sh.chain_len > 0)) sh.n_rows += sh.nA;
                 ++sh.n_layers;
                 // a residual draw at run position j needs tile sums (a layer of known width has them)
                 sh.res_j = (count < W && j > 1 && !on_demand) ? j : 0;
@@ -2186,7 +2186,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             if (a.out.req_stats) {
                 int32_t *rs = a.out.req_stats + (int64_t)DSBD_REQ_STATS * r;
                 rs[0] = sh.n_layers; rs[1] = sh.n_tests; rs[2] = sh.n_exact; rs[3] = sh.n_respass;
-                rs[4] = sh.n_near; rs[5] = sh.n_rows; rs[6] = sh.n_wrapped; rs[7] = 0;
+                rs[4] = sh.n_near; rs[5] = sh.n_rows; rs[6] = sh.n_wrapped; rs[7] = n_pass - sh.n_exact - sh.n_respass;
             }
         }
         if (sh.err) report(a.status, sh.err);

@@ -338,7 +338,8 @@ def test_layers_of_known_width(V, beams, W_min, W_max):
     zp = (zp + rng.normal(0, 1.0, zp.shape)).astype(np.float32)
     prm.update(W_min_r=None, W_min=W_min, W_max=W_max)
     dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
-    exempt = decisions = 0
+    exempt = decisions = on_demand = 0
+    n0 = np.concatenate([forest["beam_node_off"][forest["req_beam_off"][:-1]], [forest["N"]]])
     for step in range(12):
         prm["step"] = step
         gpu, status = run_gpu_verify(forest, prm, *dev)
@@ -346,7 +347,15 @@ def test_layers_of_known_width(V, beams, W_min, W_max):
         e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
         exempt += e
         decisions += d
+        # a pass takes a rejection, and the rows are looked into by layers that make one or build a histogram
+        st = gpu["req_stats"].reshape(-1, 8)
+        rejected = np.array([(gpu["node_status"][a:b] == binding.NODE_REJECTED).sum() for a, b in zip(n0[:-1], n0[1:])])
+        assert np.all(st[:, 7] <= rejected)
+        assert np.all(st[rejected == 0][:, [5, 7]] == 0)
+        on_demand += int(st[:, 7].sum())
     check_exempt(exempt, decisions)
+    if beams <= W_min:
+        assert on_demand > 0
 
 
 @pytest.mark.parametrize("V,beams,seeds", [(128256, 2, 3), (50257, 2, 2), (1025, 2, 1)])

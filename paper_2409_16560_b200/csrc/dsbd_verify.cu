@@ -1330,8 +1330,14 @@ __device__ void finish_supports(WarpScratch &ws, bool have_q, int lane) {
 #define TS(slot) do {} while (0)
 #endif
 
-// Drafts behind the first rejection of a layer of known width up to which its residual masses are computed on demand.
-constexpr int kOnDemandLeft = 3;
+// Drafts behind the first rejection of a layer of known width up to which its residual masses are computed on demand: a pass
+// for that rejection and at most one for each of them, against one histogram, and a pass more where the layer ends in a residual
+// draw behind a second rejection.  A histogram costs about 1.9 passes where a warp has eight tiles of a pass and 2.8 where it
+// has one or two, its merge and chain being as long for few tiles.  Layers of three and four drafts, mean of the benchmark's
+// distributions with as many accepts and with fewer, against a histogram for every rejection: 64 requests of 128256
+// tokens up to 2 drafts 1.03 and 1.01 times as fast, up to 3 0.97 and 0.93; 160 of 32000 1.05 and 1.03, 1.00 and 0.95; 16
+// of 128256 1.16 and 1.11, 1.20 and 1.14; one of 32000 1.12 and 1.07, 1.14 and 1.09.
+__device__ __forceinline__ int on_demand_left(int n_tiles, int n_warps) { return n_tiles <= 2 * n_warps ? 3 : 2; }
 
 // dynamic shared memory of k_verify: the histogram of a layer as four 32-bit arrays while it is
 // being built, then (over the same bytes) this CTA's slice of the suffix sums of its p and q mass
@@ -1804,10 +1810,10 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         } else if (m >= 1 && !sh.err && !a.select_mode && (m <= W_min || W_max <= W_min)) {
             // ---- the width is W_min whatever the residual masses are (W~ <= m): the drafts are tested at once.  Up to
             // the first rejection that takes no pass over the rows at all, and every rejection one pass, without a histogram,
-            // whose sums also serve the completion draw.  With more than kOnDemandLeft drafts behind the first
-            // rejection the histogram is the better way: one pass of it costs two to three of these.  (Two live rows of
-            // 128256, 4 CTAs: a layer of accepted drafts 5 us instead of 38; a rejection 16 instead of 37.  64 requests x
-            // 8 rows 986 -> 922 us for the call, 16 ragged requests 222 -> 174, one request of V = 32000 60 -> 52.) ----
+            // whose sums also serve the completion draw.  With more drafts behind the first rejection (on_demand_left) the
+            // histogram is the better way.  (Two live rows of 128256, 4 CTAs: a layer of accepted drafts 5 us instead of 38; a
+            // rejection 16 instead of 37.  Calls, W_min = 2: 64 requests x 8 rows 978 -> 907 us, 16 ragged requests 222 -> 164,
+            // one request of V = 32000 61 -> 53.) ----
             if (warp == 0) {
                 draft_tests(l, m);
                 const int W = W_min < W_max ? W_min : W_max;
@@ -1818,7 +1824,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     if (rejects) first = base + __ffs(rejects) - 1;
                 }
                 if (lane == 0) {
-                    sh.on_demand = first >= W || m - 1 - first <= kOnDemandLeft;
+                    sh.on_demand = first >= W || m - 1 - first <= on_demand_left(sh.nA * a.T, n_cta * kVWarps);
                     sh.need_exact = 0;
                     if (sh.on_demand) accept_loop(W, true);
                 }

@@ -330,8 +330,8 @@ def test_requests_around_the_node_cache_and_half_tiles(beams, gamma, V):
                                                  (9000, 40, 3, 3), (33000, 4, 4, 9), (50257, 3, 3, 3)])
 def test_layers_of_known_width(V, beams, W_min, W_max):
     """Layers whose width does not depend on the residual masses (at most W_min drafts, or W_min = W_max): no rejection,
-    a rejection with none, three, four and many drafts behind it (passes on demand up to three, the histogram from
-    four on), several rejections in a row, accepts between them; clusters of 1 to 16 CTAs, whole and half tiles, vocabularies of
+    a rejection with none, three, four and many drafts behind it (passes on demand up to two or three, else the
+    histogram), several rejections in a row, accepts between them; clusters of 1 to 16 CTAs, whole and half tiles, vocabularies of
     one token, one more than a tile and rows that are not aligned."""
     rng = np.random.default_rng(V + beams)
     forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=4, V=V, gamma=3, max_w=beams, min_w=beams)
@@ -451,6 +451,42 @@ def test_inputs_written_right_before_the_call(V, R):
     for k in range(24):
         for name in alone[k]:
             assert torch.equal(alone[k][name], behind[k][name]), (k, name)
+
+
+@pytest.mark.parametrize("R,pattern,W,passes", [(160, "RRRA", 1, 0), (160, "ARRA", 2, 2), (160, "AARR", 3, 2), (160, "RARA", 1, 0),
+                                                (4, "RRRA", 1, 3), (4, "RRRR", 1, 4), (4, "RARR", 2, 2), (4, "RRRRA", 1, 0),
+                                                (4, "AAAA", 4, 0), (4, "AARR", 1, 0)])
+def test_passes_on_demand_are_few(R, pattern, W, passes):
+    """One layer of known width whose drafts are accepted (A: far more likely under the large model) or rejected (R: impossible
+    under it) by construction.  A rejection behind a rejection takes a pass, and so does the first; one behind an accept has the
+    residual mass already.  With more than two drafts (three, where a warp has at most two tiles: 4 requests here) behind the
+    first rejection the layer takes the histogram instead; it ends with W accepts."""
+    V, m = 16400, len(pattern)
+    forest, _, _ = inputs.build_forest(dict(R=R, W=m, tree=inputs._chain(1), prefix=(1, 1)), np.random.default_rng(1))
+    rng = np.random.default_rng(V + R)
+    zq = rng.normal(0, 1.5, size=(forest["N"], V)).astype(np.float32)
+    zp = (zq + rng.normal(0, 1.0, size=zq.shape)).astype(np.float32)
+    token = np.zeros(forest["N"], np.int32)
+    drafts = np.nonzero(forest["parent"] >= 0)[0]
+    for i, n in enumerate(drafts):
+        row, token[n] = forest["parent"][n], rng.integers(0, V)
+        accept = pattern[i % m] == "A"
+        zp[row, token[n]] = 9.0 if accept else -60.0
+        zq[row, token[n]] = -20.0 if accept else 1.0
+    forest["token"] = token
+    rp = rq = np.zeros(forest["B"], np.float32)
+    prm = dict(V=V, temperature=1.0, thresh=0.7, W_min=W, W_max=W, W_nom=W, seed=3, step=0, top_k=0, top_p=1.0)
+    gpu, status = run_gpu_verify(forest, prm, *(torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)))
+    assert status == 0
+    e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+    check_exempt(e, d)
+    seen = {"A": binding.NODE_ACCEPTED, "R": binding.NODE_REJECTED}
+    want = [seen[c] for c in pattern]
+    stop = [i for i in range(m) if pattern[:i + 1].count("A") == W]
+    if stop:
+        want[stop[0] + 1:] = [binding.NODE_CUT] * (m - 1 - stop[0])
+    assert np.array_equal(gpu["node_status"][drafts].reshape(R, m), np.tile(want, (R, 1)))
+    assert np.all(gpu["req_stats"].reshape(R, -1)[:, 7] == passes)
 
 
 @pytest.mark.parametrize("V", [2000, 40000])

@@ -85,20 +85,16 @@ __device__ __forceinline__ void load_tile(const float *row, int e0, int V, bool 
     }
 }
 
-__device__ __forceinline__ void load_half_tile(const float *__restrict__ row, int e0, int V, bool aligned,
-                                               int lane, float4 (&v)[4]) {
+// Half a tile of a row that is not aligned, or ends in it (whole aligned ones are loaded where they are used).
+__device__ __forceinline__ void load_half_tile(const float *__restrict__ row, int e0, int V, int lane, float4 (&v)[4]) {
     const float ninf = -INFINITY;
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
         const int e = e0 + it * 128 + lane * 4;
-        if (aligned && e + 3 < V) {
-            v[it] = ldg_stream(reinterpret_cast<const float4 *>(row + e));
-        } else {
-            v[it].x = e < V ? __ldg(row + e) : ninf;
-            v[it].y = e + 1 < V ? __ldg(row + e + 1) : ninf;
-            v[it].z = e + 2 < V ? __ldg(row + e + 2) : ninf;
-            v[it].w = e + 3 < V ? __ldg(row + e + 3) : ninf;
-        }
+        v[it].x = e < V ? __ldg(row + e) : ninf;
+        v[it].y = e + 1 < V ? __ldg(row + e + 1) : ninf;
+        v[it].z = e + 2 < V ? __ldg(row + e + 2) : ninf;
+        v[it].w = e + 3 < V ? __ldg(row + e + 3) : ninf;
     }
 }
 
@@ -727,8 +723,8 @@ __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const f
 #pragma unroll
                 for (int it = 0; it < 4; ++it) vq[it] = ldg_stream(reinterpret_cast<const float4 *>(rq + e0 + it * 128) + lane);
             } else {
-                load_half_tile(rp, e0, V, false, lane, vp);
-                load_half_tile(rq, e0, V, false, lane, vq);
+                load_half_tile(rp, e0, V, lane, vp);
+                load_half_tile(rq, e0, V, lane, vq);
             }
             if (kFirst) {
                 float sd = 0.f, sq = 0.f;
@@ -838,8 +834,8 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float bins
 #pragma unroll
                 for (int it = 0; it < 4; ++it) vq[it] = ldg_stream(reinterpret_cast<const float4 *>(rq + e0 + it * 128) + lane);
             } else {
-                load_half_tile(rp, e0, a.V, false, lane, vp);
-                load_half_tile(rq, e0, a.V, false, lane, vq);
+                load_half_tile(rp, e0, a.V, lane, vp);
+                load_half_tile(rq, e0, a.V, lane, vq);
             }
             float sd = 0.f, sq = 0.f;
             hist_half_tile<true>(vp, vq, a.k2, ro, binscale, half_bin, top, wbase, over_bits, sd, sq, nullptr);

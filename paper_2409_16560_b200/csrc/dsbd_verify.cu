@@ -690,12 +690,14 @@ __device__ __forceinline__ void hist_half_tile(const float4 (&vp)[4], const floa
 // Else: any s, in the arithmetic of the search inside a tile (cell_mass), so that a tile with a sum has a cell that the search
 // finds; whole tiles.  sh.warp_part gets the total of each warp's items as whole numbers, so the order in which warps and CTAs add
 // up changes nothing.  Unless kFirst, in two words, so that a small F keeps its digits, and the q mass of the cells with
-// p_beam > s q_beam.
-// Bound by latency: few clusters make such a pass at a time, a warp takes about 1.8 us a half tile.  Straight-line loads for whole
-// aligned halves.  (The next item prefetched into L2: no difference.  Totals in registers: spills, a call 1 per cent slower.)
+// p_beam > s q_beam.  kTotal = false: the item sums alone.
+// Bound by latency where a cluster is alone with its pass (a warp takes about 1.8 us a half tile), by issue where many are at it:
+// 54 requests x 7 rows of 90496, 18 of which make a pass for a draw, 198 us the call with totals that nobody reads, 194 without.
+// Straight-line loads for whole aligned halves.  (The next item prefetched into L2: no difference.  Totals in registers: spills,
+// a call 1 per cent slower.)
 // Functions of their own: the callers would each carry the unrolled loop.
 constexpr double kSumUnit = 1152921504606846976.0;               // 2^60
-template <bool kFirst>
+template <bool kFirst, bool kTotal>
 __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const float *__restrict__ zq, int64_t stride,
                                                 int V, int T, float k2, Shared &sh, float s, float half_bin, double *sums,
                                                 int warp, int nwarps, int halves) {
@@ -731,24 +733,32 @@ __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const f
                 hist_half_tile<false>(vp, vq, k2, ro, 0.f, half_bin, 0.f, 0u, 0u, sd, sq, &units);
                 res1 += (double)sd;
             } else {
-                auto cell = [&](float vpc, float vqc) {
-                    float q;
-                    const float d = cell_mass(vpc, vqc, k2, ro, s, &q);
-                    acc += d;
-                    q_acc += d > 0.f ? q : 0.f;
-                };
+                // cell_mass, two cells to an instruction around the exponentials
+                const unsigned long long k22 = pack2(k2, k2), bp2 = pack2(ro.bp, ro.bp), bq2 = pack2(ro.bq, ro.bq);
+                const unsigned long long cp2 = pack2(ro.cp, ro.cp), cq2 = pack2(ro.cq, ro.cq), s2 = pack2(-s, -s);
 #pragma unroll
-                for (int it = 0; it < 4; ++it) {
-                    cell(vp[it].x, vq[it].x); cell(vp[it].y, vq[it].y);
-                    cell(vp[it].z, vq[it].z); cell(vp[it].w, vq[it].w);
-                }
+                for (int it = 0; it < 4; ++it)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float2 pe = unpack2(fma2(h ? pack2(vp[it].z, vp[it].w) : pack2(vp[it].x, vp[it].y), k22, bp2));
+                        const float2 qe = unpack2(fma2(h ? pack2(vq[it].z, vq[it].w) : pack2(vq[it].x, vq[it].y), k22, bq2));
+                        const unsigned long long p2 = mul2(pack2(exp2f(pe.x), exp2f(pe.y)), cp2);
+                        const unsigned long long q2 = mul2(pack2(exp2f(qe.x), exp2f(qe.y)), cq2);
+                        const float2 d = unpack2(fma2(s2, q2, p2)), q = unpack2(q2);
+                        acc += fmaxf(d.x, 0.f);
+                        acc += fmaxf(d.y, 0.f);
+                        if (kTotal) {
+                            q_acc += d.x > 0.f ? q.x : 0.f;
+                            q_acc += d.y > 0.f ? q.y : 0.f;
+                        }
+                    }
             }
         }
         const double tot = kFirst ? warp_sum(res1) * kUnfix : warp_sum((double)acc);
-        const double q = kFirst ? 0.0 : warp_sum((double)q_acc) * (double)kFix;
+        const double q = kFirst || !kTotal ? 0.0 : warp_sum((double)q_acc) * (double)kFix;
         if (lane == 0) {
             sums[item] = tot;
-            if (!kFirst) {
+            if (!kFirst && kTotal) {
                 const long long hi = __double2ll_rn(tot * kSumUnit);
                 sh.warp_part[0][threadIdx.x >> 5] += hi;
                 sh.warp_part[1][threadIdx.x >> 5] += __double2ll_rn((tot * kSumUnit - (double)hi) * kSumUnit);
@@ -774,8 +784,9 @@ __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, do
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float s_hi = (float)s;
     const int w = cta_rank * kVWarps + warp, nw = n_cta * kVWarps;
-    if (first) residual_pass<true>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, half_bin, sums, w, nw, halves);
-    else residual_pass<false>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, 0.f, sums, w, nw, halves);
+    if (first) residual_pass<true, true>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, half_bin, sums, w, nw, halves);
+    else if (want_total) residual_pass<false, true>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, 0.f, sums, w, nw, halves);
+    else residual_pass<false, false>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, 0.f, sums, w, nw, halves);
     if (!want_total) {
         cluster.sync();
         return 0.0;

@@ -34,7 +34,7 @@ UNIT = "nodes/s"
 # (the traffic is proportional to the number of requests).  verify_step_total = the dense pass plus the
 # per-request kernel, which re-reads the live rows (unwarped; with a top-k 0.018e9).
 NCU_TRAFFIC_BYTES = {"C5": {"forest_attention": 8.776e9, "verify_dense_pass": 4.748e9,
-                            "verify_step_total": 4.748e9 + 0.729e9}}
+                            "verify_step_total": 4.748e9 + 0.707e9}}
 
 
 def _peaks():

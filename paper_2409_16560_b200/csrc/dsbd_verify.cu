@@ -15,7 +15,8 @@
 //                  residual masses c_{j+1} = F(s_j) of the layer follow without touching the
 //                  rows again; the acceptance-count recursion; the accept loop; the
 //                  inverse-CDF completion draws.  A layer whose width does not depend on the residual
-//                  masses tests its drafts at once and makes a plain pass for each rejection.
+//                  masses tests its drafts at once and, unless many are left behind the first
+//                  rejection, makes a plain pass for each rejection in place of the histogram.
 //
 // The residual chain uses the closed form of the paper's recursion p_{k+1} = norm(max(p_k -
 // q_beam, 0)):  with F(s) = sum max(p_beam - s q_beam, 0), c_1 = 1, s_0 = 0, s_j = s_{j-1} + c_j
@@ -1351,7 +1352,7 @@ __device__ __forceinline__ int on_demand_left(int n_tiles, int n_warps) { return
 constexpr size_t kVerifyDynSmem = kHistArrays * sizeof(uint32_t) * kHistWords;
 
 // Two instances, with warped joints and without: neither carries the other's code, whose registers it would spill around
-// (64 requests x 8 rows of 128256 with top-k 10: the call 781 -> 772 us).
+// (64 requests x 8 rows of 128256 with top-k 10: a call 781 us as one kernel, 772 as two; unwarped calls alike).
 template <bool kWarped>
 __global__ void __launch_bounds__(kVThreads, 2)
 k_verify(const __grid_constant__ VerifyArgs a) {

@@ -498,7 +498,12 @@ def test_histograms_with_a_layer_of_known_width_between(V):
     zq = (zp + rng.normal(0, 0.4, zp.shape)).astype(np.float32)      # most drafts are accepted
     prm.update(W_min_r=None, W_min=2)
     dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
-    exempt = decisions = deep = 0
+    depth = np.zeros(forest["N"], np.int64)
+    for n, par in enumerate(forest["parent"]):
+        depth[n] = 0 if par < 0 else depth[par] + 1
+    n0 = np.concatenate([forest["beam_node_off"][forest["req_beam_off"][:-1]], [forest["N"]]])
+    tested = (binding.NODE_ACCEPTED, binding.NODE_REJECTED, binding.NODE_CUT)
+    exempt = decisions = between = 0
     for step in range(16):
         prm.update(step=step, thresh=0.7 + 0.015 * step)
         gpu, status = run_gpu_verify(forest, prm, *dev)
@@ -506,9 +511,12 @@ def test_histograms_with_a_layer_of_known_width_between(V):
         e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
         exempt += e
         decisions += d
-        deep += int((gpu["l_last"] >= 3).sum())
+        for r in np.nonzero(gpu["l_last"] >= 3)[0]:
+            d, st = depth[n0[r]:n0[r + 1]], gpu["node_status"][n0[r]:n0[r + 1]]
+            drafts = [int((np.isin(st, tested) & (d == l)).sum()) for l in (1, 2, 3)]
+            between += drafts[0] > 2 and drafts[1] <= 2 and drafts[2] > 2      # W_min = 2
     check_exempt(exempt, decisions)
-    assert deep > 0
+    assert between > 0
 
 
 @pytest.mark.parametrize("V", [1000, 2000, 4000, 8000, 32000])

@@ -163,11 +163,13 @@ k_tile_stats(const float *zp, const float *zq, int64_t stride, int V, int T, int
 // log-sum-exp of a tempered row from its tile statistics, by one warp (same value on every lane;
 // the order of the sums depends on T only).
 __device__ __forceinline__ double row_lse(const TileStat *s, int T, double inv_tau, int lane) {
-    double mx = -INFINITY;
-    for (int t = lane; t < T; t += 32) mx = fmax(mx, (double)s[t].mx);
-    mx = warp_max(mx);
+    float top = -INFINITY;
+#pragma unroll 4
+    for (int t = lane; t < T; t += 32) top = fmaxf(top, s[t].mx);
+    const double mx = (double)warp_max(top);
     double acc = 0.0;
     if (mx > -INFINITY)
+#pragma unroll 1
         for (int t = lane; t < T; t += 32)
             if (s[t].sum > 0.f) acc += (double)s[t].sum * exp(((double)s[t].mx - mx) * inv_tau);
     acc = warp_sum(acc);
@@ -241,8 +243,12 @@ struct VerifyArgs {
     int out_stride;
 };
 
+constexpr int kBins = 4096;
+constexpr int kOverSlots = 256;                   // copies of the last bin (rho beyond the last edge): one per
+                                                  // warp and half-warp lane, so that none collects enough to wrap
+
 struct Shared {
-    int nA, m, W, count, done, chain_len, err;
+    int nA, m, W, count, chain_len, err;         // m: -1 if too many
     int A[kMaxLive];
     int S[kMaxLive];
     int S_parent_idx[kMaxLive];
@@ -261,20 +267,30 @@ struct Shared {
     double col_a[kMaxLive + 1], col_b[kMaxLive + 1];
     double tail[kMaxLive + 2];
     int bank, halves, need_exact, res_j, run_j, chain_pos;
+    int n_draw;                             // completion draws of the request
+    float binscale[kMaxLive + 1];           // by m: bins of a layer's histogram to a power of two
     int on_demand, next_i;                  // a layer of known width: its passes are made when the accept loop asks
     // sums of an exact pass, in units of 2^-60, 2^-120 (what the first leaves) and 2^-44 (q): of this CTA's warps; of every
     // CTA, two passes in turn
     long long warp_part[3][kVWarps], part[2][3][16];
-    int n_out, n_fill;                      // output beams so far; p_beam fills left to the whole CTA
+    int n_out;                              // output beams
     int n_layers, n_tests, n_exact, n_respass;
     int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows of layers that looked into them
-    unsigned long long wtot_p[kVWarps], wtot_q[kVWarps];
-    unsigned long long slice_p[16], slice_q[16];   // mass of the bins of every CTA's slice
-    unsigned long long above_p[16], above_q[16];   // mass of the bins above every CTA's slice
-    unsigned long long w_tot[2][10];        // per bank, sums of one histogram pass: see histogram_pass / hist_fold_over
-    int n_wrapped;                          // layers where a w word of the histogram wrapped
-    double rho[kMaxLive], uu[kMaxLive];     // per live draft: p_beam/q_beam and its uniform
+    unsigned long long wtot[2][kVWarps], over[2][kOverSlots / 32];   // mass (p, q) of every warp's bins and copies of the last bin
+    unsigned long long added;               // mass that this CTA's histogram pass added (p and q), by floating-point sums
+    int wrapped;                            // a w word of this CTA's histogram wrapped
+    int n_wrapped;                          // layers where one did
+#ifdef DSBD_PHASE_TIMING
+    unsigned long long *ts, *ts_end;        // next and last time stamp of the CTA that writes
+#endif
+    double rho[kMaxLive], uu[kMaxLive];     // per live draft: p_beam/q_beam and its uniform (before: its log-probs under p, q)
 };
+
+#ifdef DSBD_PHASE_TIMING
+#define TS(slot) do { if (threadIdx.x == 0 && sh.ts) { unsigned long long t_; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_)); *sh.ts = ((unsigned long long)(slot) << 48) | (t_ & 0xFFFFFFFFFFFFull); if (sh.ts < sh.ts_end) ++sh.ts; } } while (0)
+#else
+#define TS(slot) do {} while (0)
+#endif
 
 // mass of one cell of the residual max(p_beam - s q_beam, 0); s == 0 gives p_beam
 struct RowOff { float bp, bq, cp, cq, dc; };
@@ -298,73 +314,85 @@ __device__ __forceinline__ RowOff row_off(const Shared &sh, int i) {
     return RowOff{sh.bp[i], sh.bq[i], sh.cp[i], sh.cq[i], (float)(sh.rp[i] - sh.rq[i])};
 }
 
-// Inverse-CDF search over tile masses (canonical order).  mass(i) must be the same on every
-// lane.  Returns the tile holding the first cell whose running sum reaches the target, and the
-// target minus the mass before that tile; if rounding leaves the target beyond the total, the last
-// tile with mass.  -1 if there is no mass at all.  The target is u * total when of_total, else u.
-// Every round cuts the range by 32: a lane sums its share (its loads are independent, one memory
-// latency a round instead of one per 32 tiles), the lanes' sums are scanned, one lane is chosen.
-template <class F>
-__device__ int locate_tile(F mass, int n, double u, bool of_total, int lane, double *rest) {
-    int lo = 0, len = n;
-    double target = u;
+// A value that the compiler takes for a new one: keeps it from making copies of a loop for its first round or for a flag.
+__device__ __forceinline__ void one_copy(int &x) { asm volatile("" : "+r"(x)); }
+
+// Inverse-CDF search over n weights in shared memory, by one warp.  Returns the first index whose running sum reaches the
+// target and leaves in target what that takes off the sum before it; if rounding leaves the target beyond the total, the last
+// index with mass (open: n, and the total taken off, where more weights follow).  -1 if there is no mass at all.  The target
+// is target * total when of_total.  Every round cuts the range by 32: a lane sums its share, the lanes' sums are
+// scanned, one lane is chosen.
+// One copy for all searches of a kernel, over weights that its callers have put side by side: text is what a draw waits for
+// (a search of its own in global memory for each kind of weight, unrolled: 24 KB, and 17 KB for the search inside a tile).
+__device__ __noinline__ int locate(const double *w, int n, double &target, bool of_total, bool open, int lane) {
+    int lo = 0, len = n, scale = of_total, go_on = open;
+#pragma unroll 1
     while (true) {
+        one_copy(scale); one_copy(go_on);
         const int per = (len + 31) >> 5, i0 = lo + lane * per, i1 = min(i0 + per, lo + len);
         double v = 0.0;
-#pragma unroll 4
-        for (int i = i0; i < i1; ++i) v += mass(i);
+#pragma unroll 1
+        for (int i = i0; i < i1; ++i) v += w[i];
         const double incl = warp_scan(v, lane);
-        if (of_total) { target = u * __shfl_sync(kFull, incl, 31); of_total = false; }
+        const double total = __shfl_sync(kFull, incl, 31);
+        if (scale) target *= total;
+        scale = 0;
         const unsigned pos = __ballot_sync(kFull, v > 0.0);
-        if (!pos) return -1;
         const unsigned hits = __ballot_sync(kFull, v > 0.0 && incl >= target);
+        if (!hits && go_on) { target -= total; return n; }
+        if (!pos) return -1;
         const int l = hits ? __ffs(hits) - 1 : 31 - __clz(pos);
         target -= __shfl_sync(kFull, incl - v, l);
         lo += l * per;
         len = min(per, len - l * per);
-        if (per == 1) { *rest = target; return lo; }
+        go_on = 0;
+        if (per == 1) return lo;
     }
 }
 
-// Inverse-CDF search inside one tile of row `row` (and its q row when s > 0): the first
+// Inverse-CDF search inside one tile of row `row` (and its q row when s > 0), by one warp: the first
 // token whose running mass reaches `target`, else the last token with mass.  -1: no mass.
-// A lane sums 32 consecutive tokens (two batches of independent loads), then the lanes take the 32 tokens
-// of the lane that was hit.
+// mass: 33 x 32 words of shared memory.  All sectors of the tile are asked for at once; then the lanes take the tokens side by side,
+// and each sums 32 consecutive ones.
+constexpr int kTokWords = 33 * 32;
 __device__ __noinline__ int locate_token(const float *__restrict__ rp, const float *__restrict__ rq, int V, float k2,
-                                         int t, const RowOff ro, float s, double target, int lane) {
-    const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
-    const int e0 = t * kTile + lane * 32;
-    float q;
-    auto mass = [&](float zp, float zq) { return s > 0.f ? cell_mass(zp, zq, k2, ro, s, &q) : exp2f(fmaf(zp, k2, ro.bp)) * ro.cp; };
-    double v = 0.0;
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-        float4 zp[4], zq[4];
+                                         int t, const RowOff ro, float s, double target, int lane, float *mass) {
+    const int e0 = t * kTile, n = min(kTile, V - e0);
+    rp += e0; rq += e0;
+    const bool res = s > 0.f;
+    float first_of[8];                               // (of a sector; all in flight together)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int e = e0 + half * 16 + i * 4;
-            zq[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (al && e + 3 < V) {
-                zp[i] = __ldg(reinterpret_cast<const float4 *>(rp + e));
-                if (s > 0.f) zq[i] = __ldg(reinterpret_cast<const float4 *>(rq + e));
-            } else {
-                const float ninf = -INFINITY;
-                zp[i].x = e < V ? __ldg(rp + e) : ninf;         zp[i].y = e + 1 < V ? __ldg(rp + e + 1) : ninf;
-                zp[i].z = e + 2 < V ? __ldg(rp + e + 2) : ninf; zp[i].w = e + 3 < V ? __ldg(rp + e + 3) : ninf;
-                if (s > 0.f) {
-                    zq[i].x = e < V ? __ldg(rq + e) : ninf;         zq[i].y = e + 1 < V ? __ldg(rq + e + 1) : ninf;
-                    zq[i].z = e + 2 < V ? __ldg(rq + e + 2) : ninf; zq[i].w = e + 3 < V ? __ldg(rq + e + 3) : ninf;
-                }
-            }
+    for (int i = 0; i < 4; ++i) {
+        const int e = (i * 32 + lane) * 8;
+        first_of[i] = e < n ? __ldg(rp + e) : 0.f;
+        first_of[4 + i] = res && e < n ? __ldg(rq + e) : 0.f;
+    }
+    asm volatile("" :: "f"(first_of[0]), "f"(first_of[1]), "f"(first_of[2]), "f"(first_of[3]), "f"(first_of[4]), "f"(first_of[5]),
+                       "f"(first_of[6]), "f"(first_of[7]));
+#pragma unroll 1
+    for (int i0 = 0; i0 < 32; i0 += 8) {
+        float zp[8], zq[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int e = (i0 + i) * 32 + lane;
+            zp[i] = e < n ? __ldg(rp + e) : -INFINITY;
+            zq[i] = res && e < n ? __ldg(rq + e) : -INFINITY;
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v += (double)mass(zp[i].x, zq[i].x); v += (double)mass(zp[i].y, zq[i].y);
-            v += (double)mass(zp[i].z, zq[i].z); v += (double)mass(zp[i].w, zq[i].w);
+        for (int i = 0; i < 8; ++i) {
+            float q, m = exp2f(fmaf(zp[i], k2, ro.bp)) * ro.cp;
+            if (res) m = cell_mass(zp[i], zq[i], k2, ro, s, &q);
+            mass[(i0 + i) * 33 + lane] = m;
         }
     }
+    __syncwarp();
+    double v = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < 32; ++i) v += (double)mass[lane * 33 + i];
     int first = 0;                                               // the hit lane's first token
+#pragma unroll 1
     for (int level = 0; ; ++level) {
+        one_copy(level);
         const double incl = warp_scan(v, lane);
         const unsigned pos = __ballot_sync(kFull, v > 0.0);
         if (!pos) return -1;
@@ -372,9 +400,8 @@ __device__ __noinline__ int locate_token(const float *__restrict__ rp, const flo
         const int l = hits ? __ffs(hits) - 1 : 31 - __clz(pos);
         if (level) return first + l;
         target -= __shfl_sync(kFull, incl - v, l);
-        first = t * kTile + l * 32;
-        const int e = first + lane;
-        v = e < V ? (double)mass(__ldg(rp + e), s > 0.f ? __ldg(rq + e) : 0.f) : 0.0;
+        first = e0 + l * 32;
+        v = (double)mass[l * 33 + lane];
     }
 }
 
@@ -391,7 +418,7 @@ struct NodeCache {
 
 // Writes output beam number `index` of request r (the caller has checked the slot range).  nc: the
 // request's node cache or nullptr; n_lo: first node of the request.
-__device__ void emit_at(const VerifyArgs &a, int r, int index, int parent, int node, int tok, int source,
+__device__ __forceinline__ void emit_at(const VerifyArgs &a, int r, int index, int parent, int node, int tok, int source,
                         const NodeCache *nc, int n_lo) {
     const int s = a.out.out_off[r] + index;
     const float zp = a.zp[(int64_t)parent * a.stride + tok], zq = a.zq[(int64_t)parent * a.stride + tok];
@@ -407,6 +434,7 @@ __device__ void emit_at(const VerifyArgs &a, int r, int index, int parent, int n
         int root = parent;
         while (a.parent[root] >= 0) root = a.parent[root];
         const int hi = a.req_beam_off[r + 1];
+#pragma unroll 1
         for (int b = lo; b < hi; ++b) if (a.beam_node_off[b] == root) beam = b;
         lse_p = a.lse[parent]; lse_q = a.lse[a.N + parent]; score_p = a.score[parent]; score_q = a.score[a.N + parent];
     }
@@ -423,12 +451,15 @@ __device__ void emit_at(const VerifyArgs &a, int r, int index, int parent, int n
 // Natural log of the softmax of n scores, by one warp (lanes over the scores).
 __device__ __forceinline__ void log_softmax_warp(const double *s, int n, int lane, double *out) {
     double mx = -INFINITY;
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) mx = fmax(mx, s[i]);
     mx = warp_max(mx);
     double t = 0.0;
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) t += exp(s[i] - mx);
     t = warp_sum(t);
     const double lt = log(t);
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) out[i] = (s[i] - mx) - lt;
     __syncwarp();
 }
@@ -441,6 +472,7 @@ __device__ void live_weights(const VerifyArgs &a, Shared &sh, int model, const d
     double *lw = model ? sh.lwq : sh.lwp;
     log_softmax_warp(scores, sh.nA, lane, lw);
     const double *lse = nc ? (model ? nc->lse_q : nc->lse_p) - n_lo : a.lse + (int64_t)model * a.N;
+#pragma unroll 1
     for (int i = lane; i < sh.nA; i += 32) {
         if (!model) sh.wp[i] = exp(lw[i]);
         split_offset((lw[i] - lse[sh.A[i]]) * (1.0 / kLn2), model ? &sh.bq[i] : &sh.bp[i],
@@ -455,17 +487,19 @@ __device__ void live_weights(const VerifyArgs &a, Shared &sh, int model, const d
 __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop) {
     if (lane == 0) {
         double none = 1.0;
+        sh.col_a[0] = 1.0;
+        sh.tail[0] = 1.0;
+#pragma unroll 2
         for (int i = 1; i <= m; ++i) {
             sh.first[i] = sh.alpha[i] * none;
             none *= (1.0 - sh.alpha[i]);
             sh.col_a[i] = none;                    // P(n, 0) = prod_{j<=n}(1 - alpha_j)
         }
-        sh.col_a[0] = 1.0;
-        sh.tail[0] = 1.0;
     }
     __syncwarp();
     double *prev = sh.col_a, *cur = sh.col_b;
     double below = 0.0;
+#pragma unroll 1
     for (int k = 0; k <= m; ++k) {
         // prev = P(., k); record tail
         below += prev[m];
@@ -473,12 +507,15 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
         if (k == m) break;
         // tails only fall: past the first one below the threshold, or past the cap, nothing changes W
         if (k_stop >= 0 && (1.0 - below < thresh || k + 1 >= k_stop)) {
+#pragma unroll 1
             for (int K = k + 2 + lane; K <= m + 1; K += 32) sh.tail[K] = 0.0;
             break;
         }
+#pragma unroll 1
         for (int n = lane; n <= m; n += 32) {
             double acc = 0.0;
             if (n >= k + 1)
+#pragma unroll 2
                 for (int i = 1; i <= n; ++i) acc += sh.first[i] * prev[n - i];
             cur[n] = acc;                          // P(n, k+1), zero for n < k+1
         }
@@ -487,6 +524,7 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
     }
     __syncwarp();
     int wt = 0;
+#pragma unroll 1
     for (int K = 0; K <= m; ++K) if (sh.tail[K] >= thresh) wt = K;
     if (lane == 0) sh.tail[m + 1] = 0.0;
     return wt;
@@ -518,9 +556,6 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
 // all words; a difference marks the layer, whose residual masses are
 // then all computed by exact passes over the rows.
 // ---------------------------------------------------------------------------------------
-constexpr int kBins = 4096;
-constexpr int kOverSlots = 256;                   // copies of the last bin (rho beyond the last edge): one per
-                                                  // warp and half-warp lane, so that none collects enough to wrap
 constexpr int kHistWords = kBins + kOverSlots + 16;  // bins 0..kBins-1, the copies of bin kBins, spare words
 static_assert(kHistWords % 4 == 0, "the arrays that share this memory need 16-byte alignment");
 constexpr float kFix = 17592186044416.f;          // 2^44
@@ -801,6 +836,7 @@ __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, do
     }
     cluster.sync();                                    // (two buffers: who is here has read those of the pass before)
     long long hi = 0ll, lo = 0ll, q = 0ll;
+#pragma unroll 2
     for (int c = 0; c < n_cta; ++c) {
         hi += sh.part[n_pass & 1][0][c];
         lo += sh.part[n_pass & 1][1][c];
@@ -813,9 +849,9 @@ __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, do
 }
 
 // One cluster-wide pass over the live rows; every CTA fills its own shared-memory histogram.
-// tot (shared memory, zero before the call): [0] the mass that the CTA added (p and q), from floating-point sums.
-__device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float binscale, const HistSmem &h,
-                               double *sums1, int cta_rank, int n_cta, int halves, unsigned long long *tot) {
+// sh.added (zero before the call) += the mass that the CTA added (p and q), from floating-point sums.
+__device__ __forceinline__ void histogram_pass(const VerifyArgs &a, Shared &sh, float binscale, const HistSmem &h,
+                               double *sums1, int cta_rank, int n_cta, int halves) {
     // halves = 2: an item is a half tile (when the cluster has a warp for each), with a sum of its own
     const int lane = threadIdx.x & 31;
     const int warp = cta_rank * kVWarps + (threadIdx.x >> 5);
@@ -861,160 +897,228 @@ __device__ void histogram_pass(const VerifyArgs &a, const Shared &sh, float bins
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) added += __shfl_xor_sync(kFull, added, o);
-    if (lane == 0 && added) atomicAdd(tot, added);
+    if (lane == 0 && added) atomicAdd(&sh.added, added);
 }
 
-// The copies of the last bin (rho beyond the last edge), folded by each CTA and added to every CTA's total
-// (tot[7], tot[8]); before the cluster barrier that follows the pass.  Also tot[6] += what the CTA's threads
-// added minus what these copies hold of it.
-__device__ void hist_fold_over(cg::cluster_group &cluster, const HistSmem &h, unsigned long long *tot, int n_cta) {
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x < kOverSlots) {
+// This CTA's histogram into suffix sums (p and q mass of its bins >= k, units of 2^-44), in place of the words: w words the
+// low, b words the high halves.  Entry kBins is the last bin, whose copies are folded here.  A thread takes eight bins, all their words in
+// flight together.  Each CTA keeps the sums of its own cells; the chain adds the few that it looks up over the
+// CTAs (a merge of the 4096 bins over the cluster before it took 4.5 us a layer and another cluster barrier, for at most 2 m bins that
+// anybody looks at).
+static_assert(kBins == 8 * kVThreads, "eight bins to a thread");
+__device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i0 = threadIdx.x * 8;
+    unsigned long long v[2][8];                              // p, q
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const uint32_t *w = x ? h.wq : h.wp, *b = x ? h.bq : h.bp;
+#pragma unroll
+        for (int k = 0; k < 8; k += 4) {
+            const uint4 lo = *reinterpret_cast<const uint4 *>(w + i0 + k), hi = *reinterpret_cast<const uint4 *>(b + i0 + k);
+            v[x][k] = ((unsigned long long)hi.x << 16) + lo.x; v[x][k + 1] = ((unsigned long long)hi.y << 16) + lo.y;
+            v[x][k + 2] = ((unsigned long long)hi.z << 16) + lo.z; v[x][k + 3] = ((unsigned long long)hi.w << 16) + lo.w;
+        }
+#pragma unroll
+        for (int k = 6; k >= 0; --k) v[x][k] += v[x][k + 1];
+    }
+    unsigned long long above[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        unsigned long long s = v[x][0];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_down_sync(kFull, s, o);
+            if (lane + o < 32) s += t;
+        }
+        above[x] = s - v[x][0];
+        if (lane == 0) sh.wtot[x][warp] = s;
+    }
+    if (warp < kOverSlots / 32) {
         const int i = kBins + (int)threadIdx.x;
-        unsigned long long P = ((unsigned long long)h.bp[i] << 16) + h.wp[i], Q = ((unsigned long long)h.bq[i] << 16) + h.wq[i];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            P += __shfl_xor_sync(kFull, P, o);
-            Q += __shfl_xor_sync(kFull, Q, o);
-        }
-        unsigned long long w = P + Q;
-        if (threadIdx.x < 32) w -= tot[0];
-        if (lane < n_cta) {
-            unsigned long long *to = cluster.map_shared_rank(tot, lane);
-            if (w) atomicAdd(to + 6, 0ull - w);
-            if (P) atomicAdd(to + 7, P);
-            if (Q) atomicAdd(to + 8, Q);
-        }
-    }
-}
-
-// Merge of the cluster's histograms, after a cluster barrier that follows the pass: every CTA sums one slice of
-// the bins over all CTAs' shared memory.  A lane takes four bins of two CTAs (eight bins when there is one CTA), so
-// that all its loads are in flight together; the lanes that share bins add up by shuffles, and with 16 CTAs two
-// warps share bins.  The CTA's suffix sums (p and q mass of the slice's bins >= k, units of 2^-44) replace the words of
-// its own slice, which no other CTA reads here: w words the low, b words the high halves.  Every CTA
-// gets the slice's totals.  The caller puts a cluster barrier behind this before anyone looks at another's slice.
-// Bound by distributed shared memory (64 KB a CTA, 4.5 us), as long as an instruction takes at least 128 bytes from
-// each CTA it reads: with 64 bytes from each of 8, one warp to the bins, 16 CTAs took 7 to 10 us.  (512 bytes
-// an instruction and the sums of 2 to 8 warps through a stage of 16 KB were no faster with 8 CTAs, and the shared
-// memory came off the L1 cache: 64 requests x 8 rows of 128256 30 us slower.  Half the words to fetch, by b words
-// that are added at once in the CTA that will merge them: merge 4.4 -> 3.3 us, but the pass 110 -> 115 and, for one request
-// of V = 32000, 7.5 -> 9.5: an atomic add to another CTA's shared memory costs its warp more than a local one.  Half the
-// bins for layers of few drafts: merge 4.4 -> 3.1, but their w words wrap on ordinary data when one CTA has the whole layer.)
-__device__ void hist_merge(cg::cluster_group &cluster, const HistSmem &h, Shared &sh, int cta_rank, int n_cta) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int share = n_cta > 1 ? min(n_cta / 2, 4) : 1;     // lanes that share four bins
-    const int parts = n_cta > 8 ? 2 : 1;                     // warps that share them
-    const int per_warp = 32 / share, place = lane % per_warp, segs = kVWarps / parts;
-    const int seg = warp % segs, part = warp / segs;
-    const int n_bins = n_cta > 1 ? 4 : 8;                    // of a lane
-    const int i0 = cta_rank * (kBins / n_cta) + (seg * per_warp + place) * n_bins;
-    unsigned long long P[8] = {}, Q[8] = {};
-    auto add4 = [&](int c, int i, unsigned long long *p, unsigned long long *q) {
-        const uint4 wp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wp, c) + i);
-        const uint4 wq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.wq, c) + i);
-        const uint4 bp = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bp, c) + i);
-        const uint4 bq = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(h.bq, c) + i);
-        p[0] += ((unsigned long long)bp.x << 16) + wp.x; p[1] += ((unsigned long long)bp.y << 16) + wp.y;
-        p[2] += ((unsigned long long)bp.z << 16) + wp.z; p[3] += ((unsigned long long)bp.w << 16) + wp.w;
-        q[0] += ((unsigned long long)bq.x << 16) + wq.x; q[1] += ((unsigned long long)bq.y << 16) + wq.y;
-        q[2] += ((unsigned long long)bq.z << 16) + wq.z; q[3] += ((unsigned long long)bq.w << 16) + wq.w;
-    };
-    const int c0 = part * 8 + lane / per_warp;
-    if (n_cta > 1) {
-        add4(c0, i0, P, Q);
-        add4(c0 + share, i0, P, Q);
-    } else {
-        add4(0, i0, P, Q);
-        add4(0, i0 + 4, P + 4, Q + 4);
-    }
-    for (int o = per_warp; o < 32; o <<= 1) {
+        for (int x = 0; x < 2; ++x) {
+            unsigned long long s = ((unsigned long long)(x ? h.bq : h.bp)[i] << 16) + (x ? h.wq : h.wp)[i];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            P[k] += __shfl_xor_sync(kFull, P[k], o);
-            Q[k] += __shfl_xor_sync(kFull, Q[k], o);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+            if (lane == 0) sh.over[x][warp] = s;
         }
     }
-    auto store4 = [&](int i, const unsigned long long *p, const unsigned long long *q, unsigned long long rp, unsigned long long rq) {
-        auto words = [&](uint32_t *low, uint32_t *high, const unsigned long long *v, unsigned long long r) {
-            *reinterpret_cast<uint4 *>(low + i) = make_uint4((uint32_t)(v[0] + r), (uint32_t)(v[1] + r), (uint32_t)(v[2] + r), (uint32_t)(v[3] + r));
-            *reinterpret_cast<uint4 *>(high + i) = make_uint4((uint32_t)((v[0] + r) >> 32), (uint32_t)((v[1] + r) >> 32),
-                                                             (uint32_t)((v[2] + r) >> 32), (uint32_t)((v[3] + r) >> 32));
-        };
-        words(h.wp, h.bp, p, rp);
-        words(h.wq, h.bq, q, rq);
-    };
-    if (parts == 2) {
-        // the second warp's sums through the slice itself, once the whole CTA has read its own words there
-        __syncthreads();
-        if (part == 1 && lane < per_warp) store4(i0, P, Q, 0ull, 0ull);
-        __syncthreads();
-        if (part == 0) {
-            const uint4 lp = *reinterpret_cast<const uint4 *>(h.wp + i0), up = *reinterpret_cast<const uint4 *>(h.bp + i0);
-            const uint4 lq = *reinterpret_cast<const uint4 *>(h.wq + i0), uq = *reinterpret_cast<const uint4 *>(h.bq + i0);
-            auto whole = [](uint32_t low, uint32_t high) { return ((unsigned long long)high << 32) | low; };
-            P[0] += whole(lp.x, up.x); P[1] += whole(lp.y, up.y); P[2] += whole(lp.z, up.z); P[3] += whole(lp.w, up.w);
-            Q[0] += whole(lq.x, uq.x); Q[1] += whole(lq.y, uq.y); Q[2] += whole(lq.z, uq.z); Q[3] += whole(lq.w, uq.w);
-        }
-    }
-    // suffix sums: in the lane, over the lanes' places, over the warps of part 0
-#pragma unroll
-    for (int k = 6; k >= 0; --k) { P[k] += P[k + 1]; Q[k] += Q[k + 1]; }
-    unsigned long long ap = P[0], aq = Q[0];
-    for (int o = 1; o < per_warp; o <<= 1) {
-        const unsigned long long tp = __shfl_down_sync(kFull, ap, o), tq = __shfl_down_sync(kFull, aq, o);
-        if (place + o < per_warp) { ap += tp; aq += tq; }
-    }
-    if (part == 0 && lane == 0) { sh.wtot_p[seg] = ap; sh.wtot_q[seg] = aq; }
     __syncthreads();
-    if (part > 0) return;
-    unsigned long long rp = ap - P[0], rq = aq - Q[0];
-    for (int w = seg + 1; w < segs; ++w) { rp += sh.wtot_p[w]; rq += sh.wtot_q[w]; }
-    if (lane < per_warp) {
-        store4(i0, P, Q, rp, rq);
-        if (n_cta == 1) store4(i0 + 4, P + 4, Q + 4, rp, rq);
-    }
-    if (seg == 0) {
-        // place 0: the whole slice
-        const unsigned long long tp = __shfl_sync(kFull, P[0] + rp, 0), tq = __shfl_sync(kFull, Q[0] + rq, 0);
-        if (lane < n_cta) {
-            Shared *to = cluster.map_shared_rank(&sh, lane);
-            to->slice_p[cta_rank] = tp;
-            to->slice_q[cta_rank] = tq;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        unsigned long long over = 0ull;
+#pragma unroll
+        for (int w = 0; w < kOverSlots / 32; ++w) over += sh.over[x][w];
+        above[x] += over;
+#pragma unroll 1
+        for (int w = warp + 1; w < kVWarps; ++w) above[x] += sh.wtot[x][w];
+        uint32_t *low = x ? h.wq : h.wp, *high = x ? h.bq : h.bp;
+#pragma unroll
+        for (int k = 0; k < 8; k += 4) {
+            const unsigned long long a0 = v[x][k] + above[x], a1 = v[x][k + 1] + above[x], a2 = v[x][k + 2] + above[x], a3 = v[x][k + 3] + above[x];
+            *reinterpret_cast<uint4 *>(low + i0 + k) = make_uint4((uint32_t)a0, (uint32_t)a1, (uint32_t)a2, (uint32_t)a3);
+            *reinterpret_cast<uint4 *>(high + i0 + k) = make_uint4((uint32_t)(a0 >> 32), (uint32_t)(a1 >> 32), (uint32_t)(a2 >> 32), (uint32_t)(a3 >> 32));
         }
+        if (threadIdx.x == 0) { low[kBins] = (uint32_t)over; high[kBins] = (uint32_t)(over >> 32); }
     }
+    // what the threads added, by their floating-point sums, minus what the words hold.  Without a wrap that is rounding: half a
+    // unit for each cell and 2^-20 of the mass (16 cells in a float sum), less than 2^26 units; a wrap lowers the words by 2^32
+    if (threadIdx.x == 0) sh.wrapped = (long long)(sh.added - (v[0][0] + above[0]) - (v[1][0] + above[1])) > (1ll << 31);
 }
 
-// One completion draw (residual if s_res > 0 else p_beam) by one warp; returns the token or -1
-// and the index of the live parent.
-__device__ int draw_cell(const VerifyArgs &a, const Shared &sh, double u, bool use_res, float s_res,
-                         const double *res_sums, int halves, int lane, int *ia_out) {
-    int ia, t;
-    double target;
+// Per live draft of layer l: rho = p_beam/q_beam of its cell and its uniform, by one warp.
+__device__ __noinline__ void draft_tests(Shared &sh, uint64_t seed, uint64_t step, int r, int l, int m, int lane) {
+#pragma unroll 1
+    for (int i = lane; i < m; i += 32) {
+        const int ai = sh.S_parent_idx[i];
+        const double lp = sh.rho[i], lq = sh.uu[i];
+        double rho;
+        if (lq == -INFINITY || sh.lwq[ai] == -INFINITY)
+            rho = (lp > -INFINITY && sh.lwp[ai] > -INFINITY) ? INFINITY : 0.0;
+        else
+            rho = exp((sh.lwp[ai] - sh.lwq[ai]) + (lp - lq));
+        sh.rho[i] = rho;
+        sh.uu[i] = decision_uniform(seed, step, (uint32_t)r, (uint32_t)l, 0u, (uint32_t)i);
+    }
+    __syncwarp();
+}
+
+// The accept loop from draft sh.next_i on, by one warp.  The run position rises by one with every rejection and falls back to 1
+// with an accept, so the drafts behind one another are tested side by side, each at the position that it has if
+// all before it are rejected; the first accept among them ends the round.
+// on_demand: ends with sh.need_exact = 1 after a rejection whose residual mass c_{j+1} is not known yet.
+// node_status: nullptr in a CTA that writes no results.
+__device__ __noinline__ void accept_drafts(Shared &sh, int8_t *st, int8_t *node_status, int n_lo, int m, int W, bool on_demand, int lane) {
+    int i = sh.next_i, count = sh.count, j = sh.run_j, tests = 0, near = 0, need = 0;
+    const int len = sh.chain_len;
+#pragma unroll 1
+    while (i < m && count < W && !need) {
+        const int n = min(m - i, 32);
+        // an empty residual means p' == q_beam: the rejected draft lay outside the support of q_beam, there is nothing to
+        // subtract and p' stays, and so does the run position
+        const unsigned rises = __ballot_sync(kFull, j + lane <= len && sh.c_arr[min(j + lane, kMaxLive) + 1] > 0.0);
+        const int stop = ~rises ? __ffs(~rises) - 1 : 32;         // positions j .. j + stop are reached
+        const int jt = j + min(lane, stop);
+        const bool asks = on_demand && j + stop == len + 1;       // a rejection at the last position asks for its residual mass
+        const int lanes = asks ? min(n, stop + 1) : n;
+        bool accept = false, close = false;
+        if (lane < lanes) {
+            double ratio = sh.rho[i + lane];
+            if (jt > 1) ratio = fmax(ratio - sh.s_arr[jt - 1], 0.0) / sh.c_arr[jt];
+            if (ratio > 1.0) ratio = 1.0;
+            const double u = sh.uu[i + lane];
+            accept = u <= ratio;
+            close = fabs(u - ratio) < 1e-5;
+        }
+        const unsigned accepts = __ballot_sync(kFull, accept);
+        const int done = accepts ? __ffs(accepts) : lanes;        // drafts tested in this round
+        near += __popc(__ballot_sync(kFull, close && lane < done));
+        if (lane < done) {
+            const int node = sh.S[i + lane], status = lane == done - 1 && accepts ? DSBD_NODE_ACCEPTED : DSBD_NODE_REJECTED;
+            st[node - n_lo] = (int8_t)status;
+            if (node_status) node_status[node] = (int8_t)status;
+            if (status == DSBD_NODE_ACCEPTED) sh.acc[count] = node;
+        }
+        tests += done;
+        i += done;
+        if (accepts) { ++count; j = 1; }
+        else if (asks && done == stop + 1) {
+            j += stop;
+            if (lane == 0) sh.s_arr[j] = sh.s_arr[j - 1] + sh.c_arr[j];
+            need = 1;
+        } else j += min(done, stop);
+    }
+    __syncwarp();
+    if (lane == 0) {
+        sh.next_i = i;
+        sh.count = count;
+        sh.run_j = j;
+        sh.n_tests += tests;
+        sh.n_near += near;
+        sh.need_exact = need;
+        sh.chain_pos = j;                          // (the position whose residual mass is asked for)
+    }
+    __syncwarp();
+}
+
+// Where the warps of a CTA keep what a draw searches (the histogram arrays are idle then): a warp's token masses or a piece of
+// its tile masses, and behind them, for the residual draw, the sums of kParts equal shares of the layer's item sums.
+constexpr int kParts = 256, kPiece = 512;
+static_assert(kPiece * sizeof(double) <= kTokWords * sizeof(float), "a piece of tile masses fits a warp's words");
+static_assert(kVWarps * kTokWords * sizeof(float) + kParts * sizeof(double) <= kHistArrays * kHistWords * sizeof(uint32_t),
+              "what the draws search overlays the histogram arrays");
+
+// One completion draw by one warp: from p_beam, or (use_res) from the residual at s_res; returns the token or -1
+// and the index of the live parent.  parts: see draw_shares.
+__device__ __forceinline__ int draw_cell(const VerifyArgs &a, const Shared &sh, double u, bool use_res, float s_res,
+                                         const double *res_sums, int halves, const double *parts, float *words, int lane, int *ia_out) {
+    double *piece = reinterpret_cast<double *>(words);
+    double target = u;
+    int ia, t = 0;
+    int n = a.T;                                     // tile masses to search, from `at` on
+    int at = 0;
+    double wpa = 0.0, lse_row = 0.0;
+    const TileStat *st = a.stats;
     if (use_res) {
         // (res_sums: one per tile, or two when the pass that wrote them worked on half tiles)
-        auto sum = [&](int i) { return halves == 1 ? __ldcg(res_sums + i) : __ldcg(res_sums + 2 * i) + __ldcg(res_sums + 2 * i + 1); };
-        const int tile = locate_tile(sum, sh.nA * a.T, u, true, lane, &target);
-        if (tile < 0) return -1;
-        ia = tile / a.T; t = tile - ia * a.T;
+        const int tiles = sh.nA * a.T, per = (tiles + kParts - 1) / kParts;
+        at = locate(parts, kParts, target, true, false, lane);
+        if (at < 0) return -1;
+        at *= per;
+        n = min(per, tiles - at);
+        ia = 0;
     } else {
         // p_beam: first the live parent (its row holds exactly its beam weight), then the tile
-        ia = locate_tile([&](int i) { return sh.wp[i]; }, sh.nA, u, true, lane, &target);
+        ia = locate(sh.wp, sh.nA, target, true, false, lane);
         if (ia < 0) return -1;
         const int row = sh.A[ia];
-        const double wpa = sh.wp[ia], lse_row = a.lse[row];
-        const TileStat *st = a.stats + (int64_t)row * a.T;
-        t = locate_tile([&](int i) {
-            const TileStat ts = st[i];
-            if (!(ts.sum > 0.f)) return 0.0;
-            return wpa * (double)ts.sum * exp((double)ts.mx * a.inv_tau - lse_row);
-        }, a.T, target, false, lane, &target);
-        if (t < 0) return -1;
+        wpa = sh.wp[ia]; lse_row = a.lse[row];
+        st += (int64_t)row * a.T;
     }
+#pragma unroll 1
+    for (int base = 0; ; base += kPiece) {
+        const int len = min(kPiece, n - base);
+        if (use_res) {
+#pragma unroll 1
+            for (int i = lane; i < len; i += 32) {
+                const int k = at + base + i;
+                piece[i] = halves == 1 ? __ldcg(res_sums + k) : __ldcg(res_sums + 2 * k) + __ldcg(res_sums + 2 * k + 1);
+            }
+        } else {
+#pragma unroll 2
+            for (int i = lane; i < len; i += 32) {
+                const TileStat ts = st[base + i];
+                piece[i] = ts.sum > 0.f ? wpa * (double)ts.sum * exp((double)ts.mx * a.inv_tau - lse_row) : 0.0;
+            }
+        }
+        __syncwarp();
+        const bool more = base + len < n;
+        t = locate(piece, len, target, false, more, lane);
+        __syncwarp();
+        if (t >= 0 && !(more && t == len)) { t += at + base; break; }
+        if (t < 0) {
+            if (base == 0) return -1;
+            n = base;                                // no mass from here on: the last tile with mass before
+            target = INFINITY;
+            base -= 2 * kPiece;
+        }
+    }
+    if (use_res) { ia = t / a.T; t -= ia * a.T; }
     *ia_out = ia;
     const RowOff ro = row_off(sh, ia);
     const int64_t row = (int64_t)sh.A[ia] * a.stride;
-    return locate_token(a.zp + row, a.zq + row, a.V, a.k2, t, ro, use_res ? s_res : 0.f, target, lane);
+    return locate_token(a.zp + row, a.zq + row, a.V, a.k2, t, ro, use_res ? s_res : 0.f, target, lane, words);
+}
+
+// Sums of kParts equal shares of the layer's item sums, by the CTA's first kParts threads: what a residual draw searches first.
+__device__ __forceinline__ void draw_shares(const double *res_sums, int halves, int tiles, double *parts) {
+    if (threadIdx.x >= kParts) return;
+    const int per = (tiles + kParts - 1) / kParts * halves;
+    const int i1 = min(((int)threadIdx.x + 1) * per, tiles * halves);
+    double v = 0.0;
+#pragma unroll 4
+    for (int i = (int)threadIdx.x * per; i < i1; ++i) v += __ldcg(res_sums + i);
+    parts[threadIdx.x] = v;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1081,6 +1185,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     const double *lse = a.lse + (int64_t)model * a.N;
     const float *z = model ? a.zq : a.zp;
     const float inv_tau_f = (float)a.inv_tau;
+#pragma unroll 1
     for (int i = tl; i < sh.nA; i += NT) tp.off[i] = (float)(lw[i] - lse[sh.A[i]]);
     if (tl < 3) tp.count[tl] = 0;
     if (tl == 0) { tp.low = 0xffffffffu; tp.n_sel = 0; tp.n_cand = 0; tp.err = 0; ws.n[model] = 0; }
@@ -1104,7 +1209,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     {
         unsigned lo = 0xffffffffu, hi = 0u;
         int finite = 0;
-#pragma unroll 4
+#pragma unroll 2
         for (int i = tl; i < nt; i += NT) {
             const float v = bound(i);
             const unsigned u = image(v);
@@ -1127,7 +1232,13 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         for (int round = 0; hi - lo > 1; ++round) {
             const unsigned mid = lo + (hi - lo) / 2;
             int n = 0;
-            for (int i = tl; i < nt; i += NT) n += (cached ? bcache[i] : image(bound(i))) >= mid;
+            if (cached) {
+#pragma unroll 4
+                for (int i = tl; i < nt; i += NT) n += bcache[i] >= mid;
+            } else {
+#pragma unroll 1
+                for (int i = tl; i < nt; i += NT) n += image(bound(i)) >= mid;
+            }
             n = __reduce_add_sync(kFull, n);
             if (lane == 0 && n) atomicAdd(&tp.count[round % 3], n);
             if (tl == 0) tp.count[(round + 1) % 3] = 0;           // (last read two rounds ago)
@@ -1145,6 +1256,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     float theta = -INFINITY, cut = finite >= k ? slack(value(lo)) : -INFINITY;
     for (int again = 0; ; ++again) {
         unsigned low = 0xffffffffu;
+#pragma unroll 1
         for (int i = tl; i < nt; i += NT) {
             const float bv = cached ? value(bcache[i]) : bound(i);
             if (bv >= cut && bv > -INFINITY) {
@@ -1166,102 +1278,95 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         part_sync<NT>(model);
     }
     const int n_sel = tp.n_sel;
-    // One sweep over the selected tiles by all warps: counts the cells whose key reaches th and,
-    // when asked, appends them to the candidate list (order is irrelevant: the final choice is
-    // by (key, cell)).
-    auto sweep = [&](float th, bool collect) {
-        part_sync<NT>(model);                      // every thread has taken the previous sweep's count
-        if (tl == 0) tp.n_cand = 0;
-        part_sync<NT>(model);
-        // this warp's tiles into L2 first (a tile is 32 lines of 128 bytes: one per lane), so that
-        // the dependent tile loads below do not each pay a trip to HBM
-        for (int sidx = warp; sidx < n_sel; sidx += kPartWarps) {
-            const int ti = tp.sel[sidx], ia = ti / T, t = ti - ia * T;
-            const int e = t * kTile + lane * 32;
-            if (e < a.V) asm volatile("prefetch.global.L2 [%0];" ::"l"(z + (int64_t)sh.A[ia] * a.stride + e));
-        }
+    // Sweeps over the selected tiles by all warps: each counts the cells whose key reaches th and, when collect is set, lists
+    // them (order is irrelevant: the final choice is by (key, cell)).  The first one nearly always fits the list.  Too many
+    // cells reach the conservative threshold where there are few tiles, a large k or near ties: then a bisection, by sweeps that
+    // only count, finds a threshold with between k and kMaxCand cells above it, and one more sweep lists those.
+    // (One copy of the sweep, and lanes that walk their hits: the three copies with an unrolled list each were 60 KB of code.)
+    float th = theta, lo_t = 0.f, hi_t = 0.f;
+    bool collect = true;
+    int n_cand;
+#pragma unroll 1
+    for (int itn = -1; ; ++itn) {
+        const float th_f = fmaxf(th, -3.402823466e38f);      // (a key of -infinity has no mass)
+#pragma unroll 1
         for (int sidx = warp; sidx < n_sel; sidx += kPartWarps) {
             const int ti = tp.sel[sidx], ia = ti / T, t = ti - ia * T, row = sh.A[ia];
             const float *rowp = z + (int64_t)row * a.stride;
             const bool al = (reinterpret_cast<uintptr_t>(rowp) & 15) == 0;
             float4 v[8];
             load_tile<false>(rowp, t * kTile, a.V, al, lane, v);
+            // the warp's next tile on its way to L2 (a tile is 32 lines of 128 bytes: one per lane)
+            if (sidx + kPartWarps < n_sel) {
+                const int tn = tp.sel[sidx + kPartWarps], in = tn / T, e = (tn - in * T) * kTile + lane * 32;
+                if (e < a.V) asm volatile("prefetch.global.L2 [%0];" ::"l"(z + (int64_t)sh.A[in] * a.stride + e));
+            }
             const float off_f = tp.off[ia];
-            const double off_d = lw[ia] - lse[row];
             unsigned hits = 0;                               // bit (it*4+c) of this lane's 32 cells
 #pragma unroll
             for (int it = 0; it < 8; ++it) {
                 const float zz[4] = {v[it].x, v[it].y, v[it].z, v[it].w};
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float kf = fmaf(zz[c], inv_tau_f, off_f);
-                    if (kf >= th && kf > -INFINITY) hits |= 1u << (it * 4 + c);
-                }
+                for (int c = 0; c < 4; ++c)
+                    if (fmaf(zz[c], inv_tau_f, off_f) >= th_f) hits |= 1u << (it * 4 + c);
             }
-            const int mine = __popc(hits);
-            int incl = mine;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int tmp = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += tmp;
-            }
-            const int total = __shfl_sync(kFull, incl, 31);
-            int base_pos = 0;
-            if (lane == 0 && total) base_pos = atomicAdd(&tp.n_cand, total);
-            base_pos = __shfl_sync(kFull, base_pos, 0);
-            if (collect && mine) {
-                int pos = base_pos + incl - mine;
-#pragma unroll
-                for (int it = 0; it < 8; ++it) {
-                    const float zz[4] = {v[it].x, v[it].y, v[it].z, v[it].w};
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (hits & (1u << (it * 4 + c))) {
-                            if (pos < kMaxCand) {
-                                cand_key[pos] = off_d + (double)zz[c] * a.inv_tau;
-                                cand_cell[pos] = ia * a.V + t * kTile + it * 128 + lane * 4 + c;
-                            }
-                            ++pos;
-                        }
+            if (hits) {
+                int pos = atomicAdd(&tp.n_cand, __popc(hits));
+                if (collect) {
+                    const double off_d = lw[ia] - lse[row];
+#pragma unroll 1
+                    for (; hits && pos < kMaxCand; hits &= hits - 1, ++pos) {
+                        const int bit = __ffs(hits) - 1, tok = t * kTile + (bit >> 2) * 128 + lane * 4 + (bit & 3);
+                        cand_key[pos] = off_d + (double)__ldg(rowp + tok) * a.inv_tau;
+                        cand_cell[pos] = ia * a.V + tok;
+                    }
                 }
             }
         }
         part_sync<NT>(model);
-        return tp.n_cand;
-    };
-    int n_cand = sweep(theta, true);
-    if (n_cand > kMaxCand) {
-        // too many cells reach the conservative threshold (few tiles, large k, or near ties):
-        // bisect for a threshold with between k and kMaxCand cells above it
-        float lo_t = theta, hi_t = -INFINITY;
-        for (int sidx = 0; sidx < n_sel; ++sidx) hi_t = fmaxf(hi_t, bound(tp.sel[sidx]));
-        if (!(lo_t > -INFINITY)) lo_t = hi_t - 400.f;
-        bool found = false;
-        for (int itn = 0; itn < 60 && hi_t > lo_t; ++itn) {
+        n_cand = tp.n_cand;
+        if (collect) {
+            if (n_cand <= kMaxCand || itn >= 0) break;
+            lo_t = theta; hi_t = -INFINITY;
+#pragma unroll 1
+            for (int sidx = 0; sidx < n_sel; ++sidx) hi_t = fmaxf(hi_t, bound(tp.sel[sidx]));
+            if (!(lo_t > -INFINITY)) lo_t = hi_t - 400.f;
+            collect = false;
+        } else if (n_cand > kMaxCand) lo_t = th;
+        else if (n_cand < k) hi_t = th;
+        else collect = true;
+        if (!collect) {
+            if (itn + 1 >= 60 || !(hi_t > lo_t)) return DSBD_DEV_CAPACITY;              // a huge tie at the cut
             // (first out of the gap above a mask of finite values: halving does not come back from -1e30)
-            const float half = 0.5f * (lo_t + hi_t), mid = itn ? half : fmaxf(half, hi_t - 400.f);
-            const int c = sweep(mid, false);
-            if (c > kMaxCand) lo_t = mid;
-            else if (c < k) hi_t = mid;
-            else { theta = mid; found = true; break; }
+            const float half = 0.5f * (lo_t + hi_t);
+            th = itn < 0 ? fmaxf(half, hi_t - 400.f) : half;
         }
-        if (!found) return DSBD_DEV_CAPACITY;              // a huge tie at the cut
-        n_cand = sweep(theta, true);
+        part_sync<NT>(model);                      // every thread has taken the count
+        if (tl == 0) tp.n_cand = 0;
+        part_sync<NT>(model);
     }
     // exact top k of the candidates: every candidate counts those that beat it (key descending,
     // cell ascending -- a total order, cells are unique) and, if fewer than k do, that count is its
-    // place in the support
+    // place in the support.  Eight lanes to a candidate: a few dozen candidates take one round.
     if (n_cand > kMaxCand) n_cand = kMaxCand;
-    for (int jc = tl; jc < n_cand; jc += NT) {
-        const double key = cand_key[jc];
-        const int cell = cand_cell[jc];
-        int rank = 0;
-#pragma unroll 4
-        for (int i = 0; i < n_cand; ++i) {
-            const double ki = cand_key[i];
-            rank += (ki > key) || (ki == key && cand_cell[i] < cell);
+#pragma unroll 1
+    for (int j0 = 0; j0 < n_cand; j0 += NT / 8) {
+        const int jc = j0 + (tl >> 3);
+        double key = 0.0;
+        int cell = 0, rank = 0;
+        if (jc < n_cand) {
+            key = cand_key[jc];
+            cell = cand_cell[jc];
+#pragma unroll 2
+            for (int i = tl & 7; i < n_cand; i += 8) {
+                const double ki = cand_key[i];
+                rank += (ki > key) || (ki == key && cand_cell[i] < cell);
+            }
         }
-        if (rank < k) {
+        rank += __shfl_xor_sync(kFull, rank, 1);
+        rank += __shfl_xor_sync(kFull, rank, 2);
+        rank += __shfl_xor_sync(kFull, rank, 4);
+        if (jc < n_cand && (tl & 7) == 0 && rank < k) {
             ws.prob[model][rank] = exp(key);
             ws.cell[model][rank] = cell;
         }
@@ -1293,6 +1398,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
 
 __device__ __forceinline__ double support_lookup(const WarpScratch &ws, int model, int cell) {
     int at = -1;
+#pragma unroll 2
     for (int j = 0, n = ws.n[model]; j < n; ++j) at = ws.cell[model][j] == cell ? j : at;      // (cells are unique)
     return at >= 0 ? ws.prob[model][at] : 0.0;
 }
@@ -1310,6 +1416,7 @@ __device__ int draw_support(const WarpScratch &ws, double u, double s, int lane)
     const double target = u * zsum;
     int pick = -1;
     bool found = false;
+#pragma unroll 1
     for (int l = 0; 2 * l < n; ++l) {
         const double c0 = __shfl_sync(kFull, cum0, l), c1 = __shfl_sync(kFull, incl, l);
         if (!found && (m0 >> l & 1)) { pick = 2 * l; found = c0 >= target; }
@@ -1320,23 +1427,20 @@ __device__ int draw_support(const WarpScratch &ws, double u, double s, int lane)
 
 // After build_support(p) [and q]: q~ at the p cells and the canonical order of the p support.
 __device__ void finish_supports(WarpScratch &ws, bool have_q, int lane) {
+#pragma unroll 1
     for (int i = lane; i < ws.n[0]; i += 32) ws.qat[i] = have_q ? support_lookup(ws, 1, ws.cell[0][i]) : 0.0;
     // canonical order: the place of a cell is the number of support cells below it (cells are unique)
     const int n = ws.n[0];
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) {
         const int c = ws.cell[0][i];
         int place = 0;
+#pragma unroll 2
         for (int j = 0; j < n; ++j) place += ws.cell[0][j] < c;
         ws.order[place] = i;
     }
     __syncwarp();
 }
-
-#ifdef DSBD_PHASE_TIMING
-#define TS(slot) do { if (threadIdx.x == 0 && writer) { unsigned long long t_; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_)); a.dbg[(int64_t)r * 256 + ts_n] = ((unsigned long long)(slot) << 48) | (t_ & 0xFFFFFFFFFFFFull); if (ts_n < 255) ++ts_n; } } while (0)
-#else
-#define TS(slot) do {} while (0)
-#endif
 
 // Drafts behind the first rejection of a layer of known width up to which its residual masses are computed on demand: a pass
 // for that rejection and at most one for each of them, against one histogram, and a pass more where the layer ends in a residual
@@ -1386,15 +1490,15 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     if (bad_widths) { W_min = W_max = W_nom = 1; }
     double *sums_base = a.tile_sums + (int64_t)r * 2 * (a.max_m + 1) * ((int64_t)a.max_live * a.T);
     const int64_t slot_stride = (int64_t)a.max_live * a.T;
-    int n_out = 0, n_pass = 0, n_hist = 0;
+    int n_pass = 0;
 #ifdef DSBD_PHASE_TIMING
-    int ts_n = 0;
+    if (threadIdx.x == 0) { sh.ts = writer ? a.dbg + (int64_t)r * 256 : nullptr; sh.ts_end = sh.ts + 255; }
 #endif
 
     TS(1);
     // (a CTA may store into another's shared memory once that CTA runs: arrived here, waited for below)
-    if (threadIdx.x < 20) sh.w_tot[threadIdx.x / 10][threadIdx.x % 10] = 0ull;
     cluster.barrier_arrive();
+    if (!kWarped && threadIdx.x <= kMaxLive) sh.binscale[threadIdx.x] = (float)((double)kBins / log2((double)max((int)threadIdx.x, 2)));    // s_j <= j <= m
     const int n_req_nodes = n_hi - n_lo, n_trees = min(b_hi - b_lo, kMaxLive);
     const bool cached = !a.select_mode && n_req_nodes <= kCacheNodes && a.gamma < 256;
     if (!a.select_mode) {
@@ -1428,6 +1532,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         TS(13);
         // ---- log-sum-exp of every row of the request from the dense pass's tile statistics ----
+#pragma unroll 1
         for (int task = cw; task < 2 * n_req; task += ncw) {
             const int model = task / n_req, row = n_lo + (task - model * n_req);
             const double v = row_lse(a.stats + ((int64_t)model * a.N + row) * a.T, a.T, a.inv_tau, lane);
@@ -1476,6 +1581,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 nc.score_p[i] = sp; nc.score_q[i] = sq;
                 nc.depth[i] = (uint8_t)min(dep, 255);
                 int tree = 0;
+#pragma unroll 1
                 while (tree + 1 < n_trees && nc.root[tree + 1] <= n_lo + i) ++tree;
                 nc.tree[i] = (uint8_t)tree;
                 if (writer) {
@@ -1491,6 +1597,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         __threadfence();
         cluster.sync();
         // ---- log-prob of every draft token given its parent (all nodes at once) ----
+#pragma unroll 1
         for (int i = cta_rank * kVThreads + threadIdx.x; i < n_req; i += n_cta * kVThreads) {
             const int n = n_lo + i, par = a.parent[n];
             double lp = 0.0, lq = 0.0;
@@ -1518,11 +1625,13 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 // stage the per-node log-probs in shared memory (the histogram arrays are idle
                 // here), then every node sums its own path to the root
                 double *slp = reinterpret_cast<double *>(hp), *slq = reinterpret_cast<double *>(hq);
+#pragma unroll 1
                 for (int i = threadIdx.x; i < n_req; i += kVThreads) {
                     slp[i] = a.score_w[n_lo + i];
                     slq[i] = a.score_w[a.N + n_lo + i];
                 }
                 __syncthreads();
+#pragma unroll 1
                 for (int b = b_lo + (int)threadIdx.x; b < b_hi; b += kVThreads) {
                     const int root = a.beam_node_off[b];
                     if (a.parent[root] != -1) report(a.status, DSBD_DEV_BAD_FOREST);
@@ -1530,6 +1639,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     slq[root - n_lo] = (double)a.root_logq[b];
                 }
                 __syncthreads();
+#pragma unroll 1
                 for (int i = threadIdx.x; i < n_req; i += kVThreads) {
                     double sp = 0.0, sq = 0.0;
                     int dep = 0, cur = i;
@@ -1551,6 +1661,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             } else {
                 for (int b = b_lo + (int)threadIdx.x; b < b_hi; b += kVThreads) {
                     const int lo = a.beam_node_off[b], hi = a.beam_node_off[b + 1];
+#pragma unroll 1
                     for (int n = lo; n < hi; ++n) {
                         const int par = a.parent[n];
                         double sp, sq;
@@ -1593,7 +1704,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     auto is_root = [&](int i) { return cached ? nc.parent[i] == -1 : a.parent[n_lo + i] < 0; };
     if (warp == 0) {
         if (lane == 0) {
-            sh.err = 0; sh.done = 0; sh.n_out = 0; sh.n_fill = 0;
+            sh.err = 0; sh.n_out = 0; sh.n_draw = 0;
             sh.n_layers = sh.n_tests = sh.n_exact = sh.n_respass = 0;
             sh.n_wrapped = 0; sh.n_near = 0; sh.n_rows = 0;
             if (a.select_mode) {
@@ -1604,9 +1715,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     sh.err = DSBD_DEV_BAD_FOREST;
                     sh.nA = 0;
                 }
+#pragma unroll 1
                 for (int i = 0; i < sh.nA; ++i)
                     if (a.live_nodes[lo + i] < 0 || a.live_nodes[lo + i] >= a.N) sh.err = DSBD_DEV_BAD_FOREST;
                 if (sh.err) sh.nA = 0;
+#pragma unroll 1
                 for (int i = 0; i < sh.nA; ++i) {
                     sh.A[i] = a.live_nodes[lo + i];
                     sp_live[i] = (double)a.sel_logp[sh.A[i]];
@@ -1619,6 +1732,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         }
         __syncwarp();
         if (!a.select_mode) {
+#pragma unroll 1
             for (int i = lane; i < sh.nA; i += 32) {
                 const int root = a.beam_node_off[b_lo + i];
                 sh.A[i] = root;
@@ -1626,20 +1740,22 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 sq_live[i] = cached ? nc.score_q[root - n_lo] : a.score[a.N + root];
             }
             if (writer) {
+#pragma unroll 1
                 for (int l = lane; l <= a.gamma; l += 32) a.out.layer_width[(int64_t)r * (a.gamma + 1) + l] = -1;
                 if (lane == 0) { a.out.l_last[r] = a.gamma + 1; a.out.out_width[r] = 0; }
             }
         }
         __syncwarp();
         if (!a.select_mode && writer)
+#pragma unroll 1
             for (int n = n_lo + lane; n < n_hi; n += 32)
                 a.out.node_status[n] = is_root(n - n_lo) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     }
     // Every CTA of the cluster takes identical decisions from identical data, so each keeps its
     // own copy of the node statuses and only rank 0 writes results.
-    const int n_layers = a.select_mode ? 1 : a.gamma;
     const bool st_ok = n_req_nodes <= kMaxLive * kMaxLive;
     if (!a.select_mode)
+#pragma unroll 1
         for (int n = threadIdx.x; n < n_req_nodes && st_ok; n += blockDim.x)
             st[n] = is_root(n) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     __syncthreads();
@@ -1653,36 +1769,21 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         return cached ? (model ? nc.score_q[i] : nc.score_p[i]) : a.score[(int64_t)model * a.N + n_lo + i];
     };
 
-    // per live draft of layer l: index of its parent in A, rho = p_beam/q_beam of its cell, its uniform (one warp)
-    auto draft_tests = [&](int l, int m) {
-        for (int i = lane; i < m; i += 32) {
-            const int n = sh.S[i];
-            const int pl = nd_parent(n - n_lo), par = n_lo + pl;
-            int ai = 0;
-            while (ai < sh.nA && sh.A[ai] != par) ++ai;
-            sh.S_parent_idx[i] = ai;
-            const double lp = nd_score(0, n - n_lo) - nd_score(0, pl);
-            const double lq = nd_score(1, n - n_lo) - nd_score(1, pl);
-            double rho;
-            if (lq == -INFINITY || sh.lwq[ai] == -INFINITY)
-                rho = (lp > -INFINITY && sh.lwp[ai] > -INFINITY) ? INFINITY : 0.0;
-            else
-                rho = exp((sh.lwp[ai] - sh.lwq[ai]) + (lp - lq));
-            sh.rho[i] = rho;
-            sh.uu[i] = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 0u, (uint32_t)i);
-        }
-        __syncwarp();
-    };
-
-    for (int l = 1; l <= n_layers && !sh.done && !sh.err; ++l) {
+    const bool failed = sh.err != 0;
+    // Layers 1 .. gamma; then, in the CTA that writes, the extra layer: no drafts, W_nom beams from p_beam^(gamma+1).
+    const int n_layers = a.select_mode ? 1 : a.gamma + (writer ? 1 : 0);
+#pragma unroll 1
+    for (int l = 1; l <= n_layers && !failed; ++l) {
+        const bool extra = !a.select_mode && l > a.gamma;
         // ---- live drafts of layer l, in draw order; beam weights ----
         TS(2);
         if (warp == 0) {
             int m = 0;
             if (a.select_mode) {
                 m = a.m_in[r];
-                if (m < 0 || m > kMaxLive) { if (lane == 0) sh.err = DSBD_DEV_BAD_FOREST; m = 0; }
-            } else {
+                if (m < 0 || m > kMaxLive) m = -1;
+            } else if (!extra) {
+#pragma unroll 1
                 for (int base = 0; base < n_req_nodes; base += 32) {
                     const int n = base + lane;
                     bool live = false;
@@ -1699,20 +1800,36 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     if (live && pos < kMaxLive) sh.S[pos] = n_lo + n;
                     m += __popc(mask);
                 }
-                if (m > kMaxLive) { if (lane == 0) sh.err = DSBD_DEV_BAD_FOREST; m = 0; }
+                if (m > kMaxLive) m = -1;
                 __syncwarp();
                 if (a.draft_rank) {
                     // order of (draft_rank, node id), ids being ascending: a draft's place is the number before it
+#pragma unroll 1
                     for (int i = lane; i < m; i += 32) sh.S_parent_idx[i] = a.draft_rank[sh.S[i]];
                     __syncwarp();
+#pragma unroll 1
                     for (int i = lane; i < m; i += 32) {
                         const int key = sh.S_parent_idx[i];
                         int place = 0;
+#pragma unroll 2
                         for (int j = 0; j < m; ++j) place += sh.S_parent_idx[j] < key || (j < i && sh.S_parent_idx[j] == key);
                         sh.acc[place] = sh.S[i];
                     }
                     __syncwarp();
+#pragma unroll 1
                     for (int i = lane; i < m; i += 32) sh.S[i] = sh.acc[i];
+                    __syncwarp();
+                }
+                // index of a draft's parent in A, and its log-prob under either model given that parent
+#pragma unroll 1
+                for (int i = lane; i < m; i += 32) {
+                    const int n = sh.S[i] - n_lo, pl = nd_parent(n);
+                    int ai = 0;
+#pragma unroll 1
+                    while (ai < sh.nA && sh.A[ai] != n_lo + pl) ++ai;
+                    sh.S_parent_idx[i] = ai;
+                    sh.rho[i] = nd_score(0, n) - nd_score(0, pl);
+                    sh.uu[i] = nd_score(1, n) - nd_score(1, pl);
                 }
             }
             __syncwarp();
@@ -1722,72 +1839,45 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 sh.c_arr[1] = 1.0;
                 sh.chain_len = 0;          // c_{j+1} is known for j = 1..chain_len
                 sh.next_i = sh.count = 0;
-                sh.run_j = 1;
+                sh.run_j = sh.chain_pos = 1;
                 sh.bank = l & 1;
+                sh.added = 0ull;
             }
         } else if (warp <= 2) {
             live_weights(a, sh, warp - 1, warp == 1 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
-        } else {
+        } else if (!kWarped) {
             uint4 *words = reinterpret_cast<uint4 *>(hp);
+#pragma unroll 4
             for (int i = threadIdx.x - 96; i < kHistArrays * kHistWords / 4; i += kVThreads - 96) words[i] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
         const int m = sh.m;
+        if (m < 0) {
+            if (threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
+            break;
+        }
         bool looked_up = false, on_demand = false;
+        const int W_known = extra ? W_nom : W_min < W_max ? W_min : W_max;
         TS(3);
 
-        // The accept loop (lane 0 of warp 0), from draft sh.next_i on.  on_demand: ends with sh.need_exact = 1 after a
-        // rejection whose residual mass c_{j+1} is not known yet.
-        auto accept_loop = [&](int W, bool on_demand) {
-            int i = sh.next_i, count = sh.count, j = sh.run_j, tests = 0, near = 0, need = 0;
-            for (; i < m && count < W && !need; ++i) {
-                const int n = sh.S[i];
-                const double rho = sh.rho[i];
-                double ratio;
-                if (j == 1) ratio = rho;
-                else ratio = fmax(rho - sh.s_arr[j - 1], 0.0) / sh.c_arr[j];
-                if (ratio > 1.0) ratio = 1.0;
-                const double u = sh.uu[i];
-                ++tests;
-                near += fabs(u - ratio) < 1e-5;
-                if (u <= ratio) {
-                    st[n - n_lo] = DSBD_NODE_ACCEPTED;
-                    if (writer) a.out.node_status[n] = DSBD_NODE_ACCEPTED;
-                    sh.acc[count++] = n;
-                    j = 1;
-                } else {
-                    st[n - n_lo] = DSBD_NODE_REJECTED;
-                    if (writer) a.out.node_status[n] = DSBD_NODE_REJECTED;
-                    // an empty residual means p' == q_beam: the rejected draft lay outside the
-                    // support of q_beam, there is nothing to subtract and p' stays
-                    if (on_demand && j > sh.chain_len) { sh.s_arr[j] = sh.s_arr[j - 1] + sh.c_arr[j]; need = 1; }
-                    else if (j <= sh.chain_len && sh.c_arr[j + 1] > 0.0) ++j;
-                }
-            }
-            sh.next_i = i;
-            sh.count = count;
-            sh.run_j = j;
-            sh.n_tests += tests;
-            sh.n_near += near;
-            sh.need_exact = need;
-        };
         constexpr bool warped = kWarped;
         WarpScratch &wsup = *reinterpret_cast<WarpScratch *>(hq);       // the histogram arrays are idle when warped
         if (warped) {
             // ---- supports of T o p_beam and T o q_beam, then the whole chain on <= 64 cells ----
-            if (!sh.err) {
-                // the first half of the warps builds the support of p, the second that of q, side by side
+            {
+                // the first half of the warps builds the support of p, the second that of q, side by side (p alone in the extra layer)
                 const int half = warp / (kHalf / 32);
-                const int e_half = build_support<kHalf>(a, sh, half, hp, hq);
+                const int e_half = extra && half ? 0 : build_support<kHalf>(a, sh, half, hp, hq);
                 if (e_half && (threadIdx.x & (kHalf - 1)) == 0) wsup.tmp[half].err = e_half;
                 __syncthreads();
-                const int e = wsup.tmp[0].err ? wsup.tmp[0].err : wsup.tmp[1].err;
+                const int e = wsup.tmp[0].err ? wsup.tmp[0].err : extra ? 0 : wsup.tmp[1].err;
                 if (e) { if (threadIdx.x == 0) sh.err = e; }
                 else if (warp == 0) {
-                    finish_supports(wsup, true, lane);
+                    finish_supports(wsup, !extra, lane);
                     // rho of every live draft from the warped joints
                     if (!a.select_mode) {
-                        draft_tests(l, m);
+                        draft_tests(sh, a.seed, a.step, r, l, m, lane);
+#pragma unroll 1
                         for (int i = lane; i < m; i += 32) {
                             const int cell = sh.S_parent_idx[i] * a.V + a.token[sh.S[i]];
                             const double pw = support_lookup(wsup, 0, cell), qw = support_lookup(wsup, 1, cell);
@@ -1801,6 +1891,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     const double p1 = lane + 32 < ns ? wsup.prob[0][lane + 32] : 0.0;
                     const double q1 = lane + 32 < ns ? wsup.qat[lane + 32] : 0.0;
                     double s_prev = 0.0, c_cur = 1.0;
+#pragma unroll 1
                     for (int j = 1; j <= m; ++j) {
                         const double s_j = s_prev + c_cur;
                         double acc = fmax(p0 - s_j * q0, 0.0);
@@ -1815,179 +1906,141 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 }
             }
             __syncthreads();
-        } else if (m >= 1 && !sh.err && !a.select_mode && (m <= W_min || W_max <= W_min)) {
-            // ---- the width is W_min whatever the residual masses are (W~ <= m): the drafts are tested at once.  Up to
-            // the first rejection that takes no pass over the rows at all, and every rejection one pass, without a histogram,
-            // whose sums also serve the completion draw.  With more drafts behind the first rejection (on_demand_left) the
-            // histogram is the better way.  (Two live rows of 128256, 4 CTAs: a layer of accepted drafts 5 us instead of 38; a
-            // rejection 16 instead of 37.  Calls, W_min = 2: 64 requests x 8 rows 978 -> 907 us, 16 ragged requests 222 -> 164,
-            // one request of V = 32000 61 -> 53.) ----
-            if (warp == 0) {
-                draft_tests(l, m);
-                const int W = W_min < W_max ? W_min : W_max;
-                int first = m;                         // the first rejection
-                for (int base = 0; base < m && first == m; base += 32) {
-                    const int i = base + lane;
-                    const unsigned rejects = __ballot_sync(kFull, i < m && sh.uu[i] > fmin(sh.rho[i], 1.0));
-                    if (rejects) first = base + __ffs(rejects) - 1;
-                }
-                if (lane == 0) {
-                    sh.on_demand = first >= W || m - 1 - first <= on_demand_left(sh.nA * a.T, n_cta * kVWarps);
-                    sh.need_exact = 0;
-                    if (sh.on_demand) accept_loop(W, true);
-                }
-            }
-            __syncthreads();
-            on_demand = sh.on_demand;
-            while (on_demand && sh.need_exact) {
-                const int j = sh.run_j;
-                const int halves = j == 1 ? item_halves(sh.nA * a.T, n_cta * kVWarps) : 1;   // (slot 0 has room for half tiles)
-                const float half_bin = 0.5f / (float)((double)kBins / log2((double)(m > 2 ? m : 2)));
-                const double c_next = exact_pass(a, sh, sh.s_arr[j], sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride,
-                                                 j == 1, half_bin, halves, true, n_pass++);
-                if (threadIdx.x == 0) {
-                    if (j == 1) sh.halves = halves;
-                    sh.c_arr[j + 1] = c_next;
-                    sh.chain_len = j;
-                    if (c_next > 0.0) sh.run_j = j + 1;
-                    accept_loop(W_min < W_max ? W_min : W_max, true);
+        } else if (m >= 1) {
+            const bool known = !a.select_mode && (m <= W_min || W_max <= W_min);
+            if (known) {
+                // ---- the width is W_min whatever the residual masses are (W~ <= m): the drafts are tested at once.  Up to
+                // the first rejection that takes no pass over the rows at all, and every rejection one pass, without a histogram,
+                // whose sums also serve the completion draw.  With more drafts behind the first rejection (on_demand_left) the
+                // histogram is the better way.  (Two live rows of 128256, 4 CTAs: a layer of accepted drafts 5 us instead of 38; a
+                // rejection 16 instead of 37.  Calls, W_min = 2: 64 requests x 8 rows 978 -> 907 us, 16 ragged requests 222 -> 164,
+                // one request of V = 32000 61 -> 53.) ----
+                if (warp == 0) {
+                    draft_tests(sh, a.seed, a.step, r, l, m, lane);
+                    int first = m;                         // the first rejection
+#pragma unroll 1
+                    for (int base = 0; base < m && first == m; base += 32) {
+                        const int i = base + lane;
+                        const unsigned rejects = __ballot_sync(kFull, i < m && sh.uu[i] > fmin(sh.rho[i], 1.0));
+                        if (rejects) first = base + __ffs(rejects) - 1;
+                    }
+                    if (lane == 0) sh.on_demand = first >= W_known || m - 1 - first <= on_demand_left(sh.nA * a.T, n_cta * kVWarps);
                 }
                 __syncthreads();
+                on_demand = sh.on_demand;
             }
-        }
-        if (m >= 1 && !sh.err && !warped && !on_demand) {
-            // ---- one pass: ratio histogram of the layer over the live rows ----
-            const double top = log2((double)(m > 2 ? m : 2));          // s_j <= j <= m
-            const float binscale = (float)((double)kBins / top);
-            // (counted by histograms, not by layers: the other bank is cleared between the barriers of this one)
-            const int bank = n_hist++ & 1;
-            unsigned long long *tot = sh.w_tot[bank];
-            const int halves = item_halves(sh.nA * a.T, n_cta * kVWarps);
-            histogram_pass(a, sh, binscale, hs, sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride, cta_rank,
-                           n_cta, halves, tot);
-            __syncthreads();
-            hist_fold_over(cluster, hs, tot, n_cta);
-            TS(4);
-            cluster.sync();                            // every CTA's histogram is complete
-            TS(6);
-            if (threadIdx.x < 10) sh.w_tot[bank ^ 1][threadIdx.x] = 0ull;     // the next layer's; nobody adds to it before
-                                                       // the barrier below
-            hist_merge(cluster, hs, sh, cta_rank, n_cta);
-            TS(7);
-            cluster.sync();                            // every slice of the suffix sums is complete
-            TS(5);
-            if (threadIdx.x == 32) sh.halves = halves;
-            if (warp == 1 && !a.select_mode) draft_tests(l, m);
-            // lane c of warp 0: mass of the bins above CTA c's slice
-            unsigned long long above_p = 0ull, above_q = 0ull;
-            double n_cells = 0.0;
-            bool wrapped = false;
-            const int slice = kBins / n_cta;
-            if (warp == 0) {
-                const unsigned long long own_p = lane < n_cta ? sh.slice_p[lane] : 0ull, own_q = lane < n_cta ? sh.slice_q[lane] : 0ull;
-                above_p = own_p; above_q = own_q;
+            const float binscale = sh.binscale[m];
+            if (!on_demand) {
+                // ---- one pass: ratio histogram of the layer over the live rows ----
+                const int halves = item_halves(sh.nA * a.T, n_cta * kVWarps);
+                histogram_pass(a, sh, binscale, hs, sums_base + ((int64_t)sh.bank * (a.max_m + 1)) * slot_stride, cta_rank,
+                               n_cta, halves);
+                __syncthreads();
+                TS(4);
+                hist_suffix(hs, sh);
+                TS(7);
+                cluster.sync();                            // every CTA's suffix sums are complete
+                TS(5);
+                if (threadIdx.x == 32) sh.halves = halves;
+                if (warp == 1 && !a.select_mode && !known) draft_tests(sh, a.seed, a.step, r, l, m, lane);
+            }
+            // The chain c_{j+1} = F(s_j) from sh.chain_pos on (warp 0).  sh.need_exact = 1 where the histogram leaves one open.
+            auto walk_chain = [&]() {
+                int j = sh.chain_pos, need = 0;
+                // lane 2 c + e looks up bin k + e in CTA c
+                const int c = min(lane >> 1, n_cta - 1);
+                const bool has = lane < 2 * n_cta;
+                const uint32_t *words = cluster.map_shared_rank(hs.wp, c) + (lane & 1);
+                const bool wrapped = __any_sync(kFull, *cluster.map_shared_rank(&sh.wrapped, c) != 0);
+                if (lane == 0 && wrapped && j == 1) ++sh.n_wrapped;
+                const double n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
+                double s_j = sh.s_arr[j - 1], c_j = sh.c_arr[j];
+#pragma unroll 1
+                for (; j <= m; ++j) {
+                    s_j += c_j;
+                    if (lane == 0) { sh.s_arr[j] = s_j; sh.chain_len = j; }
+                    // every partial sum of the histogram is off by at most half a unit per cell
+                    const double fix_err = n_cells * (0.5 * kUnfix) * (1.0 + s_j);
+                    if (wrapped) { need = 1; break; }                // a wrapped word: exact passes only
+                    // (up to s = 64 the bin found is off by at most 9e-7 of an edge: the logarithm's last place 3.3e-7, s as a
+                    // float 0.6e-7, the product with binscale 5e-7; an edge by 6e-7.  The bracket below takes the edges
+                    // 2e-6 wider.  Approximate logarithm and exponential, reciprocals for the division: 1 us less, 1.6e-6)
+                    int k = (int)(log2f((float)s_j) * binscale);
+                    if (k < 0 || j == 1) k = 0;                      // s_1 = 1, the first edge
+                    if (k >= kBins) { need = 1; break; }             // cannot happen for s_j <= m
+                    double P = 0.0, Q = 0.0;                         // (whole numbers below 2^46: the sums are exact)
+                    if (has) {
+                        const uint32_t *at = words + k;
+                        P = (double)(((unsigned long long)at[2 * kHistWords] << 32) | at[0]);
+                        Q = (double)(((unsigned long long)at[3 * kHistWords] << 32) | at[kHistWords]);
+                    }
 #pragma unroll
-                for (int o = 1; o < 16; o <<= 1) {
-                    const unsigned long long tp = __shfl_down_sync(kFull, above_p, o), tq = __shfl_down_sync(kFull, above_q, o);
-                    if (lane + o < 32) { above_p += tp; above_q += tq; }
+                    for (int o = 2; o < 32; o <<= 1) {
+                        P += __shfl_xor_sync(kFull, P, o);
+                        Q += __shfl_xor_sync(kFull, Q, o);
+                    }
+                    const double P0 = __shfl_sync(kFull, P, 0), Q0 = __shfl_sync(kFull, Q, 0);
+                    const double P1 = __shfl_sync(kFull, P, 1), Q1 = __shfl_sync(kFull, Q, 1);
+                    double lo_b = 0.0, hi_b = 0.0, c_next;
+                    if (j == 1) c_next = (P0 - Q0) * kUnfix;
+                    else {
+                        const double Pk = (P0 - P1) * kUnfix, Qk = (Q0 - Q1) * kUnfix;
+                        const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
+                        const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
+                        lo_b = fmax(Pk - s_j * Qk, 0.0);
+                        double q_hi = (Pk - r_lo * Qk) / (r_hi - r_lo);
+                        q_hi = fmin(fmax(q_hi, 0.0), Qk);
+                        hi_b = fmax(q_hi * (r_hi - s_j), lo_b);
+                        c_next = fmax(P1 * kUnfix - s_j * (Q1 * kUnfix), 0.0) + 0.5 * (lo_b + hi_b);
+                    }
+                    // the midpoint of the bracket is used: half its width plus the fixed-point term
+                    if (0.5 * (hi_b - lo_b) + fix_err > kErrTol) { need = 1; break; }
+                    if (lane == 0) sh.c_arr[j + 1] = c_next;
+                    c_j = c_next;
+                    if (!(c_next > 0.0)) { j = m; }               // chain exhausted: stop walking
                 }
-                // what all threads added, by their floating-point sums, minus what the words hold.  Without a wrap
-                // that is rounding: half a unit for each cell and 2^-20 of the mass (16 cells in a float sum), less
-                // than 2^26 units; a wrap lowers the words by 2^32
-                wrapped = (long long)(tot[6] - __shfl_sync(kFull, above_p + above_q, 0)) > (1ll << 31);
-                above_p += tot[7] - own_p; above_q += tot[8] - own_q;
-                n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
-                if (lane == 0 && wrapped) ++sh.n_wrapped;
-            }
-            if (warp == 0) {
-                if (lane < n_cta) { sh.above_p[lane] = above_p; sh.above_q[lane] = above_q; }
-                __syncwarp();
-            }
-            // suffix sums of bin k (warp 0; the same on every lane): one word of each kind from the CTA that has it
-            const int shift = 31 - __clz(slice);
-            auto suffix = [&](int k, unsigned long long &P, unsigned long long &Q) {
-                if (k >= kBins) { P = tot[7]; Q = tot[8]; return; }
-                const int c = k >> shift;
-                const uint32_t lp = cluster.map_shared_rank(hs.wp, c)[k], hi_p = cluster.map_shared_rank(hs.bp, c)[k];
-                const uint32_t lq = cluster.map_shared_rank(hs.wq, c)[k], hi_q = cluster.map_shared_rank(hs.bq, c)[k];
-                P = (((unsigned long long)hi_p << 32) | lp) + sh.above_p[c];
-                Q = (((unsigned long long)hi_q << 32) | lq) + sh.above_q[c];
+                if (lane == 0) {
+                    sh.need_exact = need;
+                    sh.chain_pos = need ? j : m + 1;
+                }
             };
-
-            int j0 = 1;
-            while (j0 <= m) {
+            // ---- the residual masses, and (on demand) the accept loop between them ----
+#pragma unroll 1
+            while (true) {
                 if (warp == 0) {
-                    int j = j0;
-                    int need = 0;
-                    double s_j = sh.s_arr[j - 1], c_j = sh.c_arr[j];
-                    for (; j <= m; ++j) {
-                        s_j += c_j;
-                        if (lane == 0) { sh.s_arr[j] = s_j; sh.chain_len = j; }
-                        double c_next;
-                        // every partial sum of the histogram is off by at most half a unit per cell
-                        const double fix_err = n_cells * (0.5 * kUnfix) * (1.0 + s_j);
-                        if (wrapped) { need = 1; break; }                // a wrapped word: exact passes only
-                        unsigned long long P[2], Q[2];
-                        if (j == 1) {
-                            P[0] = __shfl_sync(kFull, above_p, 0) + sh.slice_p[0];
-                            Q[0] = __shfl_sync(kFull, above_q, 0) + sh.slice_q[0];
-                            c_next = ((double)P[0] - (double)Q[0]) * kUnfix;
-                            if (fix_err > kErrTol) { need = 1; break; }
-                        } else {
-                            // (up to s = 64 the bin found is off by at most 9e-7 of an edge: the logarithm's last place 3.3e-7, s as a
-                            // float 0.6e-7, the product with binscale 5e-7; an edge by 6e-7.  The bracket below takes the edges
-                            // 2e-6 wider.  Approximate logarithm and exponential, reciprocals for the division: 1 us less, 1.6e-6)
-                            int k = (int)(log2f((float)s_j) * binscale);
-                            if (k < 0) k = 0;
-                            if (k >= kBins) { need = 1; break; }     // cannot happen for s_j <= m
-                            suffix(k, P[0], Q[0]);
-                            suffix(k + 1, P[1], Q[1]);
-                            const double Pa = (double)P[1] * kUnfix, Qa = (double)Q[1] * kUnfix;
-                            const double Pk = (double)(P[0] - P[1]) * kUnfix;
-                            const double Qk = (double)(Q[0] - Q[1]) * kUnfix;
-                            const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
-                            const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
-                            const double lo_b = fmax(Pk - s_j * Qk, 0.0);
-                            double q_hi = (Pk - r_lo * Qk) / (r_hi - r_lo);
-                            q_hi = fmin(fmax(q_hi, 0.0), Qk);
-                            const double hi_b = fmax(q_hi * (r_hi - s_j), lo_b);
-                            // the midpoint of the bracket is used: half its width plus the fixed-point term
-                            if (0.5 * (hi_b - lo_b) + fix_err > kErrTol) { need = 1; break; }
-                            c_next = fmax(Pa - s_j * Qa, 0.0) + 0.5 * (lo_b + hi_b);
-                        }
-                        if (lane == 0) sh.c_arr[j + 1] = c_next;
-                        c_j = c_next;
-                        if (!(c_next > 0.0)) { j = m; }               // chain exhausted: stop walking
-                    }
-                    if (lane == 0) {
-                        sh.need_exact = need;
-                        sh.chain_pos = need ? j : m + 1;
-                    }
+                    if (on_demand) accept_drafts(sh, st, writer ? a.out.node_status : nullptr, n_lo, m, W_known, true, lane);
+                    else walk_chain();
                 }
                 __syncthreads();
                 if (!sh.need_exact) break;
                 const int j = sh.chain_pos;
-                if (threadIdx.x == 0) ++sh.n_exact;
-                // (at j = 1 these are the sums that the histogram pass left in slot 0)
-                double *sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride;
-                if (j == 1 && threadIdx.x == 0) sh.halves = 1;
-                const double c_next = exact_pass(a, sh, sh.s_arr[j], sums, false, 0.f, 1, true, n_pass++);
-                if (threadIdx.x == 0) sh.c_arr[j + 1] = c_next;
+                const bool first = on_demand && j == 1;
+                // (in a layer with a histogram that pass left the sums at j = 1 in slot 0; half tiles have room there only)
+                const int halves = first ? item_halves(sh.nA * a.T, n_cta * kVWarps) : 1;
+                const double c_next = exact_pass(a, sh, sh.s_arr[j], sums_base + ((int64_t)sh.bank * (a.max_m + 1) + (j == 1 ? 0 : j)) * slot_stride,
+                                                 first, 0.5f / binscale, halves, true, n_pass++);
+                if (threadIdx.x == 0) {
+                    if (j == 1) sh.halves = halves;
+                    sh.c_arr[j + 1] = c_next;
+                    sh.chain_len = j;
+                    if (!on_demand) { ++sh.n_exact; sh.chain_pos = c_next > 0.0 ? j + 1 : m + 1; }
+                    else if (c_next > 0.0) sh.run_j = j + 1;
+                }
                 __syncthreads();
-                if (!(sh.c_arr[j + 1] > 0.0)) break;
-                j0 = j + 1;
             }
-            cluster.barrier_arrive();                  // this CTA has done with the others' slices
-            looked_up = true;
+            if (!on_demand) {
+                cluster.barrier_arrive();                  // this CTA has done with the others' sums
+                looked_up = true;
+            }
         }
-        __syncthreads();
 
         TS(8);
         // ---- width and accept loop (warp 0) ----
         if (warp == 0 && !sh.err) {
-            int W = W_min < W_max ? W_min : W_max;
-            if (!on_demand) {
+            int W = W_known;
+            if (!on_demand && !extra) {
                 // alpha_j = 1 - c_{j+1}/c_j; once a residual has no mass every later alpha is 1
+#pragma unroll 1
                 for (int j = 1 + lane; j <= m; j += 32) {
                     double al = 1.0;
                     if (j <= sh.chain_len && sh.c_arr[j] > 0.0 && sh.c_arr[j + 1] > 0.0)
@@ -2005,32 +2058,34 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 if (writer && lane == 0) {
                     a.width_out[r] = W;
                     if (a.alpha_out)
+#pragma unroll 1
                         for (int j = 0; j < m && j < a.out_stride; ++j)
                             a.alpha_out[(int64_t)r * a.out_stride + j] = (float)sh.alpha[j + 1];
                     if (a.tail_out)
+#pragma unroll 1
                         for (int K = 0; K <= m && K < a.out_stride; ++K)
                             a.tail_out[(int64_t)r * a.out_stride + K] = (float)sh.tail[K];
                 }
-                if (lane == 0) sh.done = 1;
-            } else if (lane == 0) {
-                if (writer) a.out.layer_width[(int64_t)r * (a.gamma + 1) + (l - 1)] = W;
-                if (!on_demand) accept_loop(W, false);
-                const int count = sh.count, j = sh.run_j;
-                for (int i = 0; i < m; ++i)
-                    if (st[sh.S[i] - n_lo] == DSBD_NODE_UNREACHED) {
-                        st[sh.S[i] - n_lo] = DSBD_NODE_CUT;
-                        if (writer) a.out.node_status[sh.S[i]] = DSBD_NODE_CUT;
-                    }
-                sh.W = W;
-                if (m >= 1 && (!on_demand || sh.chain_len > 0)) sh.n_rows += sh.nA;
-                ++sh.n_layers;
-                // a residual draw at run position j needs tile sums (a layer of known width has them)
-                sh.res_j = (count < W && j > 1 && !on_demand) ? j : 0;
+            } else {
+                if (!on_demand) accept_drafts(sh, st, writer ? a.out.node_status : nullptr, n_lo, m, W, false, lane);
+#pragma unroll 1
+                for (int i = sh.next_i + lane; i < m; i += 32) {
+                    st[sh.S[i] - n_lo] = DSBD_NODE_CUT;
+                    if (writer) a.out.node_status[sh.S[i]] = DSBD_NODE_CUT;
+                }
+                if (lane == 0) {
+                    if (writer) a.out.layer_width[(int64_t)r * (a.gamma + 1) + (l - 1)] = W;
+                    sh.W = W;
+                    if (m >= 1 && (!on_demand || sh.chain_len > 0)) sh.n_rows += sh.nA;
+                    if (!extra) ++sh.n_layers;
+                    // a residual draw at run position j needs tile sums (a layer of known width has them)
+                    sh.res_j = (sh.count < W && sh.run_j > 1 && !on_demand) ? sh.run_j : 0;
+                }
             }
         }
         __syncthreads();
 
-        if (looked_up) cluster.barrier_wait();         // the others have done with this CTA's slice
+        if (looked_up) cluster.barrier_wait();         // the others have done with this CTA's sums
         TS(9);
         // ---- a residual draw locates its tile through tile sums of max(p_beam - s_{j-1} q_beam, 0) ----
         // slot 0 of the bank; in a layer of known width that of the rejection before the draw
@@ -2042,55 +2097,12 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         }
 
         TS(10);
-        // ---- completion of a short layer, or the next layer's input beams (warp 0) ----
-        if (warp == 0 && !a.select_mode && !sh.err) {
-            const int W = sh.W, count = sh.count, j = sh.run_j;
-            int err = 0;
-            if (count < W) {
-                // accepted drafts, then the residual draw, then fills from p_beam, all independent of one another:
-                // spread over lanes when the joint is warped, else over the warps of the CTA (below)
-                const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
-                const NodeCache *cache = cached ? &nc : nullptr;
-                const int n_acc = min(count, max(cap - n_out, 0));
-                if (writer)
-                    for (int i = lane; i < n_acc; i += 32)
-                        emit_at(a, r, n_out + i, a.parent[sh.acc[i]], sh.acc[i], a.token[sh.acc[i]], DSBD_SRC_DRAFT, cache,
-                                n_lo);
-                n_out += n_acc;
-                if (n_acc < count) err = DSBD_DEV_CAPACITY;
-                const bool use_res = j > 1;
-                if (warped && !err) {
-                    const int want = W - count, n_draw = min(want, max(cap - n_out, 0));
-                    for (int k0 = 0; k0 < n_draw; k0 += 32) {
-                        const int kk = k0 + lane;
-                        const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, kk ? 2u : 1u,
-                                                          kk ? (uint32_t)(kk - 1) : 0u);
-                        int pick = draw_support(wsup, u, 0.0, lane);
-                        if (k0 == 0 && use_res) {
-                            const int of_res = draw_support(wsup, u, sh.s_arr[j - 1], lane);
-                            if (kk == 0) pick = of_res;
-                        }
-                        if (kk >= n_draw) continue;
-                        if (pick < 0) { err = DSBD_DEV_EXHAUSTED; continue; }
-                        const int ia = wsup.cell[0][pick] / a.V, tok = wsup.cell[0][pick] - ia * a.V;
-                        if (writer)
-                            emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, kk ? DSBD_SRC_FILL : DSBD_SRC_RESIDUAL, cache, n_lo);
-                    }
-                    if (__any_sync(kFull, err)) err = DSBD_DEV_EXHAUSTED;
-                    else {
-                        n_out += n_draw;
-                        if (n_draw < want) err = DSBD_DEV_CAPACITY;
-                    }
-                }
-                if (lane == 0) {
-                    sh.done = 1;
-                    if (writer) a.out.l_last[r] = l;
-                    sh.n_out = n_out;
-                    sh.n_fill = (!warped && !err) ? W - count : 0;
-                }
-            } else {
-                // the accepted drafts, ascending node id, are the next layer's input beams
+        if (a.select_mode || sh.err) break;
+        if (sh.count >= sh.W) {
+            // ---- the accepted drafts, ascending node id, are the next layer's input beams (warp 0) ----
+            if (warp == 0) {
                 int nA = 0;
+#pragma unroll 1
                 for (int base = 0; base < n_req_nodes; base += 32) {
                     const int n = base + lane;
                     const bool in = n < n_req_nodes && nd_depth(n) == l && st[n] == DSBD_NODE_ACCEPTED;
@@ -2105,97 +2117,68 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 }
                 if (lane == 0) sh.nA = nA;
             }
-            if (lane == 0 && err) sh.err = err;
-        }
-        __syncthreads();
-        if (writer && !a.select_mode && sh.done && sh.n_fill > 0 && !sh.err) {
-            // draw f is output beam n_out + f: the residual draw at the run position where the layer ended, then the
-            // fills from p_beam, each with its own uniform
-            const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
-            const int base = sh.n_out, want = sh.n_fill, j = sh.run_j;
-            const int n_draw = min(want, max(cap - base, 0));
             __syncthreads();
-            for (int f = warp; f < n_draw; f += kVWarps) {
-                const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, f ? 2u : 1u, f ? (uint32_t)(f - 1) : 0u);
-                const bool use_res = f == 0 && j > 1;
+            continue;
+        }
+        // ---- a short layer ends the request: accepted drafts, then the residual draw, then fills from p_beam (in the extra layer
+        // draws from p_beam alone), all independent of one another: a warp for each ----
+        if (!writer) break;
+        const int count = sh.count, want = sh.W - count, j = sh.run_j;
+        const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
+        const int n_acc = min(count, max(cap, 0)), n_draw = n_acc < count ? 0 : min(want, max(cap - n_acc, 0));
+        const bool use_res = j > 1;
+        const int halves = res_slot ? 1 : sh.halves;
+        float *words = reinterpret_cast<float *>(hp) + warp * kTokWords;
+        double *parts = reinterpret_cast<double *>(reinterpret_cast<float *>(hp) + kVWarps * kTokWords);
+        if (!warped && use_res) {
+            draw_shares(res_sums, halves, sh.nA * a.T, parts);
+            __syncthreads();
+        }
+#pragma unroll 1
+        for (int b = warp; b < n_acc + n_draw; b += kVWarps) {
+            int parent, node = -1, tok, source = DSBD_SRC_DRAFT;
+            if (b < n_acc) {
+                node = sh.acc[b];
+                parent = a.parent[node];
+                tok = a.token[node];
+            } else {
+                // draw f: the residual draw at the run position where the layer ended, then the fills, each with its own uniform
+                const int f = b - n_acc;
+                const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, extra ? 3u : f ? 2u : 1u,
+                                                  extra || !f ? (uint32_t)f : (uint32_t)(f - 1));
+                const bool res = f == 0 && use_res;
+                source = extra ? DSBD_SRC_EXTRA : f ? DSBD_SRC_FILL : DSBD_SRC_RESIDUAL;
                 int ia = 0;
-                const int tok = draw_cell(a, sh, u, use_res, use_res ? (float)sh.s_arr[j - 1] : 0.f, res_sums, res_slot ? 1 : sh.halves, lane, &ia);
-                if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
-                else if (lane == 0)
-                    emit_at(a, r, base + f, sh.A[ia], -1, tok, f ? DSBD_SRC_FILL : DSBD_SRC_RESIDUAL, cached ? &nc : nullptr, n_lo);
+                if (warped) {
+                    const int pick = draw_support(wsup, u, res ? sh.s_arr[j - 1] : 0.0, lane);
+                    tok = -1;
+                    if (pick >= 0) { ia = wsup.cell[0][pick] / a.V; tok = wsup.cell[0][pick] - ia * a.V; }
+                } else {
+                    tok = draw_cell(a, sh, u, res, res ? (float)sh.s_arr[j - 1] : 0.f, res_sums, halves, parts, words, lane, &ia);
+                }
+                parent = sh.A[ia];
             }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                if (!sh.err) { sh.n_out = base + n_draw; if (want > n_draw) sh.err = DSBD_DEV_CAPACITY; }
-                sh.n_fill = 0;
+            if (lane == 0) {
+                if (tok < 0) sh.n_draw = -1;
+                else emit_at(a, r, b, parent, node, tok, source, cached ? &nc : nullptr, n_lo);
             }
-            __syncthreads();
-            n_out = sh.n_out;
-        }
-    }
-
-    TS(11);
-    // ---- every layer passed: W_nom beams from p_beam^(gamma+1) ----
-    const bool extra = writer && !a.select_mode && !sh.done && !sh.err;
-    WarpScratch &wsx = *reinterpret_cast<WarpScratch *>(hq);
-    int extra_err = 0;
-    if (extra) {
-        if (warp < 2) live_weights(a, sh, warp, warp == 0 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
-        __syncthreads();
-        if (kWarped) {
-            extra_err = build_support<kVThreads>(a, sh, 0, hp, hq);       // one model only: by the whole CTA
-            if (!extra_err && warp == 0) finish_supports(wsx, false, lane);
-        }
-    }
-    if (extra && !kWarped) {
-        // W_nom independent draws from p_beam, one warp each
-        const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
-        const int n_draw = min(W_nom, max(cap - n_out, 0));
-        if (threadIdx.x == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
-        for (int kk = warp; kk < n_draw; kk += kVWarps) {
-            const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1), 3u,
-                                              (uint32_t)kk);
-            int ia = 0;
-            const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, 1, lane, &ia);
-            if (tok < 0) { if (lane == 0) sh.err = DSBD_DEV_EXHAUSTED; }
-            else if (lane == 0)
-                emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
         }
         __syncthreads();
-        if (!sh.err) {
-            n_out += n_draw;
-            if (W_nom > n_draw && threadIdx.x == 0) sh.err = DSBD_DEV_CAPACITY;
-        }
-    } else if (extra && warp == 0) {
-        // independent draws from the support, one lane each
-        int err = extra_err;
-        if (lane == 0) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;
-        const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
-        const int n_draw = err ? 0 : min(W_nom, max(cap - n_out, 0));
-        for (int k0 = 0; k0 < n_draw; k0 += 32) {
-            const int kk = k0 + lane;
-            const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)(a.gamma + 1), 3u,
-                                              (uint32_t)kk);
-            const int pick = draw_support(wsx, u, 0.0, lane);
-            if (kk >= n_draw) continue;
-            if (pick < 0) { err = DSBD_DEV_EXHAUSTED; continue; }
-            const int ia = wsx.cell[0][pick] / a.V, tok = wsx.cell[0][pick] - ia * a.V;
-            emit_at(a, r, n_out + kk, sh.A[ia], -1, tok, DSBD_SRC_EXTRA, cached ? &nc : nullptr, n_lo);
-        }
-        if (!extra_err) {
-            if (__any_sync(kFull, err)) err = DSBD_DEV_EXHAUSTED;
+        if (threadIdx.x == 0) {
+            a.out.l_last[r] = l;
+            if (sh.n_draw < 0) { sh.err = DSBD_DEV_EXHAUSTED; sh.n_out = n_acc; }
             else {
-                n_out += n_draw;
-                if (n_draw < W_nom) err = DSBD_DEV_CAPACITY;
+                sh.n_out = n_acc + n_draw;
+                if (n_acc < count || n_draw < want) sh.err = DSBD_DEV_CAPACITY;
             }
         }
-        if (lane == 0 && err) sh.err = err;
+        break;
     }
     __syncthreads();
-    TS(12);
+    TS(11);
     if (threadIdx.x == 0 && writer) {
         if (!a.select_mode) {
-            a.out.out_width[r] = n_out;
+            a.out.out_width[r] = sh.n_out;
             if (a.out.req_error) a.out.req_error[r] = sh.err;
             if (a.out.req_stats) {
                 int32_t *rs = a.out.req_stats + (int64_t)DSBD_REQ_STATS * r;
@@ -2458,6 +2441,7 @@ k_draft(const __grid_constant__ DraftArgs d) {
     }
     if (threadIdx.x == 0) { sh.nA = nA; s_err = 0; }
     asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll 1
     for (int i = warp; i < nA; i += kVWarps) {
         const double v = row_lse(a.stats + (int64_t)(b_lo + i) * a.T, a.T, a.inv_tau, lane);
         if (lane == 0) { lse[i] = v; a.lse_w[b_lo + i] = v; }
@@ -2477,6 +2461,7 @@ k_draft(const __grid_constant__ DraftArgs d) {
         if (!err) err = build_support<kVThreads>(a, sh, 0, hp, hq);
         if (!err && warp == 0) {
             finish_supports(ws, false, lane);
+#pragma unroll 1
             for (int k0 = 0; k0 < n_draw; k0 += 32) {
                 const int kk = k0 + lane;
                 const double u = decision_uniform(a.seed, a.step, (uint32_t)r, d.layer, 3u, (uint32_t)kk);
@@ -2488,10 +2473,11 @@ k_draft(const __grid_constant__ DraftArgs d) {
             }
         }
     } else {
+#pragma unroll 1
         for (int kk = warp; kk < n_draw; kk += kVWarps) {
             const double u = decision_uniform(a.seed, a.step, (uint32_t)r, d.layer, 3u, (uint32_t)kk);
             int ia = 0;
-            const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, 1, lane, &ia);
+            const int tok = draw_cell(a, sh, u, false, 0.f, nullptr, 1, nullptr, reinterpret_cast<float *>(hp) + warp * kTokWords, lane, &ia);
             if (lane == 0) {
                 if (tok < 0) s_err = DSBD_DEV_EXHAUSTED;
                 else emit(kk, ia, tok);
@@ -2575,9 +2561,9 @@ extern "C" int dsbd_draft_layer(int32_t R, int32_t n_beams, const int32_t *req_b
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)R);
     cfg.blockDim = dim3(kVThreads);
-    cfg.dynamicSmemBytes = p->top_k > 0 ? kVerifyDynSmem : 0;           // the support's scratch
+    cfg.dynamicSmemBytes = kVerifyDynSmem;                             // the support's scratch, or what the draws search
     cfg.stream = stream;
-    if (p->top_k > 0 && cudaFuncSetAttribute(k_draft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_draft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess)
         return DSBD_ERR_CUDA;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;       // see launch_verify

@@ -49,6 +49,12 @@ constexpr int kMaxLive = DSBD_MAX_LIVE;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr double kLn2 = 0.6931471805599453;
 
+// The value of lane 0, for one that all lanes of the warp have: the compiler then knows that a branch on it leaves the warp together.
+// Behind a branch on a thread index, a function's argument or a word of memory it does not, and gathers the lanes anew for every
+// shuffle: about 300 cycles each instead of 23, and three times the code (a warp_sum of doubles 1.5 us instead of 0.12).
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(kFull, x, 0); }
+__device__ __forceinline__ int warp_index() { return uniform((int)(threadIdx.x >> 5)); }
+
 // A load before griddepcontrol.wait: from L2.
 template <class V>
 __device__ __forceinline__ V ld_early(const V *p) { return __ldcg(p); }
@@ -115,16 +121,16 @@ k_tile_stats(const float *zp, const float *zq, int64_t stride, int V, int T, int
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    if (n_rows_dev) n_rows = min(max(*n_rows_dev, 0), n_rows);
+    const int64_t warp = (int64_t)blockIdx.x * kWarps + warp_index();
+    const int64_t nwarps = (int64_t)gridDim.x * kWarps;
+    if (n_rows_dev) n_rows = uniform(min(max(*n_rows_dev, 0), n_rows));
     const int64_t total = (int64_t)(one_model ? 1 : 2) * n_rows * T;
     for (int64_t item = warp; item < total; item += nwarps) {
         const int t = (int)(item % T);
         const int64_t rm = item / T;
         const int model = (int)(rm / n_rows);
         const int ri = (int)(rm % n_rows);
-        const int row = rows ? rows[ri] : ri;
+        const int row = rows ? uniform(rows[ri]) : ri;
         if (row < 0 || row >= N) continue;
         const float *z = (model ? zq : zp) + (int64_t)row * stride;
         const bool aligned = (reinterpret_cast<uintptr_t>(z) & 15) == 0;
@@ -165,12 +171,14 @@ k_tile_stats(const float *zp, const float *zq, int64_t stride, int V, int T, int
 __device__ __forceinline__ double row_lse(const TileStat *s, int T, double inv_tau, int lane) {
     float top = -INFINITY;
 #pragma unroll 4
-    for (int t = lane; t < T; t += 32) top = fmaxf(top, s[t].mx);
+    for (int t0 = 0; t0 < T; t0 += 32)
+        if (const int t = t0 + lane; t < T) top = fmaxf(top, s[t].mx);
     const double mx = (double)warp_max(top);
     double acc = 0.0;
     if (mx > -INFINITY)
 #pragma unroll 1
-        for (int t = lane; t < T; t += 32)
+        for (int t0 = 0; t0 < T; t0 += 32)
+            if (const int t = t0 + lane; t < T)
             if (s[t].sum > 0.f) acc += (double)s[t].sum * exp(((double)s[t].mx - mx) * inv_tau);
     acc = warp_sum(acc);
     return (mx > -INFINITY) ? mx * inv_tau + log(acc) : -INFINITY;
@@ -182,12 +190,12 @@ __global__ void k_row_finish(const TileStat *__restrict__ stats, int T, int N, i
                              double inv_tau, double *__restrict__ lse /*[2][N]*/,
                              float *__restrict__ lse_p_out, float *__restrict__ lse_q_out) {
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (n_rows_dev) n_rows = min(max(*n_rows_dev, 0), n_rows);
+    const int64_t warp = (int64_t)blockIdx.x * kWarps + warp_index();
+    if (n_rows_dev) n_rows = uniform(min(max(*n_rows_dev, 0), n_rows));
     if (warp >= (int64_t)2 * n_rows) return;
     const int model = (int)(warp / n_rows);
     const int ri = (int)(warp % n_rows);
-    const int row = rows ? rows[ri] : ri;
+    const int row = rows ? uniform(rows[ri]) : ri;
     if (row < 0 || row >= N) return;
     const double v = row_lse(stats + ((int64_t)model * N + row) * T, T, inv_tau, lane);
     if (lane == 0) {
@@ -325,7 +333,7 @@ __device__ __forceinline__ void one_copy(int &x) { asm volatile("" : "+r"(x)); }
 // One copy for all searches of a kernel, over weights that its callers have put side by side: text is what a draw waits for
 // (a search of its own in global memory for each kind of weight, unrolled: 24 KB, and 17 KB for the search inside a tile).
 __device__ __noinline__ int locate(const double *w, int n, double &target, bool of_total, bool open, int lane) {
-    int lo = 0, len = n, scale = of_total, go_on = open;
+    int lo = 0, len = uniform(n), scale = uniform(of_total), go_on = uniform(open);
 #pragma unroll 1
     while (true) {
         one_copy(scale); one_copy(go_on);
@@ -359,7 +367,7 @@ __device__ __noinline__ int locate_token(const float *__restrict__ rp, const flo
                                          int t, const RowOff ro, float s, double target, int lane, float *mass) {
     const int e0 = t * kTile, n = min(kTile, V - e0);
     rp += e0; rq += e0;
-    const bool res = s > 0.f;
+    const bool res = uniform(s > 0.f);
     float first_of[8];                               // (of a sector; all in flight together)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -452,15 +460,18 @@ __device__ __forceinline__ void emit_at(const VerifyArgs &a, int r, int index, i
 __device__ __forceinline__ void log_softmax_warp(const double *s, int n, int lane, double *out) {
     double mx = -INFINITY;
 #pragma unroll 1
-    for (int i = lane; i < n; i += 32) mx = fmax(mx, s[i]);
+    for (int i0 = 0; i0 < n; i0 += 32)
+        if (const int i = i0 + lane; i < n) mx = fmax(mx, s[i]);
     mx = warp_max(mx);
     double t = 0.0;
 #pragma unroll 1
-    for (int i = lane; i < n; i += 32) t += exp(s[i] - mx);
+    for (int i0 = 0; i0 < n; i0 += 32)
+        if (const int i = i0 + lane; i < n) t += exp(s[i] - mx);
     t = warp_sum(t);
     const double lt = log(t);
 #pragma unroll 1
-    for (int i = lane; i < n; i += 32) out[i] = (s[i] - mx) - lt;
+    for (int i0 = 0; i0 < n; i0 += 32)
+        if (const int i = i0 + lane; i < n) out[i] = (s[i] - mx) - lt;
     __syncwarp();
 }
 
@@ -470,10 +481,13 @@ __device__ __forceinline__ void log_softmax_warp(const double *s, int n, int lan
 __device__ void live_weights(const VerifyArgs &a, Shared &sh, int model, const double *scores, int lane,
                              const NodeCache *nc, int n_lo) {
     double *lw = model ? sh.lwq : sh.lwp;
-    log_softmax_warp(scores, sh.nA, lane, lw);
+    const int nA = uniform(sh.nA);
+    log_softmax_warp(scores, nA, lane, lw);
     const double *lse = nc ? (model ? nc->lse_q : nc->lse_p) - n_lo : a.lse + (int64_t)model * a.N;
 #pragma unroll 1
-    for (int i = lane; i < sh.nA; i += 32) {
+    for (int i0 = 0; i0 < nA; i0 += 32) {
+        const int i = i0 + lane;
+        if (i >= nA) continue;
         if (!model) sh.wp[i] = exp(lw[i]);
         split_offset((lw[i] - lse[sh.A[i]]) * (1.0 / kLn2), model ? &sh.bq[i] : &sh.bp[i],
                      model ? &sh.cq[i] : &sh.cp[i], model ? &sh.rq[i] : &sh.rp[i]);
@@ -506,18 +520,20 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
         if (lane == 0) sh.tail[k + 1] = 1.0 - below;
         if (k == m) break;
         // tails only fall: past the first one below the threshold, or past the cap, nothing changes W
-        if (k_stop >= 0 && (1.0 - below < thresh || k + 1 >= k_stop)) {
+        if (k_stop >= 0 && (uniform(1.0 - below < thresh) || k + 1 >= k_stop)) {
 #pragma unroll 1
-            for (int K = k + 2 + lane; K <= m + 1; K += 32) sh.tail[K] = 0.0;
+            for (int K0 = k + 2; K0 <= m + 1; K0 += 32)
+                if (K0 + lane <= m + 1) sh.tail[K0 + lane] = 0.0;
             break;
         }
 #pragma unroll 1
-        for (int n = lane; n <= m; n += 32) {
+        for (int n0 = 0; n0 <= m; n0 += 32) {
+            const int n = n0 + lane;
             double acc = 0.0;
-            if (n >= k + 1)
 #pragma unroll 2
-                for (int i = 1; i <= n; ++i) acc += sh.first[i] * prev[n - i];
-            cur[n] = acc;                          // P(n, k+1), zero for n < k+1
+            for (int i = 1; i <= m; ++i)
+                if (i <= n && n <= m) acc += sh.first[i] * prev[n - i];
+            if (n <= m) cur[n] = n > k ? acc : 0.0;         // P(n, k+1), zero for n < k+1
         }
         __syncwarp();
         double *tmp = prev; prev = cur; cur = tmp;
@@ -738,16 +754,18 @@ __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const f
                                                 int V, int T, float k2, Shared &sh, float s, float half_bin, double *sums,
                                                 int warp, int nwarps, int halves) {
     const int lane = threadIdx.x & 31;
-    const int row_items = T * halves, items = sh.nA * row_items;
+    nwarps = uniform(nwarps); halves = uniform(halves);
+    const int row_items = T * halves, items = uniform(sh.nA * row_items);
     if (lane < 3) sh.warp_part[lane][threadIdx.x >> 5] = 0ll;
     __syncwarp();
     long long units = 0ll;
-    for (int item = warp; item < items; item += nwarps) {
+    for (int item = uniform(warp); item < items; item += nwarps) {
         const int i = item / row_items, t = item - i * row_items;
-        const int row = sh.A[i];
+        const int row = uniform(sh.A[i]);
         const float *rp = zp + (int64_t)row * stride;
         const float *rq = zq + (int64_t)row * stride;
-        const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
+        const bool al = uniform(((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0);
+        V = uniform(V);
         const RowOff ro = row_off(sh, i);
         double res1 = 0.0;
         float acc = 0.f, q_acc = 0.f;
@@ -816,8 +834,8 @@ __device__ __noinline__ void residual_pass(const float *__restrict__ zp, const f
 __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, double s, double *sums, bool first, float half_bin,
                                           int halves, bool want_total, int n_pass) {
     cg::cluster_group cluster = cg::this_cluster();
-    const int n_cta = (int)cluster.num_blocks(), cta_rank = (int)cluster.block_rank();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_cta = uniform((int)cluster.num_blocks()), cta_rank = uniform((int)cluster.block_rank());
+    const int lane = threadIdx.x & 31, warp = warp_index();
     const float s_hi = (float)s;
     const int w = cta_rank * kVWarps + warp, nw = n_cta * kVWarps;
     if (first) residual_pass<true, true>(a.zp, a.zq, a.stride, a.V, a.T, a.k2, sh, s_hi, half_bin, sums, w, nw, halves);
@@ -854,9 +872,9 @@ __device__ __forceinline__ void histogram_pass(const VerifyArgs &a, Shared &sh, 
                                double *sums1, int cta_rank, int n_cta, int halves) {
     // halves = 2: an item is a half tile (when the cluster has a warp for each), with a sum of its own
     const int lane = threadIdx.x & 31;
-    const int warp = cta_rank * kVWarps + (threadIdx.x >> 5);
+    const int warp = cta_rank * kVWarps + warp_index();
     const int nwarps = n_cta * kVWarps;
-    const int items = sh.nA * a.T * halves;
+    const int items = uniform(sh.nA) * a.T * halves;
     unsigned long long added = 0ull;
     const uint32_t magic_bits = __float_as_uint(kBinMagic);
     const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(h.wp) - (magic_bits << 2);
@@ -866,7 +884,7 @@ __device__ __forceinline__ void histogram_pass(const VerifyArgs &a, Shared &sh, 
     const int row_items = a.T * halves;
     for (int item = warp; item < items; item += nwarps) {
         const int i = item / row_items, t = item - i * row_items;
-        const int row = sh.A[i];
+        const int row = uniform(sh.A[i]);
         const float *rp = a.zp + (int64_t)row * a.stride;
         const float *rq = a.zq + (int64_t)row * a.stride;
         const bool al = ((reinterpret_cast<uintptr_t>(rp) | reinterpret_cast<uintptr_t>(rq)) & 15) == 0;
@@ -907,7 +925,7 @@ __device__ __forceinline__ void histogram_pass(const VerifyArgs &a, Shared &sh, 
 // anybody looks at).
 static_assert(kBins == 8 * kVThreads, "eight bins to a thread");
 __device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i0 = threadIdx.x * 8;
+    const int lane = threadIdx.x & 31, warp = warp_index(), i0 = threadIdx.x * 8;
     unsigned long long v[2][8];                              // p, q
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
@@ -968,8 +986,11 @@ __device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
 
 // Per live draft of layer l: rho = p_beam/q_beam of its cell and its uniform, by one warp.
 __device__ __noinline__ void draft_tests(Shared &sh, uint64_t seed, uint64_t step, int r, int l, int m, int lane) {
+    m = uniform(m);
 #pragma unroll 1
-    for (int i = lane; i < m; i += 32) {
+    for (int i0 = 0; i0 < m; i0 += 32) {
+        const int i = i0 + lane;
+        if (i >= m) continue;
         const int ai = sh.S_parent_idx[i];
         const double lp = sh.rho[i], lq = sh.uu[i];
         double rho;
@@ -989,8 +1010,9 @@ __device__ __noinline__ void draft_tests(Shared &sh, uint64_t seed, uint64_t ste
 // on_demand: ends with sh.need_exact = 1 after a rejection whose residual mass c_{j+1} is not known yet.
 // node_status: nullptr in a CTA that writes no results.
 __device__ __noinline__ void accept_drafts(Shared &sh, int8_t *st, int8_t *node_status, int n_lo, int m, int W, bool on_demand, int lane) {
-    int i = sh.next_i, count = sh.count, j = sh.run_j, tests = 0, near = 0, need = 0;
-    const int len = sh.chain_len;
+    int i = uniform(sh.next_i), count = uniform(sh.count), j = uniform(sh.run_j), tests = 0, near = 0, need = 0;
+    const int len = uniform(sh.chain_len);
+    m = uniform(m); W = uniform(W); on_demand = uniform(on_demand);
 #pragma unroll 1
     while (i < m && count < W && !need) {
         const int n = min(m - i, 32);
@@ -1054,46 +1076,35 @@ __device__ __forceinline__ int draw_cell(const VerifyArgs &a, const Shared &sh, 
                                          const double *res_sums, int halves, const double *parts, float *words, int lane, int *ia_out) {
     double *piece = reinterpret_cast<double *>(words);
     double target = u;
-    int ia, t = 0;
-    int n = a.T;                                     // tile masses to search, from `at` on
-    int at = 0;
-    double wpa = 0.0, lse_row = 0.0;
-    const TileStat *st = a.stats;
-    if (use_res) {
-        // (res_sums: one per tile, or two when the pass that wrote them worked on half tiles)
-        const int tiles = sh.nA * a.T, per = (tiles + kParts - 1) / kParts;
-        at = locate(parts, kParts, target, true, false, lane);
-        if (at < 0) return -1;
-        at *= per;
-        n = min(per, tiles - at);
-        ia = 0;
-    } else {
-        // p_beam: first the live parent (its row holds exactly its beam weight), then the tile
-        ia = locate(sh.wp, sh.nA, target, true, false, lane);
-        if (ia < 0) return -1;
-        const int row = sh.A[ia];
-        wpa = sh.wp[ia]; lse_row = a.lse[row];
-        st += (int64_t)row * a.T;
-    }
+    // p_beam: first the live parent (its row holds exactly its beam weight), then the tile.  Residual: the share, then the tile
+    const int tiles = sh.nA * a.T, per = (tiles + kParts - 1) / kParts;
+    int ia = uniform(locate(use_res ? parts : sh.wp, use_res ? kParts : sh.nA, target, true, false, lane));
+    if (ia < 0) return -1;
+    const int at = use_res ? ia * per : 0, row_a = use_res ? 0 : sh.A[ia];
+    int n = use_res ? min(per, tiles - at) : a.T, t = 0;          // tile masses to search, from `at` on
+    const double wpa = use_res ? 0.0 : sh.wp[ia], lse_row = use_res ? 0.0 : a.lse[row_a];
+    const TileStat *st = a.stats + (int64_t)row_a * a.T;
 #pragma unroll 1
     for (int base = 0; ; base += kPiece) {
         const int len = min(kPiece, n - base);
-        if (use_res) {
 #pragma unroll 1
-            for (int i = lane; i < len; i += 32) {
-                const int k = at + base + i;
-                piece[i] = halves == 1 ? __ldcg(res_sums + k) : __ldcg(res_sums + 2 * k) + __ldcg(res_sums + 2 * k + 1);
-            }
-        } else {
-#pragma unroll 2
-            for (int i = lane; i < len; i += 32) {
+        for (int i0 = 0; i0 < len; i0 += 32) {
+            const int i = i0 + lane;
+            double x = 0.0;
+            if (use_res) {
+                // (one per tile, or two when the pass that wrote them worked on half tiles)
+                const double *k = res_sums + (int64_t)(at + base + min(i, len - 1)) * halves;
+                x = __ldcg(k);
+                if (halves > 1) x += __ldcg(k + 1);
+            } else if (i < len) {
                 const TileStat ts = st[base + i];
-                piece[i] = ts.sum > 0.f ? wpa * (double)ts.sum * exp((double)ts.mx * a.inv_tau - lse_row) : 0.0;
+                if (ts.sum > 0.f) x = wpa * (double)ts.sum * exp((double)ts.mx * a.inv_tau - lse_row);
             }
+            if (i < len) piece[i] = x;
         }
         __syncwarp();
         const bool more = base + len < n;
-        t = locate(piece, len, target, false, more, lane);
+        t = uniform(locate(piece, len, target, false, more, lane));
         __syncwarp();
         if (t >= 0 && !(more && t == len)) { t += at + base; break; }
         if (t < 0) {
@@ -1177,9 +1188,9 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     double *cand_key = reinterpret_cast<double *>(hist_p) + model * kMaxCand;
     int *cand_cell = reinterpret_cast<int *>(reinterpret_cast<double *>(hist_p) + 2 * kMaxCand) + model * kMaxCand;
     const int tl = threadIdx.x & (NT - 1);                    // thread and warp inside the part
-    const int lane = threadIdx.x & 31, warp = tl >> 5;
+    const int lane = threadIdx.x & 31, warp = uniform(tl >> 5);
     constexpr int kPartWarps = NT / 32;
-    const int T = a.T, nt = sh.nA * T, k = a.top_k;
+    const int T = a.T, nt = uniform(sh.nA) * T, k = a.top_k;
     const TileStat *stats = a.stats + (int64_t)model * a.N * T;
     const double *lw = model ? sh.lwq : sh.lwp;
     const double *lse = a.lse + (int64_t)model * a.N;
@@ -1210,7 +1221,9 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         unsigned lo = 0xffffffffu, hi = 0u;
         int finite = 0;
 #pragma unroll 2
-        for (int i = tl; i < nt; i += NT) {
+        for (int i0 = 0; i0 < nt; i0 += NT) {
+            const int i = i0 + tl;
+            if (i >= nt) continue;
             const float v = bound(i);
             const unsigned u = image(v);
             if (cached) bcache[i] = u;
@@ -1224,6 +1237,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     int finite = 0;
 #pragma unroll
     for (int w = 0; w < kPartWarps; ++w) { lo = min(lo, tp.lo[w]); hi = max(hi, tp.hi[w]); finite += tp.finite[w]; }
+    lo = uniform(lo); hi = uniform(hi); finite = uniform(finite);
     if (finite >= k) {
         // count(>= lo) >= k always holds; hi is above the k-th largest.  One or two too many are fine where they are close
         // (cells 30 below the largest have no mass to speak of)
@@ -1234,16 +1248,18 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
             int n = 0;
             if (cached) {
 #pragma unroll 4
-                for (int i = tl; i < nt; i += NT) n += bcache[i] >= mid;
+                for (int i0 = 0; i0 < nt; i0 += NT)
+                    if (const int i = i0 + tl; i < nt) n += bcache[i] >= mid;
             } else {
 #pragma unroll 1
-                for (int i = tl; i < nt; i += NT) n += image(bound(i)) >= mid;
+                for (int i0 = 0; i0 < nt; i0 += NT)
+                    if (const int i = i0 + tl; i < nt) n += image(bound(i)) >= mid;
             }
             n = __reduce_add_sync(kFull, n);
             if (lane == 0 && n) atomicAdd(&tp.count[round % 3], n);
             if (tl == 0) tp.count[(round + 1) % 3] = 0;           // (last read two rounds ago)
             part_sync<NT>(model);
-            n = tp.count[round % 3];
+            n = uniform(tp.count[round % 3]);
             if (n < k) { hi = mid; continue; }
             lo = mid;
             if (n == k || (n <= k + 2 && value(lo) > near)) break;
@@ -1257,7 +1273,9 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     for (int again = 0; ; ++again) {
         unsigned low = 0xffffffffu;
 #pragma unroll 1
-        for (int i = tl; i < nt; i += NT) {
+        for (int i0 = 0; i0 < nt; i0 += NT) {
+            const int i = i0 + tl;
+            if (i >= nt) continue;
             const float bv = cached ? value(bcache[i]) : bound(i);
             if (bv >= cut && bv > -INFINITY) {
                 const int pos = atomicAdd(&tp.n_sel, 1);
@@ -1269,7 +1287,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         if (lane == 0 && low != 0xffffffffu) atomicMin(&tp.low, low);
         part_sync<NT>(model);
         if (finite >= k) theta = slack(value(tp.low));
-        if (tp.n_sel <= 256) break;
+        if (uniform(tp.n_sel) <= 256) break;
         if (again) return DSBD_DEV_CAPACITY;                      // hundreds of tiles tie at the threshold
         // (or closely below the cut)
         part_sync<NT>(model);
@@ -1277,7 +1295,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         cut = theta;
         part_sync<NT>(model);
     }
-    const int n_sel = tp.n_sel;
+    const int n_sel = uniform(tp.n_sel);
     // Sweeps over the selected tiles by all warps: each counts the cells whose key reaches th and, when collect is set, lists
     // them (order is irrelevant: the final choice is by (key, cell)).  The first one nearly always fits the list.  Too many
     // cells reach the conservative threshold where there are few tiles, a large k or near ties: then a bisection, by sweeps that
@@ -1324,7 +1342,7 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
             }
         }
         part_sync<NT>(model);
-        n_cand = tp.n_cand;
+        n_cand = uniform(tp.n_cand);
         if (collect) {
             if (n_cand <= kMaxCand || itn >= 0) break;
             lo_t = theta; hi_t = -INFINITY;
@@ -1406,7 +1424,7 @@ __device__ __forceinline__ double support_lookup(const WarpScratch &ws, int mode
 // Inverse-CDF draws over the p support in canonical order; mass max(p~ - s q~, 0) (s = 0: p~).  By one warp, one
 // draw for each lane that wants one (u per lane).  Returns the index into the p support or -1.
 __device__ int draw_support(const WarpScratch &ws, double u, double s, int lane) {
-    const int n = ws.n[0];
+    const int n = uniform(ws.n[0]);
     double w0 = 0.0, w1 = 0.0;                                // places 2 lane and 2 lane + 1
     if (2 * lane < n) { const int i = ws.order[2 * lane]; w0 = fmax(ws.prob[0][i] - s * ws.qat[i], 0.0); }
     if (2 * lane + 1 < n) { const int i = ws.order[2 * lane + 1]; w1 = fmax(ws.prob[0][i] - s * ws.qat[i], 0.0); }
@@ -1427,17 +1445,18 @@ __device__ int draw_support(const WarpScratch &ws, double u, double s, int lane)
 
 // After build_support(p) [and q]: q~ at the p cells and the canonical order of the p support.
 __device__ void finish_supports(WarpScratch &ws, bool have_q, int lane) {
-#pragma unroll 1
-    for (int i = lane; i < ws.n[0]; i += 32) ws.qat[i] = have_q ? support_lookup(ws, 1, ws.cell[0][i]) : 0.0;
     // canonical order: the place of a cell is the number of support cells below it (cells are unique)
-    const int n = ws.n[0];
+    const int n = uniform(ws.n[0]);
 #pragma unroll 1
-    for (int i = lane; i < n; i += 32) {
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        if (i >= n) continue;
         const int c = ws.cell[0][i];
         int place = 0;
 #pragma unroll 2
         for (int j = 0; j < n; ++j) place += ws.cell[0][j] < c;
         ws.order[place] = i;
+        ws.qat[i] = have_q ? support_lookup(ws, 1, c) : 0.0;
     }
     __syncwarp();
 }
@@ -1461,11 +1480,11 @@ template <bool kWarped>
 __global__ void __launch_bounds__(kVThreads, 2)
 k_verify(const __grid_constant__ VerifyArgs a) {
     cg::cluster_group cluster = cg::this_cluster();
-    const int n_cta = (int)cluster.num_blocks();
-    const int cta_rank = (int)cluster.block_rank();
+    const int n_cta = uniform((int)cluster.num_blocks());
+    const int cta_rank = uniform((int)cluster.block_rank());
     const int r = blockIdx.x / n_cta;
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const bool writer = (cta_rank == 0);
     __shared__ Shared sh;
     __shared__ double sp_live[kMaxLive], sq_live[kMaxLive];
@@ -1479,13 +1498,14 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     // pass ahead in the stream.  That pass lets this kernel start only when each of its blocks has waited for all earlier work,
     // so what earlier kernels and the caller left lies in L2 and may be read here, from there (ld_early: the pass's wait says
     // nothing about this SM's L1); the tile statistics only after the wait.
-    const int b_lo = ld_early(a.req_beam_off + r), b_hi = ld_early(a.req_beam_off + r + 1);
-    const int n_lo = ld_early(a.beam_node_off + b_lo), n_hi = ld_early(a.beam_node_off + b_hi);
+    const int b_lo = uniform(ld_early(a.req_beam_off + r)), b_hi = uniform(ld_early(a.req_beam_off + r + 1));
+    const int n_lo = uniform(ld_early(a.beam_node_off + b_lo)), n_hi = uniform(ld_early(a.beam_node_off + b_hi));
     int W_min = a.W_min_r ? ld_early(a.W_min_r + r) : a.W_min;
     int W_max = a.W_max_r ? ld_early(a.W_max_r + r) : a.W_max;
     int W_nom = a.W_nom_r ? ld_early(a.W_nom_r + r) : a.W_nom;
     // per-request widths come from device memory: a width below 1 or a cap below the minimum is
     // reported (after the set-up below) and the request is not verified
+    W_min = uniform(W_min); W_max = uniform(W_max); W_nom = uniform(W_nom);
     const bool bad_widths = a.check_widths && (W_min < 1 || W_max < W_min || W_nom < 1);
     if (bad_widths) { W_min = W_max = W_nom = 1; }
     double *sums_base = a.tile_sums + (int64_t)r * 2 * (a.max_m + 1) * ((int64_t)a.max_live * a.T);
@@ -1732,8 +1752,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         }
         __syncwarp();
         if (!a.select_mode) {
+            const int nA = uniform(sh.nA);
 #pragma unroll 1
-            for (int i = lane; i < sh.nA; i += 32) {
+            for (int i0 = 0; i0 < nA; i0 += 32) {
+                const int i = i0 + lane;
+                if (i >= nA) continue;
                 const int root = a.beam_node_off[b_lo + i];
                 sh.A[i] = root;
                 sp_live[i] = cached ? nc.score_p[root - n_lo] : a.score[root];
@@ -1741,23 +1764,24 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             }
             if (writer) {
 #pragma unroll 1
-                for (int l = lane; l <= a.gamma; l += 32) a.out.layer_width[(int64_t)r * (a.gamma + 1) + l] = -1;
+                for (int l0 = 0; l0 <= a.gamma; l0 += 32)
+                    if (const int l = l0 + lane; l <= a.gamma) a.out.layer_width[(int64_t)r * (a.gamma + 1) + l] = -1;
                 if (lane == 0) { a.out.l_last[r] = a.gamma + 1; a.out.out_width[r] = 0; }
             }
         }
         __syncwarp();
         if (!a.select_mode && writer)
 #pragma unroll 1
-            for (int n = n_lo + lane; n < n_hi; n += 32)
-                a.out.node_status[n] = is_root(n - n_lo) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+            for (int n0 = n_lo; n0 < n_hi; n0 += 32)
+                if (const int n = n0 + lane; n < n_hi) a.out.node_status[n] = is_root(n - n_lo) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     }
     // Every CTA of the cluster takes identical decisions from identical data, so each keeps its
     // own copy of the node statuses and only rank 0 writes results.
     const bool st_ok = n_req_nodes <= kMaxLive * kMaxLive;
     if (!a.select_mode)
 #pragma unroll 1
-        for (int n = threadIdx.x; n < n_req_nodes && st_ok; n += blockDim.x)
-            st[n] = is_root(n) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+        for (int n0 = 0; n0 < n_req_nodes && st_ok; n0 += kVThreads)
+            if (const int n = n0 + threadIdx.x; n < n_req_nodes) st[n] = is_root(n) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     __syncthreads();
     if (!a.select_mode && !st_ok && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
     if (bad_widths && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_PARAM;
@@ -1769,7 +1793,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         return cached ? (model ? nc.score_q[i] : nc.score_p[i]) : a.score[(int64_t)model * a.N + n_lo + i];
     };
 
-    const bool failed = sh.err != 0;
+    const bool failed = uniform(sh.err);
     // Layers 1 .. gamma; then, in the CTA that writes, the extra layer: no drafts, W_nom beams from p_beam^(gamma+1).
     const int n_layers = a.select_mode ? 1 : a.gamma + (writer ? 1 : 0);
 #pragma unroll 1
@@ -1780,7 +1804,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         if (warp == 0) {
             int m = 0;
             if (a.select_mode) {
-                m = a.m_in[r];
+                m = uniform(a.m_in[r]);
                 if (m < 0 || m > kMaxLive) m = -1;
             } else if (!extra) {
 #pragma unroll 1
@@ -1805,10 +1829,13 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 if (a.draft_rank) {
                     // order of (draft_rank, node id), ids being ascending: a draft's place is the number before it
 #pragma unroll 1
-                    for (int i = lane; i < m; i += 32) sh.S_parent_idx[i] = a.draft_rank[sh.S[i]];
+                    for (int i0 = 0; i0 < m; i0 += 32)
+                        if (const int i = i0 + lane; i < m) sh.S_parent_idx[i] = a.draft_rank[sh.S[i]];
                     __syncwarp();
 #pragma unroll 1
-                    for (int i = lane; i < m; i += 32) {
+                    for (int i0 = 0; i0 < m; i0 += 32) {
+                        const int i = i0 + lane;
+                        if (i >= m) continue;
                         const int key = sh.S_parent_idx[i];
                         int place = 0;
 #pragma unroll 2
@@ -1817,16 +1844,20 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     }
                     __syncwarp();
 #pragma unroll 1
-                    for (int i = lane; i < m; i += 32) sh.S[i] = sh.acc[i];
+                    for (int i0 = 0; i0 < m; i0 += 32)
+                        if (const int i = i0 + lane; i < m) sh.S[i] = sh.acc[i];
                     __syncwarp();
                 }
                 // index of a draft's parent in A, and its log-prob under either model given that parent
+                const int nA = uniform(sh.nA);
 #pragma unroll 1
-                for (int i = lane; i < m; i += 32) {
+                for (int i0 = 0; i0 < m; i0 += 32) {
+                    const int i = i0 + lane;
+                    if (i >= m) continue;
                     const int n = sh.S[i] - n_lo, pl = nd_parent(n);
-                    int ai = 0;
+                    int ai = nA;
 #pragma unroll 1
-                    while (ai < sh.nA && sh.A[ai] != n_lo + pl) ++ai;
+                    for (int k = 0; k < nA; ++k) ai = sh.A[k] == n_lo + pl ? k : ai;      // (nodes are unique)
                     sh.S_parent_idx[i] = ai;
                     sh.rho[i] = nd_score(0, n) - nd_score(0, pl);
                     sh.uu[i] = nd_score(1, n) - nd_score(1, pl);
@@ -1848,10 +1879,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         } else if (!kWarped) {
             uint4 *words = reinterpret_cast<uint4 *>(hp);
 #pragma unroll 4
-            for (int i = threadIdx.x - 96; i < kHistArrays * kHistWords / 4; i += kVThreads - 96) words[i] = make_uint4(0, 0, 0, 0);
+            for (int i0 = 0; i0 < kHistArrays * kHistWords / 4; i0 += kVThreads - 96)
+                if (const int i = i0 + threadIdx.x - 96; i < kHistArrays * kHistWords / 4) words[i] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
-        const int m = sh.m;
+        const int m = uniform(sh.m);
         if (m < 0) {
             if (threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
             break;
@@ -1870,7 +1902,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 const int e_half = extra && half ? 0 : build_support<kHalf>(a, sh, half, hp, hq);
                 if (e_half && (threadIdx.x & (kHalf - 1)) == 0) wsup.tmp[half].err = e_half;
                 __syncthreads();
-                const int e = wsup.tmp[0].err ? wsup.tmp[0].err : extra ? 0 : wsup.tmp[1].err;
+                const int e = uniform(wsup.tmp[0].err ? wsup.tmp[0].err : extra ? 0 : wsup.tmp[1].err);
                 if (e) { if (threadIdx.x == 0) sh.err = e; }
                 else if (warp == 0) {
                     finish_supports(wsup, !extra, lane);
@@ -1878,7 +1910,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     if (!a.select_mode) {
                         draft_tests(sh, a.seed, a.step, r, l, m, lane);
 #pragma unroll 1
-                        for (int i = lane; i < m; i += 32) {
+                        for (int i0 = 0; i0 < m; i0 += 32) {
+                            const int i = i0 + lane;
+                            if (i >= m) continue;
                             const int cell = sh.S_parent_idx[i] * a.V + a.token[sh.S[i]];
                             const double pw = support_lookup(wsup, 0, cell), qw = support_lookup(wsup, 1, cell);
                             sh.rho[i] = qw > 0.0 ? pw / qw : (pw > 0.0 ? INFINITY : 0.0);
@@ -1900,7 +1934,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                         if (lane == 0) { sh.s_arr[j] = s_j; sh.c_arr[j + 1] = acc; sh.chain_len = j; }
                         s_prev = s_j;
                         c_cur = acc;
-                        if (!(acc > 0.0)) break;
+                        if (!uniform(acc > 0.0)) break;
                     }
                     __syncwarp();
                 }
@@ -1927,7 +1961,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     if (lane == 0) sh.on_demand = first >= W_known || m - 1 - first <= on_demand_left(sh.nA * a.T, n_cta * kVWarps);
                 }
                 __syncthreads();
-                on_demand = sh.on_demand;
+                on_demand = uniform(sh.on_demand);
             }
             const float binscale = sh.binscale[m];
             if (!on_demand) {
@@ -1946,7 +1980,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             }
             // The chain c_{j+1} = F(s_j) from sh.chain_pos on (warp 0).  sh.need_exact = 1 where the histogram leaves one open.
             auto walk_chain = [&]() {
-                int j = sh.chain_pos, need = 0;
+                int j = uniform(sh.chain_pos), need = 0;
                 // lane 2 c + e looks up bin k + e in CTA c
                 const int c = min(lane >> 1, n_cta - 1);
                 const bool has = lane < 2 * n_cta;
@@ -1966,7 +2000,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     // float 0.6e-7, the product with binscale 5e-7; an edge by 6e-7.  The bracket below takes the edges
                     // 2e-6 wider.  Approximate logarithm and exponential, reciprocals for the division: 1 us less, 1.6e-6)
                     int k = (int)(log2f((float)s_j) * binscale);
-                    if (k < 0 || j == 1) k = 0;                      // s_1 = 1, the first edge
+                    k = uniform(k < 0 || j == 1 ? 0 : k);            // (s_1 = 1, the first edge)
                     if (k >= kBins) { need = 1; break; }             // cannot happen for s_j <= m
                     double P = 0.0, Q = 0.0;                         // (whole numbers below 2^46: the sums are exact)
                     if (has) {
@@ -1994,10 +2028,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                         c_next = fmax(P1 * kUnfix - s_j * (Q1 * kUnfix), 0.0) + 0.5 * (lo_b + hi_b);
                     }
                     // the midpoint of the bracket is used: half its width plus the fixed-point term
-                    if (0.5 * (hi_b - lo_b) + fix_err > kErrTol) { need = 1; break; }
+                    need = uniform(0.5 * (hi_b - lo_b) + fix_err > kErrTol);
+                    if (need) break;
                     if (lane == 0) sh.c_arr[j + 1] = c_next;
                     c_j = c_next;
-                    if (!(c_next > 0.0)) { j = m; }               // chain exhausted: stop walking
+                    if (!uniform(c_next > 0.0)) j = m;               // chain exhausted: stop walking
                 }
                 if (lane == 0) {
                     sh.need_exact = need;
@@ -2012,8 +2047,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     else walk_chain();
                 }
                 __syncthreads();
-                if (!sh.need_exact) break;
-                const int j = sh.chain_pos;
+                if (!uniform(sh.need_exact)) break;
+                const int j = uniform(sh.chain_pos);
                 const bool first = on_demand && j == 1;
                 // (in a layer with a histogram that pass left the sums at j = 1 in slot 0; half tiles have room there only)
                 const int halves = first ? item_halves(sh.nA * a.T, n_cta * kVWarps) : 1;
@@ -2036,12 +2071,13 @@ k_verify(const __grid_constant__ VerifyArgs a) {
 
         TS(8);
         // ---- width and accept loop (warp 0) ----
-        if (warp == 0 && !sh.err) {
+        if (warp == 0 && !uniform(sh.err)) {
             int W = W_known;
             if (!on_demand && !extra) {
                 // alpha_j = 1 - c_{j+1}/c_j; once a residual has no mass every later alpha is 1
 #pragma unroll 1
-                for (int j = 1 + lane; j <= m; j += 32) {
+                for (int j0 = 1; j0 <= m; j0 += 32) {
+                    const int j = min(j0 + lane, m);         // (the last one more than once)
                     double al = 1.0;
                     if (j <= sh.chain_len && sh.c_arr[j] > 0.0 && sh.c_arr[j + 1] > 0.0)
                         al = fmin(fmax(1.0 - sh.c_arr[j + 1] / sh.c_arr[j], 0.0), 1.0);
@@ -2069,7 +2105,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             } else {
                 if (!on_demand) accept_drafts(sh, st, writer ? a.out.node_status : nullptr, n_lo, m, W, false, lane);
 #pragma unroll 1
-                for (int i = sh.next_i + lane; i < m; i += 32) {
+                for (int i0 = uniform(sh.next_i); i0 < m; i0 += 32) {
+                    const int i = i0 + lane;
+                    if (i >= m) continue;
                     st[sh.S[i] - n_lo] = DSBD_NODE_CUT;
                     if (writer) a.out.node_status[sh.S[i]] = DSBD_NODE_CUT;
                 }
@@ -2089,16 +2127,18 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         TS(9);
         // ---- a residual draw locates its tile through tile sums of max(p_beam - s_{j-1} q_beam, 0) ----
         // slot 0 of the bank; in a layer of known width that of the rejection before the draw
-        const int res_slot = on_demand && sh.run_j > 2 ? sh.run_j - 1 : 0;
+        const int err = uniform(sh.err), j = uniform(sh.run_j), res_j = uniform(sh.res_j);
+        const int res_slot = on_demand && j > 2 ? j - 1 : 0;
         double *res_sums = sums_base + ((int64_t)sh.bank * (a.max_m + 1) + res_slot) * slot_stride;
-        if (!a.select_mode && !sh.err && !warped && sh.res_j > 2) {   // run position 2 is served by the histogram pass
+        if (!a.select_mode && !err && !warped && res_j > 2) {   // run position 2 is served by the histogram pass
             if (threadIdx.x == 0) { ++sh.n_respass; sh.halves = 1; }
-            exact_pass(a, sh, sh.s_arr[sh.res_j - 1], res_sums, false, 0.f, 1, false, n_pass++);
+            exact_pass(a, sh, sh.s_arr[res_j - 1], res_sums, false, 0.f, 1, false, n_pass++);
         }
 
         TS(10);
-        if (a.select_mode || sh.err) break;
-        if (sh.count >= sh.W) {
+        if (a.select_mode || err) break;
+        const int count = uniform(sh.count), want = uniform(sh.W) - count;
+        if (want <= 0) {
             // ---- the accepted drafts, ascending node id, are the next layer's input beams (warp 0) ----
             if (warp == 0) {
                 int nA = 0;
@@ -2123,11 +2163,10 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         // ---- a short layer ends the request: accepted drafts, then the residual draw, then fills from p_beam (in the extra layer
         // draws from p_beam alone), all independent of one another: a warp for each ----
         if (!writer) break;
-        const int count = sh.count, want = sh.W - count, j = sh.run_j;
-        const int cap = a.out.out_off[r + 1] - a.out.out_off[r];
+        const int cap = uniform(a.out.out_off[r + 1] - a.out.out_off[r]);
         const int n_acc = min(count, max(cap, 0)), n_draw = n_acc < count ? 0 : min(want, max(cap - n_acc, 0));
         const bool use_res = j > 1;
-        const int halves = res_slot ? 1 : sh.halves;
+        const int halves = res_slot ? 1 : uniform(sh.halves);
         float *words = reinterpret_cast<float *>(hp) + warp * kTokWords;
         double *parts = reinterpret_cast<double *>(reinterpret_cast<float *>(hp) + kVWarps * kTokWords);
         if (!warped && use_res) {
@@ -2146,7 +2185,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 const int f = b - n_acc;
                 const double u = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, extra ? 3u : f ? 2u : 1u,
                                                   extra || !f ? (uint32_t)f : (uint32_t)(f - 1));
-                const bool res = f == 0 && use_res;
+                const bool res = uniform(f == 0 && use_res);
                 source = extra ? DSBD_SRC_EXTRA : f ? DSBD_SRC_FILL : DSBD_SRC_RESIDUAL;
                 int ia = 0;
                 if (warped) {
@@ -2429,7 +2468,7 @@ k_draft(const __grid_constant__ DraftArgs d) {
     __shared__ int s_err;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     uint32_t *hp = reinterpret_cast<uint32_t *>(dyn_smem), *hq = hp + kHistWords;
-    const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r = blockIdx.x, lane = threadIdx.x & 31, warp = warp_index();
     // (before the wait as in k_verify: what earlier work left, from L2)
     const int b_lo = ld_early(a.req_beam_off + r), o_lo = ld_early(d.out_off + r), cap = ld_early(d.out_off + r + 1) - o_lo;
     const int W = d.W_r ? ld_early(d.W_r + r) : d.W;

@@ -503,7 +503,7 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
         double none = 1.0;
         sh.col_a[0] = 1.0;
         sh.tail[0] = 1.0;
-#pragma unroll 2
+#pragma unroll 4
         for (int i = 1; i <= m; ++i) {
             sh.first[i] = sh.alpha[i] * none;
             none *= (1.0 - sh.alpha[i]);
@@ -530,7 +530,7 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
         for (int n0 = 0; n0 <= m; n0 += 32) {
             const int n = n0 + lane;
             double acc = 0.0;
-#pragma unroll 2
+#pragma unroll 4
             for (int i = 1; i <= m; ++i)
                 if (i <= n && n <= m) acc += sh.first[i] * prev[n - i];
             if (n <= m) cur[n] = n > k ? acc : 0.0;         // P(n, k+1), zero for n < k+1
@@ -964,12 +964,11 @@ __device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
     __syncthreads();
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
-        unsigned long long over = 0ull;
+        // lanes 0 to 15: the warps behind this one; 16 to 23: the copies of the last bin
+        unsigned long long t = lane < kVWarps ? (lane > warp ? sh.wtot[x][lane] : 0ull) : lane < kVWarps + kOverSlots / 32 ? sh.over[x][lane - kVWarps] : 0ull;
 #pragma unroll
-        for (int w = 0; w < kOverSlots / 32; ++w) over += sh.over[x][w];
-        above[x] += over;
-#pragma unroll 1
-        for (int w = warp + 1; w < kVWarps; ++w) above[x] += sh.wtot[x][w];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+        above[x] += t;
         uint32_t *low = x ? h.wq : h.wp, *high = x ? h.bq : h.bp;
 #pragma unroll
         for (int k = 0; k < 8; k += 4) {
@@ -977,7 +976,7 @@ __device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
             *reinterpret_cast<uint4 *>(low + i0 + k) = make_uint4((uint32_t)a0, (uint32_t)a1, (uint32_t)a2, (uint32_t)a3);
             *reinterpret_cast<uint4 *>(high + i0 + k) = make_uint4((uint32_t)(a0 >> 32), (uint32_t)(a1 >> 32), (uint32_t)(a2 >> 32), (uint32_t)(a3 >> 32));
         }
-        if (threadIdx.x == 0) { low[kBins] = (uint32_t)over; high[kBins] = (uint32_t)(over >> 32); }
+        if (threadIdx.x == kVThreads - 1) { low[kBins] = (uint32_t)above[x]; high[kBins] = (uint32_t)(above[x] >> 32); }
     }
     // what the threads added, by their floating-point sums, minus what the words hold.  Without a wrap that is rounding: half a
     // unit for each cell and 2^-20 of the mass (16 cells in a float sum), less than 2^26 units; a wrap lowers the words by 2^32
@@ -1025,12 +1024,10 @@ __device__ __noinline__ void accept_drafts(Shared &sh, int8_t *st, int8_t *node_
         const int lanes = asks ? min(n, stop + 1) : n;
         bool accept = false, close = false;
         if (lane < lanes) {
-            double ratio = sh.rho[i + lane];
-            if (jt > 1) ratio = fmax(ratio - sh.s_arr[jt - 1], 0.0) / sh.c_arr[jt];
-            if (ratio > 1.0) ratio = 1.0;
-            const double u = sh.uu[i + lane];
-            accept = u <= ratio;
-            close = fabs(u - ratio) < 1e-5;
+            // u <= min(max(rho - s, 0) / c, 1), times c
+            const double c = sh.c_arr[jt], u = sh.uu[i + lane] * c, top = fmin(fmax(sh.rho[i + lane] - sh.s_arr[jt - 1], 0.0), c);
+            accept = u <= top;
+            close = fabs(u - top) < 1e-5 * c;
         }
         const unsigned accepts = __ballot_sync(kFull, accept);
         const int done = accepts ? __ffs(accepts) : lanes;        // drafts tested in this round
@@ -2002,12 +1999,17 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     int k = (int)(log2f((float)s_j) * binscale);
                     k = uniform(k < 0 || j == 1 ? 0 : k);            // (s_1 = 1, the first edge)
                     if (k >= kBins) { need = 1; break; }             // cannot happen for s_j <= m
-                    double P = 0.0, Q = 0.0;                         // (whole numbers below 2^46: the sums are exact)
+                    uint32_t w[4] = {0u, 0u, 0u, 0u};
                     if (has) {
-                        const uint32_t *at = words + k;
-                        P = (double)(((unsigned long long)at[2 * kHistWords] << 32) | at[0]);
-                        Q = (double)(((unsigned long long)at[3 * kHistWords] << 32) | at[kHistWords]);
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) w[x] = words[x * kHistWords + k];
                     }
+                    // (the edges while the words are on their way)
+                    const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
+                    const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
+                    const double inv = 1.0 / (r_hi - r_lo);
+                    double P = (double)(((unsigned long long)w[2] << 32) | w[0]);        // (whole numbers below 2^46: their sums
+                    double Q = (double)(((unsigned long long)w[3] << 32) | w[1]);        // are exact)
 #pragma unroll
                     for (int o = 2; o < 32; o <<= 1) {
                         P += __shfl_xor_sync(kFull, P, o);
@@ -2015,15 +2017,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     }
                     const double P0 = __shfl_sync(kFull, P, 0), Q0 = __shfl_sync(kFull, Q, 0);
                     const double P1 = __shfl_sync(kFull, P, 1), Q1 = __shfl_sync(kFull, Q, 1);
-                    double lo_b = 0.0, hi_b = 0.0, c_next;
-                    if (j == 1) c_next = (P0 - Q0) * kUnfix;
-                    else {
+                    double lo_b = 0.0, hi_b = 0.0, c_next = (P0 - Q0) * kUnfix;
+                    if (j > 1) {
                         const double Pk = (P0 - P1) * kUnfix, Qk = (Q0 - Q1) * kUnfix;
-                        const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
-                        const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
                         lo_b = fmax(Pk - s_j * Qk, 0.0);
-                        double q_hi = (Pk - r_lo * Qk) / (r_hi - r_lo);
-                        q_hi = fmin(fmax(q_hi, 0.0), Qk);
+                        const double q_hi = fmin(fmax((Pk - r_lo * Qk) * inv, 0.0), Qk);
                         hi_b = fmax(q_hi * (r_hi - s_j), lo_b);
                         c_next = fmax(P1 * kUnfix - s_j * (Q1 * kUnfix), 0.0) + 0.5 * (lo_b + hi_b);
                     }
@@ -2284,12 +2282,14 @@ int check_params(const dsbd_verify_params_t *p) {
 }
 
 // Cluster size: as many CTAs per request as its tile count can use, but few enough that all
-// requests are resident at once (two CTAs per SM fit).
+// requests are resident at once (two CTAs per SM fit).  16 from six tiles a CTA on (half a tile a warp instead of one): requests of four
+// live rows, 128 tiles 41.9 us instead of 44.3 with 8 CTAs (one request), 252 tiles 43.5 for 47.9; eight requests 56.7 for 59.6 and
+// 66.4 for 74.2.  64 tiles: 41.3 for 40.5, so 8 stay.
 int cluster_size_for(int tiles, int R) {
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int cs = 1;
-    if (tiles >= 256) cs = 16;
+    if (tiles >= 96) cs = 16;
     else if (tiles >= 64) cs = 8;
     else if (tiles >= 32) cs = 4;
     else if (tiles >= 16) cs = 2;

@@ -255,6 +255,11 @@ constexpr int kBins = 4096;
 constexpr int kOverSlots = 256;                   // copies of the last bin (rho beyond the last edge): one per
                                                   // warp and half-warp lane, so that none collects enough to wrap
 
+// The bins of a layer of m drafts: scale bins to a power of two; the upper edge of a bin over 2^(k / scale), and one over the width
+// of a bin over the same, both with the edges' tolerance (2e-6).
+struct BinEdges { float scale, inv_scale; double hi, inv_width; };
+constexpr double kEdgeTol = 2e-6;
+
 struct Shared {
     int nA, m, W, count, chain_len, err;         // m: -1 if too many
     int A[kMaxLive];
@@ -276,7 +281,6 @@ struct Shared {
     double tail[kMaxLive + 2];
     int bank, halves, need_exact, res_j, run_j, chain_pos;
     int n_draw;                             // completion draws of the request
-    float binscale[kMaxLive + 1];           // by m: bins of a layer's histogram to a power of two
     int on_demand, next_i;                  // a layer of known width: its passes are made when the accept loop asks
     // sums of an exact pass, in units of 2^-60, 2^-120 (what the first leaves) and 2^-44 (q): of this CTA's warps; of every
     // CTA, two passes in turn
@@ -286,12 +290,13 @@ struct Shared {
     int n_near, n_rows;                     // accept tests inside the 1e-5 tie band; live rows of layers that looked into them
     unsigned long long wtot[2][kVWarps], over[2][kOverSlots / 32];   // mass (p, q) of every warp's bins and copies of the last bin
     unsigned long long added;               // mass that this CTA's histogram pass added (p and q), by floating-point sums
-    int wrapped;                            // a w word of this CTA's histogram wrapped
     int n_wrapped;                          // layers where one did
 #ifdef DSBD_PHASE_TIMING
     unsigned long long *ts, *ts_end;        // next and last time stamp of the CTA that writes
 #endif
-    double rho[kMaxLive], uu[kMaxLive];     // per live draft: p_beam/q_beam and its uniform (before: its log-probs under p, q)
+    double rho[kMaxLive], lq[kMaxLive];     // per live draft: p_beam/q_beam (before: its log-prob under p); log-prob under q
+    double uu[kMaxLive];                    // and its uniform
+    BinEdges bins[kMaxLive + 1];            // by m
 };
 
 #ifdef DSBD_PHASE_TIMING
@@ -499,17 +504,18 @@ __device__ void live_weights(const VerifyArgs &a, Shared &sh, int model, const d
 // returns W~ = max{K : tail[K] >= thresh}.
 // k_stop >= 0: stop once W = min(W_max = k_stop, max(W_min, W~)) is decided; -1: the whole tail
 __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop) {
-    if (lane == 0) {
-        double none = 1.0;
-        sh.col_a[0] = 1.0;
-        sh.tail[0] = 1.0;
-#pragma unroll 4
-        for (int i = 1; i <= m; ++i) {
-            sh.first[i] = sh.alpha[i] * none;
-            none *= (1.0 - sh.alpha[i]);
-            sh.col_a[i] = none;                    // P(n, 0) = prod_{j<=n}(1 - alpha_j)
-        }
+    // With 1 - alpha_j = c_{j+1} / c_j and c_1 = 1: P(n, 0) = prod_{j<=n}(1 - alpha_j) = c_{n+1}, and the first accept is the i-th
+    // draft's with alpha_i prod_{j<i}(1 - alpha_j) = c_i - c_{i+1}.  No residual mass from some c on: every later alpha is 1
+    const int len = uniform(sh.chain_len);
+#pragma unroll 1
+    for (int i0 = 0; i0 <= m; i0 += 32) {
+        const int i = min(i0 + lane, m);                     // (the last one more than once)
+        auto mass = [&](int j) { return j <= len + 1 && sh.c_arr[j] > 0.0 ? sh.c_arr[j] : 0.0; };
+        const double c = mass(i + 1);
+        sh.col_a[i] = c;
+        if (i > 0) sh.first[i] = fmax(mass(i) - c, 0.0);
     }
+    if (lane == 0) sh.tail[0] = 1.0;
     __syncwarp();
     double *prev = sh.col_a, *cur = sh.col_b;
     double below = 0.0;
@@ -541,7 +547,10 @@ __device__ int width_rule(Shared &sh, int m, double thresh, int lane, int k_stop
     __syncwarp();
     int wt = 0;
 #pragma unroll 1
-    for (int K = 0; K <= m; ++K) if (sh.tail[K] >= thresh) wt = K;
+    for (int K0 = 0; K0 <= m; K0 += 32) {
+        const unsigned reach = __ballot_sync(kFull, K0 + lane <= m && sh.tail[min(K0 + lane, m)] >= thresh);
+        if (reach) wt = K0 + 31 - __clz(reach);
+    }
     if (lane == 0) sh.tail[m + 1] = 0.0;
     return wt;
 }
@@ -578,6 +587,7 @@ constexpr float kFix = 17592186044416.f;          // 2^44
 constexpr double kUnfix = 1.0 / 17592186044416.0;
 constexpr double kErrTol = 2.5e-7;                // error bound of F(s) above which it is recomputed exactly
 constexpr int kHistArrays = 4;
+constexpr uint32_t kWrapped = 0x80000000u;
 struct HistSmem { uint32_t *wp, *wq, *bp, *bq; };
 
 __device__ __forceinline__ HistSmem hist_arrays(uint32_t *base) {
@@ -588,6 +598,18 @@ __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// Shared memory of CTA c of the cluster: the address of what p is here, and 16 bytes from there.
+__device__ __forceinline__ uint32_t cluster_address(const void *p, int c) {
+    uint32_t to;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(c));
+    return to;
+}
+__device__ __forceinline__ uint4 ld_cluster(uint32_t at) {
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+    return v;
 }
 
 // Two fp32 values in one 64-bit register: an instruction does both (rounding as the plain ones).
@@ -918,12 +940,14 @@ __device__ __forceinline__ void histogram_pass(const VerifyArgs &a, Shared &sh, 
     if (lane == 0 && added) atomicAdd(&sh.added, added);
 }
 
-// This CTA's histogram into suffix sums (p and q mass of its bins >= k, units of 2^-44), in place of the words: w words the
-// low, b words the high halves.  Entry kBins is the last bin, whose copies are folded here.  A thread takes eight bins, all their words in
-// flight together.  Each CTA keeps the sums of its own cells; the chain adds the few that it looks up over the
+// This CTA's histogram into suffix sums (p and q mass of its bins >= k, units of 2^-44), over the words: entry k is 16 bytes, p
+// low and high half, then q, so that a look-up is one load.  Entry kBins is the last bin, whose copies are folded here.  Entries of
+// eight bins are rotated against one another: a thread takes eight bins, and eight threads that store an entry each touch all banks.  Each CTA keeps the sums of its own cells; the chain adds the few that it looks up over the
 // CTAs (a merge of the 4096 bins over the cluster before it took 4.5 us a layer and another cluster barrier, for at most 2 m bins that
 // anybody looks at).
 static_assert(kBins == 8 * kVThreads, "eight bins to a thread");
+__device__ __forceinline__ int suffix_entry(int k) { return k ^ ((k >> 3) & 7); }
+static_assert((kBins + 8) * 16 <= kHistArrays * kHistWords * 4, "an entry for every bin and the last one");
 __device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
     const int lane = threadIdx.x & 31, warp = warp_index(), i0 = threadIdx.x * 8;
     unsigned long long v[2][8];                              // p, q
@@ -969,36 +993,38 @@ __device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
         above[x] += t;
-        uint32_t *low = x ? h.wq : h.wp, *high = x ? h.bq : h.bp;
-#pragma unroll
-        for (int k = 0; k < 8; k += 4) {
-            const unsigned long long a0 = v[x][k] + above[x], a1 = v[x][k + 1] + above[x], a2 = v[x][k + 2] + above[x], a3 = v[x][k + 3] + above[x];
-            *reinterpret_cast<uint4 *>(low + i0 + k) = make_uint4((uint32_t)a0, (uint32_t)a1, (uint32_t)a2, (uint32_t)a3);
-            *reinterpret_cast<uint4 *>(high + i0 + k) = make_uint4((uint32_t)(a0 >> 32), (uint32_t)(a1 >> 32), (uint32_t)(a2 >> 32), (uint32_t)(a3 >> 32));
-        }
-        if (threadIdx.x == kVThreads - 1) { low[kBins] = (uint32_t)above[x]; high[kBins] = (uint32_t)(above[x] >> 32); }
     }
     // what the threads added, by their floating-point sums, minus what the words hold.  Without a wrap that is rounding: half a
-    // unit for each cell and 2^-20 of the mass (16 cells in a float sum), less than 2^26 units; a wrap lowers the words by 2^32
-    if (threadIdx.x == 0) sh.wrapped = (long long)(sh.added - (v[0][0] + above[0]) - (v[1][0] + above[1])) > (1ll << 31);
+    // unit for each cell and 2^-20 of the mass (16 cells in a float sum), less than 2^26 units; a wrap lowers the words by 2^32.
+    // The top bit of the first entry tells (a sum takes 46 bits)
+    uint32_t wrapped = 0u;
+    if (threadIdx.x == 0 && (long long)(sh.added - (v[0][0] + above[0]) - (v[1][0] + above[1])) > (1ll << 31)) wrapped = kWrapped;
+    uint4 *entries = reinterpret_cast<uint4 *>(h.wp);
+    auto entry = [](unsigned long long p, unsigned long long q) { return make_uint4((uint32_t)p, (uint32_t)(p >> 32), (uint32_t)q, (uint32_t)(q >> 32)); };
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        uint4 e = entry(v[0][k] + above[0], v[1][k] + above[1]);
+        if (k == 0) e.y |= wrapped;
+        entries[suffix_entry(i0 + k)] = e;
+    }
+    if (threadIdx.x == kVThreads - 1) entries[suffix_entry(kBins)] = entry(above[0], above[1]);
 }
 
-// Per live draft of layer l: rho = p_beam/q_beam of its cell and its uniform, by one warp.
-__device__ __noinline__ void draft_tests(Shared &sh, uint64_t seed, uint64_t step, int r, int l, int m, int lane) {
+// Per live draft: rho = p_beam/q_beam of its cell, by one warp.
+__device__ __noinline__ void draft_tests(Shared &sh, int m, int lane) {
     m = uniform(m);
 #pragma unroll 1
     for (int i0 = 0; i0 < m; i0 += 32) {
         const int i = i0 + lane;
         if (i >= m) continue;
         const int ai = sh.S_parent_idx[i];
-        const double lp = sh.rho[i], lq = sh.uu[i];
+        const double lp = sh.rho[i], lq = sh.lq[i];
         double rho;
         if (lq == -INFINITY || sh.lwq[ai] == -INFINITY)
             rho = (lp > -INFINITY && sh.lwp[ai] > -INFINITY) ? INFINITY : 0.0;
         else
             rho = exp((sh.lwp[ai] - sh.lwq[ai]) + (lp - lq));
         sh.rho[i] = rho;
-        sh.uu[i] = decision_uniform(seed, step, (uint32_t)r, (uint32_t)l, 0u, (uint32_t)i);
     }
     __syncwarp();
 }
@@ -1515,7 +1541,15 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     TS(1);
     // (a CTA may store into another's shared memory once that CTA runs: arrived here, waited for below)
     cluster.barrier_arrive();
-    if (!kWarped && threadIdx.x <= kMaxLive) sh.binscale[threadIdx.x] = (float)((double)kBins / log2((double)max((int)threadIdx.x, 2)));    // s_j <= j <= m
+    if (!kWarped && threadIdx.x <= kMaxLive) {
+        const double range = log2((double)max((int)threadIdx.x, 2));        // s_j <= j <= m
+        BinEdges e;
+        e.scale = (float)((double)kBins / range);
+        e.inv_scale = 1.f / e.scale;
+        e.hi = exp2(1.0 / (double)e.scale) * (1.0 + kEdgeTol);
+        e.inv_width = 1.0 / (e.hi - (1.0 - kEdgeTol));
+        sh.bins[threadIdx.x] = e;
+    }
     const int n_req_nodes = n_hi - n_lo, n_trees = min(b_hi - b_lo, kMaxLive);
     const bool cached = !a.select_mode && n_req_nodes <= kCacheNodes && a.gamma < 256;
     if (!a.select_mode) {
@@ -1857,7 +1891,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     for (int k = 0; k < nA; ++k) ai = sh.A[k] == n_lo + pl ? k : ai;      // (nodes are unique)
                     sh.S_parent_idx[i] = ai;
                     sh.rho[i] = nd_score(0, n) - nd_score(0, pl);
-                    sh.uu[i] = nd_score(1, n) - nd_score(1, pl);
+                    sh.lq[i] = nd_score(1, n) - nd_score(1, pl);
                 }
             }
             __syncwarp();
@@ -1873,11 +1907,16 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             }
         } else if (warp <= 2) {
             live_weights(a, sh, warp - 1, warp == 1 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
+        } else if (warp == 3) {
+            // the drafts' uniforms, as many as there can be
+            if (!extra)
+#pragma unroll 1
+                for (int i = lane; i < kMaxLive; i += 32) sh.uu[i] = decision_uniform(a.seed, a.step, (uint32_t)r, (uint32_t)l, 0u, (uint32_t)i);
         } else if (!kWarped) {
             uint4 *words = reinterpret_cast<uint4 *>(hp);
 #pragma unroll 4
-            for (int i0 = 0; i0 < kHistArrays * kHistWords / 4; i0 += kVThreads - 96)
-                if (const int i = i0 + threadIdx.x - 96; i < kHistArrays * kHistWords / 4) words[i] = make_uint4(0, 0, 0, 0);
+            for (int i0 = 0; i0 < kHistArrays * kHistWords / 4; i0 += kVThreads - 128)
+                if (const int i = i0 + threadIdx.x - 128; i < kHistArrays * kHistWords / 4) words[i] = make_uint4(0, 0, 0, 0);
         }
         __syncthreads();
         const int m = uniform(sh.m);
@@ -1905,7 +1944,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     finish_supports(wsup, !extra, lane);
                     // rho of every live draft from the warped joints
                     if (!a.select_mode) {
-                        draft_tests(sh, a.seed, a.step, r, l, m, lane);
+                        draft_tests(sh, m, lane);
 #pragma unroll 1
                         for (int i0 = 0; i0 < m; i0 += 32) {
                             const int i = i0 + lane;
@@ -1947,7 +1986,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 // rejection 16 instead of 37.  Calls, W_min = 2: 64 requests x 8 rows 978 -> 907 us, 16 ragged requests 222 -> 164,
                 // one request of V = 32000 61 -> 53.) ----
                 if (warp == 0) {
-                    draft_tests(sh, a.seed, a.step, r, l, m, lane);
+                    draft_tests(sh, m, lane);
                     int first = m;                         // the first rejection
 #pragma unroll 1
                     for (int base = 0; base < m && first == m; base += 32) {
@@ -1960,7 +1999,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 __syncthreads();
                 on_demand = uniform(sh.on_demand);
             }
-            const float binscale = sh.binscale[m];
+            const BinEdges bins = sh.bins[m];
+            const float binscale = bins.scale;
             if (!on_demand) {
                 // ---- one pass: ratio histogram of the layer over the live rows ----
                 const int halves = item_halves(sh.nA * a.T, n_cta * kVWarps);
@@ -1973,67 +2013,67 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 cluster.sync();                            // every CTA's suffix sums are complete
                 TS(5);
                 if (threadIdx.x == 32) sh.halves = halves;
-                if (warp == 1 && !a.select_mode && !known) draft_tests(sh, a.seed, a.step, r, l, m, lane);
+                if (warp == 1 && !a.select_mode && !known) draft_tests(sh, m, lane);
             }
+            bool wrapped = false;
             // The chain c_{j+1} = F(s_j) from sh.chain_pos on (warp 0).  sh.need_exact = 1 where the histogram leaves one open.
             auto walk_chain = [&]() {
                 int j = uniform(sh.chain_pos), need = 0;
-                // lane 2 c + e looks up bin k + e in CTA c
-                const int c = min(lane >> 1, n_cta - 1);
-                const bool has = lane < 2 * n_cta;
-                const uint32_t *words = cluster.map_shared_rank(hs.wp, c) + (lane & 1);
-                const bool wrapped = __any_sync(kFull, *cluster.map_shared_rank(&sh.wrapped, c) != 0);
-                if (lane == 0 && wrapped && j == 1) ++sh.n_wrapped;
+                // lane c looks up bins k and k + 1 in CTA c
+                const uint32_t mine = lane < n_cta ? 0xffffffffu : 0u;
+                const uint32_t entries = cluster_address(hs.wp, min(lane, n_cta - 1));
                 const double n_cells = (double)sh.nA * (double)a.V;      // every cell of the live rows, at most
                 double s_j = sh.s_arr[j - 1], c_j = sh.c_arr[j];
 #pragma unroll 1
                 for (; j <= m; ++j) {
                     s_j += c_j;
                     if (lane == 0) { sh.s_arr[j] = s_j; sh.chain_len = j; }
-                    // every partial sum of the histogram is off by at most half a unit per cell
-                    const double fix_err = n_cells * (0.5 * kUnfix) * (1.0 + s_j);
-                    if (wrapped) { need = 1; break; }                // a wrapped word: exact passes only
                     // (up to s = 64 the bin found is off by at most 9e-7 of an edge: the logarithm's last place 3.3e-7, s as a
                     // float 0.6e-7, the product with binscale 5e-7; an edge by 6e-7.  The bracket below takes the edges
-                    // 2e-6 wider.  Approximate logarithm and exponential, reciprocals for the division: 1 us less, 1.6e-6)
-                    int k = (int)(log2f((float)s_j) * binscale);
-                    k = uniform(k < 0 || j == 1 ? 0 : k);            // (s_1 = 1, the first edge)
-                    if (k >= kBins) { need = 1; break; }             // cannot happen for s_j <= m
-                    uint32_t w[4] = {0u, 0u, 0u, 0u};
-                    if (has) {
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) w[x] = words[x * kHistWords + k];
-                    }
-                    // (the edges while the words are on their way)
-                    const double r_lo = (double)exp2f((float)k / binscale) * (1.0 - 2e-6);
-                    const double r_hi = (double)exp2f((float)(k + 1) / binscale) * (1.0 + 2e-6);
-                    const double inv = 1.0 / (r_hi - r_lo);
-                    double P = (double)(((unsigned long long)w[2] << 32) | w[0]);        // (whole numbers below 2^46: their sums
-                    double Q = (double)(((unsigned long long)w[3] << 32) | w[1]);        // are exact)
-#pragma unroll
-                    for (int o = 2; o < 32; o <<= 1) {
-                        P += __shfl_xor_sync(kFull, P, o);
-                        Q += __shfl_xor_sync(kFull, Q, o);
-                    }
-                    const double P0 = __shfl_sync(kFull, P, 0), Q0 = __shfl_sync(kFull, Q, 0);
-                    const double P1 = __shfl_sync(kFull, P, 1), Q1 = __shfl_sync(kFull, Q, 1);
-                    double lo_b = 0.0, hi_b = 0.0, c_next = (P0 - Q0) * kUnfix;
+                    // 2e-6 wider.)
+                    const int found = j == 1 ? 0 : (int)(log2f((float)s_j) * binscale), k = min(max(found, 0), kBins - 1);   // (s_1 = 1, the first edge)
+                    uint4 e0 = ld_cluster(entries + suffix_entry(k) * 16);
+                    const uint4 e1 = ld_cluster(entries + suffix_entry(k + 1) * 16);
+                    // the bin's edges while the words are on their way: t = k / binscale, correctly rounded but for rare last places
+                    const float t0 = (float)k * bins.inv_scale, t = fmaf(fmaf(-t0, binscale, (float)k), bins.inv_scale, t0);
+                    const double edge = (double)exp2f(t), inv = (double)exp2f(-t) * bins.inv_width;
+                    const double r_lo = edge * (1.0 - kEdgeTol), r_hi = edge * bins.hi;
+                    // every partial sum of the histogram is off by at most half a unit per cell
+                    const double fix_err = n_cells * (0.5 * kUnfix) * (1.0 + s_j);
+                    if (j == 1 && __any_sync(kFull, e0.y & mine & kWrapped)) wrapped = true;
+                    e0.y &= ~kWrapped;
+                    // the sums over the CTAs in two parts of 24 and 22 bits, so that a part's sum is one word; [0] above the bin, [1] in it
+                    double P[2], Q[2];
+                    auto add = [&](uint32_t low0, uint32_t high0, uint32_t low1, uint32_t high1, double (&sum)[2]) {
+                        const unsigned lo0 = __reduce_add_sync(kFull, low0 & mine & 0xffffffu), hi0 = __reduce_add_sync(kFull, __funnelshift_l(low0, high0, 8) & mine);
+                        const unsigned lo1 = __reduce_add_sync(kFull, low1 & mine & 0xffffffu), hi1 = __reduce_add_sync(kFull, __funnelshift_l(low1, high1, 8) & mine);
+                        sum[0] = fma((double)hi1, 16777216.0, (double)lo1);
+                        sum[1] = fma((double)(int)(hi0 - hi1), 16777216.0, (double)(int)(lo0 - lo1));
+                    };
+                    add(e0.x, e0.y, e1.x, e1.y, P);
+                    add(e0.z, e0.w, e1.z, e1.w, Q);
+                    // (in units of 2^-44)
+                    double lo_b = 0.0, hi_b = 0.0, c_next = (P[0] + P[1]) - (Q[0] + Q[1]);
                     if (j > 1) {
-                        const double Pk = (P0 - P1) * kUnfix, Qk = (Q0 - Q1) * kUnfix;
-                        lo_b = fmax(Pk - s_j * Qk, 0.0);
-                        const double q_hi = fmin(fmax((Pk - r_lo * Qk) * inv, 0.0), Qk);
-                        hi_b = fmax(q_hi * (r_hi - s_j), lo_b);
-                        c_next = fmax(P1 * kUnfix - s_j * (Q1 * kUnfix), 0.0) + 0.5 * (lo_b + hi_b);
+                        auto larger = [](double x, double y) { return x > y ? x : y; };
+                        lo_b = larger(P[1] - s_j * Q[1], 0.0);
+                        double q_hi = larger((P[1] - r_lo * Q[1]) * inv, 0.0);
+                        q_hi = q_hi < Q[1] ? q_hi : Q[1];
+                        hi_b = larger(q_hi * (r_hi - s_j), lo_b);
+                        c_next = larger(P[0] - s_j * Q[0], 0.0) + 0.5 * (lo_b + hi_b);
                     }
+                    c_next *= kUnfix;
                     // the midpoint of the bracket is used: half its width plus the fixed-point term
-                    need = uniform(0.5 * (hi_b - lo_b) + fix_err > kErrTol);
+                    // (a wrapped word: exact passes only)
+                    need = __any_sync(kFull, 0.5 * kUnfix * (hi_b - lo_b) + fix_err > kErrTol || found >= kBins || wrapped);
                     if (need) break;
                     if (lane == 0) sh.c_arr[j + 1] = c_next;
                     c_j = c_next;
-                    if (!uniform(c_next > 0.0)) j = m;               // chain exhausted: stop walking
+                    if (!__any_sync(kFull, c_next > 0.0)) j = m;     // chain exhausted: stop walking
                 }
                 if (lane == 0) {
                     sh.need_exact = need;
+                    if (need && wrapped && j == 1) ++sh.n_wrapped;
                     sh.chain_pos = need ? j : m + 1;
                 }
             };
@@ -2072,16 +2112,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         if (warp == 0 && !uniform(sh.err)) {
             int W = W_known;
             if (!on_demand && !extra) {
-                // alpha_j = 1 - c_{j+1}/c_j; once a residual has no mass every later alpha is 1
-#pragma unroll 1
-                for (int j0 = 1; j0 <= m; j0 += 32) {
-                    const int j = min(j0 + lane, m);         // (the last one more than once)
-                    double al = 1.0;
-                    if (j <= sh.chain_len && sh.c_arr[j] > 0.0 && sh.c_arr[j + 1] > 0.0)
-                        al = fmin(fmax(1.0 - sh.c_arr[j + 1] / sh.c_arr[j], 0.0), 1.0);
-                    sh.alpha[j] = al;
-                }
-                __syncwarp();
                 // (the verification only needs W~ up to W_max and can stop at the first tail below the
                 // threshold; dsbd_select_width returns the whole tail)
                 const int wt = width_rule(sh, m, a.thresh, lane, a.select_mode ? -1 : W_max);
@@ -2091,6 +2121,14 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             if (a.select_mode) {
                 if (writer && lane == 0) {
                     a.width_out[r] = W;
+                    // alpha_j = 1 - c_{j+1}/c_j; once a residual has no mass every later alpha is 1
+#pragma unroll 1
+                    for (int j = 1; j <= m; ++j) {
+                        double al = 1.0;
+                        if (j <= sh.chain_len && sh.c_arr[j] > 0.0 && sh.c_arr[j + 1] > 0.0)
+                            al = fmin(fmax(1.0 - sh.c_arr[j + 1] / sh.c_arr[j], 0.0), 1.0);
+                        sh.alpha[j] = al;
+                    }
                     if (a.alpha_out)
 #pragma unroll 1
                         for (int j = 0; j < m && j < a.out_stride; ++j)

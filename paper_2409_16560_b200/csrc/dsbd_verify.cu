@@ -172,14 +172,16 @@ __device__ __forceinline__ double row_lse(const TileStat *s, int T, double inv_t
     float top = -INFINITY;
 #pragma unroll 4
     for (int t0 = 0; t0 < T; t0 += 32)
-        if (const int t = t0 + lane; t < T) top = fmaxf(top, s[t].mx);
+        if (t0 + lane < T) top = fmaxf(top, s[t0 + lane].mx);
     const double mx = (double)warp_max(top);
     double acc = 0.0;
     if (mx > -INFINITY)
-#pragma unroll 1
-        for (int t0 = 0; t0 < T; t0 += 32)
-            if (const int t = t0 + lane; t < T)
-            if (s[t].sum > 0.f) acc += (double)s[t].sum * exp(((double)s[t].mx - mx) * inv_tau);
+#pragma unroll 2
+        for (int t0 = 0; t0 < T; t0 += 32) {
+            const TileStat x = s[min(t0 + lane, T - 1)];
+            const double e = (double)x.sum * exp(((double)x.mx - mx) * inv_tau);
+            if (t0 + lane < T && x.sum > 0.f) acc += e;
+        }
     acc = warp_sum(acc);
     return (mx > -INFINITY) ? mx * inv_tau + log(acc) : -INFINITY;
 }
@@ -482,13 +484,11 @@ __device__ __forceinline__ void log_softmax_warp(const double *s, int n, int lan
 
 // The weights of one model (0: p, 1: q) over the live set: softmax of the cumulative scores over A (Eq. 1 factorised),
 // by one warp; the two models' warps work side by side.
-// nc: the request's node cache or nullptr; n_lo: first node of the request.
-__device__ void live_weights(const VerifyArgs &a, Shared &sh, int model, const double *scores, int lane,
-                             const NodeCache *nc, int n_lo) {
+// lse: the model's log-sum-exps by node.
+__device__ __forceinline__ void live_weights(Shared &sh, int model, const double *scores, const double *lse, int lane) {
     double *lw = model ? sh.lwq : sh.lwp;
     const int nA = uniform(sh.nA);
     log_softmax_warp(scores, nA, lane, lw);
-    const double *lse = nc ? (model ? nc->lse_q : nc->lse_p) - n_lo : a.lse + (int64_t)model * a.N;
 #pragma unroll 1
     for (int i0 = 0; i0 < nA; i0 += 32) {
         const int i = i0 + lane;
@@ -1172,7 +1172,7 @@ struct SupportTmp {
     int sel[256];                 // tiles whose bound reaches the threshold
     unsigned lo[kVWarps], hi[kVWarps];   // per warp, images of the smallest finite and of the largest bound
     int finite[kVWarps];          // per warp, finite bounds
-    int count[3];                 // of the bisection's rounds, in turn
+    int count[3][3];              // of a round's three cuts, for three rounds in turn
     unsigned low;                 // image of the smallest bound from the cut on
     int n_sel, n_cand, err;
 };
@@ -1198,14 +1198,15 @@ __device__ __forceinline__ void part_sync(int model) {
 // Support of the warped joint of one model by NT threads: a half of the CTA for each model (warps 0-7: p, warps
 // 8-15: q) side by side on their own scratch, or the whole CTA where only p is wanted.  hist_p / hist_q: the first two
 // of the idle histogram arrays.  Returns 0 or a DSBD_DEV_* code (the same on every thread of the part).
-// Latency decides (a chain of short steps between barriers): the threshold is a bisection whose rounds have one
-// barrier each and that stops at the first cut with k to k + 2 tiles above it, about 8 rounds.  Exact radix
+// Latency decides (a chain of short steps between barriers): the threshold is a search whose rounds have one
+// barrier each, try three cuts and stop at the first with k tiles above it or not many more, about 4 rounds (with one cut a round and at most
+// k + 2 tiles 8 rounds, 2.3 us of a draft layer's 11).  Exact radix
 // selection (4 rounds of three barriers with colliding atomics), one warp that lists the tiles, one thread that cuts
 // at top-p and half the CTA for a draft layer's only model took, for a draft of 5 layers of 16 x 8 rows of 128256 with
 // top-k 10, 419 us instead of 337; 20 requests with top-k 50 took 169 instead of 144.  (As a function that is
 // not inlined, with generic loads: 363 and 165.)
 template <int NT>
-__device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, uint32_t *hist_p, uint32_t *hist_q) {
+__device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, const double *lse, uint32_t *hist_p, uint32_t *hist_q) {
     WarpScratch &ws = *reinterpret_cast<WarpScratch *>(hist_q);
     SupportTmp &tp = ws.tmp[model];
     double *cand_key = reinterpret_cast<double *>(hist_p) + model * kMaxCand;
@@ -1216,12 +1217,11 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
     const int T = a.T, nt = uniform(sh.nA) * T, k = a.top_k;
     const TileStat *stats = a.stats + (int64_t)model * a.N * T;
     const double *lw = model ? sh.lwq : sh.lwp;
-    const double *lse = a.lse + (int64_t)model * a.N;
     const float *z = model ? a.zq : a.zp;
     const float inv_tau_f = (float)a.inv_tau;
 #pragma unroll 1
     for (int i = tl; i < sh.nA; i += NT) tp.off[i] = (float)(lw[i] - lse[sh.A[i]]);
-    if (tl < 3) tp.count[tl] = 0;
+    if (tl < 3) tp.count[0][tl] = 0;
     if (tl == 0) { tp.low = 0xffffffffu; tp.n_sel = 0; tp.n_cand = 0; tp.err = 0; ws.n[model] = 0; }
     part_sync<NT>(model);
     // float upper bound of log(joint probability) over tile i
@@ -1256,36 +1256,45 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, u
         if (lane == 0) { tp.lo[warp] = lo; tp.hi[warp] = hi; tp.finite[warp] = finite; }
     }
     part_sync<NT>(model);
-    unsigned lo = 0xffffffffu, hi = 0u;
-    int finite = 0;
-#pragma unroll
-    for (int w = 0; w < kPartWarps; ++w) { lo = min(lo, tp.lo[w]); hi = max(hi, tp.hi[w]); finite += tp.finite[w]; }
-    lo = uniform(lo); hi = uniform(hi); finite = uniform(finite);
+    unsigned lo = __reduce_min_sync(kFull, tp.lo[lane & (kPartWarps - 1)]), hi = __reduce_max_sync(kFull, tp.hi[lane & (kPartWarps - 1)]);
+    const int finite = __reduce_add_sync(kFull, lane < kPartWarps ? tp.finite[lane] : 0);
     if (finite >= k) {
-        // count(>= lo) >= k always holds; hi is above the k-th largest.  One or two too many are fine where they are close
-        // (cells 30 below the largest have no mass to speak of)
+        // count(>= lo) >= k always holds; hi is above the k-th largest.  A tile for every warp costs no more than k of them, and one or
+        // two too many are fine, where they are close (cells 30 below the largest have no mass to speak of)
         const float near = value(hi) - 30.f;
+        const int enough = max(k + 2, kPartWarps);
         ++hi;
+#pragma unroll 1
         for (int round = 0; hi - lo > 1; ++round) {
-            const unsigned mid = lo + (hi - lo) / 2;
-            int n = 0;
+            const unsigned step = max((hi - lo) >> 2, 1u);           // (a cut at hi or above it counts fewer than k)
+            int n[3] = {0, 0, 0};
+            auto count = [&](unsigned u) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) n[c] += u >= lo + (c + 1) * step;
+            };
             if (cached) {
-#pragma unroll 4
+#pragma unroll 2
                 for (int i0 = 0; i0 < nt; i0 += NT)
-                    if (const int i = i0 + tl; i < nt) n += bcache[i] >= mid;
+                    if (const int i = i0 + tl; i < nt) count(bcache[i]);
             } else {
 #pragma unroll 1
                 for (int i0 = 0; i0 < nt; i0 += NT)
-                    if (const int i = i0 + tl; i < nt) n += image(bound(i)) >= mid;
+                    if (const int i = i0 + tl; i < nt) count(image(bound(i)));
             }
-            n = __reduce_add_sync(kFull, n);
-            if (lane == 0 && n) atomicAdd(&tp.count[round % 3], n);
-            if (tl == 0) tp.count[(round + 1) % 3] = 0;           // (last read two rounds ago)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) n[c] = __reduce_add_sync(kFull, n[c]);
+            int *counts = tp.count[round % 3], *next = tp.count[(round + 1) % 3];
+            if (lane < 3) {
+                atomicAdd(&counts[lane], lane == 0 ? n[0] : lane == 1 ? n[1] : n[2]);
+                if (warp == 0) next[lane] = 0;                       // (last read two rounds ago)
+            }
             part_sync<NT>(model);
-            n = uniform(tp.count[round % 3]);
-            if (n < k) { hi = mid; continue; }
-            lo = mid;
-            if (n == k || (n <= k + 2 && value(lo) > near)) break;
+            const int mine = counts[min(lane, 2)], at = __popc(__ballot_sync(kFull, mine >= k) & 7u);      // cuts with at least k
+            if (at < 3) hi = min(hi, lo + (at + 1) * step);
+            lo += at * step;
+            if (at == 0) continue;
+            const int reached = __shfl_sync(kFull, mine, at - 1);
+            if (reached == k || (reached <= enough && value(lo) > near)) break;
         }
     }
     // The tiles from the cut on, and the smallest bound among them, which is the threshold: a cut may lie far down in
@@ -1820,6 +1829,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     // node data by local index, from the cache when there is one
     auto nd_depth = [&](int i) -> int { return cached ? (int)nc.depth[i] : a.depth[n_lo + i]; };
     auto nd_parent = [&](int i) -> int { return cached ? (int)nc.parent[i] : a.parent[n_lo + i] - n_lo; };
+    auto node_lse = [&](int model) -> const double * {
+        return cached ? (model ? nc.lse_q : nc.lse_p) - n_lo : a.lse + (int64_t)model * a.N;
+    };
     auto nd_score = [&](int model, int i) -> double {
         return cached ? (model ? nc.score_q[i] : nc.score_p[i]) : a.score[(int64_t)model * a.N + n_lo + i];
     };
@@ -1906,7 +1918,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 sh.added = 0ull;
             }
         } else if (warp <= 2) {
-            live_weights(a, sh, warp - 1, warp == 1 ? sp_live : sq_live, lane, cached ? &nc : nullptr, n_lo);
+            live_weights(sh, warp - 1, warp == 1 ? sp_live : sq_live, node_lse(warp - 1), lane);
         } else if (warp == 3) {
             // the drafts' uniforms, as many as there can be
             if (!extra)
@@ -1935,7 +1947,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             {
                 // the first half of the warps builds the support of p, the second that of q, side by side (p alone in the extra layer)
                 const int half = warp / (kHalf / 32);
-                const int e_half = extra && half ? 0 : build_support<kHalf>(a, sh, half, hp, hq);
+                const int e_half = extra && half ? 0 : build_support<kHalf>(a, sh, half, node_lse(half), hp, hq);
                 if (e_half && (threadIdx.x & (kHalf - 1)) == 0) wsup.tmp[half].err = e_half;
                 __syncthreads();
                 const int e = uniform(wsup.tmp[0].err ? wsup.tmp[0].err : extra ? 0 : wsup.tmp[1].err);
@@ -2524,7 +2536,7 @@ k_draft(const __grid_constant__ DraftArgs d) {
         if (lane == 0) { lse[i] = v; a.lse_w[b_lo + i] = v; }
     }
     __syncthreads();
-    if (warp == 0) live_weights(a, sh, 0, score, lane, nullptr, 0);
+    if (warp == 0) live_weights(sh, 0, score, lse - b_lo, lane);
     __syncthreads();
     const int n_draw = err ? 0 : min(W, max(cap, 0));
     auto emit = [&](int kk, int ia, int tok) {
@@ -2535,7 +2547,7 @@ k_draft(const __grid_constant__ DraftArgs d) {
     };
     if (a.top_k > 0) {
         WarpScratch &ws = *reinterpret_cast<WarpScratch *>(hq);
-        if (!err) err = build_support<kVThreads>(a, sh, 0, hp, hq);
+        if (!err) err = build_support<kVThreads>(a, sh, 0, lse - b_lo, hp, hq);
         if (!err && warp == 0) {
             finish_supports(ws, false, lane);
 #pragma unroll 1

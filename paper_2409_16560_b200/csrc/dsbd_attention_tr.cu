@@ -68,8 +68,14 @@ struct Shape {
     static constexpr int kHalves = D / 64;                    // 64-column halves of a row of Q, K or V
     static constexpr uint32_t kSlot = kTile * D * 2;          // one K or V tile
     static constexpr uint32_t kPTerm = kHalfStride;                                     // [token][128 B]
-    static constexpr uint32_t kPBuf = (kSplit ? 2 : 1) * kPTerm;
-    static constexpr int kPBufs = 2;
+    // Up to 32 rows: both terms in one operand (a token's 128 bytes: 32 rows of the first term, 32 of the second) and in columns of their
+    // own of the accumulators, which the output adds.  A product of 48 or 64 columns takes as long as one of 32 (the
+    // traffic of A), so a tile's O^T is issued in 500 cycles instead of 975; and four P buffers fit instead of two, so that S^T
+    // no longer waits for the O^T two tiles back.  (8 x 4 beams after 512 to 2047 tokens: 31.5 us a call -> 30.5.)
+    static constexpr bool kJoint = kSplit && NMAX == 32;
+    static constexpr uint32_t kPBuf = (kSplit && !kJoint ? 2 : 1) * kPTerm;
+    static constexpr int kPBufs = kJoint ? 4 : 2;
+    static constexpr uint32_t kOCols = kJoint ? 2 * NMAX : NMAX;                        // of one unit's accumulators
     static constexpr bool kSWaits = D == 64 || NMAX == 64;                  // S^T waits until the tile's P buffer is free
     // query rows of one unit, or of two when they fit (a unit's copy then runs a whole unit ahead; with one
     // buffer its latency, 2800 cycles while HBM is saturated, shows at every unit's start)
@@ -145,7 +151,7 @@ struct __align__(16) Seg {
 constexpr int kMaxSlots = 4, kSegs = 8;
 struct Barriers {
     unsigned long long k_full[kMaxSlots], k_empty[kMaxSlots], v_full[kMaxSlots], v_empty[kMaxSlots];
-    unsigned long long s_full[4], p_full[4], pv_done[2], q_full[2], q_empty[2];
+    unsigned long long s_full[4], p_full[4], pv_done[4], q_full[2], q_empty[2];
     unsigned long long sum_full[2], o_full[2], o_empty[2];     // by unit parity
     unsigned long long drain[2];
     unsigned long long seg_full[kSegs], seg_empty[kSegs];
@@ -412,9 +418,9 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
             mbar_init(&sb.k_full[s], 1); mbar_init(&sb.k_empty[s], 1);
             mbar_init(&sb.v_full[s], 1); mbar_init(&sb.v_empty[s], 1);
         }
-        for (int b = 0; b < 4; ++b) { mbar_init(&sb.s_full[b], 1); mbar_init(&sb.p_full[b], kGroups * 4); }
+        for (int b = 0; b < 4; ++b) { mbar_init(&sb.s_full[b], 1); mbar_init(&sb.p_full[b], kGroups * 4); mbar_init(&sb.pv_done[b], 1); }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&sb.pv_done[b], 1); mbar_init(&sb.q_full[b], 1); mbar_init(&sb.q_empty[b], 1);
+            mbar_init(&sb.q_full[b], 1); mbar_init(&sb.q_empty[b], 1);
             mbar_init(&sb.sum_full[b], kGroups * 4); mbar_init(&sb.o_full[b], 1); mbar_init(&sb.o_empty[b], 4);
             mbar_init(&sb.drain[b], 1);
         }
@@ -538,10 +544,10 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                 const uint32_t s = tile % S::kKSlots, sbuf = tile % S::kSBufs;
                 ok = warp_wait(&sb.k_full[s], (tile / S::kKSlots) & 1, &sb);
                 // The softmax has read what the buffer held.  Where the softmax sets the pace (d = 64, more than 32
-                // rows): wait for the O^T product two tiles back, which came after; S^T then also says that the
-                // tile's P buffer is free.  Where HBM does: no longer than needed, so that the K slot is free early.
+                // rows): wait for the O^T product that last read the tile's P buffer, which came after; S^T then also says
+                // that the buffer is free.  Where HBM does: no longer than needed, so that the K slot is free early.
                 if (S::kSWaits) {
-                    if (ok && tile >= 2) ok = warp_wait(&sb.pv_done[tile & 1], ((tile - 2) >> 1) & 1, &sb);
+                    if (ok && tile >= S::kPBufs) ok = warp_wait(&sb.pv_done[tile % S::kPBufs], (tile / S::kPBufs - 1) & 1, &sb);
                 } else if (ok && tile >= S::kSBufs) {
                     ok = warp_wait(&sb.p_full[sbuf], (tile / S::kSBufs - 1) & 1, &sb);
                 }
@@ -565,8 +571,8 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
         uint32_t tile = 0, unit = 0;
         bool ok = true;
         while (ok && get_seg(sb, unit, sg)) {
-            const uint32_t idesc = instr_desc(128, max(16, (sg.rows + 15) & ~15), 1, 1);
-            const uint32_t col = tmem + S::kColO + (unit & 1) * NMAX;
+            const uint32_t idesc = instr_desc(128, (S::kJoint ? NMAX : 0) + max(16, (sg.rows + 15) & ~15), 1, 1);
+            const uint32_t col = tmem + S::kColO + (unit & 1) * S::kOCols;
             // the accumulators were last used two units ago
             ok = warp_wait(&sb.o_empty[unit & 1], ((unit >> 1) & 1) ^ 1, &sb);
 #pragma unroll 1
@@ -594,7 +600,7 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                 const bool both = sg.nh - 2 * j >= 2;        // a lone box: 64 tokens
                 const uint32_t acc = j > sg.t0 ? 1u : 0u;
 #pragma unroll
-                for (int term = 0; term < (S::kSplit ? 2 : 1); ++term) {
+                for (int term = 0; term < (S::kSplit && !S::kJoint ? 2 : 1); ++term) {
                     const uint64_t pd = desc_mn_major(
                         smem_u32(p_s + (tile % S::kPBufs) * S::kPBuf + term * S::kPTerm), kHalfStride);
 #pragma unroll
@@ -603,7 +609,7 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                                pd + (uint64_t)(ks * ((16 * 128) >> 4)), idesc, (term + ks > 0) ? 1u : acc);
                 }
                 tc_commit(on, &sb.v_empty[s]);
-                tc_commit(on, &sb.pv_done[tile & 1]);
+                tc_commit(on, &sb.pv_done[tile % S::kPBufs]);
             }
             if (ok) tc_commit(on, &sb.o_full[unit & 1]);
             ++unit;
@@ -640,7 +646,7 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
             if (sg.layer != rec_layer) { put_rec(rec_layer); rec = CutRec{}; rec_layer = sg.layer; }
             const int rows = sg.rows;
             const uint32_t ub = unit & 1;
-            const uint32_t o_addr = tmem + lane_base + S::kColO + ub * NMAX;
+            const uint32_t o_addr = tmem + lane_base + S::kColO + ub * S::kOCols;
             bool ok = warp_wait(&sb.sum_full[ub], (unit >> 1) & 1, &sb);
             if (ok) ok = warp_wait(&sb.o_full[ub], (unit >> 1) & 1, &sb);
             if (group_any(kGroups, !ok)) break;
@@ -670,9 +676,14 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                                      (tid & ~1);
 #pragma unroll 1
                 for (int r0 = 0; r0 < rows; r0 += 8) {
-                    uint32_t ov[8];
+                    uint32_t ov[8], ow[8];
                     tmem_ld8(o_addr + r0, ov);
+                    if (S::kJoint) tmem_ld8(o_addr + NMAX + r0, ow);
                     tmem_wait_ld();
+                    if (S::kJoint) {
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) + __uint_as_float(ow[c]));
+                    }
                     float v[8];
 #pragma unroll
                     for (int c = 0; c < 8; c += 4) {
@@ -717,7 +728,7 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
             const int rows = sg.rows;
             const int n8 = (rows + 7) / 8, per = (n8 + kGroups - 1) / kGroups;
             const int cbase = grp * per * 8, nch = min(max(n8 - grp * per, 0), per);
-            const uint32_t o_addr = tmem + lane_base + S::kColO + (unit & 1) * NMAX + cbase;
+            const uint32_t o_addr = tmem + lane_base + S::kColO + (unit & 1) * S::kOCols + cbase;
             float l[S::kCols];
 #pragma unroll
             for (int c = 0; c < S::kCols; ++c) l[c] = 0.f;
@@ -807,7 +818,7 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                 }
                 // the P buffer is free once the product that last read it has landed
                 if (!S::kSWaits && ok && tile >= S::kPBufs)
-                    ok = warp_wait(&sb.pv_done[(tile - S::kPBufs) & 1], ((tile - S::kPBufs) >> 1) & 1, &sb);
+                    ok = warp_wait(&sb.pv_done[tile % S::kPBufs], (tile / S::kPBufs - 1) & 1, &sb);
                 // the weights: bf16 pairs (SPLIT: the sums of their two terms) of the group's rows
                 constexpr int kW = S::kSplit ? S::kCols : S::kCols / 2;
                 uint32_t w[kW];
@@ -847,9 +858,11 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                                 }
                             }
                             const int r8 = cbase / 8 + ch;   // eight rows are one 16-byte piece of the token's line
-                            unsigned char *to = p_s + (tile % S::kPBufs) * S::kPBuf + tok * 128 + ((r8 ^ (tok & 7)) << 4);
-                            *reinterpret_cast<uint4 *>(to) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                            if (S::kSplit) *reinterpret_cast<uint4 *>(to + S::kPTerm) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                            unsigned char *line = p_s + (tile % S::kPBufs) * S::kPBuf + tok * 128;
+                            const int at = (r8 ^ (tok & 7)) << 4;
+                            *reinterpret_cast<uint4 *>(line + at) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                            if (S::kSplit)             // (joint: rows + 32, four pieces on)
+                                *reinterpret_cast<uint4 *>(line + (S::kJoint ? at ^ 64 : at + (int)S::kPTerm)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 if (S::kSplit) {
@@ -865,7 +878,7 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                     if (!group_any(grp, !ok || over > S::kMoveRef) || attempt == 2) break;
                     // rare: some reference has to move (or a wait ran out): O^T is rescaled, so the previous
                     // product must have landed
-                    if (ok && j > sg.t0) ok = warp_wait(&sb.pv_done[(tile - 1) & 1], ((tile - 1) >> 1) & 1, &sb);
+                    if (ok && j > sg.t0) ok = warp_wait(&sb.pv_done[(tile - 1) % S::kPBufs], ((tile - 1) / S::kPBufs) & 1, &sb);
                     if (group_any(grp, !ok)) { ok = false; break; }
                     tc_fence_after();
 const float m = column_max();
@@ -878,14 +891,16 @@ const float m = column_max();
                     group_sync(grp);
                     if (j > sg.t0) {
 #pragma unroll 1
-                        for (int ch = 0; ch < nch; ++ch) {
+                        for (int i = 0; i < (S::kJoint ? 2 : 1) * nch; ++i) {
+                            const int ch = i < nch ? i : i - nch;                      // (the second term's columns)
+                            const uint32_t at = o_addr + ch * 8 + (i < nch ? 0 : NMAX);
                             uint32_t ov[8];
-                            tmem_ld8(o_addr + ch * 8, ov);
+                            tmem_ld8(at, ov);
                             tmem_wait_ld();
 #pragma unroll
                             for (int c = 0; c < 8; ++c)
                                 ov[c] = __float_as_uint(__uint_as_float(ov[c]) * sx.move[grp][ch * 8 + c]);
-                            tmem_st8(o_addr + ch * 8, ov);
+                            tmem_st8(at, ov);
                         }
                         tmem_wait_st();
 #pragma unroll

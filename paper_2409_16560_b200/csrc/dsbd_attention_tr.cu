@@ -104,9 +104,9 @@ constexpr uint32_t kWaitTries = 250;
 constexpr uint32_t kWaitTries = 500000;
 #endif
 
-// What a run left for the merge.  tail: its last unit starts here and goes on in the next run; head_ends:
-// the part of a unit that the run began with is the last one of that unit.
-struct CutRec { int tail, head_ends, b, g, rb, pad0, pad1, pad2; };
+// What a run left for the merge.  tail: its last unit (of the tree n_lo .. n_lo + n_tree) starts here and goes on in the next run;
+// head_ends: the part of a unit that the run began with is the last one of that unit.
+struct CutRec { int tail, head_ends, g, rb, n_lo, n_tree, pad0, pad1; };
 
 struct TcArgs {
     int B, N, Hq, Hkv, group;
@@ -335,7 +335,7 @@ __device__ __forceinline__ int share(int n, int r, int G) { return n / G * r + m
 // Finds the run of this CTA: first unit and tile, number of tiles (all threads).
 template <int kThreads>
 __device__ void find_run(const TcArgs &a, Barriers &sb) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(kFull, tid >> 5, 0);
     const bool joint = a.whole && a.uni_nt;                   // the units of all layers in one sequence
     const int r = joint ? (int)blockIdx.x : (int)blockIdx.x % a.runs, G = joint ? (int)gridDim.x : a.runs;
     const int units = a.B * a.Hkv * (joint ? a.n_layers : 1);     // (where row blocks are one per tree)
@@ -361,9 +361,10 @@ __device__ void find_run(const TcArgs &a, Barriers &sb) {
     const int per = (a.B + kThreads - 1) / kThreads;
     const int b0 = min(tid * per, a.B), b1 = min(b0 + per, a.B);
     int sum = 0;
+    BeamFacts f = {};                                        // of the last beam of the share (nearly always its only one)
 #pragma unroll 1
     for (int b = b0; b < b1; ++b) {
-        const BeamFacts f = beam_facts(a, b);
+        f = beam_facts(a, b);
         sum += (f.nt + a.unit_cost) * f.nrb * a.Hkv;
     }
     int incl = sum;
@@ -375,15 +376,15 @@ __device__ void find_run(const TcArgs &a, Barriers &sb) {
     if (lane == 31) sb.scan[warp] = incl;
     if (tid == 0) { sb.start[0] = 0; sb.start[1] = 0; sb.start[2] = 0; sb.run = 0; }
     __syncthreads();
-    int before = incl - sum, total = 0;
-#pragma unroll 1
-    for (int w = 0; w < kThreads / 32; ++w) { if (w < warp) before += sb.scan[w]; total += sb.scan[w]; }
+    static_assert(kThreads <= 1024, "the warps' sums fit the lanes");
+    const int scan = lane < kThreads / 32 ? sb.scan[lane] : 0;
+    const int before = incl - sum + __reduce_add_sync(kFull, lane < warp ? scan : 0), total = __reduce_add_sync(kFull, scan);
     const int lo = share(total, r, G), hi = share(total, r + 1, G);
     if (lo < hi && lo >= before && lo < before + sum) {
         int at = before;
 #pragma unroll 1
         for (int b = b0; b < b1; ++b) {
-            const BeamFacts f = beam_facts(a, b);
+            if (per > 1) f = beam_facts(a, b);
             const int cost = f.nt + a.unit_cost, w = cost * f.nrb * a.Hkv;
             if (lo < at + w) {
                 sb.start[0] = b; sb.start[1] = (lo - at) / cost; sb.start[2] = (lo - at) % cost;
@@ -657,7 +658,7 @@ k_forest_attn_tr(const __grid_constant__ CUtensorMap map_kp, const __grid_consta
                 part += (2 * ((int64_t)sg.layer * a.runs + (int)blockIdx.x % a.runs) + (sg.t0 == 0 ? 1 : 0)) *
                         NMAX * (D + 2);
                 if (sg.t0 > 0) rec.head_ends = sg.last;
-                else { rec.tail = 1; rec.b = sg.b; rec.g = sg.g; rec.rb = sg.rb; }
+                else { rec.tail = 1; rec.g = sg.g; rec.rb = sg.rb; rec.n_lo = sg.n_lo; rec.n_tree = sg.n_tree; }
             }
             if (tid < rows) {
                 const float sum = (sx.red[ub][0][tid] + sx.red[ub][1][tid]) + (sx.red[ub][2][tid] + sx.red[ub][3][tid]);
@@ -956,7 +957,8 @@ const float m = column_max();
 }
 
 // Merge of the units that were cut: block (i, y, layer) takes the unit that starts as the last one of run i,
-// warps over its rows; out = sum_p O_p 2^(m_p - m) / sum_p l_p 2^(m_p - m).
+// a warp to a row (a chain of four loads from L2 each; with 32 rows to a block of 8 warps the kernel took 5.6 us, 3.5 now);
+// out = sum_p O_p 2^(m_p - m) / sum_p l_p 2^(m_p - m).
 constexpr int kMergeThreads = 256;
 template <int D, int NMAX>
 __global__ void __launch_bounds__(kMergeThreads)
@@ -964,14 +966,15 @@ k_attn_merge(TcArgs a) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int layer = blockIdx.z, i0 = layer * a.runs + (int)blockIdx.x, end = (layer + 1) * a.runs - 1;
     const CutRec rec = a.recs[i0];
+    int last = min(i0 + 1, end);                             // the runs that hold the other parts
+    int ends = a.recs[last].head_ends;
     if (!rec.tail) return;
     // (no unit of this forest: a CTA that left before it wrote its records)
-    if ((unsigned)rec.b >= (unsigned)a.B || (unsigned)rec.g >= (unsigned)a.Hkv || (unsigned)rec.rb > (unsigned)kMaxTree) return;
-    int last = min(i0 + 1, end);                             // the runs that hold the other parts
-    while (last < end && !a.recs[last].head_ends) ++last;
-    const int n_lo = a.beam_node_off[rec.b];
-    const int n_tree = min(a.beam_node_off[rec.b + 1] - n_lo, kMaxTree);
-    const int rows = min(a.block_rows, n_tree * a.group - rec.rb * a.block_rows);
+    if (rec.n_lo < 0 || (unsigned)rec.n_tree > (unsigned)kMaxTree || rec.n_lo + rec.n_tree > a.N || (unsigned)rec.g >= (unsigned)a.Hkv ||
+        (unsigned)rec.rb > (unsigned)kMaxTree) return;
+    while (last < end && !ends) ends = a.recs[++last].head_ends;
+    const int n_lo = rec.n_lo;
+    const int rows = min(a.block_rows, rec.n_tree * a.group - rec.rb * a.block_rows);
     const int lane = threadIdx.x & 31;
     constexpr int kPer = D / 32;                             // values per lane: 2 (d = 64) or 4
     for (int row = (blockIdx.y * kMergeThreads + threadIdx.x) >> 5; row < rows; row += gridDim.y * kMergeThreads / 32) {
@@ -1083,7 +1086,7 @@ int launch(const TcPlan &p, const CUtensorMap (&maps)[5], TcArgs a, cudaStream_t
         cudaSuccess)
         return DSBD_ERR_CUDA;
     if (p.whole) return DSBD_OK;
-    cfg.gridDim = dim3((unsigned)p.runs, (unsigned)((p.block_rows + 31) / 32), (unsigned)a.n_layers);
+    cfg.gridDim = dim3((unsigned)p.runs, (unsigned)((p.block_rows + kMergeThreads / 32 - 1) / (kMergeThreads / 32)), (unsigned)a.n_layers);
     cfg.blockDim = dim3(kMergeThreads);
     cfg.dynamicSmemBytes = 0;
     return cudaLaunchKernelEx(&cfg, k_attn_merge<D, NMAX>, a) == cudaSuccess ? DSBD_OK : DSBD_ERR_CUDA;

@@ -429,6 +429,8 @@ struct NodeCache {
     uint8_t depth[kCacheNodes];
     uint8_t tree[kCacheNodes];            // tree of the node, inside the request
     int root[kMaxLive];                   // first node of every tree
+    int rank[kCacheNodes];                // draft_rank, where the caller gave one
+    uint8_t live[kCacheNodes];            // index of an accepted node among the live rows
 };
 
 // Writes output beam number `index` of request r (the caller has checked the slot range).  nc: the
@@ -1550,14 +1552,14 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     TS(1);
     // (a CTA may store into another's shared memory once that CTA runs: arrived here, waited for below)
     cluster.barrier_arrive();
-    if (!kWarped && threadIdx.x <= kMaxLive) {
-        const double range = log2((double)max((int)threadIdx.x, 2));        // s_j <= j <= m
+    if (!kWarped && threadIdx.x >= kVThreads - 1 - kMaxLive) {               // (the last warps: the first ones read the nodes)
+        const int m = threadIdx.x - (kVThreads - 1 - kMaxLive);
         BinEdges e;
-        e.scale = (float)((double)kBins / range);
+        e.scale = (float)((double)kBins / log2((double)max(m, 2)));          // s_j <= j <= m
         e.inv_scale = 1.f / e.scale;
         e.hi = exp2(1.0 / (double)e.scale) * (1.0 + kEdgeTol);
         e.inv_width = 1.0 / (e.hi - (1.0 - kEdgeTol));
-        sh.bins[threadIdx.x] = e;
+        sh.bins[m] = e;
     }
     const int n_req_nodes = n_hi - n_lo, n_trees = min(b_hi - b_lo, kMaxLive);
     const bool cached = !a.select_mode && n_req_nodes <= kCacheNodes && a.gamma < 256;
@@ -1570,12 +1572,17 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         // the caller gave is read while the dense pass drains: 5.6 us instead of 8.5 (4 beams of 4 nodes, V = 32000),
         // 9 instead of 15 with 84 nodes.  Node i is thread i's.
         int par = -1, tok = -1;
-        float zp_tok = 0.f, zq_tok = 0.f;
+        float zp_tok = 0.f, zq_tok = 0.f, root_p = 0.f, root_q = 0.f;          // (the last two: of tree threadIdx.x)
         if (cached) {
-            if ((int)threadIdx.x < n_trees) nc.root[threadIdx.x] = ld_early(a.beam_node_off + b_lo + threadIdx.x);
+            if ((int)threadIdx.x < n_trees) {
+                nc.root[threadIdx.x] = ld_early(a.beam_node_off + b_lo + threadIdx.x);
+                root_p = ld_early(a.root_logp + b_lo + threadIdx.x);
+                root_q = ld_early(a.root_logq + b_lo + threadIdx.x);
+            }
             const int i = threadIdx.x, n = n_lo + i;
             if (i < n_req) {
                 par = ld_early(a.parent + n);
+                if (a.draft_rank) nc.rank[i] = ld_early(a.draft_rank + n);
                 if (par >= 0) {
                     tok = ld_early(a.token + n);
                     if (par < n_lo || par >= n) { if (writer) report(a.status, DSBD_DEV_BAD_FOREST); tok = -2; }
@@ -1620,11 +1627,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 slp[i] = lp; slq[i] = lq;
             }
             __syncthreads();
-            if (i < b_hi - b_lo && a.beam_node_off[b_lo + i] < n_hi) {
-                const int root = a.beam_node_off[b_lo + i];
-                if (writer && a.parent[root] != -1) report(a.status, DSBD_DEV_BAD_FOREST);
-                slp[root - n_lo] = (double)a.root_logp[b_lo + i];
-                slq[root - n_lo] = (double)a.root_logq[b_lo + i];
+            if (i < n_trees && nc.root[i] >= n_lo && nc.root[i] < n_hi) {
+                const int root = nc.root[i] - n_lo;
+                if (writer && nc.parent[root] != -1) report(a.status, DSBD_DEV_BAD_FOREST);
+                slp[root] = (double)root_p;
+                slq[root] = (double)root_q;
             }
             __syncthreads();
             if (i < n_req) {
@@ -1797,8 +1804,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             for (int i0 = 0; i0 < nA; i0 += 32) {
                 const int i = i0 + lane;
                 if (i >= nA) continue;
-                const int root = a.beam_node_off[b_lo + i];
+                const int root = cached ? nc.root[i] : a.beam_node_off[b_lo + i];
                 sh.A[i] = root;
+                if (cached) nc.live[root - n_lo] = (uint8_t)i;
                 sp_live[i] = cached ? nc.score_p[root - n_lo] : a.score[root];
                 sq_live[i] = cached ? nc.score_q[root - n_lo] : a.score[a.N + root];
             }
@@ -1873,7 +1881,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     // order of (draft_rank, node id), ids being ascending: a draft's place is the number before it
 #pragma unroll 1
                     for (int i0 = 0; i0 < m; i0 += 32)
-                        if (const int i = i0 + lane; i < m) sh.S_parent_idx[i] = a.draft_rank[sh.S[i]];
+                        if (const int i = i0 + lane; i < m) sh.S_parent_idx[i] = cached ? nc.rank[sh.S[i] - n_lo] : a.draft_rank[sh.S[i]];
                     __syncwarp();
 #pragma unroll 1
                     for (int i0 = 0; i0 < m; i0 += 32) {
@@ -1899,8 +1907,10 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     if (i >= m) continue;
                     const int n = sh.S[i] - n_lo, pl = nd_parent(n);
                     int ai = nA;
+                    if (cached) ai = nc.live[pl];
+                    else
 #pragma unroll 1
-                    for (int k = 0; k < nA; ++k) ai = sh.A[k] == n_lo + pl ? k : ai;      // (nodes are unique)
+                        for (int k = 0; k < nA; ++k) ai = sh.A[k] == n_lo + pl ? k : ai;      // (nodes are unique)
                     sh.S_parent_idx[i] = ai;
                     sh.rho[i] = nd_score(0, n) - nd_score(0, pl);
                     sh.lq[i] = nd_score(1, n) - nd_score(1, pl);
@@ -2198,6 +2208,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     const int pos = nA + __popc(mask & ((1u << lane) - 1));
                     if (in && pos < kMaxLive) {
                         sh.A[pos] = n_lo + n;
+                        if (cached) nc.live[n] = (uint8_t)pos;
                         sp_live[pos] = nd_score(0, n);
                         sq_live[pos] = nd_score(1, n);
                     }

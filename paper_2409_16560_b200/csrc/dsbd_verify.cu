@@ -49,7 +49,7 @@ constexpr int kMaxLive = DSBD_MAX_LIVE;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr double kLn2 = 0.6931471805599453;
 
-// The value of lane 0, for one that all lanes of the warp have: the compiler then knows that a branch on it leaves the warp together.
+// By a whole warp (never behind a branch on the lane): the value of lane 0, for one that all lanes have.  The compiler then knows that a branch on it leaves the warp together.
 // Behind a branch on a thread index, a function's argument or a word of memory it does not, and gathers the lanes anew for every
 // shuffle: about 300 cycles each instead of 23, and three times the code (a warp_sum of doubles 1.5 us instead of 0.12).
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(kFull, x, 0); }
@@ -877,13 +877,16 @@ __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, do
         if (lane < n_cta) cluster.map_shared_rank(&sh, lane)->part[n_pass & 1][warp][cta_rank] = v;
     }
     cluster.sync();                                    // (two buffers: who is here has read those of the pass before)
-    long long hi = 0ll, lo = 0ll, q = 0ll;
-#pragma unroll 2
-    for (int c = 0; c < n_cta; ++c) {
-        hi += sh.part[n_pass & 1][0][c];
-        lo += sh.part[n_pass & 1][1][c];
-        q += sh.part[n_pass & 1][2][c];
+    // (warp 0's lanes: only its first thread goes on with the mass)
+    long long sum[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+        sum[x] = lane < n_cta ? sh.part[n_pass & 1][x][lane] : 0ll;
+        if (x && first) continue;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) sum[x] += __shfl_xor_sync(kFull, sum[x], o);
     }
+    const long long hi = sum[0], lo = sum[1], q = sum[2];
     if (first) return (double)hi * (1.0 / kSumUnit);
     const double total = ((double)lo * (1.0 / kSumUnit) + (double)hi) * (1.0 / kSumUnit);
     const double rest = (s - (double)s_hi) * ((double)q * kUnfix);
@@ -891,7 +894,7 @@ __device__ __forceinline__ double exact_pass(const VerifyArgs &a, Shared &sh, do
 }
 
 // One cluster-wide pass over the live rows; every CTA fills its own shared-memory histogram.
-// sh.added (zero before the call) += the mass that the CTA added (p and q), from floating-point sums.
+// sh.warp_part[0]: the mass that each warp added (p and q), from floating-point sums.
 __device__ __forceinline__ void histogram_pass(const VerifyArgs &a, Shared &sh, float binscale, const HistSmem &h,
                                double *sums1, int cta_rank, int n_cta, int halves) {
     // halves = 2: an item is a half tile (when the cluster has a warp for each), with a sum of its own
@@ -937,9 +940,9 @@ __device__ __forceinline__ void histogram_pass(const VerifyArgs &a, Shared &sh, 
         const double tot1 = warp_sum(res1) * kUnfix;
         if (lane == 0) sums1[item] = tot1;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) added += __shfl_xor_sync(kFull, added, o);
-    if (lane == 0 && added) atomicAdd(&sh.added, added);
+    // (below 2^46: two parts of 23 bits)
+    const unsigned lo = __reduce_add_sync(kFull, (unsigned)added & 0x7fffffu), hi = __reduce_add_sync(kFull, (unsigned)(added >> 23));
+    if (lane == 0) sh.warp_part[0][threadIdx.x >> 5] = (long long)hi * 0x800000ll + lo;
 }
 
 // This CTA's histogram into suffix sums (p and q mass of its bins >= k, units of 2^-44), over the words: entry k is 16 bytes, p
@@ -986,6 +989,11 @@ __device__ __forceinline__ void hist_suffix(const HistSmem &h, Shared &sh) {
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
             if (lane == 0) sh.over[x][warp] = s;
         }
+    } else if (warp == kOverSlots / 32) {
+        long long s = lane < kVWarps ? sh.warp_part[0][lane] : 0ll;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        if (lane == 0) sh.added = (unsigned long long)s;
     }
     __syncthreads();
 #pragma unroll
@@ -1291,7 +1299,8 @@ __device__ int build_support(const VerifyArgs &a, const Shared &sh, int model, c
                 if (warp == 0) next[lane] = 0;                       // (last read two rounds ago)
             }
             part_sync<NT>(model);
-            const int mine = counts[min(lane, 2)], at = __popc(__ballot_sync(kFull, mine >= k) & 7u);      // cuts with at least k
+            // the cuts with at least k tiles (below hi: bounds that are not numbers count above every cut)
+            const int mine = counts[min(lane, 2)], at = __popc(__ballot_sync(kFull, lane < 3 && mine >= k && (lane + 1) * step < hi - lo));
             if (at < 3) hi = min(hi, lo + (at + 1) * step);
             lo += at * step;
             if (at == 0) continue;
@@ -1925,7 +1934,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 sh.next_i = sh.count = 0;
                 sh.run_j = sh.chain_pos = 1;
                 sh.bank = l & 1;
-                sh.added = 0ull;
             }
         } else if (warp <= 2) {
             live_weights(sh, warp - 1, warp == 1 ? sp_live : sq_live, node_lse(warp - 1), lane);

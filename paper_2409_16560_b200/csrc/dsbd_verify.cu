@@ -1507,14 +1507,15 @@ __device__ void finish_supports(WarpScratch &ws, bool have_q, int lane) {
 // Drafts behind the first rejection of a layer of known width up to which its residual masses are computed on demand: a pass
 // for that rejection and at most one for each of them, against one histogram, and a pass more where the layer ends in a residual
 // draw behind a second rejection.  A histogram costs about 1.9 passes where a warp has eight tiles of a pass and 2.8 where it
-// has one or two, its merge and chain being as long for few tiles.  Layers of three and four drafts, mean of the benchmark's
+// has one or two, its merge (that there was) and chain being as long for few tiles; without the merge two, three and four are within 2 per
+// cent on seven shapes, but for a call 11 per cent slower with four.  Layers of three and four drafts, mean of the benchmark's
 // distributions with as many accepts and with fewer, against a histogram for every rejection: 64 requests of 128256
 // tokens up to 2 drafts 1.03 and 1.01 times as fast, up to 3 0.97 and 0.93; 160 of 32000 1.05 and 1.03, 1.00 and 0.95; 16
 // of 128256 1.16 and 1.11, 1.20 and 1.14; one of 32000 1.12 and 1.07, 1.14 and 1.09.
 __device__ __forceinline__ int on_demand_left(int n_tiles, int n_warps) { return n_tiles <= 2 * n_warps ? 3 : 2; }
 
 // dynamic shared memory of k_verify: the histogram of a layer as four 32-bit arrays while it is
-// being built, then (over the same bytes) this CTA's slice of the suffix sums of its p and q mass
+// being built, then (over the same bytes) the suffix sums of this CTA's p and q mass
 constexpr size_t kVerifyDynSmem = kHistArrays * sizeof(uint32_t) * kHistWords;
 
 // Two instances, with warped joints and without: neither carries the other's code, whose registers it would spill around

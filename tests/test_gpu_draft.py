@@ -160,3 +160,18 @@ def test_top_k_with_masked_tiles(V, top_k, extra, value):
     ref, gpu, W_r, out_off = _both(rbo, z, s, prm, 1, 16)
     assert int(gpu["status"][0]) == 0
     _compare(ref, gpu, W_r, out_off)
+
+
+@pytest.mark.parametrize("V,top_k", [(16384, 10), (33000, 10), (72000, 64)])
+def test_a_row_with_an_infinite_logit(V, top_k):
+    """Its log-sum-exp is no number and neither are its tiles' bounds, as many as the support has cells or more: the search for the
+    support's cut ends all the same, and the other request draws what it draws alone."""
+    rng = np.random.default_rng(V)
+    rbo, z, s = _problem(rng, [2, 2], V)
+    prm = dict(V=V, temperature=1.0, seed=3, step=5, top_k=top_k, top_p=0.9)
+    ok, W_r, out_off = _both(rbo, z, s, prm, 1, 4)[1:]
+    z[0, 1] = np.inf
+    gpu = _both(rbo, z, s, prm, 1, 4)[1]
+    for k in ("out_parent", "out_token"):
+        assert np.array_equal(gpu[k][out_off[1]:], ok[k][out_off[1]:])
+    assert gpu["req_error"][1] == 0

@@ -538,6 +538,25 @@ def test_every_cluster_size(V):
     check_exempt(exempt, decisions)
 
 
+@pytest.mark.parametrize("V,beams", [(524288, 2), (524289, 2), (600001, 3), (1050000, 1), (20000, 13), (4000, 64)])
+def test_draws_over_pieces_and_shares(V, beams):
+    """A draw from p_beam searches its row's tile masses 512 at a time: 512, 513, 586 and 1026 tiles.  A residual draw searches 256
+    shares of the layer's tiles first: shares of 4, 5 and 7 tiles, of one (13 x 20 = 260 tiles: two), of one (64 x 4)."""
+    rng = np.random.default_rng(V + beams)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=1, V=V, gamma=2 if V < 100000 else 1, max_w=beams, min_w=beams)
+    zp = (zp + rng.normal(0, 2.0, zp.shape)).astype(np.float32)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = 0
+    for step in range(4):
+        prm.update(step=step, thresh=0.3, W_min=min(2, beams), W_min_r=None)
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+    check_exempt(exempt, decisions)
+
+
 @pytest.mark.parametrize("beams,V,top_k,top_p", [(64, 72000, 10, 0.8), (64, 72000, 64, 0.9), (36, 121900, 1, 1.0)])
 def test_warped_layers_with_more_tiles_than_the_bound_cache(beams, V, top_k, top_p):
     """64 x 71 = 4544 tile bounds, more than are kept in shared memory (4368), and 36 x 120 = 4320, just fewer."""

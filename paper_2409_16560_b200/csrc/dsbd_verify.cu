@@ -33,6 +33,8 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <atomic>
+
 #include "dsbd_common.cuh"
 
 namespace cg = cooperative_groups;
@@ -2351,29 +2353,53 @@ int check_params(const dsbd_verify_params_t *p) {
     return DSBD_OK;
 }
 
-// Cluster size: as many CTAs per request as its tile count can use, but few enough that all
-// requests are resident at once (two CTAs per SM fit).  16 from six tiles a CTA on (half a tile a warp instead of one): requests of four
+// Clusters of 1 << log2 CTAs of k_verify that the current device holds at once.  Clusters stay inside a GPC, and GPCs have different numbers
+// of SMs, so this is less than the CTAs that fit over the cluster's size; asked once per device (it takes some 10 us).
+constexpr int kMaxDevices = 64;
+int resident_clusters(void (*kernel)(VerifyArgs), bool warped, int log2) {
+    static std::atomic<int> known[kMaxDevices][2][5];       // 0: not asked yet
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    std::atomic<int> &slot = known[dev][warped][log2];
+    int n = slot.load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << log2);
+    cfg.blockDim = dim3(kVThreads);
+    cfg.dynamicSmemBytes = kVerifyDynSmem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << log2;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (n > 0) slot.store(n, std::memory_order_relaxed);
+    return n;
+}
+
+// Cluster size (its logarithm): as many CTAs per request as its tile count can use, but few enough that all requests are resident at
+// once.  16 from six tiles a CTA on (half a tile a warp instead of one): requests of four
 // live rows, 128 tiles 41.9 us instead of 44.3 with 8 CTAs (one request), 252 tiles 43.5 for 47.9; eight requests 56.7 for 59.6 and
-// 66.4 for 74.2.  64 tiles: 41.3 for 40.5, so 8 stay.
-int cluster_size_for(int tiles, int R) {
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int cs = 1;
-    if (tiles >= 96) cs = 16;
-    else if (tiles >= 64) cs = 8;
-    else if (tiles >= 32) cs = 4;
-    else if (tiles >= 16) cs = 2;
-    while (cs > 1 && (long long)R * cs > 2ll * sms) cs >>= 1;
-    return cs;
+// 66.4 for 74.2.  64 tiles: 41.3 for 40.5, so 8 stay.  Clusters that do not fit wait for a whole request: 18 requests of 128
+// tiles 80 us with 16 CTAs, of which 16 clusters fit, 67 with 8; 14 requests 65 and 69.
+int cluster_log2_for(void (*kernel)(VerifyArgs), bool warped, int tiles, int R) {
+    int log2 = tiles >= 96 ? 4 : tiles >= 64 ? 3 : tiles >= 32 ? 2 : tiles >= 16 ? 1 : 0;
+    while (log2 > 0 && R > resident_clusters(kernel, warped, log2)) --log2;
+    return log2;
 }
 
 int launch_verify(const VerifyArgs &args, int R, int tiles, cudaStream_t stream) {
-    const auto kernel = args.top_k > 0 ? k_verify<true> : k_verify<false>;
-    const int cs = cluster_size_for(tiles, R);
-    if (cs > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-        return DSBD_ERR_CUDA;
+    const bool warped = args.top_k > 0;
+    const auto kernel = warped ? k_verify<true> : k_verify<false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess)
         return DSBD_ERR_CUDA;
+    if (tiles >= 96 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        return DSBD_ERR_CUDA;
+    const int cs = 1 << cluster_log2_for(kernel, warped, tiles, R);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(R * cs));
     cfg.blockDim = dim3(kVThreads);
@@ -2690,7 +2716,6 @@ extern "C" int dsbd_draft_layer(int32_t R, int32_t n_beams, const int32_t *req_b
 static __device__ __align__(256) unsigned char g_static_scratch[DSBD_STATIC_SCRATCH_BYTES];
 
 namespace {
-constexpr int kMaxDevices = 64;
 unsigned char *g_static_scratch_ptr[kMaxDevices];   // device address of the array, per device
 
 // The array's name is only a host-side handle; the device address a kernel can use has to be

@@ -538,6 +538,17 @@ def test_every_cluster_size(V):
     check_exempt(exempt, decisions)
 
 
+@pytest.mark.parametrize("R", [9, 14, 18, 36, 80])
+def test_as_many_clusters_as_the_device_holds(R):
+    """6 rows of 16 tiles: clusters of 16 CTAs as long as all requests' fit at once, then of 8, 4 and 2."""
+    rng = np.random.default_rng(R)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=R, V=16384, gamma=1, max_w=6, min_w=6)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    gpu, status = run_gpu_verify(forest, prm, *dev)
+    assert status == 0
+    check_exempt(*compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest))
+
+
 @pytest.mark.parametrize("V,beams", [(524288, 2), (524289, 2), (600001, 3), (1050000, 1), (20000, 13), (4000, 64)])
 def test_draws_over_pieces_and_shares(V, beams):
     """A draw from p_beam searches its row's tile masses 512 at a time: 512, 513, 586 and 1026 tiles.  A residual draw searches 256

@@ -2385,7 +2385,7 @@ int resident_clusters(void (*kernel)(VerifyArgs), bool warped, int log2) {
 // once.  16 from six tiles a CTA on (half a tile a warp instead of one): requests of four
 // live rows, 128 tiles 41.9 us instead of 44.3 with 8 CTAs (one request), 252 tiles 43.5 for 47.9; eight requests 56.7 for 59.6 and
 // 66.4 for 74.2.  64 tiles: 41.3 for 40.5, so 8 stay.  Clusters that do not fit wait for a whole request: 18 requests of 128
-// tiles 80 us with 16 CTAs, of which 16 clusters fit, 67 with 8; 14 requests 65 and 69.
+// tiles 80 us with 16 CTAs, of which 14 clusters fit, 67 with 8; 12 requests 65 and 68.
 int cluster_log2_for(void (*kernel)(VerifyArgs), bool warped, int tiles, int R) {
     int log2 = tiles >= 96 ? 4 : tiles >= 64 ? 3 : tiles >= 32 ? 2 : tiles >= 16 ? 1 : 0;
     while (log2 > 0 && R > resident_clusters(kernel, warped, log2)) --log2;

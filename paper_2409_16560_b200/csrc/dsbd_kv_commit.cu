@@ -73,37 +73,55 @@ struct CommitArgs {
     int32_t *status;
 };
 
-// exclusive scan of v[0..n) in place by one CTA; returns the total in every thread
+// Sum of the totals of the warps before this one, and of all warps, by shuffles of the totals (a walk over 32 of them is 32 loads one after
+// the other, 1000 cycles).  By whole warps.
 template <typename T>
-__device__ T block_exclusive_scan(T *v, int n, T *warp_tot /*[32]*/) {
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int lo = min((int)threadIdx.x * per, n), hi = min(lo + per, n);
-    T local = 0;
-    for (int i = lo; i < hi; ++i) local += v[i];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T incl = local;
+__device__ __forceinline__ T warps_before(const T *warp_tot, T *total) {
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    const T own = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : T(0);
+    T incl = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const T t = __shfl_up_sync(kFull, incl, o);
         if (lane >= o) incl += t;
     }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    T base = 0, total = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        if (w < warp) base += warp_tot[w];
-        total += warp_tot[w];
+    *total = __shfl_sync(kFull, incl, 31);
+    return __shfl_sync(kFull, incl - own, warp);
+}
+
+// exclusive scans of v[0][0..n) .. v[K-1][0..n) in place by one CTA; the totals in every thread
+template <typename T, int K>
+__device__ __forceinline__ void block_exclusive_scan(T *const (&v)[K], int n, T (*warp_tot)[32] /*[K]*/, T (&total)[K]) {
+    const int per = (n + blockDim.x - 1) / blockDim.x;
+    const int lo = min((int)threadIdx.x * per, n), hi = min(lo + per, n);
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    T before[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        T local = 0;
+        for (int i = lo; i < hi; ++i) local += v[k][i];
+        T incl = local;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const T t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) warp_tot[k][warp] = incl;
+        before[k] = incl - local;
     }
-    T run = base + incl - local;
-    for (int i = lo; i < hi; ++i) { const T x = v[i]; v[i] = run; run += x; }
     __syncthreads();
-    return total;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        T run = before[k] + warps_before(warp_tot[k], &total[k]);
+        for (int i = lo; i < hi; ++i) { const T x = v[k][i]; v[k][i] = run; run += x; }
+    }
+    __syncthreads();
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
 k_commit_plan(CommitArgs a) {
-    __shared__ int64_t tot64[32];
-    __shared__ int32_t tot32[32];
+    __shared__ int64_t tot64[3][32];
+    __shared__ int32_t tot32[1][32];
     __shared__ int bad;
     if (threadIdx.x == 0) bad = 0;
     __syncthreads();
@@ -153,7 +171,10 @@ k_commit_plan(CommitArgs a) {
         a.req_best[r] = best;
     }
     __syncthreads();
-    const int n_beams = block_exclusive_scan<int32_t>(a.req_count, a.R, tot32);
+    int32_t *const counts[1] = {a.req_count};
+    int32_t sums[1];
+    block_exclusive_scan<int32_t, 1>(counts, a.R, tot32, sums);
+    const int n_beams = sums[0];
     if (n_beams > a.n_slots) { if (threadIdx.x == 0) bad = DSBD_DEV_CAPACITY; }
     __syncthreads();
     const bool fits = !bad;
@@ -194,10 +215,17 @@ k_commit_plan(CommitArgs a) {
         if (a.paged) a.new_page_off[j] = 0;
     }
     __syncthreads();
-    const int64_t total = block_exclusive_scan<int64_t>(a.new_prefix_off, a.n_slots, tot64);
-    const int64_t chunks = block_exclusive_scan<int64_t>(a.chunk_off, a.n_slots, tot64);
-    int64_t table_len = 0;
-    if (a.paged) table_len = block_exclusive_scan<int64_t>(a.new_page_off, a.n_slots, tot64);
+    int64_t offs[3] = {0, 0, 0};
+    if (a.paged) {
+        int64_t *const v[3] = {a.new_prefix_off, a.chunk_off, a.new_page_off};
+        block_exclusive_scan<int64_t, 3>(v, a.n_slots, tot64, offs);
+    } else {
+        int64_t *const v[2] = {a.new_prefix_off, a.chunk_off};
+        int64_t two[2];
+        block_exclusive_scan<int64_t, 2>(v, a.n_slots, tot64, two);
+        offs[0] = two[0]; offs[1] = two[1];
+    }
+    const int64_t total = offs[0], chunks = offs[1], table_len = offs[2];
     if (threadIdx.x == 0) {
         a.new_prefix_off[a.n_slots] = total;
         a.chunk_off[a.n_slots] = chunks;
@@ -352,7 +380,7 @@ k_commit_free(CommitArgs a) {
             if (pg >= 0 && pg < n) atomicAnd(&bits[pg >> 5], ~(1u << (pg & 31)));
         }
         __syncthreads();
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
         for (int base = 0; base < words; base += kPlanThreads) {
             const int w = base + threadIdx.x;
             uint32_t m = w < words ? bits[w] : 0u;
@@ -365,11 +393,8 @@ k_commit_free(CommitArgs a) {
             }
             if (lane == 31) warp_tot[warp] = incl;
             __syncthreads();
-            int before = carry, tile_total = 0;
-            for (int x = 0; x < kPlanThreads / 32; ++x) {
-                if (x < warp) before += warp_tot[x];
-                tile_total += warp_tot[x];
-            }
+            int tile_total;
+            const int before = carry + warps_before(warp_tot, &tile_total);
             int pos = before + incl - cnt;
             while (m) {
                 const int b = __ffs(m) - 1;
@@ -393,7 +418,7 @@ k_commit_free(CommitArgs a) {
         if (pg >= 0 && pg < n) a.used[pg] = 0;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
     for (int base = 0; base < n_pad; base += kPlanThreads * 16) {
         const int i0 = base + threadIdx.x * 16;
         int4 f[4];
@@ -411,11 +436,8 @@ k_commit_free(CommitArgs a) {
         }
         if (lane == 31) warp_tot[warp] = incl;
         __syncthreads();
-        int before = carry, tile_total = 0;
-        for (int w = 0; w < kPlanThreads / 32; ++w) {
-            if (w < warp) before += warp_tot[w];
-            tile_total += warp_tot[w];
-        }
+        int tile_total;
+        const int before = carry + warps_before(warp_tot, &tile_total);
         int pos = before + incl - cnt;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {

@@ -214,7 +214,7 @@ __global__ void k_row_finish(const TileStat *__restrict__ stats, int T, int N, i
 // ---------------------------------------------------------------------------------------
 struct VerifyArgs {
     // forest
-    int R, N, gamma;
+    int R, B, N, gamma;
     const int32_t *req_beam_off, *beam_node_off, *parent, *token, *draft_rank;
     // parameters
     int V, T;
@@ -1544,8 +1544,21 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     // pass ahead in the stream.  That pass lets this kernel start only when each of its blocks has waited for all earlier work,
     // so what earlier kernels and the caller left lies in L2 and may be read here, from there (ld_early: the pass's wait says
     // nothing about this SM's L1); the tile statistics only after the wait.
-    const int b_lo = uniform(ld_early(a.req_beam_off + r)), b_hi = uniform(ld_early(a.req_beam_off + r + 1));
-    const int n_lo = uniform(ld_early(a.beam_node_off + b_lo)), n_hi = uniform(ld_early(a.beam_node_off + b_hi));
+    int b_lo = uniform(ld_early(a.req_beam_off + r)), b_hi = uniform(ld_early(a.req_beam_off + r + 1));
+    // Every tree has nodes and every offset lies inside the forest (then so does every root): what is below uses them as indexes, and a
+    // root that two trees share would get either's score, another one in every CTA.  A request whose offsets say otherwise is reported
+    // and taken as empty.  All warps look, so that nobody waits for another's answer: a lane's loads come back with n_lo.
+    bool bad_off = b_lo < 0 || b_hi > a.B || b_lo > b_hi;
+    if (bad_off) b_lo = b_hi = 0;
+    int n_lo = ld_early(a.beam_node_off + b_lo), n_hi = ld_early(a.beam_node_off + b_hi);
+#pragma unroll 1
+    for (int t0 = b_lo; t0 < b_hi; t0 += 32) {
+        const int t = min(t0 + lane, b_hi - 1);
+        bad_off |= ld_early(a.beam_node_off + t) >= ld_early(a.beam_node_off + t + 1);
+    }
+    n_lo = uniform(n_lo); n_hi = uniform(n_hi);
+    bad_off = __any_sync(kFull, bad_off || n_lo < 0 || n_hi > a.N || n_lo > n_hi);
+    if (bad_off) b_lo = b_hi = n_lo = n_hi = 0;
     int W_min = a.W_min_r ? ld_early(a.W_min_r + r) : a.W_min;
     int W_max = a.W_max_r ? ld_early(a.W_max_r + r) : a.W_max;
     int W_nom = a.W_nom_r ? ld_early(a.W_nom_r + r) : a.W_nom;
@@ -1843,7 +1856,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         for (int n0 = 0; n0 < n_req_nodes && st_ok; n0 += kVThreads)
             if (const int n = n0 + threadIdx.x; n < n_req_nodes) st[n] = is_root(n) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     __syncthreads();
-    if (!a.select_mode && !st_ok && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
+    if (!a.select_mode && (!st_ok || bad_off) && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
     if (bad_widths && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_PARAM;
     __syncthreads();
     // node data by local index, from the cache when there is one
@@ -2487,7 +2500,7 @@ extern "C" int dsbd_verify_step(const dsbd_forest_t *f, const dsbd_verify_params
     if (cudaGetLastError() != cudaSuccess) return DSBD_ERR_CUDA;
 
     VerifyArgs a = {};
-    a.R = f->R; a.N = f->N; a.gamma = f->max_depth;
+    a.R = f->R; a.B = f->B; a.N = f->N; a.gamma = f->max_depth;
     a.req_beam_off = f->req_beam_off; a.beam_node_off = f->beam_node_off;
     a.parent = f->parent; a.token = f->token; a.draft_rank = f->draft_rank;
     a.V = p->V; a.T = L.T; a.k2 = k2; a.inv_tau = inv_tau; a.thresh = (double)p->thresh;
@@ -2806,7 +2819,7 @@ extern "C" int dsbd_select_width(const dsbd_forest_t *f, const dsbd_verify_param
     if (cudaGetLastError() != cudaSuccess) return DSBD_ERR_CUDA;
 
     VerifyArgs a = {};
-    a.R = f->R; a.N = f->N; a.gamma = f->max_depth;
+    a.R = f->R; a.B = f->B; a.N = f->N; a.gamma = f->max_depth;
     a.req_beam_off = f->req_beam_off; a.beam_node_off = f->beam_node_off;
     a.parent = f->parent; a.token = f->token; a.draft_rank = f->draft_rank;
     a.V = p->V; a.T = L.T; a.k2 = k2; a.inv_tau = inv_tau; a.thresh = (double)p->thresh;

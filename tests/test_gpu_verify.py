@@ -851,3 +851,64 @@ def test_draft_ranks_up_to_the_type_s_largest():
         exempt += e
         decisions += d
     check_exempt(exempt, decisions)
+
+
+def _tampered(depth, beams, request, **arrays):
+    """Three requests of `beams` chains of `depth` drafts; the call on the forest as it is, and on one whose device arrays differ
+    (name = function of the array and of the first tree of `request`).  Returns the forest and both outputs with their status."""
+    rng = np.random.default_rng(depth * beams)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=3, V=600, gamma=depth, max_w=beams, min_w=beams)
+    prm.update(W_min=1, W_min_r=None, thresh=0.3)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    res = []
+    for change in (False, True):
+        f = dsbd.Forest(forest, "cuda")
+        if change:
+            for name, fn in arrays.items():
+                x = forest[name].copy()
+                fn(x, int(forest["req_beam_off"][request]))
+                f.dev[name] = torch.as_tensor(x).cuda()
+        out = dsbd.alloc_verify_out(f, oracle.default_out_off(forest, prm), "cuda")
+        status = dsbd.verify_step(f, dict(prm), *dev, out)
+        res.append(({k: v.cpu().numpy() for k, v in out.items()}, int(status.item())))
+    return forest, prm, res
+
+
+# nodes of a request: kept in shared memory (up to 256), scores by the writer's threads (up to 1024), by its trees' threads
+REQUEST_SIZES = [(3, 6), (3, 64), (9, 30), (17, 64)]
+
+
+def _others_unchanged(forest, prm, request, good, bad):
+    out_off, bno, rbo = oracle.default_out_off(forest, prm), forest["beam_node_off"], forest["req_beam_off"]
+    for r in set(range(forest["R"])) - {request}:
+        w = good["out_width"][r]
+        assert bad["out_width"][r] == w and bad["req_error"][r] == 0 and bad["l_last"][r] == good["l_last"][r]
+        s, n = slice(out_off[r], out_off[r] + w), slice(bno[rbo[r]], bno[rbo[r + 1]])
+        for k in ("out_parent", "out_node", "out_token", "out_root_beam", "out_source", "out_logp"):
+            assert np.array_equal(good[k][s], bad[k][s]), (r, k)
+        assert np.array_equal(good["node_status"][n], bad["node_status"][n])
+
+
+@pytest.mark.parametrize("depth,beams", REQUEST_SIZES)
+@pytest.mark.parametrize("tree,value", [(2, "empty"), (-1, "empty"), (1, 1 << 30), (1, -5), (-1, 1 << 30), (1, "next request")])
+def test_tree_offsets_that_contradict_the_forest(depth, beams, tree, value):
+    """A tree without nodes (inside, or the last one), a root far outside the forest, before it or in the next request: reported, the
+    request is not verified, and the others are what they are without it."""
+    def change(off, b0):
+        t = b0 + (tree if tree > 0 else beams + tree)
+        off[t] = {"empty": off[t + 1], "next request": off[b0 + beams] + 2}.get(value, value)
+    forest, prm, ((good, ok), (bad, status)) = _tampered(depth, beams, 1, beam_node_off=change)
+    assert ok == 0 and status == 4 and bad["req_error"].tolist() == [0, 4, 0]         # DSBD_DEV_BAD_FOREST
+    assert bad["out_width"][1] == 0
+    _others_unchanged(forest, prm, 1, good, bad)
+
+
+@pytest.mark.parametrize("first,last", [(-1, None), (None, 1 << 30), (None, 0)])
+def test_request_offsets_that_contradict_the_forest(first, last):
+    """Requests whose trees lie outside the forest or end before they begin."""
+    def change(off, b0):
+        off[0 if first is not None else 3] = first if first is not None else last
+    r = 0 if first is not None else 2
+    forest, prm, ((good, ok), (bad, status)) = _tampered(3, 6, r, req_beam_off=change)
+    assert ok == 0 and status == 4 and bad["req_error"][r] == 4 and bad["out_width"][r] == 0
+    _others_unchanged(forest, prm, r, good, bad)

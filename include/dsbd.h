@@ -47,7 +47,8 @@ enum {
     DSBD_DEV_BAD_FOREST = 4,     /* an index that contradicts the forest: parent outside its
                                     tree, beam outside its request, too many live beams; to
                                     dsbd_verify_step also a tree without nodes or an offset
-                                    outside the forest (the request is then not verified)    */
+                                    outside the forest (the request is then not verified), or
+                                    a second root in a tree (the node stays unreached)       */
     DSBD_DEV_TIMEOUT = 5,        /* a bounded wait gave up                                   */
     DSBD_DEV_BAD_PARAM = 6       /* a per-request width (W_min_r, W_max_r, W_nom_r) below 1, or
                                     W_max_r below W_min_r                                    */

@@ -1669,6 +1669,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
 #pragma unroll 1
                 while (tree + 1 < n_trees && nc.root[tree + 1] <= n_lo + i) ++tree;
                 nc.tree[i] = (uint8_t)tree;
+                if (nc.parent[i] == -1 && nc.root[tree] != n_lo + i) {
+                    // a second root inside a tree (paths end there whichever negative value they see)
+                    nc.parent[i] = -2;
+                    if (writer) report(a.status, DSBD_DEV_BAD_FOREST);
+                }
                 if (writer) {
                     a.score_w[n_lo + i] = sp;
                     a.score_w[a.N + n_lo + i] = sq;
@@ -1788,7 +1793,18 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     if (kWarped && !writer) return;
 
     // ---- set-up ----
-    auto is_root = [&](int i) { return cached ? nc.parent[i] == -1 : a.parent[n_lo + i] < 0; };
+    // The roots are accepted: the first node of each tree.  Another node without a parent would be a live parent that has no place among the
+    // input beams; it is reported and stays unreached.
+    auto is_root = [&](int i) {
+        if (cached) return nc.parent[i] == -1;
+        if (a.parent[n_lo + i] >= 0) return false;
+        int lo = b_lo, hi = b_hi;                            // first tree that starts at the node or behind it
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (a.beam_node_off[mid] < n_lo + i) lo = mid + 1; else hi = mid;
+        }
+        return a.beam_node_off[lo] == n_lo + i;
+    };
     if (warp == 0) {
         if (lane == 0) {
             sh.err = 0; sh.n_out = 0; sh.n_draw = 0;
@@ -1852,7 +1868,11 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         if (!a.select_mode && writer)
 #pragma unroll 1
             for (int n0 = n_lo; n0 < n_hi; n0 += 32)
-                if (const int n = n0 + lane; n < n_hi) a.out.node_status[n] = is_root(n - n_lo) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+                if (const int n = n0 + lane; n < n_hi) {
+                    const bool root = is_root(n - n_lo);
+                    a.out.node_status[n] = root ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
+                    if (!cached && !root && a.parent[n] < 0) report(a.status, DSBD_DEV_BAD_FOREST);
+                }
     }
     // Every CTA of the cluster takes identical decisions from identical data, so each keeps its
     // own copy of the node statuses and only rank 0 writes results.

@@ -912,3 +912,21 @@ def test_request_offsets_that_contradict_the_forest(first, last):
     forest, prm, ((good, ok), (bad, status)) = _tampered(3, 6, r, req_beam_off=change)
     assert ok == 0 and status == 4 and bad["req_error"][r] == 4 and bad["out_width"][r] == 0
     _others_unchanged(forest, prm, r, good, bad)
+
+
+@pytest.mark.parametrize("depth,beams", REQUEST_SIZES)
+def test_a_second_root_inside_a_tree(depth, beams):
+    """A node behind its tree's first one that names no parent: reported, it stays unreached and no draft behind it is tested; the other
+    requests are what they are without it."""
+    n = (beams + 1) * (depth + 1) + 1                    # request 1, second tree, layer 1
+
+    def change(parent, b0):
+        parent[n] = -1
+    forest, prm, ((good, ok), (bad, status)) = _tampered(depth, beams, 1, parent=change)
+    bno = forest["beam_node_off"]
+    assert n == bno[forest["req_beam_off"][1] + 1] + 1 and forest["parent"][n + 1] == n
+    assert ok == 0 and status == 4 and bad["req_error"].tolist() == [0, 0, 0]
+    assert bad["node_status"][n] == 0 and bad["node_status"][n + 1] in (0, 4)        # unreached, pruned
+    assert not np.any(np.isin(bad["node_status"][n:bno[forest["req_beam_off"][1] + 2]], (1, 2, 3)))
+    assert bad["out_width"][1] >= 1
+    _others_unchanged(forest, prm, 1, good, bad)

@@ -107,6 +107,11 @@ constexpr uint32_t kWaitTries = 500000;
 // What a run left for the merge.  tail: its last unit (of the tree n_lo .. n_lo + n_tree) starts here and goes on in the next run;
 // head_ends: the part of a unit that the run began with is the last one of that unit.
 struct CutRec { int tail, head_ends, g, rb, n_lo, n_tree, pad0, pad1; };
+// Whether a record names a unit of the forest.  One that nobody wrote (a CTA that left before) may hold anything, so no sum is made of it.
+__host__ __device__ inline bool names_unit(const CutRec &rec, int N, int Hkv) {
+    return (unsigned)rec.n_tree <= (unsigned)kMaxTree && rec.n_lo >= 0 && rec.n_lo <= N - rec.n_tree && (unsigned)rec.g < (unsigned)Hkv &&
+           (unsigned)rec.rb <= (unsigned)kMaxTree;
+}
 
 struct TcArgs {
     int B, N, Hq, Hkv, group;
@@ -969,9 +974,7 @@ k_attn_merge(TcArgs a) {
     int last = min(i0 + 1, end);                             // the runs that hold the other parts
     int ends = a.recs[last].head_ends;
     if (!rec.tail) return;
-    // (no unit of this forest: a CTA that left before it wrote its records)
-    if (rec.n_lo < 0 || (unsigned)rec.n_tree > (unsigned)kMaxTree || rec.n_lo + rec.n_tree > a.N || (unsigned)rec.g >= (unsigned)a.Hkv ||
-        (unsigned)rec.rb > (unsigned)kMaxTree) return;
+    if (!names_unit(rec, a.N, a.Hkv)) return;
     while (last < end && !ends) ends = a.recs[++last].head_ends;
     const int n_lo = rec.n_lo;
     const int rows = min(a.block_rows, rec.n_tree * a.group - rec.rb * a.block_rows);
@@ -1170,3 +1173,13 @@ int launch_attention_tr(const dsbd_forest_t *f, const dsbd_attn_desc_t *d, const
 }
 
 }  // namespace dsbd
+
+#ifdef DSBD_TEST_WAIT_TIMEOUT
+// The merge's check of a record, on the host (records are 8 words; see CutRec).
+extern "C" int dsbd_test_names_unit(const int32_t *rec, int32_t N, int32_t Hkv) {
+    CutRec r;
+    static_assert(sizeof(r) == 8 * sizeof(int32_t), "a record is 8 words");
+    std::copy(rec, rec + 8, reinterpret_cast<int32_t *>(&r));
+    return names_unit(r, N, Hkv);
+}
+#endif

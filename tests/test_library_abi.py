@@ -86,3 +86,17 @@ def test_the_current_stream_without_torch_s_raw_calls(monkeypatch):
     for reader in (binding._stream_reader(types.SimpleNamespace()), binding._stream_reader(raw)):
         assert reader(types.SimpleNamespace(cuda_stream=5)) == 5
     assert binding._stream_reader(raw)(None) == 72
+
+
+def test_a_merge_record_that_nobody_wrote_names_no_unit():
+    """Records of cut attention units: tail, head_ends, g, rb, n_lo, n_tree.  N = 1000 nodes, 8 heads."""
+    from paper_2409_16560_b200 import build
+    lib = ctypes.CDLL(build.build_wait_test())
+    ok = lambda *rec: bool(lib.dsbd_test_names_unit((ctypes.c_int32 * 8)(*rec), 1000, 8))
+    big = 2 ** 31 - 1
+    for n_lo, n_tree in [(0, 1), (999, 1), (936, 64), (0, 64), (1000, 0)]:
+        assert ok(1, 0, 7, 2, n_lo, n_tree)
+    for n_lo, n_tree in [(big, 1), (big, 64), (big - 63, 64), (1000, 1), (937, 64), (-1, 1), (-big - 1, 64), (0, 65), (0, -1),
+                         (0, -big - 1), (0x11111111, 0x11111111), (big, -1)]:
+        assert not ok(1, 0, 7, 2, n_lo, n_tree), (n_lo, n_tree)
+    assert not ok(1, 0, 8, 2, 0, 1) and not ok(1, 0, -1, 2, 0, 1) and not ok(1, 0, 7, 65, 0, 1) and not ok(1, 0, 7, -1, 0, 1)

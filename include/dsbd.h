@@ -260,6 +260,10 @@ int dsbd_verify_step(const dsbd_forest_t *forest, const dsbd_verify_params_t *pa
 
 size_t dsbd_verify_workspace(const dsbd_forest_t *forest, const dsbd_verify_params_t *params);
 
+/* CTAs that dsbd_verify_step gives to a request of this shape on the current device, 0 for invalid arguments; *resident (host, may
+ * be NULL): how many such clusters the device holds at once.  For launch accounting; host-only. */
+int dsbd_verify_cluster_ctas(const dsbd_forest_t *forest, const dsbd_verify_params_t *params, int32_t *resident);
+
 /* Step 1 of dsbd_verify_step on its own: the large and the small model's next-token
  * distribution of every node (Overview: "predict the distribution for the next token of each
  * node in parallel"), returned as the log-sum-exp of each tempered logits row,

@@ -22,7 +22,7 @@ MAX_LIVE = 64
 REQ_STATS = 8                # DSBD_REQ_STATS: counters per request in req_stats
 
 EXPORTS = ["dsbd_forest_attention", "dsbd_forest_attention_workspace", "dsbd_forest_attention_launches", "dsbd_verify_step",
-           "dsbd_verify_workspace", "dsbd_select_width", "dsbd_node_stats", "dsbd_node_stats_static",
+           "dsbd_verify_workspace", "dsbd_verify_cluster_ctas", "dsbd_select_width", "dsbd_node_stats", "dsbd_node_stats_static",
            "dsbd_kv_commit", "dsbd_kv_commit_workspace", "dsbd_draft_layer", "dsbd_draft_workspace",
            "dsbd_forest_attention_paged", "dsbd_forest_attention_paged_workspace", "dsbd_kv_commit_paged", "dsbd_kv_commit_paged_workspace",
            "dsbd_forest_build",
@@ -96,6 +96,8 @@ def _declare(lib):
     lib.dsbd_forest_attention_launches.argtypes = [_vp, _vp]
     lib.dsbd_verify_workspace.restype = C.c_size_t
     lib.dsbd_verify_workspace.argtypes = [_vp, _vp]
+    lib.dsbd_verify_cluster_ctas.restype = C.c_int
+    lib.dsbd_verify_cluster_ctas.argtypes = [_vp, _vp, _vp]
     lib.dsbd_forest_attention.restype = C.c_int
     lib.dsbd_forest_attention.argtypes = [_vp] * 10 + [C.c_size_t, _vp, _vp]
     lib.dsbd_verify_step.restype = C.c_int
@@ -503,6 +505,16 @@ def verify_workspace(forest, params):
     f = forest.struct()
     p = _params(params, keep)
     return int(load().dsbd_verify_workspace(C.addressof(f), C.addressof(p)))
+
+
+def verify_cluster_ctas(forest, params):
+    """dsbd_verify_cluster_ctas: CTAs per request, and how many such clusters the device holds at once."""
+    keep = []
+    f = forest.struct()
+    p = _params(params, keep)
+    resident = C.c_int32(0)
+    ctas = int(load().dsbd_verify_cluster_ctas(C.addressof(f), C.addressof(p), C.addressof(resident)))
+    return ctas, resident.value
 
 
 def default_out_off(arrays, params):

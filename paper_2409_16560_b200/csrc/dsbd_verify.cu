@@ -2393,15 +2393,17 @@ int check_params(const dsbd_verify_params_t *p) {
 }
 
 // Clusters of 1 << log2 CTAs of k_verify that the current device holds at once.  Clusters stay inside a GPC, and GPCs have different numbers
-// of SMs, so this is less than the CTAs that fit over the cluster's size; asked once per device (it takes some 10 us).
+// of SMs, so this is less than the CTAs that fit over the cluster's size; asked once per device (it takes some 10 us).  Where the
+// device has no answer: the CTAs that fit (two per SM) over the cluster's size, none of the 16 that not every device takes, and asked
+// again by the next call.
 constexpr int kMaxDevices = 64;
 int resident_clusters(void (*kernel)(VerifyArgs), bool warped, int log2) {
-    static std::atomic<int> known[kMaxDevices][2][5];       // 0: not asked yet
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-    std::atomic<int> &slot = known[dev][warped][log2];
-    int n = slot.load(std::memory_order_relaxed);
-    if (n > 0) return n;
+    static std::atomic<int> known[kMaxDevices][2][5];       // the answer plus one; 0: not asked yet
+    int dev = -1, sms = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    std::atomic<int> *slot = dev >= 0 && dev < kMaxDevices ? &known[dev][warped][log2] : nullptr;
+    int n = slot ? slot->load(std::memory_order_relaxed) - 1 : -1;
+    if (n >= 0) return n;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1u << log2);
     cfg.blockDim = dim3(kVThreads);
@@ -2412,12 +2414,13 @@ int resident_clusters(void (*kernel)(VerifyArgs), bool warped, int log2) {
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
+    if (dev >= 0 && cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 0) {
+        if (slot) slot->store(n + 1, std::memory_order_relaxed);
+        return n;
     }
-    if (n > 0) slot.store(n, std::memory_order_relaxed);
-    return n;
+    if (dev >= 0) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaGetLastError();
+    return log2 > 3 ? 0 : 2 * sms >> log2;
 }
 
 // Cluster size (its logarithm): as many CTAs per request as its tile count can use, but few enough that all requests are resident at
@@ -2425,8 +2428,13 @@ int resident_clusters(void (*kernel)(VerifyArgs), bool warped, int log2) {
 // live rows, 128 tiles 41.9 us instead of 44.3 with 8 CTAs (one request), 252 tiles 43.5 for 47.9; eight requests 56.7 for 59.6 and
 // 66.4 for 74.2.  64 tiles: 41.3 for 40.5, so 8 stay.  Clusters that do not fit wait for a whole request: 18 requests of 128
 // tiles 80 us with 16 CTAs, of which 14 clusters fit, 67 with 8; 12 requests 65 and 68.
+// Where the kernel may not have 16, 8.
 int cluster_log2_for(void (*kernel)(VerifyArgs), bool warped, int tiles, int R) {
     int log2 = tiles >= 96 ? 4 : tiles >= 64 ? 3 : tiles >= 32 ? 2 : tiles >= 16 ? 1 : 0;
+    if (log2 == 4 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        log2 = 3;
+    }
     while (log2 > 0 && R > resident_clusters(kernel, warped, log2)) --log2;
     return log2;
 }
@@ -2435,8 +2443,6 @@ int launch_verify(const VerifyArgs &args, int R, int tiles, cudaStream_t stream)
     const bool warped = args.top_k > 0;
     const auto kernel = warped ? k_verify<true> : k_verify<false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess)
-        return DSBD_ERR_CUDA;
-    if (tiles >= 96 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return DSBD_ERR_CUDA;
     const int cs = 1 << cluster_log2_for(kernel, warped, tiles, R);
     cudaLaunchConfig_t cfg = {};
@@ -2488,6 +2494,17 @@ int launch_tile_stats(int64_t items, cudaStream_t stream, const float *zp, const
 extern "C" size_t dsbd_verify_workspace(const dsbd_forest_t *forest, const dsbd_verify_params_t *params) {
     if (check_forest(forest) != DSBD_OK || check_params(params) != DSBD_OK) return 0;
     return make_layout(forest, params->V).total;
+}
+
+extern "C" int dsbd_verify_cluster_ctas(const dsbd_forest_t *forest, const dsbd_verify_params_t *params, int32_t *resident) {
+    if (check_forest(forest) != DSBD_OK || check_params(params) != DSBD_OK) return 0;
+    const Layout L = make_layout(forest, params->V);
+    const bool warped = params->top_k > 0;
+    const auto kernel = warped ? k_verify<true> : k_verify<false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVerifyDynSmem) != cudaSuccess) cudaGetLastError();
+    const int log2 = cluster_log2_for(kernel, warped, L.max_live * L.T, forest->R);
+    if (resident) *resident = resident_clusters(kernel, warped, log2);
+    return 1 << log2;
 }
 
 extern "C" int dsbd_verify_step(const dsbd_forest_t *f, const dsbd_verify_params_t *p,

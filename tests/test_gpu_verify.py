@@ -930,3 +930,24 @@ def test_a_second_root_inside_a_tree(depth, beams):
     assert not np.any(np.isin(bad["node_status"][n:bno[forest["req_beam_off"][1] + 2]], (1, 2, 3)))
     assert bad["out_width"][1] >= 1
     _others_unchanged(forest, prm, 1, good, bad)
+
+
+@pytest.mark.parametrize("top_k", [0, 10])
+def test_cluster_sizes_are_the_largest_of_which_all_requests_fit(top_k):
+    """6 rows of 16 tiles: 16 CTAs to a request up to as many requests as the device says it holds such clusters, from one more on 8, and
+    so on down to 1; fewer tiles, smaller clusters.  Clusters stay inside a GPC and two CTAs fit an SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+
+    def asked(R, rows, V):
+        arrays = dict(req_beam_off=None, beam_node_off=None, parent=None, token=None)
+        f = dsbd.Forest.from_device(R, R, R, 1, {k: torch.zeros(4, dtype=torch.int32, device="cuda") for k in arrays}, 1, rows, rows)
+        return dsbd.verify_cluster_ctas(f, dict(V=V, W_min=1, W_max=1, W_nom=1, top_k=top_k))
+
+    R = 1
+    for ctas in (16, 8, 4, 2):
+        got, resident = asked(R, 6, 16384)
+        assert got == ctas and sms // 2 < resident * ctas <= 2 * sms
+        assert asked(resident, 6, 16384) == (ctas, resident)
+        R = resident + 1
+    assert asked(R, 6, 16384)[0] == 1
+    assert [asked(1, rows, 16384)[0] for rows in (5, 4, 3, 2, 1)] == [8, 8, 4, 4, 2] and asked(1, 1, 15000)[0] == 1

@@ -100,3 +100,25 @@ def test_a_merge_record_that_nobody_wrote_names_no_unit():
                          (0, -big - 1), (0x11111111, 0x11111111), (big, -1)]:
         assert not ok(1, 0, 7, 2, n_lo, n_tree), (n_lo, n_tree)
     assert not ok(1, 0, 8, 2, 0, 1) and not ok(1, 0, -1, 2, 0, 1) and not ok(1, 0, 7, 65, 0, 1) and not ok(1, 0, 7, -1, 0, 1)
+
+
+def _verify_shape(R, rows, V, top_k):
+    f = binding.ForestT(R, R, R, 1, 1, 1, 1, 1, 0, 1, rows, rows)          # (the pointers are not followed)
+    return f, binding.VerifyParamsT(V=V, temperature=1.0, thresh=0.7, W_min=1, W_max=1, W_nom=1, top_k=top_k, top_p=1.0)
+
+
+def test_cluster_sizes_without_a_device_s_answer():
+    """148 SMs of two CTAs over the cluster's size, and no clusters of 16, which not every device takes."""
+    import pytest
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("the device answers")
+    lib = dsbd.load()
+    resident = ctypes.c_int32()
+    for top_k in (0, 10):
+        for R, ctas in [(1, 8), (37, 8), (38, 4), (74, 4), (75, 2), (148, 2), (149, 1), (5000, 1)]:
+            f, p = _verify_shape(R, 6, 16384, top_k)
+            assert lib.dsbd_verify_cluster_ctas(ctypes.addressof(f), ctypes.addressof(p), ctypes.addressof(resident)) == ctas
+            assert resident.value == 296 // ctas
+    f, p = _verify_shape(0, 6, 16384, 0)
+    assert lib.dsbd_verify_cluster_ctas(ctypes.addressof(f), ctypes.addressof(p), None) == 0

@@ -2011,8 +2011,12 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 if (e_half && (threadIdx.x & (kHalf - 1)) == 0) wsup.tmp[half].err = e_half;
                 __syncthreads();
                 const int e = uniform(wsup.tmp[0].err ? wsup.tmp[0].err : extra ? 0 : wsup.tmp[1].err);
-                if (e) { if (threadIdx.x == 0) sh.err = e; }
-                else if (warp == 0) {
+                if (e) {
+                    if (threadIdx.x == 0) {
+                        sh.err = e;
+                        if (extra) a.out.layer_width[(int64_t)r * (a.gamma + 1) + a.gamma] = W_nom;      // (reached, and its width known)
+                    }
+                } else if (warp == 0) {
                     finish_supports(wsup, !extra, lane);
                     // rho of every live draft from the warped joints
                     if (!a.select_mode) {

@@ -951,3 +951,17 @@ def test_cluster_sizes_are_the_largest_of_which_all_requests_fit(top_k):
         R = resident + 1
     assert asked(R, 6, 16384)[0] == 1
     assert [asked(1, rows, 16384)[0] for rows in (5, 4, 3, 2, 1)] == [8, 8, 4, 4, 2] and asked(1, 1, 15000)[0] == 1
+
+
+def test_an_extra_layer_whose_support_does_not_fit():
+    """300 tiles of equal bounds, more than the search for a support keeps: reported, no beam is drawn, and the width of the layer that was
+    reached is told as for any other."""
+    V, W = 300 * 1024, 2
+    forest = dict(R=1, B=W, N=W, max_depth=0, req_beam_off=np.array([0, W], np.int32), beam_node_off=np.arange(W + 1, dtype=np.int32),
+                  parent=np.full(W, -1, np.int32), token=np.zeros(W, np.int32))
+    prm = dict(V=V, temperature=1.0, thresh=0.5, W_min=W, W_max=W, W_nom=5, seed=1, step=0, top_k=10, top_p=1.0)
+    z, zero = torch.zeros(W, V, device="cuda"), torch.zeros(W, device="cuda")
+    gpu, status = run_gpu_verify(forest, prm, z, z, zero, zero)
+    assert status == 3 and gpu["req_error"][0] == 3                      # DSBD_DEV_CAPACITY
+    assert gpu["l_last"][0] == 1 and gpu["out_width"][0] == 0
+    assert gpu["layer_width"][0].tolist() == [5]

@@ -285,6 +285,7 @@ struct Shared {
     double tail[kMaxLive + 2];
     int bank, halves, need_exact, res_j, run_j, chain_pos;
     int n_draw;                             // completion draws of the request
+    int empty_tree;                         // some tree of the request has no nodes
     int on_demand, next_i;                  // a layer of known width: its passes are made when the accept loop asks
     // sums of an exact pass, in units of 2^-60, 2^-120 (what the first leaves) and 2^-44 (q): of this CTA's warps; of every
     // CTA, two passes in turn
@@ -1546,7 +1547,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
     // nothing about this SM's L1); the tile statistics only after the wait.
     int b_lo = uniform(ld_early(a.req_beam_off + r)), b_hi = uniform(ld_early(a.req_beam_off + r + 1));
     // (what is below uses the offsets as indexes: a request whose own contradict the forest is reported and taken as empty.  Those of its
-    // trees are looked at by the set-up; all warps together here cost 16 requests 0.9 us)
+    // trees are looked at further down, by a thread each: all warps together here cost 16 requests 0.9 us, warp 0 alone in the
+    // set-up one request 0.3)
     bool bad_off = b_lo < 0 || b_hi > a.B || b_lo > b_hi;
     if (bad_off) b_lo = b_hi = 0;
     int n_lo = uniform(ld_early(a.beam_node_off + b_lo)), n_hi = uniform(ld_early(a.beam_node_off + b_hi));
@@ -1568,6 +1570,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
 #endif
 
     TS(1);
+    if (threadIdx.x == 0) sh.empty_tree = 0;
     // (a CTA may store into another's shared memory once that CTA runs: arrived here, waited for below)
     cluster.barrier_arrive();
     if (!kWarped && threadIdx.x >= kVThreads - 1 - kMaxLive) {               // (the last warps: the first ones read the nodes)
@@ -1645,6 +1648,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 slp[i] = lp; slq[i] = lq;
             }
             __syncthreads();
+            // Every tree has nodes: then every root lies in the request and is one tree's only (else it would have either's score, another one in
+            // every CTA).
+            if (i < n_trees && nc.root[i] >= (i + 1 < n_trees ? nc.root[i + 1] : n_hi)) sh.empty_tree = 1;
             if (i < n_trees && nc.root[i] >= n_lo && nc.root[i] < n_hi) {
                 const int root = nc.root[i] - n_lo;
                 if (writer && nc.parent[root] != -1) report(a.status, DSBD_DEV_BAD_FOREST);
@@ -1684,6 +1690,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
             }
             __syncthreads();
         } else {
+#pragma unroll 1
+        for (int b = b_lo + (int)threadIdx.x; b < b_hi; b += kVThreads)
+            if (a.beam_node_off[b] >= a.beam_node_off[b + 1]) sh.empty_tree = 1;
         __threadfence();
         cluster.sync();
         // ---- log-prob of every draft token given its parent (all nodes at once) ----
@@ -1724,7 +1733,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
 #pragma unroll 1
                 for (int b = b_lo + (int)threadIdx.x; b < b_hi; b += kVThreads) {
                     const int root = a.beam_node_off[b];
-                    if (root < n_lo || root >= n_hi) continue;                // (the set-up reports it)
+                    if (root < n_lo || root >= n_hi) continue;                // (an empty tree's)
                     if (a.parent[root] != -1) report(a.status, DSBD_DEV_BAD_FOREST);
                     slp[root - n_lo] = (double)a.root_logp[b];
                     slq[root - n_lo] = (double)a.root_logq[b];
@@ -1830,28 +1839,17 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                 }
             } else {
                 sh.nA = b_hi - b_lo;
-                if (sh.nA > kMaxLive) { sh.err = DSBD_DEV_BAD_FOREST; sh.nA = 0; }
+                if (sh.nA > kMaxLive || sh.empty_tree || bad_off) { sh.err = DSBD_DEV_BAD_FOREST; sh.nA = 0; }
             }
         }
         __syncwarp();
         if (!a.select_mode) {
-            int nA = uniform(sh.nA);
-            auto tree_start = [&](int i) { return i < nA ? (cached ? nc.root[i] : a.beam_node_off[b_lo + i]) : n_hi; };
-            // Every tree has nodes, so that every root lies in the request and is one tree's only (else it would have either's score, another
-            // one in every CTA).
-            bool empty = false;
-#pragma unroll 1
-            for (int i0 = 0; i0 < nA; i0 += 32)
-                if (const int i = i0 + lane; i < nA) empty |= tree_start(i) >= tree_start(i + 1);
-            if (__any_sync(kFull, empty)) {
-                nA = 0;
-                if (lane == 0) { sh.nA = 0; sh.err = DSBD_DEV_BAD_FOREST; }
-            }
+            const int nA = uniform(sh.nA);
 #pragma unroll 1
             for (int i0 = 0; i0 < nA; i0 += 32) {
                 const int i = i0 + lane;
                 if (i >= nA) continue;
-                const int root = tree_start(i);
+                const int root = cached ? nc.root[i] : a.beam_node_off[b_lo + i];
                 sh.A[i] = root;
                 if (cached) nc.live[root - n_lo] = (uint8_t)i;
                 sp_live[i] = cached ? nc.score_p[root - n_lo] : a.score[root];
@@ -1882,7 +1880,7 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         for (int n0 = 0; n0 < n_req_nodes && st_ok; n0 += kVThreads)
             if (const int n = n0 + threadIdx.x; n < n_req_nodes) st[n] = is_root(n) ? DSBD_NODE_ACCEPTED : DSBD_NODE_UNREACHED;
     __syncthreads();
-    if (!a.select_mode && (!st_ok || bad_off) && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
+    if (!a.select_mode && !st_ok && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_FOREST;
     if (bad_widths && threadIdx.x == 0) sh.err = DSBD_DEV_BAD_PARAM;
     __syncthreads();
     // node data by local index, from the cache when there is one

@@ -2020,7 +2020,6 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     finish_supports(wsup, !extra, lane);
                     // rho of every live draft from the warped joints
                     if (!a.select_mode) {
-                        draft_tests(sh, m, lane);
 #pragma unroll 1
                         for (int i0 = 0; i0 < m; i0 += 32) {
                             const int i = i0 + lane;

@@ -261,7 +261,7 @@ constexpr int kOverSlots = 256;                   // copies of the last bin (rho
 
 // The bins of a layer of m drafts: scale bins to a power of two; the upper edge of a bin over 2^(k / scale), and one over the width
 // of a bin over the same, both with the edges' tolerance (2e-6).
-struct BinEdges { float scale, inv_scale; double hi, inv_width; };
+struct BinEdges { float scale; double inv_scale, hi, inv_width; };
 constexpr double kEdgeTol = 2e-6;
 
 struct Shared {
@@ -1577,8 +1577,8 @@ k_verify(const __grid_constant__ VerifyArgs a) {
         const int m = threadIdx.x - (kVThreads - 1 - kMaxLive);
         BinEdges e;
         e.scale = (float)((double)kBins / log2((double)max(m, 2)));          // s_j <= j <= m
-        e.inv_scale = 1.f / e.scale;
-        e.hi = exp2(1.0 / (double)e.scale) * (1.0 + kEdgeTol);
+        e.inv_scale = 1.0 / (double)e.scale;
+        e.hi = exp2(e.inv_scale) * (1.0 + kEdgeTol);
         e.inv_width = 1.0 / (e.hi - (1.0 - kEdgeTol));
         sh.bins[m] = e;
     }
@@ -2109,8 +2109,9 @@ k_verify(const __grid_constant__ VerifyArgs a) {
                     const int found = j == 1 ? 0 : (int)(log2f((float)s_j) * binscale), k = min(max(found, 0), kBins - 1);   // (s_1 = 1, the first edge)
                     uint4 e0 = ld_cluster(entries + suffix_entry(k) * 16);
                     const uint4 e1 = ld_cluster(entries + suffix_entry(k + 1) * 16);
-                    // the bin's edges while the words are on their way: t = k / binscale, correctly rounded but for rare last places
-                    const float t0 = (float)k * bins.inv_scale, t = fmaf(fmaf(-t0, binscale, (float)k), bins.inv_scale, t0);
+                    // the bin's edges while the words are on their way; k / scale, rounded to a float (a division of floats: 0.6 us of
+                    // 36.9, one request of V = 32000)
+                    const float t = (float)((double)k * bins.inv_scale);
                     const double edge = (double)exp2f(t), inv = (double)exp2f(-t) * bins.inv_width;
                     const double r_lo = edge * (1.0 - kEdgeTol), r_hi = edge * bins.hi;
                     // every partial sum of the histogram is off by at most half a unit per cell

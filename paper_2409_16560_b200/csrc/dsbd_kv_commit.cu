@@ -118,7 +118,9 @@ __device__ __forceinline__ void block_exclusive_scan(T *const (&v)[K], int n, T 
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kPlanThreads)
+// (One CTA to an SM, said to the compiler: else it keeps to 32 registers and spills 56 bytes; paged update of 32 requests 29.7 us -> 28.9, of
+// 4 19.6 -> 18.8.)
+__global__ void __launch_bounds__(kPlanThreads, 1)
 k_commit_plan(CommitArgs a) {
     __shared__ int64_t tot64[3][32];
     __shared__ int32_t tot32[1][32];

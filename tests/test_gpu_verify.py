@@ -965,3 +965,29 @@ def test_an_extra_layer_whose_support_does_not_fit():
     assert status == 3 and gpu["req_error"][0] == 3                      # DSBD_DEV_CAPACITY
     assert gpu["l_last"][0] == 1 and gpu["out_width"][0] == 0
     assert gpu["layer_width"][0].tolist() == [5]
+
+
+@pytest.mark.parametrize("V", [524289, 525312, 600001, 1050000])
+def test_draws_from_the_last_of_a_row_s_tile_masses(V):
+    """A draw from p_beam searches its row's tile masses 512 at a time: here most of each row's mass lies behind the first (second) 512, in
+    one token, one tile, 74 and two tiles there."""
+    rng = np.random.default_rng(V + 1)
+    forest, prm, zp, zq, rp, rq, _ = _random_problem(rng, R=2, V=V, gamma=1, max_w=2, min_w=2)
+    last = (V - 1) // (512 * 1024) * (512 * 1024)
+    for z in (zp, zq):
+        z[:, last:] += np.log(20.0 * V / (V - last)).astype(np.float32)
+    dev = [torch.as_tensor(x).cuda() for x in (zp, zq, rp, rq)]
+    exempt = decisions = behind = 0
+    for step in range(8):
+        prm.update(step=step, thresh=0.3, W_min=2, W_min_r=None, W_nom=8)
+        gpu, status = run_gpu_verify(forest, prm, *dev)
+        assert status == 0
+        e, d = compare_verify(_oracle(forest, prm, zp, zq, rp, rq), gpu, forest)
+        exempt += e
+        decisions += d
+        out_off = oracle.default_out_off(forest, prm)
+        for r in range(2):
+            s = slice(out_off[r], out_off[r] + gpu["out_width"][r])
+            behind += int(((gpu["out_token"][s] >= last) & (gpu["out_source"][s] >= 2)).sum())        # fills, extra draws
+    check_exempt(exempt, decisions)
+    assert behind > 0

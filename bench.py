@@ -299,11 +299,12 @@ def _side_workload(dsbd, inputs, dev, name, steps, warmup, top_k=0, top_p=1.0, p
     return res
 
 
+# by stamp: the phase that ends there
 PHASE_NAMES = {1: "start", 2: "prologue / previous layer's completion", 3: "layer set-up", 4: "histogram pass",
-               5: "wait for the cluster's slices", 6: "wait for the cluster's passes",
-               7: "merge and suffix sums of a slice", 8: "residual chain",
-               9: "width and accept loop", 10: "residual pass for a completion draw", 11: "completion draws",
-               12: "extra layer and final writes", 13: "wait for the dense pass", 14: "log-sum-exps"}
+               5: "wait for the cluster's suffix sums", 7: "suffix sums",
+               8: "residual chain, warped supports or passes on demand", 9: "width and accept loop",
+               10: "residual pass for a completion draw", 11: "completion draws", 13: "wait for the dense pass",
+               14: "log-sum-exps"}
 
 
 def run_verify_phases(args):

@@ -122,3 +122,9 @@ def test_cluster_sizes_without_a_device_s_answer():
             assert resident.value == 296 // ctas
     f, p = _verify_shape(0, 6, 16384, 0)
     assert lib.dsbd_verify_cluster_ctas(ctypes.addressof(f), ctypes.addressof(p), None) == 0
+
+
+def test_every_time_stamp_of_the_verification_has_a_name():
+    import bench
+    text = open(os.path.join(ROOT, "paper_2409_16560_b200", "csrc", "dsbd_verify.cu")).read()
+    assert {int(x) for x in re.findall(r"\bTS\((\d+)\)", text)} == set(bench.PHASE_NAMES)

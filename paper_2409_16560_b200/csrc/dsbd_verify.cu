@@ -1509,12 +1509,17 @@ __device__ void finish_supports(WarpScratch &ws, bool have_q, int lane) {
 
 // Drafts behind the first rejection of a layer of known width up to which its residual masses are computed on demand: a pass
 // for that rejection and at most one for each of them, against one histogram, and a pass more where the layer ends in a residual
-// draw behind a second rejection.  A histogram costs about 1.9 passes where a warp has eight tiles of a pass and 2.8 where it
-// has one or two, its merge (that there was) and chain being as long for few tiles; without the merge two, three and four are within 2 per
-// cent on seven shapes, but for a call 11 per cent slower with four.  Layers of three and four drafts, mean of the benchmark's
-// distributions with as many accepts and with fewer, against a histogram for every rejection: 64 requests of 128256
-// tokens up to 2 drafts 1.03 and 1.01 times as fast, up to 3 0.97 and 0.93; 160 of 32000 1.05 and 1.03, 1.00 and 0.95; 16
-// of 128256 1.16 and 1.11, 1.20 and 1.14; one of 32000 1.12 and 1.07, 1.14 and 1.09.
+// draw behind a second rejection.  Us a call with limits of none to four, every layer of known width, mean of three to six inputs of
+// the benchmark's distributions (without passes on demand: 31.4, 43.7, 55.3, 130, 460, 925):
+//                                             0      1      2      3      4
+//    one request, 4 beams, V = 32000       31.4   31.4   29.4   29.0   29.1      a warp has at most two tiles of a pass
+//    one request, 4 beams, V = 128256      42.1   40.8   40.5   39.8   39.8      likewise
+//    16 requests, 4 beams, V = 32000       54.9   53.2   52.9   56.0   56.0      likewise: the slowest of 16 counts
+//    16 requests, 4 beams, V = 128256       130    129    131    139    139
+//    64 requests, 4 beams, V = 128256       460    457    463    492    490
+//    64 requests, 8 beams, V = 128256       925    922    920    935    977
+// 2 is within 1.5 per cent of the best wherever there are many tiles.  Where there are few, 3 gains 1 to 2 per cent for a single request
+// and loses 6 for 16 of them.
 __device__ __forceinline__ int on_demand_left(int n_tiles, int n_warps) { return n_tiles <= 2 * n_warps ? 3 : 2; }
 
 // dynamic shared memory of k_verify: the histogram of a layer as four 32-bit arrays while it is
